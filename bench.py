@@ -556,9 +556,8 @@ def run_e2e(args, wl, pg, cu_list, host, dev, world, barrier, binding):
 
 def run_widened(args):
     """Builder-run lines for the rows widened after the hot path (not the driver's metric):
-    --workload SIM     the dense redundancy-analysis map (block 16) of the keys of a C3 layer, a
-                       tensor-core contraction: roofline bound "tensor" against the measured bf16
-                       peak, algorithmic flops = 2 L^2 d per head;
+    --workload SIM     the redundancy-analysis map (block 16) of the keys of a C3 layer: rows read and
+                       cells written per second against the measured copy peak;
     --workload DECODE  one decode token over the C3b compact cache (28 layers x 4 heads x 512
                        rows): bytes of cache read per second against the measured copy peak."""
     import torch
@@ -599,20 +598,21 @@ def run_widened(args):
             it[0] += 1
 
         ms = timed(fn, max(4, min(args.steps, 20)))
-        flops = 2.0 * L * L * 128 * H
-        ach = flops / (ms * 1e-3) / 1e12
+        T = -(-L // block)
+        nbytes = H * (L * 256.0 + T * T * 4.0)     # rows read once, cells written once
+        ach = nbytes / (ms * 1e-3) / 1e9
         line = {"metric": "similarity_rows_per_s", "value": H * L / (ms * 1e-3), "unit": "rows/s",
-                "n_gpus": 1, "ms_per_step": ms, "higher_is_better": True, "dtype": "bf16 hi/lo in, f32 accumulate",
+                "n_gpus": 1, "ms_per_step": ms, "higher_is_better": True, "dtype": "bf16 parts in, f32 accumulate",
                 "data": "synthetic",
                 "config": {"workload": f"SIM: block-{block} cosine map of the keys of a C3 layer, "
                                        f"H={H}, L={L}, d=128, {args.variant} keys; inputs of 4 layers cycled"},
-                "roofline": {"bound": "tensor", "achieved": ach, "peak": pk["bf16_tflops"],
-                             "unit": "TFLOP/s", "frac": ach / pk["bf16_tflops"], "traffic": None,
-                             "peak_source": "measured cuBLAS bf16 (burst)",
-                             "algorithmic_flops_per_launch": flops,
-                             "executed_flops_per_launch": flops * 1.5,
-                             "note": "executed = upper triangle (x 1/2) of three bf16 products "
-                                     "(hi.hi, hi.lo, lo.hi: x 3)"}}
+                "roofline": {"bound": "hbm", "achieved": ach, "peak": pk["hbm_gbs"],
+                             "unit": "GB/s", "frac": ach / pk["hbm_gbs"], "traffic": None,
+                             "peak_source": "measured copy bandwidth",
+                             "algorithmic_bytes_per_launch": nbytes,
+                             "executed_flops_per_launch": H * T * (T + 128) * 128.0 * 6,
+                             "note": "executed = upper triangle of tiles of the Gram matrix of the block "
+                                     "sums, six products of bf16 parts"}}
     else:
         NL, H, G, B = 28, 4, 7, 512
         rows = H * B

@@ -274,12 +274,10 @@ int mixkv_layer_budget_schedule(int32_t n_layers, int32_t budget, int32_t window
  *   mean_opt   device, [heads] fp32 or NULL: mean over all ordered pairs i != j of the head,
  *              the redundancy of Eq. 4
  *   workspace  device, mixkv_similarity_workspace_size bytes, 16-byte aligned, caller-owned
- * A zero row has cosine 0 with every row.  Two routes: for block = 1, 2, 4, 8 or 16 the dense
- * matrix X^ X^T of Eq. 3 is formed on the tensor cores (rows normalised once into two bf16
- * halves, upper triangle of 128 x 128 tiles, cells reduced in the epilogue); for every other
- * block size the cells come from the Gram matrix of the per-block sums of unit rows (one
- * streaming pass over X).  The workspace size depends on the route.  Errors as for the other
- * entry points. */
+ * A zero row has cosine 0 with every row.  The cells come from the Gram matrix of the
+ * per-block sums of unit rows (one streaming pass over X, then the upper triangle of tiles on the
+ * tensor cores, the sums as two (block == 1) or three bf16 parts).  Errors as for the other entry
+ * points. */
 int mixkv_similarity_workspace_size(int32_t heads, int32_t L, int32_t block, size_t* bytes);
 int mixkv_similarity_map(const void* X, int32_t heads, int32_t L, int32_t head_dim, int32_t block,
                          void* workspace, size_t workspace_bytes, float* cells, float* mean_opt,

@@ -118,12 +118,18 @@ __host__ __device__ __forceinline__ size_t ppos(const SeqTable& st, int layer, i
   return ((size_t)layer * st.H + h) * st.Ptot + (st.cu[b] - b * st.W) + i;
 }
 
-// Dense (tensor-core) route of the similarity map for block = 1, 2, 4, 8, 16 (similarity_tc.cu).
-bool similarity_dense_block(int block);
-size_t similarity_dense_workspace(int heads, int L);
-cudaError_t launch_similarity_dense(const void* X, int heads, int L, int block, void* workspace,
-                                    float* cells, float** u_out, int** nz_out, int* slices_out,
-                                    cudaStream_t s);
+// Gram matrix of the block sums of a similarity map (similarity_tc.cu).
+struct GramArgs {
+  const void* parts;   // [nparts][heads][T][d] bf16: the block sums as 2 or 3 bf16 parts
+  int nparts;
+  const int* nz;       // [heads][T]       non-zero rows of a block
+  const float* us;     // [heads][slices][d]  partial sums of all unit rows of a head
+  const int* nzs;      // [heads][slices]
+  int slices, heads, L, block, T;
+  float* cells;        // [heads][T][T]
+  float* mean;         // [heads] or nullptr
+};
+cudaError_t launch_gram(const GramArgs& g, cudaStream_t s);
 
 struct TailArgs {
   const float* scores;

@@ -1,169 +1,326 @@
 // Redundancy analysis (the pairwise key / value similarity the paper plots as heat maps and
-// summarises per head, Sec. 1 and Sec. 3.1): block-mean cosine similarity map of the rows of
-// one tensor.  The mean of cos(x_i, x_j) over a cell (i in block I, j in block J) is
-// u_I . u_J / (n_I n_J) with u_I the sum of the unit rows of block I, the same identity that
-// turns the mean of the whole matrix into Eq. 4; so the map needs one streaming pass over the
-// rows (HBM bound) and a small Gram matrix of the block sums, not the L x L matrix.  That is the
-// route for coarse maps; with 1 .. 16 rows per cell the Gram of block sums is the L x L
-// contraction itself and runs on the tensor cores (similarity_tc.cu).
+// summarises per head, Sec. 1 and Sec. 3.1): block-mean cosine similarity map of the rows of one
+// tensor.  The mean of cos(x_i, x_j) over a cell (i in block I, j in block J) is
+// u_I . u_J / (n_I n_J) with u_I the sum of the unit rows of block I, the same identity that turns
+// the mean of the whole matrix into Eq. 4.  So a map needs one streaming pass over the rows, which
+// leaves the block sums (k_block_sums, here), and the Gram matrix of the block sums on the tensor
+// cores (k_gram, similarity_tc.cu): never more than T x T x d multiply-adds for T x T cells, T = L
+// only where a cell is one pair of rows.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace mixkv {
 namespace {
 
-constexpr int kSimThreads = 256;
-constexpr int kSimRows = 256;   // rows one CTA of the first kernel reads
+constexpr int kSumWarps = 8;
+constexpr int kSumThreads = kSumWarps * 32;
+constexpr int kSumRows = 32;        // rows a warp holds in registers at a time (8 KB of loads in flight)
+constexpr int kSumMaxCluster = 8;
 
-// grid (T * S, H): unit-row sum and number of non-zero rows of one slice (kSimRows rows at most;
-// S slices per block) of one block of one head.  A warp takes four rows at a time (all loads in
-// flight); lane l holds elements 4l .. 4l+3 of a row.  u, nz: [H, T * S, ...].
-__global__ void __launch_bounds__(kSimThreads)
-k_block_unit_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block, const int S,
-                  float* __restrict__ u, int* __restrict__ nz) {
-  __shared__ float part[kSimThreads / 32][kHeadDim];
-  __shared__ int cnt[kSimThreads / 32];
-  const int I = blockIdx.x / S, sl = blockIdx.x % S, h = blockIdx.y, T = gridDim.x;   // T: slices per head
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int b1 = min(L, (I + 1) * block);
-  const int r0 = min(b1, I * block + sl * kSimRows), r1 = min(b1, r0 + kSimRows);
-  const __nv_bfloat16* base = X + (size_t)h * L * kHeadDim;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  int nonzero = 0;
-  constexpr int kW = kSimThreads / 32, kInFlight = 4;   // rows a warp loads before it reduces any
-  for (int r = r0 + warp; r < r1; r += kInFlight * kW) {
-    uint2 v[kInFlight];
+// Three layouts of the work of k_block_sums, by the rows per block.
+enum { kRowsOne = 0,    // block == 1: every row leaves as its own "sum"
+       kRowsFew = 1,    // block <= 32: a warp takes whole blocks
+       kRowsMany = 2 }; // longer blocks: the warps of a CTA (or of a cluster) share one
+
+__host__ __device__ constexpr int sum_mode(int block) {
+  return block == 1 ? kRowsOne : block <= kSumRows ? kRowsFew : kRowsMany;
+}
+// Blocks one CTA (or cluster) takes.
+__host__ __device__ inline int blocks_per_cta(int block) {
+  if (block <= kSumRows) return kSumWarps * (kSumRows / block);
+  const int sub = (block + kSumRows - 1) / kSumRows;
+  return sub < kSumWarps ? kSumWarps / sub : 1;
+}
+// Bits of the rows a .. b-1 of a warp's 32 rows, where row 2 i + half is bit 16 half + i.
+__device__ __forceinline__ unsigned row_bits(const int a, const int b) {
+  const unsigned even = ((1u << ((b + 1) >> 1)) - 1u) & ~((1u << ((a + 1) >> 1)) - 1u);
+  const unsigned odd = ((1u << (b >> 1)) - 1u) & ~((1u << (a >> 1)) - 1u);
+  return even | (odd << 16);
+}
+
+// x as a sum of bf16 parts, most significant first (8 mantissa bits each).
+template <int P>
+__device__ __forceinline__ void split_parts(const float (&x)[8], uint4 (&part)[P]) {
+  __nv_bfloat16 h[P][8];
 #pragma unroll
-    for (int k = 0; k < kInFlight; ++k) {
-      const int rk = r + k * kW;
-      v[k] = rk < r1 ? *reinterpret_cast<const uint2*>(base + (size_t)rk * kHeadDim + 4 * lane)
-                     : make_uint2(0u, 0u);
-    }
-    float f[kInFlight][4], n2[kInFlight];
+  for (int e = 0; e < 8; ++e) {
+    float r = x[e];
 #pragma unroll
-    for (int k = 0; k < kInFlight; ++k) {
-      const float2 p = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v[k].x));
-      const float2 q = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v[k].y));
-      f[k][0] = p.x, f[k][1] = p.y, f[k][2] = q.x, f[k][3] = q.y;
-      n2[k] = (p.x * p.x + p.y * p.y) + (q.x * q.x + q.y * q.y);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-      for (int k = 0; k < kInFlight; ++k) n2[k] += __shfl_xor_sync(0xffffffffu, n2[k], o);
-#pragma unroll
-    for (int k = 0; k < kInFlight; ++k) {
-      const float inv = n2[k] > 0.f ? rsqrtf(n2[k]) : 0.f;
-      nonzero += n2[k] > 0.f;
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[e] = fmaf(f[k][e], inv, acc[e]);
+    for (int p = 0; p < P; ++p) {
+      h[p][e] = __float2bfloat16_rn(r);
+      r -= __bfloat162float(h[p][e]);
     }
   }
 #pragma unroll
-  for (int e = 0; e < 4; ++e) part[warp][4 * lane + e] = acc[e];
-  if (lane == 0) cnt[warp] = nonzero;
+  for (int p = 0; p < P; ++p) part[p] = *reinterpret_cast<const uint4*>(h[p]);
+}
+
+// grid (slices * cluster, H).  Sums of the unit rows of every block, written as P bf16 parts
+// ([P][H][T][d]: two parts where a row stands for itself, three, fp32's 24 bits, for sums), the
+// number of non-zero rows of every block, and per slice (what one CTA or cluster read) the sum of
+// its unit rows and its non-zero rows, from which the head mean comes.
+//
+// HBM bound: every row is read once, 16 lanes of 16 bytes to a row, all 32 rows of a warp's step
+// asked for before the first is used (8 KB per warp, 16 warps per SM).  The 32 squared norms of a
+// step are reduced by folding (15 exchanges per lane instead of 64 for 16 butterflies).  131072 rows
+// (four heads of 32768) in blocks of 256: 13.3 us before (four rows per warp in flight), see the
+// dispatch for the present figure.
+template <int MODE, int P>
+__global__ void __launch_bounds__(kSumThreads, 2)
+k_block_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block, const int T,
+             __nv_bfloat16* __restrict__ parts, int* __restrict__ nz, float* __restrict__ us,
+             int* __restrict__ nzs) {
+  __shared__ float part[kSumWarps][kHeadDim];
+  __shared__ int cnt[kSumWarps];
+  __shared__ float csum[kHeadDim];
+  __shared__ int ccnt;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int S = MODE == kRowsMany ? (int)cluster.num_blocks() : 1;
+  const int rank = MODE == kRowsMany ? (int)cluster.block_rank() : 0;
+  const int slice = blockIdx.x / S, h = blockIdx.y, H = gridDim.y, nslices = gridDim.x / S;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, half = lane >> 4, c = lane & 15;
+  const int bpc = blocks_per_cta(block);
+  const size_t part_stride = (size_t)H * T * kHeadDim;
+  const __nv_bfloat16* base = X + (size_t)h * L * kHeadDim + 8 * c;
+  __nv_bfloat16* prow = parts + (size_t)h * T * kHeadDim + 8 * c;
+  pdl_launch_dependents();
+  pdl_wait();
+
+  float tot[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) tot[e] = 0.f;
+  int tot_nz = 0;
+
+  // The warp's rows: whole blocks (few rows per block), or a share of one block.
+  int first, end, stride;      // first row, end of the warp's range, rows between its steps
+  int blk = 0;                 // block the range starts in
+  if (MODE != kRowsMany) {
+    const int per_warp = kSumRows / block;
+    blk = slice * bpc + warp * per_warp;
+    first = blk * block;
+    end = min(L, first + per_warp * block);
+    stride = kSumRows;
+  } else {
+    const int sub = (block + kSumRows - 1) / kSumRows;   // steps of a block
+    const int share = sub < kSumWarps ? sub : kSumWarps; // warps of a CTA on one block
+    const int slot = warp / share;
+    blk = slice * bpc + slot;
+    first = blk * block + (rank * share + warp - slot * share) * kSumRows;
+    end = slot < bpc ? min(L, (blk + 1) * block) : 0;
+    stride = S * share * kSumRows;
+  }
+#pragma unroll 1
+  for (int r0 = first; r0 < end; r0 += stride) {
+    uint4 v[16];
+    float p[16];
+    const uint4* rp = reinterpret_cast<const uint4*>(base + (size_t)(r0 + half) * kHeadDim);
+    const int left = end - r0 - half;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {   // one address, constant offsets
+      v[i] = make_uint4(0, 0, 0, 0);
+      if (2 * i < left) v[i] = __ldg(rp + 2 * i * (kHeadDim / 8));
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const uint32_t* w = reinterpret_cast<const uint32_t*>(&v[i]);
+      float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        // (byte permutes here, shifts below: with the same instructions in both sweeps the 256
+        // widened values would be kept, which does not fit the registers)
+        const float a = __uint_as_float(__byte_perm(w[e], 0u, 0x1044)),
+                    b = __uint_as_float(__byte_perm(w[e], 0u, 0x3244));
+        s0 = fmaf(a, a, s0);
+        s1 = fmaf(b, b, s1);
+      }
+      p[i] = s0 + s1;
+    }
+    // folding: lane c of a half is left with the squared norm of row 2 c + half
+#pragma unroll
+    for (int o = 8; o >= 1; o >>= 1) {
+      const bool up = (c & o) != 0;
+#pragma unroll
+      for (int k = 0; k < o; ++k) {
+        const float send = up ? p[k] : p[k + o], keep = up ? p[k + o] : p[k];
+        p[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    }
+    const float inv = p[0] > 0.f ? rsqrtf(p[0]) : 0.f;
+    const unsigned alive = __ballot_sync(0xffffffffu, p[0] > 0.f);
+    tot_nz += __popc(alive);
+    float acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+    // sum of the two halves' accumulators -> the parts of block `blk` (rows a .. b-1 of the step)
+    auto flush = [&](const float (&mine)[8], const int a, const int b) {
+      float s[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        s[e] = mine[e] + __shfl_xor_sync(0xffffffffu, mine[e], 16);
+        tot[e] += s[e];
+      }
+      if (blk < T) {
+        uint4 q[P];
+        split_parts<P>(s, q);
+        // half 0 writes parts 0 and 2, half 1 part 1
+        *reinterpret_cast<uint4*>(prow + (size_t)half * part_stride + (size_t)blk * kHeadDim) =
+            half ? q[1] : q[0];
+        if (P == 3 && half == 0)
+          *reinterpret_cast<uint4*>(prow + 2 * part_stride + (size_t)blk * kHeadDim) = q[P - 1];
+        if (lane == 0) nz[(size_t)h * T + blk] = __popc(alive & row_bits(a, b));
+      }
+      ++blk;
+    };
+    int next = block, a0 = 0;   // kRowsFew: row of the step at which the current block ends / starts
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const float w = __shfl_sync(0xffffffffu, inv, (lane & 16) | i);
+      const uint32_t* q = reinterpret_cast<const uint32_t*>(&v[i]);
+      float x[8];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        x[2 * e] = __uint_as_float(q[e] << 16) * w;
+        x[2 * e + 1] = __uint_as_float(q[e] & 0xffff0000u) * w;
+      }
+      if (MODE == kRowsOne) {
+        const int r = r0 + 2 * i + half;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) tot[e] += x[e];
+        if (r < end) {
+          uint4 o2[P];
+          split_parts<P>(x, o2);
+#pragma unroll
+          for (int k = 0; k < P; ++k)
+            *reinterpret_cast<uint4*>(prow + k * part_stride + (size_t)r * kHeadDim) = o2[k];
+          if (c == 0) nz[(size_t)h * T + r] = w > 0.f ? 1 : 0;
+        }
+      } else if (MODE == kRowsFew) {
+        if (next == 2 * i + 1) {   // the block ends between the two rows of this pair
+#pragma unroll
+          for (int e = 0; e < 8; ++e) acc[e] += half == 0 ? x[e] : 0.f;
+          flush(acc, a0, next);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) acc[e] = half == 0 ? 0.f : x[e];
+          a0 = next;
+          next += block;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) acc[e] += x[e];
+        }
+        if (next == 2 * i + 2) {
+          flush(acc, a0, next);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+          a0 = next;
+          next += block;
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) tot[e] += x[e];
+      }
+    }
+  }
+  // per-warp sums of unit rows (kRowsFew: the two halves already hold the same totals)
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const float s = MODE == kRowsFew ? tot[e] : tot[e] + __shfl_xor_sync(0xffffffffu, tot[e], 16);
+    if (half == 0) part[warp][8 * c + e] = s;
+  }
+  if (lane == 0) cnt[warp] = tot_nz;
   __syncthreads();
-  if (threadIdx.x < kHeadDim) {
+  if (MODE == kRowsMany) {
+    const int sub = (block + kSumRows - 1) / kSumRows;
+    const int share = sub < kSumWarps ? sub : kSumWarps;
+    if (S > 1) {   // one block per cluster: every CTA's sum, then rank 0 adds them in rank order
+      if (tid < kHeadDim) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < kSumWarps; ++w) s += part[w][tid];
+        csum[tid] = s;
+      }
+      if (tid == 0) {
+        int n = 0;
+        for (int w = 0; w < kSumWarps; ++w) n += cnt[w];
+        ccnt = n;
+      }
+      cluster.sync();
+      if (rank == 0) {
+        if (tid < kHeadDim) {
+          float s = 0.f;
+          for (int r = 0; r < S; ++r) s += *cluster.map_shared_rank(&csum[tid], r);
+          part[0][tid] = s;
+#pragma unroll
+          for (int w = 1; w < kSumWarps; ++w) part[w][tid] = 0.f;
+        }
+        if (tid == 0) {
+          int n = 0;
+          for (int r = 0; r < S; ++r) n += *cluster.map_shared_rank(&ccnt, r);
+          cnt[0] = n;
+          for (int w = 1; w < kSumWarps; ++w) cnt[w] = 0;
+        }
+      }
+      cluster.sync();   // the peers' shared memory stays alive until rank 0 has read it
+      if (rank != 0) return;
+    }
+    // block sums: one warp per block of the CTA, lane -> four dimensions
+    if (warp < bpc && slice * bpc + warp < T) {
+      const int I = slice * bpc + warp;
+      float s[4] = {0.f, 0.f, 0.f, 0.f};
+      int n = 0;
+      for (int w = warp * share; w < (warp + 1) * share; ++w) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[e] += part[w][4 * lane + e];
+        n += cnt[w];
+      }
+#pragma unroll
+      for (int k = 0; k < P; ++k) {
+        __nv_bfloat16 o[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          o[e] = __float2bfloat16_rn(s[e]);
+          s[e] -= __bfloat162float(o[e]);
+        }
+        *reinterpret_cast<uint2*>(parts + k * part_stride + ((size_t)h * T + I) * kHeadDim + 4 * lane) =
+            *reinterpret_cast<const uint2*>(o);
+      }
+      if (lane == 0) nz[(size_t)h * T + I] = n;
+    }
+  }
+  if (tid < kHeadDim) {
     float s = 0.f;
 #pragma unroll
-    for (int w = 0; w < kSimThreads / 32; ++w) s += part[w][threadIdx.x];
-    u[((size_t)h * T + blockIdx.x) * kHeadDim + threadIdx.x] = s;
+    for (int w = 0; w < kSumWarps; ++w) s += part[w][tid];
+    us[((size_t)h * nslices + slice) * kHeadDim + tid] = s;
   }
-  if (threadIdx.x == 0) {
-    int c = 0;
-    for (int w = 0; w < kSimThreads / 32; ++w) c += cnt[w];
-    nz[h * T + blockIdx.x] = c;
-  }
-}
-
-// grid (T, H), 128 threads: adds the S slices of a block (blocks longer than kSimRows rows).
-__global__ void __launch_bounds__(kHeadDim)
-k_fold_slices(const float* __restrict__ us, const int* __restrict__ nzs, const int S,
-              float* __restrict__ u, int* __restrict__ nz) {
-  const int I = blockIdx.x, h = blockIdx.y, T = gridDim.x, c = threadIdx.x;
-  float s = 0.f;
-  for (int k = 0; k < S; ++k) s += us[(((size_t)h * T + I) * S + k) * kHeadDim + c];
-  u[((size_t)h * T + I) * kHeadDim + c] = s;
-  if (c == 0) {
-    int z = 0;
-    for (int k = 0; k < S; ++k) z += nzs[(h * T + I) * S + k];
-    nz[h * T + I] = z;
-  }
-}
-
-// grid (ceil(T/16), ceil(T/16), H), 16 x 16 threads: cells of the map.
-__global__ void __launch_bounds__(256)
-k_block_map(const float* __restrict__ u, const int* __restrict__ nz, const int L, const int block,
-            const int T, float* __restrict__ cells) {
-  __shared__ float ui[16][kHeadDim + 1], uj[16][kHeadDim + 1];
-  const int h = blockIdx.z, I0 = blockIdx.y * 16, J0 = blockIdx.x * 16;
-  const int ty = threadIdx.y, tx = threadIdx.x, t = ty * 16 + tx;
-  {
-    // thread t stages column t % 128 of rows t / 128, t / 128 + 2, ... : all sixteen loads in flight
-    const int c = t & (kHeadDim - 1), rb = t >> 7;
-    float a[8], b[8];
+  if (tid == 0) {
+    int n = 0;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int r = rb + 2 * k;
-      a[k] = I0 + r < T ? u[((size_t)h * T + I0 + r) * kHeadDim + c] : 0.f;
-      b[k] = J0 + r < T ? u[((size_t)h * T + J0 + r) * kHeadDim + c] : 0.f;
-    }
-#pragma unroll
-    for (int k = 0; k < 8; ++k) ui[rb + 2 * k][c] = a[k], uj[rb + 2 * k][c] = b[k];
-  }
-  __syncthreads();
-  const int I = I0 + ty, J = J0 + tx;
-  if (I >= T || J >= T) return;
-  float dot = 0.f;
-#pragma unroll 8
-  for (int c = 0; c < kHeadDim; ++c) dot = fmaf(ui[ty][c], uj[tx][c], dot);
-  const float nI = (float)(min(L, (I + 1) * block) - I * block);
-  const float nJ = (float)(min(L, (J + 1) * block) - J * block);
-  float v;
-  if (I != J) {
-    v = dot / (nI * nJ);
-  } else {   // the pairs i == j are left out: each non-zero row has cosine 1 with itself
-    const float pairs = nI * (nI - 1.f);
-    v = pairs > 0.f ? (dot - (float)nz[h * T + I]) / pairs : 0.f;
-  }
-  cells[((size_t)h * T + I) * T + J] = v;
-}
-
-// grid H, 1024 threads: mean over all ordered pairs i != j of the head (Eq. 4).  Eight groups of
-// 128 threads walk the blocks side by side.
-__global__ void __launch_bounds__(1024)
-k_head_mean(const float* __restrict__ u, const int* __restrict__ nz, const int L, const int T,
-            float* __restrict__ mean) {
-  __shared__ float part[8][kHeadDim];
-  __shared__ float red[4];
-  __shared__ int zs[32];
-  const int h = blockIdx.x, c = threadIdx.x & (kHeadDim - 1), g = threadIdx.x >> 7;
-  float s = 0.f;
-#pragma unroll 16
-  for (int I = g; I < T; I += 8) s += u[((size_t)h * T + I) * kHeadDim + c];
-  part[g][c] = s;
-  int z = 0;
-  for (int I = threadIdx.x; I < T; I += 1024) z += nz[h * T + I];
-  for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-  if ((threadIdx.x & 31) == 0) zs[threadIdx.x >> 5] = z;
-  __syncthreads();
-  if (threadIdx.x < kHeadDim) {
-    float t = 0.f;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) t += part[k][c];
-    const float n2 = warp_sum(t * t);
-    if ((c & 31) == 0) red[c >> 5] = n2;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int total_nz = 0;
-    for (int w = 0; w < 32; ++w) total_nz += zs[w];
-    const double nn = ((double)red[0] + (double)red[1]) + ((double)red[2] + (double)red[3]);
-    const double Ld = (double)L;
-    mean[h] = L > 1 ? (float)((nn - (double)total_nz) / (Ld * (Ld - 1.0))) : 0.f;
+    for (int w = 0; w < kSumWarps; ++w) n += cnt[w];
+    nzs[(size_t)h * nslices + slice] = n;
   }
 }
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
+
+// What a call of this shape needs between its two kernels.
+struct SimPlan {
+  int T, slices, nparts;
+  size_t parts_bytes, nz_bytes, us_bytes, nzs_bytes;
+  SimPlan(int heads, int L, int block) {
+    T = (int)(((long long)L + block - 1) / block);
+    const int bpc = blocks_per_cta(block);
+    slices = (T + bpc - 1) / bpc;
+    nparts = block == 1 ? 2 : 3;
+    parts_bytes = align256((size_t)nparts * heads * T * kHeadDim * 2);
+    nz_bytes = align256((size_t)heads * T * 4);
+    us_bytes = align256((size_t)heads * slices * kHeadDim * 4);
+    nzs_bytes = align256((size_t)heads * slices * 4);
+  }
+  size_t bytes() const { return parts_bytes + nz_bytes + us_bytes + nzs_bytes; }
+};
 
 }  // namespace
 }  // namespace mixkv
@@ -174,14 +331,7 @@ extern "C" {
 
 int mixkv_similarity_workspace_size(int32_t heads, int32_t L, int32_t block, size_t* bytes) {
   if (!bytes || heads < 1 || L < 1 || block < 1) return MIXKV_ERR_INVALID_ARG;
-  if (similarity_dense_block(block)) {
-    *bytes = similarity_dense_workspace(heads, L);
-    return MIXKV_OK;
-  }
-  const size_t T = ((size_t)L + block - 1) / block;
-  const size_t S = ((size_t)block + kSimRows - 1) / kSimRows;   // slices per block
-  *bytes = align256((size_t)heads * T * kHeadDim * 4) + align256((size_t)heads * T * 4);
-  if (S > 1) *bytes += align256((size_t)heads * T * S * kHeadDim * 4) + align256((size_t)heads * T * S * 4);
+  *bytes = SimPlan(heads, L, block).bytes();
   return MIXKV_OK;
 }
 
@@ -192,47 +342,53 @@ int mixkv_similarity_map(const void* X, int32_t heads, int32_t L, int32_t head_d
   if (head_dim != kHeadDim) return MIXKV_ERR_UNSUPPORTED;
   if ((reinterpret_cast<uintptr_t>(X) & 15u) || (reinterpret_cast<uintptr_t>(workspace) & 15u))
     return MIXKV_ERR_INVALID_ARG;
+  if (block > L) block = L;   // one block either way
+  const SimPlan pl(heads, L, block);
   size_t need = 0;
   mixkv_similarity_workspace_size(heads, L, block, &need);
   if (workspace_bytes < need) return MIXKV_ERR_WORKSPACE_TOO_SMALL;
-  const long long T = ((long long)L + block - 1) / block;
-  const long long S = ((long long)block + kSimRows - 1) / kSimRows;
-  if (T > 65535 || heads > 65535 || T * S > 0x7fffffffLL) return MIXKV_ERR_UNSUPPORTED;   // grid limits
+  if (pl.T > 65535 || heads > 65535) return MIXKV_ERR_UNSUPPORTED;   // grid limits
   {
     const int rc = device_check(nullptr);
     if (rc != MIXKV_OK) return rc;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  if (similarity_dense_block(block)) {
-    float* ud = nullptr;
-    int* nzd = nullptr;
-    int slices = 0;
-    if (launch_similarity_dense(X, heads, L, block, workspace, cells, &ud, &nzd, &slices, s) !=
-        cudaSuccess)
-      return MIXKV_ERR_CUDA;
-    if (mean_opt) k_head_mean<<<(unsigned)heads, 1024, 0, s>>>(ud, nzd, L, slices, mean_opt);
-    return cudaGetLastError() == cudaSuccess ? MIXKV_OK : MIXKV_ERR_CUDA;
-  }
   unsigned char* wsb = reinterpret_cast<unsigned char*>(workspace);
-  float* u = reinterpret_cast<float*>(wsb);
-  wsb += align256((size_t)heads * T * kHeadDim * 4);
+  __nv_bfloat16* parts = reinterpret_cast<__nv_bfloat16*>(wsb);
+  wsb += pl.parts_bytes;
   int* nz = reinterpret_cast<int*>(wsb);
-  wsb += align256((size_t)heads * T * 4);
-  if (S == 1) {
-    k_block_unit_sums<<<dim3((unsigned)T, (unsigned)heads), kSimThreads, 0, s>>>(
-        reinterpret_cast<const __nv_bfloat16*>(X), L, block, 1, u, nz);
-  } else {
-    float* us = reinterpret_cast<float*>(wsb);
-    wsb += align256((size_t)heads * T * S * kHeadDim * 4);
-    int* nzs = reinterpret_cast<int*>(wsb);
-    k_block_unit_sums<<<dim3((unsigned)(T * S), (unsigned)heads), kSimThreads, 0, s>>>(
-        reinterpret_cast<const __nv_bfloat16*>(X), L, block, (int)S, us, nzs);
-    k_fold_slices<<<dim3((unsigned)T, (unsigned)heads), kHeadDim, 0, s>>>(us, nzs, (int)S, u, nz);
+  wsb += pl.nz_bytes;
+  float* us = reinterpret_cast<float*>(wsb);
+  wsb += pl.us_bytes;
+  int* nzs = reinterpret_cast<int*>(wsb);
+  // Long blocks of which there are too few to fill the GPU: a cluster of CTAs per block, as long as
+  // every warp keeps a full step of 32 rows.
+  int S = 1;
+  while (S < kSumMaxCluster && (long long)heads * pl.slices * S < device_sm_count() &&
+         (long long)2 * S * kSumWarps * kSumRows <= block)
+    S *= 2;
+  const dim3 grid((unsigned)(pl.slices * S), (unsigned)heads);
+  const __nv_bfloat16* x = reinterpret_cast<const __nv_bfloat16*>(X);
+  cudaError_t e;
+  switch (sum_mode(block)) {
+    case kRowsOne:
+      e = launch_pdl(k_block_sums<kRowsOne, 2>, grid, dim3(kSumThreads), 0, s, 1, x, L, block, pl.T, parts,
+                     nz, us, nzs);
+      break;
+    case kRowsFew:
+      e = launch_pdl(k_block_sums<kRowsFew, 3>, grid, dim3(kSumThreads), 0, s, 1, x, L, block, pl.T, parts,
+                     nz, us, nzs);
+      break;
+    default:
+      e = launch_pdl(k_block_sums<kRowsMany, 3>, grid, dim3(kSumThreads), 0, s, S, x, L, block, pl.T, parts,
+                     nz, us, nzs);
+      break;
   }
-  const unsigned g = (unsigned)((T + 15) / 16);
-  k_block_map<<<dim3(g, g, (unsigned)heads), dim3(16, 16), 0, s>>>(u, nz, L, block, (int)T, cells);
-  if (mean_opt) k_head_mean<<<(unsigned)heads, 1024, 0, s>>>(u, nz, L, (int)T, mean_opt);
-  return cudaGetLastError() == cudaSuccess ? MIXKV_OK : MIXKV_ERR_CUDA;
+  if (e != cudaSuccess) return MIXKV_ERR_CUDA;
+  GramArgs g;
+  g.parts = parts, g.nparts = pl.nparts, g.nz = nz, g.us = us, g.nzs = nzs, g.slices = pl.slices;
+  g.heads = heads, g.L = L, g.block = block, g.T = pl.T, g.cells = cells, g.mean = mean_opt;
+  return launch_gram(g, s) == cudaSuccess ? MIXKV_OK : MIXKV_ERR_CUDA;
 }
 
 }  // extern "C"

@@ -1,17 +1,21 @@
-// Redundancy analysis at fine resolution (block = 1, 2, 4, 8 or 16 rows per cell): the dense
-// cosine-similarity matrix R = X^ X^T of Eq. 3 on the tensor cores.  With few rows per cell the
-// Gram of block sums IS the L x L contraction, so it runs as tcgen05 tiles:
+// Second kernel of the redundancy analysis: the Gram matrix of the block sums on the tensor cores,
+// cell (I, J) = u_I . u_J / pairs (similarity.cu leaves the sums u as bf16 parts).
 //
-//   k_unit_rows   one streaming pass over X: every row is normalised in fp32 and written as two
-//                 bf16 arrays, hi = bf16(x^) and lo = bf16(x^ - hi) (together 16 mantissa bits,
-//                 which keeps a cell within 1e-6 of the fp32 dot product); per 256-row slice the
-//                 sum of the unit rows and the number of non-zero rows (for the head mean).
-//   k_gram_tc     persistent CTAs, one row of 128 x 128 tiles at a time (rows I and nT-1-I
-//                 paired so that every work item has the same length); only tiles J >= I are
-//                 computed, the mirrored cells are written from the same registers.  Per tile
-//                 24 tcgen05.mma steps accumulate hi.hi + hi.lo + lo.hi in tensor memory; the
-//                 epilogue reduces the block x block sub-squares (columns in the thread, rows by
-//                 warp shuffles), drops the i == j pairs and divides by the pair count.
+// The sums come as P bf16 parts, so a product is the sum of the part products that carry fp32's bits:
+//   P = 2 (one row per block: x = hi + lo, 16 mantissa bits)      hi.hi + lo.hi + hi.lo
+//   P = 3 (hi + mid + lo, 24 bits)    hi.hi + mid.hi + lo.hi + hi.mid + mid.mid + hi.lo
+// Persistent CTAs walk a contiguous run of tiles (head, I, J): 128 blocks I on M, NT blocks J on N,
+// only tiles that touch or lie right of the diagonal.  The parts of I stay in shared memory while
+// J runs (P x 32 KB), the parts of J go through a three-stage ring one part at a time, and two
+// accumulator stages let the epilogue of a tile overlap the MMA of the next.
+//
+// What bounds it: the output, T x T x 4 bytes per head, once T is large.  Every store is a full
+// 128-byte line per warp: the cells of the mirrored tile straight from the registers (a thread holds
+// one I and 32 J, so for one J the lanes are 32 consecutive I), the tile itself after a 32 x 32
+// transposition through shared memory (swizzled, no bank conflicts).
+//
+// NT = 128 where there are tiles enough for every SM, NT = 32 below that: a small map is one chain
+// of load, MMA and store per CTA, and a quarter of the columns shortens all three.
 #include <cuda.h>
 
 #include "tc_common.cuh"
@@ -19,183 +23,164 @@
 namespace mixkv {
 namespace {
 
-constexpr int kURows = 256;      // rows per slice of k_unit_rows
-constexpr int kUThreads = 256;
-
-// grid (ceil(L / 256), H).  A warp takes four rows at a time; lane l holds elements 4l .. 4l+3.
-__global__ void __launch_bounds__(kUThreads)
-k_unit_rows(const __nv_bfloat16* __restrict__ X, const int L, __nv_bfloat16* __restrict__ hi,
-            __nv_bfloat16* __restrict__ lo, float* __restrict__ u, int* __restrict__ nz) {
-  __shared__ float part[kUThreads / 32][kHeadDim];
-  __shared__ int cnt[kUThreads / 32];
-  const int sl = blockIdx.x, h = blockIdx.y, S = gridDim.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r0 = sl * kURows, r1 = min(L, r0 + kURows);
-  const size_t hbase = (size_t)h * L * kHeadDim;
-  float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  int nonzero = 0;
-  constexpr int kW = kUThreads / 32, kInFlight = 4;
-  for (int r = r0 + warp; r < r1; r += kInFlight * kW) {
-    uint2 v[kInFlight];
-#pragma unroll
-    for (int k = 0; k < kInFlight; ++k) {
-      const int rk = r + k * kW;
-      v[k] = rk < r1 ? *reinterpret_cast<const uint2*>(X + hbase + (size_t)rk * kHeadDim + 4 * lane)
-                     : make_uint2(0u, 0u);
-    }
-    float f[kInFlight][4], n2[kInFlight];
-#pragma unroll
-    for (int k = 0; k < kInFlight; ++k) {
-      const float2 p = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v[k].x));
-      const float2 q = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v[k].y));
-      f[k][0] = p.x, f[k][1] = p.y, f[k][2] = q.x, f[k][3] = q.y;
-      n2[k] = (p.x * p.x + p.y * p.y) + (q.x * q.x + q.y * q.y);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-      for (int k = 0; k < kInFlight; ++k) n2[k] += __shfl_xor_sync(0xffffffffu, n2[k], o);
-#pragma unroll
-    for (int k = 0; k < kInFlight; ++k) {
-      const int rk = r + k * kW;
-      const float inv = n2[k] > 0.f ? rsqrtf(n2[k]) : 0.f;
-      nonzero += n2[k] > 0.f;
-      __nv_bfloat16 hh[4], ll[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float x = f[k][e] * inv;
-        acc[e] += x;
-        hh[e] = __float2bfloat16_rn(x);
-        ll[e] = __float2bfloat16_rn(x - __bfloat162float(hh[e]));
-      }
-      if (rk < r1) {
-        *reinterpret_cast<uint2*>(hi + hbase + (size_t)rk * kHeadDim + 4 * lane) =
-            *reinterpret_cast<const uint2*>(hh);
-        *reinterpret_cast<uint2*>(lo + hbase + (size_t)rk * kHeadDim + 4 * lane) =
-            *reinterpret_cast<const uint2*>(ll);
-      }
-    }
-  }
-#pragma unroll
-  for (int e = 0; e < 4; ++e) part[warp][4 * lane + e] = acc[e];
-  if (lane == 0) cnt[warp] = nonzero;
-  __syncthreads();
-  if (threadIdx.x < kHeadDim) {
-    float s = 0.f;
-#pragma unroll
-    for (int w = 0; w < kUThreads / 32; ++w) s += part[w][threadIdx.x];
-    u[((size_t)h * S + sl) * kHeadDim + threadIdx.x] = s;
-  }
-  if (threadIdx.x == 0) {
-    int c = 0;
-    for (int w = 0; w < kUThreads / 32; ++w) c += cnt[w];
-    nz[h * S + sl] = c;
-  }
-}
-
-// ------------------------------------------------------------------------------- Gram tiles
-constexpr int kGThreads = 12 * 32;   // TMA, MMA, 2 idle, 8 epilogue warps
+constexpr int kGThreads = 12 * 32;   // TMA, MMA, 2 head-mean, 8 epilogue warps
 constexpr int kGEpiWarp0 = 4, kGEpiWarps = 8;
-constexpr int kOperandBytes = 4 * 16384;   // hi and lo of 128 rows: [part][64-column half][128 x 128 B]
+constexpr int kPartBytes = 128 * 256;   // one part of 128 blocks: two 64-column halves of 16 KB
+constexpr int kGStages = 3;
 
 struct GBars {
   uint64_t afull, afree;
-  uint64_t bfull[2], bempty[2];
+  uint64_t bfull[kGStages], bempty[kGStages];
   uint64_t tfull[2], tempty[2];
   uint32_t tmem_base;
   int abort;
 };
 
-// The (head, row of tiles) items of one CTA: item m pairs rows m and nT-1-m of a head.
+// Column tiles of tile row I: J starts at the diagonal (I * 128).
+template <int NT>
+__host__ __device__ __forceinline__ int row_tiles(const int T, const int I) {
+  return (T - I * 128 + NT - 1) / NT;
+}
+
+// The tiles [lo, hi) of one CTA in (head, I, c) order; column tile c covers blocks I * 128 + c * NT ...
+template <int NT>
 struct GramWalk {
-  int nT, half, items, m, which, h, I;
-  __device__ GramWalk(int nT_, int H) : nT(nT_), half((nT_ + 1) / 2), items(H * ((nT_ + 1) / 2)) {
-    m = blockIdx.x;
-    which = 0;
-    set();
-  }
-  __device__ __forceinline__ bool valid() const { return m < items; }
-  __device__ __forceinline__ void set() {
-    if (m < items) {
-      h = m / half;
-      const int mi = m - h * half;
-      I = which == 0 ? mi : nT - 1 - mi;
+  int id, hi, T, nT, h, I, c, nc;
+  bool fresh;   // first tile of this CTA in its (head, I): the parts of I have to be loaded
+  __device__ GramWalk(const int T_, const int per_head, const int lo, const int hi_)
+      : id(lo), hi(hi_), T(T_), nT((T_ + 127) / 128) {
+    fresh = true;
+    h = lo / per_head;
+    c = lo - h * per_head;
+    I = 0;
+    nc = row_tiles<NT>(T, 0);
+    while (c >= nc) {
+      c -= nc;
+      nc = row_tiles<NT>(T, ++I);
     }
   }
+  __device__ __forceinline__ bool valid() const { return id < hi; }
+  // the last tile of this CTA in its (head, I)
+  __device__ __forceinline__ bool row_last() const { return id + 1 == hi || c + 1 == nc; }
   __device__ __forceinline__ void next() {
-    const int mi = m % half;
-    if (which == 0 && nT - 1 - mi != mi) {
-      which = 1;
-    } else {
-      which = 0;
-      m += gridDim.x;
+    ++id;
+    fresh = false;
+    if (++c == nc) {
+      c = 0;
+      fresh = true;
+      if (++I == nT) {
+        I = 0;
+        ++h;
+      }
+      nc = row_tiles<NT>(T, I);
     }
-    set();
   }
 };
 
-__device__ __forceinline__ void load_operand(unsigned char* dst, const CUtensorMap* tmHi,
-                                             const CUtensorMap* tmLo, int row0, int h, uint64_t* bar) {
-  tma_load_3d(dst, tmHi, 0, row0, h, bar);
-  tma_load_3d(dst + 16384, tmHi, 64, row0, h, bar);
-  tma_load_3d(dst + 32768, tmLo, 0, row0, h, bar);
-  tma_load_3d(dst + 49152, tmLo, 64, row0, h, bar);
+// Mean over all ordered pairs i != j of a head (Eq. 4), by two warps that have nothing else to do:
+// thread t holds dimensions 2t, 2t + 1.
+__device__ void head_mean(const float* __restrict__ us, const int* __restrict__ nzs, const int slices,
+                          const int h, const int L, const int t, float* red, float* __restrict__ mean) {
+  float2 s = make_float2(0.f, 0.f);
+  int z = 0;
+  const float2* row = reinterpret_cast<const float2*>(us + (size_t)h * slices * kHeadDim) + t;
+  constexpr int kDepth = 16;
+  for (int k0 = 0; k0 < slices; k0 += kDepth) {
+    float2 v[kDepth];
+#pragma unroll
+    for (int k = 0; k < kDepth; ++k)
+      v[k] = k0 + k < slices ? __ldcg(row + (size_t)(k0 + k) * (kHeadDim / 2)) : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < kDepth; ++k) s.x += v[k].x, s.y += v[k].y;
+  }
+  for (int k = t; k < slices; k += 64) z += __ldcg(nzs + (size_t)h * slices + k);
+  const float n2 = warp_sum(s.x * s.x + s.y * s.y);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+  if ((t & 31) == 0) {
+    red[t >> 5] = n2;
+    reinterpret_cast<int*>(red)[2 + (t >> 5)] = z;
+  }
+  named_bar_sync(1, 64);
+  if (t == 0) {
+    const double nn = (double)red[0] + (double)red[1], Ld = (double)L;
+    const int nz = reinterpret_cast<int*>(red)[2] + reinterpret_cast<int*>(red)[3];
+    mean[h] = L > 1 ? (float)((nn - (double)nz) / (Ld * (Ld - 1.0))) : 0.f;
+  }
+  named_bar_sync(1, 64);
 }
 
-template <int B>
+template <int P, int NT>
 __global__ void __launch_bounds__(kGThreads, 1)
-k_gram_tc(const __grid_constant__ CUtensorMap tmHi, const __grid_constant__ CUtensorMap tmLo,
-          const int L, const int H, const int T, float* __restrict__ cells) {
+k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+       const int* __restrict__ nz, const float* __restrict__ us, const int* __restrict__ nzs,
+       const int slices, const int H, const int L, const int block, const int T, const int per_head,
+       float* __restrict__ cells, float* __restrict__ mean) {
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
-  unsigned char* sA = base;                      // 64 KB
-  unsigned char* sB = sA + kOperandBytes;        // 2 x 64 KB
-  GBars* bars = reinterpret_cast<GBars*>(sB + 2 * kOperandBytes);
+  constexpr int kBPart = NT * 256, kBHalf = NT * 128;   // one part of the NT blocks on N
+  unsigned char* sA = base;                             // P parts
+  unsigned char* sB = sA + P * kPartBytes;              // kGStages x one part
+  float* sT = reinterpret_cast<float*>(sB + kGStages * kBPart);   // [8 warps][32 x 32]
+  GBars* bars = reinterpret_cast<GBars*>(sT + kGEpiWarps * 1024);
+  __shared__ float red[4];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int nT = (L + kTile - 1) / kTile;
+  const long long total = (long long)H * per_head;
+  const int lo = (int)(total * blockIdx.x / gridDim.x), hi = (int)(total * (blockIdx.x + 1) / gridDim.x);
   volatile int* abort = &bars->abort;
 
+  pdl_launch_dependents();
   if (tid == 0) {
     mbar_init(&bars->afull, 1);
     mbar_init(&bars->afree, 1);
-    for (int s = 0; s < 2; ++s) {
+    for (int s = 0; s < kGStages; ++s) {
       mbar_init(&bars->bfull[s], 1);
       mbar_init(&bars->bempty[s], 1);
+    }
+    for (int s = 0; s < 2; ++s) {
       mbar_init(&bars->tfull[s], 1);
-      mbar_init(&bars->tempty[s], kGEpiWarps);
+      mbar_init(&bars->tempty[s], NT == 128 ? kGEpiWarps : 4);
     }
     bars->abort = 0;
     mbar_init_fence();
   }
   if (warp == 1) tmem_alloc(&bars->tmem_base, 256);
   if (warp == 0 && lane == 0) {
-    tma_prefetch_desc(&tmHi);
-    tma_prefetch_desc(&tmLo);
+    tma_prefetch_desc(&tmA);
+    tma_prefetch_desc(&tmB);
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
+  pdl_wait();
 
   if (warp == 0) {
     // -------------------------------------------------------------------- TMA producer
     if (lane == 0) {
       int it = 0, rown = 0;
       bool ok = true;
-      for (GramWalk w(nT, H); w.valid() && ok; w.next()) {
-        if (rown > 0 && !mbar_wait(&bars->afree, (rown - 1) & 1, abort)) break;
-        mbar_expect_tx(&bars->afull, kOperandBytes);
-        load_operand(sA, &tmHi, &tmLo, w.I * kTile, w.h, &bars->afull);
-        ++rown;
-        for (int J = w.I; J < nT; ++J) {
-          const int s = it & 1, ph = (it >> 1) & 1;
+      for (GramWalk<NT> w(T, per_head, lo, hi); w.valid() && ok; w.next()) {
+        if (w.fresh) {
+          if (rown > 0 && !mbar_wait(&bars->afree, (rown - 1) & 1, abort)) break;
+          mbar_expect_tx(&bars->afull, P * kPartBytes);
+          for (int p = 0; p < P; ++p) {
+            tma_load_3d(sA + p * kPartBytes, &tmA, 0, w.I * 128, p * H + w.h, &bars->afull);
+            tma_load_3d(sA + p * kPartBytes + 16384, &tmA, 64, w.I * 128, p * H + w.h, &bars->afull);
+          }
+          ++rown;
+        }
+        for (int p = 0; p < P; ++p) {
+          const int s = it % kGStages, ph = (it / kGStages) & 1;
           if (!mbar_wait(&bars->bempty[s], ph ^ 1, abort)) {
             ok = false;
             break;
           }
-          mbar_expect_tx(&bars->bfull[s], kOperandBytes);
-          load_operand(sB + s * kOperandBytes, &tmHi, &tmLo, J * kTile, w.h, &bars->bfull[s]);
+          mbar_expect_tx(&bars->bfull[s], kBPart);
+          unsigned char* dst = sB + s * kBPart;
+          tma_load_3d(dst, &tmB, 0, w.I * 128 + w.c * NT, p * H + w.h, &bars->bfull[s]);
+          tma_load_3d(dst + kBHalf, &tmB, 64, w.I * 128 + w.c * NT, p * H + w.h, &bars->bfull[s]);
           ++it;
         }
       }
@@ -208,128 +193,131 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmHi, const __grid_constant__ CUte
   } else if (warp == 1) {
     // -------------------------------------------------------------------- MMA issuer
     if (lane == 0) {
-      constexpr uint32_t idesc = umma_idesc_bf16(128, kTile);
+      constexpr uint32_t idesc = umma_idesc_bf16(128, NT);
       const uint32_t a0 = umma_desc_lo(smem_u32(sA)), b0 = umma_desc_lo(smem_u32(sB));
-      int it = 0, rown = 0;
+      int it = 0, rown = 0, tile = 0;
       bool ok = true;
-      for (GramWalk w(nT, H); w.valid() && ok; w.next()) {
-        if (!mbar_wait(&bars->afull, rown & 1, abort)) break;
-        ++rown;
-        for (int J = w.I; J < nT; ++J) {
-          const int s = it & 1, ph = (it >> 1) & 1;
-          if (!mbar_wait(&bars->bfull[s], ph, abort) || !mbar_wait(&bars->tempty[s], ph ^ 1, abort)) {
+      for (GramWalk<NT> w(T, per_head, lo, hi); w.valid() && ok; w.next()) {
+        if (w.fresh) {
+          if (!mbar_wait(&bars->afull, rown & 1, abort)) break;
+          ++rown;
+        }
+        const int ts = tile & 1, tph = (tile >> 1) & 1;
+        if (!mbar_wait(&bars->tempty[ts], tph ^ 1, abort)) break;
+        // part p of J meets the parts of I whose product with it carries weight
+#pragma unroll
+        for (int p = 0; p < P; ++p) {
+          const int s = it % kGStages, ph = (it / kGStages) & 1;
+          if (!mbar_wait(&bars->bfull[s], ph, abort)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t bs = b0 + (uint32_t)s * (kOperandBytes >> 4);
-          // x^.y^ = hi.hi + hi.lo + lo.hi (lo.lo is below 2^-17): parts (A, B) = (0,0), (0,1), (1,0)
+          const uint32_t bs = b0 + (uint32_t)s * (kBPart >> 4);
 #pragma unroll
-          for (int seg = 0; seg < 3; ++seg) {
-            const uint32_t pa = (seg == 2 ? 32768u : 0u) >> 4, pb = (seg == 1 ? 32768u : 0u) >> 4;
+          for (int pa = 0; pa < P - p; ++pa) {
 #pragma unroll
             for (int ks = 0; ks < 8; ++ks) {
-              const uint32_t o = (uint32_t)((ks >> 2) * (16384 >> 4) + (ks & 3) * 2);
-              if (seg == 0 && ks == 0)
-                umma_bf16_lo<0>(tmem + s * 128, a0 + pa + o, bs + pb + o, idesc);
+              const uint32_t oa = (uint32_t)(pa * (kPartBytes >> 4) + (ks >> 2) * (16384 >> 4) + (ks & 3) * 2);
+              const uint32_t ob = (uint32_t)((ks >> 2) * (kBHalf >> 4) + (ks & 3) * 2);
+              if (p == 0 && pa == 0 && ks == 0)
+                umma_bf16_lo<0>(tmem + ts * 128, a0 + oa, bs + ob, idesc);
               else
-                umma_bf16_lo<1>(tmem + s * 128, a0 + pa + o, bs + pb + o, idesc);
+                umma_bf16_lo<1>(tmem + ts * 128, a0 + oa, bs + ob, idesc);
             }
           }
           umma_commit(&bars->bempty[s]);
-          umma_commit(&bars->tfull[s]);
           ++it;
         }
-        umma_commit(&bars->afree);
+        umma_commit(&bars->tfull[ts]);
+        if (w.row_last()) umma_commit(&bars->afree);
+        ++tile;
       }
     }
-  } else if (warp >= kGEpiWarp0) {
+  } else if (warp < kGEpiWarp0) {
+    // -------------------------------------------------------------------- head means
+    if (mean)
+      for (int h = blockIdx.x; h < H; h += gridDim.x)
+        head_mean(us, nzs, slices, h, L, tid - 64, red, mean);
+  } else if (NT == 128 || warp < kGEpiWarp0 + 4) {
     // -------------------------------------------------------------------- epilogue
-    // warp % 4 = TMEM lane quarter (32 rows of the tile), (warp - 4) / 4 = 64-column half.
+    // warp % 4 = TMEM lane quarter (32 blocks I of the tile), (warp - 4) / 4 = 64-column half.
     const int quarter = warp & 3, ch = (warp - kGEpiWarp0) >> 2;
-    const int r = quarter * 32 + lane;
-    constexpr int G = 32 / B;   // cells per 32-column chunk and row group
-    int it = 0;
-    bool ok = true;
-    for (GramWalk w(nT, H); w.valid() && ok; w.next()) {
-      const int i = w.I * kTile + r;            // row of the matrix
-      const int ci = i / B;                     // its cell row
-      const int nI = min(B, L - ci * B);
+    constexpr int kChunks = NT == 128 ? 2 : 1;
+    float* st = sT + (warp - kGEpiWarp0) * 1024;
+    const float inv_b = 1.0f / (float)block, last_n = (float)(L - (T - 1) * block);
+    int tile = 0;
+    for (GramWalk<NT> w(T, per_head, lo, hi); w.valid(); w.next()) {
+      const int i0 = w.I * 128 + quarter * 32, i = i0 + lane;   // this thread's block I
+      const bool last_i = i == T - 1;
+      const float inv_i = last_i ? 1.0f / last_n : inv_b;
+      const bool on_diag = w.c * NT < 128;    // inside the diagonal 128 x 128 tile: no mirrored store
       float* out = cells + (size_t)w.h * T * T;
-      for (int J = w.I; J < nT; ++J) {
-        const int s = it & 1, ph = (it >> 1) & 1;
-        if (!mbar_wait(&bars->tfull[s], ph, abort)) {
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + s * 128 + ch * 64;
+      const int ts = tile & 1, tph = (tile >> 1) & 1;
+      if (!mbar_wait(&bars->tfull[ts], tph, abort)) break;
+      tc_fence_after();
+      const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + ts * 128 + ch * 64;
 #pragma unroll 1
-        for (int k = 0; k < 2; ++k) {
-          uint32_t v[32];
-          tmem_ld32(taddr + k * 32, v);
-          tmem_ld_wait();
-          tmem_ld_fence(v);
-          const int c0 = ch * 64 + k * 32;      // first column of the chunk inside the tile
-          if (J == w.I) {                       // the pairs i == j are left out
+      for (int k = 0; k < kChunks; ++k) {
+        const int j0 = w.I * 128 + w.c * NT + ch * 64 + k * 32;   // first block J of the chunk
+        uint32_t v[32];
+        tmem_ld32(taddr + k * 32, v);
+        tmem_ld_wait();
+        tmem_ld_fence(v);
+        if (k + 1 == kChunks) {   // the accumulator stage is read: the MMA may fill it again
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bars->tempty[ts]);
+        }
+        if (j0 >= T || i0 >= T) continue;
+        const float sc = inv_i * inv_b;
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (c0 + j == r) v[j] = 0u;
+        for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * sc);
+        if (j0 + 31 >= T - 1 || j0 == i0) {   // the last block, or cells of the diagonal
+          const bool diag = j0 == i0;
+          const float n = last_i ? last_n : (float)block, pairs = n * (n - 1.0f);
+          // the pairs of a row with itself are left out: cosine 1 each
+          const float own = pairs > 0.f ? 1.0f / pairs : 0.f;
+          const float z = diag && i < T ? (float)nz[(size_t)w.h * T + i] : 0.f;
+          const float fix = (float)block / last_n;   // columns of the last block
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            float x = __uint_as_float(v[j]);
+            if (j0 + j == T - 1) x *= fix;
+            if (diag && j == lane) x = (x * n * n - z) * own;
+            v[j] = __float_as_uint(x);
           }
-          float sgrp[G];
+        }
+        if (!on_diag) {   // mirrored tile: row J, 32 consecutive I per store
+          float* p = out + (size_t)j0 * T + i;
+          if (i < T) {
+            if (j0 + 32 <= T) {
 #pragma unroll
-          for (int g = 0; g < G; ++g) {
-            float t = __uint_as_float(v[g * B]);
+              for (int j = 0; j < 32; ++j) p[(size_t)j * T] = __uint_as_float(v[j]);
+            } else {
 #pragma unroll
-            for (int e = 1; e < B; ++e) t += __uint_as_float(v[g * B + e]);
-            sgrp[g] = t;
-          }
-#pragma unroll
-          for (int o = 1; o < B; o <<= 1)
-#pragma unroll
-            for (int g = 0; g < G; ++g) sgrp[g] += __shfl_xor_sync(0xffffffffu, sgrp[g], o);
-          if (B == 1 && (T & 3) == 0 && ci < T) {
-            // one row per thread: 16-byte stores along the row, the mirrored cells lane by lane
-            // (consecutive lanes, consecutive addresses)
-            const int cj0 = J * kTile + c0;
-            if (cj0 < T) {
-#pragma unroll
-              for (int g = 0; g < 32; g += 4) {
-                if (cj0 + g < T) {
-                  float4 q4;
-                  q4.x = ci != cj0 + g ? sgrp[g] : 0.f;
-                  q4.y = ci != cj0 + g + 1 ? sgrp[g + 1] : 0.f;
-                  q4.z = ci != cj0 + g + 2 ? sgrp[g + 2] : 0.f;
-                  q4.w = ci != cj0 + g + 3 ? sgrp[g + 3] : 0.f;
-                  *reinterpret_cast<float4*>(out + (size_t)ci * T + cj0 + g) = q4;
-                }
-              }
-              if (J != w.I) {
-#pragma unroll
-                for (int g = 0; g < 32; ++g)
-                  if (cj0 + g < T) out[(size_t)(cj0 + g) * T + ci] = sgrp[g];
-              }
-            }
-          } else if ((lane & (B - 1)) == 0 && ci < T) {
-            const int cj0 = (J * kTile + c0) / B;
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-              const int cj = cj0 + g;
-              if (cj < T) {
-                const int nJ = min(B, L - cj * B);
-                const float pairs = ci != cj ? (float)(nI * nJ) : (float)(nI * (nI - 1));
-                const float val = pairs > 0.f ? sgrp[g] / pairs : 0.f;
-                out[(size_t)ci * T + cj] = val;
-                if (J != w.I) out[(size_t)cj * T + ci] = val;   // the mirrored tile
-              }
+              for (int j = 0; j < 32; ++j)
+                if (j0 + j < T) p[(size_t)j * T] = __uint_as_float(v[j]);
             }
           }
         }
-        tc_fence_before();
+        // the tile itself: rows I, 32 consecutive J per store
         __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->tempty[s]);
-        ++it;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) st[lane * 32 + (j ^ lane)] = __uint_as_float(v[j]);
+        __syncwarp();
+        if (j0 + lane < T) {
+          float* p = out + (size_t)i0 * T + j0 + lane;
+          if (i0 + 32 <= T) {
+#pragma unroll
+            for (int r = 0; r < 32; ++r) p[(size_t)r * T] = st[r * 32 + (lane ^ r)];
+          } else {
+#pragma unroll 1
+            for (int r = 0; r < T - i0; ++r) p[(size_t)r * T] = st[r * 32 + (lane ^ r)];
+          }
+        }
       }
+      ++tile;
     }
   }
   tc_fence_before();
@@ -337,79 +325,51 @@ k_gram_tc(const __grid_constant__ CUtensorMap tmHi, const __grid_constant__ CUte
   if (warp == 1) tmem_dealloc(tmem, 256);
 }
 
-size_t align256(size_t x) { return (x + 255) / 256 * 256; }
-
-template <int B>
-cudaError_t launch_gram(const CUtensorMap& tmHi, const CUtensorMap& tmLo, int L, int H, int T,
-                        float* cells, cudaStream_t s) {
+template <int P, int NT>
+cudaError_t launch_gram_t(const GramArgs& g, const long long per_head, cudaStream_t s) {
   static bool done[64] = {false};
-  const size_t smem = 1024 + 3 * (size_t)kOperandBytes + sizeof(GBars);
+  const size_t smem = 1024 + (size_t)P * kPartBytes + (size_t)kGStages * NT * 256 +
+                      (size_t)kGEpiWarps * 4096 + sizeof(GBars);
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64 || !done[dev]) {
-    e = cudaFuncSetAttribute(k_gram_tc<B>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_gram<P, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) done[dev] = true;
   }
-  const int nT = (L + kTile - 1) / kTile;
-  const int items = H * ((nT + 1) / 2);
-  const int grid = items < device_sm_count() ? items : device_sm_count();
-  k_gram_tc<B><<<grid, kGThreads, smem, s>>>(tmHi, tmLo, L, H, T, cells);
-  return cudaGetLastError();
+  const long long total = per_head * g.heads;
+  if (total > 0x7fffffffLL) return cudaErrorInvalidValue;
+  CUtensorMap tmA, tmB;
+  const unsigned long long dims[3] = {(unsigned long long)kHeadDim, (unsigned long long)g.T,
+                                      (unsigned long long)P * g.heads};
+  const unsigned long long strides[2] = {(unsigned long long)kHeadDim * 2,
+                                         (unsigned long long)g.T * kHeadDim * 2};
+  const unsigned boxA[3] = {64, 128, 1}, boxB[3] = {64, (unsigned)NT, 1};
+  if (!encode_bf16_map(&tmA, g.parts, 3, dims, strides, boxA) ||
+      !encode_bf16_map(&tmB, g.parts, 3, dims, strides, boxB))
+    return cudaErrorInvalidValue;
+  const int grid = (int)(total < device_sm_count() ? total : device_sm_count());
+  return launch_pdl(k_gram<P, NT>, dim3((unsigned)grid), dim3(kGThreads), smem, s, 1, tmA, tmB, g.nz, g.us,
+                    g.nzs, g.slices, g.heads, g.L, g.block, g.T, (int)per_head, g.cells, g.mean);
+}
+
+template <int NT>
+long long tiles_per_head(const int T) {
+  long long n = 0;
+  for (int I = 0; I < (T + 127) / 128; ++I) n += row_tiles<NT>(T, I);
+  return n;
 }
 
 }  // namespace
 
-bool similarity_dense_block(int block) {
-  return block == 1 || block == 2 || block == 4 || block == 8 || block == 16;
-}
-
-size_t similarity_dense_workspace(int heads, int L) {
-  const size_t S = ((size_t)L + kURows - 1) / kURows;
-  return 2 * align256((size_t)heads * L * kHeadDim * 2) + align256((size_t)heads * S * kHeadDim * 4) +
-         align256((size_t)heads * S * 4);
-}
-
-// Dense route of mixkv_similarity_map.  u_out / nz_out / slices_out: the per-slice unit-row sums
-// for the head mean.
-cudaError_t launch_similarity_dense(const void* X, int heads, int L, int block, void* workspace,
-                                    float* cells, float** u_out, int** nz_out, int* slices_out,
-                                    cudaStream_t s) {
-  unsigned char* wsb = reinterpret_cast<unsigned char*>(workspace);
-  __nv_bfloat16* hi = reinterpret_cast<__nv_bfloat16*>(wsb);
-  wsb += align256((size_t)heads * L * kHeadDim * 2);
-  __nv_bfloat16* lo = reinterpret_cast<__nv_bfloat16*>(wsb);
-  wsb += align256((size_t)heads * L * kHeadDim * 2);
-  const int S = (L + kURows - 1) / kURows;
-  float* u = reinterpret_cast<float*>(wsb);
-  wsb += align256((size_t)heads * S * kHeadDim * 4);
-  int* nz = reinterpret_cast<int*>(wsb);
-  k_unit_rows<<<dim3((unsigned)S, (unsigned)heads), kUThreads, 0, s>>>(
-      reinterpret_cast<const __nv_bfloat16*>(X), L, hi, lo, u, nz);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  CUtensorMap tmHi, tmLo;
-  const unsigned long long dims[3] = {(unsigned long long)kHeadDim, (unsigned long long)L,
-                                      (unsigned long long)heads};
-  const unsigned long long strides[2] = {(unsigned long long)kHeadDim * 2,
-                                         (unsigned long long)L * kHeadDim * 2};
-  const unsigned box[3] = {64, (unsigned)kTile, 1};
-  if (!encode_bf16_map(&tmHi, hi, 3, dims, strides, box) ||
-      !encode_bf16_map(&tmLo, lo, 3, dims, strides, box))
-    return cudaErrorInvalidValue;
-  const int T = (L + block - 1) / block;
-  switch (block) {
-    case 1: e = launch_gram<1>(tmHi, tmLo, L, heads, T, cells, s); break;
-    case 2: e = launch_gram<2>(tmHi, tmLo, L, heads, T, cells, s); break;
-    case 4: e = launch_gram<4>(tmHi, tmLo, L, heads, T, cells, s); break;
-    case 8: e = launch_gram<8>(tmHi, tmLo, L, heads, T, cells, s); break;
-    default: e = launch_gram<16>(tmHi, tmLo, L, heads, T, cells, s); break;
-  }
-  *u_out = u;
-  *nz_out = nz;
-  *slices_out = S;
-  return e;
+cudaError_t launch_gram(const GramArgs& g, cudaStream_t s) {
+  const long long wide = tiles_per_head<128>(g.T);
+  const bool narrow = wide * g.heads < device_sm_count();
+  const long long per_head = narrow ? tiles_per_head<32>(g.T) : wide;
+  if (g.nparts == 2)
+    return narrow ? launch_gram_t<2, 32>(g, per_head, s) : launch_gram_t<2, 128>(g, per_head, s);
+  return narrow ? launch_gram_t<3, 32>(g, per_head, s) : launch_gram_t<3, 128>(g, per_head, s);
 }
 
 }  // namespace mixkv

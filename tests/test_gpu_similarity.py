@@ -48,6 +48,19 @@ def test_dense_route_small_maps(H, L, block):
         assert (np.diagonal(c, axis1=1, axis2=2) == 0).all()
 
 
+@pytest.mark.parametrize("H,L,block", [
+    (2, 331, 3), (1, 997, 31), (2, 1000, 32), (1, 1101, 33), (2, 2049, 255), (1, 1030, 257),   # steps of 32 rows
+    (1, 4500, 513), (1, 5000, 4096), (1, 300, 512),                 # a cluster of CTAs per block, one block
+    (1, 127, 1), (1, 129, 1), (3, 770, 6), (1, 4112, 16), (2, 2054, 2), (13, 1290, 10)])   # map edges, many heads
+def test_block_and_tile_edges(H, L, block):
+    rng = np.random.default_rng(7 * block + L)
+    X = rng.standard_normal((H, L, 128)) + 0.9 * rng.standard_normal((H, 1, 128))
+    X[0, L // 2] = 0.0
+    X[0, L - 1] = 0.0
+    cells, _ = run(synth.f32_to_bf16_bits(X.astype(np.float32)), block)
+    assert torch.allclose(cells, cells.transpose(1, 2), rtol=0, atol=1e-6)
+
+
 @pytest.mark.parametrize("L,block", [(8192, 1), (32768, 16)])
 def test_dense_route_full_size_sampled(L, block):
     # The dense map of the keys of two heads at full size.  The pairwise oracle needs the L x L
