@@ -1,13 +1,18 @@
-"""ctypes binding of the MixKV C ABI (``include/mixkv.h``).
+"""Python binding of the MixKV C ABI (``include/mixkv.h``).
 
 Argument marshalling only: every function hands device pointers of torch tensors to the
 library entry point of the same name and returns the tensors it filled.  No arithmetic of
 the method happens here, and nothing falls back to PyTorch ops or the CPU: if
-``libmixkv.so`` is missing, :func:`load_library` raises.
+``libmixkv.so`` or ``_mixkv_host.so`` is missing, :func:`load_library` raises.
+
+The calls that enqueue work go through the native module ``_mixkv_host``
+(``csrc/host/host_binding.cpp``), the rest through ctypes.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass
 from typing import Dict, Optional, Sequence
@@ -16,6 +21,7 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libmixkv.so")
+HOST_PATH = os.path.join(_PKG, "_mixkv_host.so")
 
 EXPORTS = ("mixkv_default_params", "mixkv_workspace_size", "mixkv_scores", "mixkv_select",
            "mixkv_compress_layer", "mixkv_compress_layer_traced", "mixkv_launches_per_layer",
@@ -66,6 +72,7 @@ class Params:
 
 
 _lib: Optional[C.CDLL] = None
+_host_module = None
 
 
 def load_library() -> C.CDLL:
@@ -125,24 +132,32 @@ def status_string(status: int) -> str:
     return load_library().mixkv_status_string(int(status)).decode()
 
 
-def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
-    if t is None:
-        return None
-    assert t.is_contiguous(), "tensors handed to the library must be contiguous"
-    return t.data_ptr()
-
-
-def _cu_array(cu: Optional[Sequence[int]]):
-    if cu is None:
-        return None, 1
-    arr = (C.c_int32 * len(cu))(*[int(x) for x in cu])
-    return arr, len(cu) - 1
+def _host():
+    """The native half of the binding (loads the library first)."""
+    global _host_module
+    if _host_module is None:
+        load_library()
+        if not os.path.exists(HOST_PATH):
+            raise FileNotFoundError(
+                f"{HOST_PATH} not found: build it with `python -m paper_2510_20707_b200.build`")
+        loader = importlib.machinery.ExtensionFileLoader("_mixkv_host", HOST_PATH)
+        spec = importlib.util.spec_from_file_location("_mixkv_host", HOST_PATH, loader=loader)
+        module = importlib.util.module_from_spec(spec)
+        loader.exec_module(module)
+        module.setup(LIB_PATH, MixKVError)
+        _host_module = module
+    return _host_module
 
 
 def _stream(stream) -> int:
     if stream is None:
         stream = torch.cuda.current_stream()
     return stream.cuda_stream
+
+
+def _events(trace_events):
+    """Address and length of a ctypes array of cudaEvent_t handles (see mixkv_compress_layer_traced)."""
+    return (0, 0) if trace_events is None else (C.addressof(trace_events), len(trace_events))
 
 
 def workspace_size(params: Params, batch: int, total_tokens: int, max_seq_len: int) -> int:
@@ -194,40 +209,13 @@ def device_check():
     return rc, int(major.value)
 
 
-def _workspace(params, cu, Ltot, device, workspace):
-    batch = 1 if cu is None else len(cu) - 1
-    max_len = Ltot if cu is None else max(int(cu[b + 1]) - int(cu[b]) for b in range(batch))
-    need = workspace_size(params, batch, Ltot, max_len)
-    if workspace is None:
-        workspace = torch.empty(need, dtype=torch.uint8, device=device)
-    return workspace, batch
-
-
 def scores(K: torch.Tensor, V: Optional[torch.Tensor], Q: torch.Tensor, params: Params,
            cu_seqlens: Optional[Sequence[int]] = None, rbar_in: Optional[torch.Tensor] = None,
            workspace: Optional[torch.Tensor] = None, stream=None,
            want_parts: bool = True) -> Dict[str, torch.Tensor]:
     """mixkv_scores: K, V [H, Ltot, 128] bf16, Q [batch, H*G, W, 128] bf16 (device tensors)."""
-    H, Ltot, d = K.shape
-    workspace, batch = _workspace(params, cu_seqlens, Ltot, K.device, workspace)
-    Ptot = Ltot - batch * params.window
-    f32 = dict(dtype=torch.float32, device=K.device)
-    out = {"s_comp": torch.empty((H, Ptot), **f32)}
-    if want_parts:
-        out["s_ex"] = torch.empty((H, Ptot), **f32)
-        out["s_div"] = torch.empty((H, Ptot), **f32)
-        out["rbar"] = torch.empty((batch, H), **f32)
-    status = torch.zeros(1, dtype=torch.int32, device=K.device)
-    cu, _ = _cu_array(cu_seqlens)
-    pc = params.c()
-    rc = load_library().mixkv_scores(
-        _ptr(K), _ptr(V), _ptr(Q), cu, batch, Ltot, C.byref(pc), _ptr(workspace),
-        workspace.numel(), _ptr(out["s_comp"]), _ptr(out.get("s_ex")), _ptr(out.get("s_div")),
-        _ptr(out.get("rbar")), _ptr(rbar_in), _ptr(status), _stream(stream))
-    if rc != 0:
-        raise MixKVError(rc, "mixkv_scores")
-    out["status"] = status
-    return out
+    return (_host_module or _host()).scores(K, V, Q, params, cu_seqlens, rbar_in, workspace, stream,
+                                            want_parts, False)
 
 
 def scores_static(K: torch.Tensor, V: Optional[torch.Tensor], Q: torch.Tensor, params: Params,
@@ -239,46 +227,14 @@ def scores_static(K: torch.Tensor, V: Optional[torch.Tensor], Q: torch.Tensor, p
     and outputs only; the output tensors below are the caller's, as in :func:`scores`.
     Raises MixKVError (status -6) when the problem is too large for the built-in array.
     Calls on one device share that array: do not let two of them overlap on the GPU."""
-    H, Ltot, d = K.shape
-    batch = 1 if cu_seqlens is None else len(cu_seqlens) - 1
-    Ptot = Ltot - batch * params.window
-    f32 = dict(dtype=torch.float32, device=K.device)
-    out = {"s_comp": torch.empty((H, Ptot), **f32), "s_ex": torch.empty((H, Ptot), **f32),
-           "s_div": torch.empty((H, Ptot), **f32), "rbar": torch.empty((batch, H), **f32)}
-    status = torch.zeros(1, dtype=torch.int32, device=K.device)
-    cu, _ = _cu_array(cu_seqlens)
-    pc = params.c()
-    rc = load_library().mixkv_scores_static(
-        _ptr(K), _ptr(V), _ptr(Q), cu, batch, Ltot, C.byref(pc), _ptr(out["s_comp"]),
-        _ptr(out["s_ex"]), _ptr(out["s_div"]), _ptr(out["rbar"]), _ptr(rbar_in), _ptr(status),
-        _stream(stream))
-    if rc != 0:
-        raise MixKVError(rc, "mixkv_scores_static")
-    out["status"] = status
-    return out
+    return (_host_module or _host()).scores(K, V, Q, params, cu_seqlens, rbar_in, None, stream, True,
+                                            True)
 
 
 def select(s: torch.Tensor, params: Params, cu_seqlens: Optional[Sequence[int]] = None,
            workspace: Optional[torch.Tensor] = None, stream=None) -> Dict[str, torch.Tensor]:
     """mixkv_select on scores [H, Ptot] fp32 (device tensor)."""
-    H, Ptot = s.shape
-    batch = 1 if cu_seqlens is None else len(cu_seqlens) - 1
-    Ltot = Ptot + batch * params.window
-    workspace, batch = _workspace(params, cu_seqlens, Ltot, s.device, workspace)
-    i32 = dict(dtype=torch.int32, device=s.device)
-    cap = max(batch * H * (params.budget - params.window), 1)
-    out = {"idx": torch.empty(cap, **i32), "counts": torch.empty(batch * H, **i32),
-           "idx_offsets": torch.empty(batch * H + 1, **i32)}
-    status = torch.zeros(1, **i32)
-    cu, _ = _cu_array(cu_seqlens)
-    pc = params.c()
-    rc = load_library().mixkv_select(_ptr(s), cu, batch, Ltot, C.byref(pc), _ptr(workspace),
-                                     workspace.numel(), _ptr(out["idx"]), _ptr(out["counts"]),
-                                     _ptr(out["idx_offsets"]), _ptr(status), _stream(stream))
-    if rc != 0:
-        raise MixKVError(rc, "mixkv_select")
-    out["status"] = status
-    return out
+    return (_host_module or _host()).select(s, params, cu_seqlens, workspace, stream)
 
 
 def compress_layer(K: torch.Tensor, V: torch.Tensor, Q: torch.Tensor, params: Params,
@@ -290,37 +246,9 @@ def compress_layer(K: torch.Tensor, V: torch.Tensor, Q: torch.Tensor, params: Pa
     """mixkv_compress_layer.  Returns K_out / V_out [batch*H*B, 128] (rows beyond
     out_row_offsets[-1] are untouched), out_row_offsets and, if want_aux, idx / counts /
     idx_offsets / s_comp.  `out` lets a caller reuse output tensors across calls."""
-    H, Ltot, d = K.shape
-    workspace, batch = _workspace(params, cu_seqlens, Ltot, K.device, workspace)
-    Ptot = Ltot - batch * params.window
-    if out is None:
-        i32 = dict(dtype=torch.int32, device=K.device)
-        rows = batch * H * params.budget
-        out = {"K_out": torch.empty((rows, d), dtype=torch.bfloat16, device=K.device),
-               "V_out": torch.empty((rows, d), dtype=torch.bfloat16, device=K.device),
-               "out_row_offsets": torch.empty(batch * H + 1, **i32),
-               "status": torch.zeros(1, **i32)}
-        if want_aux:
-            cap = max(batch * H * (params.budget - params.window), 1)
-            out["idx"] = torch.empty(cap, **i32)
-            out["counts"] = torch.empty(batch * H, **i32)
-            out["idx_offsets"] = torch.empty(batch * H + 1, **i32)
-            out["s_comp"] = torch.empty((H, Ptot), dtype=torch.float32, device=K.device)
-    cu, _ = _cu_array(cu_seqlens)
-    pc = params.c()
-    args = (_ptr(K), _ptr(V), _ptr(Q), cu, batch, Ltot, C.byref(pc), _ptr(workspace),
-            workspace.numel(), _ptr(rbar_in), _ptr(out["K_out"]), _ptr(out["V_out"]),
-            _ptr(out["out_row_offsets"]), _ptr(out.get("idx")), _ptr(out.get("counts")),
-            _ptr(out.get("idx_offsets")), _ptr(out.get("s_comp")), _ptr(out["status"]),
-            _stream(stream))
-    if trace_events is None:
-        rc = load_library().mixkv_compress_layer(*args)
-    else:
-        # trace_events: a ctypes array of cudaEvent_t handles (see mixkv_compress_layer_traced)
-        rc = load_library().mixkv_compress_layer_traced(*args, trace_events, len(trace_events))
-    if rc != 0:
-        raise MixKVError(rc, "mixkv_compress_layer")
-    return out
+    events, n_events = (0, 0) if trace_events is None else _events(trace_events)
+    return (_host_module or _host()).compress_layer(K, V, Q, params, cu_seqlens, rbar_in, workspace, stream,
+                                                    out, want_aux, events, n_events)
 
 
 def compress_layers(K: torch.Tensor, V: torch.Tensor, Q: torch.Tensor, params: Params,
@@ -336,57 +264,9 @@ def compress_layers(K: torch.Tensor, V: torch.Tensor, Q: torch.Tensor, params: P
     want_aux, idx [n_layers, cap] / counts / idx_offsets / s_comp.  With head_budgets (int32
     device tensor [n_layers, batch*H], rows to keep per head, window included) the call goes to
     mixkv_compress_layers_budgeted."""
-    NL, H, Ltot, d = K.shape
-    batch = 1 if cu_seqlens is None else len(cu_seqlens) - 1
-    max_len = Ltot if cu_seqlens is None else max(int(cu_seqlens[b + 1]) - int(cu_seqlens[b])
-                                                 for b in range(batch))
-    if workspace is None:
-        workspace = torch.empty(workspace_size_layers(params, NL, batch, Ltot, max_len),
-                                dtype=torch.uint8, device=K.device)
-    for t in (K, V, Q):
-        assert t[0].is_contiguous(), "each layer must be contiguous"
-    assert V.stride(0) == K.stride(0), "K and V must share their layer stride"
-    Ptot = Ltot - batch * params.window
-    lens = [Ltot] if cu_seqlens is None else [int(cu_seqlens[b + 1]) - int(cu_seqlens[b])
-                                              for b in range(batch)]
-    cap = max(sum(H * min(params.budget - params.window, L - params.window) for L in lens), 1)
-    if out is None:
-        i32 = dict(dtype=torch.int32, device=K.device)
-        rows = batch * H * params.budget
-        out = {"K_out": torch.empty((NL, rows, d), dtype=torch.bfloat16, device=K.device),
-               "V_out": torch.empty((NL, rows, d), dtype=torch.bfloat16, device=K.device),
-               "out_row_offsets": torch.empty((NL, batch * H + 1), **i32),
-               "status": torch.zeros(1, **i32)}
-        if want_aux:
-            out["idx"] = torch.empty((NL, cap), **i32)
-            out["counts"] = torch.empty((NL, batch * H), **i32)
-            out["idx_offsets"] = torch.empty((NL, batch * H + 1), **i32)
-            out["s_comp"] = torch.empty((NL, H, Ptot), dtype=torch.float32, device=K.device)
-    cu, _ = _cu_array(cu_seqlens)
-    pc = params.c()
-    ev, n_ev = (None, 0) if trace_events is None else (trace_events, len(trace_events))
-    if head_budgets is not None:
-        assert head_budgets.dtype == torch.int32 and head_budgets.is_contiguous()
-        assert tuple(head_budgets.shape) == (NL, batch * H) and trace_events is None
-        rc = load_library().mixkv_compress_layers_budgeted(
-            K.data_ptr(), V.data_ptr(), Q.data_ptr(), NL, K.stride(0), Q.stride(0), cu, batch,
-            Ltot, C.byref(pc), _ptr(workspace), workspace.numel(), _ptr(rbar_in),
-            _ptr(head_budgets), _ptr(out["K_out"]), _ptr(out["V_out"]),
-            _ptr(out["out_row_offsets"]), _ptr(out.get("idx")), _ptr(out.get("counts")),
-            _ptr(out.get("idx_offsets")), _ptr(out.get("s_comp")), _ptr(out["status"]),
-            _stream(stream))
-        if rc != 0:
-            raise MixKVError(rc, "mixkv_compress_layers_budgeted")
-        return out
-    rc = load_library().mixkv_compress_layers(
-        K.data_ptr(), V.data_ptr(), Q.data_ptr(), NL, K.stride(0), Q.stride(0), cu, batch, Ltot,
-        C.byref(pc), _ptr(workspace), workspace.numel(), _ptr(rbar_in), _ptr(out["K_out"]),
-        _ptr(out["V_out"]), _ptr(out["out_row_offsets"]), _ptr(out.get("idx")),
-        _ptr(out.get("counts")), _ptr(out.get("idx_offsets")), _ptr(out.get("s_comp")),
-        _ptr(out["status"]), _stream(stream), ev, n_ev)
-    if rc != 0:
-        raise MixKVError(rc, "mixkv_compress_layers")
-    return out
+    events, n_events = (0, 0) if trace_events is None else _events(trace_events)
+    return (_host_module or _host()).compress_layers(K, V, Q, params, cu_seqlens, rbar_in, workspace, stream,
+                                                     out, want_aux, events, n_events, head_budgets)
 
 
 def layer_budget_schedule(n_layers: int, budget: int, window: int, taper_permille: int):
@@ -402,22 +282,7 @@ def layer_budget_schedule(n_layers: int, budget: int, window: int, taper_permill
 def similarity_map(X: torch.Tensor, block: int, want_mean: bool = True, stream=None):
     """mixkv_similarity_map: X [heads, L, 128] bf16 device tensor -> (cells [heads, T, T] fp32,
     mean [heads] fp32 or None): block-mean cosine similarity of the rows of every head."""
-    heads, L, d = X.shape
-    assert X.is_contiguous() and X.dtype == torch.bfloat16
-    need = C.c_size_t(0)
-    rc = load_library().mixkv_similarity_workspace_size(heads, L, block, C.byref(need))
-    if rc != 0:
-        raise MixKVError(rc, "mixkv_similarity_workspace_size")
-    ws = torch.empty(need.value, dtype=torch.uint8, device=X.device)
-    T = (L + block - 1) // block
-    cells = torch.empty((heads, T, T), dtype=torch.float32, device=X.device)
-    mean = torch.empty(heads, dtype=torch.float32, device=X.device) if want_mean else None
-    rc = load_library().mixkv_similarity_map(X.data_ptr(), heads, L, d, block, ws.data_ptr(),
-                                             ws.numel(), cells.data_ptr(), _ptr(mean),
-                                             _stream(stream))
-    if rc != 0:
-        raise MixKVError(rc, "mixkv_similarity_map")
-    return cells, mean
+    return (_host_module or _host()).similarity_map(X, block, want_mean, stream)
 
 
 def decode_attention(K_cache: torch.Tensor, V_cache: torch.Tensor, out_row_offsets: torch.Tensor,
@@ -426,17 +291,8 @@ def decode_attention(K_cache: torch.Tensor, V_cache: torch.Tensor, out_row_offse
     """mixkv_decode_attention: K_cache / V_cache [n_layers, rows_cap, 128] bf16 (the compact
     cache), out_row_offsets [n_layers, batch*H+1] int32, q [n_layers, batch, H*G, 128] bf16 ->
     [n_layers, batch, H*G, 128] fp32."""
-    NL, rows_cap, d = K_cache.shape
-    batch = q.shape[1]
-    assert K_cache.is_contiguous() and V_cache.is_contiguous() and q.is_contiguous()
-    assert out_row_offsets.dtype == torch.int32 and out_row_offsets.is_contiguous()
-    out = torch.empty(q.shape, dtype=torch.float32, device=q.device)
-    rc = load_library().mixkv_decode_attention(
-        K_cache.data_ptr(), V_cache.data_ptr(), out_row_offsets.data_ptr(), rows_cap, q.data_ptr(),
-        NL, batch, kv_heads, gqa_ratio, d, softmax_scale, max_rows, out.data_ptr(), _stream(stream))
-    if rc != 0:
-        raise MixKVError(rc, "mixkv_decode_attention")
-    return out
+    return (_host_module or _host()).decode_attention(K_cache, V_cache, out_row_offsets, q, kv_heads,
+                                                      gqa_ratio, max_rows, softmax_scale, stream)
 
 
 def selftest_bounded_wait(stream=None):

@@ -1,41 +1,83 @@
-"""Builds libmixkv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds, in-tree, libmixkv.so (the C-ABI CUDA library, nvcc for sm_100a) and _mixkv_host.so (the native
+half of the Python binding, the host compiler against torch's headers)."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(os.path.dirname(PKG), "include")
 LIB = os.path.join(PKG, "libmixkv.so")
+HOST_SRC = os.path.join(CSRC, "host", "host_binding.cpp")
+HOST_LIB = os.path.join(PKG, "_mixkv_host.so")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-              "-Xcompiler", "-fPIC", "-shared"]
+              "--threads", "0", "-Xcompiler", "-fPIC", "-shared"]
 
 
 def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def is_stale() -> bool:
-    if not os.path.exists(LIB):
+def _older(target, deps) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    t = os.path.getmtime(target)
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _headers():
+    return (glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) +
+            glob.glob(os.path.join(INCLUDE, "*.h")))
+
+
+def is_stale() -> bool:
+    return _older(LIB, sources() + _headers())
+
+
+def host_is_stale() -> bool:
+    return _older(HOST_LIB, [HOST_SRC, os.path.join(CSRC, "internal_api.h"),
+                             os.path.join(INCLUDE, "mixkv.h")])
+
+
+def _host_command(out: str):
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    inc = [INCLUDE, os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            *[f"-I{d}" for d in inc], "-o", out, HOST_SRC, f"-L{os.path.join(root, 'lib')}",
+            "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-lc10", "-lc10_cuda", "-ldl"]
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every CUDA source of the package into libmixkv.so (no GPU needed)."""
+    """Compile every CUDA source of the package into libmixkv.so and the native binding into
+    _mixkv_host.so (no GPU needed)."""
+    jobs = []
     if force or is_stale():
         nvcc = os.environ.get("NVCC", "nvcc")
         tmp = LIB + f".tmp{os.getpid()}"
         cmd = [nvcc, *NVCC_FLAGS, f"-I{INCLUDE}", f"-I{CSRC}", "-o", tmp, *sources()]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
-        subprocess.check_call(cmd)
-        os.replace(tmp, LIB)
+        jobs.append((cmd, tmp, LIB))
+    if force or host_is_stale():
+        tmp = HOST_LIB + f".tmp{os.getpid()}"
+        jobs.append((_host_command(tmp), tmp, HOST_LIB))
+    running = [(subprocess.Popen(cmd), cmd, tmp, lib) for cmd, tmp, lib in jobs]   # side by side
+    failed = None
+    for proc, cmd, tmp, lib in running:
+        if proc.wait() != 0:
+            failed = subprocess.CalledProcessError(proc.returncode, cmd)
+        else:
+            os.replace(tmp, lib)
+    if failed:
+        raise failed
     return LIB
 
 

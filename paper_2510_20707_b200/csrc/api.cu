@@ -6,6 +6,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "internal_api.h"
 
 namespace mixkv {
 
@@ -166,6 +167,7 @@ int make_ctx(const mixkv_params* p, const int32_t* cu, int batch, int L, void* w
   c->trace_events = nullptr;
   c->n_trace_events = 0;
   c->stage = 0;
+  c->clear_status = false;
   return MIXKV_OK;
 }
 
@@ -285,13 +287,16 @@ int mixkv_workspace_size_layers(const mixkv_params* p, int32_t n_layers, int32_t
   return MIXKV_OK;
 }
 
-int mixkv_scores(const void* K, const void* V, const void* Qwin, const int32_t* cu_seqlens_host,
-                 int32_t batch, int32_t L, const mixkv_params* p, void* workspace,
-                 size_t workspace_bytes, float* s_comp, float* s_ex_opt, float* s_div_opt,
-                 float* rbar_opt, const float* rbar_in_opt, int32_t* status_dev, void* stream) {
+namespace {
+int scores_impl(const void* K, const void* V, const void* Qwin, const int32_t* cu_seqlens_host,
+                int32_t batch, int32_t L, const mixkv_params* p, void* workspace,
+                size_t workspace_bytes, float* s_comp, float* s_ex_opt, float* s_div_opt,
+                float* rbar_opt, const float* rbar_in_opt, int32_t* status_dev, bool clear_status,
+                void* stream) {
   LaunchCtx c;
   int rc = make_ctx(p, cu_seqlens_host, batch, L, workspace, workspace_bytes, stream, &c);
   if (rc != MIXKV_OK) return rc;
+  c.clear_status = clear_status;
   if (!K || !Qwin || !s_comp || (p->use_vnorm == MIXKV_INTRINSIC_VNORM && !V))
     return MIXKV_ERR_INVALID_ARG;
   if (!aligned16(K) || !aligned16(Qwin) || (V && !aligned16(V))) return MIXKV_ERR_INVALID_ARG;
@@ -300,11 +305,19 @@ int mixkv_scores(const void* K, const void* V, const void* Qwin, const int32_t* 
   return enqueue_scores(c, K, V, Qwin, s_comp, s_ex_opt, s_div_opt, rbar_opt, rbar_in_opt,
                         status_dev);
 }
+}  // namespace
 
-int mixkv_select(const float* scores, const int32_t* cu_seqlens_host, int32_t batch, int32_t L,
-                 const mixkv_params* p, void* workspace, size_t workspace_bytes, int32_t* idx,
-                 int32_t* counts, int32_t* idx_offsets, int32_t* status_dev, void* stream) {
-  (void)status_dev;
+int mixkv_scores(const void* K, const void* V, const void* Qwin, const int32_t* cu_seqlens_host,
+                 int32_t batch, int32_t L, const mixkv_params* p, void* workspace,
+                 size_t workspace_bytes, float* s_comp, float* s_ex_opt, float* s_div_opt,
+                 float* rbar_opt, const float* rbar_in_opt, int32_t* status_dev, void* stream) {
+  return scores_impl(K, V, Qwin, cu_seqlens_host, batch, L, p, workspace, workspace_bytes, s_comp,
+                     s_ex_opt, s_div_opt, rbar_opt, rbar_in_opt, status_dev, false, stream);
+}
+
+int mixkv_internal_select(const float* scores, const int32_t* cu_seqlens_host, int32_t batch, int32_t L,
+                          const mixkv_params* p, void* workspace, size_t workspace_bytes, int32_t* idx,
+                          int32_t* counts, int32_t* idx_offsets, int32_t* status_dev, void* stream) {
   LaunchCtx c;
   int rc = make_ctx(p, cu_seqlens_host, batch, L, workspace, workspace_bytes, stream, &c);
   if (rc != MIXKV_OK) return rc;
@@ -315,7 +328,16 @@ int mixkv_select(const float* scores, const int32_t* cu_seqlens_host, int32_t ba
   memset(&t, 0, sizeof(t));
   t.idx = idx;
   t.idx_offsets = idx_offsets;
+  t.status_clear = status_dev;
   return enqueue_select(c, scores, counts, t);
+}
+
+int mixkv_select(const float* scores, const int32_t* cu_seqlens_host, int32_t batch, int32_t L,
+                 const mixkv_params* p, void* workspace, size_t workspace_bytes, int32_t* idx,
+                 int32_t* counts, int32_t* idx_offsets, int32_t* status_dev, void* stream) {
+  (void)status_dev;
+  return mixkv_internal_select(scores, cu_seqlens_host, batch, L, p, workspace, workspace_bytes, idx, counts,
+                               idx_offsets, nullptr, stream);
 }
 
 namespace {
@@ -497,32 +519,49 @@ int static_scratch(void** out) {
   *out = g_scratch_addr[dev];
   return MIXKV_OK;
 }
+
+// The scratch array for a problem that fits it.  The size is worked out on the host first: too
+// large a problem is refused before anything is enqueued (only attribute queries have run by then).
+int take_static_scratch(const mixkv_params* p, const int32_t* cu_seqlens_host, int32_t batch, int32_t L,
+                        void** scratch) {
+  int rc = check_params(p);
+  if (rc != MIXKV_OK) return rc;
+  SeqTable st;
+  int max_len = 0;
+  rc = build_table(p, cu_seqlens_host, batch, L, 1, &st, &max_len);
+  if (rc != MIXKV_OK) return rc;
+  Workspace ws;
+  carve(p, st, nullptr, &ws);
+  if (ws.bytes > (size_t)MIXKV_STATIC_SCRATCH_BYTES) return MIXKV_ERR_STATIC_SCRATCH_EXCEEDED;
+  return static_scratch(scratch);
+}
 }  // namespace
+
+int mixkv_internal_scores(const void* K, const void* V, const void* Qwin, const int32_t* cu_seqlens_host,
+                          int32_t batch, int32_t L, const mixkv_params* p, int use_static_scratch,
+                          void* workspace, size_t workspace_bytes, float* s_comp, float* s_ex_opt,
+                          float* s_div_opt, float* rbar_opt, const float* rbar_in_opt, int32_t* status_dev,
+                          void* stream) {
+  if (use_static_scratch) {
+    const int rc = take_static_scratch(p, cu_seqlens_host, batch, L, &workspace);
+    if (rc != MIXKV_OK) return rc;
+    workspace_bytes = MIXKV_STATIC_SCRATCH_BYTES;
+  }
+  return scores_impl(K, V, Qwin, cu_seqlens_host, batch, L, p, workspace, workspace_bytes, s_comp,
+                     s_ex_opt, s_div_opt, rbar_opt, rbar_in_opt, status_dev, true, stream);
+}
 
 int mixkv_scores_static(const void* K, const void* V, const void* Qwin,
                         const int32_t* cu_seqlens_host, int32_t batch, int32_t L,
                         const mixkv_params* p, float* s_comp, float* s_ex_opt, float* s_div_opt,
                         float* rbar_opt, const float* rbar_in_opt, int32_t* status_dev,
                         void* stream) {
-  // size the problem on the host first: too large a problem is refused before anything is
-  // enqueued (only attribute queries have run by then)
-  {
-    int rc = check_params(p);
-    if (rc != MIXKV_OK) return rc;
-    SeqTable st;
-    int max_len = 0;
-    rc = build_table(p, cu_seqlens_host, batch, L, 1, &st, &max_len);
-    if (rc != MIXKV_OK) return rc;
-    Workspace ws;
-    carve(p, st, nullptr, &ws);
-    if (ws.bytes > (size_t)MIXKV_STATIC_SCRATCH_BYTES) return MIXKV_ERR_STATIC_SCRATCH_EXCEEDED;
-  }
   void* scratch = nullptr;
-  int rc = static_scratch(&scratch);
+  const int rc = take_static_scratch(p, cu_seqlens_host, batch, L, &scratch);
   if (rc != MIXKV_OK) return rc;
-  return mixkv_scores(K, V, Qwin, cu_seqlens_host, batch, L, p, scratch,
-                      (size_t)MIXKV_STATIC_SCRATCH_BYTES, s_comp, s_ex_opt, s_div_opt, rbar_opt,
-                      rbar_in_opt, status_dev, stream);
+  return scores_impl(K, V, Qwin, cu_seqlens_host, batch, L, p, scratch,
+                     (size_t)MIXKV_STATIC_SCRATCH_BYTES, s_comp, s_ex_opt, s_div_opt, rbar_opt,
+                     rbar_in_opt, status_dev, false, stream);
 }
 
 namespace {

@@ -79,6 +79,7 @@ struct LaunchCtx {
   void* const* trace_events;  // optional measurement hook: events recorded between kernels
   int n_trace_events;
   mutable int stage;
+  bool clear_status;          // the first kernel sets the status word to 0
 
   // Records the event that marks the start of the next kernel (or the end of the last).
   void mark() const {
@@ -145,6 +146,7 @@ struct TailArgs {
   const void* V;
   void* K_out;
   void* V_out;
+  int* status_clear;   // optional word set to 0
 };
 // counts [layers, batch*H] <- candidates to select for budgets [layers, batch*H] given by the caller
 cudaError_t launch_given_budgets(const LaunchCtx& c, const int* budgets, int* counts);

@@ -285,7 +285,7 @@ template <int MB>
 __global__ void __launch_bounds__(p1_threads(MB), 1)
 k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ,
         const SeqTable st, const Workspace ws, const float scale_log2e,
-        int* status) {
+        const int clear_status, int* status) {
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
@@ -344,6 +344,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
   pdl_wait();   // everything earlier in the stream is complete: global memory may be touched
+  if (clear_status && status && blockIdx.x == 0 && tid == 0) *status = 0;
 
   if (warp < kEpiWarp0) {
     set_regs<kP1RegsLead, kP1RegsLaunch>();
@@ -1145,13 +1146,13 @@ cudaError_t launch_pass1(const LaunchCtx& c, const void* K, const void* Q, int* 
     cudaError_t e = ensure_smem(k_pass1<1>, kSmemLimit, done1);
     if (e != cudaSuccess) return e;
     return launch_pdl(k_pass1<1>, dim3(c.st.g1), dim3(p1_threads(1)), smem, c.stream, 1, tmK, tmQ, c.st,
-                      c.ws, c.scale_log2e, status);
+                      c.ws, c.scale_log2e, (int)c.clear_status, status);
   }
   const size_t smem = pass1_smem(2, c.st.NQ);
   cudaError_t e = ensure_smem(k_pass1<2>, kSmemLimit, done2);
   if (e != cudaSuccess) return e;
   return launch_pdl(k_pass1<2>, dim3(c.st.g1), dim3(p1_threads(2)), smem, c.stream, 1, tmK, tmQ, c.st,
-                    c.ws, c.scale_log2e, status);
+                    c.ws, c.scale_log2e, (int)c.clear_status, status);
 }
 
 cudaError_t launch_pass2(const LaunchCtx& c, const void* K, const void* V, const void* Q,

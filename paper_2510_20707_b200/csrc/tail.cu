@@ -545,6 +545,7 @@ struct TailKernelArgs {
   long long kv_layer_stride;  // elements between consecutive layers of K (V)
   int idx_cap;                // index-list entries reserved per layer
   int out_rows_cap;           // output rows reserved per layer
+  int* status_clear;          // optional word set to 0
   MixParams mp;
 };
 
@@ -601,6 +602,7 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   pdl_launch_dependents();
   pdl_wait();
 
+  if (a.status_clear && blockIdx.x == 0 && tid == 0) *a.status_clear = 0;
   // ---- budget and output offsets of this (b, h)
   if (tid < 32) {
     int off = 0, cnt;
@@ -1088,6 +1090,7 @@ cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
   a.kv_layer_stride = c.kv_layer_stride;
   a.idx_cap = c.idx_cap;
   a.out_rows_cap = c.out_rows_cap;
+  a.status_clear = t.status_clear;
   a.mp = mix_params(c.p);
   const TailShape sh = tail_shape(c);
   const bool fused = t.scores == nullptr;
