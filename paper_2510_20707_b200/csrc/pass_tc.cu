@@ -40,7 +40,6 @@ constexpr int kWarpTma = 0, kWarpMma = 1;
 constexpr int kP1WarpMma = 3;                    // pass 1: see k_pass1
 constexpr int kEpiWarp0 = 4;
 constexpr int kEpiWarps = 16;                    // warps 4..19
-constexpr int kEpiThreads = kEpiWarps * 32;
 constexpr int kAuxWarp0 = kEpiWarp0 + kEpiWarps; // warps 20..: key statistics / value norms
 
 // Registers per thread of the calling warpgroup from here on: N, where the kernel was launched
@@ -145,9 +144,9 @@ __host__ __device__ constexpr int p1_stages(int NQ) { return NQ > 224 ? 4 : 5; }
 // registers per thread: at launch, then per role (7 warpgroups: 40 + 4 * 72 + 2 * 88 = 7 * 72;
 // the key-statistics warps hold a batch of eight key rows in registers between their two sweeps)
 #ifndef P1_LEAD
-#define P1_LEAD 40
-#define P1_EPI 72
-#define P1_AUX 88
+#define P1_LEAD 24
+#define P1_EPI 64
+#define P1_AUX 112
 #endif
 constexpr int kP1RegsLaunch = 72, kP1RegsLead = P1_LEAD, kP1RegsEpi = P1_EPI, kP1RegsAux = P1_AUX;
 
@@ -211,10 +210,10 @@ __device__ __forceinline__ float fold_key_sums(const float* ksum, const SegList&
   }
   return sum;
 }
-// The pass-1 segments of the head that tile iterator `ti` (of either pass) stands on.
-__device__ __forceinline__ SegList pass1_segments(const SeqTable& st, const TileIter& ti) {
-  const int per_head = (st.tile1_start[ti.b + 1] - st.tile1_start[ti.b]) / st.H;
-  return SegList(ti.layer * st.nt1 + st.tile1_start[ti.b] + ti.h * per_head, per_head, split1(st));
+// The pass-1 segments of the head that segment iterator `sg` (of either pass) stands on.
+__device__ __forceinline__ SegList pass1_segments(const SeqTable& st, const SegIter& sg) {
+  const int per_head = (st.tile1_start[sg.b + 1] - st.tile1_start[sg.b]) / st.H;
+  return SegList(sg.layer * st.nt1 + st.tile1_start[sg.b] + sg.h * per_head, per_head, split1(st));
 }
 
 // The running softmax statistics of a query row are a pair (m, z): z = sum over the keys seen
@@ -351,24 +350,26 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     if (warp == kWarpTma) {
       // ---------------------------------------------------------------- TMA producer
       if (lane == 0) {
-        int it = 0, segn = 0;
-        bool seg_start = true;
-        for (TileIter ti(st.tile1_start, st.batch, H, st.nt1, lo, hi); ti.valid(); ti.next()) {
-          if (seg_start) {
-            if (segn > 0 && !mbar_wait(&bars->qfree, (segn - 1) & 1, abort)) break;
-            mbar_expect_tx(&bars->qfull, NQ * 256);
-            tma_load_3d(sQ, &tmQ, 0, ti.bh() * NQ, ti.layer, &bars->qfull);
-            tma_load_3d(sQ + NQ * 128, &tmQ, 64, ti.bh() * NQ, ti.layer, &bars->qfull);
-            ++segn;
+        int s = 0, ph = 1, it = 0, segn = 0;
+        bool ok = true;
+        for (SegIter sg(st.tile1_start, st.batch, H, st.nt1, lo, hi); sg.valid() && ok; sg.next()) {
+          if (segn > 0 && !mbar_wait(&bars->qfree, (segn - 1) & 1, abort)) break;
+          mbar_expect_tx(&bars->qfull, NQ * 256);
+          tma_load_3d(sQ, &tmQ, 0, sg.bh() * NQ, sg.layer, &bars->qfull);
+          tma_load_3d(sQ + NQ * 128, &tmQ, 64, sg.bh() * NQ, sg.layer, &bars->qfull);
+          ++segn;
+          int y = st.cu[sg.b] + sg.t0 * kTile;
+          for (int k = 0; k < sg.n; ++k, y += kTile) {
+            if (!mbar_wait(&bars->empty[s], ph, abort)) {
+              ok = false;
+              break;
+            }
+            mbar_expect_tx(&bars->full[s], kTileBytes);
+            tma_load_4d(sK + s * kTileBytes, &tmK, 0, y, sg.h, sg.layer, &bars->full[s]);
+            tma_load_4d(sK + s * kTileBytes + kHalfBytes, &tmK, 64, y, sg.h, sg.layer, &bars->full[s]);
+            if (++s == kP1Stages) s = 0, ph ^= 1;
+            ++it;
           }
-          seg_start = ti.seg_last();
-          const int s = it % kP1Stages, ph = (it / kP1Stages) & 1;
-          if (!mbar_wait(&bars->empty[s], ph ^ 1, abort)) break;
-          mbar_expect_tx(&bars->full[s], kTileBytes);
-          const int y = st.cu[ti.b] + ti.t * kTile;
-          tma_load_4d(sK + s * kTileBytes, &tmK, 0, y, ti.h, ti.layer, &bars->full[s]);
-          tma_load_4d(sK + s * kTileBytes + kHalfBytes, &tmK, 64, y, ti.h, ti.layer, &bars->full[s]);
-          ++it;
         }
         if (*abort) {
           raise(status, abort);
@@ -377,44 +378,47 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
       }
     } else if (warp == kP1WarpMma) {
       // ---------------------------------------------------------------- MMA issuer
-      if (lane == 0) {
+      {
+        const uint32_t on = elect_one();
         constexpr uint32_t idesc = umma_idesc_bf16(128, kTile);
         const uint32_t q_lo = umma_desc_lo(smem_u32(sQ));
         const uint32_t k_lo = umma_desc_lo(smem_u32(sK));
         const uint32_t q_half = (uint32_t)(NQ * 128) >> 4;   // second 64-column half of the queries
-        int it = 0, segn = 0;
-        bool seg_start = true;
-        for (TileIter ti(st.tile1_start, st.batch, H, st.nt1, lo, hi); ti.valid(); ti.next()) {
-          if (seg_start) {
-            if (!mbar_wait(&bars->qfull, segn & 1, abort)) break;
-            ++segn;
-          }
-          seg_start = ti.seg_last();
-          const int s = it % kP1Stages, ph = (it / kP1Stages) & 1, ts = it & 1, tph = (it >> 1) & 1;
-          if (!mbar_wait(&bars->full[s], ph, abort)) break;
-          if (!mbar_wait(&bars->tempty[ts], tph ^ 1, abort)) break;
-          tc_fence_after();
-          const uint32_t kb_lo = k_lo + (uint32_t)s * (kTileBytes >> 4);
-          const uint32_t td = tmem + ts * (MB * 128);
-#pragma unroll
-          for (int mb = 0; mb < MB; ++mb) {
-            // k-steps of 16 columns: 32 bytes apart inside a 64-column half
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {
-              const uint32_t a_lo = q_lo + (ks >> 2) * q_half + (uint32_t)(mb * (16384 >> 4) + (ks & 3) * 2);
-              const uint32_t b_lo = kb_lo + (uint32_t)((ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2);
-              if (ks == 0)
-                umma_bf16_lo<0>(td + mb * 128, a_lo, b_lo, idesc);
-              else
-                umma_bf16_lo<1>(td + mb * 128, a_lo, b_lo, idesc);
+        int s = 0, ph = 0, ts = 0, tph = 1, segn = 0;
+        bool ok = true;
+        for (SegIter sg(st.tile1_start, st.batch, H, st.nt1, lo, hi); sg.valid() && ok; sg.next()) {
+          if (!mbar_wait(&bars->qfull, segn & 1, abort)) break;
+          ++segn;
+          for (int k = 0; k < sg.n; ++k) {
+            if (!mbar_wait(&bars->full[s], ph, abort) || !mbar_wait(&bars->tempty[ts], tph, abort)) {
+              ok = false;
+              break;
             }
+            tc_fence_after();
+            const uint32_t kb_lo = k_lo + (uint32_t)s * (kTileBytes >> 4);
+            const uint32_t td = tmem + ts * (MB * 128);
+#pragma unroll
+            for (int mb = 0; mb < MB; ++mb) {
+              // k-steps of 16 columns: 32 bytes apart inside a 64-column half
+#pragma unroll
+              for (int ks = 0; ks < 8; ++ks) {
+                const uint32_t a_lo = q_lo + (ks >> 2) * q_half + (uint32_t)(mb * (16384 >> 4) + (ks & 3) * 2);
+                const uint32_t b_lo = kb_lo + (uint32_t)((ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2);
+                if (ks == 0)
+                  umma_bf16_lo<0>(td + mb * 128, a_lo, b_lo, idesc, on);
+                else
+                  umma_bf16_lo<1>(td + mb * 128, a_lo, b_lo, idesc, on);
+              }
+            }
+            umma_commit(&bars->empty[s], on);
+            umma_commit(&bars->tfull[ts], on);
+            if (k + 1 == sg.n) umma_commit(&bars->qfree, on);
+            if (++s == kP1Stages) s = 0, ph ^= 1;
+            ts ^= 1;
+            tph ^= ts ^ 1;
           }
-          umma_commit(&bars->empty[s]);
-          umma_commit(&bars->tfull[ts]);
-          if (seg_start) umma_commit(&bars->qfree);
-          ++it;
         }
-        if (*abort) raise(status, abort);
+        if (*abort && on) raise(status, abort);
       }
     }
   } else if (warp < kAuxWarp0) {
@@ -437,166 +441,150 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     // per row.  Named barriers 6 + blk ("handed over") and 8 + blk ("read").
     const int xrow = (unit > 0 ? unit - 1 : 0) * 128 + (MB == 2 ? blk * 128 : 0) + quarter * 32 + lane;
     constexpr int kXThreads = NU * 128;
-    float m_run = -1e30f, z_run = 0.f;
-    int it = 0, seg_first = lo, segs_done = 0;
-    bool seg_start = true, no_ref = true;
-    for (TileIter ti(st.tile1_start, st.batch, H, st.nt1, lo, hi); ti.valid(); ti.next()) {
-      if (seg_start) {
-        m_run = -1e30f;
-        z_run = 0.f;
-        no_ref = true;   // the segment's first chunk sets the reference
-        seg_first = ti.id;
-      }
-      seg_start = ti.seg_last();
-      const int L = st.cu[ti.b + 1] - st.cu[ti.b], P = L - W;
-      const int ts = it & 1, tph = (it >> 1) & 1;
-      // (after an abort the waits fail at once; the loop goes on without work so that the
-      // segment-end barriers below stay matched)
-      const bool ok = warp_on && mbar_wait(&bars->tfull[ts], tph, abort);
-      if (ok) {
-        tc_fence_after();
-        const int k0 = ti.t * kTile + unit * NC;
-        const bool need_mask = ti.t * kTile + kTile > P;
-        const int lim = P + jrow;   // last key this row may see
-        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + ts * (MB * 128) + col0;
+    int ts = 0, tph = 0, segs_done = 0;
+    const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + col0;
+    for (SegIter sg(st.tile1_start, st.batch, H, st.nt1, lo, hi); sg.valid(); sg.next()) {
+      float m_run = -1e30f, z_run = 0.f;
+      const int P = st.cu[sg.b + 1] - st.cu[sg.b] - W;
+      const int t_mask = P / kTile;   // first tile that holds keys some row may not see
+      // a warp on padding rows only walks the segments, for the barriers below
+      for (int t = warp_on ? sg.t0 : sg.end(); t < sg.end(); ++t) {
+        // (after an abort the waits fail at once; the loop goes on without work so that the
+        // segment-end barriers below stay matched)
+        if (mbar_wait(&bars->tfull[ts], tph, abort)) {
+          tc_fence_after();
+          const uint32_t taddr = tbase + ts * (MB * 128);
 #pragma unroll 1
-        for (int c0 = 0; c0 < NC; c0 += 32) {   // kept rolled: the body must stay in the i-cache
-          bool slow = no_ref || need_mask;      // the same in every lane
-          float zc = 0.f;
-          if (!slow) {
-            uint32_t ra[32];
-            tmem_ld32(taddr + c0, ra);
-            tmem_ld_wait();
-            tmem_ld_fence(ra);
-            zc = chunk_expsum(ra, scale_log2e, m_run);
-            slow = __any_sync(0xffffffffu, !(zc < kChunkSumLimit));
+          for (int c0 = 0; c0 < NC; c0 += 32) {   // kept rolled: the body must stay in the i-cache
+            bool slow = t == sg.t0 || t >= t_mask;  // the same in every lane; the first tile sets the reference
+            float zc = 0.f;
+            if (!slow) {
+              uint32_t ra[32];
+              tmem_ld32(taddr + c0, ra);
+              tmem_ld_wait();
+              tmem_ld_fence(ra);
+              zc = chunk_expsum(ra, scale_log2e, m_run);
+              slow = __any_sync(0xffffffffu, !(zc < kChunkSumLimit));
+            }
+            if (slow) {
+              const float2 mz = softmax_chunk_ref(taddr + c0, t >= t_mask, t * kTile + unit * NC + c0, P + jrow,
+                                                  scale_log2e, m_run, z_run);
+              m_run = mz.x;
+              z_run = mz.y;
+            } else {
+              z_run += zc;
+            }
           }
-          if (slow) {
-            const float2 mz =
-                softmax_chunk_ref(taddr + c0, need_mask, k0 + c0, lim, scale_log2e, m_run, z_run);
-            m_run = mz.x;
-            z_run = mz.y;
-            no_ref = false;
-          } else {
-            z_run += zc;
-          }
+          tc_fence_before();
+          __syncwarp();   // one arrival per warp: 512 single arrivals on one word cost more than a chunk
+          if (lane == 0) mbar_arrive(&bars->tempty[ts]);
         }
+        ts ^= 1;
+        tph ^= ts ^ 1;
       }
-      if (warp_on) {
-        tc_fence_before();
-        __syncwarp();   // one arrival per warp: 512 single arrivals on one word cost more than a chunk
-        if (lane == 0) mbar_arrive(&bars->tempty[ts]);
-      }
-      if (seg_start) {   // (here: this was the segment's last tile)
-        if (unit > 0) {
-          if (segs_done > 0) named_bar_sync(8 + blk, kXThreads);   // the last hand-over was read
-          sxs[xrow] = make_float2(m_run, z_run);
-          named_bar_arrive(6 + blk, kXThreads);
-        } else {
-          named_bar_sync(6 + blk, kXThreads);
-          float2 mz = make_float2(m_run, z_run);
+      if (unit > 0) {
+        if (segs_done > 0) named_bar_sync(8 + blk, kXThreads);   // the last hand-over was read
+        sxs[xrow] = make_float2(m_run, z_run);
+        named_bar_arrive(6 + blk, kXThreads);
+      } else {
+        named_bar_sync(6 + blk, kXThreads);
+        float2 mz = make_float2(m_run, z_run);
 #pragma unroll
-          for (int u = 1; u < NU; ++u) mz = merge_stats(mz, sxs[xrow + (u - 1) * 128]);
-          named_bar_arrive(8 + blk, kXThreads);
-          if (row < NQ) ws.rowstat[(size_t)seg_first * NQ + row] = mz;
-        }
-        ++segs_done;
+        for (int u = 1; u < NU; ++u) mz = merge_stats(mz, sxs[xrow + (u - 1) * 128]);
+        named_bar_arrive(8 + blk, kXThreads);
+        if (row < NQ) ws.rowstat[(size_t)sg.id * NQ + row] = mz;
       }
-      ++it;
+      ++segs_done;
     }
   } else {
     // ------------------------------------------------------------------ key statistics
-    // Sixteen lanes share a key row (one 16-byte chunk each); a pair of 8-row batches is one
-    // warp-wide step (one batch per 16-lane group).  Sweep 1 squares, a butterfly leaves the
-    // squared norm of row r with lanes 2r and 2r+1, sweep 2 adds the rows scaled by 1/|k| into
-    // eight per-thread sums (dims 8c .. 8c+7).
+    // A warp takes 16 rows of a tile in four steps of four; eight lanes share a row, lane c of them with
+    // 16-byte chunk c of either 64-column half (conflict-free in the swizzled tile).  The bf16 are widened
+    // once and stay in registers as fp32 pairs between their two uses: squares, whose sums are folded so
+    // that lanes 2k, 2k + 1 end with the squared norm of their row of step k, then the rows scaled by 1/|k|
+    // into sixteen per-thread sums.  These warps paced the whole pass (3900 clocks per tile of G*W = 224, 3600
+    // of 128) when sixteen lanes shared a row and every bf16 was widened twice.
     set_regs<kP1RegsAux, kP1RegsLaunch>();
     const int aux_w = warp - kAuxWarp0;
-    const int c = lane & 15, lg = lane >> 4;
-    const int chalf = c >> 3, cc = c & 7;
+    const int c = lane & 7, lg = lane >> 3;
     constexpr int aux_threads = kP1AuxWarps * 32;
     const int kt = tid - kAuxWarp0 * 32;
-    f32x2 acc2[4];   // dims 8c .. 8c+7 as four packed pairs
+    // this lane's chunk of row 16 aux_w + 4 k + lg in half 0: the row's swizzle is (row & 7) = 4 (k & 1) + lg
+    const uint32_t off0 = (uint32_t)(16 * aux_w + lg) * 128 + ((uint32_t)(c ^ lg) << 4);
+    const uint32_t off1 = (uint32_t)(16 * aux_w + lg) * 128 + ((uint32_t)(c ^ (lg + 4)) << 4);
+    const int my_row = 16 * aux_w + 4 * (c >> 1) + lg;   // the row whose norm this lane ends with
+    int s = 0, ph = 0;
+    for (SegIter sg(st.tile1_start, st.batch, H, st.nt1, lo, hi); sg.valid(); sg.next()) {
+      f32x2 acc2[8];   // dims 8c .. 8c+7 of half 0, then of half 1, as packed pairs
 #pragma unroll
-    for (int e = 0; e < 4; ++e) acc2[e] = pack2(0.f, 0.f);
-    int it = 0, seg_first = lo;
-    bool seg_start = true;
-    for (TileIter ti(st.tile1_start, st.batch, H, st.nt1, lo, hi); ti.valid(); ti.next()) {
-      if (seg_start) {
+      for (int e = 0; e < 8; ++e) acc2[e] = pack2(0.f, 0.f);
+      const int L = st.cu[sg.b + 1] - st.cu[sg.b];
+      float* kinv = ws.kinv + kpos(st, sg.layer, sg.h, sg.b, 0);
+      int i = sg.t0 * kTile + my_row;
+      for (int k = 0; k < sg.n; ++k, i += kTile) {
+        const bool ok = mbar_wait(&bars->full[s], ph, abort);
+        const unsigned char* tile = sK + s * kTileBytes;
+        f32x2 f[4][8];
+        float p[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc2[e] = pack2(0.f, 0.f);
-        seg_first = ti.id;
-      }
-      seg_start = ti.seg_last();
-      const int L = st.cu[ti.b + 1] - st.cu[ti.b];
-      const int s = it % kP1Stages, ph = (it / kP1Stages) & 1;
-      const bool ok = mbar_wait(&bars->full[s], ph, abort);
-      const unsigned char* tile = sK + s * kTileBytes + chalf * kHalfBytes;
-      {
-        const int row0 = (2 * aux_w + lg) * 8;
-        uint4 u[8];
-        float p[8];
-#pragma unroll
-        for (int rr = 0; rr < 8; ++rr) {
-          u[rr] = *reinterpret_cast<const uint4*>(tile + sw128_offset(row0 + rr, cc));
-          const uint32_t* p2 = reinterpret_cast<const uint32_t*>(&u[rr]);
+        for (int r = 0; r < 4; ++r) {
           f32x2 sq = pack2(0.f, 0.f);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const f32x2 f2 = bf16x2_wide(p2[e]);
-            sq = fma2(f2, f2, sq);
+          for (int hf = 0; hf < 2; ++hf) {
+            const uint4 u = *reinterpret_cast<const uint4*>(tile + hf * kHalfBytes + r * 512 + ((r & 1) ? off1 : off0));
+            f[r][4 * hf] = bf16x2_wide(u.x), f[r][4 * hf + 1] = bf16x2_wide(u.y);
+            f[r][4 * hf + 2] = bf16x2_wide(u.z), f[r][4 * hf + 3] = bf16x2_wide(u.w);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sq = fma2(f[r][4 * hf + e], f[r][4 * hf + e], sq);
           }
           float s0, s1;
           unpack2(sq, s0, s1);
-          p[rr] = s0 + s1;
+          p[r] = s0 + s1;
         }
         // the tile now lives in registers: hand the stage back
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars->empty[s]);
-#pragma unroll
-        for (int o = 8; o >= 2; o >>= 1) {
-          const bool up = (c & o) != 0;
-#pragma unroll
-          for (int k = 0; k < o / 2; ++k) {
-            const float send = up ? p[k] : p[k + o / 2];
-            const float keep = up ? p[k + o / 2] : p[k];
-            p[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-          }
+        if (++s == kP1Stages) s = 0, ph ^= 1;
+        {
+          const bool up = (c & 4) != 0;
+          const float k0 = up ? p[2] : p[0], k1 = up ? p[3] : p[1], g0 = up ? p[0] : p[2], g1 = up ? p[1] : p[3];
+          p[0] = k0 + __shfl_xor_sync(0xffffffffu, g0, 4);
+          p[1] = k1 + __shfl_xor_sync(0xffffffffu, g1, 4);
+          const bool up2 = (c & 2) != 0;
+          p[0] = (up2 ? p[1] : p[0]) + __shfl_xor_sync(0xffffffffu, up2 ? p[0] : p[1], 2);
+          p[0] += __shfl_xor_sync(0xffffffffu, p[0], 1);
         }
-        p[0] += __shfl_xor_sync(0xffffffffu, p[0], 1);
-        const int i = ti.t * kTile + row0 + (c >> 1);
         const float inv = (ok && i < L && p[0] > 0.f) ? rsqrtf(p[0]) : 0.f;
-        if (i < L && (c & 1) == 0) ws.kinv[kpos(st, ti.layer, ti.h, ti.b, i)] = inv;
+        if (i < L && (c & 1) == 0) kinv[i] = inv;
 #pragma unroll
-        for (int rr = 0; rr < 8; ++rr) {
-          const float w = __shfl_sync(0xffffffffu, inv, (lane & 16) | (rr << 1));
-          const uint32_t* p2 = reinterpret_cast<const uint32_t*>(&u[rr]);
+        for (int r = 0; r < 4; ++r) {
+          const float w = __shfl_sync(0xffffffffu, inv, (lane & 24) | (2 * r));
           const f32x2 w2 = pack2(w, w);
 #pragma unroll
-          for (int e = 0; e < 4; ++e) acc2[e] = fma2(bf16x2_wide(p2[e]), w2, acc2[e]);
+          for (int e = 0; e < 8; ++e) acc2[e] = fma2(f[r][e], w2, acc2[e]);
         }
+        // (no barrier per tile: after an abort the waits fail at once and every warp still walks
+        // the same tiles, so the segment-end barriers below stay matched)
       }
-      // (no barrier per tile: after an abort the waits fail at once and every warp still walks
-      // the same tiles, so the segment-end barriers below stay matched)
-      if (seg_start) {
-        float acc[8];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) unpack2(acc2[e], acc[2 * e], acc[2 * e + 1]);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          const float v = acc[e] + __shfl_xor_sync(0xffffffffu, acc[e], 16);
-          if (lane < 16) sks[aux_w * 128 + c * 8 + e] = v;
-        }
-        named_bar_sync(2, aux_threads);
-        if (kt < kHeadDim) {
-          float t = 0.f;
-#pragma unroll
-          for (int w = 0; w < kP1AuxWarps; ++w) t += sks[w * 128 + kt];
-          ws.ksum[(size_t)seg_first * kHeadDim + kt] = t;
-        }
-        named_bar_sync(2, aux_threads);
+      for (int e = 0; e < 8; ++e) {
+        float a0, a1;
+        unpack2(acc2[e], a0, a1);
+        a0 += __shfl_xor_sync(0xffffffffu, a0, 8);
+        a1 += __shfl_xor_sync(0xffffffffu, a1, 8);
+        a0 += __shfl_xor_sync(0xffffffffu, a0, 16);
+        a1 += __shfl_xor_sync(0xffffffffu, a1, 16);
+        if (lane < 8)
+          *reinterpret_cast<float2*>(sks + aux_w * 128 + (e >> 2) * 64 + 8 * c + 2 * (e & 3)) = make_float2(a0, a1);
       }
-      ++it;
+      named_bar_sync(2, aux_threads);
+      if (kt < kHeadDim) {
+        float t = 0.f;
+#pragma unroll
+        for (int w = 0; w < kP1AuxWarps; ++w) t += sks[w * 128 + kt];
+        ws.ksum[(size_t)sg.id * kHeadDim + kt] = t;
+      }
+      named_bar_sync(2, aux_threads);
     }
   }
   tc_fence_before();
@@ -688,7 +676,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&bars->tfull[s], 1);
-      mbar_init(&bars->tempty[s], 128);    // the warpgroup that owns the accumulator stage
+      mbar_init(&bars->tempty[s], 4);      // the warps of the warpgroup that owns the accumulator stage
     }
     mbar_init(&bars->qfull, 1);
     mbar_init(&bars->qfree, 1);
@@ -711,24 +699,26 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   if (warp == kWarpTma) {
     // ------------------------------------------------------------------ K / Q producer
     if (lane == 0) {
-      int it = 0, segn = 0;
-      bool seg_start = true;
-      for (TileIter ti(st.tile2_start, st.batch, H, st.nt2, lo, hi); ti.valid(); ti.next()) {
-        if (seg_start) {
-          if (segn > 0 && !mbar_wait(&bars->qfree, (segn - 1) & 1, abort)) break;
-          mbar_expect_tx(&bars->qfull, NQ * 256);
-          tma_load_3d(sQ, &tmQ, 0, ti.bh() * NQ, ti.layer, &bars->qfull);
-          tma_load_3d(sQ + NB * 128, &tmQ, 64, ti.bh() * NQ, ti.layer, &bars->qfull);
-          ++segn;
+      int s = 0, ph = 1, it = 0, segn = 0;
+      bool ok = true;
+      for (SegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
+        if (segn > 0 && !mbar_wait(&bars->qfree, (segn - 1) & 1, abort)) break;
+        mbar_expect_tx(&bars->qfull, NQ * 256);
+        tma_load_3d(sQ, &tmQ, 0, sg.bh() * NQ, sg.layer, &bars->qfull);
+        tma_load_3d(sQ + NB * 128, &tmQ, 64, sg.bh() * NQ, sg.layer, &bars->qfull);
+        ++segn;
+        int y = st.cu[sg.b] + sg.t0 * kTile;
+        for (int k = 0; k < sg.n; ++k, y += kTile) {
+          if (!mbar_wait(&bars->kempty[s], ph, abort)) {
+            ok = false;
+            break;
+          }
+          mbar_expect_tx(&bars->kfull[s], kTileBytes);
+          tma_load_4d(sK + s * kTileBytes, &tmK, 0, y, sg.h, sg.layer, &bars->kfull[s]);
+          tma_load_4d(sK + s * kTileBytes + kHalfBytes, &tmK, 64, y, sg.h, sg.layer, &bars->kfull[s]);
+          if (++s == kP2KStages) s = 0, ph ^= 1;
+          ++it;
         }
-        seg_start = ti.seg_last();
-        const int s = it % kP2KStages, ph = (it / kP2KStages) & 1;
-        if (!mbar_wait(&bars->kempty[s], ph ^ 1, abort)) break;
-        mbar_expect_tx(&bars->kfull[s], kTileBytes);
-        const int y = st.cu[ti.b] + ti.t * kTile;
-        tma_load_4d(sK + s * kTileBytes, &tmK, 0, y, ti.h, ti.layer, &bars->kfull[s]);
-        tma_load_4d(sK + s * kTileBytes + kHalfBytes, &tmK, 64, y, ti.h, ti.layer, &bars->kfull[s]);
-        ++it;
       }
       if (*abort) {
         raise(status, abort);
@@ -738,20 +728,20 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   } else if (warp == kWarpTmaV) {
     // ------------------------------------------------------------------ V producer
     if (lane == 0 && use_vnorm == MIXKV_INTRINSIC_VNORM) {
-      int vit = 0;
+      int vit = 0, vs = 0, vph = 1;
       bool ok = true;
-      for (TileIter ti(st.tile2_start, st.batch, H, st.nt2, lo, hi); ti.valid() && ok; ti.next()) {
-        const int y = st.cu[ti.b] + ti.t * kTile;
-        for (int sub = 0; sub < 2; ++sub) {
-          const int vs = vit % vstages, vph = (vit / vstages) & 1;
-          if (!mbar_wait(&bars->vempty[vs], vph ^ 1, abort)) {
+      for (SegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
+        int y = st.cu[sg.b] + sg.t0 * kTile;
+        for (int k = 0; k < 2 * sg.n; ++k, y += 64) {   // half tiles of 64 rows
+          if (!mbar_wait(&bars->vempty[vs], vph, abort)) {
             ok = false;
             break;
           }
           mbar_expect_tx(&bars->vfull[vs], kVSubBytes);
           unsigned char* dst = sV + vs * kVSubBytes;
-          tma_load_4d(dst, &tmV, 0, y + sub * 64, ti.h, ti.layer, &bars->vfull[vs]);
-          tma_load_4d(dst + kVSubBytes / 2, &tmV, 64, y + sub * 64, ti.h, ti.layer, &bars->vfull[vs]);
+          tma_load_4d(dst, &tmV, 0, y, sg.h, sg.layer, &bars->vfull[vs]);
+          tma_load_4d(dst + kVSubBytes / 2, &tmV, 64, y, sg.h, sg.layer, &bars->vfull[vs]);
+          if (++vs == vstages) vs = 0, vph ^= 1;
           ++vit;
         }
       }
@@ -762,35 +752,42 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     }
   } else if (warp == kWarpMma) {
     // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc_bf16(128, NB);
-      int it = 0, segn = 0;
-      bool seg_start = true;
-      for (TileIter ti(st.tile2_start, st.batch, H, st.nt2, lo, hi); ti.valid(); ti.next()) {
-        if (seg_start) {
-          if (!mbar_wait(&bars->qfull, segn & 1, abort)) break;
-          if (!mbar_wait(&bars->kbready, segn & 1, abort)) break;
-          ++segn;
+    const uint32_t on = elect_one();
+    const uint32_t idesc = umma_idesc_bf16(128, NB);
+    const uint32_t k_lo = umma_desc_lo(smem_u32(sK)), q_lo = umma_desc_lo(smem_u32(sQ));
+    const uint32_t q_half = (uint32_t)(NB * 128) >> 4;   // second 64-column half of the B operand
+    int s = 0, ph = 0, ts = 0, tph = 1, segn = 0;
+    bool ok = true;
+    for (SegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
+      if (!mbar_wait(&bars->qfull, segn & 1, abort)) break;
+      if (!mbar_wait(&bars->kbready, segn & 1, abort)) break;
+      ++segn;
+      for (int k = 0; k < sg.n; ++k) {
+        if (!mbar_wait(&bars->kfull[s], ph, abort) || !mbar_wait(&bars->tempty[ts], tph, abort)) {
+          ok = false;
+          break;
         }
-        seg_start = ti.seg_last();
-        const int s = it % kP2KStages, ph = (it / kP2KStages) & 1, ts = it & 1, tph = (it >> 1) & 1;
-        if (!mbar_wait(&bars->kfull[s], ph, abort)) break;
-        if (!mbar_wait(&bars->tempty[ts], tph ^ 1, abort)) break;
         tc_fence_after();
-        const uint32_t kaddr = smem_u32(sK + s * kTileBytes);
+        const uint32_t kb_lo = k_lo + (uint32_t)s * (kTileBytes >> 4);
+        const uint32_t td = tmem + ts * 256;
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
-          const uint64_t da = umma_desc_sw128(kaddr + (ks >> 2) * kHalfBytes + (ks & 3) * 32);
-          const uint64_t db = umma_desc_sw128(smem_u32(sQ) + (ks >> 2) * NB * 128 + (ks & 3) * 32);
-          umma_bf16(tmem + ts * 256, da, db, idesc, ks > 0);
+          const uint32_t a_lo = kb_lo + (uint32_t)((ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2);
+          const uint32_t b_lo = q_lo + (ks >> 2) * q_half + (uint32_t)((ks & 3) * 2);
+          if (ks == 0)
+            umma_bf16_lo<0>(td, a_lo, b_lo, idesc, on);
+          else
+            umma_bf16_lo<1>(td, a_lo, b_lo, idesc, on);
         }
-        umma_commit(&bars->kempty[s]);
-        umma_commit(&bars->tfull[ts]);
-        if (seg_start) umma_commit(&bars->qfree);
-        ++it;
+        umma_commit(&bars->kempty[s], on);
+        umma_commit(&bars->tfull[ts], on);
+        if (k + 1 == sg.n) umma_commit(&bars->qfree, on);
+        if (++s == kP2KStages) s = 0, ph ^= 1;
+        ts ^= 1;
+        tph ^= ts ^ 1;
       }
-      if (*abort) raise(status, abort);
     }
+    if (*abort && on) raise(status, abort);
   } else if (warp >= kEpiWarp0 && warp < kEpiWarp0 + kP2EpiWarps) {
     // ------------------------------------------------------------------ epilogue
     // The two warpgroups take alternate tiles (warpgroup g owns accumulator stage g), one key
@@ -809,28 +806,27 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     const float log2W = log2f((float)W);
     const int barid = 1 + wg;                      // named barriers 1, 2: one per warpgroup
     const f32x2 sc2 = pack2(scale_log2e, scale_log2e);
-    float dmin = INFINITY, dmax = -INFINITY, dsum = 0.f, exw = 0.f;
-    int it = 0, seg_first = lo;
-    bool seg_start = true;
-    for (TileIter ti(st.tile2_start, st.batch, H, st.nt2, lo, hi); ti.valid(); ti.next()) {
-      const int L = st.cu[ti.b + 1] - st.cu[ti.b], P = L - W;
-      if (seg_start) {
-        named_bar_sync(5, kP2EpiWarps * 32);   // the previous segment's readers of sbq are done
-        if (et < NQ) sbq[et] = fold_row_stats(ws.rowstat, pass1_segments(st, ti), NQ, et, log2W);
-        dmin = INFINITY, dmax = -INFINITY, dsum = 0.f, exw = 0.f;
-        seg_first = ti.id;
-        named_bar_sync(5, kP2EpiWarps * 32);
-      }
-      seg_start = ti.seg_last();
-      const int ts = it & 1;
-      if (ts == wg) {   // this warpgroup's tile
-        const int tph = (it >> 1) & 1;
-        const int ikey = ti.t * kTile + key;
+    int tile = 0;   // parity decides which warpgroup owns it
+    for (SegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid(); sg.next()) {
+      const int P = st.cu[sg.b + 1] - st.cu[sg.b] - W;
+      named_bar_sync(5, kP2EpiWarps * 32);   // the previous segment's readers of sbq are done
+      if (et < NQ) sbq[et] = fold_row_stats(ws.rowstat, pass1_segments(st, sg), NQ, et, log2W);
+      float dmin = INFINITY, dmax = -INFINITY, dsum = 0.f, exw = 0.f;
+      named_bar_sync(5, kP2EpiWarps * 32);
+      const float* kinv = ws.kinv + kpos(st, sg.layer, sg.h, sg.b, 0);
+      const size_t poff = ppos(st, sg.layer, sg.h, sg.b, 0);
+      float* ex_out = ws.s_ex_raw + poff;
+      float* sd_out = s_div_out + poff;
+      // this warpgroup's tiles of the segment
+      const int skip = (tile & 1) ^ wg;
+      for (int t = sg.t0 + skip, tl = tile + skip; t < sg.end(); t += 2, tl += 2) {
+        const int tph = (tl >> 1) & 1;
+        const int ikey = t * kTile + key;
         float kinv_i = 0.f;
-        if (ikey < P) kinv_i = ws.kinv[kpos(st, ti.layer, ti.h, ti.b, ikey)];
-        const bool ok = mbar_wait(&bars->tfull[ts], tph, abort);
+        if (ikey < P) kinv_i = kinv[ikey];
+        const bool ok = mbar_wait(&bars->tfull[wg], tph, abort);
         tc_fence_after();
-        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + ts * 256;
+        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + wg * 256;
         f32x2 acc = pack2(0.f, 0.f);
         float dot = 0.f;
         if (ok) {
@@ -859,15 +855,15 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
           dot = (__uint_as_float(rd[0]) + __uint_as_float(rd[1])) + __uint_as_float(rd[2]);
         }
         tc_fence_before();
-        mbar_arrive(&bars->tempty[ts]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->tempty[wg]);
         if (ok && ikey < P) {
           float acc0, acc1;
           unpack2(acc, acc0, acc1);
-          const size_t poff = ppos(st, ti.layer, ti.h, ti.b, 0);
           const float ex = acc0 + acc1;
-          ws.s_ex_raw[poff + ikey] = ex;
+          ex_out[ikey] = ex;
           const float sd = -dot * kinv_i;
-          s_div_out[poff + ikey] = sd;
+          sd_out[ikey] = sd;
           dmin = fminf(dmin, sd);
           dmax = fmaxf(dmax, sd);
           dsum += sd;
@@ -876,7 +872,8 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
           exw = fmaf(ex, (float)cover, exw);
         }
       }
-      if (seg_start) {
+      tile += sg.n;
+      {
         // this warpgroup's share of the segment's score statistics (neutral if it had no tile)
         const float a = warp_min(dmin), b2 = warp_max(dmax), c2 = warp_sum(dsum),
                     d2 = warp_sum(exw);
@@ -889,13 +886,12 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         }
         named_bar_sync(barid, 128);
         if (gt == 0) {
-          ws.dstat[(size_t)seg_first * 2 + wg] = make_float4(
+          ws.dstat[(size_t)sg.id * 2 + wg] = make_float4(
               fminf(fminf(sr[0], sr[1]), fminf(sr[2], sr[3])),
               fmaxf(fmaxf(sr[4], sr[5]), fmaxf(sr[6], sr[7])),
               (sr[8] + sr[9]) + (sr[10] + sr[11]), (sr[12] + sr[13]) + (sr[14] + sr[15]));
         }
       }
-      ++it;
     }
   } else if (warp >= kP2AuxWarp0) {
     // ------------------------------------------------------------------ mean key, value norms
@@ -906,109 +902,104 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     // tile, warps 14, 15 the last 64; one row per thread from the swizzled half tile.
     const int vt = tid - kP2AuxWarp0 * 32;         // 0..127
     const int sub = vt >> 6, vr = vt & 63;
-    float vmin = INFINITY, vmax = -INFINITY, vsum = 0.f;
-    int it = 0, segn = 0, seg_first = lo;
-    bool seg_start = true;
-    for (TileIter ti(st.tile2_start, st.batch, H, st.nt2, lo, hi); ti.valid(); ti.next()) {
-      if (seg_start) {
-        const int L = st.cu[ti.b + 1] - st.cu[ti.b];
-        const float ks = fold_key_sums(ws.ksum, pass1_segments(st, ti), vt);
-        const float kb = ks / (float)L;   // mean unit key
-        if (ti.t == 0) {                  // the same in all 128 threads
-          const float n2 = warp_sum(ks * ks);
-          if (lane == 0) sred[44 + (warp - kP2AuxWarp0)] = n2;
-          named_bar_sync(4, 128);
-          if (vt == 0) {
-            const double nn = ((double)sred[44] + (double)sred[45]) + ((double)sred[46] + (double)sred[47]);
-            const double T = (double)L;
-            const float r = (float)((nn - T) / (T * (T - 1.0)));   // Eq. 4
-            ws.rbar[ti.unit()] = r;
-            if (rbar_out) rbar_out[ti.unit()] = r;
-          }
+    int vs = sub, vph = 0, segn = 0;   // V stage of this pair of warps: half tiles sub, sub + 2, ...
+    for (SegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid(); sg.next()) {
+      const int L = st.cu[sg.b + 1] - st.cu[sg.b], P = L - W;
+      const float ks = fold_key_sums(ws.ksum, pass1_segments(st, sg), vt);
+      const float kb = ks / (float)L;   // mean unit key
+      if (sg.t0 == 0) {                 // the same in all 128 threads
+        const float n2 = warp_sum(ks * ks);
+        if (lane == 0) sred[44 + (warp - kP2AuxWarp0)] = n2;
+        named_bar_sync(4, 128);
+        if (vt == 0) {
+          const double nn = ((double)sred[44] + (double)sred[45]) + ((double)sred[46] + (double)sred[47]);
+          const double T = (double)L;
+          const float r = (float)((nn - T) / (T * (T - 1.0)));   // Eq. 4
+          ws.rbar[sg.unit()] = r;
+          if (rbar_out) rbar_out[sg.unit()] = r;
         }
-        __nv_bfloat16 parts[3];
-        parts[0] = __float2bfloat16_rn(kb);
-        const float r1 = kb - __bfloat162float(parts[0]);
-        parts[1] = __float2bfloat16_rn(r1);
-        parts[2] = __float2bfloat16_rn(r1 - __bfloat162float(parts[1]));
-        if (segn > 0) {   // the previous segment's MMAs must be done with the B rows
-          if (vt == 0) mbar_wait(&bars->qfree, (segn - 1) & 1, abort);
-          named_bar_sync(4, 128);
-        }
-        {
-          unsigned char* hb = sQ + (vt >> 6) * NB * 128 + (vt & 7) * 2;
-          const int chunk = (vt & 63) >> 3;
-#pragma unroll
-          for (int e = 0; e < kExtraRows; ++e) {
-            if (e < 3 || segn == 0)
-              *reinterpret_cast<__nv_bfloat16*>(hb + sw128_offset(NQ + e, chunk)) =
-                  e < 3 ? parts[e] : __float2bfloat16_rn(0.f);
-          }
-        }
-        fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->kbready);
-        ++segn;
-        vmin = INFINITY, vmax = -INFINITY, vsum = 0.f;
-        seg_first = ti.id;
       }
-      seg_start = ti.seg_last();
+      __nv_bfloat16 parts[3];
+      parts[0] = __float2bfloat16_rn(kb);
+      const float r1 = kb - __bfloat162float(parts[0]);
+      parts[1] = __float2bfloat16_rn(r1);
+      parts[2] = __float2bfloat16_rn(r1 - __bfloat162float(parts[1]));
+      if (segn > 0) {   // the previous segment's MMAs must be done with the B rows
+        if (vt == 0) mbar_wait(&bars->qfree, (segn - 1) & 1, abort);
+        named_bar_sync(4, 128);
+      }
+      {
+        unsigned char* hb = sQ + (vt >> 6) * NB * 128 + (vt & 7) * 2;
+        const int chunk = (vt & 63) >> 3;
+#pragma unroll
+        for (int e = 0; e < kExtraRows; ++e) {
+          if (e < 3 || segn == 0)
+            *reinterpret_cast<__nv_bfloat16*>(hb + sw128_offset(NQ + e, chunk)) =
+                e < 3 ? parts[e] : __float2bfloat16_rn(0.f);
+        }
+      }
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->kbready);
+      ++segn;
+      float vmin = INFINITY, vmax = -INFINITY, vsum = 0.f;
+      float* vnorm = ws.vnorm + ppos(st, sg.layer, sg.h, sg.b, 0);
       if (use_vnorm == MIXKV_INTRINSIC_KNORM) {
         // key-norm ablation: the intrinsic term is minus the key norm, which pass 1 left as its
         // reciprocal; no V tile is loaded
-        const int P = st.cu[ti.b + 1] - st.cu[ti.b] - W;
-        const int i = ti.t * kTile + vt;
-        if (i < P) {
-          const float ki = ws.kinv[kpos(st, ti.layer, ti.h, ti.b, i)];
+        const float* kinv = ws.kinv + kpos(st, sg.layer, sg.h, sg.b, 0);
+        for (int i = sg.t0 * kTile + vt; i < min(P, sg.end() * kTile); i += kTile) {
+          const float ki = kinv[i];
           const float n = ki > 0.f ? -1.0f / ki : 0.f;
-          ws.vnorm[ppos(st, ti.layer, ti.h, ti.b, i)] = n;
+          vnorm[i] = n;
           vmin = fminf(vmin, n);
           vmax = fmaxf(vmax, n);
           vsum += n;
         }
       } else if (use_vnorm) {
-        const int P = st.cu[ti.b + 1] - st.cu[ti.b] - W;
-        const int vit = 2 * it + sub;
-        const int vs = vit % vstages, vph = (vit / vstages) & 1;
-        const bool ok = mbar_wait(&bars->vfull[vs], vph, abort);
-        const unsigned char* tile = sV + vs * kVSubBytes;
-        f32x2 ss2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
-        if (ok) {
+        for (int t = sg.t0; t < sg.end(); ++t) {
+          const bool ok = mbar_wait(&bars->vfull[vs], vph, abort);
+          const unsigned char* tile = sV + vs * kVSubBytes;
+          f32x2 ss2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};
+          if (ok) {
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
+            for (int half = 0; half < 2; ++half) {
 #pragma unroll
-            for (int c = 0; c < 8; ++c) {
-              const uint4 u =
-                  *reinterpret_cast<const uint4*>(tile + half * (kVSubBytes / 2) + sw128_offset(vr, c));
-              const uint32_t* p2 = reinterpret_cast<const uint32_t*>(&u);
+              for (int c = 0; c < 8; ++c) {
+                const uint4 u =
+                    *reinterpret_cast<const uint4*>(tile + half * (kVSubBytes / 2) + sw128_offset(vr, c));
+                const uint32_t* p2 = reinterpret_cast<const uint32_t*>(&u);
 #pragma unroll
-              for (int e = 0; e < 4; ++e) {
-                const f32x2 f2 = bf16x2_wide(p2[e]);
-                ss2[e & 1] = fma2(f2, f2, ss2[e & 1]);
+                for (int e = 0; e < 4; ++e) {
+                  const f32x2 f2 = bf16x2_wide(p2[e]);
+                  ss2[e & 1] = fma2(f2, f2, ss2[e & 1]);
+                }
               }
             }
           }
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->vempty[vs]);
-        const int i = ti.t * kTile + sub * 64 + vr;
-        if (ok && i < P) {
-          float ss[4];
-          unpack2(ss2[0], ss[0], ss[2]);
-          unpack2(ss2[1], ss[1], ss[3]);
-          const float n = sqrtf((ss[0] + ss[1]) + (ss[2] + ss[3]));
-          ws.vnorm[ppos(st, ti.layer, ti.h, ti.b, i)] = n;
-          vmin = fminf(vmin, n);
-          vmax = fmaxf(vmax, n);
-          vsum += n;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bars->vempty[vs]);
+          vs += 2;
+          if (vs >= vstages) vs -= vstages, vph ^= 1;
+          const int i = t * kTile + sub * 64 + vr;
+          if (ok && i < P) {
+            float ss[4];
+            unpack2(ss2[0], ss[0], ss[2]);
+            unpack2(ss2[1], ss[1], ss[3]);
+            const float n = sqrtf((ss[0] + ss[1]) + (ss[2] + ss[3]));
+            vnorm[i] = n;
+            vmin = fminf(vmin, n);
+            vmax = fmaxf(vmax, n);
+            vsum += n;
+          }
+          // The four warps stay within one tile of each other.  With an odd number of V stages the
+          // two pairs of warps take turns on the same stage: a pair that ran ahead would wait for
+          // a phase of vfull whose predecessor it never saw complete, and a parity wait on a
+          // barrier that is still one phase behind returns at once.
+          named_bar_sync(3, 128);
         }
       }
-      // The four warps stay within one tile of each other.  With an odd number of V stages the
-      // two pairs of warps take turns on the same stage: a pair that ran ahead would wait for
-      // a phase of vfull whose predecessor it never saw complete, and a parity wait on a
-      // barrier that is still one phase behind returns at once.
-      named_bar_sync(3, 128);
-      if (seg_start && use_vnorm) {
+      if (use_vnorm) {
         const float a = warp_min(vmin), b2 = warp_max(vmax), c2 = warp_sum(vsum);
         const int vw = warp - kP2AuxWarp0;
         if (lane == 0) {
@@ -1018,14 +1009,13 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         }
         named_bar_sync(4, 128);
         if (vt == 0) {
-          ws.vstat[seg_first] = make_float4(
+          ws.vstat[sg.id] = make_float4(
               fminf(fminf(sred[32], sred[33]), fminf(sred[34], sred[35])),
               fmaxf(fmaxf(sred[36], sred[37]), fmaxf(sred[38], sred[39])),
               (sred[40] + sred[41]) + (sred[42] + sred[43]), 0.f);
         }
         named_bar_sync(4, 128);
       }
-      ++it;
     }
   }
   tc_fence_before();

@@ -192,7 +192,8 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
     }
   } else if (warp == 1) {
     // -------------------------------------------------------------------- MMA issuer
-    if (lane == 0) {
+    {
+      const uint32_t on = elect_one();
       constexpr uint32_t idesc = umma_idesc_bf16(128, NT);
       const uint32_t a0 = umma_desc_lo(smem_u32(sA)), b0 = umma_desc_lo(smem_u32(sB));
       int it = 0, rown = 0, tile = 0;
@@ -221,16 +222,16 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
               const uint32_t oa = (uint32_t)(pa * (kPartBytes >> 4) + (ks >> 2) * (16384 >> 4) + (ks & 3) * 2);
               const uint32_t ob = (uint32_t)((ks >> 2) * (kBHalf >> 4) + (ks & 3) * 2);
               if (p == 0 && pa == 0 && ks == 0)
-                umma_bf16_lo<0>(tmem + ts * 128, a0 + oa, bs + ob, idesc);
+                umma_bf16_lo<0>(tmem + ts * 128, a0 + oa, bs + ob, idesc, on);
               else
-                umma_bf16_lo<1>(tmem + ts * 128, a0 + oa, bs + ob, idesc);
+                umma_bf16_lo<1>(tmem + ts * 128, a0 + oa, bs + ob, idesc, on);
             }
           }
-          umma_commit(&bars->bempty[s]);
+          umma_commit(&bars->bempty[s], on);
           ++it;
         }
-        umma_commit(&bars->tfull[ts]);
-        if (w.row_last()) umma_commit(&bars->afree);
+        umma_commit(&bars->tfull[ts], on);
+        if (w.row_last()) umma_commit(&bars->afree, on);
         ++tile;
       }
     }

@@ -54,12 +54,14 @@ __device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
 // limit passes or another thread of the CTA has already aborted.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort) {
   if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = global_ns();
+  unsigned long long t0 = 0;   // the clock is first read after a few hundred tries: most waits end before
   for (uint32_t it = 1;; ++it) {
     if (mbar_try(bar, parity)) return true;
     if ((it & 255u) == 0) {
       if (*abort) return false;
-      if (global_ns() - t0 > kWaitLimitNs) {
+      const unsigned long long now = global_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > kWaitLimitNs) {
         *abort = 1;
         return false;
       }
@@ -96,18 +98,9 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* tm) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
 }
 
-// Shared-memory matrix descriptor of a K-major bf16 operand stored as rows of 128 bytes with
-// the 128-byte swizzle (what a TMA box of 64 bf16 x rows writes): 8-row groups are 1024 bytes
-// apart.
-__device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)1 << 16;            // leading byte offset: unused for swizzled K-major
-  d |= (uint64_t)(1024 >> 4) << 32;  // stride byte offset between 8-row groups
-  d |= (uint64_t)1 << 46;            // descriptor version (Blackwell)
-  d |= (uint64_t)2 << 61;            // SWIZZLE_128B
-  return d;
-}
+// Shared-memory matrix descriptors are for K-major bf16 operands stored as rows of 128 bytes with the
+// 128-byte swizzle (what a TMA box of 64 bf16 x rows writes): 8-row groups 1024 bytes apart (stride byte
+// offset), leading byte offset unused, version 1 (bit 46), SWIZZLE_128B (2 in bits 61 ..).
 
 // Instruction descriptor: D f32, A and B bf16, both K-major, M x N tile.
 __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
@@ -115,39 +108,47 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
          ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t da, uint64_t db,
-                                          uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d),
-      "l"(da), "l"(db), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-// The same descriptor as two 32-bit halves: the high half is a constant, the low half is
+// A descriptor as two 32-bit halves: the high half is a constant, the low half is
 // ((address >> 4) & 0x3fff) | 1 << 16, so stepping an operand by n bytes (n a multiple of 16,
-// inside shared memory) is an integer add of n >> 4 to the low half: the issuing thread
-// builds a descriptor with one add instead of a dozen 64-bit operations.
+// inside shared memory) is an integer add of n >> 4 to the low half.
+//
+// Issuing: ONE thread issues an MMA, but the whole warp walks the tile loop and `on` (elect_one, nonzero
+// in one lane) predicates the instruction itself.  The operands of the instruction live in uniform
+// registers; under a branch of a single lane they are moved there one by one, and behind seven busy warps of
+// its scheduler that serial stream took 165 clocks per 128 x 128 x 16 step (64 of tensor time): it, not the
+// tensor cores or the epilogue, paced pass 1.  With converged control flow the compiler computes them in
+// the uniform registers in the first place.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t on;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(on));
+  return on;
+}
 constexpr uint32_t kUmmaDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint32_t umma_desc_lo(uint32_t saddr) {
   return ((saddr >> 4) & 0x3FFFu) | (1u << 16);
 }
 template <int ACC>
 __device__ __forceinline__ void umma_bf16_lo(uint32_t tmem_d, uint32_t a_lo, uint32_t b_lo,
-                                             uint32_t idesc) {
+                                             uint32_t idesc, uint32_t on) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "setp.ne.b32 p, %5, 0;\n\t"
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\t"
+      "setp.ne.b32 p, %5, 0;\n\tsetp.ne.b32 q, %6, 0;\n\t"
       "mov.b64 da, {%1, %3};\n\t"
       "mov.b64 db, {%2, %3};\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(tmem_d),
-      "r"(a_lo), "r"(b_lo), "r"(kUmmaDescHi), "r"(idesc), "n"(ACC)
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}" ::"r"(tmem_d),
+      "r"(a_lo), "r"(b_lo), "r"(kUmmaDescHi), "r"(idesc), "n"(ACC), "r"(on)
       : "memory");
 }
-// Arrives on the barrier once every MMA issued so far by this thread has completed.
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                   smem_u32(bar))
-               : "memory");
+// Arrives on the barrier once every MMA issued so far by the elected thread has completed.
+__device__ __forceinline__ void umma_commit(uint64_t* bar, uint32_t on) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(
+          smem_u32(bar)),
+      "r"(on)
+      : "memory");
 }
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -278,41 +279,41 @@ __host__ __device__ __forceinline__ int tile_owner(int t, const Split& sp) {
   return t < big ? t / (sp.q + 1) : sp.r + (t - big) / sp.q;
 }
 
-// Walks the tiles [lo, hi) of one CTA in (layer, b, h, t) order without dividing per tile.
-// Tile ids run over all layers: id = layer * nt + (tile of the layer).
-struct TileIter {
-  int id, hi, layer, b, h, t, per_head, H, batch, nt;
+// Walks the tiles [lo, hi) of one CTA segment by segment: a segment is a run of tiles t0 .. t0 + n - 1 of
+// one (layer, sequence, head), so that a role's loop over the tiles of a segment carries nothing but the
+// tile index.  Tile ids run over all layers: id = layer * nt + (tile of the layer).
+struct SegIter {
+  int id, hi, layer, b, h, t0, n, per_head, H, batch;
   const int* tile_start;
-  __device__ TileIter(const int* tile_start_, int batch_, int H_, int nt_, int lo, int hi_)
-      : id(lo), hi(hi_), H(H_), batch(batch_), nt(nt_), tile_start(tile_start_) {
-    layer = b = h = t = 0;
+  __device__ SegIter(const int* tile_start_, int batch_, int H_, int nt, int lo, int hi_)
+      : id(lo), hi(hi_), H(H_), batch(batch_), tile_start(tile_start_) {
+    layer = b = h = t0 = n = 0;
     per_head = 1;
     if (lo < hi_) {
-      layer = lo / nt_;
-      const TileCoord c = tile_coord(tile_start_, batch_, H_, lo - layer * nt_);
-      b = c.b, h = c.h, t = c.t;
+      layer = lo / nt;
+      const TileCoord c = tile_coord(tile_start_, batch_, H_, lo - layer * nt);
+      b = c.b, h = c.h, t0 = c.t;
       per_head = (tile_start_[b + 1] - tile_start_[b]) / H_;
+      n = min(per_head - t0, hi_ - lo);
     }
   }
   __device__ __forceinline__ bool valid() const { return id < hi; }
-  // (sequence, head) of the tile inside its layer, and over all layers
+  // (sequence, head) of the segment inside its layer, and over all layers
   __device__ __forceinline__ int bh() const { return b * H + h; }
   __device__ __forceinline__ int unit() const { return (layer * batch + b) * H + h; }
-  // last tile of a segment: a run of tiles of one (layer, b, h) inside this CTA's range
-  __device__ __forceinline__ bool seg_last() const { return id + 1 == hi || t + 1 == per_head; }
+  __device__ __forceinline__ int end() const { return t0 + n; }
   __device__ __forceinline__ void next() {
-    ++id;
-    if (++t == per_head) {
-      t = 0;
-      if (++h == H) {
-        h = 0;
-        if (++b == batch) {
-          b = 0;
-          ++layer;
-        }
-        if (id < hi) per_head = (tile_start[b + 1] - tile_start[b]) / H;
+    id += n;
+    t0 = 0;
+    if (++h == H) {
+      h = 0;
+      if (++b == batch) {
+        b = 0;
+        ++layer;
       }
+      per_head = (tile_start[b + 1] - tile_start[b]) / H;
     }
+    n = min(per_head, hi - id);
   }
 };
 
