@@ -86,37 +86,7 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
   return d;
 }
 
-// exp2 of both halves of t on the FMA pipe, for the share of the exponentials that the
-// special-function unit (16 results per clock and SM, the bound of both passes) cannot take:
-// t = j + f with j the nearest integer (the magic-number add leaves j in the low mantissa bits),
-// 2^f by a cubic (relative error below 7.5e-5 on [-0.5, 0.5]), j added to the exponent field.
-// t is clamped at -125 (a masked logit, -inf, gives 2^-125 instead of 0).
-__device__ __forceinline__ f32x2 ex2_poly2(f32x2 t2) {
-  float t0, t1;
-  unpack2(t2, t0, t1);
-  t2 = pack2(fmaxf(t0, -125.f), fmaxf(t1, -125.f));
-  const f32x2 y = add2(t2, pack2(12582912.f, 12582912.f));             // 1.5 * 2^23 + j
-  const f32x2 jf = add2(y, pack2(-12582912.f, -12582912.f));
-  const f32x2 f = fma2(jf, pack2(-1.f, -1.f), t2);
-  f32x2 p = fma2(pack2(0.0551716536f, 0.0551716536f), f, pack2(0.242611125f, 0.242611125f));
-  p = fma2(p, f, pack2(0.693260968f, 0.693260968f));
-  p = fma2(p, f, pack2(0.999928057f, 0.999928057f));
-  float p0, p1, y0, y1;
-  unpack2(p, p0, p1);
-  unpack2(y, y0, y1);
-  return pack2(__uint_as_float(__float_as_uint(p0) + (__float_as_uint(y0) << 23)),
-               __uint_as_float(__float_as_uint(p1) + (__float_as_uint(y1) << 23)));
-}
-// Of every 16 pairs of exponentials, kPolyPairs go through ex2_poly2, spread evenly.
-#ifndef MIXKV_POLY_PAIRS
-#define MIXKV_POLY_PAIRS 0
-#endif
-constexpr int kPolyPairs = MIXKV_POLY_PAIRS;
-__host__ __device__ constexpr bool poly_pair(int k) {
-  return ((k % 16) * kPolyPairs) % 16 < kPolyPairs && kPolyPairs > 0;
-}
-__device__ __forceinline__ f32x2 ex2_pair(f32x2 t2, const bool poly) {
-  if (poly) return ex2_poly2(t2);
+__device__ __forceinline__ f32x2 ex2_pair(f32x2 t2) {
   float a0, a1;
   unpack2(t2, a0, a1);
   return pack2(ex2(a0), ex2(a1));
@@ -153,8 +123,8 @@ constexpr int kP1RegsLaunch = 72, kP1RegsLead = P1_LEAD, kP1RegsEpi = P1_EPI, kP
 struct P1Bars {
   uint64_t full[kP1MaxStages];
   uint64_t empty[kP1MaxStages];
-  uint64_t tfull[2];
-  uint64_t tempty[2];
+  uint64_t tfull[4];
+  uint64_t tempty[4];
   uint64_t qfull;
   uint64_t qfree;
   uint32_t tmem_base;
@@ -222,29 +192,21 @@ __device__ __forceinline__ SegList pass1_segments(const SeqTable& st, const SegI
 // carries 2^±126 around it, and searching the maximum of every chunk costs a quarter of the
 // epilogue's instructions on its critical path.
 //
-// Fast path, one 32-column chunk: the sum of exp2(logit * c - m) with the standing reference.
-__device__ __forceinline__ float chunk_expsum(const uint32_t (&r)[32], const float scale_log2e,
-                                              const float m_run) {
-  const f32x2 sc2 = pack2(scale_log2e, scale_log2e), nm2 = pack2(-m_run, -m_run);
-  f32x2 za = pack2(0.f, 0.f), zb = za;
+// Fast path, 16 columns: adds exp2(logit * c - m) under the standing reference to two packed sums.
+__device__ __forceinline__ void expsum16(const uint32_t (&r)[16], const f32x2 sc2, const f32x2 nm2, f32x2& za,
+                                         f32x2& zb) {
 #pragma unroll
-  for (int j = 0; j < 32; j += 4) {
-    const f32x2 ta = fma2(pack2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])), sc2, nm2);
-    const f32x2 tb = fma2(pack2(__uint_as_float(r[j + 2]), __uint_as_float(r[j + 3])), sc2, nm2);
-    za = add2(za, ex2_pair(ta, poly_pair(j / 2)));
-    zb = add2(zb, ex2_pair(tb, poly_pair(j / 2 + 1)));
+  for (int j = 0; j < 16; j += 4) {
+    za = add2(za, ex2_pair(fma2(pack2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])), sc2, nm2)));
+    zb = add2(zb, ex2_pair(fma2(pack2(__uint_as_float(r[j + 2]), __uint_as_float(r[j + 3])), sc2, nm2)));
   }
-  float z0, z1;
-  unpack2(add2(za, zb), z0, z1);
-  return z0 + z1;
 }
-// A chunk sum at or above this means a logit about 2^99 above the reference (or no reference
-// yet): the chunk is redone on the slow path.  Below it nothing can overflow: 1024 chunks of a
-// head add up to less than 2^110.
-constexpr float kChunkSumLimit = 1e30f;
+// A tile's sum at or above this means a logit about 2^99 above the reference (or no reference yet): the tile
+// is redone on the slow path.  Below it nothing can overflow: the tiles of a head add up to less than 2^113.
+constexpr float kTileSumLimit = 1e30f;
 
-// Slow path: the chunk again from tensor memory with the causal mask and a maximum search; the
-// reference moves up to the chunk's maximum if that is larger.  Taken for the first chunk of
+// Slow path: a 32-column chunk from tensor memory with the causal mask and a maximum search; the
+// reference moves up to the chunk's maximum if that is larger.  Taken for the first tile of
 // a segment, for the tiles that need the mask, and when the fast path's sum says that the
 // reference is too low.  Every lane of the warp takes part (the load is warp-wide).  Returns
 // the new (m, z).
@@ -271,8 +233,13 @@ __device__ __noinline__ float2 softmax_chunk_ref(const uint32_t taddr, const boo
     z_run *= ex2(m_run - mn);
     m_run = mn;
   }
-  z_run += chunk_expsum(r, scale_log2e, m_run);
-  return make_float2(m_run, z_run);
+  const f32x2 sc2 = pack2(scale_log2e, scale_log2e), nm2 = pack2(-m_run, -m_run);
+  f32x2 za = pack2(0.f, 0.f), zb = za;
+  expsum16(reinterpret_cast<const uint32_t(&)[16]>(r[0]), sc2, nm2, za, zb);
+  expsum16(reinterpret_cast<const uint32_t(&)[16]>(r[16]), sc2, nm2, za, zb);
+  float z0, z1;
+  unpack2(add2(za, zb), z0, z1);
+  return make_float2(m_run, z_run + (z0 + z1));
 }
 
 // grid = g1 persistent CTAs of 28 warps: TMA, 2 idle, MMA, 16 epilogue, 8 key-statistics.  The
@@ -291,6 +258,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   const int kP1Stages = p1_stages(st.NQ);
   constexpr int kP1AuxWarps = p1_aux_warps(MB);
   constexpr int NU = MB == 2 ? 2 : 4;   // warpgroups that share a query row
+  constexpr int TS = MB == 2 ? 2 : 4;   // accumulator stages (512 columns of tensor memory)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int NQ = st.NQ, W = st.W, H = st.H;
   // The query tile holds exactly NQ rows per 64-column half.  The MMA reads MB * 128 rows: the
@@ -321,7 +289,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
       mbar_init(&bars->full[s], 1);
       mbar_init(&bars->empty[s], 1 + kP1AuxWarps);   // MMA commit + the key-statistics warps
     }
-    for (int s = 0; s < 2; ++s) {
+    for (int s = 0; s < TS; ++s) {
       mbar_init(&bars->tfull[s], 1);
       // every epilogue warp that owns query rows reads every tile; warps on padding rows (the
       // last lane quarters of the last block) neither wait nor arrive: a warp that polls a
@@ -333,7 +301,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     bars->abort = 0;
     mbar_init_fence();
   }
-  if (warp == kP1WarpMma) tmem_alloc(&bars->tmem_base, MB * 256);
+  if (warp == kP1WarpMma) tmem_alloc(&bars->tmem_base, 512);
   if (warp == kWarpTma && lane == 0) {
     tma_prefetch_desc(&tmK);
     tma_prefetch_desc(&tmQ);
@@ -414,8 +382,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
             umma_commit(&bars->tfull[ts], on);
             if (k + 1 == sg.n) umma_commit(&bars->qfree, on);
             if (++s == kP1Stages) s = 0, ph ^= 1;
-            ts ^= 1;
-            tph ^= ts ^ 1;
+            if (++ts == TS) ts = 0, tph ^= 1;
           }
         }
         if (*abort && on) raise(status, abort);
@@ -423,8 +390,8 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     }
   } else if (warp < kAuxWarp0) {
     // ------------------------------------------------------------------ epilogue
-    // All sixteen warps read every tile (two accumulator stages: the MMA of the next tile fills
-    // the other stage meanwhile).  Warpgroup wg = 0..3:
+    // All sixteen warps read every tile (the MMA of the next tiles fills the other accumulator
+    // stages meanwhile).  Warpgroup wg = 0..3:
     // MB == 2: query rows (wg / 2) * 128 .. +127, keys (wg % 2) * 64 .. +63 of the tile;
     // MB == 1: query rows 0 .. 127, keys wg * 32 .. +31.
     set_regs<kP1RegsEpi, kP1RegsLaunch>();
@@ -447,40 +414,54 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
       float m_run = -1e30f, z_run = 0.f;
       const int P = st.cu[sg.b + 1] - st.cu[sg.b] - W;
       const int t_mask = P / kTile;   // first tile that holds keys some row may not see
-      // a warp on padding rows only walks the segments, for the barriers below
+      // A tile goes in pieces of 16 columns: while one is exponentiated the next is on its way from tensor
+      // memory, so that the four warps of a scheduler, which move in step, do not all wait for their loads
+      // at the same time (G*W = 224, 28 layers of 4 x 32768 keys: 305 -> 283 us).  The first piece of the
+      // next tile is not asked for ahead: with its accumulator not ready yet this tile's would be held back
+      // (310 us).  A warp on padding rows only walks the segments, for the barriers below.
       for (int t = warp_on ? sg.t0 : sg.end(); t < sg.end(); ++t) {
         // (after an abort the waits fail at once; the loop goes on without work so that the
         // segment-end barriers below stay matched)
         if (mbar_wait(&bars->tfull[ts], tph, abort)) {
           tc_fence_after();
           const uint32_t taddr = tbase + ts * (MB * 128);
-#pragma unroll 1
-          for (int c0 = 0; c0 < NC; c0 += 32) {   // kept rolled: the body must stay in the i-cache
-            bool slow = t == sg.t0 || t >= t_mask;  // the same in every lane; the first tile sets the reference
-            float zc = 0.f;
-            if (!slow) {
-              uint32_t ra[32];
-              tmem_ld32(taddr + c0, ra);
+          const bool masked = t >= t_mask;
+          bool slow = t == sg.t0 || masked;   // the same in every lane; the first tile sets the reference
+          if (!slow) {
+            const f32x2 sc2 = pack2(scale_log2e, scale_log2e), nm2 = pack2(-m_run, -m_run);
+            f32x2 za = pack2(0.f, 0.f), zb = za;
+            uint32_t ra[16], rb[16];
+            tmem_ld16(taddr, ra);
+#pragma unroll
+            for (int c0 = 0; c0 < NC; c0 += 32) {
               tmem_ld_wait();
               tmem_ld_fence(ra);
-              zc = chunk_expsum(ra, scale_log2e, m_run);
-              slow = __any_sync(0xffffffffu, !(zc < kChunkSumLimit));
+              tmem_ld16(taddr + c0 + 16, rb);
+              expsum16(ra, sc2, nm2, za, zb);
+              tmem_ld_wait();
+              tmem_ld_fence(rb);
+              if (c0 + 32 < NC) tmem_ld16(taddr + c0 + 32, ra);
+              expsum16(rb, sc2, nm2, za, zb);
             }
-            if (slow) {
-              const float2 mz = softmax_chunk_ref(taddr + c0, t >= t_mask, t * kTile + unit * NC + c0, P + jrow,
+            float z0, z1;
+            unpack2(add2(za, zb), z0, z1);
+            slow = __any_sync(0xffffffffu, !(z0 + z1 < kTileSumLimit));
+            if (!slow) z_run += z0 + z1;
+          }
+          if (slow) {
+#pragma unroll 1
+            for (int c0 = 0; c0 < NC; c0 += 32) {
+              const float2 mz = softmax_chunk_ref(taddr + c0, masked, t * kTile + unit * NC + c0, P + jrow,
                                                   scale_log2e, m_run, z_run);
               m_run = mz.x;
               z_run = mz.y;
-            } else {
-              z_run += zc;
             }
           }
           tc_fence_before();
           __syncwarp();   // one arrival per warp: 512 single arrivals on one word cost more than a chunk
           if (lane == 0) mbar_arrive(&bars->tempty[ts]);
         }
-        ts ^= 1;
-        tph ^= ts ^ 1;
+        if (++ts == TS) ts = 0, tph ^= 1;
       }
       if (unit > 0) {
         if (segs_done > 0) named_bar_sync(8 + blk, kXThreads);   // the last hand-over was read
@@ -589,7 +570,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == kP1WarpMma) tmem_dealloc(tmem, MB * 256);
+  if (warp == kP1WarpMma) tmem_dealloc(tmem, 512);
   if (tid == 0 && bars->abort && status) atomicExch(status, MIXKV_ERR_TIMEOUT);
   // every partial result of this CTA's segments is written: pass 2 folds them per head
 }
@@ -629,14 +610,10 @@ __device__ __forceinline__ void colsum_chunk(const uint32_t (&r)[N], const float
 #pragma unroll
   for (int j = 0; j < N; j += 4) {
     const float4 nb = *reinterpret_cast<const float4*>(nb_smem + j);   // negated normalisers
-    float a0, a1, b0, b1;
-    unpack2(fma2(pack2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])), sc2, pack2(nb.x, nb.y)),
-            a0, a1);
-    unpack2(fma2(pack2(__uint_as_float(r[j + 2]), __uint_as_float(r[j + 3])), sc2,
-                 pack2(nb.z, nb.w)),
-            b0, b1);
-    acc = add2(acc, pack2(ex2(a0), ex2(a1)));
-    acc = add2(acc, pack2(ex2(b0), ex2(b1)));
+    acc = add2(acc, ex2_pair(fma2(pack2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])), sc2,
+                                  pack2(nb.x, nb.y))));
+    acc = add2(acc, ex2_pair(fma2(pack2(__uint_as_float(r[j + 2]), __uint_as_float(r[j + 3])), sc2,
+                                  pack2(nb.z, nb.w))));
   }
 }
 
