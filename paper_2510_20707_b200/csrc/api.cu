@@ -386,7 +386,7 @@ int compress_impl(const void* K, const void* V, const void* Qwin, int n_layers,
     // one kernel: mix, select, gather
     t.s_div = c.ws.s_div;
     t.rbar_in = rbar_in_opt;
-    t.s_comp_out = s_comp;
+    t.s_comp_out = s_comp_opt;   // nobody else reads the mixed scores
     t.counts_dev = head_budgets ? counts : nullptr;
     t.counts_out = head_budgets ? nullptr : counts;
     c.mark();

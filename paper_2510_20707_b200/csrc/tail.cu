@@ -1,9 +1,9 @@
 // Everything after the two K passes: the per-head scalars, pooling, the head-wise mix (Eq. 2,
 // Eq. 5), budgets, per-head top-B selection and the gather (Algorithm 1, step 2 and the TopB
-// line).  The fixed-budget layer call runs all of it in ONE kernel, k_tail: a cluster of eight
-// CTAs per (sequence, head) mixes the scores of its slice, finds the selection threshold by
-// radix passes whose histograms are combined through distributed shared memory, compacts the
-// kept positions in ascending order and copies the kept K / V rows.
+// line).  The fixed-budget layer call runs all of it in ONE kernel, k_tail: one CTA or a cluster of
+// them per (sequence, head) mixes the scores of its slice, finds the selection threshold (binned counts,
+// combined through distributed shared memory), compacts the kept positions in ascending order and
+// copies the kept K / V rows.
 #include <cooperative_groups.h>
 
 #include "tc_common.cuh"
@@ -221,7 +221,7 @@ k_mixpool(const SeqTable st, const Workspace ws, const float* __restrict__ s_div
   }
 }
 
-// ------------------------------------------------------------------- radix selection
+// ------------------------------------------------------------------- threshold search
 // Order-preserving map float -> uint32 (larger float, larger key); -0 is folded into +0 so
 // that equal floats have equal keys.
 __device__ __forceinline__ unsigned order_key(float f) {
@@ -230,208 +230,225 @@ __device__ __forceinline__ unsigned order_key(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Adds the 32 digits of a warp (0xffffffff = none) to a shared-memory histogram.  The digit of
-// the lowest lane, then the digit of the lowest lane left, are counted with one vote and one add
-// each (the first passes of a selection see one or two digits almost everywhere); what is left
-// after that is spread over the bins and is added lane by lane.
-__device__ __forceinline__ void count_digits(int* hist, const unsigned digit, const int lane) {
-  unsigned left = 0xffffffffu;
+constexpr int kSelBinBits = 11, kSelBins = 1 << kSelBinBits;
+constexpr int kSelListCap = 256;   // candidates ranked directly
+
+struct SelSmem {
+  int hist[2][kSelBins];
+  unsigned list[kSelListCap];    // this CTA's candidates
+  unsigned all[kSelListCap];     // those of every CTA of the cluster, in rank order
+  unsigned wlo[32], whi[32];
+  unsigned range[2];             // this CTA's smallest and largest key
+  int scan[32];
+  int off[9];                    // cluster: where each rank's candidates start in `all`
+  int nlist, gt, eq;             // this CTA's candidates, its keys above them, its keys equal to the threshold
+  int bin, remaining, count;     // bin that holds the threshold, keys still needed from it, keys in it
+  unsigned tau;
+  int need_eq, eq_total;
+  int gt_before, eq_before;
+};
+
+struct Threshold {
+  unsigned tau;              // the want-th largest key
+  int need_eq, eq_total;     // keys equal to it that are wanted / that there are
+  int gt_before, eq_before;  // keys above it and equal to it in the CTAs of lower rank
+};
+
+// Sum of v over the threads after the caller (suffix = true) or before it; every thread of the CTA takes
+// part.  Ends with every warp past its reads of `scan` only after the caller's next CTA barrier.
+template <int T, bool SUFFIX>
+__device__ __forceinline__ int block_scan(const int v, int* scan, const int lane, const int warp) {
+  int incl = v;
 #pragma unroll
-  for (int round = 0; round < 2; ++round) {
-    const int src = __ffs(left) - 1;                       // lowest lane not counted yet
-    const unsigned d = __shfl_sync(0xffffffffu, digit, src);
-    const unsigned same = __ballot_sync(0xffffffffu, digit == d) & left;
-    if (lane == src && d != 0xffffffffu) atomicAdd(&hist[d], __popc(same));
-    left &= ~same;
-    if (left == 0) return;                                 // uniform across the warp
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = SUFFIX ? __shfl_down_sync(0xffffffffu, incl, o) : __shfl_up_sync(0xffffffffu, incl, o);
+    if (SUFFIX ? lane + o < 32 : lane >= o) incl += x;
   }
-  if (((left >> lane) & 1u) && digit != 0xffffffffu) atomicAdd(&hist[digit], 1);
+  if (lane == (SUFFIX ? 0 : 31)) scan[warp] = incl;
+  __syncthreads();
+  const bool other = lane < T / 32 && (SUFFIX ? lane > warp : lane < warp);
+  return incl - v + __reduce_add_sync(0xffffffffu, other ? scan[lane] : 0);
 }
 
-// Adds eight digits per lane (0xffffffff = none) to a shared-memory histogram.  A lane first counts
-// how many of its own digits equal its first live one (the leading digits of a selection put
-// almost every key of a CTA into two or three bins: one add per key on those words would
-// serialise the CTA).  Then, as in count_digits, the first digit of the lowest lane and that of
-// the lowest lane left are added with one vote, one warp sum and one add each; the lanes left
-// after that add their own count, and the digits that differ from a lane's first go in one by
-// one.
-__device__ __forceinline__ void count_digits8(int* hist, const unsigned (&dg)[8], const int lane) {
-  unsigned d0 = 0xffffffffu;
-#pragma unroll
-  for (int e = 0; e < 8; ++e)
-    if (d0 == 0xffffffffu) d0 = dg[e];
-  int c0 = 0;
-#pragma unroll
-  for (int e = 0; e < 8; ++e) c0 += (dg[e] == d0);
-  unsigned left = 0xffffffffu;
-#pragma unroll
-  for (int round = 0; round < 2; ++round) {
-    const int src = __ffs(left) - 1;                       // lowest lane not counted yet
-    const unsigned d = __shfl_sync(0xffffffffu, d0, src);
-    const bool mine = d0 == d && ((left >> lane) & 1u);
-    const unsigned same = __ballot_sync(0xffffffffu, mine);
-    const int tot = __reduce_add_sync(0xffffffffu, mine ? c0 : 0);
-    if (lane == src && d != 0xffffffffu) atomicAdd(&hist[d], tot);
-    left &= ~same;
-    if (left == 0) break;                                  // uniform across the warp
-  }
-  if (((left >> lane) & 1u) && d0 != 0xffffffffu) atomicAdd(&hist[d0], c0);
-#pragma unroll
-  for (int e = 0; e < 8; ++e)
-    if (dg[e] != 0xffffffffu && dg[e] != d0) atomicAdd(&hist[dg[e]], 1);
-}
-
-// Threshold of the `want` largest keys of a set spread over the CTAs of a cluster (one CTA: a
-// cluster of one): the want-th largest key and how many keys equal to it are still needed.  All
-// threads of all CTAs take part; key_at(e), e < total, gives the keys of this CTA (any order).
-// A first sweep finds the smallest and the largest key: the bits they share are the same in
-// every key and are skipped, so the first digit pass already sees digits that differ (scores of
-// one sequence share sign and most of the exponent; counting those bits would send every warp
-// to the same one or two bins).  Then digit passes of up to 8 bits, most significant first:
-// every CTA counts its keys, the histograms are added up through distributed shared memory
-// after a cluster barrier and every CTA finds the digit itself.  The first pass leaves one bin
-// to search; when its keys fit `list` (list_cap entries of shared memory) the second pass
-// copies this CTA's share of them there while it counts, and the later passes read the list
-// instead of all keys.  hist: 2 x 256 ints of shared memory, zeroed here.  Returns through
-// tau / need_eq (same in every thread of the cluster).
-template <typename KeyAt>
-__device__ __forceinline__ void radix_threshold(const KeyAt& key_at, const int total, const int want,
-                                                cg::cluster_group& cluster, int (*hist)[256],
-                                                unsigned* list, const int list_cap, unsigned* tau,
-                                                int* need_eq) {
-  __shared__ unsigned s_prefix, s_lo[32], s_hi[32], s_range[2];
-  __shared__ int s_remaining, s_cand, s_fill, htot[256];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = (blockDim.x + 31) >> 5;
-  const int cs = (int)cluster.num_blocks();
-  for (int t = threadIdx.x; t < 512; t += blockDim.x) hist[t >> 8][t & 255] = 0;
-  unsigned lo = 0xffffffffu, hi = 0u;
-  for (int e = threadIdx.x; e < total; e += blockDim.x) {
-    const unsigned key = key_at(e);
-    lo = min(lo, key);
-    hi = max(hi, key);
-  }
+// Threshold of the `want` largest keys (1 <= want < number of keys) of a set spread over the CTAs of a
+// cluster (cs == 1: one CTA).  All T threads of all CTAs take part; key_at(j), j < n, gives this CTA's keys,
+// lo / hi are the smallest and largest of those this thread has seen (all of them together: the CTA's).
+//
+// The keys are binned linearly between the smallest and the largest of all: 2048 bins over the range in
+// use put the keys of a head, which share sign and most of their exponent, into hundreds of bins, so the
+// counting is one shared-memory add per key without contention, and the bin of the threshold holds a few
+// dozen keys, which are listed and ranked against each other.  One sweep to count, one to list, where digits of
+// the raw key bits took two to four sweeps and as many exchanges across the cluster.  A bin with more keys
+// than the list takes is binned again (three rounds reach single key values), so any distribution, all-equal
+// keys included, ends after a bounded number of sweeps.  sm.hist must be zero on entry (visible to the CTA).
+template <int T, typename KeyAt>
+__device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const int n, const int want,
+                                                      unsigned lo, unsigned hi, SelSmem& sm,
+                                                      cg::cluster_group& cluster, const int cs,
+                                                      const int crank) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  constexpr int NW = T / 32, PER = kSelBins / T;
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
-  if (lane == 0) s_lo[warp] = lo, s_hi[warp] = hi;
+  if (lane == 0) sm.wlo[warp] = lo, sm.whi[warp] = hi;
+  if (tid == 0) sm.nlist = 0, sm.gt = 0, sm.eq = 0;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 0; w < nwarps; ++w) lo = min(lo, s_lo[w]), hi = max(hi, s_hi[w]);
-    s_range[0] = lo, s_range[1] = hi;
-  }
-  cluster.sync();
-  lo = 0xffffffffu, hi = 0u;
-  for (int r = 0; r < cs; ++r) {
-    const unsigned* rr = cluster.map_shared_rank(&s_range[0], r);
-    lo = min(lo, rr[0]);
-    hi = max(hi, rr[1]);
-  }
-  const unsigned diff = lo ^ hi;
-  int top = (hi >= lo && diff) ? 32 - __clz(diff) : 0;   // the low `top` bits differ between keys
-  unsigned mask = top == 32 ? 0u : ~((1u << top) - 1u);
-  unsigned prefix = hi & mask;
-  int remaining = want;
-  int n_list = -1;        // >= 0: this CTA's candidates are in `list`
-  bool build = false;     // this pass copies the candidates to `list`
-  for (int pass = 0; top > 0; ++pass) {
-    const int bits = min(8, top), shift = top - bits, buf = pass & 1;
-    const unsigned dmask = (1u << bits) - 1u;
-    if (threadIdx.x == 0) s_prefix = prefix, s_remaining = remaining, s_cand = 0, s_fill = 0;
-    __syncthreads();
-    if (n_list >= 0) {
-      for (int e0 = 0; e0 < n_list; e0 += blockDim.x) {   // uniform trip count: full-warp votes
-        const int e = e0 + threadIdx.x;
-        unsigned digit = 0xffffffffu;
-        if (e < n_list) {
-          const unsigned key = list[e];
-          if ((key & mask) == prefix) digit = (key >> shift) & dmask;
-        }
-        count_digits(hist[buf], digit, lane);
-      }
-    } else {
-      for (int e0 = 0; e0 < total; e0 += blockDim.x) {   // uniform trip count: full-warp votes
-        const int e = e0 + threadIdx.x;
-        unsigned digit = 0xffffffffu, key = 0u;
-        if (e < total) {
-          key = key_at(e);
-          if ((key & mask) == prefix) digit = (key >> shift) & dmask;
-        }
-        count_digits(hist[buf], digit, lane);
-        if (build) {   // one shared-memory add per warp reserves the slots of its candidates
-          const unsigned m = __ballot_sync(0xffffffffu, digit != 0xffffffffu);
-          if (m) {
-            const int leader = __ffs(m) - 1;
-            int base = 0;
-            if (lane == leader) base = atomicAdd(&s_fill, __popc(m));
-            base = __shfl_sync(0xffffffffu, base, leader);
-            if (digit != 0xffffffffu) list[base + __popc(m & ((1u << lane) - 1u))] = key;
-          }
-        }
-      }
-    }
+  lo = __reduce_min_sync(0xffffffffu, lane < NW ? sm.wlo[lane] : 0xffffffffu);
+  hi = __reduce_max_sync(0xffffffffu, lane < NW ? sm.whi[lane] : 0u);
+  if (cs > 1) {
+    if (tid == 0) sm.range[0] = lo, sm.range[1] = hi;
     cluster.sync();
-    if (threadIdx.x < 256) {
-      int tot = 0;
-      for (int r = 0; r < cs; ++r) tot += *cluster.map_shared_rank(&hist[buf][threadIdx.x], r);
-      htot[threadIdx.x] = tot;
-      hist[buf ^ 1][threadIdx.x] = 0;   // every CTA is past its reads of the other buffer
+    lo = 0xffffffffu, hi = 0u;
+    if (lane < cs) {
+      const uint2 r = *reinterpret_cast<const uint2*>(cluster.map_shared_rank(&sm.range[0], lane));
+      lo = r.x, hi = r.y;
     }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      // lane l owns bins 8l .. 8l+7; `above` = keys in higher bins
-      int h8[8], mine = 0;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) h8[k] = htot[8 * lane + k], mine += h8[k];
-      // suffix sum over lanes: keys in the bins of higher lanes
-      int incl = mine;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int v = __shfl_down_sync(0xffffffffu, incl, o);
-        if (lane + o < 32) incl += v;
-      }
-      int above = incl - mine;
-#pragma unroll
-      for (int k = 7; k >= 0; --k) {
-        if (above < remaining && remaining <= above + h8[k]) {
-          s_prefix = prefix | ((unsigned)(8 * lane + k) << shift);
-          s_remaining = remaining - above;
-          s_cand = h8[k];
-        }
-        above += h8[k];
-      }
-    }
-    __syncthreads();
-    prefix = s_prefix;
-    remaining = s_remaining;
-    mask |= dmask << shift;
-    top = shift;
-    if (build) {
-      n_list = s_fill;   // the list holds this CTA's keys under the prefix before this pass; the
-      build = false;     // next passes narrow the prefix inside it
-    } else if (n_list < 0 && pass == 0 && s_cand <= list_cap) {
-      build = true;
-    }
-    __syncthreads();
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
   }
-  *tau = prefix;
-  *need_eq = remaining;
+  unsigned base = lo, span = hi - lo;   // the candidates are the keys in [base, base + span]
+  int shift = span ? max(0, 32 - __clz(span) - kSelBinBits) : 0;
+  int remaining = want;
+  for (int round = 0;; ++round) {
+    int* hist = sm.hist[round & 1];
+    for (int j = tid; j < n; j += T) {
+      const unsigned d = key_at(j) - base;
+      if (d <= span) atomicAdd(&hist[d >> shift], 1);
+    }
+    if (cs > 1) cluster.sync();
+    else __syncthreads();
+    // thread t owns bins PER t .. PER t + PER - 1 (of all CTAs); `above` = keys in higher bins
+    int h[PER], mine = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) h[k] = 0;
+    for (int r = 0; r < cs; ++r) {
+      const int* src = cs > 1 ? cluster.map_shared_rank(&hist[PER * tid], r) : &hist[PER * tid];
+#pragma unroll
+      for (int k = 0; k < PER; k += 2) {
+        const int2 v = *reinterpret_cast<const int2*>(src + k);
+        h[k] += v.x, h[k + 1] += v.y;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+      mine += h[k];
+      sm.hist[(round & 1) ^ 1][PER * tid + k] = 0;   // every CTA is past its reads of the other buffer
+    }
+    int above = block_scan<T, true>(mine, sm.scan, lane, warp);
+    if (above < remaining && remaining <= above + mine) {
+#pragma unroll
+      for (int k = PER - 1; k >= 0; --k) {
+        if (above < remaining && remaining <= above + h[k]) {
+          sm.bin = PER * tid + k;
+          sm.remaining = remaining - above;
+          sm.count = h[k];
+        }
+        above += h[k];
+      }
+    }
+    __syncthreads();
+    base += (unsigned)sm.bin << shift;
+    remaining = sm.remaining;
+    span = (1u << shift) - 1u;
+    if (shift == 0 || sm.count <= kSelListCap) break;
+    shift = max(0, shift - kSelBinBits);
+  }
+  const int count = sm.count;
+  Threshold th;
+  th.gt_before = th.eq_before = 0;
+  if (shift == 0) {   // the bin is one key value
+    th.tau = base, th.need_eq = remaining, th.eq_total = count;
+    if (cs > 1) {
+      int gt = 0, eq = 0;
+      for (int j = tid; j < n; j += T) {
+        const unsigned key = key_at(j);
+        gt += key > base;
+        eq += key == base;
+      }
+      gt = __reduce_add_sync(0xffffffffu, gt);
+      eq = __reduce_add_sync(0xffffffffu, eq);
+      if (lane == 0) atomicAdd(&sm.gt, gt), atomicAdd(&sm.eq, eq);
+      cluster.sync();
+      const bool below = lane < crank;
+      th.gt_before = __reduce_add_sync(0xffffffffu, below ? *cluster.map_shared_rank(&sm.gt, lane) : 0);
+      th.eq_before = __reduce_add_sync(0xffffffffu, below ? *cluster.map_shared_rank(&sm.eq, lane) : 0);
+    }
+    return th;
+  }
+  // list the candidates; the keys above them are wanted in any case
+  int gt = 0;
+  for (int j = tid; j < n; j += T) {
+    const unsigned key = key_at(j);
+    if (key >= base) {
+      if (key - base <= span) sm.list[atomicAdd(&sm.nlist, 1)] = key;
+      else ++gt;
+    }
+  }
+  const unsigned* all = sm.list;
+  if (cs > 1) {
+    gt = __reduce_add_sync(0xffffffffu, gt);
+    if (lane == 0) atomicAdd(&sm.gt, gt);
+    cluster.sync();
+    if (warp < cs) {   // warp r copies rank r's candidates behind those of the lower ranks
+      const int len = lane < cs ? *cluster.map_shared_rank(&sm.nlist, lane) : 0;
+      const int start = __reduce_add_sync(0xffffffffu, lane < warp ? len : 0);
+      const int mylen = __shfl_sync(0xffffffffu, len, warp);
+      const unsigned* src = cluster.map_shared_rank(&sm.list[0], warp);
+      for (int k = lane; k < mylen; k += 32) sm.all[start + k] = src[k];
+      if (lane == 0) sm.off[warp] = start;
+    }
+    th.gt_before =
+        __reduce_add_sync(0xffffffffu, lane < crank ? *cluster.map_shared_rank(&sm.gt, lane) : 0);
+    all = sm.all;
+  }
+  __syncthreads();
+  for (int k = tid; k < count; k += T) {
+    const unsigned key = all[k];
+    int g = 0, e = 0;
+#pragma unroll 4
+    for (int x = 0; x < count; ++x) {
+      const unsigned y = all[x];
+      g += y > key;
+      e += y == key;
+    }
+    if (g < remaining && remaining <= g + e) sm.tau = key, sm.need_eq = remaining - g, sm.eq_total = e;
+  }
+  __syncthreads();
+  th.tau = sm.tau, th.need_eq = sm.need_eq, th.eq_total = sm.eq_total;
+  if (cs > 1) {
+    const int below = sm.off[crank];
+    int g = 0, e = 0;
+    for (int x = lane; x < below; x += 32) {
+      g += all[x] > th.tau;
+      e += all[x] == th.tau;
+    }
+    th.gt_before += __reduce_add_sync(0xffffffffu, g);
+    th.eq_before = __reduce_add_sync(0xffffffffu, e);
+  }
+  return th;
 }
 
 constexpr int kBudgetCluster = 8;
+
+constexpr int kBudgetThreads = 1024;
 
 // Head budgets of one sequence under the adaptive rule (see mixkv.h).  One CTA per (sequence,
 // layer) when the call has many of them, else a cluster of kBudgetCluster CTAs, each with a
 // slice of the positions of every head.  A CTA turns its H * n pooled scores into
 // order-preserving keys once and keeps them in shared memory when they fit (cache_cap keys);
-// otherwise every pass reads them from global memory.
-__global__ void __launch_bounds__(1024)
+// otherwise every sweep reads them from global memory.
+__global__ void __launch_bounds__(kBudgetThreads)
 k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ counts,
-         const int Bp, const int floor_slots, const int cache_cap, const int list_cap) {
-  extern __shared__ unsigned bkeys[];   // [cache_cap] keys, then [list_cap] candidates
-  __shared__ int hist[2][256];
+         const int Bp, const int floor_slots, const int cache_cap) {
+  extern __shared__ unsigned bkeys[];   // [cache_cap] keys
+  __shared__ __align__(16) SelSmem sm;
   __shared__ int s_gt[64], s_eq[64], t_gt[64], t_eq[64];
   cg::cluster_group cluster = cg::this_cluster();
   const int cs = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
+  const int tid = threadIdx.x, lane = tid & 31;
   pdl_launch_dependents();
+  for (int t = tid; t < 2 * kSelBins; t += kBudgetThreads) (&sm.hist[0][0])[t] = 0;
+  if (tid < 64) s_gt[tid] = 0, s_eq[tid] = 0;
   pdl_wait();
   const int b = blockIdx.x / cs, layer = blockIdx.y, H = st.H;
   counts += (size_t)layer * st.batch * H;
@@ -441,9 +458,9 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
   if (N > total) N = total;
   const float* base = scores + ppos(st, layer, 0, b, 0);
   const size_t stride = (size_t)st.Ptot;
-  if (N <= 0) {   // the same in every CTA of the cluster
+  if (N <= 0 || N == total) {   // nothing to share, or everything: the same in every CTA of the cluster
     if (crank == 0)
-      for (int h = threadIdx.x; h < H; h += blockDim.x) counts[b * H + h] = min(floor_slots, P);
+      for (int h = tid; h < H; h += kBudgetThreads) counts[b * H + h] = N <= 0 ? min(floor_slots, P) : P;
     return;
   }
   // this CTA's slice of every head: positions [p0, p0 + n)
@@ -451,54 +468,55 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
   const int p0 = min(crank * chunk, P), n = min(chunk, P - p0);
   const int local = H * n;
   const bool cached = local <= cache_cap;
-  if (cached) {
-    for (int h = 0; h < H; ++h) {
-      const float* row = base + (size_t)h * stride + p0;
-      for (int i0 = 0; i0 < n; i0 += 8 * blockDim.x) {   // eight loads in flight per thread
-        float v[8];
+  unsigned lo = 0xffffffffu, hi = 0u;
+  for (int h = 0; h < H; ++h) {
+    const float* row = base + (size_t)h * stride + p0;
+    for (int i0 = 0; i0 < n; i0 += 8 * kBudgetThreads) {   // eight loads in flight per thread
+      float v[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int i = i0 + k * blockDim.x + threadIdx.x;
-          v[k] = i < n ? row[i] : 0.f;
-        }
+      for (int k = 0; k < 8; ++k) {
+        const int i = i0 + k * kBudgetThreads + tid;
+        v[k] = i < n ? row[i] : 0.f;
+      }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int i = i0 + k * blockDim.x + threadIdx.x;
-          if (i < n) bkeys[h * n + i] = order_key(v[k]);
+      for (int k = 0; k < 8; ++k) {
+        const int i = i0 + k * kBudgetThreads + tid;
+        if (i < n) {
+          const unsigned key = order_key(v[k]);
+          if (cached) bkeys[h * n + i] = key;
+          lo = min(lo, key);
+          hi = max(hi, key);
         }
       }
     }
-    __syncthreads();
   }
+  __syncthreads();
   auto key_at = [&](const int e) -> unsigned {
     if (cached) return bkeys[e];
     const int h = e / n;
     return order_key(base[(size_t)h * stride + p0 + (e - h * n)]);
   };
-  unsigned tau;
-  int need_eq;
-  radix_threshold(key_at, local, (int)N, cluster, hist, bkeys + cache_cap, list_cap, &tau, &need_eq);
-  for (int h = threadIdx.x; h < H; h += blockDim.x) s_gt[h] = 0, s_eq[h] = 0;
-  __syncthreads();
+  const Threshold th =
+      threshold_search<kBudgetThreads>(key_at, local, (int)N, lo, hi, sm, cluster, cs, crank);
   for (int h = 0; h < H; ++h) {
     int gt = 0, eq = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    for (int i = tid; i < n; i += kBudgetThreads) {
       const unsigned key = key_at(h * n + i);
-      gt += key > tau;
-      eq += key == tau;
+      gt += key > th.tau;
+      eq += key == th.tau;
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      gt += __shfl_xor_sync(0xffffffffu, gt, o);
-      eq += __shfl_xor_sync(0xffffffffu, eq, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
+    gt = __reduce_add_sync(0xffffffffu, gt);
+    eq = __reduce_add_sync(0xffffffffu, eq);
+    if (lane == 0 && (gt | eq)) {
       atomicAdd(&s_gt[h], gt);
       atomicAdd(&s_eq[h], eq);
     }
   }
-  cluster.sync();   // every CTA's per-head counts are complete
+  // every CTA's per-head counts are complete
+  if (cs > 1) cluster.sync();
+  else __syncthreads();
   if (crank == 0) {
-    for (int h = threadIdx.x; h < H; h += blockDim.x) {
+    for (int h = tid; h < H; h += kBudgetThreads) {
       int g = 0, q = 0;
       for (int r = 0; r < cs; ++r) {
         g += *cluster.map_shared_rank(&s_gt[h], r);
@@ -507,8 +525,8 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
       t_gt[h] = g, t_eq[h] = q;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      int rem = need_eq;  // equal-to-threshold elements go to the lower (head, position) first
+    if (tid == 0) {
+      int rem = th.need_eq;  // equal-to-threshold elements go to the lower (head, position) first
       for (int h = 0; h < H; ++h) {
         const int take = min(t_eq[h], rem);
         rem -= take;
@@ -516,21 +534,25 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
       }
     }
   }
-  cluster.sync();   // the peers' shared memory stays alive until rank 0 has read it
+  if (cs > 1) cluster.sync();   // the peers' shared memory stays alive until rank 0 has read it
+}
+
+// Positions per CTA when cs CTAs share the P candidates of a head: whole words of 32.
+__host__ __device__ __forceinline__ int tail_chunk(const int P, const int cs) {
+  return (((P + cs - 1) / cs) + 31) & ~31;
 }
 
 // ------------------------------------------------------------------------------ tail
-constexpr int kTailCluster = 8;
-constexpr int kTailThreads = 512;
+constexpr int kTailMaxCluster = 8;
 constexpr int kTailCacheCap = 16384;       // positions a CTA of a cluster keeps in shared memory
 constexpr int kTailCacheCapSolo = 40960;   // positions a CTA that owns a whole head keeps
-constexpr int kTailListCap = 2048;         // keys of the threshold bin a lone CTA lists after two digits
+constexpr int kTailRowCap = 1024;          // selected rows of a CTA listed in shared memory for the gather
 
 struct TailKernelArgs {
   const float* scores;        // select on these (FUSED == false)
   const float* s_div;         // FUSED: parts of the mix
   const float* rbar_in;
-  float* s_comp_out;          // FUSED: mixed scores are written here
+  float* s_comp_out;          // FUSED: mixed scores are written here (nullptr: nobody wants them)
   const int* counts_dev;      // adaptive budgets; nullptr = fixed
   int* counts_out;
   int* idx;
@@ -558,24 +580,20 @@ __device__ __forceinline__ int fixed_offset(const SeqTable& st, int bh, int Bp) 
   return off;
 }
 
-// Shared-memory slot of local position j: one pad word per 32 keeps both the strided walk
-// (thread t, t + 512, ...) and the contiguous runs of the compaction free of bank conflicts.
-__device__ __forceinline__ int kslot(int j) { return j + (j >> 5); }
-
-// T threads per CTA; the cluster size (1 or kTailCluster CTAs per (layer, sequence, head)) is read
-// from the launch: many independent heads fill the GPU with one CTA each and need no cluster
-// traffic at all, a call with few heads spreads each head over a cluster.
+// T threads per CTA, cs CTAs (a cluster, read from the launch) per (layer, sequence, head): see tail_shape.
+//
+// Latency bound: a unit is a chain of short phases.  Mix (or load) the slice's scores into shared memory as
+// keys; threshold (threshold_search); one vote per 32 positions turns the keys into a bitmap whose prefix sums
+// place every kept position; gather.  28 layers x 4 heads x 32736 candidates: 52 -> see DESIGN's table; 896 heads of
+// 2 to 7 thousand candidates (selection and gather only): 114 us with one 1024-thread CTA per head.
 template <bool FUSED, int T>
-__global__ void __launch_bounds__(T, T == 512 ? 2 : 1)
+__global__ void __launch_bounds__(T, 1024 / T)
 k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   extern __shared__ __align__(16) unsigned char tail_smem[];
-  __shared__ int hist[2][256];
-  __shared__ int s_scan[32][2];
-  __shared__ __align__(8) int s_tot[2];
-  __shared__ int s_sel[3];      // digit, remaining, keys in the digit's bin
-  __shared__ int s_nlist;
-  __shared__ int s_off;
+  __shared__ __align__(16) SelSmem sm;
+  __shared__ int s_off, s_want;
   __shared__ float sc[8];
+  __shared__ int s_rows[kTailRowCap];
   cg::cluster_group cluster = cg::this_cluster();
   const int crank = (int)cluster.block_rank();
   const int cs = (int)cluster.num_blocks();
@@ -591,24 +609,27 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   int* counts_out = a.counts_out ? a.counts_out + (size_t)layer * BH : nullptr;
   int* idx_offsets = a.idx_offsets + (size_t)layer * (BH + 1);
   int* out_row_offsets = a.out_row_offsets ? a.out_row_offsets + (size_t)layer * (BH + 1) : nullptr;
-  // slice of this CTA: positions [c0, c0 + n)
-  const int chunk = (P + cs - 1) / cs;
-  const int R = (chunk + T - 1) / T;   // positions per thread
+  // slice of this CTA: positions [c0, c0 + n), whole words of 32 positions
+  const int chunk = tail_chunk(P, cs);
   const int c0 = min(crank * chunk, P);
   const int n = min(chunk, P - c0);
-  unsigned* skeys = reinterpret_cast<unsigned*>(tail_smem);            // [kslot(chunk) + 1]
-  float* sraw = reinterpret_cast<float*>(skeys + kslot(chunk) + 1);    // FUSED: [8 T + 64] stage; else [kTailListCap]
+  const int nwords = (n + 31) >> 5;
+  unsigned* words = reinterpret_cast<unsigned*>(tail_smem);            // [chunk / 32] bitmap of kept positions
+  unsigned* eqw = words + (chunk >> 5);                                // [chunk / 32] positions equal to the threshold
+  unsigned* skeys = eqw + (chunk >> 5);                                // [chunk] when cached
+  float* sraw = reinterpret_cast<float*>(skeys + chunk);               // FUSED: [8 T + 64] pooling stage
 
   pdl_launch_dependents();
+  for (int t = tid; t < 2 * kSelBins; t += T) (&sm.hist[0][0])[t] = 0;
   pdl_wait();
 
   if (a.status_clear && blockIdx.x == 0 && tid == 0) *a.status_clear = 0;
   // ---- budget and output offsets of this (b, h)
-  if (tid < 32) {
+  if (warp == 0) {
     int off = 0, cnt;
     if (counts_dev) {
       for (int t = lane; t < bh; t += 32) off += counts_dev[t];
-      for (int o = 16; o > 0; o >>= 1) off += __shfl_xor_sync(0xffffffffu, off, o);
+      off = __reduce_add_sync(0xffffffffu, off);
       cnt = counts_dev[bh];
     } else {
       off = fixed_offset(st, bh, a.Bp);
@@ -616,8 +637,7 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
     }
     if (lane == 0) {
       s_off = off;
-      s_nlist = 0;
-      s_sel[1] = cnt;
+      s_want = cnt;
       if (crank == 0) {
         idx_offsets[bh] = off;
         if (counts_out) counts_out[bh] = cnt;
@@ -629,10 +649,8 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
       }
     }
   }
-  for (int t = tid; t < 256; t += T) hist[0][t] = 0;   // visible after the next CTA barrier
-  const float* src = a.scores;
   const bool cached = FUSED || a.cached;
-  float held[8];   // FUSED, R <= 8: mixed scores kept until the selection is done
+  unsigned klo = 0xffffffffu, khi = 0u;   // smallest and largest key this thread has made
   if (FUSED) {
     // ---- pooling and mix of this slice (Eq. 2, Eq. 5) in blocks of 8 T consecutive positions:
     // thread t takes positions t, t + T, ... of the block
@@ -683,251 +701,127 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
       for (int u = 0; u < a.mp.pool_k; ++u) {
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          const int jb = min(e * T + tid, nb - 1);
-          const float w = sraw[jb + u];
-          ex[e] = avg ? ex[e] + w : fmaxf(ex[e], w);
+          if (e * T < nb) {   // the same in every thread
+            const float w = sraw[min(e * T + tid, nb - 1) + u];
+            ex[e] = avg ? ex[e] + w : fmaxf(ex[e], w);
+          }
         }
       }
-      unsigned top[8];   // leading digit of the block's keys: the first digit pass, taken here
 #pragma unroll
       for (int e = 0; e < 8; ++e) {
         const int jb = e * T + tid;
-        held[e] = 0.f;
-        top[e] = 0xffffffffu;
         if (jb < nb) {
-          held[e] = mix_one(avg ? ex[e] * invk : ex[e], vn[e], dv[e], sc, a.mp.use_vnorm,
-                            a.mp.mix_mode);
-          const unsigned key = order_key(held[e]);
-          skeys[kslot(j0 + jb)] = key;
-          top[e] = key >> 24;
-          if (R > 8) a.s_comp_out[poff + c0 + j0 + jb] = held[e];
+          const float s = mix_one(avg ? ex[e] * invk : ex[e], vn[e], dv[e], sc, a.mp.use_vnorm, a.mp.mix_mode);
+          const unsigned key = order_key(s);
+          skeys[j0 + jb] = key;
+          klo = min(klo, key);
+          khi = max(khi, key);
+          if (a.s_comp_out) a.s_comp_out[poff + c0 + j0 + jb] = s;
         }
       }
-      count_digits8(hist[0], top, lane);
     }
-    src = a.s_comp_out;
-  } else if (a.cached) {
-    for (int j = tid; j < n; j += T) skeys[kslot(j)] = order_key(src[poff + c0 + j]);
+  } else {
+    for (int j0 = 0; j0 < n; j0 += 4 * T) {   // four loads in flight per thread
+      float v[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int j = j0 + e * T + tid;
+        v[e] = j < n ? a.scores[poff + c0 + j] : 0.f;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int j = j0 + e * T + tid;
+        if (j < n) {
+          const unsigned key = order_key(v[e]);
+          if (cached) skeys[j] = key;
+          klo = min(klo, key);
+          khi = max(khi, key);
+        }
+      }
+    }
   }
   __syncthreads();
-  const int want = s_sel[1];
-  int* out = a.idx + (size_t)layer * a.idx_cap + s_off;
-  auto key_at = [&](int j) -> unsigned {
-    return cached ? skeys[kslot(j)] : order_key(src[poff + c0 + j]);
-  };
+  const int want = s_want;
+  auto key_at = [&](int j) -> unsigned { return cached ? skeys[j] : order_key(a.scores[poff + c0 + j]); };
 
-  bool all = false;
-  unsigned tau = 0;
-  int need_eq = 0;
-  if (want >= P) {
-    all = true;     // keep every candidate
+  int kept = 0, before = 0;   // positions this CTA keeps, and the CTAs of lower rank
+  if (want >= P) {            // every candidate
+    for (int w = tid; w < nwords; w += T) words[w] = n - 32 * w >= 32 ? 0xffffffffu : (1u << (n - 32 * w)) - 1u;
+    before = c0;
   } else if (want > 0) {
-    // ---- threshold: the want-th largest key of the head, four 8-bit digit passes
-    unsigned prefix = 0, mask = 0;
-    int remaining = want;
-    // up to eight keys per thread stay in registers for the four passes; their votes are
-    // independent, so the eight chains of a pass overlap
-    const bool inreg = cached && R <= 8;
-    unsigned rk[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int j = e * T + tid;
-      rk[e] = (inreg && j < n) ? skeys[kslot(j)] : 0u;
-    }
-    auto count_digit = [&](const unsigned digit, const int buf) {
-      count_digits(hist[buf], digit, lane);
-    };
-    // Threads 0..255 bring the number of keys in their bin: the bin that holds the left-th
-    // largest key goes to s_sel[0], how many keys are still needed from inside it to s_sel[1],
-    // its size to s_sel[2].  All threads call it; it ends on a CTA barrier.
-    auto find_digit = [&](const int tot, const int left) {
-      int incl = tot;   // suffix sums over the 256 bins: this bin and those above it
-      if (tid < 256) {
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int v = __shfl_down_sync(0xffffffffu, incl, o);
-          if (lane + o < 32) incl += v;
-        }
-        if (lane == 0) s_scan[warp][0] = incl;
-      }
-      __syncthreads();
-      if (tid < 256) {
-        int above = incl - tot;
-        for (int w = warp + 1; w < 8; ++w) above += s_scan[w][0];
-        if (above < left && left <= above + tot) {
-          s_sel[0] = tid;
-          s_sel[1] = left - above;
-          s_sel[2] = tot;
-        }
-      }
-      __syncthreads();
-    };
-    for (int pass = 0; pass < 4; ++pass) {
-      const int shift = 24 - 8 * pass, buf = pass & 1;
-      if (FUSED && pass == 0) {
-        // the leading digits were counted while the keys were made
-      } else if (inreg) {
-        unsigned dg[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-          dg[e] = (e * T + tid < n && (rk[e] & mask) == prefix) ? (rk[e] >> shift) & 255u
-                                                                : 0xffffffffu;
-        if (R > 4) {   // R is the same in every thread
-          count_digits8(hist[buf], dg, lane);
-        } else {
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (e < R) count_digit(dg[e], buf);
-        }
-      } else {
-        for (int e0 = 0; e0 < R; e0 += 8) {   // same trip count in every lane: full-warp votes
-          unsigned dg[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const int j = (e0 + e) * T + tid;
-            dg[e] = 0xffffffffu;
-            if (e0 + e < R && j < n) {
-              const unsigned key = key_at(j);
-              if ((key & mask) == prefix) dg[e] = (key >> shift) & 255u;
-            }
-          }
-          count_digits8(hist[buf], dg, lane);
-        }
-      }
-      cluster.sync();
-      // every CTA adds up the cluster's histograms and finds the digit itself
-      int tot = 0;
-      if (tid < 256) {
-        int part[kTailCluster];
-#pragma unroll
-        for (int r = 0; r < kTailCluster; ++r)
-          part[r] = r < cs ? *cluster.map_shared_rank(&hist[buf][tid], r) : 0;
-#pragma unroll
-        for (int r = 0; r < kTailCluster; ++r) tot += part[r];
-        hist[buf ^ 1][tid] = 0;   // every CTA is past its reads of the other buffer
-      }
-      find_digit(tot, remaining);
-      prefix |= (unsigned)s_sel[0] << shift;
-      remaining = s_sel[1];
-      mask |= 255u << shift;
-      // A CTA that owns a whole head and keeps its keys in shared memory: two digits fix sign,
-      // exponent and seven mantissa bits, and the bin that holds the threshold is small.  Its
-      // keys (their low 16 bits) go to a list and the last two digits are searched there, two
-      // sweeps over a few hundred entries instead of two over all keys.  (With a cluster the
-      // sweeps are short already and a list costs as much as the two histogram exchanges.)
-      if (cs == 1 && pass == 1 && !inreg && cached && s_sel[2] <= kTailListCap) {
-        unsigned* list = reinterpret_cast<unsigned*>(sraw);   // after the keys; the pooling stage is free by now
-        for (int e = 0; e < R; ++e) {
-          const int j = e * T + tid;
-          if (j < n) {
-            const unsigned key = skeys[kslot(j)];
-            if ((key & mask) == prefix) list[atomicAdd(&s_nlist, 1)] = key & 0xffffu;
-          }
-        }
-        if (tid < 256) hist[1][tid] = 0;   // hist[0] is zero already
-        __syncthreads();
-        const int nl = s_nlist;
-        for (int e = tid; e < nl; e += T) atomicAdd(&hist[0][(list[e] >> 8) & 255u], 1);
-        __syncthreads();
-        find_digit(tid < 256 ? hist[0][tid] : 0, remaining);
-        const unsigned hi8 = (unsigned)s_sel[0];
-        remaining = s_sel[1];
-        for (int e = tid; e < nl; e += T)
-          if (((list[e] >> 8) & 255u) == hi8) atomicAdd(&hist[1][list[e] & 255u], 1);
-        __syncthreads();
-        find_digit(tid < 256 ? hist[1][tid] : 0, remaining);
-        prefix |= (hi8 << 8) | (unsigned)s_sel[0];
-        remaining = s_sel[1];
-        break;
+    const Threshold th = threshold_search<T>(key_at, n, want, klo, khi, sm, cluster, cs, crank);
+    // ---- bitmap: a warp votes on 32 consecutive positions
+    const bool all_eq = th.need_eq == th.eq_total;   // no tie to split: keep every key from tau on
+    for (int j0 = 0; j0 < n; j0 += T) {
+      const int j = j0 + tid;
+      const unsigned key = j < n ? key_at(j) : 0u;
+      const unsigned m = __ballot_sync(0xffffffffu, j < n && (all_eq ? key >= th.tau : key > th.tau));
+      const unsigned q = all_eq ? 0u : __ballot_sync(0xffffffffu, j < n && key == th.tau);
+      if (lane == 0 && (j >> 5) < nwords) {
+        words[j >> 5] = m;
+        eqw[j >> 5] = q;
       }
     }
-    tau = prefix;
-    need_eq = remaining;
-  }
-
-  // ---- ordered compaction: thread t owns the run [t*R, (t+1)*R) of the slice; it keeps the
-  // positions with key > tau, plus the first need_eq (in position order) with key == tau
-  if (want > 0) {
-    const int r0 = min(tid * R, n), r1 = min(r0 + R, n);
-    int gt = 0, eq = 0;
-    if (all) {
-      gt = r1 - r0;
-    } else {
-      for (int j = r0; j < r1; ++j) {
-        const unsigned key = key_at(j);
-        gt += key > tau;
-        eq += key == tau;
-      }
-    }
-    int gt_inc = gt, eq_inc = eq;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(0xffffffffu, gt_inc, o);
-      const int y = __shfl_up_sync(0xffffffffu, eq_inc, o);
-      if (lane >= o) gt_inc += x, eq_inc += y;
-    }
-    __syncthreads();   // the threshold search is done with s_scan
-    if (lane == 31) s_scan[warp][0] = gt_inc, s_scan[warp][1] = eq_inc;
     __syncthreads();
-    int gt_before = gt_inc - gt, eq_before = eq_inc - eq;
-    for (int w = 0; w < warp; ++w) gt_before += s_scan[w][0], eq_before += s_scan[w][1];
-    if (tid == T - 1) {
-      s_tot[0] = gt_before + gt;
-      s_tot[1] = eq_before + eq;
-    }
-    cluster.sync();
-    {
-      int2 before[kTailCluster];
-#pragma unroll
-      for (int r = 0; r < kTailCluster; ++r)
-        before[r] = r < crank ? *reinterpret_cast<const int2*>(cluster.map_shared_rank(&s_tot[0], r))
-                              : make_int2(0, 0);
-#pragma unroll
-      for (int r = 0; r < kTailCluster; ++r) gt_before += before[r].x, eq_before += before[r].y;
-    }
-    // most runs hold no kept position at all: their second walk is skipped
-    const bool writes = all || gt > 0 || (eq > 0 && eq_before < need_eq);
-    for (int j = r0; writes && j < r1; ++j) {
-      const int i = c0 + j;
-      if (all) {
-        out[gt_before++] = i;
-        continue;
-      }
-      const unsigned key = key_at(j);
-      if (key > tau) {
-        out[gt_before + min(eq_before, need_eq)] = i;
-        ++gt_before;
-      } else if (key == tau) {
-        if (eq_before < need_eq) out[gt_before + eq_before] = i;
-        ++eq_before;
+    before = th.gt_before + min(th.eq_before, th.need_eq);
+    if (!all_eq) {   // the first need_eq equal keys in position order
+      int seen = th.eq_before;
+      for (int w0 = 0; w0 < nwords; w0 += T) {
+        const int w = w0 + tid;
+        unsigned q = w < nwords ? eqw[w] : 0u;
+        const int first = seen + block_scan<T, false>(__popc(q), sm.scan, lane, warp);
+        int take = max(0, min(__popc(q), th.need_eq - first));
+        unsigned keep = 0u;
+        for (; take > 0; --take) {
+          keep |= q & (0u - q);
+          q &= q - 1u;
+        }
+        if (w < nwords) words[w] |= keep;
+        __syncthreads();
+        if (tid < 32) {   // total of this round
+          const int tot = __reduce_add_sync(0xffffffffu, lane < T / 32 ? sm.scan[lane] : 0);
+          if (lane == 0) sm.bin = tot;
+        }
+        __syncthreads();
+        seen += sm.bin;
+        __syncthreads();
       }
     }
   }
-  // the index list is complete (and visible to the cluster) after this barrier; it also keeps
-  // every CTA's shared memory alive until its peers have read it
-  cluster.sync();
-  if (FUSED && R <= 8) {
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int j = e * T + tid;
-      if (j < n) a.s_comp_out[poff + c0 + j] = held[e];
+  // ---- compaction: prefix sums over the words of the bitmap place every kept position
+  int* out = a.idx + (size_t)layer * a.idx_cap + s_off;
+  if (want > 0) {
+    __syncthreads();   // the words are complete
+    for (int w0 = 0; w0 < nwords; w0 += T) {
+      const int w = w0 + tid;
+      unsigned m = w < nwords ? words[w] : 0u;
+      int k = kept + block_scan<T, false>(__popc(m), sm.scan, lane, warp);
+      kept += __reduce_add_sync(0xffffffffu, lane < T / 32 ? sm.scan[lane] : 0);
+      for (; m; m &= m - 1u, ++k) {
+        const int i = c0 + 32 * w + __ffs(m) - 1;
+        out[before + k] = i;
+        if (k < kTailRowCap) s_rows[k] = i;
+      }
+      __syncthreads();
     }
   }
+  if (cs > 1 && want > 0 && want < P) cluster.barrier_arrive();   // past this CTA's last remote read
 
-  // ---- gather: selected rows in ascending position order, then the W window rows
+  // ---- gather: the rows this CTA keeps in ascending position order; the last CTA adds the W window rows
   if (a.K_out) {
-    const int n_sel = max(want, 0) < P ? max(want, 0) : P;
-    const int rows = n_sel + W;
+    const int rows = kept + (crank == cs - 1 ? W : 0);
     const __nv_bfloat16* Ksrc = a.K + (size_t)layer * a.kv_layer_stride;
     const __nv_bfloat16* Vsrc = a.V + (size_t)layer * a.kv_layer_stride;
     const size_t srow0 = (size_t)h * st.Ltot + st.cu[b];
-    const size_t drow0 = (size_t)layer * a.out_rows_cap + (size_t)(s_off + bh * W);
+    const size_t drow0 = (size_t)layer * a.out_rows_cap + (size_t)(s_off + bh * W + before);
     const int hw = tid >> 4, l = tid & 15;                       // half-warps, 16 B per lane
-    const int rows_per_sweep = cs * (T / 16);
-    for (int rb = crank * (T / 16) + hw; rb < rows; rb += 2 * rows_per_sweep) {
-      const int ra = rb + rows_per_sweep;
-      const int sa = rb < n_sel ? __ldcg(out + rb) : P + (rb - n_sel);
-      const int sb = ra < rows ? (ra < n_sel ? __ldcg(out + ra) : P + (ra - n_sel)) : -1;
+    constexpr int kSweep = T / 16;
+    auto source = [&](const int r) {
+      return r >= kept ? P + (r - kept) : r < kTailRowCap ? s_rows[r] : __ldcg(out + before + r);
+    };
+    for (int ra = hw; ra < rows; ra += 2 * kSweep) {
+      const int rb = ra + kSweep;
+      const int sa = source(ra), sb = rb < rows ? source(rb) : -1;
       const uint4 k0 = __ldg(reinterpret_cast<const uint4*>(Ksrc + (srow0 + sa) * kHeadDim) + l);
       const uint4 v0 = __ldg(reinterpret_cast<const uint4*>(Vsrc + (srow0 + sa) * kHeadDim) + l);
       uint4 k1 = make_uint4(0, 0, 0, 0), v1 = k1;
@@ -935,14 +829,16 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
         k1 = __ldg(reinterpret_cast<const uint4*>(Ksrc + (srow0 + sb) * kHeadDim) + l);
         v1 = __ldg(reinterpret_cast<const uint4*>(Vsrc + (srow0 + sb) * kHeadDim) + l);
       }
-      reinterpret_cast<uint4*>(a.K_out + (drow0 + rb) * kHeadDim)[l] = k0;
-      reinterpret_cast<uint4*>(a.V_out + (drow0 + rb) * kHeadDim)[l] = v0;
+      reinterpret_cast<uint4*>(a.K_out + (drow0 + ra) * kHeadDim)[l] = k0;
+      reinterpret_cast<uint4*>(a.V_out + (drow0 + ra) * kHeadDim)[l] = v0;
       if (sb >= 0) {
-        reinterpret_cast<uint4*>(a.K_out + (drow0 + ra) * kHeadDim)[l] = k1;
-        reinterpret_cast<uint4*>(a.V_out + (drow0 + ra) * kHeadDim)[l] = v1;
+        reinterpret_cast<uint4*>(a.K_out + (drow0 + rb) * kHeadDim)[l] = k1;
+        reinterpret_cast<uint4*>(a.V_out + (drow0 + rb) * kHeadDim)[l] = v1;
       }
     }
   }
+  // a CTA's shared memory stays alive until its peers have read it
+  if (cs > 1 && want > 0 && want < P) cluster.barrier_wait();
 }
 
 int floor_slots(const mixkv_params& p) {
@@ -1006,13 +902,8 @@ cudaError_t launch_budget(const LaunchCtx& c, const float* scores, int* counts) 
   // the keys of a CTA's slice of the longest sequence in shared memory when they fit
   const size_t want = (size_t)c.st.H * chunk * 4;
   const size_t cap_bytes = 200 * 1024;
-  const size_t key_bytes = want <= cap_bytes - 16 * 1024 ? want : 0;
-  // the rest, up to 16 K entries, holds the candidates left after the first digit pass
-  size_t list_bytes = cap_bytes - key_bytes;
-  if (list_bytes > 64 * 1024) list_bytes = 64 * 1024;
-  if (list_bytes > want) list_bytes = want;
-  const size_t smem = key_bytes + list_bytes;
-  if (smem > 48 * 1024) {
+  const size_t smem = want <= cap_bytes ? want : 0;
+  if (smem > 24 * 1024) {   // on top of the search's static shared memory
     static bool done[64] = {false};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -1024,30 +915,30 @@ cudaError_t launch_budget(const LaunchCtx& c, const float* scores, int* counts) 
       if (dev >= 0 && dev < 64) done[dev] = true;
     }
   }
-  return launch_pdl(k_budget, dim3(c.st.batch * cs, c.st.layers), dim3(1024), smem, c.stream, cs,
-                    c.st, scores, counts, c.p.budget - c.p.window, floor_slots(c.p),
-                    (int)(key_bytes / 4), (int)(list_bytes / 4));
+  return launch_pdl(k_budget, dim3(c.st.batch * cs, c.st.layers), dim3(kBudgetThreads), smem, c.stream, cs,
+                    c.st, scores, counts, c.p.budget - c.p.window, floor_slots(c.p), (int)(smem / 4));
 }
 
-// Launch shape of k_tail: many (layer, sequence, head) units -> one 1024-thread CTA each; few ->
-// a cluster of kTailCluster 512-thread CTAs each.  Returns false when the keys of a slice do not
-// fit the shared-memory cache under either shape.
+// Launch shape of k_tail for the longest sequence of the call.
 struct TailShape {
   int cs, threads, chunk;
   bool cached;
 };
 
 TailShape tail_shape(const LaunchCtx& c) {
-  const int units = c.st.layers * c.st.batch * c.st.H;
+  const long long units = (long long)c.st.layers * c.st.batch * c.st.H;
+  const int P = c.max_prefix;
   TailShape t;
-  t.cs = 1, t.threads = 1024, t.chunk = c.max_prefix;
-  if (units >= device_sm_count() / 2 && t.chunk <= kTailCacheCapSolo) {
-    t.cached = true;
-    return t;
+  t.cs = 1;
+  if (units >= device_sm_count() / 2 && P <= kTailCacheCapSolo) {
+    // many units: one CTA each
+  } else {
+    while (t.cs < kTailMaxCluster && tail_chunk(P, t.cs) > 4096) t.cs *= 2;
   }
-  t.cs = kTailCluster, t.threads = kTailThreads;
-  t.chunk = (c.max_prefix + kTailCluster - 1) / kTailCluster;
-  t.cached = t.chunk <= kTailCacheCap;
+  t.chunk = tail_chunk(P, t.cs);
+  t.threads = t.chunk <= 2048 ? 256 : t.chunk <= 4096 ? 512 : 1024;
+  if (units * t.cs <= device_sm_count()) t.threads = t.chunk <= 1024 ? 256 : t.chunk <= 2048 ? 512 : 1024;
+  t.cached = t.chunk <= (t.cs == 1 ? kTailCacheCapSolo : kTailCacheCap);
   return t;
 }
 
@@ -1060,8 +951,8 @@ cudaError_t launch_tail_t(const LaunchCtx& c, const TailKernelArgs& a, const Tai
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  if (smem > 48 * 1024 && (dev < 0 || dev >= 64 || have[dev] < smem)) {
-    const size_t ask = 216 * 1024;
+  if (smem > 20 * 1024 && (dev < 0 || dev >= 64 || have[dev] < smem)) {   // on top of the static part
+    const size_t ask = 203 * 1024;
     e = cudaFuncSetAttribute(k_tail<FUSED, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)ask);
     if (e != cudaSuccess) return e;
@@ -1096,13 +987,15 @@ cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
   const bool fused = t.scores == nullptr;
   a.cached = sh.cached ? 1 : 0;
   if (fused && !a.cached) return cudaErrorInvalidValue;   // callers check tail_can_fuse() first
-  size_t smem = 0;
-  if (a.cached) smem += ((size_t)sh.chunk + (sh.chunk >> 5) + 1) * 4;
-  if (fused) smem += ((size_t)8 * sh.threads + 64) * 4;          // pooling stage, later the key list
-  else if (a.cached) smem += (size_t)kTailListCap * 4;           // key list of a lone CTA
-  if (sh.threads == 1024)
-    return fused ? launch_tail_t<true, 1024>(c, a, sh, smem) : launch_tail_t<false, 1024>(c, a, sh, smem);
-  return fused ? launch_tail_t<true, 512>(c, a, sh, smem) : launch_tail_t<false, 512>(c, a, sh, smem);
+  // bitmaps of kept and of equal positions, the keys, the pooling stage
+  size_t smem = (size_t)(sh.chunk / 32) * 8;
+  if (a.cached) smem += (size_t)sh.chunk * 4;
+  if (fused) smem += ((size_t)8 * sh.threads + 64) * 4;
+  switch (sh.threads) {
+    case 256: return fused ? launch_tail_t<true, 256>(c, a, sh, smem) : launch_tail_t<false, 256>(c, a, sh, smem);
+    case 512: return fused ? launch_tail_t<true, 512>(c, a, sh, smem) : launch_tail_t<false, 512>(c, a, sh, smem);
+    default: return fused ? launch_tail_t<true, 1024>(c, a, sh, smem) : launch_tail_t<false, 1024>(c, a, sh, smem);
+  }
 }
 
 }  // namespace mixkv
