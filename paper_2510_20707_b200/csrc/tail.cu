@@ -20,8 +20,8 @@ namespace {
 //   s_in_scaled  = (|V_i| - sc[0]) * sc[1]
 //   s_div_scaled = (s_div_i - sc[2]) * sc[3]
 //   sc[4]        = redundancy used by the mix
-__device__ void head_scalars(const SeqTable& st, const Workspace& ws, const int layer, const int b,
-                             const int h, const int pool_k, const int pool_mode, const int use_vnorm,
+__device__ void head_scalars(const SeqTable& st, const Workspace& ws, const SegList& sl, const int layer,
+                             const int b, const int h, const int pool_k, const int pool_mode, const int use_vnorm,
                              const float eps, const float* __restrict__ rbar_in, const int lane,
                              float* sc) {
   const int unit = (layer * st.batch + b) * st.H + h;
@@ -31,8 +31,6 @@ __device__ void head_scalars(const SeqTable& st, const Workspace& ws, const int 
   float rbar = 0.f;
   if (lane == 0) rbar = rbar_in ? rbar_in[unit] : ws.rbar[unit];
   {
-    const int per_head = (st.tile2_start[b + 1] - st.tile2_start[b]) / st.H;
-    const SegList sl(layer * st.nt2 + st.tile2_start[b] + h * per_head, per_head, split2(st));
     // lanes take segments side by side, two per lane and round; all loads of a round are
     // issued before the first is used
     for (int e0 = lane; e0 < sl.nseg; e0 += 64) {
@@ -114,19 +112,35 @@ __device__ __forceinline__ float pool_window(const float* w, const int k, const 
   return v;
 }
 
+// Eq. 5 with VNorm (Eq. 2); v0 .. r: the head scalars.  Rounding written out, so that every kernel that
+// mixes gives the same bits.
+__device__ __forceinline__ float mix_headwise(const float ex, const float vn, const float dv, const float v0,
+                                              const float vs, const float d0, const float ds, const float r) {
+  const float imp = __fmaf_rn(vn - v0, vs, ex);
+  const float dsc = __fmul_rn(dv - d0, ds);
+  return __fmaf_rn(1.0f - r, imp, __fmul_rn(r, dsc));
+}
+
 __device__ __forceinline__ float mix_one(const float ex, const float vn, const float dv,
                                          const float* sc, const int use_vnorm,
                                          const int mix_mode) {
-  float imp = ex;
-  if (use_vnorm) imp += (vn - sc[0]) * sc[1];
-  const float dsc = (dv - sc[2]) * sc[3];
+  if (use_vnorm && mix_mode == MIXKV_MIX_HEADWISE)
+    return mix_headwise(ex, vn, dv, sc[0], sc[1], sc[2], sc[3], sc[4]);
+  const float imp = use_vnorm ? __fmaf_rn(vn - sc[0], sc[1], ex) : ex;
+  const float dsc = __fmul_rn(dv - sc[2], sc[3]);
   const float r = sc[4];
   switch (mix_mode) {
-    case MIXKV_MIX_HEADWISE: return (1.0f - r) * imp + r * dsc;   // Eq. 5
+    case MIXKV_MIX_HEADWISE: return __fmaf_rn(1.0f - r, imp, __fmul_rn(r, dsc));   // Eq. 5
     case MIXKV_MIX_IMPORTANCE_ONLY: return imp;
     case MIXKV_MIX_DIVERSITY_ONLY: return dv;
-    default: return imp + dsc;
+    default: return __fadd_rn(imp, dsc);
   }
+}
+
+// The pass-2 segments of a head.
+__device__ __forceinline__ SegList pass2_segments(const SeqTable& st, const int layer, const int b, const int h) {
+  const int per_head = (st.tile2_start[b + 1] - st.tile2_start[b]) / st.H;
+  return SegList(layer * st.nt2 + st.tile2_start[b] + h * per_head, per_head, split2(st));
 }
 
 struct MixParams {
@@ -185,8 +199,8 @@ k_mixpool(const SeqTable st, const Workspace ws, const float* __restrict__ s_div
   const int half = mp.pool_k >> 1;
   const float pad = mp.pool_mode == MIXKV_POOL_AVG ? 0.f : -INFINITY;
   if (threadIdx.x < 32)
-    head_scalars(st, ws, layer, b, h, mp.pool_k, mp.pool_mode, mp.use_vnorm, mp.eps, rbar_in,
-                 threadIdx.x, sc);
+    head_scalars(st, ws, pass2_segments(st, layer, b, h), layer, b, h, mp.pool_k, mp.pool_mode, mp.use_vnorm,
+                 mp.eps, rbar_in, threadIdx.x, sc);
   // a chunk is eight rounds of 256 positions (+ the pooling halo in a ninth); every load of the
   // chunk is issued before the first use
   constexpr int kRounds = kPChunk / 256;
@@ -236,6 +250,7 @@ constexpr int kSelListCap = 256;   // candidates ranked directly
 struct SelSmem {
   int hist[2][kSelBins];
   unsigned list[kSelListCap];    // this CTA's candidates
+  int pos[kSelListCap];          // and which of its keys they are
   unsigned all[kSelListCap];     // those of every CTA of the cluster, in rank order
   unsigned wlo[32], whi[32];
   unsigned range[2];             // this CTA's smallest and largest key
@@ -252,6 +267,8 @@ struct Threshold {
   unsigned tau;              // the want-th largest key
   int need_eq, eq_total;     // keys equal to it that are wanted / that there are
   int gt_before, eq_before;  // keys above it and equal to it in the CTAs of lower rank
+  bool listed;               // above(j) was called for this CTA's keys above the last bin, whose sm.nlist keys
+                             // are in sm.list / sm.pos
 };
 
 // Sum of v over the threads after the caller (suffix = true) or before it; every thread of the CTA takes
@@ -280,10 +297,11 @@ __device__ __forceinline__ int block_scan(const int v, int* scan, const int lane
 // dozen keys, which are listed and ranked against each other.  One sweep to count, one to list, where digits of
 // the raw key bits took two to four sweeps and as many exchanges across the cluster.  A bin with more keys
 // than the list takes is binned again (three rounds reach single key values), so any distribution, all-equal
-// keys included, ends after a bounded number of sweeps.  sm.hist must be zero on entry (visible to the CTA).
-template <int T, typename KeyAt>
-__device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const int n, const int want,
-                                                      unsigned lo, unsigned hi, SelSmem& sm,
+// keys included, ends after a bounded number of sweeps.  The listing sweep calls above(j) for the keys that
+// are wanted in any case.  sm.hist must be zero on entry (visible to the CTA).
+template <int T, typename KeyAt, typename Above>
+__device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const Above& above_bin, const int n,
+                                                      const int want, unsigned lo, unsigned hi, SelSmem& sm,
                                                       cg::cluster_group& cluster, const int cs,
                                                       const int crank) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -356,6 +374,7 @@ __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const
   const int count = sm.count;
   Threshold th;
   th.gt_before = th.eq_before = 0;
+  th.listed = shift != 0;
   if (shift == 0) {   // the bin is one key value
     th.tau = base, th.need_eq = remaining, th.eq_total = count;
     if (cs > 1) {
@@ -380,8 +399,13 @@ __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const
   for (int j = tid; j < n; j += T) {
     const unsigned key = key_at(j);
     if (key >= base) {
-      if (key - base <= span) sm.list[atomicAdd(&sm.nlist, 1)] = key;
-      else ++gt;
+      if (key - base <= span) {
+        const int at = atomicAdd(&sm.nlist, 1);
+        sm.list[at] = key, sm.pos[at] = j;
+      } else {
+        ++gt;
+        above_bin(j);
+      }
     }
   }
   const unsigned* all = sm.list;
@@ -497,7 +521,7 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
     return order_key(base[(size_t)h * stride + p0 + (e - h * n)]);
   };
   const Threshold th =
-      threshold_search<kBudgetThreads>(key_at, local, (int)N, lo, hi, sm, cluster, cs, crank);
+      threshold_search<kBudgetThreads>(key_at, [](int) {}, local, (int)N, lo, hi, sm, cluster, cs, crank);
   for (int h = 0; h < H; ++h) {
     int gt = 0, eq = 0;
     for (int i = tid; i < n; i += kBudgetThreads) {
@@ -537,6 +561,9 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
   if (cs > 1) cluster.sync();   // the peers' shared memory stays alive until rank 0 has read it
 }
 
+// Word at which the keys of a slice start in k_tail's dynamic shared memory: behind the two bitmaps, on a
+// 16-byte boundary.
+__host__ __device__ __forceinline__ int tail_keys_at(const int chunk) { return ((chunk >> 4) + 3) & ~3; }
 // Positions per CTA when cs CTAs share the P candidates of a head: whole words of 32.
 __host__ __device__ __forceinline__ int tail_chunk(const int P, const int cs) {
   return (((P + cs - 1) / cs) + 31) & ~31;
@@ -584,8 +611,9 @@ __device__ __forceinline__ int fixed_offset(const SeqTable& st, int bh, int Bp) 
 //
 // Latency bound: a unit is a chain of short phases.  Mix (or load) the slice's scores into shared memory as
 // keys; threshold (threshold_search); one vote per 32 positions turns the keys into a bitmap whose prefix sums
-// place every kept position; gather.  28 layers x 4 heads x 32736 candidates: 52 -> see DESIGN's table; 896 heads of
-// 2 to 7 thousand candidates (selection and gather only): 114 us with one 1024-thread CTA per head.
+// place every kept position; gather.  28 layers x 4 heads x 32736 candidates: 35 us (57 with digit passes over the
+// raw keys and a position per thread and step in the mix); 896 heads of 2 to 7 thousand candidates (selection and
+// gather only): 47 us (119).
 template <bool FUSED, int T>
 __global__ void __launch_bounds__(T, 1024 / T)
 k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
@@ -616,11 +644,14 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   const int nwords = (n + 31) >> 5;
   unsigned* words = reinterpret_cast<unsigned*>(tail_smem);            // [chunk / 32] bitmap of kept positions
   unsigned* eqw = words + (chunk >> 5);                                // [chunk / 32] positions equal to the threshold
-  unsigned* skeys = eqw + (chunk >> 5);                                // [chunk] when cached
-  float* sraw = reinterpret_cast<float*>(skeys + chunk);               // FUSED: [8 T + 64] pooling stage
+  unsigned* skeys = reinterpret_cast<unsigned*>(tail_smem) + tail_keys_at(chunk);   // [chunk] when cached
+  float* sraw = reinterpret_cast<float*>(skeys + chunk);               // FUSED: [4 T + 64] raw scores of a block
+  float* sdv = sraw + 4 * T + 64;                                      // FUSED: [4 T] diversity scores
 
   pdl_launch_dependents();
   for (int t = tid; t < 2 * kSelBins; t += T) (&sm.hist[0][0])[t] = 0;
+  const SegList sl2 = pass2_segments(st, layer, b, h);   // (divisions: ahead of the wait)
+  const int fixed_off = fixed_offset(st, bh, a.Bp);
   pdl_wait();
 
   if (a.status_clear && blockIdx.x == 0 && tid == 0) *a.status_clear = 0;
@@ -632,7 +663,7 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
       off = __reduce_add_sync(0xffffffffu, off);
       cnt = counts_dev[bh];
     } else {
-      off = fixed_offset(st, bh, a.Bp);
+      off = fixed_off;
       cnt = min(a.Bp, P);
     }
     if (lane == 0) {
@@ -652,72 +683,124 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   const bool cached = FUSED || a.cached;
   unsigned klo = 0xffffffffu, khi = 0u;   // smallest and largest key this thread has made
   if (FUSED) {
-    // ---- pooling and mix of this slice (Eq. 2, Eq. 5) in blocks of 8 T consecutive positions:
-    // thread t takes positions t, t + T, ... of the block
+    // ---- pooling and mix of this slice (Eq. 2, Eq. 5) in blocks of 4 T positions.  A block is read from
+    // global memory one block ahead (consecutive threads, consecutive positions), staged in shared memory
+    // (raw scores with the pooling halo; value norms in the slots of the block's keys), and every
+    // thread then takes four CONSECUTIVE positions: a window of up to nine raw scores around them is three
+    // 16-byte loads instead of four times the window.
+    constexpr int BL = 4 * T;
     const int half = a.mp.pool_k >> 1;
-    const bool avg = a.mp.pool_mode == MIXKV_POOL_AVG;
+    const bool avg = a.mp.pool_mode == MIXKV_POOL_AVG, vnorm_on = a.mp.use_vnorm != 0;
     const float pad = avg ? 0.f : -INFINITY;
     const float invk = 1.0f / (float)a.mp.pool_k;
     if (warp == 1)
-      head_scalars(st, ws, layer, b, h, a.mp.pool_k, a.mp.pool_mode, a.mp.use_vnorm, a.mp.eps,
+      head_scalars(st, ws, sl2, layer, b, h, a.mp.pool_k, a.mp.pool_mode, a.mp.use_vnorm, a.mp.eps,
                    a.rbar_in, lane, sc);
-    // The block and its pooling halo (62 positions at most) are nine rounds of T raw scores.
-    // They are loaded one block ahead: the raw scores of block b + 1 fly while block b is pooled
-    // and mixed, and the two per-position terms of a block are asked for before its pooling and
-    // used after it.
-    float raw[9];
-    auto load_raw = [&](const int j0) {
-      const int nstage = min(8 * T, n - j0) + 2 * half;
+    const float* g_raw = ws.s_ex_raw + poff;
+    const float* g_vn = ws.vnorm + poff + c0;
+    const float* g_dv = a.s_div + poff + c0;
+    float* svn = reinterpret_cast<float*>(skeys);
+    float raw[5], vn[4], dv[4];   // the fifth raw score: the halo (62 positions at most)
+    auto load_block = [&](const int j0) {
+      const int nb = min(BL, n - j0), i0 = c0 + j0 - half;
+      if (nb == BL && i0 >= 0 && i0 + BL + 2 * half <= P) {   // inside the sequence: nothing to test
+        const float* r = g_raw + i0 + tid;
+        const float* d = g_dv + j0 + tid;
+        const float* v = g_vn + j0 + tid;
 #pragma unroll
-      for (int e = 0; e < 9; ++e) {
-        const int t = e * T + tid, i = c0 + j0 - half + t;
-        raw[e] = (j0 < n && t < nstage && i >= 0 && i < P) ? ws.s_ex_raw[poff + i] : pad;
+        for (int e = 0; e < 4; ++e) {
+          raw[e] = r[e * T];
+          dv[e] = d[e * T];
+          vn[e] = vnorm_on ? v[e * T] : 0.f;
+        }
+        if (tid < 2 * half) raw[4] = r[4 * T];
+        return;
+      }
+#pragma unroll
+      for (int e = 0; e < 5; ++e) {
+        const int t = e * T + tid, i = i0 + t;
+        raw[e] = (t < nb + 2 * half && i >= 0 && i < P) ? g_raw[i] : pad;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int t = e * T + tid;
+        vn[e] = (vnorm_on && t < nb) ? g_vn[j0 + t] : 0.f;
+        dv[e] = t < nb ? g_dv[j0 + t] : 0.f;
       }
     };
-    load_raw(0);
-    for (int j0 = 0; j0 < n; j0 += 8 * T) {
-      const int nb = min(8 * T, n - j0);   // positions of this block
-      float vn[8], dv[8];
-      const int nstage = nb + 2 * half;
+    if (n > 0) load_block(0);
+    for (int j0 = 0; j0 < n; j0 += BL) {
+      const int nb = min(BL, n - j0);   // positions of this block
+      __syncthreads();                  // the previous block's readers of the stage are done
+      if (nb == BL) {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int jb = e * T + tid;
-        vn[e] = (a.mp.use_vnorm && jb < nb) ? ws.vnorm[poff + c0 + j0 + jb] : 0.f;
-        dv[e] = jb < nb ? a.s_div[poff + c0 + j0 + jb] : 0.f;
-      }
-      __syncthreads();                     // the previous block's readers of sraw are done
+        for (int e = 0; e < 4; ++e)
+          sraw[e * T + tid] = raw[e], sdv[e * T + tid] = dv[e], svn[j0 + e * T + tid] = vn[e];
+        if (tid < 2 * half) sraw[BL + tid] = raw[4];
+      } else {
 #pragma unroll
-      for (int e = 0; e < 9; ++e) {
-        const int t = e * T + tid;
-        if (t < nstage) sraw[t] = raw[e];
+        for (int e = 0; e < 5; ++e) {
+          const int t = e * T + tid;
+          if (t < nb + 2 * half) sraw[t] = raw[e];
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int t = e * T + tid;
+          if (t < nb) sdv[t] = dv[e], svn[j0 + t] = vn[e];
+        }
       }
-      load_raw(j0 + 8 * T);
+      if (j0 + BL < n) load_block(j0 + BL);
       __syncthreads();
-      // the eight pooling windows advance together (same order of additions as pool_window),
-      // so their shared-memory loads overlap instead of forming eight serial chains
-      float ex[8];
+      const int q = 4 * tid;            // this thread's positions q .. q + 3 of the block
+      if (q < nb) {
+        float ex[4];
+        if (a.mp.pool_k <= 9) {
+          float w[12];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) ex[e] = avg ? 0.f : -INFINITY;
-      for (int u = 0; u < a.mp.pool_k; ++u) {
+          for (int u = 0; u < 3; ++u)
+            *reinterpret_cast<float4*>(w + 4 * u) = *reinterpret_cast<const float4*>(sraw + q + 4 * u);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          if (e * T < nb) {   // the same in every thread
-            const float w = sraw[min(e * T + tid, nb - 1) + u];
-            ex[e] = avg ? ex[e] + w : fmaxf(ex[e], w);
+          for (int e = 0; e < 4; ++e) ex[e] = avg ? 0.f : -INFINITY;
+#pragma unroll
+          for (int u = 0; u < 9; ++u) {   // (same order of additions as pool_window)
+            if (u < a.mp.pool_k) {
+#pragma unroll
+              for (int e = 0; e < 4; ++e) ex[e] = avg ? ex[e] + w[e + u] : fmaxf(ex[e], w[e + u]);
+            }
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) ex[e] = avg ? ex[e] * invk : ex[e];
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) ex[e] = pool_window(sraw + q + e, a.mp.pool_k, a.mp.pool_mode, invk);
+        }
+        const float4 v4 = *reinterpret_cast<const float4*>(svn + j0 + q);
+        const float4 d4 = *reinterpret_cast<const float4*>(sdv + q);
+        const float vv[4] = {v4.x, v4.y, v4.z, v4.w}, dd[4] = {d4.x, d4.y, d4.z, d4.w};
+        float m[4];
+        unsigned key[4];
+        if (a.mp.mix_mode == MIXKV_MIX_HEADWISE && vnorm_on) {   // (scalars in registers)
+          const float r = sc[4], v0 = sc[0], vs = sc[1], d0 = sc[2], ds = sc[3];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) m[e] = mix_headwise(ex[e], vv[e], dd[e], v0, vs, d0, ds, r);
+        } else {
+#pragma unroll
+          for (int e = 0; e < 4; ++e) m[e] = mix_one(ex[e], vv[e], dd[e], sc, a.mp.use_vnorm, a.mp.mix_mode);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          key[e] = order_key(m[e]);
+          if (q + e < nb) {
+            klo = min(klo, key[e]);
+            khi = max(khi, key[e]);
           }
         }
-      }
+        if (a.s_comp_out) {
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int jb = e * T + tid;
-        if (jb < nb) {
-          const float s = mix_one(avg ? ex[e] * invk : ex[e], vn[e], dv[e], sc, a.mp.use_vnorm, a.mp.mix_mode);
-          const unsigned key = order_key(s);
-          skeys[j0 + jb] = key;
-          klo = min(klo, key);
-          khi = max(khi, key);
-          if (a.s_comp_out) a.s_comp_out[poff + c0 + j0 + jb] = s;
+          for (int e = 0; e < 4; ++e)
+            if (q + e < nb) a.s_comp_out[poff + c0 + j0 + q + e] = m[e];
         }
+        *reinterpret_cast<uint4*>(skeys + j0 + q) = make_uint4(key[0], key[1], key[2], key[3]);
       }
     }
   } else {
@@ -749,17 +832,25 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
     for (int w = tid; w < nwords; w += T) words[w] = n - 32 * w >= 32 ? 0xffffffffu : (1u << (n - 32 * w)) - 1u;
     before = c0;
   } else if (want > 0) {
-    const Threshold th = threshold_search<T>(key_at, n, want, klo, khi, sm, cluster, cs, crank);
-    // ---- bitmap: a warp votes on 32 consecutive positions
+    for (int w = tid; w < nwords; w += T) words[w] = 0u;   // visible after the search's first barrier
+    auto keep = [&](const int j) { atomicOr(&words[j >> 5], 1u << (j & 31)); };
+    const Threshold th = threshold_search<T>(key_at, keep, n, want, klo, khi, sm, cluster, cs, crank);
     const bool all_eq = th.need_eq == th.eq_total;   // no tie to split: keep every key from tau on
-    for (int j0 = 0; j0 < n; j0 += T) {
-      const int j = j0 + tid;
-      const unsigned key = j < n ? key_at(j) : 0u;
-      const unsigned m = __ballot_sync(0xffffffffu, j < n && (all_eq ? key >= th.tau : key > th.tau));
-      const unsigned q = all_eq ? 0u : __ballot_sync(0xffffffffu, j < n && key == th.tau);
-      if (lane == 0 && (j >> 5) < nwords) {
-        words[j >> 5] = m;
-        eqw[j >> 5] = q;
+    if (all_eq && th.listed) {
+      for (int k = tid; k < sm.nlist; k += T)
+        if (sm.list[k] >= th.tau) keep(sm.pos[k]);
+    } else {
+      // a warp votes on 32 consecutive positions
+      __syncthreads();
+      for (int j0 = 0; j0 < n; j0 += T) {
+        const int j = j0 + tid;
+        const unsigned key = j < n ? key_at(j) : 0u;
+        const unsigned m = __ballot_sync(0xffffffffu, j < n && (all_eq ? key >= th.tau : key > th.tau));
+        const unsigned q = __ballot_sync(0xffffffffu, j < n && key == th.tau);
+        if (lane == 0 && (j >> 5) < nwords) {
+          words[j >> 5] = m;
+          eqw[j >> 5] = q;
+        }
       }
     }
     __syncthreads();
@@ -819,21 +910,24 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
     auto source = [&](const int r) {
       return r >= kept ? P + (r - kept) : r < kTailRowCap ? s_rows[r] : __ldcg(out + before + r);
     };
-    for (int ra = hw; ra < rows; ra += 2 * kSweep) {
-      const int rb = ra + kSweep;
-      const int sa = source(ra), sb = rb < rows ? source(rb) : -1;
-      const uint4 k0 = __ldg(reinterpret_cast<const uint4*>(Ksrc + (srow0 + sa) * kHeadDim) + l);
-      const uint4 v0 = __ldg(reinterpret_cast<const uint4*>(Vsrc + (srow0 + sa) * kHeadDim) + l);
-      uint4 k1 = make_uint4(0, 0, 0, 0), v1 = k1;
-      if (sb >= 0) {
-        k1 = __ldg(reinterpret_cast<const uint4*>(Ksrc + (srow0 + sb) * kHeadDim) + l);
-        v1 = __ldg(reinterpret_cast<const uint4*>(Vsrc + (srow0 + sb) * kHeadDim) + l);
+    for (int r0 = hw; r0 < rows; r0 += 4 * kSweep) {   // four rows of K and V in flight
+      uint4 kk[4], vv[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int r = r0 + e * kSweep;
+        if (r < rows) {
+          const size_t src = (srow0 + source(r)) * kHeadDim;
+          kk[e] = __ldg(reinterpret_cast<const uint4*>(Ksrc + src) + l);
+          vv[e] = __ldg(reinterpret_cast<const uint4*>(Vsrc + src) + l);
+        }
       }
-      reinterpret_cast<uint4*>(a.K_out + (drow0 + ra) * kHeadDim)[l] = k0;
-      reinterpret_cast<uint4*>(a.V_out + (drow0 + ra) * kHeadDim)[l] = v0;
-      if (sb >= 0) {
-        reinterpret_cast<uint4*>(a.K_out + (drow0 + rb) * kHeadDim)[l] = k1;
-        reinterpret_cast<uint4*>(a.V_out + (drow0 + rb) * kHeadDim)[l] = v1;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int r = r0 + e * kSweep;
+        if (r < rows) {
+          reinterpret_cast<uint4*>(a.K_out + (drow0 + r) * kHeadDim)[l] = kk[e];
+          reinterpret_cast<uint4*>(a.V_out + (drow0 + r) * kHeadDim)[l] = vv[e];
+        }
       }
     }
   }
@@ -927,17 +1021,23 @@ struct TailShape {
 
 TailShape tail_shape(const LaunchCtx& c) {
   const long long units = (long long)c.st.layers * c.st.batch * c.st.H;
-  const int P = c.max_prefix;
+  const int P = c.max_prefix, sms = device_sm_count();
   TailShape t;
   t.cs = 1;
-  if (units >= device_sm_count() / 2 && P <= kTailCacheCapSolo) {
-    // many units: one CTA each
-  } else {
+  // Many heads, or heads of a block of positions or less: a CTA each (an exchange across a cluster costs
+  // more than another block).  Few long heads: up to eight CTAs each.
+  if (!(units >= sms / 2 && P <= kTailCacheCapSolo))
     while (t.cs < kTailMaxCluster && tail_chunk(P, t.cs) > 4096) t.cs *= 2;
-  }
   t.chunk = tail_chunk(P, t.cs);
-  t.threads = t.chunk <= 2048 ? 256 : t.chunk <= 4096 ? 512 : 1024;
-  if (units * t.cs <= device_sm_count()) t.threads = t.chunk <= 1024 ? 256 : t.chunk <= 2048 ? 512 : 1024;
+  // A CTA alone on its SM: 1024 threads (a block of 4096 positions), fewer when the slice is shorter.  More
+  // CTAs than SMs: smaller ones side by side, as many as there are and as shared memory holds (heads of
+  // 7300: 256 threads 47 us, 1024 70; 256 heads of 16352: 512 threads 41 us, 1024 47).
+  const long long per_sm = (units * t.cs + sms - 1) / sms;
+  t.threads = per_sm >= 3 ? 256 : per_sm == 2 ? 512 : t.chunk <= 1024 ? 256 : t.chunk <= 2048 ? 512 : 1024;
+  if (per_sm > 1)
+    while (t.threads < 1024 &&
+           (1024 / t.threads) * (24576 + (size_t)t.chunk * 17 / 4 + (size_t)t.threads * 32) > 226 * 1024)
+      t.threads *= 2;
   t.cached = t.chunk <= (t.cs == 1 ? kTailCacheCapSolo : kTailCacheCap);
   return t;
 }
@@ -988,7 +1088,7 @@ cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
   a.cached = sh.cached ? 1 : 0;
   if (fused && !a.cached) return cudaErrorInvalidValue;   // callers check tail_can_fuse() first
   // bitmaps of kept and of equal positions, the keys, the pooling stage
-  size_t smem = (size_t)(sh.chunk / 32) * 8;
+  size_t smem = (size_t)tail_keys_at(sh.chunk) * 4;
   if (a.cached) smem += (size_t)sh.chunk * 4;
   if (fused) smem += ((size_t)8 * sh.threads + 64) * 4;
   switch (sh.threads) {
