@@ -293,7 +293,7 @@ int mixkv_similarity_map(const void* X, int32_t heads, int32_t L, int32_t head_d
  *   q                  device, [n_layers, batch, H * G, d] bf16: the token's query per layer
  *   max_rows           upper bound on the rows of one (layer, b, h), e.g. B, or L for a cache
  *                      that was not compressed; rows beyond it are not read.  It only steers
- *                      how many CTAs share one head (the warps of a cluster of 1, 2, 4 or 8
+ *                      how many CTAs share one head (the warps of a cluster of 1 to 8
  *                      CTAs take the rows 16 at a time, each with a running softmax), so any
  *                      length is accepted
  *   out                device, [n_layers, batch, H * G, d] fp32; a head without rows gets zeros

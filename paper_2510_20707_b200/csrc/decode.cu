@@ -3,23 +3,32 @@
 // in one launch.  With one query token and G query heads per KV head the two contractions have
 // 7 .. 16 rows on one side: too few for the 64- or 128-row tcgen05 tiles (nine tenths of such a
 // tile would be padding), too many multiply-adds for the fp32 pipe at HBM speed (2 * 2 * G * 128
-// per 512-byte row pair), so they run as warp-level mma.sync m16n8k16 (bf16 x bf16 -> fp32) with
-// every operand loaded from global memory straight into its fragment, no shared-memory staging:
+// per 512-byte row pair), so they run as warp-level mma.sync m16n8k16 (bf16 x bf16 -> fp32):
 //
-//   * a warp takes 16 cache rows per step.  logits: D[head, row] = q[head, :] . K[row, :],
-//     A = q (held in registers for the whole kernel), B = K rows.  The contraction index may be
-//     permuted freely as long as A and B agree, so a lane takes 64 CONTIGUOUS bytes of its row
-//     (four 16-byte loads) and deals them out over the eight k-steps.
+//   * a warp takes 16 cache rows per step, copied asynchronously into a ring of two (K, V) slot pairs of its own
+//     (rows on a 272-byte pitch); a slot is asked for again as soon as its rows are used.  logits:
+//     D[head, row] = q[head, :] . K[row, :], A = q (held in registers for the whole kernel), B = K rows.  The
+//     contraction index may be permuted freely as long as A and B agree, so a lane takes 64
+//     CONTIGUOUS bytes of its row (four 16-byte loads, in an order that keeps the shared-memory banks
+//     apart) and deals them out over the eight k-steps.
 //   * softmax weights with a running (reference, sum) per head in log2 units; the weights leave
 //     as TWO bf16 (value and remainder), so the value sum is fp32-grade.
 //   * values: D[head, dim] += P[head, row] . V[row, dim].  B wants two rows of one dim per
 //     register: a lane loads 32 contiguous bytes of four rows and byte-permutes pairs of rows
 //     together; which output column a lane's dim lands in is again a free permutation.
 //
+// What bounds it: a step is a serial chain of about 1000 clocks in one warp (two dependent contractions with a
+// softmax between them) behind a DRAM round trip, so the rate is set by the warps per SM and by how far ahead
+// each of them asks.  With the operands of two steps in registers (255 of them) eight warps fit an SM: 896
+// ragged heads of 512 rows on average 69.7 us (3.4 TB/s).  Sixteen warps with one slot pair each: 59.6 us; twelve
+// with two: 52.4 us (4.6 TB/s), and the short chains of few warps gain too (one head of 8192 rows 18.6 -> 15.3 us).
+// (Eight persistent warps that run through the unit boundaries, the next unit taken from the hardware's launch
+// control: 82 us.)
+//
 // The rows of a (layer, sequence, KV head) unit are dealt out in steps of 16 over the warps of a
-// thread-block cluster (1, 2, 4 or 8 CTAs of four warps; as many as fit the GPU in one wave), and
-// a warp keeps two register sets so that the loads of its next step fly while it works.  Warps merge through shared memory, the CTAs of a cluster through distributed
-// shared memory, every CTA taking a slice of the outputs.  Every row is read once.
+// thread-block cluster (1 to 8 CTAs of four warps; as many as fit the GPU in one wave).  Warps
+// merge through shared memory, the CTAs of a cluster through distributed shared memory, every CTA taking a
+// slice of the outputs.  Every row is read once.
 #include <cooperative_groups.h>
 
 #include "tc_common.cuh"
@@ -34,13 +43,22 @@ constexpr int kDecThreads = kDecWarps * 32;
 constexpr int kDecMaxG = 16;
 constexpr int kDecStep = 16;     // cache rows per warp step
 
+constexpr int kDecPitch = 272;                      // bytes between the rows of a slot
+constexpr int kDecSlot = kDecStep * kDecPitch;      // one K or V slot
+constexpr int kDecDepth = 2;                        // steps a warp has on their way or in work
+
 // Floats of dynamic shared memory for GP = 8 or 16 head slots: wacc [warps][GP][132] per-warp
 // value sums, xo [GP][128] the CTA's, wm / wz [warps][16], xm / xz [16], allm / allz [8][16]
 // every rank's (reference, sum) during the cluster merge.
 constexpr int kDecHeadPitch = kHeadDim + 4;   // floats between the heads of a warp's value sums
+__host__ __device__ constexpr size_t dec_warp_bytes(int GP) {
+  const size_t ring = 2 * (size_t)kDecDepth * kDecSlot, sums = (size_t)GP * kDecHeadPitch * 4;
+  return ring > sums ? ring : sums;
+}
 __host__ __device__ constexpr size_t dec_floats(int GP) {
-  return (size_t)kDecWarps * GP * kDecHeadPitch + (size_t)GP * kHeadDim + 2 * kDecWarps * kDecMaxG +
-         2 * kDecMaxG + 2 * 8 * kDecMaxG;
+  return (size_t)GP * kHeadDim + 2 * kDecWarps * kDecMaxG + 2 * kDecMaxG + 2 * 8 * kDecMaxG +
+         // per warp: the K and the V slot, then (the steps are over) its value sums
+         kDecWarps * (dec_warp_bytes(GP) / 4);
 }
 // Slot of dimension `dim` inside a head of a warp's value sums: one pad word per 32 dimensions
 // and a head pitch of 132 put the 32 lanes of a fragment store (8 heads x 4 dimensions 32 apart)
@@ -58,6 +76,16 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
       "{%8, %9}, {%0, %1, %2, %3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// The same with rows 8 .. 15 of A (and of D) zero: two accumulator registers.
+__device__ __forceinline__ void mma_bf16_low(float (&d)[2], const uint32_t a0, const uint32_t a2,
+                                             const uint32_t b0, const uint32_t b1) {
+  asm volatile(
+      "{\n\t.reg .f32 u, v;\n\t"
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, u, v}, {%2, %3, %4, %3}, "
+      "{%5, %6}, {%0, %1, %7, %7};\n\t}"
+      : "+f"(d[0]), "+f"(d[1])
+      : "r"(a0), "r"(0u), "r"(a2), "r"(b0), "r"(b1), "f"(0.f));
 }
 // bf16 pair (x in the low half) of two floats, and what rounding left over.
 __device__ __forceinline__ uint32_t pack_bf16(const float x, const float y) {
@@ -80,18 +108,178 @@ __device__ __forceinline__ float quad_sum(float v) {
   return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
 
+// Sixteen rows of X into a slot: chunk c (16 bytes) of row r at r * 272 + 16 c.  Rows past the end repeat
+// the last row; their weights are zero.
+__device__ __forceinline__ void copy_rows(unsigned char* slot, const __nv_bfloat16* X, const int rb, const int n,
+                                          const int lane) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int r = 2 * i + (lane >> 4), c = lane & 15;
+    const int row = min(rb + r, n - 1);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(slot + r * kDecPitch + 16 * c)),
+                 "l"(X + (size_t)row * kHeadDim + 8 * c)
+                 : "memory");
+  }
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// All copies of this lane but the newest groups (everything asked for after the tile needed now) have landed;
+// with every lane of the warp past this, all rows of that tile.
+__device__ __forceinline__ void copy_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(2 * kDecDepth - 1) : "memory");
+  __syncwarp();
+}
+
+// What a warp holds of a unit: query fragments, value sums, running softmax.  Register pair i of lane (g, t)
+// covers dimensions 32 t + 8 c .. + 7, c = (i + 2 (t / 2)) % 4, of heads g and g + 8 (two k-steps: the first two
+// of four dimensions as a0 / a1, the last two as a2 / a3).  Value sums: tile dt, registers 0 1 = head g,
+// dimensions 16 (2t) + dt and 16 (2t + 1) + (dt ^ 8); registers 2 3 = head g + 8.
+template <bool WIDE>
+struct DecState {
+  static constexpr int R = WIDE ? 4 : 2;
+  uint32_t qa[8][R];
+  float acc[16][R];
+  float m0, m1, z0, z1;
+
+  __device__ __forceinline__ void start(const __nv_bfloat16* q, const int G, const int g, const int t) {
+    const uint4* q0 = reinterpret_cast<const uint4*>(q + (size_t)g * kHeadDim + 32 * t);
+    const uint4* q1 = reinterpret_cast<const uint4*>(q + (size_t)(g + 8) * kHeadDim + 32 * t);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int c = (i + 2 * (t >> 1)) & 3;
+      uint4 u0 = make_uint4(0, 0, 0, 0), u1 = u0;
+      if (g < G) u0 = __ldg(q0 + c);
+      if (WIDE && g + 8 < G) u1 = __ldg(q1 + c);
+      if constexpr (WIDE) {
+        qa[2 * i][0] = u0.x, qa[2 * i][2] = u0.y, qa[2 * i + 1][0] = u0.z, qa[2 * i + 1][2] = u0.w;
+        qa[2 * i][1] = u1.x, qa[2 * i][3] = u1.y, qa[2 * i + 1][1] = u1.z, qa[2 * i + 1][3] = u1.w;
+      } else {
+        qa[2 * i][0] = u0.x, qa[2 * i][1] = u0.y, qa[2 * i + 1][0] = u0.z, qa[2 * i + 1][1] = u0.w;
+      }
+    }
+#pragma unroll
+    for (int dt = 0; dt < 16; ++dt)
+#pragma unroll
+      for (int c = 0; c < R; ++c) acc[dt][c] = 0.f;
+    m0 = m1 = -INFINITY, z0 = z1 = 0.f;
+  }
+
+  // logits of a step: s[j] registers 0 1 = head g, rows 8 j + 2t, + 1; 2 3 = head g + 8
+  __device__ __forceinline__ void logits(const unsigned char* slot, const int g, const int t, float (&s)[2][R]) const {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const unsigned char* row = slot + (8 * j + g) * kDecPitch + 64 * t;
+#pragma unroll
+      for (int c = 0; c < R; ++c) s[j][c] = 0.f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint4 k = *reinterpret_cast<const uint4*>(row + 16 * ((i + 2 * (t >> 1)) & 3));
+        if constexpr (WIDE) {
+          mma_bf16(s[j], qa[2 * i], k.x, k.y);
+          mma_bf16(s[j], qa[2 * i + 1], k.z, k.w);
+        } else {
+          mma_bf16_low(s[j], qa[2 * i][0], qa[2 * i][1], k.x, k.y);
+          mma_bf16_low(s[j], qa[2 * i + 1][0], qa[2 * i + 1][1], k.z, k.w);
+        }
+      }
+    }
+  }
+
+  // softmax weights of one head (registers c0, c0 + 1 of s) under its running reference, log2 units; `left`: rows
+  // of the unit from this step on
+  template <int C0>
+  __device__ __forceinline__ void weights(float (&s)[2][R], float& m, float& z, const int left,
+                                          const float scale_log2e, const int t) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        s[j][C0 + c] = 8 * j + 2 * t + c < left ? s[j][C0 + c] * scale_log2e : -INFINITY;
+    const float mx = quad_max(fmaxf(fmaxf(s[0][C0], s[0][C0 + 1]), fmaxf(s[1][C0], s[1][C0 + 1])));
+    const float mn = fmaxf(m, mx), f = exp2f(m - mn);   // mx is finite: the step has a row
+    if (f != 1.f) {
+      z *= f;
+#pragma unroll
+      for (int dt = 0; dt < 16; ++dt) acc[dt][C0] *= f, acc[dt][C0 + 1] *= f;
+    }
+    m = mn;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      s[j][C0] = exp2f(s[j][C0] - mn);
+      s[j][C0 + 1] = exp2f(s[j][C0 + 1] - mn);
+      z += s[j][C0] + s[j][C0 + 1];
+    }
+  }
+
+  // values: the weights as bf16 value + bf16 remainder (A fragments over the 16 rows of the step) times V;
+  // tile dt takes dimension 16 g + (dt ^ 8 (g & 1)) of this lane's four rows
+  __device__ __forceinline__ void values(const unsigned char* slot, const int g, const int t, const float (&p)[2][R]) {
+    uint32_t ahi[4] = {0, 0, 0, 0}, alo[4] = {0, 0, 0, 0};
+    split_bf16(p[0][0], p[0][1], ahi[0], alo[0]);
+    split_bf16(p[1][0], p[1][1], ahi[2], alo[2]);
+    if constexpr (WIDE) {
+      split_bf16(p[0][2], p[0][3], ahi[1], alo[1]);
+      split_bf16(p[1][2], p[1][3], ahi[3], alo[3]);
+    }
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+      uint4 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        v[u] = *reinterpret_cast<const uint4*>(slot + (2 * t + (u & 1) + 8 * (u >> 1)) * kDecPitch + 32 * g +
+                                               16 * (half ^ (g & 1)));
+#pragma unroll
+      for (int d = 0; d < 8; ++d) {
+        const int dt = 8 * half + d;
+        const uint32_t sel = (d & 1) ? 0x7632u : 0x5410u;
+        const uint32_t b0 = __byte_perm(word_of(v[0], d >> 1), word_of(v[1], d >> 1), sel);
+        const uint32_t b1 = __byte_perm(word_of(v[2], d >> 1), word_of(v[3], d >> 1), sel);
+        if constexpr (WIDE) {
+          mma_bf16(acc[dt], ahi, b0, b1);
+          mma_bf16(acc[dt], alo, b0, b1);
+        } else {
+          mma_bf16_low(acc[dt], ahi[0], ahi[2], b0, b1);
+          mma_bf16_low(acc[dt], alo[0], alo[2], b0, b1);
+        }
+      }
+    }
+  }
+};
+
+// A warp's value sums and (reference, sum) pairs into shared memory.
+template <bool WIDE>
+__device__ __forceinline__ void store_partial(const DecState<WIDE>& st, float* wacc, float* wm, float* wz,
+                                              const int g, const int t) {
+  const float z0 = quad_sum(st.z0), z1 = quad_sum(st.z1);
+  float* w0 = wacc + (size_t)g * kDecHeadPitch;
+#pragma unroll
+  for (int dt = 0; dt < 16; ++dt) {
+    w0[dec_slot(16 * (2 * t) + dt)] = st.acc[dt][0];
+    w0[dec_slot(16 * (2 * t + 1) + (dt ^ 8))] = st.acc[dt][1];
+    if constexpr (WIDE) {
+      w0[8 * kDecHeadPitch + dec_slot(16 * (2 * t) + dt)] = st.acc[dt][2];
+      w0[8 * kDecHeadPitch + dec_slot(16 * (2 * t + 1) + (dt ^ 8))] = st.acc[dt][3];
+    }
+  }
+  if (t == 0) {
+    wm[g] = st.m0, wz[g] = z0;
+    wm[g + 8] = WIDE ? st.m1 : -INFINITY, wz[g + 8] = WIDE ? z1 : 0.f;
+  }
+}
+
 // grid: n_layers * batch * H * S, clusters of S.  WIDE: more than eight query heads per KV head
 // (head slots 8..15 of the tiles carry data).
+constexpr int kDecPerSm = 3;   // CTAs per SM (12 warps, 208 KB of slots)
 template <bool WIDE>
-__global__ void __launch_bounds__(kDecThreads, 2)
+__global__ void __launch_bounds__(kDecThreads, kDecPerSm)
 k_decode_attention(const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __restrict__ Vc,
                    const int* __restrict__ row_offsets, const long long rows_cap,
                    const __nv_bfloat16* __restrict__ q, const int BH, const int H, const int G,
                    const float scale_log2e, const int max_rows, float* __restrict__ out) {
   constexpr int GP = WIDE ? 16 : 8;
   extern __shared__ __align__(16) float dsm[];
-  float* wacc = dsm;                                   // [warps][GP][kDecHeadPitch]
-  float* xo = wacc + kDecWarps * GP * kDecHeadPitch;   // [GP][128]
+  constexpr int kWarpFloats = (int)(dec_warp_bytes(GP) / 4);
+  float* wacc = dsm;                                   // [warps]: slots, then [GP][kDecHeadPitch]
+  float* xo = wacc + kDecWarps * kWarpFloats;          // [GP][128]
   float* wm = xo + GP * kHeadDim;                      // [warps][16]
   float* wz = wm + kDecWarps * kDecMaxG;               // [warps][16]
   float* xm = wz + kDecWarps * kDecMaxG;               // [16]
@@ -103,164 +291,54 @@ k_decode_attention(const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __
   const int unit = blockIdx.x / S, layer = unit / BH, bh = unit % BH, b = bh / H, h = bh % H;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, t = lane & 3;
+  const size_t qoff = (((size_t)layer * (BH / H) + b) * H + h) * (size_t)G * kHeadDim;
   pdl_launch_dependents();
   pdl_wait();
   const int* ro = row_offsets + (size_t)layer * (BH + 1);
   const int r0 = ro[bh], n = min(ro[bh + 1] - r0, max_rows);
   const __nv_bfloat16* Kb = Kc + ((size_t)layer * rows_cap + r0) * kHeadDim;
   const __nv_bfloat16* Vb = Vc + ((size_t)layer * rows_cap + r0) * kHeadDim;
-  const size_t qoff = (((size_t)layer * (BH / H) + b) * H + h) * (size_t)G * kHeadDim;
-
-  // ---- query fragments: k-step kt of lane (g, t) covers dimensions 32 t + 4 kt .. + 3 of heads
-  // g and g + 8, the first two as a0 / a1, the last two as a2 / a3
-  uint32_t qa[8][4];
-  {
-    const uint4* q0 = reinterpret_cast<const uint4*>(q + qoff + (size_t)g * kHeadDim + 32 * t);
-    const uint4* q1 = reinterpret_cast<const uint4*>(q + qoff + (size_t)(g + 8) * kHeadDim + 32 * t);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      uint4 u0 = make_uint4(0, 0, 0, 0), u1 = u0;
-      if (g < G) u0 = __ldg(q0 + i);
-      if (WIDE && g + 8 < G) u1 = __ldg(q1 + i);
-      qa[2 * i][0] = u0.x, qa[2 * i][2] = u0.y, qa[2 * i + 1][0] = u0.z, qa[2 * i + 1][2] = u0.w;
-      qa[2 * i][1] = u1.x, qa[2 * i][3] = u1.y, qa[2 * i + 1][1] = u1.z, qa[2 * i + 1][3] = u1.w;
-    }
-  }
-  // value sums: tile dt, registers 0 1 = head g, dimensions 16 (2t) + dt and 16 (2t + 1) + dt;
-  // registers 2 3 = head g + 8
-  float acc[16][4];
-#pragma unroll
-  for (int dt = 0; dt < 16; ++dt)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[dt][c] = 0.f;
-  float m0 = -INFINITY, m1 = -INFINITY, z0 = 0.f, z1 = 0.f;
-
+  DecState<WIDE> st;
   const int nsteps = (n + kDecStep - 1) / kDecStep;
-  // All loads of a step: K rows rb + 8 j + g (64 bytes from 64 t), V rows rb + 2t, 2t + 1,
-  // 2t + 8, 2t + 9 (32 bytes from 32 g).  Rows past the end repeat the last row; their weights
-  // are zero.
-  auto load_step = [&](const int step, uint4 (&kq)[2][4], uint4 (&vq)[4][2]) {
-    const int rb = step * kDecStep;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int row = min(rb + 8 * j + g, n - 1);
-      const uint4* p = reinterpret_cast<const uint4*>(Kb + (size_t)row * kHeadDim + 32 * t);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) kq[j][i] = __ldg(p + i);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int row = min(rb + 2 * t + (u & 1) + 8 * (u >> 1), n - 1);
-      const uint4* p = reinterpret_cast<const uint4*>(Vb + (size_t)row * kHeadDim + 16 * g);
-      vq[u][0] = __ldg(p);
-      vq[u][1] = __ldg(p + 1);
-    }
-  };
-  auto work_step = [&](const int step, const uint4 (&kq)[2][4], const uint4 (&vq)[4][2]) {
-    const int rb = step * kDecStep;
-    // ---- logits: s[j] registers 0 1 = head g, rows rb + 8 j + 2t, + 1; 2 3 = head g + 8
-    float s[2][4];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) s[j][c] = 0.f;
-#pragma unroll
-      for (int kt = 0; kt < 8; ++kt)
-        mma_bf16(s[j], qa[kt], word_of(kq[j][kt >> 1], 2 * (kt & 1)),
-                 word_of(kq[j][kt >> 1], 2 * (kt & 1) + 1));
-    }
-    // ---- softmax weights under the running reference of each head (log2 units)
-    float p[2][4];
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        p[j][c] = rb + 8 * j + 2 * t + (c & 1) < n ? s[j][c] * scale_log2e : -INFINITY;
-    {
-      const float mx = quad_max(fmaxf(fmaxf(p[0][0], p[0][1]), fmaxf(p[1][0], p[1][1])));
-      const float mn = fmaxf(m0, mx), f = exp2f(m0 - mn);   // mx is finite: the step has a row
-      if (f != 1.f) {
-        z0 *= f;
-#pragma unroll
-        for (int dt = 0; dt < 16; ++dt) acc[dt][0] *= f, acc[dt][1] *= f;
-      }
-      m0 = mn;
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        p[j][0] = exp2f(p[j][0] - mn);
-        p[j][1] = exp2f(p[j][1] - mn);
-        z0 += p[j][0] + p[j][1];
-      }
-    }
-    if (WIDE) {
-      const float mx = quad_max(fmaxf(fmaxf(p[0][2], p[0][3]), fmaxf(p[1][2], p[1][3])));
-      const float mn = fmaxf(m1, mx), f = exp2f(m1 - mn);
-      if (f != 1.f) {
-        z1 *= f;
-#pragma unroll
-        for (int dt = 0; dt < 16; ++dt) acc[dt][2] *= f, acc[dt][3] *= f;
-      }
-      m1 = mn;
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        p[j][2] = exp2f(p[j][2] - mn);
-        p[j][3] = exp2f(p[j][3] - mn);
-        z1 += p[j][2] + p[j][3];
-      }
-    }
-    // the weights as bf16 value + bf16 remainder: A fragments over the 16 rows of the step
-    uint32_t ahi[4] = {0, 0, 0, 0}, alo[4] = {0, 0, 0, 0};
-    split_bf16(p[0][0], p[0][1], ahi[0], alo[0]);
-    split_bf16(p[1][0], p[1][1], ahi[2], alo[2]);
-    if (WIDE) {
-      split_bf16(p[0][2], p[0][3], ahi[1], alo[1]);
-      split_bf16(p[1][2], p[1][3], ahi[3], alo[3]);
-    }
-    // ---- values: tile dt takes dimension 16 g + dt of this lane's four rows
-#pragma unroll
-    for (int dt = 0; dt < 16; ++dt) {
-      const int w = dt >> 1;
-      const uint32_t sel = (dt & 1) ? 0x7632u : 0x5410u;
-      const uint32_t b0 = __byte_perm(word_of(vq[0][w >> 2], w & 3), word_of(vq[1][w >> 2], w & 3), sel);
-      const uint32_t b1 = __byte_perm(word_of(vq[2][w >> 2], w & 3), word_of(vq[3][w >> 2], w & 3), sel);
-      mma_bf16(acc[dt], ahi, b0, b1);
-      mma_bf16(acc[dt], alo, b0, b1);
-    }
-  };
-  // two register sets: the loads of a warp's next step are in flight while it works on this one
+  float* mine = wacc + warp * kWarpFloats;
   {
+    unsigned char* ring = reinterpret_cast<unsigned char*>(mine);   // [depth] x (K slot, V slot)
     const int stride = S * kDecWarps;
-    uint4 kA[2][4], vA[4][2], kB[2][4], vB[4][2];
     int step = crank * kDecWarps + warp;
-    if (step < nsteps) load_step(step, kA, vA);
-    while (step < nsteps) {
-      if (step + stride < nsteps) load_step(step + stride, kB, vB);
-      work_step(step, kA, vA);
-      step += stride;
-      if (step >= nsteps) break;
-      if (step + stride < nsteps) load_step(step + stride, kA, vA);
-      work_step(step, kB, vB);
-      step += stride;
+#pragma unroll
+    for (int d = 0; d < kDecDepth; ++d) {
+      const int ahead = step + d * stride;
+      if (ahead < nsteps) copy_rows(ring + 2 * d * kDecSlot, Kb, ahead * kDecStep, n, lane);
+      copy_commit();
+      if (ahead < nsteps) copy_rows(ring + (2 * d + 1) * kDecSlot, Vb, ahead * kDecStep, n, lane);
+      copy_commit();
     }
+    st.start(q + qoff, G, g, t);
+    for (int d = 0; step < nsteps; step += stride, d = d + 1 == kDecDepth ? 0 : d + 1) {
+      unsigned char* sK = ring + 2 * d * kDecSlot;
+      unsigned char* sV = sK + kDecSlot;
+      const int ahead = step + kDecDepth * stride;
+      const int left = n - step * kDecStep;
+      float p[2][DecState<WIDE>::R];
+      copy_wait();     // K of this step
+      st.logits(sK, g, t, p);
+      __syncwarp();    // every lane has read the slot
+      if (ahead < nsteps) copy_rows(sK, Kb, ahead * kDecStep, n, lane);
+      copy_commit();
+      st.template weights<0>(p, st.m0, st.z0, left, scale_log2e, t);
+      if constexpr (WIDE) st.template weights<2>(p, st.m1, st.z1, left, scale_log2e, t);
+      copy_wait();     // V of this step
+      st.values(sV, g, t, p);
+      __syncwarp();
+      if (ahead < nsteps) copy_rows(sV, Vb, ahead * kDecStep, n, lane);
+      copy_commit();
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
   }
 
   // ---- the warps of the CTA merge through shared memory
-  z0 = quad_sum(z0);
-  z1 = quad_sum(z1);
-#pragma unroll
-  for (int dt = 0; dt < 16; ++dt) {
-    float* w0 = wacc + ((size_t)warp * GP + g) * kDecHeadPitch;
-    w0[dec_slot(16 * (2 * t) + dt)] = acc[dt][0];
-    w0[dec_slot(16 * (2 * t + 1) + dt)] = acc[dt][1];
-    if (WIDE) {
-      w0[8 * kDecHeadPitch + dec_slot(16 * (2 * t) + dt)] = acc[dt][2];
-      w0[8 * kDecHeadPitch + dec_slot(16 * (2 * t + 1) + dt)] = acc[dt][3];
-    }
-  }
-  if (t == 0) {
-    wm[warp * kDecMaxG + g] = m0, wz[warp * kDecMaxG + g] = z0;
-    wm[warp * kDecMaxG + g + 8] = WIDE ? m1 : -INFINITY, wz[warp * kDecMaxG + g + 8] = WIDE ? z1 : 0.f;
-  }
+  store_partial(st, mine, wm + warp * kDecMaxG, wz + warp * kDecMaxG, g, t);
   __syncthreads();
   for (int e = tid; e < GP * kHeadDim; e += kDecThreads) {
     const int head = e / kHeadDim, dim = e % kHeadDim;
@@ -272,7 +350,7 @@ k_decode_attention(const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __
     for (int w = 0; w < kDecWarps; ++w) {
       const float mw = wm[w * kDecMaxG + head];
       const float sc = mw == -INFINITY ? 0.f : exp2f(mw - M);
-      num = fmaf(wacc[((size_t)w * GP + head) * kDecHeadPitch + dec_slot(dim)], sc, num);
+      num = fmaf(wacc[w * kWarpFloats + head * kDecHeadPitch + dec_slot(dim)], sc, num);
       den = fmaf(wz[w * kDecMaxG + head], sc, den);
     }
     xo[e] = num;
@@ -307,6 +385,7 @@ k_decode_attention(const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __
   cluster.sync();   // a CTA's shared memory stays alive until its peers have read it
 }
 
+
 }  // namespace
 }  // namespace mixkv
 
@@ -332,21 +411,31 @@ extern "C" int mixkv_decode_attention(const void* K_cache, const void* V_cache,
   }
   const long long units = (long long)n_layers * batch * kv_heads;
   if (units * 8 > 0x7fffffffLL) return MIXKV_ERR_UNSUPPORTED;
-  // CTAs per unit: as many as still fit the GPU in one wave (two CTAs of four warps per SM: the
-  // two register sets of a warp hold 16 KB of loads in flight) while every warp keeps at least
-  // two steps to overlap
-  const long long steps = ((long long)max_rows + kDecStep - 1) / kDecStep;
-  int S = 1;
-  while (S < 8 && units * (2 * S) <= 2LL * device_sm_count() && 2LL * (2 * S) * kDecWarps <= steps)
-    S *= 2;
   const bool wide = gqa_ratio > 8;
+  // CTAs per unit: as many as still fit the GPU in one wave while every warp keeps a step (one head of 512
+  // rows on 8 CTAs 5.8 us, on 4 6.4; 112 heads of 512 rows on 3 CTAs each 11.5 us, on 2 12.8)
+  const long long slots = (long long)kDecPerSm * device_sm_count();
+  const long long steps = ((long long)max_rows + kDecStep - 1) / kDecStep;
+  long long most = slots / units < steps / kDecWarps ? slots / units : steps / kDecWarps;
+  const int S = most < 1 ? 1 : most > 8 ? 8 : (int)most;
   const size_t smem = dec_floats(wide ? 16 : 8) * 4;
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)kHeadDim);
-  const cudaError_t e = launch_pdl(
-      wide ? k_decode_attention<true> : k_decode_attention<false>, dim3((unsigned)(units * S)),
-      dim3(kDecThreads), smem, (cudaStream_t)stream, S,
-      reinterpret_cast<const __nv_bfloat16*>(K_cache), reinterpret_cast<const __nv_bfloat16*>(V_cache),
-      out_row_offsets, (long long)rows_cap, reinterpret_cast<const __nv_bfloat16*>(q), batch * kv_heads,
-      kv_heads, gqa_ratio, scale * kLog2e, max_rows, out);
+  const __nv_bfloat16 *K = reinterpret_cast<const __nv_bfloat16*>(K_cache),
+                      *V = reinterpret_cast<const __nv_bfloat16*>(V_cache),
+                      *qq = reinterpret_cast<const __nv_bfloat16*>(q);
+  auto kernel = wide ? k_decode_attention<true> : k_decode_attention<false>;
+  if (smem > 48 * 1024) {
+    static bool done[2][64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return MIXKV_ERR_CUDA;
+    if (dev < 0 || dev >= 64 || !done[wide][dev]) {
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return MIXKV_ERR_CUDA;
+      if (dev >= 0 && dev < 64) done[wide][dev] = true;
+    }
+  }
+  const cudaError_t e = launch_pdl(kernel, dim3((unsigned)(units * S)), dim3(kDecThreads), smem, (cudaStream_t)stream, S,
+                                   K, V, out_row_offsets, (long long)rows_cap, qq, batch * kv_heads, kv_heads,
+                                   gqa_ratio, scale * kLog2e, max_rows, out);
   return e == cudaSuccess ? MIXKV_OK : MIXKV_ERR_CUDA;
 }

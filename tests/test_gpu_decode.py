@@ -96,6 +96,38 @@ def test_step_edges_and_head_counts(G):
         assert np.allclose(out[l], ref, rtol=RTOL, atol=ATOL), f"layer {l}"
 
 
+@pytest.mark.parametrize("NL,batch,H,G,lo,hi", [
+    (4, 16, 8, 7, 0, 40),          # 512 units: empty heads, fewer rows than the warps of a CTA take
+    (3, 13, 9, 16, 1, 300),        # wide heads, a unit count that no number of CTAs divides
+    (28, 3, 4, 1, 120, 140)])      # steps of all eight warps and one more
+def test_more_units_than_one_wave(NL, batch, H, G, lo, hi):
+    rng = np.random.default_rng(NL * batch)
+    counts = rng.integers(lo, hi + 1, (NL, batch * H))
+    counts[0, 0], counts[-1, -1] = lo, hi
+    cap = int(counts.sum(1).max())
+    K = synth.f32_to_bf16_bits(rng.standard_normal((NL, cap, 128)).astype(np.float32))
+    V = synth.f32_to_bf16_bits(rng.standard_normal((NL, cap, 128)).astype(np.float32))
+    q = synth.f32_to_bf16_bits(rng.standard_normal((NL, batch, H * G, 128)).astype(np.float32))
+    offs = np.concatenate([np.zeros((NL, 1), np.int64), counts.cumsum(1)], 1).astype(np.int32)
+    dev = [torch.from_numpy(x.view(np.int16)).cuda().view(torch.bfloat16) for x in (K, V, q)]
+    out = binding.decode_attention(dev[0], dev[1], torch.from_numpy(offs).cuda(), dev[2], H, G, hi)
+    again = binding.decode_attention(dev[0], dev[1], torch.from_numpy(offs).cuda(), dev[2], H, G, hi)
+    torch.cuda.synchronize()
+    assert torch.equal(out, again)
+    k, v, qq = (synth.bf16_bits_to_f32(x).astype(np.float64) for x in (K, V, q))
+    got = out.cpu().numpy()
+    for l in range(NL):
+        for u in range(batch * H):
+            a, e = offs[l, u], offs[l, u + 1]
+            rows = got[l, u // H, (u % H) * G:(u % H + 1) * G]
+            if a == e:
+                assert (rows == 0).all()
+                continue
+            s = qq[l, u // H, (u % H) * G:(u % H + 1) * G] @ k[l, a:e].T / np.sqrt(128.0)
+            p = np.exp(s - s.max(1, keepdims=True))
+            assert np.allclose(rows, p @ v[l, a:e] / p.sum(1, keepdims=True), rtol=2e-4, atol=2e-5), (l, u)
+
+
 def test_repeated_calls_are_bit_identical():
     # the steps of a head go to fixed warps and the partial results are merged in a fixed order
     # (warps through shared memory, CTAs through distributed shared memory): twenty calls on the

@@ -280,28 +280,29 @@ def test_whole_head_ctas_select_exactly(levels):
 @pytest.mark.parametrize("H,n,levels,want", [
     (3, 31, 0, 7), (2, 257, 4, 100), (2, 1025, 0, 3), (2, 4064, 1, 500),      # one CTA per head, 256 to 1024 threads
     (2, 9000, 0, 700), (2, 9000, 40, 2000), (1, 33000, 0, 1), (1, 33000, 700, 1500),   # clusters of 4 and 8
-    (150, 300, 20, 60), (300, 5000, 0, 129),                                  # more CTAs than SMs
+    (200, 300, 20, 60), (500, 2000, 0, 129),                                  # more CTAs than SMs
     (1, 140000, 300, 900)])                                                   # keys not held in shared memory
 def test_threshold_search_edges(H, n, levels, want):
     # one, a few or no repeated values (levels = number of distinct scores), the range spread over many
     # octaves and both signs
     rng = np.random.default_rng(H * n + want)
-    W = 32
-    heads = min(H, 60)
-    layers_of = -(-H // heads)
-    for rep in range(layers_of):
-        s = rng.standard_normal((heads, n)).astype(np.float32) * np.exp2(rng.integers(-20, 20, (heads, n)))
-        if levels:
-            s = rng.choice(s.reshape(-1)[:levels], size=(heads, n))
-        s = s.astype(np.float32)
-        s[0, 0], s[0, -1] = 0.0, -0.0
-        pg = binding.Params(kv_heads=heads, gqa_ratio=1, window=W, budget=W + want)
-        out = binding.select(torch.from_numpy(s).cuda(), pg)
-        torch.cuda.synchronize()
-        idx = out["idx"].cpu().numpy().reshape(heads, want)
+    W, batch = 32, max(1, H // 50)            # many heads: several sequences of 50
+    heads = H // batch
+    s = rng.standard_normal((heads, batch * n)).astype(np.float32) * np.exp2(rng.integers(-20, 20, (heads, batch * n)))
+    if levels:
+        s = rng.choice(s.reshape(-1)[:levels], size=(heads, batch * n))
+    s = s.astype(np.float32)
+    s[0, 0], s[0, -1] = 0.0, -0.0
+    pg = binding.Params(kv_heads=heads, gqa_ratio=1, window=W, budget=W + want)
+    cu = None if batch == 1 else [b * (n + W) for b in range(batch + 1)]
+    out = binding.select(torch.from_numpy(s).cuda(), pg, cu_seqlens=cu)
+    torch.cuda.synchronize()
+    idx = out["idx"].cpu().numpy().reshape(batch, heads, want)
+    for b in range(batch):
         for h in range(heads):
-            order = np.lexsort((np.arange(n), -s[h].astype(np.float64)))
-            assert (idx[h] == np.sort(order[:want])).all(), (rep, h)
+            row = s[h, b * n:(b + 1) * n]
+            order = np.lexsort((np.arange(n), -row.astype(np.float64)))
+            assert (idx[b, h] == np.sort(order[:want])).all(), (b, h)
 
 
 def test_long_sequence_cluster_tail():
