@@ -65,37 +65,10 @@ __device__ __forceinline__ void drain_ring(uint64_t* full, int stages, int it) {
   }
 }
 
-// Packed fp32 pairs (one instruction for two lanes of arithmetic).
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float a, float b) {
-  f32x2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
 __device__ __forceinline__ f32x2 ex2_pair(f32x2 t2) {
   float a0, a1;
   unpack2(t2, a0, a1);
   return pack2(ex2(a0), ex2(a1));
-}
-
-// The two bf16 of a word as a packed fp32 pair (low half first), built in place in the 64-bit
-// register (a pair assembled from two separate floats costs moves).
-__device__ __forceinline__ f32x2 bf16x2_wide(const uint32_t w) {
-  return ((unsigned long long)(w & 0xffff0000u) << 32) | (unsigned long long)(w << 16);
 }
 
 constexpr size_t kSmemLimit = 227 * 1024;   // dynamic shared memory a CTA may ask for
@@ -667,6 +640,13 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     tma_prefetch_desc(&tmQ);
   }
   if (warp == kWarpTmaV && lane == 0) tma_prefetch_desc(&tmV);
+  if (warp >= kP2AuxWarp0) {   // B rows past the three parts of the mean key stay zero
+    const int vt = tid - kP2AuxWarp0 * 32;
+    unsigned char* hb = sQ + (vt >> 6) * NB * 128 + (vt & 7) * 2;
+#pragma unroll
+    for (int e = 3; e < kExtraRows; ++e)
+      *reinterpret_cast<__nv_bfloat16*>(hb + sw128_offset(NQ + e, (vt & 63) >> 3)) = __float2bfloat16_rn(0.f);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -884,18 +864,6 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
       const int L = st.cu[sg.b + 1] - st.cu[sg.b], P = L - W;
       const float ks = fold_key_sums(ws.ksum, pass1_segments(st, sg), vt);
       const float kb = ks / (float)L;   // mean unit key
-      if (sg.t0 == 0) {                 // the same in all 128 threads
-        const float n2 = warp_sum(ks * ks);
-        if (lane == 0) sred[44 + (warp - kP2AuxWarp0)] = n2;
-        named_bar_sync(4, 128);
-        if (vt == 0) {
-          const double nn = ((double)sred[44] + (double)sred[45]) + ((double)sred[46] + (double)sred[47]);
-          const double T = (double)L;
-          const float r = (float)((nn - T) / (T * (T - 1.0)));   // Eq. 4
-          ws.rbar[sg.unit()] = r;
-          if (rbar_out) rbar_out[sg.unit()] = r;
-        }
-      }
       __nv_bfloat16 parts[3];
       parts[0] = __float2bfloat16_rn(kb);
       const float r1 = kb - __bfloat162float(parts[0]);
@@ -909,15 +877,24 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         unsigned char* hb = sQ + (vt >> 6) * NB * 128 + (vt & 7) * 2;
         const int chunk = (vt & 63) >> 3;
 #pragma unroll
-        for (int e = 0; e < kExtraRows; ++e) {
-          if (e < 3 || segn == 0)
-            *reinterpret_cast<__nv_bfloat16*>(hb + sw128_offset(NQ + e, chunk)) =
-                e < 3 ? parts[e] : __float2bfloat16_rn(0.f);
-        }
+        for (int e = 0; e < 3; ++e)
+          *reinterpret_cast<__nv_bfloat16*>(hb + sw128_offset(NQ + e, chunk)) = parts[e];
       }
       fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->kbready);
+      if (lane == 0) mbar_arrive(&bars->kbready);   // the MMA may start: the rest is off its path
+      if (sg.t0 == 0) {                 // the same in all 128 threads
+        const float n2 = warp_sum(ks * ks);
+        if (lane == 0) sred[44 + (warp - kP2AuxWarp0)] = n2;
+        named_bar_sync(4, 128);
+        if (vt == 0) {
+          const double nn = ((double)sred[44] + (double)sred[45]) + ((double)sred[46] + (double)sred[47]);
+          const double T = (double)L;
+          const float r = (float)((nn - T) / (T * (T - 1.0)));   // Eq. 4
+          ws.rbar[sg.unit()] = r;
+          if (rbar_out) rbar_out[sg.unit()] = r;
+        }
+      }
       ++segn;
       float vmin = INFINITY, vmax = -INFINITY, vsum = 0.f;
       float* vnorm = ws.vnorm + ppos(st, sg.layer, sg.h, sg.b, 0);

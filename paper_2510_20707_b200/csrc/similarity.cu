@@ -17,28 +17,24 @@ namespace {
 
 constexpr int kSumWarps = 8;
 constexpr int kSumThreads = kSumWarps * 32;
-constexpr int kSumRows = 32;        // rows a warp holds in registers at a time (8 KB of loads in flight)
+constexpr int kSumStep = 16;        // rows a warp holds in registers at a time (4 KB of loads in flight)
+constexpr int kSumSteps = 2;        // steps of a warp, at least
+constexpr int kSumRows = kSumStep * kSumSteps;
 constexpr int kSumMaxCluster = 8;
 
 // Three layouts of the work of k_block_sums, by the rows per block.
 enum { kRowsOne = 0,    // block == 1: every row leaves as its own "sum"
-       kRowsFew = 1,    // block <= 32: a warp takes whole blocks
+       kRowsFew = 1,    // block <= 16: a warp takes whole blocks
        kRowsMany = 2 }; // longer blocks: the warps of a CTA (or of a cluster) share one
 
 __host__ __device__ constexpr int sum_mode(int block) {
-  return block == 1 ? kRowsOne : block <= kSumRows ? kRowsFew : kRowsMany;
+  return block == 1 ? kRowsOne : block <= kSumStep ? kRowsFew : kRowsMany;
 }
 // Blocks one CTA (or cluster) takes.
 __host__ __device__ inline int blocks_per_cta(int block) {
-  if (block <= kSumRows) return kSumWarps * (kSumRows / block);
+  if (block <= kSumStep) return kSumWarps * kSumSteps * (kSumStep / block);
   const int sub = (block + kSumRows - 1) / kSumRows;
   return sub < kSumWarps ? kSumWarps / sub : 1;
-}
-// Bits of the rows a .. b-1 of a warp's 32 rows, where row 2 i + half is bit 16 half + i.
-__device__ __forceinline__ unsigned row_bits(const int a, const int b) {
-  const unsigned even = ((1u << ((b + 1) >> 1)) - 1u) & ~((1u << ((a + 1) >> 1)) - 1u);
-  const unsigned odd = ((1u << (b >> 1)) - 1u) & ~((1u << (a >> 1)) - 1u);
-  return even | (odd << 16);
 }
 
 // x as a sum of bf16 parts, most significant first (8 mantissa bits each).
@@ -63,17 +59,16 @@ __device__ __forceinline__ void split_parts(const float (&x)[8], uint4 (&part)[P
 // number of non-zero rows of every block, and per slice (what one CTA or cluster read) the sum of
 // its unit rows and its non-zero rows, from which the head mean comes.
 //
-// HBM bound: every row is read once, 16 lanes of 16 bytes to a row, all 32 rows of a warp's step
-// asked for before the first is used (8 KB per warp, 16 warps per SM).  The 32 squared norms of a
-// step are reduced by folding (15 exchanges per lane instead of 64 for 16 butterflies).  131072 rows
-// (four heads of 32768) in blocks of 256: 13.3 us before (four rows per warp in flight), see the
-// dispatch for the present figure.
+// HBM bound: every row is read once, 16 lanes of 16 bytes to a row, the 16 rows of a warp's step asked for
+// before the first is used (4 KB per warp, 32 warps per SM: with 32 rows per step and 16 warps the last of two
+// waves was half empty).  The squared norms of a step are reduced by folding (8 exchanges per lane instead of 32
+// for 8 butterflies), bf16 pairs are widened in place and multiplied as packed fp32.
 template <int MODE, int P>
-__global__ void __launch_bounds__(kSumThreads, 2)
+__global__ void __launch_bounds__(kSumThreads, MODE == kRowsFew ? 3 : 4)
 k_block_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block, const int T,
              __nv_bfloat16* __restrict__ parts, int* __restrict__ nz, float* __restrict__ us,
              int* __restrict__ nzs) {
-  __shared__ float part[kSumWarps][kHeadDim];
+  __shared__ __align__(16) float part[kSumWarps][kHeadDim];
   __shared__ int cnt[kSumWarps];
   __shared__ float csum[kHeadDim];
   __shared__ int ccnt;
@@ -89,78 +84,86 @@ k_block_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block, 
   pdl_launch_dependents();
   pdl_wait();
 
-  float tot[8];
+  f32x2 tot[4];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) tot[e] = 0.f;
+  for (int e = 0; e < 4; ++e) tot[e] = pack2(0.f, 0.f);
   int tot_nz = 0;
 
   // The warp's rows: whole blocks (few rows per block), or a share of one block.
-  int first, end, stride;      // first row, end of the warp's range, rows between its steps
-  int blk = 0;                 // block the range starts in
+  int r0, end, step;           // first row of a step, end of the warp's range, rows between its steps
+  int again = 0, blk = 0;      // rows skipped after every second step (a cluster's turns); block of the step
   if (MODE != kRowsMany) {
-    const int per_warp = kSumRows / block;
-    blk = slice * bpc + warp * per_warp;
-    first = blk * block;
-    end = min(L, first + per_warp * block);
-    stride = kSumRows;
+    const int per_step = kSumStep / block;
+    blk = slice * bpc + warp * kSumSteps * per_step;
+    r0 = blk * block;
+    step = per_step * block;
+    end = min(L, r0 + kSumSteps * step);
   } else {
-    const int sub = (block + kSumRows - 1) / kSumRows;   // steps of a block
+    const int sub = (block + kSumRows - 1) / kSumRows;   // shares of kSumRows rows in a block
     const int share = sub < kSumWarps ? sub : kSumWarps; // warps of a CTA on one block
     const int slot = warp / share;
     blk = slice * bpc + slot;
-    first = blk * block + (rank * share + warp - slot * share) * kSumRows;
+    r0 = blk * block + (rank * share + warp - slot * share) * kSumRows;
     end = slot < bpc ? min(L, (blk + 1) * block) : 0;
-    stride = S * share * kSumRows;
+    step = kSumStep;
+    again = (S * share - 1) * kSumRows;
   }
 #pragma unroll 1
-  for (int r0 = first; r0 < end; r0 += stride) {
-    uint4 v[16];
-    float p[16];
+  for (int turn = 0; r0 < end; ++turn, r0 += step + ((turn & 1) ? 0 : again)) {
+    const int stop = MODE == kRowsMany ? end : min(end, r0 + step);
+    uint4 v[8];
+    float p[8];
     const uint4* rp = reinterpret_cast<const uint4*>(base + (size_t)(r0 + half) * kHeadDim);
-    const int left = end - r0 - half;
+    const int left = stop - r0 - half;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {   // one address, constant offsets
+    for (int i = 0; i < 8; ++i) {   // one address, constant offsets
       v[i] = make_uint4(0, 0, 0, 0);
       if (2 * i < left) v[i] = __ldg(rp + 2 * i * (kHeadDim / 8));
     }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const uint32_t* w = reinterpret_cast<const uint32_t*>(&v[i]);
-      float s0 = 0.f, s1 = 0.f;
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+      f32x2 sq = pack2(0.f, 0.f);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        // (byte permutes here, shifts below: with the same instructions in both sweeps the 256
-        // widened values would be kept, which does not fit the registers)
-        const float a = __uint_as_float(__byte_perm(w[e], 0u, 0x1044)),
-                    b = __uint_as_float(__byte_perm(w[e], 0u, 0x3244));
-        s0 = fmaf(a, a, s0);
-        s1 = fmaf(b, b, s1);
+        // (byte permutes here, bf16x2_wide below: widened by the same instructions in both sweeps, all values
+        // would be kept in between, which does not fit the registers)
+        const f32x2 f = pack2(__uint_as_float(__byte_perm(w[e], 0u, 0x1044)),
+                              __uint_as_float(__byte_perm(w[e], 0u, 0x3244)));
+        sq = fma2(f, f, sq);
       }
+      float s0, s1;
+      unpack2(sq, s0, s1);
       p[i] = s0 + s1;
     }
-    // folding: lane c of a half is left with the squared norm of row 2 c + half
+    // folding: lanes 2 i, 2 i + 1 of a half are left with the squared norm of row 2 i + half
 #pragma unroll
-    for (int o = 8; o >= 1; o >>= 1) {
+    for (int o = 8; o >= 2; o >>= 1) {
       const bool up = (c & o) != 0;
 #pragma unroll
-      for (int k = 0; k < o; ++k) {
-        const float send = up ? p[k] : p[k + o], keep = up ? p[k + o] : p[k];
+      for (int k = 0; k < o / 2; ++k) {
+        const float send = up ? p[k] : p[k + o / 2], keep = up ? p[k + o / 2] : p[k];
         p[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
       }
     }
+    p[0] += __shfl_xor_sync(0xffffffffu, p[0], 1);
     const float inv = p[0] > 0.f ? rsqrtf(p[0]) : 0.f;
-    const unsigned alive = __ballot_sync(0xffffffffu, p[0] > 0.f);
+    // bit r of `alive`: row r of the step is not zero (row r = 2 i + half stands with lane 16 half + 2 i)
+    const float of_row = __shfl_sync(0xffffffffu, inv, ((lane & 1) << 4) | (lane & 14));
+    const unsigned alive = __ballot_sync(0xffffffffu, of_row > 0.f) & 0xffffu;
     tot_nz += __popc(alive);
-    float acc[8];
+    f32x2 acc[4];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+    for (int e = 0; e < 4; ++e) acc[e] = pack2(0.f, 0.f);
     // sum of the two halves' accumulators -> the parts of block `blk` (rows a .. b-1 of the step)
-    auto flush = [&](const float (&mine)[8], const int a, const int b) {
+    auto flush = [&](const int a, const int b) {
       float s[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        s[e] = mine[e] + __shfl_xor_sync(0xffffffffu, mine[e], 16);
-        tot[e] += s[e];
+      for (int e = 0; e < 4; ++e) {
+        unpack2(acc[e], s[2 * e], s[2 * e + 1]);
+        s[2 * e] += __shfl_xor_sync(0xffffffffu, s[2 * e], 16);
+        s[2 * e + 1] += __shfl_xor_sync(0xffffffffu, s[2 * e + 1], 16);
+        tot[e] = add2(tot[e], pack2(s[2 * e], s[2 * e + 1]));
       }
       if (blk < T) {
         uint4 q[P];
@@ -170,26 +173,30 @@ k_block_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block, 
             half ? q[1] : q[0];
         if (P == 3 && half == 0)
           *reinterpret_cast<uint4*>(prow + 2 * part_stride + (size_t)blk * kHeadDim) = q[P - 1];
-        if (lane == 0) nz[(size_t)h * T + blk] = __popc(alive & row_bits(a, b));
+        if (lane == 0) nz[(size_t)h * T + blk] = __popc(alive & ((1u << b) - (1u << a)));
       }
       ++blk;
     };
     int next = block, a0 = 0;   // kRowsFew: row of the step at which the current block ends / starts
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-      const float w = __shfl_sync(0xffffffffu, inv, (lane & 16) | i);
-      const uint32_t* q = reinterpret_cast<const uint32_t*>(&v[i]);
-      float x[8];
+    for (int i = 0; i < 8; ++i) {
+      const float w = __shfl_sync(0xffffffffu, inv, (lane & 16) | (2 * i));
+      const f32x2 w2 = pack2(w, w);
+      const uint32_t q[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+      f32x2 f[4];
 #pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        x[2 * e] = __uint_as_float(q[e] << 16) * w;
-        x[2 * e + 1] = __uint_as_float(q[e] & 0xffff0000u) * w;
-      }
+      for (int e = 0; e < 4; ++e) f[e] = bf16x2_wide(q[e]);
       if (MODE == kRowsOne) {
         const int r = r0 + 2 * i + half;
+        float x[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) tot[e] += x[e];
-        if (r < end) {
+        for (int e = 0; e < 4; ++e) {
+          tot[e] = fma2(f[e], w2, tot[e]);
+          float x0, x1;
+          unpack2(f[e], x0, x1);
+          x[2 * e] = x0 * w, x[2 * e + 1] = x1 * w;
+        }
+        if (r < stop) {
           uint4 o2[P];
           split_parts<P>(x, o2);
 #pragma unroll
@@ -199,35 +206,41 @@ k_block_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block, 
         }
       } else if (MODE == kRowsFew) {
         if (next == 2 * i + 1) {   // the block ends between the two rows of this pair
+          const f32x2 mine = half == 0 ? w2 : pack2(0.f, 0.f), rest = half == 0 ? pack2(0.f, 0.f) : w2;
 #pragma unroll
-          for (int e = 0; e < 8; ++e) acc[e] += half == 0 ? x[e] : 0.f;
-          flush(acc, a0, next);
+          for (int e = 0; e < 4; ++e) acc[e] = fma2(f[e], mine, acc[e]);
+          flush(a0, next);
 #pragma unroll
-          for (int e = 0; e < 8; ++e) acc[e] = half == 0 ? 0.f : x[e];
+          for (int e = 0; e < 4; ++e) acc[e] = fma2(f[e], rest, pack2(0.f, 0.f));
           a0 = next;
           next += block;
         } else {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) acc[e] += x[e];
+          for (int e = 0; e < 4; ++e) acc[e] = fma2(f[e], w2, acc[e]);
         }
         if (next == 2 * i + 2) {
-          flush(acc, a0, next);
+          flush(a0, next);
 #pragma unroll
-          for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+          for (int e = 0; e < 4; ++e) acc[e] = pack2(0.f, 0.f);
           a0 = next;
           next += block;
         }
       } else {
 #pragma unroll
-        for (int e = 0; e < 8; ++e) tot[e] += x[e];
+        for (int e = 0; e < 4; ++e) tot[e] = fma2(f[e], w2, tot[e]);
       }
     }
   }
   // per-warp sums of unit rows (kRowsFew: the two halves already hold the same totals)
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    const float s = MODE == kRowsFew ? tot[e] : tot[e] + __shfl_xor_sync(0xffffffffu, tot[e], 16);
-    if (half == 0) part[warp][8 * c + e] = s;
+  for (int e = 0; e < 4; ++e) {
+    float s0, s1;
+    unpack2(tot[e], s0, s1);
+    if (MODE != kRowsFew) {
+      s0 += __shfl_xor_sync(0xffffffffu, s0, 16);
+      s1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+    }
+    if (half == 0) *reinterpret_cast<float2*>(&part[warp][8 * c + 2 * e]) = make_float2(s0, s1);
   }
   if (lane == 0) cnt[warp] = tot_nz;
   __syncthreads();
@@ -362,7 +375,7 @@ int mixkv_similarity_map(const void* X, int32_t heads, int32_t L, int32_t head_d
   wsb += pl.us_bytes;
   int* nzs = reinterpret_cast<int*>(wsb);
   // Long blocks of which there are too few to fill the GPU: a cluster of CTAs per block, as long as
-  // every warp keeps a full step of 32 rows.
+  // every warp keeps a full share of 32 rows.
   int S = 1;
   while (S < kSumMaxCluster && (long long)heads * pl.slices * S < device_sm_count() &&
          (long long)2 * S * kSumWarps * kSumRows <= block)

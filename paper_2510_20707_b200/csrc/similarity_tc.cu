@@ -9,10 +9,8 @@
 // J runs (P x 32 KB), the parts of J go through a three-stage ring one part at a time, and two
 // accumulator stages let the epilogue of a tile overlap the MMA of the next.
 //
-// What bounds it: the output, T x T x 4 bytes per head, once T is large.  Every store is a full
-// 128-byte line per warp: the cells of the mirrored tile straight from the registers (a thread holds
-// one I and 32 J, so for one J the lanes are 32 consecutive I), the tile itself after a 32 x 32
-// transposition through shared memory (swizzled, no bank conflicts).
+// What bounds it: the output, T x T x 4 bytes per head, once T is large: a tile and its mirror image leave
+// through shared memory as 16-byte stores of full 128-byte lines.
 //
 // NT = 128 where there are tiles enough for every SM, NT = 32 below that: a small map is one chain
 // of load, MMA and store per CTA, and a quarter of the columns shortens all three.
@@ -289,33 +287,50 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
             v[j] = __float_as_uint(x);
           }
         }
-        if (!on_diag) {   // mirrored tile: row J, 32 consecutive I per store
-          float* p = out + (size_t)j0 * T + i;
-          if (i < T) {
-            if (j0 + 32 <= T) {
+        // Both images go through a swizzled 32 x 32 tile in shared memory (cell (i, j) of the chunk at word
+        // 4 ((j / 4) ^ (i & 7)) + j % 4 of row i) and leave as 16-byte stores, four rows of 128 bytes per
+        // instruction; where the rows of the map are not 16-byte aligned, or the chunk is cut by its edge, as
+        // 4-byte stores, one row per instruction.
+        const bool vec = (T & 3) == 0 && i0 + 32 <= T && j0 + 32 <= T;
+        const int sub = lane >> 3, quad = lane & 7;   // row of a group of four, four columns of it
+        if (!on_diag) {   // mirrored tile: rows J
+          if (vec) {
+            __syncwarp();
 #pragma unroll
-              for (int j = 0; j < 32; ++j) p[(size_t)j * T] = __uint_as_float(v[j]);
-            } else {
+            for (int j = 0; j < 32; ++j)
+              st[j * 32 + 4 * ((lane >> 2) ^ (j & 7)) + (lane & 3)] = __uint_as_float(v[j]);
+            __syncwarp();
+            float* p = out + (size_t)(j0 + sub) * T + i0 + 4 * quad;
 #pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (j0 + j < T) p[(size_t)j * T] = __uint_as_float(v[j]);
-            }
+            for (int r = 0; r < 32; r += 4)
+              *reinterpret_cast<float4*>(p + (size_t)r * T) =
+                  *reinterpret_cast<const float4*>(st + (r + sub) * 32 + 4 * (quad ^ ((r + sub) & 7)));
+          } else if (i < T) {
+            float* p = out + (size_t)j0 * T + i;   // straight from the registers
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (j0 + j < T) p[(size_t)j * T] = __uint_as_float(v[j]);
           }
         }
-        // the tile itself: rows I, 32 consecutive J per store
+        // the tile itself: rows I
         __syncwarp();
 #pragma unroll
-        for (int j = 0; j < 32; ++j) st[lane * 32 + (j ^ lane)] = __uint_as_float(v[j]);
+        for (int j = 0; j < 32; j += 4)
+          *reinterpret_cast<float4*>(st + lane * 32 + 4 * ((j >> 2) ^ (lane & 7))) =
+              make_float4(__uint_as_float(v[j]), __uint_as_float(v[j + 1]), __uint_as_float(v[j + 2]),
+                          __uint_as_float(v[j + 3]));
         __syncwarp();
-        if (j0 + lane < T) {
+        if (vec) {
+          float* p = out + (size_t)(i0 + sub) * T + j0 + 4 * quad;
+#pragma unroll
+          for (int r = 0; r < 32; r += 4)
+            *reinterpret_cast<float4*>(p + (size_t)r * T) =
+                *reinterpret_cast<const float4*>(st + (r + sub) * 32 + 4 * (quad ^ ((r + sub) & 7)));
+        } else if (j0 + lane < T) {
           float* p = out + (size_t)i0 * T + j0 + lane;
-          if (i0 + 32 <= T) {
 #pragma unroll
-            for (int r = 0; r < 32; ++r) p[(size_t)r * T] = st[r * 32 + (lane ^ r)];
-          } else {
-#pragma unroll 1
-            for (int r = 0; r < T - i0; ++r) p[(size_t)r * T] = st[r * 32 + (lane ^ r)];
-          }
+          for (int r = 0; r < 32; ++r)
+            if (i0 + r < T) p[(size_t)r * T] = st[r * 32 + 4 * ((lane >> 2) ^ (r & 7)) + (lane & 3)];
         }
       }
       ++tile;

@@ -148,6 +148,43 @@ struct MixParams {
   float eps;
 };
 
+// Pooled scores of four consecutive positions from staged windows (16-byte aligned; a window of up to nine raw
+// scores around each of the four is three 16-byte loads), additions in the order of pool_window.
+__device__ __forceinline__ void pool4(const float* w0, const int k, const bool avg, const int mode, const float invk,
+                                      float (&ex)[4]) {
+  if (k <= 9) {
+    float w[12];
+#pragma unroll
+    for (int u = 0; u < 3; ++u) *reinterpret_cast<float4*>(w + 4 * u) = *reinterpret_cast<const float4*>(w0 + 4 * u);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) ex[e] = avg ? 0.f : -INFINITY;
+#pragma unroll
+    for (int u = 0; u < 9; ++u) {
+      if (u < k) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) ex[e] = avg ? ex[e] + w[e + u] : fmaxf(ex[e], w[e + u]);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) ex[e] = avg ? ex[e] * invk : ex[e];
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) ex[e] = pool_window(w0 + e, k, mode, invk);
+  }
+}
+__device__ __forceinline__ void mix4(const float (&ex)[4], const float4 v4, const float4 d4, const float* sc,
+                                     const int use_vnorm, const int mix_mode, float (&m)[4]) {
+  const float vv[4] = {v4.x, v4.y, v4.z, v4.w}, dd[4] = {d4.x, d4.y, d4.z, d4.w};
+  if (mix_mode == MIXKV_MIX_HEADWISE && use_vnorm) {   // (scalars in registers)
+    const float r = sc[4], a0 = sc[0], a1 = sc[1], d0 = sc[2], d1 = sc[3];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) m[e] = mix_headwise(ex[e], vv[e], dd[e], a0, a1, d0, d1, r);
+  } else {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) m[e] = mix_one(ex[e], vv[e], dd[e], sc, use_vnorm, mix_mode);
+  }
+}
+
 // --------------------------------------------------------------------------- poolsum
 // Max pooling only: per-chunk sums of the pooled score (its mean enters Eq. 2).
 __global__ void __launch_bounds__(256)
@@ -181,56 +218,72 @@ k_poolsum(const SeqTable st, const Workspace ws, const int k) {
 }
 
 // --------------------------------------------------------------------------- mixpool
-// Pooling and the mix over a grid of position chunks (the scores entry point, adaptive budgets).
-__global__ void __launch_bounds__(256)
+// Pooling and the mix over a grid of position chunks (the scores entry point, adaptive budgets).  A chunk is read
+// with consecutive threads on consecutive positions, all loads in flight at once, staged in shared memory and
+// mixed four consecutive positions per thread, as in k_tail.
+__global__ void __launch_bounds__(256, 4)
 k_mixpool(const SeqTable st, const Workspace ws, const float* __restrict__ s_div,
           const float* __restrict__ rbar_in, float* __restrict__ s_ex_out,
           float* __restrict__ s_comp, const MixParams mp) {
-  __shared__ float tile[kPChunk + 64];
+  __shared__ __align__(16) float tile[kPChunk + 64], svn[kPChunk], sdv[kPChunk];
   __shared__ float sc[8];
   pdl_launch_dependents();
-  pdl_wait();
-  const int pcx = blockIdx.x, h = blockIdx.y, layer = blockIdx.z;
+  const int pcx = blockIdx.x, h = blockIdx.y, layer = blockIdx.z, tid = threadIdx.x;
   const int b = find_seq(st.pchunk_start, st.batch, pcx);
   const int P = st.cu[b + 1] - st.cu[b] - st.W;
   const int p0 = (pcx - st.pchunk_start[b]) * kPChunk;
-  const int p1 = min(p0 + kPChunk, P);
+  const int n = min(kPChunk, P - p0);
   const size_t poff = ppos(st, layer, h, b, 0);
   const int half = mp.pool_k >> 1;
-  const float pad = mp.pool_mode == MIXKV_POOL_AVG ? 0.f : -INFINITY;
-  if (threadIdx.x < 32)
-    head_scalars(st, ws, pass2_segments(st, layer, b, h), layer, b, h, mp.pool_k, mp.pool_mode, mp.use_vnorm,
-                 mp.eps, rbar_in, threadIdx.x, sc);
-  // a chunk is eight rounds of 256 positions (+ the pooling halo in a ninth); every load of the
-  // chunk is issued before the first use
+  const bool avg = mp.pool_mode == MIXKV_POOL_AVG;
+  const float pad = avg ? 0.f : -INFINITY;
+  const SegList sl = pass2_segments(st, layer, b, h);   // (divisions: ahead of the wait)
+  pdl_wait();
+  // eight rounds of 256 positions (+ the pooling halo in a ninth)
   constexpr int kRounds = kPChunk / 256;
-  const int nstage = (p1 - p0) + 2 * half;
+  const int nstage = n + 2 * half;
   float raw[kRounds + 1], vn[kRounds], dv[kRounds];
 #pragma unroll
   for (int e = 0; e <= kRounds; ++e) {
-    const int t = e * 256 + threadIdx.x, i = p0 - half + t;
+    const int t = e * 256 + tid, i = p0 - half + t;
     raw[e] = (t < nstage && i >= 0 && i < P) ? ws.s_ex_raw[poff + i] : pad;
   }
 #pragma unroll
   for (int e = 0; e < kRounds; ++e) {
-    const int i = p0 + e * 256 + threadIdx.x;
-    vn[e] = (mp.use_vnorm && i < p1) ? ws.vnorm[poff + i] : 0.f;
-    dv[e] = i < p1 ? s_div[poff + i] : 0.f;
+    const int t = e * 256 + tid;
+    vn[e] = (mp.use_vnorm && t < n) ? ws.vnorm[poff + p0 + t] : 0.f;
+    dv[e] = t < n ? s_div[poff + p0 + t] : 0.f;
   }
+  if (tid < 32)
+    head_scalars(st, ws, sl, layer, b, h, mp.pool_k, mp.pool_mode, mp.use_vnorm, mp.eps, rbar_in, tid, sc);
 #pragma unroll
   for (int e = 0; e <= kRounds; ++e) {
-    const int t = e * 256 + threadIdx.x;
+    const int t = e * 256 + tid;
     if (t < nstage) tile[t] = raw[e];
   }
+#pragma unroll
+  for (int e = 0; e < kRounds; ++e) svn[e * 256 + tid] = vn[e], sdv[e * 256 + tid] = dv[e];
   __syncthreads();
   const float invk = 1.0f / (float)mp.pool_k;
+  // the pooled scores take the place of the value norms, the mixed ones that of the diversity scores
+#pragma unroll
+  for (int g = 0; g < kPChunk / 1024; ++g) {
+    const int q = g * 1024 + 4 * tid;
+    if (q >= n) break;
+    float ex[4], m[4];
+    pool4(tile + q, mp.pool_k, avg, mp.pool_mode, invk, ex);
+    const float4 v4 = *reinterpret_cast<const float4*>(svn + q), d4 = *reinterpret_cast<const float4*>(sdv + q);
+    mix4(ex, v4, d4, sc, mp.use_vnorm, mp.mix_mode, m);
+    *reinterpret_cast<float4*>(svn + q) = make_float4(ex[0], ex[1], ex[2], ex[3]);
+    *reinterpret_cast<float4*>(sdv + q) = make_float4(m[0], m[1], m[2], m[3]);
+  }
+  __syncthreads();
 #pragma unroll
   for (int e = 0; e < kRounds; ++e) {
-    const int t = e * 256 + threadIdx.x, i = p0 + t;
-    if (i < p1) {
-      const float ex = pool_window(tile + t, mp.pool_k, mp.pool_mode, invk);
-      if (s_ex_out) s_ex_out[poff + i] = ex;
-      s_comp[poff + i] = mix_one(ex, vn[e], dv[e], sc, mp.use_vnorm, mp.mix_mode);
+    const int t = e * 256 + tid;
+    if (t < n) {
+      if (s_ex_out) s_ex_out[poff + p0 + t] = svn[t];
+      s_comp[poff + p0 + t] = sdv[t];
     }
   }
 }
@@ -246,6 +299,7 @@ __device__ __forceinline__ unsigned order_key(float f) {
 
 constexpr int kSelBinBits = 11, kSelBins = 1 << kSelBinBits;
 constexpr int kSelListCap = 256;   // candidates ranked directly
+constexpr int kSelMaxCluster = 8;
 
 struct SelSmem {
   int hist[2][kSelBins];
@@ -255,7 +309,7 @@ struct SelSmem {
   unsigned wlo[32], whi[32];
   unsigned range[2];             // this CTA's smallest and largest key
   int scan[32];
-  int off[9];                    // cluster: where each rank's candidates start in `all`
+  int off[kSelMaxCluster];       // cluster: where each rank's candidates start in `all`
   int nlist, gt, eq;             // this CTA's candidates, its keys above them, its keys equal to the threshold
   int bin, remaining, count;     // bin that holds the threshold, keys still needed from it, keys in it
   unsigned tau;
@@ -339,13 +393,22 @@ __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const
     int h[PER], mine = 0;
 #pragma unroll
     for (int k = 0; k < PER; ++k) h[k] = 0;
-    for (int r = 0; r < cs; ++r) {
-      const int* src = cs > 1 ? cluster.map_shared_rank(&hist[PER * tid], r) : &hist[PER * tid];
+    if (cs > 1) {
+      // every rank's loads are under way before the first is used: a remote load takes half a microsecond
+      int2 v[kSelMaxCluster][PER / 2];
 #pragma unroll
-      for (int k = 0; k < PER; k += 2) {
-        const int2 v = *reinterpret_cast<const int2*>(src + k);
-        h[k] += v.x, h[k + 1] += v.y;
-      }
+      for (int r = 0; r < kSelMaxCluster; ++r)
+#pragma unroll
+        for (int k = 0; k < PER / 2; ++k)
+          v[r][k] = r < cs ? reinterpret_cast<const int2*>(cluster.map_shared_rank(&hist[PER * tid], r))[k]
+                           : make_int2(0, 0);
+#pragma unroll
+      for (int r = 0; r < kSelMaxCluster; ++r)
+#pragma unroll
+        for (int k = 0; k < PER / 2; ++k) h[2 * k] += v[r][k].x, h[2 * k + 1] += v[r][k].y;
+    } else {
+#pragma unroll
+      for (int k = 0; k < PER; ++k) h[k] = hist[PER * tid + k];
     }
 #pragma unroll
     for (int k = 0; k < PER; ++k) {
@@ -469,7 +532,7 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
   __shared__ int s_gt[64], s_eq[64], t_gt[64], t_eq[64];
   cg::cluster_group cluster = cg::this_cluster();
   const int cs = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
-  const int tid = threadIdx.x, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_launch_dependents();
   for (int t = tid; t < 2 * kSelBins; t += kBudgetThreads) (&sm.hist[0][0])[t] = 0;
   if (tid < 64) s_gt[tid] = 0, s_eq[tid] = 0;
@@ -487,53 +550,54 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
       for (int h = tid; h < H; h += kBudgetThreads) counts[b * H + h] = N <= 0 ? min(floor_slots, P) : P;
     return;
   }
-  // this CTA's slice of every head: positions [p0, p0 + n)
+  // This CTA's slice of every head: positions [p0, p0 + n).  Its keys stand head after head, every head padded
+  // to whole words of 32 with key 0 (below every key of a number), so that a word belongs to one head.
   const int chunk = (P + cs - 1) / cs;
   const int p0 = min(crank * chunk, P), n = min(chunk, P - p0);
-  const int local = H * n;
+  const int npad = (n + 31) & ~31, local = H * npad;
   const bool cached = local <= cache_cap;
   unsigned lo = 0xffffffffu, hi = 0u;
-  for (int h = 0; h < H; ++h) {
-    const float* row = base + (size_t)h * stride + p0;
-    for (int i0 = 0; i0 < n; i0 += 8 * kBudgetThreads) {   // eight loads in flight per thread
-      float v[8];
+  for (int i0 = 0; i0 < npad; i0 += 2 * kBudgetThreads) {   // up to eight loads in flight per thread
+    for (int h0 = 0; h0 < H; h0 += 4) {
+      float v[2][4];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int i = i0 + k * kBudgetThreads + tid;
-        v[k] = i < n ? row[i] : 0.f;
-      }
+      for (int u = 0; u < 2; ++u)
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int i = i0 + k * kBudgetThreads + tid;
-        if (i < n) {
-          const unsigned key = order_key(v[k]);
-          if (cached) bkeys[h * n + i] = key;
-          lo = min(lo, key);
-          hi = max(hi, key);
+        for (int k = 0; k < 4; ++k) {
+          const int i = i0 + u * kBudgetThreads + tid;
+          v[u][k] = i < n && h0 + k < H ? base[(size_t)(h0 + k) * stride + p0 + i] : 0.f;
         }
-      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int i = i0 + u * kBudgetThreads + tid;
+          if (i < npad && h0 + k < H) {
+            const unsigned key = i < n ? order_key(v[u][k]) : 0u;
+            if (cached) bkeys[(h0 + k) * npad + i] = key;
+            if (i < n) lo = min(lo, key), hi = max(hi, key);
+          }
+        }
     }
   }
   __syncthreads();
   auto key_at = [&](const int e) -> unsigned {
     if (cached) return bkeys[e];
-    const int h = e / n;
-    return order_key(base[(size_t)h * stride + p0 + (e - h * n)]);
+    const int h = e / npad, i = e - h * npad;
+    return i < n ? order_key(base[(size_t)h * stride + p0 + i]) : 0u;
   };
   const Threshold th =
       threshold_search<kBudgetThreads>(key_at, [](int) {}, local, (int)N, lo, hi, sm, cluster, cs, crank);
+  // a vote per word of 32; most words hold nothing that counts
   for (int h = 0; h < H; ++h) {
-    int gt = 0, eq = 0;
-    for (int i = tid; i < n; i += kBudgetThreads) {
-      const unsigned key = key_at(h * n + i);
-      gt += key > th.tau;
-      eq += key == th.tau;
-    }
-    gt = __reduce_add_sync(0xffffffffu, gt);
-    eq = __reduce_add_sync(0xffffffffu, eq);
-    if (lane == 0 && (gt | eq)) {
-      atomicAdd(&s_gt[h], gt);
-      atomicAdd(&s_eq[h], eq);
+    for (int i0 = warp * 32; i0 < npad; i0 += kBudgetThreads) {
+      const unsigned key = key_at(h * npad + i0 + lane);
+      const int gt = __popc(__ballot_sync(0xffffffffu, key > th.tau)),
+                eq = __popc(__ballot_sync(0xffffffffu, key == th.tau));
+      if (lane == 0 && (gt | eq)) {
+        if (gt) atomicAdd(&s_gt[h], gt);
+        if (eq) atomicAdd(&s_eq[h], eq);
+      }
     }
   }
   // every CTA's per-head counts are complete
@@ -693,9 +757,6 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
     const bool avg = a.mp.pool_mode == MIXKV_POOL_AVG, vnorm_on = a.mp.use_vnorm != 0;
     const float pad = avg ? 0.f : -INFINITY;
     const float invk = 1.0f / (float)a.mp.pool_k;
-    if (warp == 1)
-      head_scalars(st, ws, sl2, layer, b, h, a.mp.pool_k, a.mp.pool_mode, a.mp.use_vnorm, a.mp.eps,
-                   a.rbar_in, lane, sc);
     const float* g_raw = ws.s_ex_raw + poff;
     const float* g_vn = ws.vnorm + poff + c0;
     const float* g_dv = a.s_div + poff + c0;
@@ -729,6 +790,9 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
       }
     };
     if (n > 0) load_block(0);
+    if (warp == 1)   // (its own share of the first block is on the way)
+      head_scalars(st, ws, sl2, layer, b, h, a.mp.pool_k, a.mp.pool_mode, a.mp.use_vnorm, a.mp.eps,
+                   a.rbar_in, lane, sc);
     for (int j0 = 0; j0 < n; j0 += BL) {
       const int nb = min(BL, n - j0);   // positions of this block
       __syncthreads();                  // the previous block's readers of the stage are done
@@ -753,40 +817,11 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
       __syncthreads();
       const int q = 4 * tid;            // this thread's positions q .. q + 3 of the block
       if (q < nb) {
-        float ex[4];
-        if (a.mp.pool_k <= 9) {
-          float w[12];
-#pragma unroll
-          for (int u = 0; u < 3; ++u)
-            *reinterpret_cast<float4*>(w + 4 * u) = *reinterpret_cast<const float4*>(sraw + q + 4 * u);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) ex[e] = avg ? 0.f : -INFINITY;
-#pragma unroll
-          for (int u = 0; u < 9; ++u) {   // (same order of additions as pool_window)
-            if (u < a.mp.pool_k) {
-#pragma unroll
-              for (int e = 0; e < 4; ++e) ex[e] = avg ? ex[e] + w[e + u] : fmaxf(ex[e], w[e + u]);
-            }
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e) ex[e] = avg ? ex[e] * invk : ex[e];
-        } else {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) ex[e] = pool_window(sraw + q + e, a.mp.pool_k, a.mp.pool_mode, invk);
-        }
-        const float4 v4 = *reinterpret_cast<const float4*>(svn + j0 + q);
-        const float4 d4 = *reinterpret_cast<const float4*>(sdv + q);
-        const float vv[4] = {v4.x, v4.y, v4.z, v4.w}, dd[4] = {d4.x, d4.y, d4.z, d4.w};
-        float m[4];
+        float ex[4], m[4];
+        pool4(sraw + q, a.mp.pool_k, avg, a.mp.pool_mode, invk, ex);
+        mix4(ex, *reinterpret_cast<const float4*>(svn + j0 + q), *reinterpret_cast<const float4*>(sdv + q), sc,
+             a.mp.use_vnorm, a.mp.mix_mode, m);
         unsigned key[4];
-        if (a.mp.mix_mode == MIXKV_MIX_HEADWISE && vnorm_on) {   // (scalars in registers)
-          const float r = sc[4], v0 = sc[0], vs = sc[1], d0 = sc[2], ds = sc[3];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) m[e] = mix_headwise(ex[e], vv[e], dd[e], v0, vs, d0, ds, r);
-        } else {
-#pragma unroll
-          for (int e = 0; e < 4; ++e) m[e] = mix_one(ex[e], vv[e], dd[e], sc, a.mp.use_vnorm, a.mp.mix_mode);
-        }
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           key[e] = order_key(m[e]);
@@ -994,7 +1029,7 @@ cudaError_t launch_budget(const LaunchCtx& c, const float* scores, int* counts) 
   const int cs = c.st.batch * c.st.layers < device_sm_count() / kBudgetCluster ? kBudgetCluster : 1;
   const size_t chunk = ((size_t)c.max_prefix + cs - 1) / cs;
   // the keys of a CTA's slice of the longest sequence in shared memory when they fit
-  const size_t want = (size_t)c.st.H * chunk * 4;
+  const size_t want = (size_t)c.st.H * ((chunk + 31) / 32) * 128;
   const size_t cap_bytes = 200 * 1024;
   const size_t smem = want <= cap_bytes ? want : 0;
   if (smem > 24 * 1024) {   // on top of the search's static shared memory
