@@ -153,8 +153,8 @@ __device__ __forceinline__ float fold_key_sums(const float* ksum, const SegList&
   }
   return sum;
 }
-// The pass-1 segments of the head that segment iterator `sg` (of either pass) stands on.
-__device__ __forceinline__ SegList pass1_segments(const SeqTable& st, const SegIter& sg) {
+// The pass-1 segments of the head that segment iterator `sg` of pass 2 stands on.
+__device__ __forceinline__ SegList pass1_segments(const SeqTable& st, const RevSegIter& sg) {
   const int per_head = (st.tile1_start[sg.b + 1] - st.tile1_start[sg.b]) / st.H;
   return SegList(sg.layer * st.nt1 + st.tile1_start[sg.b] + sg.h * per_head, per_head, split1(st));
 }
@@ -554,6 +554,10 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
 // of its G*W logit columns, so nothing is exchanged between warps), 4 value-norm warps.  More
 // epilogue warps splitting the columns of a tile were measured slower (C3: 13.4 against 11.7 us per
 // layer): the exchange of partial sums and the extra warps cost more than they hide.
+//
+// A CTA walks its tiles backwards: pass 1 has read (about) the same tiles in ascending order, so the K that is
+// still in L2 from there is the end of every CTA's range.  K and V are loaded evict-first, which keeps those lines,
+// and the scores written for the tail, from being driven out by what is not read again.
 constexpr int kP2Threads = 16 * 32;
 constexpr int kP2EpiWarps = 8;                   // warps 4..11
 constexpr int kP2AuxWarp0 = 12;                  // warps 12..15: value norms
@@ -656,23 +660,24 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   if (warp == kWarpTma) {
     // ------------------------------------------------------------------ K / Q producer
     if (lane == 0) {
+      const uint64_t policy = l2_evict_first();
       int s = 0, ph = 1, it = 0, segn = 0;
       bool ok = true;
-      for (SegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
+      for (RevSegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
         if (segn > 0 && !mbar_wait(&bars->qfree, (segn - 1) & 1, abort)) break;
         mbar_expect_tx(&bars->qfull, NQ * 256);
         tma_load_3d(sQ, &tmQ, 0, sg.bh() * NQ, sg.layer, &bars->qfull);
         tma_load_3d(sQ + NB * 128, &tmQ, 64, sg.bh() * NQ, sg.layer, &bars->qfull);
         ++segn;
-        int y = st.cu[sg.b] + sg.t0 * kTile;
-        for (int k = 0; k < sg.n; ++k, y += kTile) {
+        int y = st.cu[sg.b] + (sg.end() - 1) * kTile;
+        for (int k = 0; k < sg.n; ++k, y -= kTile) {
           if (!mbar_wait(&bars->kempty[s], ph, abort)) {
             ok = false;
             break;
           }
           mbar_expect_tx(&bars->kfull[s], kTileBytes);
-          tma_load_4d(sK + s * kTileBytes, &tmK, 0, y, sg.h, sg.layer, &bars->kfull[s]);
-          tma_load_4d(sK + s * kTileBytes + kHalfBytes, &tmK, 64, y, sg.h, sg.layer, &bars->kfull[s]);
+          tma_load_4d(sK + s * kTileBytes, &tmK, 0, y, sg.h, sg.layer, &bars->kfull[s], policy);
+          tma_load_4d(sK + s * kTileBytes + kHalfBytes, &tmK, 64, y, sg.h, sg.layer, &bars->kfull[s], policy);
           if (++s == kP2KStages) s = 0, ph ^= 1;
           ++it;
         }
@@ -685,19 +690,20 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   } else if (warp == kWarpTmaV) {
     // ------------------------------------------------------------------ V producer
     if (lane == 0 && use_vnorm == MIXKV_INTRINSIC_VNORM) {
+      const uint64_t policy = l2_evict_first();
       int vit = 0, vs = 0, vph = 1;
       bool ok = true;
-      for (SegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
-        int y = st.cu[sg.b] + sg.t0 * kTile;
-        for (int k = 0; k < 2 * sg.n; ++k, y += 64) {   // half tiles of 64 rows
+      for (RevSegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
+        int y = st.cu[sg.b] + (sg.end() - 1) * kTile;
+        for (int k = 0; k < 2 * sg.n; ++k, y += (k & 1) ? 64 : -64 - kTile) {   // half tiles of 64 rows
           if (!mbar_wait(&bars->vempty[vs], vph, abort)) {
             ok = false;
             break;
           }
           mbar_expect_tx(&bars->vfull[vs], kVSubBytes);
           unsigned char* dst = sV + vs * kVSubBytes;
-          tma_load_4d(dst, &tmV, 0, y, sg.h, sg.layer, &bars->vfull[vs]);
-          tma_load_4d(dst + kVSubBytes / 2, &tmV, 64, y, sg.h, sg.layer, &bars->vfull[vs]);
+          tma_load_4d(dst, &tmV, 0, y, sg.h, sg.layer, &bars->vfull[vs], policy);
+          tma_load_4d(dst + kVSubBytes / 2, &tmV, 64, y, sg.h, sg.layer, &bars->vfull[vs], policy);
           if (++vs == vstages) vs = 0, vph ^= 1;
           ++vit;
         }
@@ -715,7 +721,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     const uint32_t q_half = (uint32_t)(NB * 128) >> 4;   // second 64-column half of the B operand
     int s = 0, ph = 0, ts = 0, tph = 1, segn = 0;
     bool ok = true;
-    for (SegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
+    for (RevSegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
       if (!mbar_wait(&bars->qfull, segn & 1, abort)) break;
       if (!mbar_wait(&bars->kbready, segn & 1, abort)) break;
       ++segn;
@@ -764,7 +770,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     const int barid = 1 + wg;                      // named barriers 1, 2: one per warpgroup
     const f32x2 sc2 = pack2(scale_log2e, scale_log2e);
     int tile = 0;   // parity decides which warpgroup owns it
-    for (SegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid(); sg.next()) {
+    for (RevSegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid(); sg.next()) {
       const int P = st.cu[sg.b + 1] - st.cu[sg.b] - W;
       named_bar_sync(5, kP2EpiWarps * 32);   // the previous segment's readers of sbq are done
       if (et < NQ) sbq[et] = fold_row_stats(ws.rowstat, pass1_segments(st, sg), NQ, et, log2W);
@@ -776,7 +782,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
       float* sd_out = s_div_out + poff;
       // this warpgroup's tiles of the segment
       const int skip = (tile & 1) ^ wg;
-      for (int t = sg.t0 + skip, tl = tile + skip; t < sg.end(); t += 2, tl += 2) {
+      for (int t = sg.end() - 1 - skip, tl = tile + skip; t >= sg.t0; t -= 2, tl += 2) {
         const int tph = (tl >> 1) & 1;
         const int ikey = t * kTile + key;
         float kinv_i = 0.f;
@@ -860,7 +866,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     const int vt = tid - kP2AuxWarp0 * 32;         // 0..127
     const int sub = vt >> 6, vr = vt & 63;
     int vs = sub, vph = 0, segn = 0;   // V stage of this pair of warps: half tiles sub, sub + 2, ...
-    for (SegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid(); sg.next()) {
+    for (RevSegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid(); sg.next()) {
       const int L = st.cu[sg.b + 1] - st.cu[sg.b], P = L - W;
       const float ks = fold_key_sums(ws.ksum, pass1_segments(st, sg), vt);
       const float kb = ks / (float)L;   // mean unit key
@@ -911,7 +917,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
           vsum += n;
         }
       } else if (use_vnorm) {
-        for (int t = sg.t0; t < sg.end(); ++t) {
+        for (int t = sg.end() - 1; t >= sg.t0; --t) {
           const bool ok = mbar_wait(&bars->vfull[vs], vph, abort);
           const unsigned char* tile = sV + vs * kVSubBytes;
           f32x2 ss2[2] = {pack2(0.f, 0.f), pack2(0.f, 0.f)};

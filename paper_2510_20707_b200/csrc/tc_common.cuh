@@ -94,6 +94,20 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* tm, in
       "l"(tm), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar))
       : "memory");
 }
+// The same with an L2 eviction policy.
+__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* tm, int x, int y, int z,
+                                            int w, uint64_t* bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], "
+      "[%1, {%2, %3, %4, %5}], [%6], %7;" ::"r"(smem_u32(dst)),
+      "l"(tm), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar)), "l"(policy)
+      : "memory");
+}
+__device__ __forceinline__ uint64_t l2_evict_first() {
+  uint64_t policy;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  return policy;
+}
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* tm) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory");
 }
@@ -314,6 +328,43 @@ struct SegIter {
       per_head = (tile_start[b + 1] - tile_start[b]) / H;
     }
     n = min(per_head, hi - id);
+  }
+};
+
+// The same tiles from the last to the first: segments in descending order, tiles end() - 1 down to t0 inside
+// them.  id is the first (lowest) tile of the segment, as in SegIter.
+struct RevSegIter {
+  int id, lo, left, layer, b, h, t0, n, H, batch;
+  const int* tile_start;
+  __device__ RevSegIter(const int* tile_start_, int batch_, int H_, int nt, int lo_, int hi)
+      : lo(lo_), left(hi), H(H_), batch(batch_), tile_start(tile_start_) {
+    layer = b = h = t0 = n = id = 0;
+    if (lo_ < hi) {
+      layer = (hi - 1) / nt;
+      const TileCoord c = tile_coord(tile_start_, batch_, H_, hi - 1 - layer * nt);
+      b = c.b, h = c.h;
+      set(c.t + 1);
+    }
+  }
+  __device__ __forceinline__ void set(int end) {   // the segment ends before tile `end` of its head
+    n = min(end, left - lo);
+    t0 = end - n;
+    id = left - n;
+  }
+  __device__ __forceinline__ bool valid() const { return left > lo; }
+  __device__ __forceinline__ int bh() const { return b * H + h; }
+  __device__ __forceinline__ int unit() const { return (layer * batch + b) * H + h; }
+  __device__ __forceinline__ int end() const { return t0 + n; }
+  __device__ __forceinline__ void next() {
+    left -= n;
+    if (--h < 0) {
+      h = H - 1;
+      if (--b < 0) {
+        b = batch - 1;
+        --layer;
+      }
+    }
+    set((tile_start[b + 1] - tile_start[b]) / H);
   }
 };
 
