@@ -113,43 +113,43 @@ __device__ __forceinline__ float2 merge_stats(const float2 a, const float2 b) {
 // ---- per-head folds (pass 2, at the start of a segment): what the segments of pass 1 left
 // for a (layer, sequence, head) becomes what pass 2 needs of it.
 //
-// kFoldDepth loads are in flight per round: a head that a one-layer call spreads over a quarter
-// of the GPU's CTAs is folded in one round trip to L2.
-constexpr int kFoldDepth = 40;
-// Window row q: the (reference, sum) pairs of all segments merged under the largest reference,
-// returned as the negated log2 normaliser of the row with the 1/W of the window mean folded in.
-__device__ __forceinline__ float fold_row_stats(const float2* rowstat, const SegList& sl,
-                                                const int NQ, const int q, const float log2W) {
+// kFoldRows row statistics and kFoldSums key sums are in flight per round and thread, two threads share a window
+// row: a head that a one-layer call spreads over a quarter of the GPU's CTAs is folded in a round trip or two to
+// L2.
+constexpr int kFoldRows = 12, kFoldSums = 40;
+// Window row q over segments [e_lo, e_hi): their (reference, sum) pairs merged under the largest reference.
+__device__ __forceinline__ float2 fold_row_stats(const float2* rowstat, const SegList& sl, const int e_lo,
+                                                 const int e_hi, const int NQ, const int q) {
   float M = -1e30f, Z = 0.f;
 #pragma unroll 1
-  for (int e0 = 0; e0 < sl.nseg; e0 += kFoldDepth) {
-    float2 v[kFoldDepth];
+  for (int e0 = e_lo; e0 < e_hi; e0 += kFoldRows) {
+    float2 v[kFoldRows];
 #pragma unroll
-    for (int k = 0; k < kFoldDepth; ++k) {
+    for (int k = 0; k < kFoldRows; ++k) {
       v[k] = make_float2(-1e30f, 0.f);
-      if (e0 + k < sl.nseg) v[k] = __ldcg(rowstat + (size_t)sl.start(e0 + k) * NQ + q);
+      if (e0 + k < e_hi) v[k] = __ldcg(rowstat + (size_t)sl.start(e0 + k) * NQ + q);
     }
     float mx = M;
 #pragma unroll
-    for (int k = 0; k < kFoldDepth; ++k) mx = fmaxf(mx, v[k].x);
+    for (int k = 0; k < kFoldRows; ++k) mx = fmaxf(mx, v[k].x);
     Z *= ex2(M - mx);
 #pragma unroll
-    for (int k = 0; k < kFoldDepth; ++k) Z = fmaf(v[k].y, ex2(v[k].x - mx), Z);
+    for (int k = 0; k < kFoldRows; ++k) Z = fmaf(v[k].y, ex2(v[k].x - mx), Z);
     M = mx;
   }
-  return -(M + log2f(Z)) - log2W;
+  return make_float2(M, Z);
 }
 // Component kt of the unit-key sum over all segments of the head.
 __device__ __forceinline__ float fold_key_sums(const float* ksum, const SegList& sl, const int kt) {
   float sum = 0.f;
 #pragma unroll 1
-  for (int e0 = 0; e0 < sl.nseg; e0 += kFoldDepth) {
-    float v[kFoldDepth];
+  for (int e0 = 0; e0 < sl.nseg; e0 += kFoldSums) {
+    float v[kFoldSums];
 #pragma unroll
-    for (int k = 0; k < kFoldDepth; ++k)
+    for (int k = 0; k < kFoldSums; ++k)
       v[k] = e0 + k < sl.nseg ? __ldcg(ksum + (size_t)sl.start(e0 + k) * kHeadDim + kt) : 0.f;
 #pragma unroll
-    for (int k = 0; k < kFoldDepth; ++k) sum += v[k];
+    for (int k = 0; k < kFoldSums; ++k) sum += v[k];
   }
   return sum;
 }
@@ -549,18 +549,19 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
 }
 
 // ======================================================================== pass 2
-// Pass 2 streams K and V and sits at the HBM bound with sixteen warps: K/Q producer, MMA, V
-// producer, 1 idle, two epilogue warpgroups that own alternate tiles (every thread one key and all
-// of its G*W logit columns, so nothing is exchanged between warps), 4 value-norm warps.  More
-// epilogue warps splitting the columns of a tile were measured slower (C3: 13.4 against 11.7 us per
-// layer): the exchange of partial sums and the extra warps cost more than they hide.
+// Pass 2 streams K and V.  24 warps: K/Q producer, MMA, V producer, 1 idle, four epilogue warpgroups, 4
+// value-norm warps.  Epilogue warpgroup g works on accumulator stage g & 1 (alternate tiles), column half
+// g >> 1: one key per thread and half of its G*W logit columns, in pieces of 16 with the next piece on its way
+// from tensor memory; the two halves of a key meet in one word of shared memory per tile.  (With two warpgroups
+// and all columns in a thread, two warps per scheduler kept the exp2 unit busy for half of the time: 28 layers of
+// 4 x 32768 keys, G*W = 224, 359 us; as here 333 us; split like this but without the pieces 359 us again.)
 //
 // A CTA walks its tiles backwards: pass 1 has read (about) the same tiles in ascending order, so the K that is
 // still in L2 from there is the end of every CTA's range.  K and V are loaded evict-first, which keeps those lines,
 // and the scores written for the tail, from being driven out by what is not read again.
-constexpr int kP2Threads = 16 * 32;
-constexpr int kP2EpiWarps = 8;                   // warps 4..11
-constexpr int kP2AuxWarp0 = 12;                  // warps 12..15: value norms
+constexpr int kP2EpiWarps = 16;                  // warps 4..19
+constexpr int kP2AuxWarp0 = kEpiWarp0 + kP2EpiWarps;   // warps 20..23: value norms
+constexpr int kP2Threads = (kP2AuxWarp0 + 4) * 32;
 
 constexpr int kP2KStages = 3;              // K tiles (32 KB each)
 constexpr int kP2VStagesMax = 4;           // V half tiles: 64 rows, 16 KB each
@@ -579,22 +580,23 @@ struct P2Bars {
   int abort;
 };
 
-// N logit columns of one key (registers r[0..N)): adds exp2(logit * scale - normaliser of the
-// column) to acc; nb_smem holds the negated normalisers of these columns.
-template <int N>
-__device__ __forceinline__ void colsum_chunk(const uint32_t (&r)[N], const float* nb_smem,
-                                             const f32x2 sc2, f32x2& acc) {
+// 16 logit columns of one key: adds exp2(logit * scale - normaliser of the column) to two packed sums;
+// nb_smem holds the negated normalisers of these columns.
+__device__ __forceinline__ void colsum16(const uint32_t (&r)[16], const float* nb_smem, const f32x2 sc2,
+                                         f32x2& acc_a, f32x2& acc_b) {
 #pragma unroll
-  for (int j = 0; j < N; j += 4) {
+  for (int j = 0; j < 16; j += 4) {
     const float4 nb = *reinterpret_cast<const float4*>(nb_smem + j);   // negated normalisers
-    acc = add2(acc, ex2_pair(fma2(pack2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])), sc2,
-                                  pack2(nb.x, nb.y))));
-    acc = add2(acc, ex2_pair(fma2(pack2(__uint_as_float(r[j + 2]), __uint_as_float(r[j + 3])), sc2,
-                                  pack2(nb.z, nb.w))));
+    acc_a = add2(acc_a, ex2_pair(fma2(pack2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])), sc2,
+                                      pack2(nb.x, nb.y))));
+    acc_b = add2(acc_b, ex2_pair(fma2(pack2(__uint_as_float(r[j + 2]), __uint_as_float(r[j + 3])), sc2,
+                                      pack2(nb.z, nb.w))));
   }
 }
 
-// grid = g2 persistent CTAs: K producer, MMA, V producer, 1 idle, 8 epilogue, 4 value-norm warps.
+// grid = g2 persistent CTAs: K producer, MMA, V producer, 1 idle, 16 epilogue, 4 value-norm warps.
+// NCH: pieces of 16 query columns per epilogue warp, at most.
+template <int NCH>
 __global__ void __launch_bounds__(kP2Threads, 1)
 k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
         const __grid_constant__ CUtensorMap tmQ, const SeqTable st, const Workspace ws,
@@ -608,8 +610,10 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   unsigned char* sQ = base;                   // 2 halves x [NB x 128 B]
   unsigned char* sK = sQ + 2 * NB * 128;      // kP2KStages x 32 KB
   unsigned char* sV = sK + kP2KStages * kTileBytes;   // vstages x 16 KB
-  float* sbq = reinterpret_cast<float*>(sV + vstages * kVSubBytes);  // [256] negated normalisers (+ 256 spare)
-  float* sred = sbq + 512;                    // [64]: 2 x 16 epilogue, 12 value norms, 4 mean key
+  float* sbq = reinterpret_cast<float*>(sV + vstages * kVSubBytes);  // [256] negated normalisers
+  float* sxp = sbq + 256;                     // [2][128] partial column sums of the second column halves
+  float2* sxf = reinterpret_cast<float2*>(sxp + 256);   // [256] row statistics of the second half of the segments
+  float* sred = reinterpret_cast<float*>(sxf + 256);    // [64]: 2 x 16 epilogue, 12 value norms, 4 mean key
   P2Bars* bars = reinterpret_cast<P2Bars*>(sred + 64);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -630,7 +634,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&bars->tfull[s], 1);
-      mbar_init(&bars->tempty[s], 4);      // the warps of the warpgroup that owns the accumulator stage
+      mbar_init(&bars->tempty[s], 8);      // the warps of the two warpgroups that read the stage
     }
     mbar_init(&bars->qfull, 1);
     mbar_init(&bars->qfree, 1);
@@ -753,91 +757,118 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     if (*abort && on) raise(status, abort);
   } else if (warp >= kEpiWarp0 && warp < kEpiWarp0 + kP2EpiWarps) {
     // ------------------------------------------------------------------ epilogue
-    // The two warpgroups take alternate tiles (warpgroup g owns accumulator stage g), one key
-    // per thread and all G*W columns of it, so a tile needs no exchange between warpgroups and
-    // inside a segment the groups never wait for each other; each leaves its own partial score
-    // statistics.  At the start of a segment the 256 threads fold the row statistics of the
-    // head together, one window row per thread, into the normaliser table both groups read.
-    // Nobody leaves the tile loop early: after an abort every wait fails at once, so the
-    // named barriers of the segment boundaries stay matched.
-    const int quarter = warp & 3, wg = (warp - kEpiWarp0) >> 2;
+    // Alternate tiles belong to alternate pairs of warpgroups, so inside a segment the pairs never wait
+    // for each other; each pair leaves its own partial score statistics.  At the start of a segment the
+    // 512 threads fold the row statistics of the head together, two threads to a window row, into the
+    // normaliser table all groups read.  Nobody leaves the tile loop early: after an abort every
+    // wait fails at once, so the named barriers stay matched.
+    const int quarter = warp & 3, grp = (warp - kEpiWarp0) >> 2;
+    const int wg = grp & 1, chalf = grp >> 1;      // accumulator stage, column half
     const int gt = (tid - kEpiWarp0 * 32) & 127;   // thread inside the warpgroup
     const int gw = gt >> 5;                        // warp inside the warpgroup
     const int key = quarter * 32 + lane;
     const int nch = NQ / 16;
-    const int et = tid - kEpiWarp0 * 32;           // thread inside the epilogue, 0..255
+    const int ch_lo = chalf ? nch / 2 : 0, ch_n = chalf ? nch - nch / 2 : nch / 2;   // ch_n <= NCH
+    const int et = tid - kEpiWarp0 * 32;           // thread inside the epilogue, 0..511
     const float log2W = log2f((float)W);
-    const int barid = 1 + wg;                      // named barriers 1, 2: one per warpgroup
+    const int barid = 1 + wg;                      // named barriers 1, 2: first column halves
+    const int xbar = 6 + wg;                       // named barriers 6, 7: partial sums handed over
     const f32x2 sc2 = pack2(scale_log2e, scale_log2e);
-    int tile = 0;   // parity decides which warpgroup owns it
+    const uint32_t tstage = tmem + ((uint32_t)(quarter * 32) << 16) + wg * 256, taddr = tstage + ch_lo * 16;
+    const float* nb = sbq + ch_lo * 16;
+    int tile = 0;   // parity decides which pair owns it
     for (RevSegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid(); sg.next()) {
       const int P = st.cu[sg.b + 1] - st.cu[sg.b] - W;
-      named_bar_sync(5, kP2EpiWarps * 32);   // the previous segment's readers of sbq are done
-      if (et < NQ) sbq[et] = fold_row_stats(ws.rowstat, pass1_segments(st, sg), NQ, et, log2W);
+      {
+        const SegList sl = pass1_segments(st, sg);
+        const int q = et & 255, mid = sl.nseg > kFoldRows ? (sl.nseg + 1) >> 1 : sl.nseg;
+        float2 mz = make_float2(-1e30f, 0.f);
+        if (q < NQ) {
+          if (et < 256) mz = fold_row_stats(ws.rowstat, sl, 0, mid, NQ, q);
+          else sxf[q] = fold_row_stats(ws.rowstat, sl, mid, sl.nseg, NQ, q);
+        }
+        named_bar_sync(5, kP2EpiWarps * 32);   // (also: the previous segment's readers of sbq are done)
+        // the negated log2 normaliser of the row with the 1/W of the window mean folded in
+        if (et < NQ) {
+          if (mid < sl.nseg) mz = merge_stats(mz, sxf[et]);
+          sbq[et] = -(mz.x + log2f(mz.y)) - log2W;
+        }
+        named_bar_sync(5, kP2EpiWarps * 32);
+      }
       float dmin = INFINITY, dmax = -INFINITY, dsum = 0.f, exw = 0.f;
-      named_bar_sync(5, kP2EpiWarps * 32);
       const float* kinv = ws.kinv + kpos(st, sg.layer, sg.h, sg.b, 0);
       const size_t poff = ppos(st, sg.layer, sg.h, sg.b, 0);
       float* ex_out = ws.s_ex_raw + poff;
       float* sd_out = s_div_out + poff;
-      // this warpgroup's tiles of the segment
+      // this pair's tiles of the segment
       const int skip = (tile & 1) ^ wg;
       for (int t = sg.end() - 1 - skip, tl = tile + skip; t >= sg.t0; t -= 2, tl += 2) {
         const int tph = (tl >> 1) & 1;
         const int ikey = t * kTile + key;
         float kinv_i = 0.f;
-        if (ikey < P) kinv_i = kinv[ikey];
+        if (chalf == 0 && ikey < P) kinv_i = kinv[ikey];
         const bool ok = mbar_wait(&bars->tfull[wg], tph, abort);
         tc_fence_after();
-        const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + wg * 256;
-        f32x2 acc = pack2(0.f, 0.f);
-        float dot = 0.f;
+        f32x2 acc = pack2(0.f, 0.f), acc_b = acc;
+        uint32_t rd[4];
         if (ok) {
-          uint32_t rd[4];
-          tmem_ld4(taddr + NQ, rd);
-          // 32-column chunks (the other warpgroup's tile keeps the SM busy while this load is
-          // in flight), then a 16-column rest; kept rolled: the body must stay in the i-cache
-          const int n32 = nch >> 1;
-#pragma unroll 1
-          for (int ci = 0; ci < n32; ++ci) {
-            uint32_t ra[32];
-            tmem_ld32(taddr + ci * 32, ra);
+          uint32_t ra[16], rb[16];
+          tmem_ld16(taddr, ra);   // (a piece past this half is another half's or the mean key's: read, not used)
+#pragma unroll
+          for (int ci = 0; ci < NCH; ci += 2) {
             tmem_ld_wait();
             tmem_ld_fence(ra);
-            colsum_chunk<32>(ra, sbq + ci * 32, sc2, acc);
+            if (ci + 1 < NCH) tmem_ld16(taddr + ci * 16 + 16, rb);
+            else if (chalf == 0) tmem_ld4(tstage + NQ, rd);
+            if (ci < NCH - 1 || ci < ch_n) colsum16(ra, nb + ci * 16, sc2, acc, acc_b);
+            if (ci + 1 < NCH) {
+              tmem_ld_wait();
+              tmem_ld_fence(rb);
+              if (ci + 2 < NCH) tmem_ld16(taddr + ci * 16 + 32, ra);
+              else if (chalf == 0) tmem_ld4(tstage + NQ, rd);
+              if (ci + 1 < NCH - 1 || ci + 1 < ch_n) colsum16(rb, nb + ci * 16 + 16, sc2, acc, acc_b);
+            }
           }
-          if (nch & 1) {
-            uint32_t rb[16];
-            tmem_ld16(taddr + n32 * 32, rb);
-            tmem_ld_wait();
-            tmem_ld_fence(rb);
-            colsum_chunk<16>(rb, sbq + n32 * 32, sc2, acc);
-          }
-          tmem_ld_wait();
-          tmem_ld_fence(rd);
-          dot = (__uint_as_float(rd[0]) + __uint_as_float(rd[1])) + __uint_as_float(rd[2]);
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&bars->tempty[wg]);
-        if (ok && ikey < P) {
-          float acc0, acc1;
-          unpack2(acc, acc0, acc1);
-          const float ex = acc0 + acc1;
-          ex_out[ikey] = ex;
-          const float sd = -dot * kinv_i;
-          sd_out[ikey] = sd;
-          dmin = fminf(dmin, sd);
-          dmax = fmaxf(dmax, sd);
-          dsum += sd;
-          // number of pooling windows (centres in [0, P)) that cover this position
-          const int cover = min(ikey, pool_half) + min(P - 1 - ikey, pool_half) + 1;
-          exw = fmaf(ex, (float)cover, exw);
+        float acc0, acc1;
+        unpack2(add2(acc, acc_b), acc0, acc1);
+        const float part = acc0 + acc1;
+        if (chalf) {
+          // The other half reads this word before it arrives on tempty, and the next tile of this stage is
+          // not complete before that: no barrier for the way back.
+          sxp[wg * 128 + key] = part;
+          named_bar_arrive(xbar, 256);
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bars->tempty[wg]);
+        } else {
+          float dot = 0.f;
+          if (ok) {
+            tmem_ld_wait();
+            tmem_ld_fence(rd);
+            dot = (__uint_as_float(rd[0]) + __uint_as_float(rd[1])) + __uint_as_float(rd[2]);
+          }
+          named_bar_sync(xbar, 256);
+          const float ex = part + sxp[wg * 128 + key];
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&bars->tempty[wg]);
+          if (ok && ikey < P) {
+            ex_out[ikey] = ex;
+            const float sd = -dot * kinv_i;
+            sd_out[ikey] = sd;
+            dmin = fminf(dmin, sd);
+            dmax = fmaxf(dmax, sd);
+            dsum += sd;
+            // number of pooling windows (centres in [0, P)) that cover this position
+            const int cover = min(ikey, pool_half) + min(P - 1 - ikey, pool_half) + 1;
+            exw = fmaf(ex, (float)cover, exw);
+          }
         }
       }
       tile += sg.n;
-      {
-        // this warpgroup's share of the segment's score statistics (neutral if it had no tile)
+      if (chalf == 0) {
+        // this pair's share of the segment's score statistics (neutral if it had no tile)
         const float a = warp_min(dmin), b2 = warp_max(dmax), c2 = warp_sum(dsum),
                     d2 = warp_sum(exw);
         float* sr = sred + wg * 16;
@@ -1041,7 +1072,7 @@ size_t pass1_smem(int MB, int NQ) {
 }
 size_t pass2_smem(int NQ, int vstages) {
   return 1024 + (size_t)2 * (NQ + kExtraRows) * 128 + kP2KStages * kTileBytes +
-         (size_t)vstages * kVSubBytes + 512 * 4 + 64 * 4 + sizeof(P2Bars) + 64;
+         (size_t)vstages * kVSubBytes + 1024 * 4 + 64 * 4 + sizeof(P2Bars) + 64;
 }
 
 // cudaFuncSetAttribute once per (kernel, device).
@@ -1105,21 +1136,41 @@ cudaError_t launch_pass1(const LaunchCtx& c, const void* K, const void* Q, int* 
                     c.ws, c.scale_log2e, (int)c.clear_status, status);
 }
 
+namespace {
+struct P2Maps {
+  CUtensorMap K, V, Q;
+};
+template <int NCH>
+cudaError_t launch_pass2_t(const LaunchCtx& c, const P2Maps& m, float* s_div_out, float* rbar_out, int vstages,
+                           int* status) {
+  static bool done[64] = {false};
+  cudaError_t e = ensure_smem(k_pass2<NCH>, kSmemLimit, done);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_pass2<NCH>, dim3(c.st.g2), dim3(kP2Threads), pass2_smem(c.st.NQ, vstages), c.stream, 1, m.K, m.V,
+                    m.Q, c.st, c.ws, s_div_out, rbar_out, c.scale_log2e, c.p.use_vnorm, c.p.pool_kernel >> 1,
+                    vstages, status);
+}
+}  // namespace
+
 cudaError_t launch_pass2(const LaunchCtx& c, const void* K, const void* V, const void* Q,
                          float* s_div_out, float* rbar_out, int* status) {
   CUtensorMap tmK, tmV, tmQ;
   const void* Vsrc = c.p.use_vnorm == MIXKV_INTRINSIC_VNORM ? V : K;   // the V map is never used without VNorm
   if (!map_kv(c, K, kTile, &tmK) || !map_kv(c, Vsrc, 64, &tmV) || !map_q(c, Q, &tmQ))
     return cudaErrorInvalidValue;
-  static bool done[64] = {false};
-  cudaError_t e = ensure_smem(k_pass2, kSmemLimit, done);
-  if (e != cudaSuccess) return e;
   int vstages = kP2VStagesMax;
   while (vstages > 2 && pass2_smem(c.st.NQ, vstages) > kSmemLimit) --vstages;
-  const size_t smem = pass2_smem(c.st.NQ, vstages);
-  return launch_pdl(k_pass2, dim3(c.st.g2), dim3(kP2Threads), smem, c.stream, 1, tmK, tmV, tmQ, c.st,
-                    c.ws, s_div_out, rbar_out, c.scale_log2e, c.p.use_vnorm, c.p.pool_kernel >> 1,
-                    vstages, status);
+  const P2Maps m{tmK, tmV, tmQ};
+  switch ((c.st.NQ / 16 + 1) / 2) {   // pieces of 16 columns per epilogue warp
+    case 1: return launch_pass2_t<1>(c, m, s_div_out, rbar_out, vstages, status);
+    case 2: return launch_pass2_t<2>(c, m, s_div_out, rbar_out, vstages, status);
+    case 3: return launch_pass2_t<3>(c, m, s_div_out, rbar_out, vstages, status);
+    case 4: return launch_pass2_t<4>(c, m, s_div_out, rbar_out, vstages, status);
+    case 5: return launch_pass2_t<5>(c, m, s_div_out, rbar_out, vstages, status);
+    case 6: return launch_pass2_t<6>(c, m, s_div_out, rbar_out, vstages, status);
+    case 7: return launch_pass2_t<7>(c, m, s_div_out, rbar_out, vstages, status);
+    default: return launch_pass2_t<8>(c, m, s_div_out, rbar_out, vstages, status);
+  }
 }
 
 }  // namespace mixkv
