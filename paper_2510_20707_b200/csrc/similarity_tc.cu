@@ -6,8 +6,9 @@
 //   P = 3 (hi + mid + lo, 24 bits)    hi.hi + mid.hi + lo.hi + hi.mid + mid.mid + hi.lo
 // Persistent CTAs walk a contiguous run of tiles (head, I, J): 128 blocks I on M, NT blocks J on N,
 // only tiles that touch or lie right of the diagonal.  The parts of I stay in shared memory while
-// J runs (P x 32 KB), the parts of J go through a three-stage ring one part at a time, and two
-// accumulator stages let the epilogue of a tile overlap the MMA of the next.
+// J runs (P x 32 KB), the parts of J go through a ring of six half parts (with three whole ones a stage was asked
+// for again only half a tile ahead of its use, less than a round trip to L2), and two accumulator stages let the
+// epilogue of a tile overlap the MMA of the next.
 //
 // What bounds it: the output, T x T x 4 bytes per head, once T is large: a tile and its mirror image leave
 // through shared memory as 16-byte stores of full 128-byte lines.
@@ -24,7 +25,7 @@ namespace {
 constexpr int kGThreads = 12 * 32;   // TMA, MMA, 2 head-mean, 8 epilogue warps
 constexpr int kGEpiWarp0 = 4, kGEpiWarps = 8;
 constexpr int kPartBytes = 128 * 256;   // one part of 128 blocks: two 64-column halves of 16 KB
-constexpr int kGStages = 3;
+constexpr int kGStages = 6;            // halves (64 columns) of one part of the blocks on N
 
 struct GBars {
   uint64_t afull, afree;
@@ -117,10 +118,10 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
-  constexpr int kBPart = NT * 256, kBHalf = NT * 128;   // one part of the NT blocks on N
+  constexpr int kBHalf = NT * 128;                      // half a part of the NT blocks on N
   unsigned char* sA = base;                             // P parts
-  unsigned char* sB = sA + P * kPartBytes;              // kGStages x one part
-  float* sT = reinterpret_cast<float*>(sB + kGStages * kBPart);   // [8 warps][32 x 32]
+  unsigned char* sB = sA + P * kPartBytes;              // kGStages x half a part
+  float* sT = reinterpret_cast<float*>(sB + kGStages * kBHalf);   // [8 warps][32 x 32]
   GBars* bars = reinterpret_cast<GBars*>(sT + kGEpiWarps * 1024);
   __shared__ float red[4];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -157,7 +158,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
   if (warp == 0) {
     // -------------------------------------------------------------------- TMA producer
     if (lane == 0) {
-      int it = 0, rown = 0;
+      int s = 0, ph = 1, rown = 0;
       bool ok = true;
       for (GramWalk<NT> w(T, per_head, lo, hi); w.valid() && ok; w.next()) {
         if (w.fresh) {
@@ -169,17 +170,14 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
           }
           ++rown;
         }
-        for (int p = 0; p < P; ++p) {
-          const int s = it % kGStages, ph = (it / kGStages) & 1;
-          if (!mbar_wait(&bars->bempty[s], ph ^ 1, abort)) {
+        for (int x = 0; x < 2 * P && ok; ++x) {   // half x / P of part x % P
+          if (!mbar_wait(&bars->bempty[s], ph, abort)) {
             ok = false;
             break;
           }
-          mbar_expect_tx(&bars->bfull[s], kBPart);
-          unsigned char* dst = sB + s * kBPart;
-          tma_load_3d(dst, &tmB, 0, w.I * 128 + w.c * NT, p * H + w.h, &bars->bfull[s]);
-          tma_load_3d(dst + kBHalf, &tmB, 64, w.I * 128 + w.c * NT, p * H + w.h, &bars->bfull[s]);
-          ++it;
+          mbar_expect_tx(&bars->bfull[s], kBHalf);
+          tma_load_3d(sB + s * kBHalf, &tmB, x / P * 64, w.I * 128 + w.c * NT, x % P * H + w.h, &bars->bfull[s]);
+          if (++s == kGStages) s = 0, ph ^= 1;
         }
       }
       if (*abort) {   // let the copies in flight land before the shared memory goes away
@@ -194,7 +192,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
       const uint32_t on = elect_one();
       constexpr uint32_t idesc = umma_idesc_bf16(128, NT);
       const uint32_t a0 = umma_desc_lo(smem_u32(sA)), b0 = umma_desc_lo(smem_u32(sB));
-      int it = 0, rown = 0, tile = 0;
+      int s = 0, ph = 0, rown = 0, tile = 0;
       bool ok = true;
       for (GramWalk<NT> w(T, per_head, lo, hi); w.valid() && ok; w.next()) {
         if (w.fresh) {
@@ -203,30 +201,30 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
         }
         const int ts = tile & 1, tph = (tile >> 1) & 1;
         if (!mbar_wait(&bars->tempty[ts], tph ^ 1, abort)) break;
-        // part p of J meets the parts of I whose product with it carries weight
+        // half by half of the contraction, part p of J meets the parts of I whose product with it carries weight
 #pragma unroll
-        for (int p = 0; p < P; ++p) {
-          const int s = it % kGStages, ph = (it / kGStages) & 1;
+        for (int x = 0; x < 2 * P; ++x) {
+          const int p = x % P, half = x / P;
           if (!mbar_wait(&bars->bfull[s], ph, abort)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t bs = b0 + (uint32_t)s * (kBPart >> 4);
+          const uint32_t bs = b0 + (uint32_t)s * (kBHalf >> 4);
 #pragma unroll
           for (int pa = 0; pa < P - p; ++pa) {
 #pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {
-              const uint32_t oa = (uint32_t)(pa * (kPartBytes >> 4) + (ks >> 2) * (16384 >> 4) + (ks & 3) * 2);
-              const uint32_t ob = (uint32_t)((ks >> 2) * (kBHalf >> 4) + (ks & 3) * 2);
-              if (p == 0 && pa == 0 && ks == 0)
+            for (int ks = 0; ks < 4; ++ks) {
+              const uint32_t oa = (uint32_t)(pa * (kPartBytes >> 4) + half * (16384 >> 4) + ks * 2);
+              const uint32_t ob = (uint32_t)(ks * 2);
+              if (x == 0 && pa == 0 && ks == 0)
                 umma_bf16_lo<0>(tmem + ts * 128, a0 + oa, bs + ob, idesc, on);
               else
                 umma_bf16_lo<1>(tmem + ts * 128, a0 + oa, bs + ob, idesc, on);
             }
           }
           umma_commit(&bars->bempty[s], on);
-          ++it;
+          if (++s == kGStages) s = 0, ph ^= 1;
         }
         umma_commit(&bars->tfull[ts], on);
         if (w.row_last()) umma_commit(&bars->afree, on);
@@ -344,7 +342,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
 template <int P, int NT>
 cudaError_t launch_gram_t(const GramArgs& g, const long long per_head, cudaStream_t s) {
   static bool done[64] = {false};
-  const size_t smem = 1024 + (size_t)P * kPartBytes + (size_t)kGStages * NT * 256 +
+  const size_t smem = 1024 + (size_t)P * kPartBytes + (size_t)kGStages * NT * 128 +
                       (size_t)kGEpiWarps * 4096 + sizeof(GBars);
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
