@@ -114,9 +114,10 @@ __device__ __forceinline__ float2 merge_stats(const float2 a, const float2 b) {
 // for a (layer, sequence, head) becomes what pass 2 needs of it.
 //
 // kFoldRows row statistics and kFoldSums key sums are in flight per round and thread, two threads share a window
-// row: a head that a one-layer call spreads over a quarter of the GPU's CTAs is folded in a round trip or two to
-// L2.
-constexpr int kFoldRows = 12, kFoldSums = 40;
+// row.  Short rounds: code that runs once per segment costs its instruction fetches, and forty loads unrolled were
+// 6 KB of it (one layer of 4 x 1024 keys 23.6 us, with short rounds 22.5; 37 segments per head, a one-layer
+// call of 4 x 32768, cost the same either way).
+constexpr int kFoldRows = 6, kFoldSums = 8;
 // Window row q over segments [e_lo, e_hi): their (reference, sum) pairs merged under the largest reference.
 __device__ __forceinline__ float2 fold_row_stats(const float2* rowstat, const SegList& sl, const int e_lo,
                                                  const int e_hi, const int NQ, const int q) {

@@ -6,6 +6,8 @@
 // copies the kept K / V rows.
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "tc_common.cuh"
 
 namespace cg = cooperative_groups;
@@ -121,7 +123,9 @@ __device__ __forceinline__ float mix_headwise(const float ex, const float vn, co
   return __fmaf_rn(1.0f - r, imp, __fmul_rn(r, dsc));
 }
 
-__device__ __forceinline__ float mix_one(const float ex, const float vn, const float dv,
+// The other modes, out of line: in the kernels that pool and mix, code that a call does not run only lengthens the way
+// to the code that it does (one layer of 4 x 1024 keys 22.5 -> 21.9 us).
+__device__ __noinline__ float mix_one(const float ex, const float vn, const float dv,
                                          const float* sc, const int use_vnorm,
                                          const int mix_mode) {
   if (use_vnorm && mix_mode == MIXKV_MIX_HEADWISE)
@@ -148,6 +152,10 @@ struct MixParams {
   float eps;
 };
 
+__device__ __noinline__ float pool_wide(const float* w, const int k, const int mode, const float invk) {
+  return pool_window(w, k, mode, invk);
+}
+
 // Pooled scores of four consecutive positions from staged windows (16-byte aligned; a window of up to nine raw
 // scores around each of the four is three 16-byte loads), additions in the order of pool_window.
 __device__ __forceinline__ void pool4(const float* w0, const int k, const bool avg, const int mode, const float invk,
@@ -169,7 +177,7 @@ __device__ __forceinline__ void pool4(const float* w0, const int k, const bool a
     for (int e = 0; e < 4; ++e) ex[e] = avg ? ex[e] * invk : ex[e];
   } else {
 #pragma unroll
-    for (int e = 0; e < 4; ++e) ex[e] = pool_window(w0 + e, k, mode, invk);
+    for (int e = 0; e < 4; ++e) ex[e] = pool_wide(w0 + e, k, mode, invk);
   }
 }
 __device__ __forceinline__ void mix4(const float (&ex)[4], const float4 v4, const float4 d4, const float* sc,
@@ -678,7 +686,8 @@ __device__ __forceinline__ int fixed_offset(const SeqTable& st, int bh, int Bp) 
 // place every kept position; gather.  28 layers x 4 heads x 32736 candidates: 35 us (57 with digit passes over the
 // raw keys and a position per thread and step in the mix); 896 heads of 2 to 7 thousand candidates (selection and
 // gather only): 47 us (119).
-template <bool FUSED, int T>
+// CL: launched as a cluster (else one CTA per unit, and none of the cluster's code is there to be stepped over).
+template <bool FUSED, int T, bool CL>
 __global__ void __launch_bounds__(T, 1024 / T)
 k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   extern __shared__ __align__(16) unsigned char tail_smem[];
@@ -687,8 +696,8 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   __shared__ float sc[8];
   __shared__ int s_rows[kTailRowCap];
   cg::cluster_group cluster = cg::this_cluster();
-  const int crank = (int)cluster.block_rank();
-  const int cs = (int)cluster.num_blocks();
+  const int crank = CL ? (int)cluster.block_rank() : 0;
+  const int cs = CL ? (int)cluster.num_blocks() : 1;
   const int BH = st.batch * st.H;
   const int unit = blockIdx.x / cs;                    // (layer, sequence, head)
   const int layer = unit / BH, bh = unit % BH, b = bh / st.H, h = bh % st.H;
@@ -1079,7 +1088,7 @@ TailShape tail_shape(const LaunchCtx& c) {
 
 bool tail_can_fuse(const LaunchCtx& c) { return tail_shape(c).cached; }
 
-template <bool FUSED, int T>
+template <bool FUSED, int T, bool CL>
 cudaError_t launch_tail_t(const LaunchCtx& c, const TailKernelArgs& a, const TailShape& sh,
                           size_t smem) {
   static size_t have[64] = {0};
@@ -1088,13 +1097,13 @@ cudaError_t launch_tail_t(const LaunchCtx& c, const TailKernelArgs& a, const Tai
   if (e != cudaSuccess) return e;
   if (smem > 20 * 1024 && (dev < 0 || dev >= 64 || have[dev] < smem)) {   // on top of the static part
     const size_t ask = 203 * 1024;
-    e = cudaFuncSetAttribute(k_tail<FUSED, T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(k_tail<FUSED, T, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)ask);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) have[dev] = ask;
   }
   const dim3 grid(c.st.layers * c.st.batch * c.st.H * sh.cs);
-  return launch_pdl(k_tail<FUSED, T>, grid, dim3(T), smem, c.stream, sh.cs, c.st, c.ws, a);
+  return launch_pdl(k_tail<FUSED, T, CL>, grid, dim3(T), smem, c.stream, sh.cs, c.st, c.ws, a);
 }
 
 cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
@@ -1126,10 +1135,15 @@ cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
   size_t smem = (size_t)tail_keys_at(sh.chunk) * 4;
   if (a.cached) smem += (size_t)sh.chunk * 4;
   if (fused) smem += ((size_t)8 * sh.threads + 64) * 4;
+  auto launch = [&](auto threads) {
+    constexpr int T = decltype(threads)::value;
+    if (sh.cs > 1) return fused ? launch_tail_t<true, T, true>(c, a, sh, smem) : launch_tail_t<false, T, true>(c, a, sh, smem);
+    return fused ? launch_tail_t<true, T, false>(c, a, sh, smem) : launch_tail_t<false, T, false>(c, a, sh, smem);
+  };
   switch (sh.threads) {
-    case 256: return fused ? launch_tail_t<true, 256>(c, a, sh, smem) : launch_tail_t<false, 256>(c, a, sh, smem);
-    case 512: return fused ? launch_tail_t<true, 512>(c, a, sh, smem) : launch_tail_t<false, 512>(c, a, sh, smem);
-    default: return fused ? launch_tail_t<true, 1024>(c, a, sh, smem) : launch_tail_t<false, 1024>(c, a, sh, smem);
+    case 256: return launch(std::integral_constant<int, 256>());
+    case 512: return launch(std::integral_constant<int, 512>());
+    default: return launch(std::integral_constant<int, 1024>());
   }
 }
 
