@@ -4,8 +4,8 @@
 //
 // Why it is native: a call of the library enqueues two to six kernels, and the smallest calls keep the
 // GPU busy for less time than interpreted marshalling takes.  Through ctypes one decode call cost 15 us of
-// host time for 7 us of GPU time and a scores + select pair 89 us; the figures of this module stand in
-// binding.py.  Output tensors come from torch's caching allocator without the dispatcher.
+// host time for 7 us of GPU time and a scores + select pair 89 us; here they cost 5.5 and 24 us, one
+// layer's compression 8.6 us.  Output tensors come from torch's caching allocator without the dispatcher.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 

@@ -30,12 +30,10 @@ namespace {
 constexpr int kTileBytes = kTile * 256;    // 128 keys x 128 bf16
 constexpr int kHalfBytes = kTile * 128;    // one 64-column half of a K tile
 
-// Warp roles.  Warpgroup 0 (warps 0..3) holds the single-thread roles: TMA producer, MMA
-// issuer, (pass 2) V producer.  Pass 1: warps 4..19 are the epilogue (all sixteen work on every
-// tile), warps 20..27 compute the key statistics; register budgets per role are set with
-// setmaxnreg (the single-thread roles hand most of theirs to the others).  Pass 2: warps 4..11
-// are the epilogue (two warpgroups that own alternate tiles), warps 12..15 the value norms.  A
-// warp's TMEM lane quarter is warp % 4.
+// Warp roles.  Warpgroup 0 (warps 0..3) holds the single-thread roles: TMA producer, MMA issuer, (pass 2) V
+// producer.  Warps 4..19 are the epilogue.  From warp 20 on: pass 1, eight warps for the key statistics; pass 2,
+// four for the value norms.  Pass 1 shares its registers out by role with setmaxnreg (the single-thread roles hand
+// most of theirs to the others).  A warp's TMEM lane quarter is warp % 4.
 constexpr int kWarpTma = 0, kWarpMma = 1;
 constexpr int kP1WarpMma = 3;                    // pass 1: see k_pass1
 constexpr int kEpiWarp0 = 4;
@@ -74,24 +72,19 @@ __device__ __forceinline__ f32x2 ex2_pair(f32x2 t2) {
 constexpr size_t kSmemLimit = 227 * 1024;   // dynamic shared memory a CTA may ask for
 
 // ======================================================================== pass 1
-// Eight key-statistics warps (from warp 20 on): one tile = 8 pairs of 8-row batches, one pair per
-// warp.  28 warps per CTA.
-__host__ __device__ constexpr int p1_aux_warps(int MB) { return 8; }
-__host__ __device__ constexpr int p1_threads(int MB) { return (kAuxWarp0 + p1_aux_warps(MB)) * 32; }
+// Eight key-statistics warps (from warp 20 on), each with 16 rows of every tile: 28 warps per CTA.
+constexpr int kP1AuxWarps = 8;
+constexpr int kP1Threads = (kAuxWarp0 + kP1AuxWarps) * 32;
 constexpr int kP1MaxStages = 6;
 constexpr int kP1XRows = 3 * 128;   // row statistics exchanged between the warpgroups of a query row
 // K tile ring: as deep as shared memory allows next to the query tile (the deeper the ring, the
 // more bytes in flight towards HBM)
 // (the widest query tiles leave room for four)
 __host__ __device__ constexpr int p1_stages(int NQ) { return NQ > 224 ? 4 : 5; }
-// registers per thread: at launch, then per role (7 warpgroups: 40 + 4 * 72 + 2 * 88 = 7 * 72;
-// the key-statistics warps hold a batch of eight key rows in registers between their two sweeps)
-#ifndef P1_LEAD
-#define P1_LEAD 24
-#define P1_EPI 64
-#define P1_AUX 112
-#endif
-constexpr int kP1RegsLaunch = 72, kP1RegsLead = P1_LEAD, kP1RegsEpi = P1_EPI, kP1RegsAux = P1_AUX;
+// Registers per thread: at launch, then per role (7 warpgroups: 24 + 4 * 64 + 2 * 112 = 7 * 72).  The
+// key-statistics warps keep four widened rows between their two sweeps; two 16-column pieces fit the epilogue's 64.
+constexpr int kP1RegsLaunch = 72, kP1RegsLead = 24, kP1RegsEpi = 64, kP1RegsAux = 112;
+static_assert(kP1RegsLead + 4 * kP1RegsEpi + 2 * kP1RegsAux == 7 * kP1RegsLaunch, "setmaxnreg shares");
 
 struct P1Bars {
   uint64_t full[kP1MaxStages];
@@ -222,7 +215,7 @@ __device__ __noinline__ float2 softmax_chunk_ref(const uint32_t taddr, const boo
 // stream that shares a scheduler with many busy warps issues slowly enough to pace the tile
 // loop.
 template <int MB>
-__global__ void __launch_bounds__(p1_threads(MB), 1)
+__global__ void __launch_bounds__(kP1Threads, 1)
 k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmQ,
         const SeqTable st, const Workspace ws, const float scale_log2e,
         const int clear_status, int* status) {
@@ -230,7 +223,6 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   unsigned char* base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
   const int kP1Stages = p1_stages(st.NQ);
-  constexpr int kP1AuxWarps = p1_aux_warps(MB);
   constexpr int NU = MB == 2 ? 2 : 4;   // warpgroups that share a query row
   constexpr int TS = MB == 2 ? 2 : 4;   // accumulator stages (512 columns of tensor memory)
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1066,7 +1058,7 @@ bool map_q(const LaunchCtx& c, const void* Q, CUtensorMap* tm) {
 size_t pass1_smem(int MB, int NQ) {
   // up to 1023 bytes of alignment slack in front of the carve-up; never beyond the limit (the
   // kernel checks that its carve-up fits behind the aligned base)
-  const size_t need = (size_t)2 * NQ * 128 + (size_t)p1_stages(NQ) * kTileBytes + p1_aux_warps(MB) * 128 * 4 +
+  const size_t need = (size_t)2 * NQ * 128 + (size_t)p1_stages(NQ) * kTileBytes + kP1AuxWarps * 128 * 4 +
                       kP1XRows * 8 + sizeof(P1Bars);
   const size_t want = need + 1024;
   return want < kSmemLimit ? want : kSmemLimit;
@@ -1127,13 +1119,13 @@ cudaError_t launch_pass1(const LaunchCtx& c, const void* K, const void* Q, int* 
     const size_t smem = pass1_smem(1, c.st.NQ);
     cudaError_t e = ensure_smem(k_pass1<1>, kSmemLimit, done1);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_pass1<1>, dim3(c.st.g1), dim3(p1_threads(1)), smem, c.stream, 1, tmK, tmQ, c.st,
+    return launch_pdl(k_pass1<1>, dim3(c.st.g1), dim3(kP1Threads), smem, c.stream, 1, tmK, tmQ, c.st,
                       c.ws, c.scale_log2e, (int)c.clear_status, status);
   }
   const size_t smem = pass1_smem(2, c.st.NQ);
   cudaError_t e = ensure_smem(k_pass1<2>, kSmemLimit, done2);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_pass1<2>, dim3(c.st.g1), dim3(p1_threads(2)), smem, c.stream, 1, tmK, tmQ, c.st,
+  return launch_pdl(k_pass1<2>, dim3(c.st.g1), dim3(kP1Threads), smem, c.stream, 1, tmK, tmQ, c.st,
                     c.ws, c.scale_log2e, (int)c.clear_status, status);
 }
 
