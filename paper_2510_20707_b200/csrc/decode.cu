@@ -47,19 +47,15 @@ constexpr int kDecPitch = 272;                      // bytes between the rows of
 constexpr int kDecSlot = kDecStep * kDecPitch;      // one K or V slot
 constexpr int kDecDepth = 2;                        // steps a warp has on their way or in work
 
-// Floats of dynamic shared memory for GP = 8 or 16 head slots: wacc [warps][GP][132] per-warp
-// value sums, xo [GP][128] the CTA's, wm / wz [warps][16], xm / xz [16], allm / allz [8][16]
-// every rank's (reference, sum) during the cluster merge.
+// Dynamic shared memory for GP = 8 or 16 head slots: per warp its ring and then, the steps being over, its value
+// sums [GP][132] in the same place; the CTA's sums xo [GP][128] behind those of warp 0, in what was its ring (with
+// room of their own sixteen head slots left two CTAs on an SM where the split counts on three: 32 layers x 4
+// sequences of 603 rows and 12 heads 25.3 us); wm / wz [warps][16], xm / xz [16], allm / allz [8][16] every
+// rank's (reference, sum) during the cluster merge.
 constexpr int kDecHeadPitch = kHeadDim + 4;   // floats between the heads of a warp's value sums
-__host__ __device__ constexpr size_t dec_warp_bytes(int GP) {
-  const size_t ring = 2 * (size_t)kDecDepth * kDecSlot, sums = (size_t)GP * kDecHeadPitch * 4;
-  return ring > sums ? ring : sums;
-}
-__host__ __device__ constexpr size_t dec_floats(int GP) {
-  return (size_t)GP * kHeadDim + 2 * kDecWarps * kDecMaxG + 2 * kDecMaxG + 2 * 8 * kDecMaxG +
-         // per warp: the K and the V slot, then (the steps are over) its value sums
-         kDecWarps * (dec_warp_bytes(GP) / 4);
-}
+constexpr size_t kDecWarpBytes = 2 * (size_t)kDecDepth * kDecSlot;
+static_assert(16 * (kDecHeadPitch + kHeadDim) * 4 <= kDecWarpBytes, "sums of a warp and of the CTA fit a ring");
+constexpr size_t kDecSmem = kDecWarps * kDecWarpBytes + (2 * kDecWarps + 2 + 2 * 8) * kDecMaxG * 4;
 // Slot of dimension `dim` inside a head of a warp's value sums: one pad word per 32 dimensions
 // and a head pitch of 132 put the 32 lanes of a fragment store (8 heads x 4 dimensions 32 apart)
 // into 32 different banks.
@@ -277,10 +273,10 @@ k_decode_attention(const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __
                    const float scale_log2e, const int max_rows, float* __restrict__ out) {
   constexpr int GP = WIDE ? 16 : 8;
   extern __shared__ __align__(16) float dsm[];
-  constexpr int kWarpFloats = (int)(dec_warp_bytes(GP) / 4);
+  constexpr int kWarpFloats = (int)(kDecWarpBytes / 4);
   float* wacc = dsm;                                   // [warps]: slots, then [GP][kDecHeadPitch]
-  float* xo = wacc + kDecWarps * kWarpFloats;          // [GP][128]
-  float* wm = xo + GP * kHeadDim;                      // [warps][16]
+  float* xo = wacc + GP * kDecHeadPitch;               // [GP][128], behind the sums of warp 0
+  float* wm = wacc + kDecWarps * kWarpFloats;          // [warps][16]
   float* wz = wm + kDecWarps * kDecMaxG;               // [warps][16]
   float* xm = wz + kDecWarps * kDecMaxG;               // [16]
   float* xz = xm + kDecMaxG;                           // [16]
@@ -418,7 +414,7 @@ extern "C" int mixkv_decode_attention(const void* K_cache, const void* V_cache,
   const long long steps = ((long long)max_rows + kDecStep - 1) / kDecStep;
   long long most = slots / units < steps / kDecWarps ? slots / units : steps / kDecWarps;
   const int S = most < 1 ? 1 : most > 8 ? 8 : (int)most;
-  const size_t smem = dec_floats(wide ? 16 : 8) * 4;
+  const size_t smem = kDecSmem;
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)kHeadDim);
   const __nv_bfloat16 *K = reinterpret_cast<const __nv_bfloat16*>(K_cache),
                       *V = reinterpret_cast<const __nv_bfloat16*>(V_cache),
