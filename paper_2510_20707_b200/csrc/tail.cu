@@ -646,8 +646,7 @@ __host__ __device__ __forceinline__ int tail_chunk(const int P, const int cs) {
 
 // ------------------------------------------------------------------------------ tail
 constexpr int kTailMaxCluster = 8;
-constexpr int kTailCacheCap = 16384;       // positions a CTA of a cluster keeps in shared memory
-constexpr int kTailCacheCapSolo = 40960;   // positions a CTA that owns a whole head keeps
+constexpr int kTailCacheCap = 40960;       // positions a CTA keeps in shared memory
 constexpr int kTailRowCap = 1024;          // selected rows of a CTA listed in shared memory for the gather
 
 struct TailKernelArgs {
@@ -1071,10 +1070,17 @@ TailShape tail_shape(const LaunchCtx& c) {
   const int P = c.max_prefix, sms = device_sm_count();
   TailShape t;
   t.cs = 1;
-  // Many heads, or heads of a block of positions or less: a CTA each (an exchange across a cluster costs
-  // more than another block).  Few long heads: up to eight CTAs each.
-  if (!(units >= sms / 2 && P <= kTailCacheCapSolo))
-    while (t.cs < kTailMaxCluster && tail_chunk(P, t.cs) > 4096) t.cs *= 2;
+  // A CTA per unit when there are many units or a unit is a block of positions or less (an exchange across a
+  // cluster costs more than another block).  Few long ones: CTAs as long as all clusters are resident at once
+  // with one CTA per SM.  Pairs fill the chip; clusters of four and eight do not (they have to lie in one group of
+  // SMs, and groups differ in size): up to 112 CTAs of them ran in one wave, 128 did not (16 units of 32000
+  // positions: eight CTAs each 87 us, four 74; 48 units of 12000: eight 121, four 90, two 80).
+  if (units < sms / 2)
+    while (t.cs < kTailMaxCluster && tail_chunk(P, t.cs) > 4096 &&
+           units * 2 * t.cs <= (t.cs == 1 ? sms : sms * 4 / 5))
+      t.cs *= 2;
+  // What does not fit shared memory in that many CTAs takes more of them.
+  while (t.cs < kTailMaxCluster && tail_chunk(P, t.cs) > kTailCacheCap) t.cs *= 2;
   t.chunk = tail_chunk(P, t.cs);
   // A CTA alone on its SM: 1024 threads (a block of 4096 positions), fewer when the slice is shorter.  More
   // CTAs than SMs: smaller ones side by side, as many as there are and as shared memory holds (heads of
@@ -1085,7 +1091,7 @@ TailShape tail_shape(const LaunchCtx& c) {
     while (t.threads < 1024 &&
            (1024 / t.threads) * (24576 + (size_t)t.chunk * 17 / 4 + (size_t)t.threads * 32) > 226 * 1024)
       t.threads *= 2;
-  t.cached = t.chunk <= (t.cs == 1 ? kTailCacheCapSolo : kTailCacheCap);
+  t.cached = t.chunk <= kTailCacheCap;
   return t;
 }
 
