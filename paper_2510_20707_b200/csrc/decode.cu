@@ -45,7 +45,8 @@ constexpr int kDecStep = 16;     // cache rows per warp step
 
 constexpr int kDecPitch = 272;                      // bytes between the rows of a slot
 constexpr int kDecSlot = kDecStep * kDecPitch;      // one K or V slot
-constexpr int kDecDepth = 2;                        // steps a warp has on their way or in work
+// Steps a warp has on their way or in work: two with three CTAs on an SM, four when a CTA has an SM for itself.
+constexpr int kDecDepth = 2, kDecDepthAlone = 4;
 
 // Dynamic shared memory for GP = 8 or 16 head slots: per warp its ring and then, the steps being over, its value
 // sums [GP][132] in the same place; the CTA's sums xo [GP][128] behind those of warp 0, in what was its ring (with
@@ -53,9 +54,11 @@ constexpr int kDecDepth = 2;                        // steps a warp has on their
 // sequences of 603 rows and 12 heads 25.3 us); wm / wz [warps][16], xm / xz [16], allm / allz [8][16] every
 // rank's (reference, sum) during the cluster merge.
 constexpr int kDecHeadPitch = kHeadDim + 4;   // floats between the heads of a warp's value sums
-constexpr size_t kDecWarpBytes = 2 * (size_t)kDecDepth * kDecSlot;
-static_assert(16 * (kDecHeadPitch + kHeadDim) * 4 <= kDecWarpBytes, "sums of a warp and of the CTA fit a ring");
-constexpr size_t kDecSmem = kDecWarps * kDecWarpBytes + (2 * kDecWarps + 2 + 2 * 8) * kDecMaxG * 4;
+__host__ __device__ constexpr size_t dec_warp_bytes(int depth) { return 2 * (size_t)depth * kDecSlot; }
+static_assert(16 * (kDecHeadPitch + kHeadDim) * 4 <= dec_warp_bytes(kDecDepth), "sums of a warp and of the CTA fit a ring");
+constexpr size_t dec_smem(int depth) {
+  return kDecWarps * dec_warp_bytes(depth) + (2 * kDecWarps + 2 + 2 * 8) * kDecMaxG * 4;
+}
 // Slot of dimension `dim` inside a head of a warp's value sums: one pad word per 32 dimensions
 // and a head pitch of 132 put the 32 lanes of a fragment store (8 heads x 4 dimensions 32 apart)
 // into 32 different banks.
@@ -120,8 +123,9 @@ __device__ __forceinline__ void copy_rows(unsigned char* slot, const __nv_bfloat
 __device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 // All copies of this lane but the newest groups (everything asked for after the tile needed now) have landed;
 // with every lane of the warp past this, all rows of that tile.
+template <int DEPTH>
 __device__ __forceinline__ void copy_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(2 * kDecDepth - 1) : "memory");
+  asm volatile("cp.async.wait_group %0;" ::"n"(2 * DEPTH - 1) : "memory");
   __syncwarp();
 }
 
@@ -265,7 +269,7 @@ __device__ __forceinline__ void store_partial(const DecState<WIDE>& st, float* w
 // grid: n_layers * batch * H * S, clusters of S.  WIDE: more than eight query heads per KV head
 // (head slots 8..15 of the tiles carry data).
 constexpr int kDecPerSm = 3;   // CTAs per SM (12 warps, 208 KB of slots)
-template <bool WIDE>
+template <bool WIDE, int DEPTH>
 __global__ void __launch_bounds__(kDecThreads, kDecPerSm)
 k_decode_attention(const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __restrict__ Vc,
                    const int* __restrict__ row_offsets, const long long rows_cap,
@@ -273,7 +277,7 @@ k_decode_attention(const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __
                    const float scale_log2e, const int max_rows, float* __restrict__ out) {
   constexpr int GP = WIDE ? 16 : 8;
   extern __shared__ __align__(16) float dsm[];
-  constexpr int kWarpFloats = (int)(kDecWarpBytes / 4);
+  constexpr int kWarpFloats = (int)(dec_warp_bytes(DEPTH) / 4);
   float* wacc = dsm;                                   // [warps]: slots, then [GP][kDecHeadPitch]
   float* xo = wacc + GP * kDecHeadPitch;               // [GP][128], behind the sums of warp 0
   float* wm = wacc + kDecWarps * kWarpFloats;          // [warps][16]
@@ -302,7 +306,7 @@ k_decode_attention(const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __
     const int stride = S * kDecWarps;
     int step = crank * kDecWarps + warp;
 #pragma unroll
-    for (int d = 0; d < kDecDepth; ++d) {
+    for (int d = 0; d < DEPTH; ++d) {
       const int ahead = step + d * stride;
       if (ahead < nsteps) copy_rows(ring + 2 * d * kDecSlot, Kb, ahead * kDecStep, n, lane);
       copy_commit();
@@ -310,20 +314,20 @@ k_decode_attention(const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __
       copy_commit();
     }
     st.start(q + qoff, G, g, t);
-    for (int d = 0; step < nsteps; step += stride, d = d + 1 == kDecDepth ? 0 : d + 1) {
+    for (int d = 0; step < nsteps; step += stride, d = d + 1 == DEPTH ? 0 : d + 1) {
       unsigned char* sK = ring + 2 * d * kDecSlot;
       unsigned char* sV = sK + kDecSlot;
-      const int ahead = step + kDecDepth * stride;
+      const int ahead = step + DEPTH * stride;
       const int left = n - step * kDecStep;
       float p[2][DecState<WIDE>::R];
-      copy_wait();     // K of this step
+      copy_wait<DEPTH>();     // K of this step
       st.logits(sK, g, t, p);
       __syncwarp();    // every lane has read the slot
       if (ahead < nsteps) copy_rows(sK, Kb, ahead * kDecStep, n, lane);
       copy_commit();
       st.template weights<0>(p, st.m0, st.z0, left, scale_log2e, t);
       if constexpr (WIDE) st.template weights<2>(p, st.m1, st.z1, left, scale_log2e, t);
-      copy_wait();     // V of this step
+      copy_wait<DEPTH>();     // V of this step
       st.values(sV, g, t, p);
       __syncwarp();
       if (ahead < nsteps) copy_rows(sV, Vb, ahead * kDecStep, n, lane);
@@ -410,24 +414,45 @@ extern "C" int mixkv_decode_attention(const void* K_cache, const void* V_cache,
   const bool wide = gqa_ratio > 8;
   // CTAs per unit: as many as still fit the GPU in one wave while every warp keeps a step (one head of 512
   // rows on 8 CTAs 5.8 us, on 4 6.4; 112 heads of 512 rows on 3 CTAs each 11.5 us, on 2 12.8)
-  const long long slots = (long long)kDecPerSm * device_sm_count();
+  const int sms = device_sm_count();
+  const long long slots = (long long)kDecPerSm * sms;
   const long long steps = ((long long)max_rows + kDecStep - 1) / kDecStep;
-  long long most = slots / units < steps / kDecWarps ? slots / units : steps / kDecWarps;
-  const int S = most < 1 ? 1 : most > 8 ? 8 : (int)most;
-  const size_t smem = kDecSmem;
+  const long long most = slots / units < steps / kDecWarps ? slots / units : steps / kDecWarps;
+  int S = most < 1 ? 1 : most > 8 ? 8 : (int)most;
+  // One wave and a bit of a second: halves even that out where a warp then still has eight steps (560 ragged heads
+  // of 2500 rows on average 152 -> 130 us, with five steps per warp or a nearly empty second wave nothing)
+  if (units * 10 >= slots * 11 && units * 2 <= slots * 3 && steps >= 2 * kDecWarps * 8) S = 2;
+  // Eight to 32 units: a CTA has an SM for itself, with the deeper ring.  Where there is room for three, the CTAs
+  // of a cluster end up sharing SMs while others idle (13 units of 3500 rows 15.9 -> 10.3 us, 20 of them 16.2 -> 13.7,
+  // 30 of 1000 9.3 -> 8.5; fewer than eight units gain nothing, and 16 x 8 CTAs spread well as they are: 12.7 us
+  // against 13.0).  The clusters have to be resident all at once, or a second wave doubles the time; a
+  // cluster lies in one group of 16 or more SMs, so 15 clusters of eight fit, 22 of six, 25 of five and 32 of four.
+  const int fit[9] = {0, 0, 0, 0, 32, 25, 22, 15, 15};
+  bool alone = false;
+  if (units >= 8 && units != 16 && sms >= 148)
+    for (int x = 8; x >= 4 && !alone; --x)
+      if (units <= fit[x]) {
+        alone = steps >= kDecWarps * x;
+        if (alone) S = x;
+        break;
+      }
+  const int depth = alone ? kDecDepthAlone : kDecDepth;
+  const size_t smem = dec_smem(depth);
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)kHeadDim);
   const __nv_bfloat16 *K = reinterpret_cast<const __nv_bfloat16*>(K_cache),
                       *V = reinterpret_cast<const __nv_bfloat16*>(V_cache),
                       *qq = reinterpret_cast<const __nv_bfloat16*>(q);
-  auto kernel = wide ? k_decode_attention<true> : k_decode_attention<false>;
+  auto kernel = alone ? (wide ? k_decode_attention<true, kDecDepthAlone> : k_decode_attention<false, kDecDepthAlone>)
+                      : (wide ? k_decode_attention<true, kDecDepth> : k_decode_attention<false, kDecDepth>);
   if (smem > 48 * 1024) {
-    static bool done[2][64] = {};
+    static bool done[4][64] = {};
+    const int variant = 2 * alone + wide;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return MIXKV_ERR_CUDA;
-    if (dev < 0 || dev >= 64 || !done[wide][dev]) {
+    if (dev < 0 || dev >= 64 || !done[variant][dev]) {
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return MIXKV_ERR_CUDA;
-      if (dev >= 0 && dev < 64) done[wide][dev] = true;
+      if (dev >= 0 && dev < 64) done[variant][dev] = true;
     }
   }
   const cudaError_t e = launch_pdl(kernel, dim3((unsigned)(units * S)), dim3(kDecThreads), smem, (cudaStream_t)stream, S,

@@ -99,7 +99,9 @@ def test_step_edges_and_head_counts(G):
 @pytest.mark.parametrize("NL,batch,H,G,lo,hi", [
     (4, 16, 8, 7, 0, 40),          # 512 units: empty heads, fewer rows than the warps of a CTA take
     (3, 13, 9, 16, 1, 300),        # wide heads, a unit count that no number of CTAs divides
-    (28, 3, 4, 1, 120, 140)])      # steps of all eight warps and one more
+    (28, 3, 4, 1, 120, 140),       # steps of all eight warps and one more
+    (1, 15, 1, 4, 1500, 1600), (1, 16, 1, 9, 1500, 1600), (2, 4, 4, 7, 1, 900),   # few units, a CTA alone on its SM
+    (10, 13, 4, 7, 1, 1020)])      # a second wave that is short: two CTAs per unit
 def test_more_units_than_one_wave(NL, batch, H, G, lo, hi):
     rng = np.random.default_rng(NL * batch)
     counts = rng.integers(lo, hi + 1, (NL, batch * H))
