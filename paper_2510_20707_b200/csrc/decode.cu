@@ -426,11 +426,15 @@ extern "C" int mixkv_decode_attention(const void* K_cache, const void* V_cache,
   // of a cluster end up sharing SMs while others idle (13 units of 3500 rows 15.9 -> 10.3 us, 20 of them 16.2 -> 13.7,
   // 30 of 1000 9.3 -> 8.5; fewer than eight units gain nothing, and 16 x 8 CTAs spread well as they are: 12.7 us
   // against 13.0).  The clusters have to be resident all at once, or a second wave doubles the time; a
-  // cluster lies in one group of 16 or more SMs, so 15 clusters of eight fit, 22 of six, 25 of five and 32 of four.
+  // cluster lies in one group of SMs, and 15 clusters of eight fit, 22 of six, 25 of five and 32 of four.
+  // Fewer than eight CTAs only where the heads can be of one length (the cache holds max_rows rows of every head):
+  // else the longest head decides, and it wants eight (28 ragged heads of 2500 rows on average 21.7 us on four
+  // CTAs, 17.7 on eight).
   const int fit[9] = {0, 0, 0, 0, 32, 25, 22, 15, 15};
+  const bool even = rows_cap >= (long long)max_rows * batch * kv_heads;
   bool alone = false;
   if (units >= 8 && units != 16 && sms >= 148)
-    for (int x = 8; x >= 4 && !alone; --x)
+    for (int x = 8; x >= (even ? 4 : 8) && !alone; --x)
       if (units <= fit[x]) {
         alone = steps >= kDecWarps * x;
         if (alone) S = x;
