@@ -527,7 +527,7 @@ constexpr int kBudgetCluster = 8;
 constexpr int kBudgetThreads = 1024;
 
 // Head budgets of one sequence under the adaptive rule (see mixkv.h).  One CTA per (sequence,
-// layer) when the call has many of them, else a cluster of kBudgetCluster CTAs, each with a
+// layer) when the call has many of them, else a cluster of up to kBudgetCluster CTAs, each with a
 // slice of the positions of every head.  A CTA turns its H * n pooled scores into
 // order-preserving keys once and keeps them in shared memory when they fit (cache_cap keys);
 // otherwise every sweep reads them from global memory.
@@ -1036,8 +1036,16 @@ cudaError_t launch_given_budgets(const LaunchCtx& c, const int* budgets, int* co
 }
 
 cudaError_t launch_budget(const LaunchCtx& c, const float* scores, int* counts) {
-  // few (sequence, layer) pairs: a cluster of CTAs each; many: one CTA each
-  const int cs = c.st.batch * c.st.layers < device_sm_count() / kBudgetCluster ? kBudgetCluster : 1;
+  // CTAs per (sequence, layer) pair: one while it has 8192 keys or less of all heads (the exchanges cost as much as
+  // the sweeps they save), else as many as leave each that much and are all resident at once, one per SM (120 CTAs
+  // in clusters of four or eight ran in one wave, 136 did not).  Whole calls, eight CTAs each up to 17 pairs and one
+  // beyond that against this: 17 pairs of 3000 keys 50.1 / 37.9 us; 17, 20, 28 of 96000 217 / 204, 368 / 238, 439 /
+  // 322 us; 28, 56 of 32000 134 / 122, 227 / 224 us.
+  const int pairs = c.st.batch * c.st.layers;
+  int cs = 1;
+  while (cs < kBudgetCluster && (long long)c.st.H * c.max_prefix > 8192LL * cs &&
+         pairs * 2 * cs <= device_sm_count() * 13 / 16)
+    cs *= 2;
   const size_t chunk = ((size_t)c.max_prefix + cs - 1) / cs;
   // the keys of a CTA's slice of the longest sequence in shared memory when they fit
   const size_t want = (size_t)c.st.H * ((chunk + 31) / 32) * 128;

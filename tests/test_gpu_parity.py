@@ -307,6 +307,27 @@ def test_threshold_search_edges(H, n, levels, want):
             assert (idx[b, h] == np.sort(order[:want])).all(), (b, h)
 
 
+@pytest.mark.parametrize("batch,H,P", [
+    (1, 8, 1024), (1, 8, 1025),                                # one CTA per sequence, two
+    (15, 8, 4100), (16, 8, 4100), (30, 8, 4100),               # clusters of eight, of four
+    (31, 8, 2100), (60, 8, 1030), (61, 8, 1030)])              # of two; one CTA
+def test_adaptive_budget_cluster_edges(batch, H, P):
+    # levels: ties at the global threshold, which go to the lower (head, position)
+    W = 16
+    rng = np.random.default_rng(batch * P)
+    cu = (np.arange(batch + 1) * (P + W)).astype(np.int32)
+    s = (rng.integers(0, 700, size=(H, batch * P)) / np.float32(700)).astype(np.float32)
+    po = oracle.Params(kv_heads=H, gqa_ratio=1, window=W, budget=W + 100, budget_mode=1)
+    pg = binding.Params(kv_heads=H, gqa_ratio=1, window=W, budget=W + 100, budget_mode=1)
+    many = batch > 1
+    ref = oracle.select(s, po, cu=cu if many else None)
+    got = binding.select(torch.from_numpy(s).cuda(), pg, cu_seqlens=[int(c) for c in cu] if many else None)
+    offs = got["idx_offsets"].cpu().numpy()
+    assert np.array_equal(got["counts"].cpu().numpy(), ref["counts"].reshape(-1))
+    assert np.array_equal(offs, ref["idx_offsets"])
+    assert np.array_equal(got["idx"].cpu().numpy()[:offs[-1]], ref["idx"])
+
+
 def test_long_sequence_cluster_tail():
     # 65536 keys per head: the cluster shape of the tail kernel with 16 positions per thread
     wl = synth.small_workload(H=2, G=4, W=32, seq_lens=(65536,), pool_kernel=7, budget=512,
