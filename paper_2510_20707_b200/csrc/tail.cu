@@ -647,6 +647,7 @@ __host__ __device__ __forceinline__ int tail_chunk(const int P, const int cs) {
 // ------------------------------------------------------------------------------ tail
 constexpr int kTailMaxCluster = 8;
 constexpr int kTailCacheCap = 40960;       // positions a CTA keeps in shared memory
+constexpr int kTailCacheCapFull = 16384;   // the same in a cluster of eight: few, very long heads go unfused beyond
 constexpr int kTailRowCap = 1024;          // selected rows of a CTA listed in shared memory for the gather
 
 struct TailKernelArgs {
@@ -1099,7 +1100,7 @@ TailShape tail_shape(const LaunchCtx& c) {
     while (t.threads < 1024 &&
            (1024 / t.threads) * (24576 + (size_t)t.chunk * 17 / 4 + (size_t)t.threads * 32) > 226 * 1024)
       t.threads *= 2;
-  t.cached = t.chunk <= kTailCacheCap;
+  t.cached = t.chunk <= (t.cs == kTailMaxCluster ? kTailCacheCapFull : kTailCacheCap);
   return t;
 }
 

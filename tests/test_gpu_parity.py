@@ -282,8 +282,8 @@ def test_whole_head_ctas_select_exactly(levels):
     (2, 9000, 0, 700), (2, 9000, 40, 2000), (1, 33000, 0, 1), (1, 33000, 700, 1500),   # clusters of 4 and 8
     (14, 33000, 0, 300), (15, 33000, 9, 300), (29, 9000, 0, 50), (30, 9000, 0, 50), (60, 9000, 50, 77),   # 8, 4, 2
     (200, 300, 20, 60), (500, 2000, 0, 129),                                  # more CTAs than SMs
-    (1, 140000, 300, 900),                                                    # long slices of a cluster
-    (1, 330000, 300, 900)])                                                   # keys not held in shared memory
+    (29, 70000, 300, 900), (10, 130000, 300, 900),                            # long slices of four and of eight CTAs
+    (1, 140000, 300, 900)])                                                   # keys not held in shared memory
 def test_threshold_search_edges(H, n, levels, want):
     # one, a few or no repeated values (levels = number of distinct scores), the range spread over many
     # octaves and both signs
