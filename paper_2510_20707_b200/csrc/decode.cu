@@ -45,8 +45,9 @@ constexpr int kDecStep = 16;     // cache rows per warp step
 
 constexpr int kDecPitch = 272;                      // bytes between the rows of a slot
 constexpr int kDecSlot = kDecStep * kDecPitch;      // one K or V slot
-// Steps a warp has on their way or in work: two with three CTAs on an SM, four when a CTA has an SM for itself.
-constexpr int kDecDepth = 2, kDecDepthAlone = 4;
+// Steps a warp has on their way or in work: two with three CTAs on an SM, three with two, four when a CTA has an
+// SM for itself.
+constexpr int kDecDepth = 2, kDecDepthPair = 3, kDecDepthAlone = 4;
 
 // Dynamic shared memory for GP = 8 or 16 head slots: per warp its ring and then, the steps being over, its value
 // sums [GP][132] in the same place; the CTA's sums xo [GP][128] behind those of warp 0, in what was its ring (with
@@ -440,17 +441,22 @@ extern "C" int mixkv_decode_attention(const void* K_cache, const void* V_cache,
         if (alone) S = x;
         break;
       }
-  const int depth = alone ? kDecDepthAlone : kDecDepth;
+  // A CTA per unit and no more than two per SM: those two, with the ring of three (with room for a third some SMs
+  // get three and others one: 296 units of 3400 rows 102.8 -> 89.7 us, 280 of 5000 142.6 -> 124.4, 256 of 300
+  // 13.6 -> 12.9; 240 units of 3400 rows 77.1 -> 78.3, of 512 ragged 31.8 -> 29.7).
+  const bool pair = !alone && S == 1 && units > sms && units <= 2LL * sms;
+  const int depth = alone ? kDecDepthAlone : pair ? kDecDepthPair : kDecDepth;
   const size_t smem = dec_smem(depth);
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)kHeadDim);
   const __nv_bfloat16 *K = reinterpret_cast<const __nv_bfloat16*>(K_cache),
                       *V = reinterpret_cast<const __nv_bfloat16*>(V_cache),
                       *qq = reinterpret_cast<const __nv_bfloat16*>(q);
-  auto kernel = alone ? (wide ? k_decode_attention<true, kDecDepthAlone> : k_decode_attention<false, kDecDepthAlone>)
-                      : (wide ? k_decode_attention<true, kDecDepth> : k_decode_attention<false, kDecDepth>);
+  auto kernel = alone  ? (wide ? k_decode_attention<true, kDecDepthAlone> : k_decode_attention<false, kDecDepthAlone>)
+                : pair ? (wide ? k_decode_attention<true, kDecDepthPair> : k_decode_attention<false, kDecDepthPair>)
+                       : (wide ? k_decode_attention<true, kDecDepth> : k_decode_attention<false, kDecDepth>);
   if (smem > 48 * 1024) {
-    static bool done[4][64] = {};
-    const int variant = 2 * alone + wide;
+    static bool done[6][64] = {};
+    const int variant = 2 * (depth - kDecDepth) + wide;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return MIXKV_ERR_CUDA;
     if (dev < 0 || dev >= 64 || !done[variant][dev]) {

@@ -101,6 +101,7 @@ def test_step_edges_and_head_counts(G):
     (3, 13, 9, 16, 1, 300),        # wide heads, a unit count that no number of CTAs divides
     (28, 3, 4, 1, 120, 140),       # steps of all eight warps and one more
     (1, 15, 1, 4, 1500, 1600), (1, 16, 1, 9, 1500, 1600), (2, 4, 4, 7, 1, 900),   # few units, a CTA alone on its SM
+    (8, 7, 4, 7, 0, 200), (2, 37, 4, 16, 1, 130), (1, 149, 1, 7, 1, 120),   # one wave of two CTAs per SM
     (10, 13, 4, 7, 1, 1020)])      # a second wave that is short: two CTAs per unit
 def test_more_units_than_one_wave(NL, batch, H, G, lo, hi):
     rng = np.random.default_rng(NL * batch)
