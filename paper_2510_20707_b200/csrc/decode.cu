@@ -418,8 +418,15 @@ extern "C" int mixkv_decode_attention(const void* K_cache, const void* V_cache,
   const int sms = device_sm_count();
   const long long slots = (long long)kDecPerSm * sms;
   const long long steps = ((long long)max_rows + kDecStep - 1) / kDecStep;
-  const long long most = slots / units < steps / kDecWarps ? slots / units : steps / kDecWarps;
-  int S = most < 1 ? 1 : most > 8 ? 8 : (int)most;
+  // A cluster lies in one group of SMs, so not every place can be taken: at three CTAs per SM 48 clusters of eight
+  // were resident at once, 56 of seven, 70 of six, 82 of five, 104 of four, 142 of three, and one more of any of them
+  // cost a second wave (units of 1500 rows: 48 on eight CTAs 12.0 us, 49 17.3, on seven 13; 70 on six 15.3, 72 20.7, on
+  // five 16.2).
+  const int whole[9] = {0, 0, 222, 142, 104, 82, 70, 56, 48};
+  long long most = slots / units < 8 ? slots / units : 8;
+  while (most > 1 && units * 148 > (long long)whole[most] * sms) --most;
+  if (most > steps / kDecWarps) most = steps / kDecWarps;
+  int S = most < 1 ? 1 : (int)most;
   // One wave and a bit of a second: halves even that out where a warp then still has eight steps (560 ragged heads
   // of 2500 rows on average 152 -> 130 us, with five steps per warp or a nearly empty second wave nothing)
   if (units * 10 >= slots * 11 && units * 2 <= slots * 3 && steps >= 2 * kDecWarps * 8) S = 2;

@@ -102,6 +102,7 @@ def test_step_edges_and_head_counts(G):
     (28, 3, 4, 1, 120, 140),       # steps of all eight warps and one more
     (1, 15, 1, 4, 1500, 1600), (1, 16, 1, 9, 1500, 1600), (2, 4, 4, 7, 1, 900),   # few units, a CTA alone on its SM
     (8, 7, 4, 7, 0, 200), (2, 37, 4, 16, 1, 130), (1, 149, 1, 7, 1, 120),   # one wave of two CTAs per SM
+    (7, 7, 1, 7, 500, 700), (3, 19, 1, 12, 1, 500), (1, 143, 1, 4, 100, 200),   # one more than fits at 8, 7 and 3 CTAs
     (10, 13, 4, 7, 1, 1020)])      # a second wave that is short: two CTAs per unit
 def test_more_units_than_one_wave(NL, batch, H, G, lo, hi):
     rng = np.random.default_rng(NL * batch)
