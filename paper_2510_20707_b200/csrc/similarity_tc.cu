@@ -250,6 +250,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
     constexpr int kChunks = NT == 128 ? 2 : 1;
     float* st = sT + (warp - kGEpiWarp0) * 1024;
     const float inv_b = 1.0f / (float)block, last_n = (float)(L - (T - 1) * block);
+    const bool rows16 = (T & 3) == 0 && (reinterpret_cast<uintptr_t>(cells) & 15) == 0;
     int tile = 0;
     for (GramWalk<NT> w(T, per_head, lo, hi); w.valid(); w.next()) {
       const int i0 = w.I * 128 + quarter * 32, i = i0 + lane;   // this thread's block I
@@ -294,9 +295,9 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
         }
         // Both images go through a swizzled 32 x 32 tile in shared memory (cell (i, j) of the chunk at word
         // 4 ((j / 4) ^ (i & 7)) + j % 4 of row i) and leave as 16-byte stores, four rows of 128 bytes per
-        // instruction; where the rows of the map are not 16-byte aligned, or the chunk is cut by its edge, as
-        // 4-byte stores, one row per instruction.
-        const bool vec = (T & 3) == 0 && i0 + 32 <= T && j0 + 32 <= T;
+        // instruction; where the rows of the map are not 16-byte aligned (a caller's map need only be aligned to
+        // 4 bytes), or the chunk is cut by its edge, as 4-byte stores, one row per instruction.
+        const bool vec = rows16 && i0 + 32 <= T && j0 + 32 <= T;
         const int sub = lane >> 3, quad = lane & 7;   // row of a group of four, four columns of it
         if (!on_diag) {   // mirrored tile: rows J
           if (vec) {

@@ -99,6 +99,28 @@ def test_keys_and_values_of_a_c2_layer():
     run(x["V"], 256)
 
 
+@pytest.mark.parametrize("L,block", [(256, 1), (2048, 16), (32768, 256)])
+def test_map_on_a_four_byte_boundary(L, block):
+    # fp32 outputs need 4-byte alignment only: a map that is a slice of a larger buffer gets the same bits as an
+    # aligned one, and nothing around it is written (maps of 256, 128 and 128 cells a side: rows of whole 16 bytes)
+    import ctypes as C
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    X = torch.randn((2, L, 128), generator=gen, device="cuda").bfloat16()
+    ref, mean = binding.similarity_map(X, block)
+    lib, need = binding.load_library(), C.c_size_t(0)
+    assert lib.mixkv_similarity_workspace_size(2, L, block, C.byref(need)) == 0
+    ws = torch.empty(need.value, dtype=torch.uint8, device="cuda")
+    for skip in (1, 2, 3):
+        buf = torch.full((ref.numel() + 8,), 7.0, device="cuda")
+        m = torch.zeros(2, device="cuda")
+        rc = lib.mixkv_similarity_map(X.data_ptr(), 2, L, 128, block, ws.data_ptr(), ws.numel(),
+                                      buf.data_ptr() + 4 * skip, m.data_ptr(),
+                                      torch.cuda.current_stream().cuda_stream)
+        torch.cuda.synchronize()
+        assert rc == 0 and torch.equal(buf[skip:skip + ref.numel()].view_as(ref), ref) and torch.equal(m, mean)
+        assert (buf[:skip] == 7).all() and (buf[skip + ref.numel():] == 7).all()
+
+
 def test_rejects_bad_arguments():
     X = torch.zeros((1, 16, 64), dtype=torch.bfloat16, device="cuda")
     with pytest.raises(binding.MixKVError):
