@@ -6,6 +6,10 @@
 // GPU busy for less time than interpreted marshalling takes.  Through ctypes one decode call cost 15 us of
 // host time for 7 us of GPU time and a scores + select pair 89 us; here they cost 5.5 and 24 us, one
 // layer's compression 8.6 us.  Output tensors come from torch's caching allocator without the dispatcher.
+//
+// The interpreter lock is given up around everything that can block (Unlocked, below): a launch waits while the
+// stream's queue is full, an allocation may wait for the device, and a host callback on that stream, or any
+// other thread of the program, may need the interpreter before either goes on.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -47,6 +51,18 @@ struct Names {
 
 // A Python exception is set; unwinds to the entry point.
 struct Raised {};
+
+// No interpreter lock in this scope.
+struct Unlocked {
+  PyThreadState* state = PyEval_SaveThread();
+  ~Unlocked() { PyEval_RestoreThread(state); }
+};
+// A call of the library without the lock; the arguments are evaluated before it is given up.
+template <typename... P, typename... A>
+int enqueue(int (*fn)(P...), A... args) {
+  const Unlocked u;
+  return fn(args...);
+}
 
 [[noreturn]] void fail(PyObject* type, const char* what) {
   PyErr_SetString(type, what);
@@ -173,7 +189,12 @@ void* stream_of(PyObject* o) {
 }
 
 at::Tensor empty(at::IntArrayRef size, at::ScalarType type, const at::Tensor& like) {
+  const Unlocked u;
   return at::Tensor(at::detail::empty_cuda(size, type, like.device(), std::nullopt));
+}
+at::Tensor zero_word(const at::Tensor& like) {   // (enqueues a fill)
+  const Unlocked u;
+  return at::zeros({1}, like.options().dtype(at::kInt));
 }
 int32_t* ip(const at::Tensor& t) { return static_cast<int32_t*>(t.data_ptr()); }
 float* fp(const at::Tensor& t) { return static_cast<float*>(t.data_ptr()); }
@@ -272,8 +293,8 @@ PyObject* py_scores(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const float* rin = ptr<float>(a[5]);
     float *pe = parts ? fp(s_ex) : nullptr, *pd = parts ? fp(s_div) : nullptr,
           *pr = parts ? fp(rbar) : nullptr;
-    check_status(api.scores(k, v, q, cu.data(), cu.batch, (int)Ltot, &p, fixed ? 1 : 0, fixed ? nullptr : ws->data,
-                            fixed ? 0 : ws->bytes, fp(s_comp), pe, pd, pr, rin, ip(status), stream),
+    check_status(enqueue(api.scores, k, v, q, cu.data(), cu.batch, (int)Ltot, &p, fixed ? 1 : 0, fixed ? nullptr : ws->data,
+                         fixed ? 0 : ws->bytes, fp(s_comp), pe, pd, pr, rin, ip(status), stream),
                  fixed ? "mixkv_scores_static" : "mixkv_scores");
     Dict out;
     put(out.d, nm.s_comp, s_comp);
@@ -299,8 +320,8 @@ PyObject* py_select(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int64_t cap = std::max<int64_t>(BH * (p.budget - p.window), 1);
     at::Tensor idx = empty({cap}, at::kInt, s), counts = empty({BH}, at::kInt, s),
                offs = empty({BH + 1}, at::kInt, s), status = empty({1}, at::kInt, s);
-    check_status(api.select(ptr<const float>(a[0]), cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes,
-                            ip(idx), ip(counts), ip(offs), ip(status), stream_of(a[4])),
+    check_status(enqueue(api.select, ptr<const float>(a[0]), cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes,
+                         ip(idx), ip(counts), ip(offs), ip(status), stream_of(a[4])),
                  "mixkv_select");
     Dict out;
     put(out.d, nm.idx, idx);
@@ -329,7 +350,7 @@ PyObject* compress_outputs(PyObject* given, const bool aux, const int64_t lead, 
   put(out.d, nm.K_out, make({rows, K.size(-1)}, at::kBFloat16));
   put(out.d, nm.V_out, make({rows, K.size(-1)}, at::kBFloat16));
   put(out.d, nm.out_row_offsets, make({BH + 1}, at::kInt));
-  put(out.d, nm.status, at::zeros({1}, K.options().dtype(at::kInt)));
+  put(out.d, nm.status, zero_word(K));
   if (aux) {
     put(out.d, nm.idx, make({cap}, at::kInt));
     put(out.d, nm.counts, make({BH}, at::kInt));
@@ -380,10 +401,10 @@ PyObject* py_compress_layer(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const long long events = PyLong_AsLongLong(a[10]);
     const long n_events = PyLong_AsLong(a[11]);
     if (PyErr_Occurred()) throw Raised();
-    check_status(api.layer(ptr(a[0]), ptr(a[1]), ptr(a[2]), cu.data(), cu.batch, (int)Ltot, &p, ws.data,
-                           ws.bytes, ptr<const float>(a[5]), o.K, o.V, o.row_offsets, o.idx, o.counts,
-                           o.idx_offsets, o.s_comp, o.status, stream_of(a[7]),
-                           reinterpret_cast<void* const*>(events), (int)n_events),
+    check_status(enqueue(api.layer, ptr(a[0]), ptr(a[1]), ptr(a[2]), cu.data(), cu.batch, (int)Ltot, &p, ws.data,
+                         ws.bytes, ptr<const float>(a[5]), o.K, o.V, o.row_offsets, o.idx, o.counts,
+                         o.idx_offsets, o.s_comp, o.status, stream_of(a[7]),
+                         reinterpret_cast<void* const*>(events), (int)n_events),
                  "mixkv_compress_layer");
     return out.release();
   });
@@ -429,15 +450,15 @@ PyObject* py_compress_layers(PyObject*, PyObject* const* a, Py_ssize_t n) {
       want_contiguous(hb);
       if (hb.scalar_type() != at::kInt || hb.dim() != 2 || hb.size(0) != NL || hb.size(1) != BH || n_events)
         fail(PyExc_AssertionError, "head_budgets must be an int32 tensor [layers, batch * H], without events");
-      check_status(api.budgeted(K.data_ptr(), V.data_ptr(), Q.data_ptr(), (int)NL, K.stride(0), Q.stride(0),
-                                cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes, rin, ip(hb), o.K, o.V,
-                                o.row_offsets, o.idx, o.counts, o.idx_offsets, o.s_comp, o.status, stream),
+      check_status(enqueue(api.budgeted, K.data_ptr(), V.data_ptr(), Q.data_ptr(), (int)NL, K.stride(0), Q.stride(0),
+                           cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes, rin, ip(hb), o.K, o.V,
+                           o.row_offsets, o.idx, o.counts, o.idx_offsets, o.s_comp, o.status, stream),
                    "mixkv_compress_layers_budgeted");
     } else {
-      check_status(api.layers(K.data_ptr(), V.data_ptr(), Q.data_ptr(), (int)NL, K.stride(0), Q.stride(0),
-                              cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes, rin, o.K, o.V,
-                              o.row_offsets, o.idx, o.counts, o.idx_offsets, o.s_comp, o.status, stream,
-                              reinterpret_cast<void* const*>(events), (int)n_events),
+      check_status(enqueue(api.layers, K.data_ptr(), V.data_ptr(), Q.data_ptr(), (int)NL, K.stride(0), Q.stride(0),
+                           cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes, rin, o.K, o.V,
+                           o.row_offsets, o.idx, o.counts, o.idx_offsets, o.s_comp, o.status, stream,
+                           reinterpret_cast<void* const*>(events), (int)n_events),
                    "mixkv_compress_layers");
     }
     return out.release();
@@ -459,8 +480,8 @@ PyObject* py_similarity_map(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int64_t T = (L + block - 1) / block;
     at::Tensor ws = empty({(int64_t)need}, at::kByte, X), cells = empty({heads, T, T}, at::kFloat, X), mean;
     if (PyObject_IsTrue(a[2]) == 1) mean = empty({heads}, at::kFloat, X);
-    check_status(api.sim_map(X.data_ptr(), heads, L, (int)X.size(2), (int)block, ws.data_ptr(), need, fp(cells),
-                             mean.defined() ? fp(mean) : nullptr, stream_of(a[3])),
+    check_status(enqueue(api.sim_map, X.data_ptr(), heads, L, (int)X.size(2), (int)block, ws.data_ptr(), need, fp(cells),
+                         mean.defined() ? fp(mean) : nullptr, stream_of(a[3])),
                  "mixkv_similarity_map");
     Ref c(THPVariable_Wrap(cells)), m(mean.defined() ? THPVariable_Wrap(mean) : Py_NewRef(Py_None));
     if (!c.o || !m.o) throw Raised();
@@ -482,9 +503,9 @@ PyObject* py_decode_attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const double scale = PyFloat_AsDouble(a[7]);
     if (PyErr_Occurred()) throw Raised();
     at::Tensor out = empty(q.sizes(), at::kFloat, q);
-    check_status(api.decode(K.data_ptr(), V.data_ptr(), ip(offs), K.size(1), q.data_ptr(), (int)K.size(0),
-                            (int)q.size(1), (int)H, (int)G, (int)K.size(2), (float)scale, (int)rows, fp(out),
-                            stream_of(a[8])),
+    check_status(enqueue(api.decode, K.data_ptr(), V.data_ptr(), ip(offs), K.size(1), q.data_ptr(), (int)K.size(0),
+                         (int)q.size(1), (int)H, (int)G, (int)K.size(2), (float)scale, (int)rows, fp(out),
+                         stream_of(a[8])),
                  "mixkv_decode_attention");
     return THPVariable_Wrap(out);
   });

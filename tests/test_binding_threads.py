@@ -1,0 +1,98 @@
+"""The binding gives up the interpreter lock while a call is in the library: a launch can wait for the GPU, and
+what it waits for may be a callback or another thread that needs the interpreter.  The library is replaced by one
+whose entry points wait until another Python thread lets them go (two seconds at most)."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+from paper_2510_20707_b200 import build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+LIBRARY = r"""
+#include <stdatomic.h>
+#include <stddef.h>
+#include <time.h>
+static atomic_int inside, let_go;
+int entered(void) { return atomic_load(&inside); }
+void release(void) { atomic_store(&let_go, 1); }
+static int wait_for_release(void) {
+  atomic_store(&inside, 1);
+  const struct timespec ms = {0, 1000000};
+  int k = 0;
+  while (!atomic_load(&let_go) && k++ < 2000) nanosleep(&ms, NULL);
+  const int ok = atomic_load(&let_go);
+  atomic_store(&inside, 0);
+  atomic_store(&let_go, 0);
+  return ok ? 0 : -4;
+}
+int mixkv_internal_scores() { return wait_for_release(); }
+int mixkv_internal_select() { return wait_for_release(); }
+int mixkv_compress_layer_traced() { return wait_for_release(); }
+int mixkv_compress_layers() { return wait_for_release(); }
+int mixkv_compress_layers_budgeted() { return wait_for_release(); }
+int mixkv_similarity_map() { return wait_for_release(); }
+int mixkv_decode_attention() { return wait_for_release(); }
+int mixkv_workspace_size_layers(const void* p, int n, int b, long long t, int m, size_t* bytes) {
+  return *bytes = 256, 0;
+}
+int mixkv_similarity_workspace_size(int h, int L, int b, size_t* bytes) { return *bytes = 256, 0; }
+"""
+
+PROGRAM = r"""
+import ctypes, sys, threading, time, types
+import torch
+from paper_2510_20707_b200 import binding
+device, fake = sys.argv[1:]
+lib = ctypes.CDLL(fake)
+binding.load_library()
+binding.LIB_PATH = fake            # what the native module is bound to
+H, L, W, B = 2, 64, 16, 32
+p = binding.Params(kv_heads=H, gqa_ratio=1, window=W, budget=B)
+t = lambda *shape, dtype=torch.bfloat16: torch.zeros(shape, dtype=dtype, device=device)
+i32 = torch.int32
+K, Q = t(1, H, L, 128), t(1, 1, H, W, 128)
+# "cpu": only the calls that need no new tensor; nothing looks at the stream or at the memory
+stream = types.SimpleNamespace(cuda_stream=0) if device == "cpu" else None
+ws = t(256, dtype=torch.uint8)
+out = dict(K_out=t(1, H * B, 128), V_out=t(1, H * B, 128), out_row_offsets=t(1, H + 1, dtype=i32), status=t(1, dtype=i32))
+one = dict(out, **{k: out[k][0] for k in ("K_out", "V_out", "out_row_offsets")})
+kw = dict(workspace=ws, stream=stream)
+calls = dict(
+    layer=lambda: binding.compress_layer(K[0], K[0], Q[0], p, out=one, **kw),
+    layers=lambda: binding.compress_layers(K, K, Q, p, out=out, **kw),
+    budgeted=lambda: binding.compress_layers(K, K, Q, p, out=out, head_budgets=t(1, H, dtype=i32), **kw))
+if device != "cpu":
+    calls.update(
+        scores=lambda: binding.scores(K[0], K[0], Q[0], p), static=lambda: binding.scores_static(K[0], K[0], Q[0], p),
+        select=lambda: binding.select(t(H, L - W, dtype=torch.float32), p),
+        new_outputs=lambda: binding.compress_layer(K[0], K[0], Q[0], p),
+        similarity=lambda: binding.similarity_map(K[0], 4),
+        decode=lambda: binding.decode_attention(K[0], K[0], t(H, 2, dtype=i32), t(H, 1, 1, 128), 1, 1, 4))
+for name, call in calls.items():
+    def watch():
+        end = time.monotonic() + 10
+        while not lib.entered() and time.monotonic() < end: time.sleep(0.001)
+        lib.release()
+    th = threading.Thread(target=watch)
+    th.start()
+    try:
+        call()
+    except binding.MixKVError as e:
+        sys.exit(f"{name}: no other thread ran during the call ({e})")
+    th.join()
+print("ok", len(calls))
+"""
+
+
+@pytest.mark.parametrize("device,n", [("cpu", 3), pytest.param("cuda", 9, marks=pytest.mark.gpu)])
+def test_other_threads_run_while_a_call_is_in_the_library(device, n, tmp_path):
+    build.build()
+    src, lib = tmp_path / "waiting.c", tmp_path / "libwaiting.so"
+    src.write_text(LIBRARY)
+    subprocess.run(["gcc", "-std=gnu11", "-O1", "-shared", "-fPIC", "-w", "-o", str(lib), str(src)], check=True)
+    r = subprocess.run([sys.executable, "-c", PROGRAM, device, str(lib)], cwd=ROOT, capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == f"ok {n}", r.stdout + r.stderr
