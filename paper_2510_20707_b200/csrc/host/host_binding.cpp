@@ -171,9 +171,9 @@ struct Offsets {
   }
   const int32_t* data() const { return v.empty() ? nullptr : v.data(); }
   int len(int b, int Ltot) const { return v.empty() ? Ltot : v[(size_t)b + 1] - v[(size_t)b]; }
-  int max_len(int Ltot) const {
-    int m = len(0, Ltot);
-    for (int b = 1; b < batch; ++b) m = std::max(m, len(b, Ltot));
+  int max_len(int Ltot) const {   // (0 where there is no sequence: the library refuses that)
+    int m = 0;
+    for (int b = 0; b < batch; ++b) m = std::max(m, len(b, Ltot));
     return m;
   }
 };

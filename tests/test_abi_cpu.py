@@ -99,3 +99,17 @@ def test_device_check_without_a_device_or_with_one(lib):
         assert (rc, major) == (0, 10)
     else:
         assert rc == -4 and major == 0
+
+
+@pytest.mark.parametrize("cu", [[], [0], [0, 64, 40], [0, 8]])
+def test_binding_refuses_offsets_without_a_sequence(lib, cu):
+    # no sequence, one offset, a descending one, one shorter than the window: refused before anything is allocated
+    import torch
+    K = torch.zeros((2, 64, 128), dtype=torch.bfloat16)
+    p = binding.Params(kv_heads=2, gqa_ratio=1, window=16, budget=32)
+    with pytest.raises(binding.MixKVError) as e:
+        out = {k: torch.zeros(4) for k in ("K_out", "V_out", "out_row_offsets", "status")}
+        ws = None if len(cu) < 2 else torch.zeros(1 << 20, dtype=torch.uint8)
+        binding.compress_layer(K, K, torch.zeros((1, 2, 16, 128), dtype=torch.bfloat16), p, cu_seqlens=cu, out=out,
+                               workspace=ws, stream=type("S", (), {"cuda_stream": 0}))
+    assert e.value.status == -1
