@@ -106,6 +106,11 @@ T* item(PyObject* dict, PyObject* key, const bool required) {   // entry of an o
   return ptr<T>(o);
 }
 
+bool truth(PyObject* o) {
+  const int t = PyObject_IsTrue(o);
+  if (t < 0) throw Raised();
+  return t != 0;
+}
 long attr_int(PyObject* o, PyObject* name) {
   PyObject* v = PyObject_GetAttr(o, name);
   if (!v) throw Raised();
@@ -276,7 +281,7 @@ PyObject* py_scores(PyObject*, PyObject* const* a, Py_ssize_t n) {
     want_dims(K, 3, "K must have three dimensions [H, Ltot, d]");
     const mixkv_params p = params(a[3]);
     const Offsets cu(a[4]);
-    const bool parts = PyObject_IsTrue(a[8]) == 1, fixed = PyObject_IsTrue(a[9]) == 1;
+    const bool parts = truth(a[8]), fixed = truth(a[9]);
     const int64_t H = K.size(0), Ltot = K.size(1), Ptot = Ltot - (int64_t)cu.batch * p.window;
     std::optional<Space> ws;
     if (!fixed) ws.emplace(a[6], p, 1, cu, (int)Ltot, K);
@@ -334,7 +339,7 @@ PyObject* py_select(PyObject*, PyObject* const* a, Py_ssize_t n) {
 
 // Outputs of a compression call: the caller's dict, or a new one.  `lead` is the layer dimension (-1: the
 // one-layer call, whose tensors have none).
-PyObject* compress_outputs(PyObject* given, const bool aux, const int64_t lead, const int64_t rows,
+PyObject* compress_outputs(PyObject* given, PyObject* aux, const int64_t lead, const int64_t rows,
                            const int64_t cap, const int64_t BH, const int64_t H, const int64_t Ptot,
                            const at::Tensor& K) {
   if (given != Py_None) {
@@ -351,7 +356,7 @@ PyObject* compress_outputs(PyObject* given, const bool aux, const int64_t lead, 
   put(out.d, nm.V_out, make({rows, K.size(-1)}, at::kBFloat16));
   put(out.d, nm.out_row_offsets, make({BH + 1}, at::kInt));
   put(out.d, nm.status, zero_word(K));
-  if (aux) {
+  if (truth(aux)) {
     put(out.d, nm.idx, make({cap}, at::kInt));
     put(out.d, nm.counts, make({BH}, at::kInt));
     put(out.d, nm.idx_offsets, make({BH + 1}, at::kInt));
@@ -394,7 +399,7 @@ PyObject* py_compress_layer(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const Offsets cu(a[4]);
     const int64_t H = K.size(0), Ltot = K.size(1), BH = cu.batch * H;
     const Space ws(a[6], p, 1, cu, (int)Ltot, K);
-    Ref out(compress_outputs(a[8], PyObject_IsTrue(a[9]) == 1, -1, BH * p.budget,
+    Ref out(compress_outputs(a[8], a[9], -1, BH * p.budget,
                              std::max<int64_t>(BH * (p.budget - p.window), 1), BH, H,
                              Ltot - (int64_t)cu.batch * p.window, K));
     const OutPtrs o(out.o);
@@ -437,7 +442,7 @@ PyObject* py_compress_layers(PyObject*, PyObject* const* a, Py_ssize_t n) {
     int64_t cap = 0;
     for (int b = 0; b < cu.batch; ++b)
       cap += H * std::min<int64_t>(p.budget - p.window, cu.len(b, (int)Ltot) - p.window);
-    Ref out(compress_outputs(a[8], PyObject_IsTrue(a[9]) == 1, NL, BH * p.budget, std::max<int64_t>(cap, 1), BH,
+    Ref out(compress_outputs(a[8], a[9], NL, BH * p.budget, std::max<int64_t>(cap, 1), BH,
                              H, Ltot - (int64_t)cu.batch * p.window, K));
     const OutPtrs o(out.o);
     const long long events = PyLong_AsLongLong(a[10]);
@@ -479,7 +484,7 @@ PyObject* py_similarity_map(PyObject*, PyObject* const* a, Py_ssize_t n) {
     check_status(api.sim_ws_size(heads, L, (int)block, &need), "mixkv_similarity_workspace_size");
     const int64_t T = (L + block - 1) / block;
     at::Tensor ws = empty({(int64_t)need}, at::kByte, X), cells = empty({heads, T, T}, at::kFloat, X), mean;
-    if (PyObject_IsTrue(a[2]) == 1) mean = empty({heads}, at::kFloat, X);
+    if (truth(a[2])) mean = empty({heads}, at::kFloat, X);
     check_status(enqueue(api.sim_map, X.data_ptr(), heads, L, (int)X.size(2), (int)block, ws.data_ptr(), need, fp(cells),
                          mean.defined() ? fp(mean) : nullptr, stream_of(a[3])),
                  "mixkv_similarity_map");

@@ -113,3 +113,12 @@ def test_binding_refuses_offsets_without_a_sequence(lib, cu):
         binding.compress_layer(K, K, torch.zeros((1, 2, 16, 128), dtype=torch.bfloat16), p, cu_seqlens=cu, out=out,
                                workspace=ws, stream=type("S", (), {"cuda_stream": 0}))
     assert e.value.status == -1
+
+
+def test_binding_passes_on_what_a_truth_value_raises(lib):
+    import numpy as np
+    import torch
+    K = torch.zeros((2, 64, 128), dtype=torch.bfloat16)
+    p = binding.Params(kv_heads=2, gqa_ratio=1, window=16, budget=32)
+    with pytest.raises(ValueError):     # the truth value of an array is ambiguous
+        binding.scores(K, K, torch.zeros((1, 2, 16, 128), dtype=torch.bfloat16), p, want_parts=np.ones(2))
