@@ -479,6 +479,8 @@ PyObject* py_similarity_map(PyObject*, PyObject* const* a, Py_ssize_t n) {
       fail(PyExc_AssertionError, "X must be a contiguous bf16 tensor");
     const long block = PyLong_AsLong(a[1]);
     if (block == -1 && PyErr_Occurred()) throw Raised();
+    // (the library would see its lower 32 bits, and another number of cells than the map has)
+    if (block != (int32_t)block) check_status(MIXKV_ERR_INVALID_ARG, "mixkv_similarity_map");
     const int heads = (int)X.size(0), L = (int)X.size(1);
     size_t need = 0;
     check_status(api.sim_ws_size(heads, L, (int)block, &need), "mixkv_similarity_workspace_size");

@@ -122,3 +122,11 @@ def test_binding_passes_on_what_a_truth_value_raises(lib):
     p = binding.Params(kv_heads=2, gqa_ratio=1, window=16, budget=32)
     with pytest.raises(ValueError):     # the truth value of an array is ambiguous
         binding.scores(K, K, torch.zeros((1, 2, 16, 128), dtype=torch.bfloat16), p, want_parts=np.ones(2))
+
+
+@pytest.mark.parametrize("block", [0, -3, 1 << 31, (1 << 32) + 16])
+def test_binding_refuses_block_sizes_the_library_cannot_take(lib, block):
+    import torch
+    with pytest.raises(binding.MixKVError) as e:
+        binding.similarity_map(torch.zeros((1, 64, 128), dtype=torch.bfloat16), block)
+    assert e.value.status == -1
