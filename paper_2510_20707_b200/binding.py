@@ -1,12 +1,16 @@
 """Python binding of the MixKV C ABI (``include/mixkv.h``).
 
 Argument marshalling only: every function hands device pointers of torch tensors to the
-library entry point of the same name and returns the tensors it filled.  No arithmetic of
-the method happens here, and nothing falls back to PyTorch ops or the CPU: if
-``libmixkv.so`` or ``_mixkv_host.so`` is missing, :func:`load_library` raises.
+library and returns the tensors it filled.  No arithmetic of the method happens here, and
+nothing falls back to PyTorch ops or the CPU: if ``libmixkv.so`` is missing,
+:func:`load_library` raises, and so does the first call that enqueues work without
+``_mixkv_host.so``.
 
 The calls that enqueue work go through the native module ``_mixkv_host``
-(``csrc/host/host_binding.cpp``), the rest through ctypes.
+(``csrc/host/host_binding.cpp``), the rest through ctypes, each to the entry point of the same
+name but for :func:`scores`, :func:`scores_static` and :func:`select`, which take the variants of
+``csrc/internal_api.h`` (the call itself clears the status word it hands out), and
+:func:`compress_layer`, which is ``mixkv_compress_layer_traced`` with no events.
 """
 from __future__ import annotations
 

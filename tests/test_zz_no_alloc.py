@@ -3,7 +3,7 @@
 Some users of the library cannot hand it a workspace: an engine that gave all free HBM to
 its own KV pool at start-up, a plug-in inside another program's step loop where cudaMalloc
 would stall the device, a binding without an allocator.  For them the library carries a
-fixed scratch array of its own.  This file checks, through the C ABI, that scoring with that
+fixed scratch array of its own.  This file checks, through the binding, that scoring with that
 built-in scratch gives bit for bit what scoring with a caller workspace gives (the same
 kernels run in the same order, only the scratch address differs) and agrees with the CPU
 oracle, on two calls in a row (the second on a different, shorter problem, so stale contents
