@@ -235,16 +235,6 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   float* sks = reinterpret_cast<float*>(sK + kP1Stages * kTileBytes);  // [aux warps][128] key-sum exchange
   float2* sxs = reinterpret_cast<float2*>(sks + kP1AuxWarps * 128);    // [kP1XRows] row statistics handed over
   P1Bars* bars = reinterpret_cast<P1Bars*>(sxs + kP1XRows);
-  {
-    // the carve-up above must fit behind the (1 KB aligned) base
-    unsigned dyn;
-    asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
-    if ((size_t)(reinterpret_cast<unsigned char*>(bars + 1) - smem_dyn) > dyn) {
-      if (threadIdx.x == 0 && status) atomicExch(status, MIXKV_ERR_CUDA);
-      return;
-    }
-  }
-
   const int lo = cta_first_tile(blockIdx.x, split1(st));
   const int hi = cta_first_tile(blockIdx.x + 1, split1(st));
   volatile int* abort = &bars->abort;
@@ -1055,18 +1045,28 @@ bool map_q(const LaunchCtx& c, const void* Q, CUtensorMap* tm) {
              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-size_t pass1_smem(int MB, int NQ) {
-  // up to 1023 bytes of alignment slack in front of the carve-up; never beyond the limit (the
-  // kernel checks that its carve-up fits behind the aligned base)
-  const size_t need = (size_t)2 * NQ * 128 + (size_t)p1_stages(NQ) * kTileBytes + kP1AuxWarps * 128 * 4 +
-                      kP1XRows * 8 + sizeof(P1Bars);
-  const size_t want = need + 1024;
-  return want < kSmemLimit ? want : kSmemLimit;
+// Dynamic shared memory of the passes: what the kernels carve up, behind up to 1023 bytes that align its start.
+constexpr size_t pass1_smem(int NQ) {
+  return 1024 + (size_t)2 * NQ * 128 + (size_t)p1_stages(NQ) * kTileBytes + kP1AuxWarps * 128 * 4 +
+         kP1XRows * 8 + sizeof(P1Bars);
 }
-size_t pass2_smem(int NQ, int vstages) {
+constexpr size_t pass2_smem(int NQ, int vstages) {
   return 1024 + (size_t)2 * (NQ + kExtraRows) * 128 + kP2KStages * kTileBytes +
          (size_t)vstages * kVSubBytes + 1024 * 4 + 64 * 4 + sizeof(P2Bars) + 64;
 }
+// V stages: the two pairs of value-norm warps need one each.
+constexpr int pass2_vstages(int NQ) {
+  int n = kP2VStagesMax;
+  while (n > 2 && pass2_smem(NQ, n) > kSmemLimit) --n;
+  return n;
+}
+constexpr bool passes_fit() {
+  for (int NQ = 16; NQ <= kMaxNQ; NQ += 16)
+    if (pass1_smem(NQ) > kSmemLimit || pass2_smem(NQ, pass2_vstages(NQ)) > kSmemLimit || p1_stages(NQ) > kP1MaxStages)
+      return false;
+  return true;
+}
+static_assert(passes_fit(), "a pass asks for more shared memory than a CTA may have at some width of the query tile");
 
 // cudaFuncSetAttribute once per (kernel, device).
 template <typename F>
@@ -1116,13 +1116,13 @@ cudaError_t launch_pass1(const LaunchCtx& c, const void* K, const void* Q, int* 
   if (!map_kv(c, K, kTile, &tmK) || !map_q(c, Q, &tmQ)) return cudaErrorInvalidValue;
   static bool done1[64] = {false}, done2[64] = {false};
   if (c.st.NQ <= 128) {
-    const size_t smem = pass1_smem(1, c.st.NQ);
+    const size_t smem = pass1_smem(c.st.NQ);
     cudaError_t e = ensure_smem(k_pass1<1>, kSmemLimit, done1);
     if (e != cudaSuccess) return e;
     return launch_pdl(k_pass1<1>, dim3(c.st.g1), dim3(kP1Threads), smem, c.stream, 1, tmK, tmQ, c.st,
                       c.ws, c.scale_log2e, (int)c.clear_status, status);
   }
-  const size_t smem = pass1_smem(2, c.st.NQ);
+  const size_t smem = pass1_smem(c.st.NQ);
   cudaError_t e = ensure_smem(k_pass1<2>, kSmemLimit, done2);
   if (e != cudaSuccess) return e;
   return launch_pdl(k_pass1<2>, dim3(c.st.g1), dim3(kP1Threads), smem, c.stream, 1, tmK, tmQ, c.st,
@@ -1151,8 +1151,7 @@ cudaError_t launch_pass2(const LaunchCtx& c, const void* K, const void* V, const
   const void* Vsrc = c.p.use_vnorm == MIXKV_INTRINSIC_VNORM ? V : K;   // the V map is never used without VNorm
   if (!map_kv(c, K, kTile, &tmK) || !map_kv(c, Vsrc, 64, &tmV) || !map_q(c, Q, &tmQ))
     return cudaErrorInvalidValue;
-  int vstages = kP2VStagesMax;
-  while (vstages > 2 && pass2_smem(c.st.NQ, vstages) > kSmemLimit) --vstages;
+  const int vstages = pass2_vstages(c.st.NQ);
   const P2Maps m{tmK, tmV, tmQ};
   switch ((c.st.NQ / 16 + 1) / 2) {   // pieces of 16 columns per epilogue warp
     case 1: return launch_pass2_t<1>(c, m, s_div_out, rbar_out, vstages, status);
