@@ -144,6 +144,10 @@ def _host():
         if not os.path.exists(HOST_PATH):
             raise FileNotFoundError(
                 f"{HOST_PATH} not found: build it with `python -m paper_2510_20707_b200.build`")
+        from . import build
+        if not build.host_matches(HOST_PATH):
+            raise ImportError(f"{HOST_PATH} was built for another torch or Python: build it again with "
+                              "`python -m paper_2510_20707_b200.build`")
         loader = importlib.machinery.ExtensionFileLoader("_mixkv_host", HOST_PATH)
         spec = importlib.util.spec_from_file_location("_mixkv_host", HOST_PATH, loader=loader)
         module = importlib.util.module_from_spec(spec)

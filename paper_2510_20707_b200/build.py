@@ -3,6 +3,8 @@ half of the Python binding, the host compiler against torch's headers)."""
 from __future__ import annotations
 
 import glob
+import hashlib
+import importlib.util
 import os
 import subprocess
 import sysconfig
@@ -38,19 +40,37 @@ def is_stale() -> bool:
     return _older(LIB, sources() + _headers())
 
 
+def _torch_root() -> str:
+    return os.path.dirname(importlib.util.find_spec("torch").origin)   # (found, not imported)
+
+
+def host_tag() -> str:
+    """What _mixkv_host.so is bound to: this torch build's C++ interface and this Python's ABI.  The module
+    carries it as a string."""
+    with open(os.path.join(_torch_root(), "version.py"), "rb") as f:
+        torch_build = hashlib.sha256(f.read()).hexdigest()[:16]
+    return f"mixkv-host torch-{torch_build} {sysconfig.get_config_var('SOABI')}"
+
+
+def host_matches(path: str = HOST_LIB) -> bool:
+    """Whether the module was built for the torch and the Python in use (loading another one may crash)."""
+    with open(path, "rb") as f:
+        return host_tag().encode() + b"\0" in f.read()
+
+
 def host_is_stale() -> bool:
     return _older(HOST_LIB, [HOST_SRC, os.path.join(CSRC, "internal_api.h"),
-                             os.path.join(INCLUDE, "mixkv.h")])
+                             os.path.join(INCLUDE, "mixkv.h")]) or not host_matches()
 
 
 def _host_command(out: str):
     import torch
-    root = os.path.dirname(torch.__file__)
+    root = _torch_root()
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     inc = [INCLUDE, os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
            os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
     return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
-            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DMIXKV_HOST_TAG="{host_tag()}"',
             *[f"-I{d}" for d in inc], "-o", out, HOST_SRC, f"-L{os.path.join(root, 'lib')}",
             "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-lc10", "-lc10_cuda", "-ldl"]
 

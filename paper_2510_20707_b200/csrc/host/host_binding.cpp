@@ -25,6 +25,9 @@
 #include "../internal_api.h"
 #include "mixkv.h"
 
+// What this module was compiled against (build.py looks for the string in the file).
+extern "C" __attribute__((used)) const char mixkv_host_tag[] = MIXKV_HOST_TAG;
+
 namespace {
 
 // ---- the library and what comes from Python at start-up

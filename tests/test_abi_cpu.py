@@ -130,3 +130,14 @@ def test_binding_refuses_block_sizes_the_library_cannot_take(lib, block):
     with pytest.raises(binding.MixKVError) as e:
         binding.similarity_map(torch.zeros((1, 64, 128), dtype=torch.bfloat16), block)
     assert e.value.status == -1
+
+
+def test_native_binding_is_rebuilt_for_another_torch(lib, monkeypatch):
+    # the module is compiled against torch's C++ interface: a file newer than its sources does not show that
+    assert build.host_matches() and not build.host_is_stale()
+    tag = build.host_tag()
+    monkeypatch.setattr(build, "host_tag", lambda: tag.replace("torch-", "torch-x"))
+    assert build.host_is_stale()
+    monkeypatch.setattr(binding, "_host_module", None)
+    with pytest.raises(ImportError):
+        binding._host()
