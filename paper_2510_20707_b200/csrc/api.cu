@@ -2,7 +2,6 @@
 #include <math.h>
 #include <string.h>
 
-#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -14,17 +13,17 @@ namespace mixkv {
 // UNSUPPORTED; CUDA when the device cannot be queried.  Looked up once per device.
 int classify_cc(int major) { return major == 10 ? MIXKV_OK : MIXKV_ERR_UNSUPPORTED; }
 int device_check(int* major_out) {
-  static std::atomic<int> cached[64];   // 0 = unknown, else major + 1
+  static std::atomic<int> cached[kMaxDevices];   // 0 = unknown, else major + 1
   int dev = 0;
   if (major_out) *major_out = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return MIXKV_ERR_CUDA;
   int major = 0;
-  if (dev >= 0 && dev < 64 && cached[dev].load(std::memory_order_relaxed) != 0) {
+  if (dev >= 0 && dev < kMaxDevices && cached[dev].load(std::memory_order_relaxed) != 0) {
     major = cached[dev].load(std::memory_order_relaxed) - 1;
   } else {
     if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess)
       return MIXKV_ERR_CUDA;
-    if (dev >= 0 && dev < 64) cached[dev].store(major + 1, std::memory_order_relaxed);
+    if (dev >= 0 && dev < kMaxDevices) cached[dev].store(major + 1, std::memory_order_relaxed);
   }
   if (major_out) *major_out = major;
   return classify_cc(major);
@@ -502,7 +501,6 @@ int mixkv_compress_layer(const void* K, const void* V, const void* Qwin,
 static __device__ __align__(256) unsigned char g_static_scratch[MIXKV_STATIC_SCRATCH_BYTES];
 
 namespace {
-constexpr int kMaxDevices = 64;
 std::mutex g_scratch_mutex;
 void* g_scratch_addr[kMaxDevices] = {nullptr};
 

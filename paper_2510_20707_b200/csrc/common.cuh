@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "mixkv.h"
 
 namespace mixkv {
@@ -93,7 +95,21 @@ struct LaunchCtx {
 cudaError_t launch_pass1(const LaunchCtx& c, const void* K, const void* Q, int* status);
 cudaError_t launch_pass2(const LaunchCtx& c, const void* K, const void* V, const void* Q,
                          float* s_div_out, float* rbar_out, int* status);
+constexpr int kMaxDevices = 64;   // what is looked up or set once per device is remembered for so many
 int device_sm_count();
+// Lets `kernel` have `smem` bytes of dynamic shared memory on the current device, once per device; `done` is the
+// kernel's own array (static: entry points may run in several threads at once).
+template <typename F>
+cudaError_t ensure_smem(F kernel, size_t smem, std::atomic<bool> (&done)[kMaxDevices]) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const bool known = dev >= 0 && dev < kMaxDevices;
+  if (known && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess && known) done[dev].store(true, std::memory_order_release);
+  return e;
+}
 // Fills a CUtensorMap (passed as void*) for a bf16 tensor of the given rank: dims innermost first,
 // strides in bytes of dimensions 1 .. rank-1, box extents; 128-byte swizzle, zero fill outside.
 bool encode_bf16_map(void* tm, const void* base, int rank, const unsigned long long* dims,

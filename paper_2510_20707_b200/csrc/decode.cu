@@ -461,19 +461,11 @@ extern "C" int mixkv_decode_attention(const void* K_cache, const void* V_cache,
   auto kernel = alone  ? (wide ? k_decode_attention<true, kDecDepthAlone> : k_decode_attention<false, kDecDepthAlone>)
                 : pair ? (wide ? k_decode_attention<true, kDecDepthPair> : k_decode_attention<false, kDecDepthPair>)
                        : (wide ? k_decode_attention<true, kDecDepth> : k_decode_attention<false, kDecDepth>);
-  if (smem > 48 * 1024) {
-    static bool done[6][64] = {};
-    const int variant = 2 * (depth - kDecDepth) + wide;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return MIXKV_ERR_CUDA;
-    if (dev < 0 || dev >= 64 || !done[variant][dev]) {
-      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return MIXKV_ERR_CUDA;
-      if (dev >= 0 && dev < 64) done[variant][dev] = true;
-    }
-  }
-  const cudaError_t e = launch_pdl(kernel, dim3((unsigned)(units * S)), dim3(kDecThreads), smem, (cudaStream_t)stream, S,
-                                   K, V, out_row_offsets, (long long)rows_cap, qq, batch * kv_heads, kv_heads,
-                                   gqa_ratio, scale * kLog2e, max_rows, out);
+  static std::atomic<bool> done[6][kMaxDevices];
+  cudaError_t e = ensure_smem(kernel, smem, done[2 * (depth - kDecDepth) + wide]);
+  if (e != cudaSuccess) return MIXKV_ERR_CUDA;
+  e = launch_pdl(kernel, dim3((unsigned)(units * S)), dim3(kDecThreads), smem, (cudaStream_t)stream, S, K, V,
+                 out_row_offsets, (long long)rows_cap, qq, batch * kv_heads, kv_heads, gqa_ratio, scale * kLog2e,
+                 max_rows, out);
   return e == cudaSuccess ? MIXKV_OK : MIXKV_ERR_CUDA;
 }

@@ -1068,20 +1068,6 @@ constexpr bool passes_fit() {
 }
 static_assert(passes_fit(), "a pass asks for more shared memory than a CTA may have at some width of the query tile");
 
-// cudaFuncSetAttribute once per (kernel, device).
-template <typename F>
-cudaError_t ensure_smem(F kernel, size_t smem, bool (&done)[64]) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || !done[dev]) {
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) done[dev] = true;
-  }
-  return cudaSuccess;
-}
-
 }  // namespace
 
 bool encode_bf16_map(void* tm, const void* base, int rank, const unsigned long long* dims,
@@ -1099,22 +1085,22 @@ bool encode_bf16_map(void* tm, const void* base, int rank, const unsigned long l
 }
 
 int device_sm_count() {
-  static int cached[64] = {0};
+  static std::atomic<int> cached[kMaxDevices];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-  if (cached[dev] == 0) {
-    int n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 148;
+  int n = cached[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
       n = 148;
-    cached[dev] = n;
+    cached[dev].store(n, std::memory_order_relaxed);
   }
-  return cached[dev];
+  return n;
 }
 
 cudaError_t launch_pass1(const LaunchCtx& c, const void* K, const void* Q, int* status) {
   CUtensorMap tmK, tmQ;
   if (!map_kv(c, K, kTile, &tmK) || !map_q(c, Q, &tmQ)) return cudaErrorInvalidValue;
-  static bool done1[64] = {false}, done2[64] = {false};
+  static std::atomic<bool> done1[kMaxDevices], done2[kMaxDevices];
   if (c.st.NQ <= 128) {
     const size_t smem = pass1_smem(c.st.NQ);
     cudaError_t e = ensure_smem(k_pass1<1>, kSmemLimit, done1);
@@ -1136,7 +1122,7 @@ struct P2Maps {
 template <int NCH>
 cudaError_t launch_pass2_t(const LaunchCtx& c, const P2Maps& m, float* s_div_out, float* rbar_out, int vstages,
                            int* status) {
-  static bool done[64] = {false};
+  static std::atomic<bool> done[kMaxDevices];
   cudaError_t e = ensure_smem(k_pass2<NCH>, kSmemLimit, done);
   if (e != cudaSuccess) return e;
   return launch_pdl(k_pass2<NCH>, dim3(c.st.g2), dim3(kP2Threads), pass2_smem(c.st.NQ, vstages), c.stream, 1, m.K, m.V,

@@ -349,17 +349,11 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
 
 template <int P, int NT>
 cudaError_t launch_gram_t(const GramArgs& g, const long long per_head, cudaStream_t s) {
-  static bool done[64] = {false};
+  static std::atomic<bool> done[kMaxDevices];
   const size_t smem = 1024 + (size_t)P * kPartBytes + (size_t)kGStages * NT * 128 +
                       (size_t)kGEpiWarps * 4096 + sizeof(GBars);
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  const cudaError_t e = ensure_smem(k_gram<P, NT>, smem, done);
   if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64 || !done[dev]) {
-    e = cudaFuncSetAttribute(k_gram<P, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) done[dev] = true;
-  }
   const long long total = per_head * g.heads;
   if (total > 0x7fffffffLL) return cudaErrorInvalidValue;
   CUtensorMap tmA, tmB;

@@ -1053,16 +1053,9 @@ cudaError_t launch_budget(const LaunchCtx& c, const float* scores, int* counts) 
   const size_t cap_bytes = 200 * 1024;
   const size_t smem = want <= cap_bytes ? want : 0;
   if (smem > 24 * 1024) {   // on top of the search's static shared memory
-    static bool done[64] = {false};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    static std::atomic<bool> done[kMaxDevices];
+    const cudaError_t e = ensure_smem(k_budget, cap_bytes, done);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64 || !done[dev]) {
-      e = cudaFuncSetAttribute(k_budget, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)cap_bytes);
-      if (e != cudaSuccess) return e;
-      if (dev >= 0 && dev < 64) done[dev] = true;
-    }
   }
   return launch_pdl(k_budget, dim3(c.st.batch * cs, c.st.layers), dim3(kBudgetThreads), smem, c.stream, cs,
                     c.st, scores, counts, c.p.budget - c.p.window, floor_slots(c.p), (int)(smem / 4));
@@ -1109,16 +1102,10 @@ bool tail_can_fuse(const LaunchCtx& c) { return tail_shape(c).cached; }
 template <bool FUSED, int T, bool CL>
 cudaError_t launch_tail_t(const LaunchCtx& c, const TailKernelArgs& a, const TailShape& sh,
                           size_t smem) {
-  static size_t have[64] = {0};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (smem > 20 * 1024 && (dev < 0 || dev >= 64 || have[dev] < smem)) {   // on top of the static part
-    const size_t ask = 203 * 1024;
-    e = cudaFuncSetAttribute(k_tail<FUSED, T, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)ask);
+  if (smem > 20 * 1024) {   // on top of the static part
+    static std::atomic<bool> done[kMaxDevices];
+    const cudaError_t e = ensure_smem(k_tail<FUSED, T, CL>, 203 * 1024, done);
     if (e != cudaSuccess) return e;
-    if (dev >= 0 && dev < 64) have[dev] = ask;
   }
   const dim3 grid(c.st.layers * c.st.batch * c.st.H * sh.cs);
   return launch_pdl(k_tail<FUSED, T, CL>, grid, dim3(T), smem, c.stream, sh.cs, c.st, c.ws, a);

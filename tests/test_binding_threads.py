@@ -4,6 +4,7 @@ whose entry points wait until another Python thread lets them go (two seconds at
 import os
 import subprocess
 import sys
+import threading
 
 import pytest
 
@@ -96,3 +97,50 @@ def test_other_threads_run_while_a_call_is_in_the_library(device, n, tmp_path):
     r = subprocess.run([sys.executable, "-c", PROGRAM, device, str(lib)], cwd=ROOT, capture_output=True, text=True,
                        timeout=300)
     assert r.returncode == 0 and r.stdout.strip() == f"ok {n}", r.stdout + r.stderr
+
+
+@pytest.mark.gpu
+def test_calls_from_several_threads():
+    # four threads with a stream and a workspace each, through one-layer, adaptive, decode and map calls at the same
+    # time (what the library keeps per device is shared): every result has the bits of a call made alone
+    import torch
+    from paper_2510_20707_b200 import binding
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    rand = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
+    K, V, Q = rand(4, 3000, 128), rand(4, 3000, 128), rand(1, 16, 32, 128)
+    cache, q = rand(1, 4 * 300, 128), rand(1, 1, 16, 128)
+    offs = (torch.arange(5, dtype=torch.int32, device="cuda") * 300).view(1, 5)
+    params = [binding.Params(kv_heads=4, gqa_ratio=4, budget=128, budget_mode=m) for m in (0, 1)]
+    size = max(binding.workspace_size(p, 1, 3000, 3000) for p in params)
+
+    def work(ws):
+        out = [binding.compress_layer(K, V, Q, p, workspace=ws) for p in params]
+        res = [o[k] for o in out for k in ("s_comp", "idx_offsets", "out_row_offsets")]
+        res += [o["idx"][:4 * 96] for o in out] + [out[0]["K_out"], out[0]["V_out"]]
+        s = binding.scores(K, V, Q, params[0], workspace=ws)
+        return res + [s["s_comp"], binding.select(s["s_comp"], params[0], workspace=ws)["idx"],
+                      binding.decode_attention(cache, cache, offs, q, 4, 4, 300), *binding.similarity_map(K, 16)]
+
+    new = lambda: torch.empty(size, dtype=torch.uint8, device="cuda")
+    ref = work(new())
+    torch.cuda.synchronize()
+    found = []
+
+    def thread():
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                ws = new()
+                for _ in range(20):
+                    got = work(ws)
+                    stream.synchronize()
+                    found.append(all(torch.equal(a, b) for a, b in zip(got, ref, strict=True)))
+        except Exception as e:      # (a thread's exception would not fail the test)
+            found.append(e)
+
+    threads = [threading.Thread(target=thread) for _ in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert found == [True] * 80, found
