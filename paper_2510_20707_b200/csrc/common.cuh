@@ -19,6 +19,7 @@ constexpr int kMaxNQ = 240;          // G*W upper bound (16 spare rows carry the
 constexpr int kTile = 128;           // keys per tensor-core tile
 constexpr int kPChunk = 2048;        // candidate positions per CTA in pool / mix
 constexpr int kExtraRows = 16;       // rows appended to the query tile in pass 2
+constexpr int kMaxCluster = 8;       // CTAs of a cluster (the portable limit)
 constexpr float kLog2e = 1.4426950408889634f;
 
 // Everything a kernel needs to find its slice of the ragged batch.
@@ -97,19 +98,45 @@ cudaError_t launch_pass2(const LaunchCtx& c, const void* K, const void* V, const
                          float* s_div_out, float* rbar_out, int* status);
 constexpr int kMaxDevices = 64;   // what is looked up or set once per device is remembered for so many
 int device_sm_count();
+// The current device as an index into what is remembered per device; -1: none, or one past the end.
+inline int device_slot() {
+  int dev = -1;
+  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices ? dev : -1;
+}
 // Lets `kernel` have `smem` bytes of dynamic shared memory on the current device, once per device; `done` is the
 // kernel's own array (static: entry points may run in several threads at once).
 template <typename F>
-cudaError_t ensure_smem(F kernel, size_t smem, std::atomic<bool> (&done)[kMaxDevices]) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const bool known = dev >= 0 && dev < kMaxDevices;
-  if (known && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess && known) done[dev].store(true, std::memory_order_release);
+cudaError_t ensure_smem(F kernel, size_t smem, std::atomic<bool> (&done)[kMaxDevices], const int dev = device_slot()) {
+  if (dev >= 0 && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess && dev >= 0) done[dev].store(true, std::memory_order_release);
   return e;
 }
+// Clusters of 1 .. 8 CTAs of one kernel that the current device holds at once.  A cluster lies in one group of SMs, and
+// how the SMs of a chip fall into groups differs between chips of one model, so the runtime is asked, once per device
+// and size (0.2 us a question); `kernel` may already have its shared memory.  Without a device: as if SMs were all alike.
+struct ClusterFit {
+  std::atomic<int> known[kMaxDevices][kMaxCluster + 1];   // 0: not asked, else the answer + 1
+  template <typename F>
+  int ask(F kernel, int threads, size_t smem, int size, const int dev = device_slot()) {
+    if (dev >= 0)
+      if (const int k = known[dev][size].load(std::memory_order_relaxed)) return k - 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)size);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)size;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) return device_sm_count() / size;
+    if (dev >= 0) known[dev][size].store(n + 1, std::memory_order_relaxed);
+    return n;
+  }
+};
 // Fills a CUtensorMap (passed as void*) for a bf16 tensor of the given rank: dims innermost first,
 // strides in bytes of dimensions 1 .. rank-1, box extents; 128-byte swizzle, zero fill outside.
 bool encode_bf16_map(void* tm, const void* base, int rank, const unsigned long long* dims,
@@ -121,9 +148,6 @@ cudaError_t launch_poolsum(const LaunchCtx& c);
 cudaError_t launch_mixpool(const LaunchCtx& c, const float* s_div, const float* rbar_in,
                            float* s_ex_out, float* s_comp);
 cudaError_t launch_budget(const LaunchCtx& c, const float* scores, int* counts);
-// Selection (and optionally the mix before it and the gather after it) by one CTA cluster per
-// (sequence, head).  scores != nullptr: select on them; else mix first (s_div, rbar_in) and
-// write the mixed scores to s_comp_out.  counts_dev == nullptr: fixed budgets.
 // Index of (layer, head h, sequence b, position i) in a [layers, H, Ltot] / [layers, H, Ptot]
 // array.
 __host__ __device__ __forceinline__ size_t kpos(const SeqTable& st, int layer, int h, int b,
@@ -148,6 +172,9 @@ struct GramArgs {
 };
 cudaError_t launch_gram(const GramArgs& g, cudaStream_t s);
 
+// Selection (and optionally the mix before it and the gather after it), one CTA or cluster per
+// (layer, sequence, head).  scores != nullptr: select on them; else mix first (s_div, rbar_in) and
+// write the mixed scores to s_comp_out.  counts_dev == nullptr: fixed budgets.
 struct TailArgs {
   const float* scores;
   const float* s_div;

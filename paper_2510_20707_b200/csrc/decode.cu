@@ -31,6 +31,7 @@
 // slice of the outputs.  Every row is read once.
 #include <cooperative_groups.h>
 
+#include "internal_api.h"
 #include "tc_common.cuh"
 
 namespace cg = cooperative_groups;
@@ -386,11 +387,70 @@ k_decode_attention(const __nv_bfloat16* __restrict__ Kc, const __nv_bfloat16* __
   cluster.sync();   // a CTA's shared memory stays alive until its peers have read it
 }
 
+using DecKernel = void (*)(const __nv_bfloat16*, const __nv_bfloat16*, const int*, long long, const __nv_bfloat16*, int,
+                           int, int, float, int, float*);
+DecKernel dec_kernel(const bool wide, const int depth) {
+  switch (depth) {
+    case kDecDepthAlone: return wide ? k_decode_attention<true, kDecDepthAlone> : k_decode_attention<false, kDecDepthAlone>;
+    case kDecDepthPair: return wide ? k_decode_attention<true, kDecDepthPair> : k_decode_attention<false, kDecDepthPair>;
+    default: return wide ? k_decode_attention<true, kDecDepth> : k_decode_attention<false, kDecDepth>;
+  }
+}
+
+// CTAs per unit and depth of their rings.  shared(n) and alone(n): clusters of n CTAs that are resident at once with
+// three CTAs to an SM and with one; even: the cache has room for max_rows rows of every head, so they may be of one length.
+struct DecodeShape {
+  int S, depth;
+};
+template <typename Shared, typename Alone>
+DecodeShape decode_shape(const long long units, const int max_rows, const bool even, const int sms,
+                         const Shared& shared, const Alone& alone) {
+  // CTAs per unit: as many as still fit the GPU in one wave while every warp keeps a step (one head of 512
+  // rows on 8 CTAs 5.8 us, on 4 6.4; 112 heads of 512 rows on 3 CTAs each 11.5 us, on 2 12.8)
+  const long long slots = (long long)kDecPerSm * sms;
+  const long long steps = ((long long)max_rows + kDecStep - 1) / kDecStep;
+  // One cluster more than are resident at once costs a second wave (48 clusters of eight were, 56 of seven, 71 of
+  // six, 82 of five; units of 1500 rows: 48 on eight CTAs 12.0 us, 49 17.3, on seven 13; 70 on six 15.3, 72 20.7, on
+  // five 16.2).
+  long long most = slots / units < kMaxCluster ? slots / units : kMaxCluster;
+  while (most > 1 && units > shared((int)most)) --most;
+  if (most > steps / kDecWarps) most = steps / kDecWarps;
+  int S = most < 1 ? 1 : (int)most;
+  // One wave and a bit of a second: halves even that out where a warp then still has eight steps (560 ragged heads
+  // of 2500 rows on average 152 -> 130 us, with five steps per warp or a nearly empty second wave nothing)
+  if (units * 10 >= slots * 11 && units * 2 <= slots * 3 && steps >= 2 * kDecWarps * 8) S = 2;
+  // Eight units and more: as long as all clusters are resident with an SM to each CTA, that and the deeper ring.  Where
+  // there is room for three, the CTAs of a cluster end up sharing SMs while others idle (13 units of 3500 rows 15.9 ->
+  // 10.3 us, 20 of them 16.2 -> 13.7, 30 of 1000 9.3 -> 8.5; fewer than eight units gain nothing).
+  // Fewer than eight CTAs only where the heads can be of one length: else the longest head decides, and it wants eight
+  // (28 ragged heads of 2500 rows on average 21.7 us on four CTAs, 17.7 on eight).
+  // One cluster of eight too many: only one group of SMs has to share, and eight CTAs stay ahead of six as long as a
+  // warp has few steps (16 units where 15 fit, six CTAs against eight: 512 rows 6.4 / 6.2 us, 512 of wide heads 11.7 /
+  // 11.2, 3500 12.9 / 12.9, 8000 20.1 / 21.2; 17 units of 1500 rows 8.9 / 10.3).
+  const int eight = units >= 8 ? alone(kMaxCluster) : 0;
+  if (units >= 8 && !(units == eight + 1 && S == kMaxCluster && steps < 8 * kMaxCluster * kDecWarps)) {
+    int x = kMaxCluster;
+    while (x >= (even ? 4 : kMaxCluster) && units > alone(x)) --x;
+    if (x >= (even ? 4 : kMaxCluster) && steps >= kDecWarps * x) return {x, kDecDepthAlone};
+  }
+  // A CTA per unit and no more than two per SM: those two, with the ring of three (with room for a third some SMs
+  // get three and others one: 296 units of 3400 rows 102.8 -> 89.7 us, 280 of 5000 142.6 -> 124.4, 256 of 300
+  // 13.6 -> 12.9; 240 units of 3400 rows 77.1 -> 78.3, of 512 ragged 31.8 -> 29.7).
+  return {S, S == 1 && units > sms && units <= 2LL * sms ? kDecDepthPair : kDecDepth};
+}
 
 }  // namespace
 }  // namespace mixkv
 
 using namespace mixkv;
+
+extern "C" void mixkv_internal_decode_shape(int64_t units, int32_t max_rows, int32_t even, int32_t sms,
+                                            const int32_t* shared, const int32_t* alone, int32_t* ctas,
+                                            int32_t* depth) {
+  const DecodeShape s = decode_shape(units, max_rows, even != 0, sms, [&](const int n) { return shared[n]; },
+                                     [&](const int n) { return alone[n]; });
+  *ctas = s.S, *depth = s.depth;
+}
 
 extern "C" int mixkv_decode_attention(const void* K_cache, const void* V_cache,
                                       const int32_t* out_row_offsets, int64_t rows_cap,
@@ -413,56 +473,27 @@ extern "C" int mixkv_decode_attention(const void* K_cache, const void* V_cache,
   const long long units = (long long)n_layers * batch * kv_heads;
   if (units * 8 > 0x7fffffffLL) return MIXKV_ERR_UNSUPPORTED;
   const bool wide = gqa_ratio > 8;
-  // CTAs per unit: as many as still fit the GPU in one wave while every warp keeps a step (one head of 512
-  // rows on 8 CTAs 5.8 us, on 4 6.4; 112 heads of 512 rows on 3 CTAs each 11.5 us, on 2 12.8)
-  const int sms = device_sm_count();
-  const long long slots = (long long)kDecPerSm * sms;
-  const long long steps = ((long long)max_rows + kDecStep - 1) / kDecStep;
-  // A cluster lies in one group of SMs, so not every place can be taken: at three CTAs per SM 48 clusters of eight
-  // were resident at once, 56 of seven, 70 of six, 82 of five, 104 of four, 142 of three, and one more of any of them
-  // cost a second wave (units of 1500 rows: 48 on eight CTAs 12.0 us, 49 17.3, on seven 13; 70 on six 15.3, 72 20.7, on
-  // five 16.2).
-  const int whole[9] = {0, 0, 222, 142, 104, 82, 70, 56, 48};
-  long long most = slots / units < 8 ? slots / units : 8;
-  while (most > 1 && units * 148 > (long long)whole[most] * sms) --most;
-  if (most > steps / kDecWarps) most = steps / kDecWarps;
-  int S = most < 1 ? 1 : (int)most;
-  // One wave and a bit of a second: halves even that out where a warp then still has eight steps (560 ragged heads
-  // of 2500 rows on average 152 -> 130 us, with five steps per warp or a nearly empty second wave nothing)
-  if (units * 10 >= slots * 11 && units * 2 <= slots * 3 && steps >= 2 * kDecWarps * 8) S = 2;
-  // Eight to 32 units: a CTA has an SM for itself, with the deeper ring.  Where there is room for three, the CTAs
-  // of a cluster end up sharing SMs while others idle (13 units of 3500 rows 15.9 -> 10.3 us, 20 of them 16.2 -> 13.7,
-  // 30 of 1000 9.3 -> 8.5; fewer than eight units gain nothing, and 16 x 8 CTAs spread well as they are: 12.7 us
-  // against 13.0).  The clusters have to be resident all at once, or a second wave doubles the time; a
-  // cluster lies in one group of SMs, and 15 clusters of eight fit, 22 of six, 25 of five and 32 of four.
-  // Fewer than eight CTAs only where the heads can be of one length (the cache holds max_rows rows of every head):
-  // else the longest head decides, and it wants eight (28 ragged heads of 2500 rows on average 21.7 us on four
-  // CTAs, 17.7 on eight).
-  const int fit[9] = {0, 0, 0, 0, 32, 25, 22, 15, 15};
-  const bool even = rows_cap >= (long long)max_rows * batch * kv_heads;
-  bool alone = false;
-  if (units >= 8 && units != 16 && sms >= 148)
-    for (int x = 8; x >= (even ? 4 : 8) && !alone; --x)
-      if (units <= fit[x]) {
-        alone = steps >= kDecWarps * x;
-        if (alone) S = x;
-        break;
-      }
-  // A CTA per unit and no more than two per SM: those two, with the ring of three (with room for a third some SMs
-  // get three and others one: 296 units of 3400 rows 102.8 -> 89.7 us, 280 of 5000 142.6 -> 124.4, 256 of 300
-  // 13.6 -> 12.9; 240 units of 3400 rows 77.1 -> 78.3, of 512 ragged 31.8 -> 29.7).
-  const bool pair = !alone && S == 1 && units > sms && units <= 2LL * sms;
-  const int depth = alone ? kDecDepthAlone : pair ? kDecDepthPair : kDecDepth;
+  static std::atomic<bool> done[6][kMaxDevices];
+  static ClusterFit fit[6];   // (by variant, as `done`)
+  const int dev = device_slot();
+  auto variant = [&](const int depth) { return 2 * (depth - kDecDepth) + wide; };
+  auto resident = [&](const int depth) {
+    return [&, depth](const int size) {
+      const DecKernel k = dec_kernel(wide, depth);
+      if (ensure_smem(k, dec_smem(depth), done[variant(depth)], dev) != cudaSuccess) return 0;
+      return fit[variant(depth)].ask(k, kDecThreads, dec_smem(depth), size, dev);
+    };
+  };
+  const DecodeShape shape = decode_shape(units, max_rows, rows_cap >= (long long)max_rows * batch * kv_heads,
+                                         device_sm_count(), resident(kDecDepth), resident(kDecDepthAlone));
+  const int S = shape.S, depth = shape.depth;
   const size_t smem = dec_smem(depth);
   const float scale = softmax_scale > 0.f ? softmax_scale : 1.0f / sqrtf((float)kHeadDim);
   const __nv_bfloat16 *K = reinterpret_cast<const __nv_bfloat16*>(K_cache),
                       *V = reinterpret_cast<const __nv_bfloat16*>(V_cache),
                       *qq = reinterpret_cast<const __nv_bfloat16*>(q);
-  auto kernel = alone  ? (wide ? k_decode_attention<true, kDecDepthAlone> : k_decode_attention<false, kDecDepthAlone>)
-                : pair ? (wide ? k_decode_attention<true, kDecDepthPair> : k_decode_attention<false, kDecDepthPair>)
-                       : (wide ? k_decode_attention<true, kDecDepth> : k_decode_attention<false, kDecDepth>);
-  static std::atomic<bool> done[6][kMaxDevices];
-  cudaError_t e = ensure_smem(kernel, smem, done[2 * (depth - kDecDepth) + wide]);
+  const DecKernel kernel = dec_kernel(wide, depth);
+  cudaError_t e = ensure_smem(kernel, smem, done[variant(depth)], dev);
   if (e != cudaSuccess) return MIXKV_ERR_CUDA;
   e = launch_pdl(kernel, dim3((unsigned)(units * S)), dim3(kDecThreads), smem, (cudaStream_t)stream, S, K, V,
                  out_row_offsets, (long long)rows_cap, qq, batch * kv_heads, kv_heads, gqa_ratio, scale * kLog2e,

@@ -1,6 +1,4 @@
-// Entry points the Python binding uses beside the public C ABI (include/mixkv.h): the same calls with a
-// status word that the call itself sets to 0 first, so that a binding which hands out a new word per call
-// need not enqueue a fill for it.
+// Entry points beside the public C ABI (include/mixkv.h): two the Python binding uses, and the launch rules for tests.
 #pragma once
 #include <stddef.h>
 #include <stdint.h>
@@ -11,6 +9,9 @@
 extern "C" {
 #endif
 
+// The same calls as the public ones with a status word that the call itself sets to 0 first, so that a binding which
+// hands out a new word per call need not enqueue a fill for it.
+//
 // mixkv_scores (static_scratch == 0) or mixkv_scores_static (workspace ignored).  The word is cleared
 // by the first kernel right after its dependency wait; a kernel reports an expired wait two seconds later
 // at the earliest.
@@ -22,6 +23,14 @@ int mixkv_internal_scores(const void* K, const void* V, const void* Qwin, const 
 int mixkv_internal_select(const float* scores, const int32_t* cu_seqlens_host, int32_t batch, int32_t L,
                           const mixkv_params* p, void* workspace, size_t workspace_bytes, int32_t* idx,
                           int32_t* counts, int32_t* idx_offsets, int32_t* status_dev, void* stream);
+
+// The rules that split the work of a call over clusters, as functions of the sizes and of how many clusters of n CTAs a
+// device holds at once (alone[n] with one CTA per SM, shared[n] with three, n = 1 .. 8).  No device is needed.
+// decode: CTAs per unit and the depth of their rings; tail, budget: CTAs per unit, per (sequence, layer) pair.
+void mixkv_internal_decode_shape(int64_t units, int32_t max_rows, int32_t even, int32_t sms, const int32_t* shared,
+                                 const int32_t* alone, int32_t* ctas, int32_t* depth);
+int mixkv_internal_tail_clusters(int64_t units, int32_t candidates, int32_t sms, const int32_t* alone);
+int mixkv_internal_budget_clusters(int32_t pairs, int64_t keys_per_pair, const int32_t* alone);
 
 #ifdef __cplusplus
 }

@@ -8,6 +8,7 @@
 
 #include <type_traits>
 
+#include "internal_api.h"
 #include "tc_common.cuh"
 
 namespace cg = cooperative_groups;
@@ -307,7 +308,7 @@ __device__ __forceinline__ unsigned order_key(float f) {
 
 constexpr int kSelBinBits = 11, kSelBins = 1 << kSelBinBits;
 constexpr int kSelListCap = 256;   // candidates ranked directly
-constexpr int kSelMaxCluster = 8;
+constexpr int kSelMaxCluster = kMaxCluster;
 
 struct SelSmem {
   int hist[2][kSelBins];
@@ -523,7 +524,7 @@ __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const
   return th;
 }
 
-constexpr int kBudgetCluster = 8;
+constexpr int kBudgetCluster = kMaxCluster;
 constexpr int kBudgetThreads = 1024;
 
 // Head budgets of one sequence under the adaptive rule (see mixkv.h).  One CTA per (sequence,
@@ -645,9 +646,10 @@ __host__ __device__ __forceinline__ int tail_chunk(const int P, const int cs) {
 }
 
 // ------------------------------------------------------------------------------ tail
-constexpr int kTailMaxCluster = 8;
+constexpr int kTailMaxCluster = kMaxCluster;
 constexpr int kTailCacheCap = 40960;       // positions a CTA keeps in shared memory
 constexpr int kTailCacheCapFull = 16384;   // the same in a cluster of eight: few, very long heads go unfused beyond
+constexpr size_t kTailSmem = 203 * 1024;   // dynamic shared memory at most
 constexpr int kTailRowCap = 1024;          // selected rows of a CTA listed in shared memory for the gather
 
 struct TailKernelArgs {
@@ -1036,17 +1038,31 @@ cudaError_t launch_given_budgets(const LaunchCtx& c, const int* budgets, int* co
                     counts, c.p.budget - c.p.window);
 }
 
-cudaError_t launch_budget(const LaunchCtx& c, const float* scores, int* counts) {
-  // CTAs per (sequence, layer) pair: one while it has 8192 keys or less of all heads (the exchanges cost as much as
-  // the sweeps they save), else as many as leave each that much and are all resident at once, one per SM (120 CTAs
-  // in clusters of four or eight ran in one wave, 136 did not).  Whole calls, eight CTAs each up to 17 pairs and one
-  // beyond that against this: 17 pairs of 3000 keys 50.1 / 37.9 us; 17, 20, 28 of 96000 217 / 204, 368 / 238, 439 /
-  // 322 us; 28, 56 of 32000 134 / 122, 227 / 224 us.
-  const int pairs = c.st.batch * c.st.layers;
+namespace {
+// Clusters of `size` CTAs that the device holds at once with an SM to each CTA (k_tail and k_budget with 1024 threads;
+// 120 KB make sure of it).
+int alone_clusters(const int size) {
+  static std::atomic<bool> done[kMaxDevices];
+  static ClusterFit fit;
+  (void)ensure_smem(k_tail<true, 1024, true>, kTailSmem, done);   // (a failure shows at the launch)
+  return fit.ask(k_tail<true, 1024, true>, 1024, 120 * 1024, size);
+}
+
+// CTAs per (sequence, layer) pair: one while it has 8192 keys or less of all heads (the exchanges cost as much as
+// the sweeps they save), else as many as leave each that much and are all resident at once, one per SM (15 clusters of
+// eight are, 33 of four, 74 of two).  Whole calls, eight CTAs each up to 17 pairs and one
+// beyond that against this: 17 pairs of 3000 keys 50.1 / 37.9 us; 17, 20, 28 of 96000 217 / 204, 368 / 238, 439 /
+// 322 us; 28, 56 of 32000 134 / 122, 227 / 224 us.
+template <typename Fit>
+int budget_clusters(const int pairs, const long long keys, const Fit& alone) {
   int cs = 1;
-  while (cs < kBudgetCluster && (long long)c.st.H * c.max_prefix > 8192LL * cs &&
-         pairs * 2 * cs <= device_sm_count() * 13 / 16)
-    cs *= 2;
+  while (cs < kBudgetCluster && keys > 8192LL * cs && pairs <= alone(2 * cs)) cs *= 2;
+  return cs;
+}
+}  // namespace
+
+cudaError_t launch_budget(const LaunchCtx& c, const float* scores, int* counts) {
+  const int cs = budget_clusters(c.st.batch * c.st.layers, (long long)c.st.H * c.max_prefix, alone_clusters);
   const size_t chunk = ((size_t)c.max_prefix + cs - 1) / cs;
   // the keys of a CTA's slice of the longest sequence in shared memory when they fit
   const size_t want = (size_t)c.st.H * ((chunk + 31) / 32) * 128;
@@ -1067,20 +1083,25 @@ struct TailShape {
   bool cached;
 };
 
+// CTAs per unit.  One when there are many units or a unit is a block of positions or less (an exchange across a
+// cluster costs more than another block).  Few long ones: more of them, always so that all clusters are resident at
+// once with an SM to each CTA, and as long as pairs leave an SM over and clusters of four and eight a fifth of them: beyond
+// that the exchange costs more than it saves (selection alone, 74 units of 6000 positions on pairs 10.4 us, on one CTA
+// each 7.0; 31 of 12000 on four 10.1, on two 8.9; 15 of 30000 on eight 12.3, on four 9.9).
+template <typename Fit>
+int tail_clusters(const long long units, const int P, const int sms, const Fit& alone) {
+  int cs = 1;
+  while (cs < kTailMaxCluster && tail_chunk(P, cs) > 4096 && units * 2 * cs <= (cs == 1 ? sms - 1 : sms * 4 / 5) &&
+         units <= alone(2 * cs))
+    cs *= 2;
+  return cs;
+}
+
 TailShape tail_shape(const LaunchCtx& c) {
   const long long units = (long long)c.st.layers * c.st.batch * c.st.H;
   const int P = c.max_prefix, sms = device_sm_count();
   TailShape t;
-  t.cs = 1;
-  // A CTA per unit when there are many units or a unit is a block of positions or less (an exchange across a
-  // cluster costs more than another block).  Few long ones: CTAs as long as all clusters are resident at once
-  // with one CTA per SM.  Pairs fill the chip; clusters of four and eight do not (they have to lie in one group of
-  // SMs, and groups differ in size): up to 112 CTAs of them ran in one wave, 128 did not (16 units of 32000
-  // positions: eight CTAs each 87 us, four 74; 48 units of 12000: eight 121, four 90, two 80).
-  if (units < sms / 2)
-    while (t.cs < kTailMaxCluster && tail_chunk(P, t.cs) > 4096 &&
-           units * 2 * t.cs <= (t.cs == 1 ? sms : sms * 4 / 5))
-      t.cs *= 2;
+  t.cs = tail_clusters(units, P, sms, alone_clusters);
   // What does not fit shared memory in that many CTAs takes more of them.
   while (t.cs < kTailMaxCluster && tail_chunk(P, t.cs) > kTailCacheCap) t.cs *= 2;
   t.chunk = tail_chunk(P, t.cs);
@@ -1104,7 +1125,7 @@ cudaError_t launch_tail_t(const LaunchCtx& c, const TailKernelArgs& a, const Tai
                           size_t smem) {
   if (smem > 20 * 1024) {   // on top of the static part
     static std::atomic<bool> done[kMaxDevices];
-    const cudaError_t e = ensure_smem(k_tail<FUSED, T, CL>, 203 * 1024, done);
+    const cudaError_t e = ensure_smem(k_tail<FUSED, T, CL>, kTailSmem, done);
     if (e != cudaSuccess) return e;
   }
   const dim3 grid(c.st.layers * c.st.batch * c.st.H * sh.cs);
@@ -1153,3 +1174,10 @@ cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
 }
 
 }  // namespace mixkv
+
+extern "C" int mixkv_internal_tail_clusters(int64_t units, int32_t candidates, int32_t sms, const int32_t* alone) {
+  return mixkv::tail_clusters(units, candidates, sms, [&](const int n) { return alone[n]; });
+}
+extern "C" int mixkv_internal_budget_clusters(int32_t pairs, int64_t keys_per_pair, const int32_t* alone) {
+  return mixkv::budget_clusters(pairs, keys_per_pair, [&](const int n) { return alone[n]; });
+}

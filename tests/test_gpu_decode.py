@@ -150,6 +150,27 @@ def test_repeated_calls_are_bit_identical():
         assert torch.equal(first, again)
 
 
+def test_capture_of_shapes_that_did_not_run_before():
+    # a call outside capture is asked for once per entry point: what another shape needs (its kernel's shared memory,
+    # the clusters a device holds) may be looked up while a capture is going on
+    def problem(units, rows, G):
+        offs = (torch.arange(units + 1, dtype=torch.int32, device="cuda") * rows).view(1, -1)
+        gen = torch.Generator(device="cuda").manual_seed(units)
+        K, V = (torch.randn((1, units * rows, 128), generator=gen, device="cuda").bfloat16() for _ in range(2))
+        q = torch.randn((1, units, G, 128), generator=gen, device="cuda").bfloat16()
+        return K, V, offs, q, 1, G, rows
+    binding.decode_attention(*problem(4, 100, 4))
+    for units, rows, G in ((20, 700, 4), (20, 700, 12), (48, 600, 9), (250, 200, 4), (296, 2100, 3), (250, 200, 11)):
+        x = problem(units, rows, G)
+        graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.graph(graph, stream=side):
+            out = binding.decode_attention(*x)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(out, binding.decode_attention(*x)), (units, rows, G)
+
+
 def test_empty_head_short_rows_and_bad_arguments():
     H, G = 2, 2
     rng = np.random.default_rng(3)

@@ -1,0 +1,66 @@
+"""The rules that split a call's work over clusters of CTAs (csrc/internal_api.h), without a device: whatever number
+of clusters a device holds at once, no rule asks for more, which would cost a second wave."""
+import ctypes as C
+
+import pytest
+
+from paper_2510_20707_b200 import binding, build
+
+# resident clusters of 1 .. 8 CTAs with one CTA per SM and with three: a B200 with 148 SMs, then chips whose SMs fall
+# into other groups, and one with fewer of them
+B200 = (148, (148, 74, 45, 33, 26, 22, 15, 15), (444, 222, 142, 104, 82, 71, 56, 48))
+CHIPS = [B200, (148, (148, 70, 40, 28, 22, 18, 12, 11), (444, 210, 130, 90, 70, 60, 45, 40)),
+         (132, (132, 66, 40, 30, 22, 20, 15, 14), (396, 198, 126, 93, 72, 62, 50, 42)),
+         (64, (64, 32, 20, 16, 10, 8, 8, 4), (192, 96, 60, 48, 34, 28, 24, 16))]
+
+
+@pytest.fixture(scope="module")
+def lib():
+    build.build()
+    return binding.load_library()
+
+
+def array(limits):
+    return (C.c_int32 * 9)(0, *limits)
+
+
+def decode(lib, chip, units, rows, even=1):
+    sms, alone, shared = chip
+    ctas, depth = C.c_int32(), C.c_int32()
+    lib.mixkv_internal_decode_shape(C.c_int64(units), rows, even, sms, array(shared), array(alone), C.byref(ctas),
+                                    C.byref(depth))
+    return ctas.value, depth.value
+
+
+@pytest.mark.parametrize("chip", CHIPS)
+def test_no_more_clusters_than_are_resident(lib, chip):
+    sms, alone, shared = chip
+    for units in list(range(1, 700)) + [896, 1184, 5000]:
+        for rows in (1, 17, 300, 512, 1500, 3500, 20000):
+            for even in (0, 1):
+                S, depth = decode(lib, chip, units, rows, even)
+                assert 1 <= S <= 8 and depth in (2, 3, 4)
+                halves = S == 2 and 1.1 <= units / (3 * sms) <= 1.5      # evens out a second wave on purpose
+                assert S == 1 or halves or units <= (alone if depth == 4 else shared)[S - 1], (units, rows, S, depth)
+        for P in (100, 4097, 9000, 33000, 140000):
+            cs = lib.mixkv_internal_tail_clusters(C.c_int64(units), P, sms, array(alone))
+            assert cs in (1, 2, 4, 8) and (cs == 1 or units <= alone[cs - 1]), (units, P, cs)
+            cs = lib.mixkv_internal_budget_clusters(units, C.c_int64(8 * P), array(alone))
+            assert cs in (1, 2, 4, 8) and (cs == 1 or units <= alone[cs - 1]), (units, P, cs)
+
+
+@pytest.mark.parametrize("units,rows,even,want", [
+    (4, 512, 1, (8, 2)), (15, 1500, 1, (8, 4)), (16, 1500, 1, (8, 2)), (16, 8000, 1, (6, 4)), (17, 1500, 1, (6, 4)),
+    (28, 2500, 0, (8, 2)), (49, 1500, 1, (7, 2)), (896, 512, 0, (1, 2)), (560, 2500, 0, (2, 2)), (12, 60, 1, (1, 2))])
+def test_decode_shapes_as_measured(lib, units, rows, even, want):
+    assert decode(lib, B200, units, rows, even) == want
+
+
+def test_tail_and_budget_clusters_as_measured(lib):
+    sms, alone, _ = B200
+    tail = lambda units, P: lib.mixkv_internal_tail_clusters(C.c_int64(units), P, sms, array(alone))
+    assert [tail(14, 30000), tail(15, 30000), tail(29, 12000), tail(30, 12000), tail(73, 9000), tail(74, 9000),
+            tail(4, 4096)] == [8, 4, 4, 2, 2, 1, 1]
+    budget = lambda pairs, keys: lib.mixkv_internal_budget_clusters(pairs, C.c_int64(keys), array(alone))
+    assert [budget(1, 8192), budget(15, 60000), budget(16, 60000), budget(33, 60000), budget(34, 60000),
+            budget(74, 60000), budget(75, 60000), budget(74, 8193)] == [1, 8, 4, 4, 2, 2, 1, 2]
