@@ -60,12 +60,6 @@ struct Unlocked {
   PyThreadState* state = PyEval_SaveThread();
   ~Unlocked() { PyEval_RestoreThread(state); }
 };
-// A call of the library without the lock; the arguments are evaluated before it is given up.
-template <typename... P, typename... A>
-int enqueue(int (*fn)(P...), A... args) {
-  const Unlocked u;
-  return fn(args...);
-}
 
 [[noreturn]] void fail(PyObject* type, const char* what) {
   PyErr_SetString(type, what);
@@ -196,13 +190,9 @@ void* stream_of(PyObject* o) {
   return s;
 }
 
+// (called without the interpreter lock)
 at::Tensor empty(at::IntArrayRef size, at::ScalarType type, const at::Tensor& like) {
-  const Unlocked u;
   return at::Tensor(at::detail::empty_cuda(size, type, like.device(), std::nullopt));
-}
-at::Tensor zero_word(const at::Tensor& like) {   // (enqueues a fill)
-  const Unlocked u;
-  return at::zeros({1}, like.options().dtype(at::kInt));
 }
 int32_t* ip(const at::Tensor& t) { return static_cast<int32_t*>(t.data_ptr()); }
 float* fp(const at::Tensor& t) { return static_cast<float*>(t.data_ptr()); }
@@ -224,6 +214,7 @@ struct Space {
     if (o == Py_None) {
       size_t need = 0;
       check_status(api.ws_size(&p, layers, cu.batch, Ltot, cu.max_len(Ltot), &need), "mixkv_workspace_size");
+      const Unlocked u;
       own = empty({(int64_t)need}, at::kByte, like);
       data = own.data_ptr();
       bytes = need;
@@ -289,21 +280,25 @@ PyObject* py_scores(PyObject*, PyObject* const* a, Py_ssize_t n) {
     std::optional<Space> ws;
     if (!fixed) ws.emplace(a[6], p, 1, cu, (int)Ltot, K);
     if (Ptot < 0) check_status(MIXKV_ERR_INVALID_ARG, fixed ? "mixkv_scores_static" : "mixkv_scores");
-    at::Tensor s_comp = empty({H, Ptot}, at::kFloat, K), s_ex, s_div, rbar;
-    if (parts) {
-      s_ex = empty({H, Ptot}, at::kFloat, K);
-      s_div = empty({H, Ptot}, at::kFloat, K);
-      rbar = empty({cu.batch, H}, at::kFloat, K);
-    }
-    at::Tensor status = empty({1}, at::kInt, K);
+    at::Tensor s_comp, s_ex, s_div, rbar, status;
     void* stream = stream_of(a[7]);
     void *k = ptr(a[0]), *v = ptr(a[1]), *q = ptr(a[2]);
     const float* rin = ptr<float>(a[5]);
-    float *pe = parts ? fp(s_ex) : nullptr, *pd = parts ? fp(s_div) : nullptr,
-          *pr = parts ? fp(rbar) : nullptr;
-    check_status(enqueue(api.scores, k, v, q, cu.data(), cu.batch, (int)Ltot, &p, fixed ? 1 : 0, fixed ? nullptr : ws->data,
-                         fixed ? 0 : ws->bytes, fp(s_comp), pe, pd, pr, rin, ip(status), stream),
-                 fixed ? "mixkv_scores_static" : "mixkv_scores");
+    int rc;
+    {
+      const Unlocked u;
+      s_comp = empty({H, Ptot}, at::kFloat, K);
+      if (parts) {
+        s_ex = empty({H, Ptot}, at::kFloat, K);
+        s_div = empty({H, Ptot}, at::kFloat, K);
+        rbar = empty({cu.batch, H}, at::kFloat, K);
+      }
+      status = empty({1}, at::kInt, K);
+      rc = api.scores(k, v, q, cu.data(), cu.batch, (int)Ltot, &p, fixed ? 1 : 0, fixed ? nullptr : ws->data,
+                      fixed ? 0 : ws->bytes, fp(s_comp), parts ? fp(s_ex) : nullptr, parts ? fp(s_div) : nullptr,
+                      parts ? fp(rbar) : nullptr, rin, ip(status), stream);
+    }
+    check_status(rc, fixed ? "mixkv_scores_static" : "mixkv_scores");
     Dict out;
     put(out.d, nm.s_comp, s_comp);
     if (parts) {
@@ -326,11 +321,20 @@ PyObject* py_select(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const int64_t H = s.size(0), Ltot = s.size(1) + (int64_t)cu.batch * p.window, BH = cu.batch * H;
     const Space ws(a[3], p, 1, cu, (int)Ltot, s);
     const int64_t cap = std::max<int64_t>(BH * (p.budget - p.window), 1);
-    at::Tensor idx = empty({cap}, at::kInt, s), counts = empty({BH}, at::kInt, s),
-               offs = empty({BH + 1}, at::kInt, s), status = empty({1}, at::kInt, s);
-    check_status(enqueue(api.select, ptr<const float>(a[0]), cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes,
-                         ip(idx), ip(counts), ip(offs), ip(status), stream_of(a[4])),
-                 "mixkv_select");
+    const float* scores = ptr<const float>(a[0]);
+    void* stream = stream_of(a[4]);
+    at::Tensor idx, counts, offs, status;
+    int rc;
+    {
+      const Unlocked u;
+      idx = empty({cap}, at::kInt, s);
+      counts = empty({BH}, at::kInt, s);
+      offs = empty({BH + 1}, at::kInt, s);
+      status = empty({1}, at::kInt, s);
+      rc = api.select(scores, cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes, ip(idx), ip(counts), ip(offs),
+                      ip(status), stream);
+    }
+    check_status(rc, "mixkv_select");
     Dict out;
     put(out.d, nm.idx, idx);
     put(out.d, nm.counts, counts);
@@ -350,21 +354,32 @@ PyObject* compress_outputs(PyObject* given, PyObject* aux, const int64_t lead, c
     Py_INCREF(given);
     return given;
   }
-  auto make = [&](std::vector<int64_t> size, const at::ScalarType t) {
-    if (lead >= 0) size.insert(size.begin(), lead);
-    return empty(size, t, K);
-  };
-  Dict out;
-  put(out.d, nm.K_out, make({rows, K.size(-1)}, at::kBFloat16));
-  put(out.d, nm.V_out, make({rows, K.size(-1)}, at::kBFloat16));
-  put(out.d, nm.out_row_offsets, make({BH + 1}, at::kInt));
-  put(out.d, nm.status, zero_word(K));
-  if (truth(aux)) {
-    put(out.d, nm.idx, make({cap}, at::kInt));
-    put(out.d, nm.counts, make({BH}, at::kInt));
-    put(out.d, nm.idx_offsets, make({BH + 1}, at::kInt));
-    put(out.d, nm.s_comp, make({H, Ptot}, at::kFloat));
+  const bool with_aux = truth(aux);
+  struct {
+    PyObject* key;
+    at::ScalarType type;
+    std::vector<int64_t> size;
+    at::Tensor t;
+  } outputs[] = {{nm.K_out, at::kBFloat16, {rows, K.size(-1)}, {}},
+                 {nm.V_out, at::kBFloat16, {rows, K.size(-1)}, {}},
+                 {nm.out_row_offsets, at::kInt, {BH + 1}, {}},
+                 {nm.idx, at::kInt, {cap}, {}},
+                 {nm.counts, at::kInt, {BH}, {}},
+                 {nm.idx_offsets, at::kInt, {BH + 1}, {}},
+                 {nm.s_comp, at::kFloat, {H, Ptot}, {}}};
+  const int n = with_aux ? 7 : 3;
+  at::Tensor status;
+  {
+    const Unlocked u;
+    for (int i = 0; i < n; ++i) {
+      if (lead >= 0) outputs[i].size.insert(outputs[i].size.begin(), lead);
+      outputs[i].t = empty(outputs[i].size, outputs[i].type, K);
+    }
+    status = at::zeros({1}, K.options().dtype(at::kInt));   // (enqueues a fill)
   }
+  Dict out;
+  for (int i = 0; i < n; ++i) put(out.d, outputs[i].key, outputs[i].t);
+  put(out.d, nm.status, status);
   return out.release();
 }
 struct Ref {   // an owned reference
@@ -409,11 +424,16 @@ PyObject* py_compress_layer(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const long long events = PyLong_AsLongLong(a[10]);
     const long n_events = PyLong_AsLong(a[11]);
     if (PyErr_Occurred()) throw Raised();
-    check_status(enqueue(api.layer, ptr(a[0]), ptr(a[1]), ptr(a[2]), cu.data(), cu.batch, (int)Ltot, &p, ws.data,
-                         ws.bytes, ptr<const float>(a[5]), o.K, o.V, o.row_offsets, o.idx, o.counts,
-                         o.idx_offsets, o.s_comp, o.status, stream_of(a[7]),
-                         reinterpret_cast<void* const*>(events), (int)n_events),
-                 "mixkv_compress_layer");
+    void *k = ptr(a[0]), *v = ptr(a[1]), *q = ptr(a[2]), *stream = stream_of(a[7]);
+    const float* rin = ptr<const float>(a[5]);
+    int rc;
+    {
+      const Unlocked u;
+      rc = api.layer(k, v, q, cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes, rin, o.K, o.V, o.row_offsets,
+                     o.idx, o.counts, o.idx_offsets, o.s_comp, o.status, stream,
+                     reinterpret_cast<void* const*>(events), (int)n_events);
+    }
+    check_status(rc, "mixkv_compress_layer");
     return out.release();
   });
 }
@@ -453,22 +473,27 @@ PyObject* py_compress_layers(PyObject*, PyObject* const* a, Py_ssize_t n) {
     if (PyErr_Occurred()) throw Raised();
     const float* rin = ptr<const float>(a[5]);
     void* stream = stream_of(a[7]);
+    const int32_t* budgets = nullptr;
     if (a[12] != Py_None) {
       const at::Tensor& hb = tensor(a[12]);
       want_contiguous(hb);
       if (hb.scalar_type() != at::kInt || hb.dim() != 2 || hb.size(0) != NL || hb.size(1) != BH || n_events)
         fail(PyExc_AssertionError, "head_budgets must be an int32 tensor [layers, batch * H], without events");
-      check_status(enqueue(api.budgeted, K.data_ptr(), V.data_ptr(), Q.data_ptr(), (int)NL, K.stride(0), Q.stride(0),
-                           cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes, rin, ip(hb), o.K, o.V,
-                           o.row_offsets, o.idx, o.counts, o.idx_offsets, o.s_comp, o.status, stream),
-                   "mixkv_compress_layers_budgeted");
-    } else {
-      check_status(enqueue(api.layers, K.data_ptr(), V.data_ptr(), Q.data_ptr(), (int)NL, K.stride(0), Q.stride(0),
-                           cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes, rin, o.K, o.V,
-                           o.row_offsets, o.idx, o.counts, o.idx_offsets, o.s_comp, o.status, stream,
-                           reinterpret_cast<void* const*>(events), (int)n_events),
-                   "mixkv_compress_layers");
+      budgets = ip(hb);
     }
+    void *k = K.data_ptr(), *v = V.data_ptr(), *q = Q.data_ptr();
+    const int64_t kv_stride = K.stride(0), q_stride = Q.stride(0);
+    int rc;
+    {
+      const Unlocked u;
+      rc = budgets ? api.budgeted(k, v, q, (int)NL, kv_stride, q_stride, cu.data(), cu.batch, (int)Ltot, &p, ws.data,
+                                  ws.bytes, rin, budgets, o.K, o.V, o.row_offsets, o.idx, o.counts, o.idx_offsets,
+                                  o.s_comp, o.status, stream)
+                   : api.layers(k, v, q, (int)NL, kv_stride, q_stride, cu.data(), cu.batch, (int)Ltot, &p, ws.data,
+                                ws.bytes, rin, o.K, o.V, o.row_offsets, o.idx, o.counts, o.idx_offsets, o.s_comp,
+                                o.status, stream, reinterpret_cast<void* const*>(events), (int)n_events);
+    }
+    check_status(rc, budgets ? "mixkv_compress_layers_budgeted" : "mixkv_compress_layers");
     return out.release();
   });
 }
@@ -488,12 +513,21 @@ PyObject* py_similarity_map(PyObject*, PyObject* const* a, Py_ssize_t n) {
     size_t need = 0;
     check_status(api.sim_ws_size(heads, L, (int)block, &need), "mixkv_similarity_workspace_size");
     const int64_t T = (L + block - 1) / block;
-    at::Tensor ws = empty({(int64_t)need}, at::kByte, X), cells = empty({heads, T, T}, at::kFloat, X), mean;
-    if (truth(a[2])) mean = empty({heads}, at::kFloat, X);
-    check_status(enqueue(api.sim_map, X.data_ptr(), heads, L, (int)X.size(2), (int)block, ws.data_ptr(), need, fp(cells),
-                         mean.defined() ? fp(mean) : nullptr, stream_of(a[3])),
-                 "mixkv_similarity_map");
-    Ref c(THPVariable_Wrap(cells)), m(mean.defined() ? THPVariable_Wrap(mean) : Py_NewRef(Py_None));
+    const bool want_mean = truth(a[2]);
+    void *x = X.data_ptr(), *stream = stream_of(a[3]);
+    const int d = (int)X.size(2);
+    at::Tensor ws, cells, mean;
+    int rc;
+    {
+      const Unlocked u;
+      ws = empty({(int64_t)need}, at::kByte, X);
+      cells = empty({heads, T, T}, at::kFloat, X);
+      if (want_mean) mean = empty({heads}, at::kFloat, X);
+      rc = api.sim_map(x, heads, L, d, (int)block, ws.data_ptr(), need, fp(cells), want_mean ? fp(mean) : nullptr,
+                       stream);
+    }
+    check_status(rc, "mixkv_similarity_map");
+    Ref c(THPVariable_Wrap(cells)), m(want_mean ? THPVariable_Wrap(mean) : Py_NewRef(Py_None));
     if (!c.o || !m.o) throw Raised();
     return PyTuple_Pack(2, c.o, m.o);
   });
@@ -512,11 +546,19 @@ PyObject* py_decode_attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const long H = PyLong_AsLong(a[4]), G = PyLong_AsLong(a[5]), rows = PyLong_AsLong(a[6]);
     const double scale = PyFloat_AsDouble(a[7]);
     if (PyErr_Occurred()) throw Raised();
-    at::Tensor out = empty(q.sizes(), at::kFloat, q);
-    check_status(enqueue(api.decode, K.data_ptr(), V.data_ptr(), ip(offs), K.size(1), q.data_ptr(), (int)K.size(0),
-                         (int)q.size(1), (int)H, (int)G, (int)K.size(2), (float)scale, (int)rows, fp(out),
-                         stream_of(a[8])),
-                 "mixkv_decode_attention");
+    void *k = K.data_ptr(), *v = V.data_ptr(), *query = q.data_ptr(), *stream = stream_of(a[8]);
+    const int32_t* offsets = ip(offs);
+    const int layers = (int)K.size(0), batch = (int)q.size(1), d = (int)K.size(2);
+    const int64_t cap = K.size(1);
+    at::Tensor out;
+    int rc;
+    {
+      const Unlocked u;
+      out = empty(q.sizes(), at::kFloat, q);
+      rc = api.decode(k, v, offsets, cap, query, layers, batch, (int)H, (int)G, d, (float)scale, (int)rows, fp(out),
+                      stream);
+    }
+    check_status(rc, "mixkv_decode_attention");
     return THPVariable_Wrap(out);
   });
 }
