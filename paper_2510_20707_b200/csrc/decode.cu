@@ -5,8 +5,8 @@
 // tile would be padding), too many multiply-adds for the fp32 pipe at HBM speed (2 * 2 * G * 128
 // per 512-byte row pair), so they run as warp-level mma.sync m16n8k16 (bf16 x bf16 -> fp32):
 //
-//   * a warp takes 16 cache rows per step, copied asynchronously into a ring of two (K, V) slot pairs of its own
-//     (rows on a 272-byte pitch); a slot is asked for again as soon as its rows are used.  logits:
+//   * a warp takes 16 cache rows per step, copied asynchronously into a ring of one to four (K, V) slot pairs of its
+//     own (rows on a 272-byte pitch); a slot is asked for again as soon as its rows are used.  logits:
 //     D[head, row] = q[head, :] . K[row, :], A = q (held in registers for the whole kernel), B = K rows.  The
 //     contraction index may be permuted freely as long as A and B agree, so a lane takes 64
 //     CONTIGUOUS bytes of its row (four 16-byte loads, in an order that keeps the shared-memory banks
@@ -47,8 +47,9 @@ constexpr int kDecStep = 16;     // cache rows per warp step
 constexpr int kDecPitch = 272;                      // bytes between the rows of a slot
 constexpr int kDecSlot = kDecStep * kDecPitch;      // one K or V slot
 // Steps a warp has on their way or in work: two with three CTAs on an SM, three with two, four when a CTA has an
-// SM for itself.
+// SM for itself (decode_shape).
 constexpr int kDecDepth = 2, kDecDepthPair = 3, kDecDepthAlone = 4;
+constexpr int kDecDepthEven = 1;   // one (in the room of three) with two CTAs and long heads of one length
 
 // Dynamic shared memory for GP = 8 or 16 head slots: per warp its ring and then, the steps being over, its value
 // sums [GP][132] in the same place; the CTA's sums xo [GP][128] behind those of warp 0, in what was its ring (with
@@ -56,7 +57,9 @@ constexpr int kDecDepth = 2, kDecDepthPair = 3, kDecDepthAlone = 4;
 // sequences of 603 rows and 12 heads 25.3 us); wm / wz [warps][16], xm / xz [16], allm / allz [8][16] every
 // rank's (reference, sum) during the cluster merge.
 constexpr int kDecHeadPitch = kHeadDim + 4;   // floats between the heads of a warp's value sums
-__host__ __device__ constexpr size_t dec_warp_bytes(int depth) { return 2 * (size_t)depth * kDecSlot; }
+__host__ __device__ constexpr size_t dec_warp_bytes(int depth) {
+  return 2 * (size_t)(depth == kDecDepthEven ? kDecDepthPair : depth) * kDecSlot;
+}
 static_assert(16 * (kDecHeadPitch + kHeadDim) * 4 <= dec_warp_bytes(kDecDepth), "sums of a warp and of the CTA fit a ring");
 constexpr size_t dec_smem(int depth) {
   return kDecWarps * dec_warp_bytes(depth) + (2 * kDecWarps + 2 + 2 * 8) * kDecMaxG * 4;
@@ -392,6 +395,7 @@ using DecKernel = void (*)(const __nv_bfloat16*, const __nv_bfloat16*, const int
 DecKernel dec_kernel(const bool wide, const int depth) {
   switch (depth) {
     case kDecDepthAlone: return wide ? k_decode_attention<true, kDecDepthAlone> : k_decode_attention<false, kDecDepthAlone>;
+    case kDecDepthEven: return wide ? k_decode_attention<true, kDecDepthEven> : k_decode_attention<false, kDecDepthEven>;
     case kDecDepthPair: return wide ? k_decode_attention<true, kDecDepthPair> : k_decode_attention<false, kDecDepthPair>;
     default: return wide ? k_decode_attention<true, kDecDepth> : k_decode_attention<false, kDecDepth>;
   }
@@ -434,9 +438,14 @@ DecodeShape decode_shape(const long long units, const int max_rows, const bool e
     if (x >= (even ? 4 : kMaxCluster) && steps >= kDecWarps * x) return {x, kDecDepthAlone};
   }
   // A CTA per unit and no more than two per SM: those two, with the ring of three (with room for a third some SMs
-  // get three and others one: 296 units of 3400 rows 102.8 -> 89.7 us, 280 of 5000 142.6 -> 124.4, 256 of 300
-  // 13.6 -> 12.9; 240 units of 3400 rows 77.1 -> 78.3, of 512 ragged 31.8 -> 29.7).
-  return {S, S == 1 && units > sms && units <= 2LL * sms ? kDecDepthPair : kDecDepth};
+  // get three and others one: 280 units of 5000 rows 142.6 -> 124.4 us, 256 of 300 13.6 -> 12.9, of 512 ragged
+  // 41 -> 31).  Long heads of one length leave DRAM no gap then, and the SMs that get their rows first run ahead with
+  // their rings while the others decide the call (SMs 81 % active, with a step in registers 89): one slot pair in
+  // flight per warp keeps them level (296 units of 5000 rows 129.9 -> 120.1 us, with operands in registers 118.4; 256 of
+  // 3400 80.8 -> 74.9, registers 79.5; 296 of 1000 30.7 -> 29.5).  Ragged heads in a cache of that very size lose by it
+  // (256 units of 500 to 2000 rows 37.5 -> 39.9 us), so short ones, which gain little, keep the ring of three.
+  const bool pair = S == 1 && units > sms && units <= 2LL * sms;
+  return {S, !pair ? kDecDepth : even && steps >= 80 ? kDecDepthEven : kDecDepthPair};
 }
 
 }  // namespace
@@ -473,10 +482,10 @@ extern "C" int mixkv_decode_attention(const void* K_cache, const void* V_cache,
   const long long units = (long long)n_layers * batch * kv_heads;
   if (units * 8 > 0x7fffffffLL) return MIXKV_ERR_UNSUPPORTED;
   const bool wide = gqa_ratio > 8;
-  static std::atomic<bool> done[6][kMaxDevices];
-  static ClusterFit fit[6];   // (by variant, as `done`)
+  static std::atomic<bool> done[10][kMaxDevices];
+  static ClusterFit fit[10];   // (by variant, as `done`)
   const int dev = device_slot();
-  auto variant = [&](const int depth) { return 2 * (depth - kDecDepth) + wide; };
+  auto variant = [&](const int depth) { return 2 * depth + wide; };
   auto resident = [&](const int depth) {
     return [&, depth](const int size) {
       const DecKernel k = dec_kernel(wide, depth);

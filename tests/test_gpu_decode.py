@@ -132,6 +132,29 @@ def test_more_units_than_one_wave(NL, batch, H, G, lo, hi):
             assert np.allclose(rows, p @ v[l, a:e] / p.sum(1, keepdims=True), rtol=2e-4, atol=2e-5), (l, u)
 
 
+@pytest.mark.parametrize("units,rows,G,ragged", [
+    (224, 1280, 7, False), (296, 1265, 16, False), (296, 1300, 4, True), (223, 1281, 9, True), (296, 1264, 4, True)])
+def test_two_units_per_sm_in_a_cache_of_their_size(units, rows, G, ragged):
+    # the cache has room for max_rows rows of every head: from 80 steps on one slot pair per warp in flight, whether
+    # the heads are of one length or not (none, one, a step and one, all rows among them)
+    rng = np.random.default_rng(units + rows)
+    counts = rng.integers(0, rows + 1, units) if ragged else np.full(units, rows)
+    if ragged:
+        counts[:6] = 0, 1, 16, 17, rows - 1, rows
+    gen = torch.Generator(device="cuda").manual_seed(rows)
+    K, V = (torch.randn((1, units * rows, 128), generator=gen, device="cuda").bfloat16() for _ in range(2))
+    q = torch.randn((1, units, G, 128), generator=gen, device="cuda").bfloat16()
+    offs = np.concatenate([[0], counts.cumsum()]).astype(np.int32)
+    call = lambda: binding.decode_attention(K, V, torch.from_numpy(offs[None]).cuda(), q, 1, G, rows)
+    out = call()
+    assert torch.equal(out, call())
+    Kd, Vd, qd = K[0].double(), V[0].double(), q[0].double()
+    for u in range(units):
+        a, e = offs[u], offs[u + 1]
+        want = torch.softmax(qd[u] @ Kd[a:e].T / np.sqrt(128.0), 1) @ Vd[a:e]     # (no rows: zeros)
+        assert torch.allclose(out[0, u].double(), want, rtol=RTOL, atol=ATOL), u
+
+
 def test_repeated_calls_are_bit_identical():
     # the steps of a head go to fixed warps and the partial results are merged in a fixed order
     # (warps through shared memory, CTAs through distributed shared memory): twenty calls on the
