@@ -15,11 +15,14 @@
 
 #include <ATen/ATen.h>
 #include <ATen/cuda/EmptyTensor.h>
+#include <c10/cuda/CUDAFunctions.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include <dlfcn.h>
 
+#include <optional>
 #include <vector>
 
 #include "../internal_api.h"
@@ -180,15 +183,28 @@ struct Offsets {
   }
 };
 
-void* stream_of(PyObject* o) {
-  if (o == Py_None) return (void*)c10::cuda::getCurrentCUDAStream().stream();
-  PyObject* v = PyObject_GetAttr(o, nm.cuda_stream);
-  if (!v) throw Raised();
-  void* s = PyLong_AsVoidPtr(v);
-  Py_DECREF(v);
-  if (!s && PyErr_Occurred()) throw Raised();
-  return s;
-}
+// The stream of a call: the one it is given, else the current one.  While this lives it is the current one, so that what
+// the call allocates, fills and gives back (a workspace of its own is free again when the call returns, long before the
+// GPU is done with it) is ordered on the stream its kernels run on.
+struct CallStream {
+  void* handle;
+  std::optional<c10::cuda::CUDAStreamGuard> guard;
+  CallStream(PyObject* o, const at::Tensor& like) {
+    if (o == Py_None) {
+      handle = (void*)c10::cuda::getCurrentCUDAStream().stream();
+      return;
+    }
+    PyObject* v = PyObject_GetAttr(o, nm.cuda_stream);
+    if (!v) throw Raised();
+    handle = PyLong_AsVoidPtr(v);
+    Py_DECREF(v);
+    if (!handle && PyErr_Occurred()) throw Raised();
+    if (!like.is_cuda()) return;
+    const c10::DeviceIndex device = c10::cuda::current_device();
+    if (handle != (void*)c10::cuda::getCurrentCUDAStream(device).stream())
+      guard.emplace(c10::cuda::getStreamFromExternal((cudaStream_t)handle, device));
+  }
+};
 
 // (called without the interpreter lock)
 at::Tensor empty(at::IntArrayRef size, at::ScalarType type, const at::Tensor& like) {
@@ -277,11 +293,11 @@ PyObject* py_scores(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const Offsets cu(a[4]);
     const bool parts = truth(a[8]), fixed = truth(a[9]);
     const int64_t H = K.size(0), Ltot = K.size(1), Ptot = Ltot - (int64_t)cu.batch * p.window;
+    const CallStream stream(a[7], K);
     std::optional<Space> ws;
     if (!fixed) ws.emplace(a[6], p, 1, cu, (int)Ltot, K);
     if (Ptot < 0) check_status(MIXKV_ERR_INVALID_ARG, fixed ? "mixkv_scores_static" : "mixkv_scores");
     at::Tensor s_comp, s_ex, s_div, rbar, status;
-    void* stream = stream_of(a[7]);
     void *k = ptr(a[0]), *v = ptr(a[1]), *q = ptr(a[2]);
     const float* rin = ptr<float>(a[5]);
     int rc;
@@ -296,7 +312,7 @@ PyObject* py_scores(PyObject*, PyObject* const* a, Py_ssize_t n) {
       status = empty({1}, at::kInt, K);
       rc = api.scores(k, v, q, cu.data(), cu.batch, (int)Ltot, &p, fixed ? 1 : 0, fixed ? nullptr : ws->data,
                       fixed ? 0 : ws->bytes, fp(s_comp), parts ? fp(s_ex) : nullptr, parts ? fp(s_div) : nullptr,
-                      parts ? fp(rbar) : nullptr, rin, ip(status), stream);
+                      parts ? fp(rbar) : nullptr, rin, ip(status), stream.handle);
     }
     check_status(rc, fixed ? "mixkv_scores_static" : "mixkv_scores");
     Dict out;
@@ -319,10 +335,10 @@ PyObject* py_select(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const mixkv_params p = params(a[1]);
     const Offsets cu(a[2]);
     const int64_t H = s.size(0), Ltot = s.size(1) + (int64_t)cu.batch * p.window, BH = cu.batch * H;
+    const CallStream stream(a[4], s);
     const Space ws(a[3], p, 1, cu, (int)Ltot, s);
     const int64_t cap = std::max<int64_t>(BH * (p.budget - p.window), 1);
     const float* scores = ptr<const float>(a[0]);
-    void* stream = stream_of(a[4]);
     at::Tensor idx, counts, offs, status;
     int rc;
     {
@@ -332,7 +348,7 @@ PyObject* py_select(PyObject*, PyObject* const* a, Py_ssize_t n) {
       offs = empty({BH + 1}, at::kInt, s);
       status = empty({1}, at::kInt, s);
       rc = api.select(scores, cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes, ip(idx), ip(counts), ip(offs),
-                      ip(status), stream);
+                      ip(status), stream.handle);
     }
     check_status(rc, "mixkv_select");
     Dict out;
@@ -416,6 +432,7 @@ PyObject* py_compress_layer(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const mixkv_params p = params(a[3]);
     const Offsets cu(a[4]);
     const int64_t H = K.size(0), Ltot = K.size(1), BH = cu.batch * H;
+    const CallStream stream(a[7], K);
     const Space ws(a[6], p, 1, cu, (int)Ltot, K);
     Ref out(compress_outputs(a[8], a[9], -1, BH * p.budget,
                              std::max<int64_t>(BH * (p.budget - p.window), 1), BH, H,
@@ -424,13 +441,13 @@ PyObject* py_compress_layer(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const long long events = PyLong_AsLongLong(a[10]);
     const long n_events = PyLong_AsLong(a[11]);
     if (PyErr_Occurred()) throw Raised();
-    void *k = ptr(a[0]), *v = ptr(a[1]), *q = ptr(a[2]), *stream = stream_of(a[7]);
+    void *k = ptr(a[0]), *v = ptr(a[1]), *q = ptr(a[2]);
     const float* rin = ptr<const float>(a[5]);
     int rc;
     {
       const Unlocked u;
       rc = api.layer(k, v, q, cu.data(), cu.batch, (int)Ltot, &p, ws.data, ws.bytes, rin, o.K, o.V, o.row_offsets,
-                     o.idx, o.counts, o.idx_offsets, o.s_comp, o.status, stream,
+                     o.idx, o.counts, o.idx_offsets, o.s_comp, o.status, stream.handle,
                      reinterpret_cast<void* const*>(events), (int)n_events);
     }
     check_status(rc, "mixkv_compress_layer");
@@ -461,6 +478,7 @@ PyObject* py_compress_layers(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const mixkv_params p = params(a[3]);
     const Offsets cu(a[4]);
     const int64_t NL = K.size(0), H = K.size(1), Ltot = K.size(2), BH = cu.batch * H;
+    const CallStream stream(a[7], K);
     const Space ws(a[6], p, (int)NL, cu, (int)Ltot, K);
     int64_t cap = 0;
     for (int b = 0; b < cu.batch; ++b)
@@ -472,7 +490,6 @@ PyObject* py_compress_layers(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const long n_events = PyLong_AsLong(a[11]);
     if (PyErr_Occurred()) throw Raised();
     const float* rin = ptr<const float>(a[5]);
-    void* stream = stream_of(a[7]);
     const int32_t* budgets = nullptr;
     if (a[12] != Py_None) {
       const at::Tensor& hb = tensor(a[12]);
@@ -488,10 +505,10 @@ PyObject* py_compress_layers(PyObject*, PyObject* const* a, Py_ssize_t n) {
       const Unlocked u;
       rc = budgets ? api.budgeted(k, v, q, (int)NL, kv_stride, q_stride, cu.data(), cu.batch, (int)Ltot, &p, ws.data,
                                   ws.bytes, rin, budgets, o.K, o.V, o.row_offsets, o.idx, o.counts, o.idx_offsets,
-                                  o.s_comp, o.status, stream)
+                                  o.s_comp, o.status, stream.handle)
                    : api.layers(k, v, q, (int)NL, kv_stride, q_stride, cu.data(), cu.batch, (int)Ltot, &p, ws.data,
                                 ws.bytes, rin, o.K, o.V, o.row_offsets, o.idx, o.counts, o.idx_offsets, o.s_comp,
-                                o.status, stream, reinterpret_cast<void* const*>(events), (int)n_events);
+                                o.status, stream.handle, reinterpret_cast<void* const*>(events), (int)n_events);
     }
     check_status(rc, budgets ? "mixkv_compress_layers_budgeted" : "mixkv_compress_layers");
     return out.release();
@@ -514,7 +531,8 @@ PyObject* py_similarity_map(PyObject*, PyObject* const* a, Py_ssize_t n) {
     check_status(api.sim_ws_size(heads, L, (int)block, &need), "mixkv_similarity_workspace_size");
     const int64_t T = (L + block - 1) / block;
     const bool want_mean = truth(a[2]);
-    void *x = X.data_ptr(), *stream = stream_of(a[3]);
+    const CallStream stream(a[3], X);
+    void* x = X.data_ptr();
     const int d = (int)X.size(2);
     at::Tensor ws, cells, mean;
     int rc;
@@ -524,7 +542,7 @@ PyObject* py_similarity_map(PyObject*, PyObject* const* a, Py_ssize_t n) {
       cells = empty({heads, T, T}, at::kFloat, X);
       if (want_mean) mean = empty({heads}, at::kFloat, X);
       rc = api.sim_map(x, heads, L, d, (int)block, ws.data_ptr(), need, fp(cells), want_mean ? fp(mean) : nullptr,
-                       stream);
+                       stream.handle);
     }
     check_status(rc, "mixkv_similarity_map");
     Ref c(THPVariable_Wrap(cells)), m(want_mean ? THPVariable_Wrap(mean) : Py_NewRef(Py_None));
@@ -546,7 +564,8 @@ PyObject* py_decode_attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const long H = PyLong_AsLong(a[4]), G = PyLong_AsLong(a[5]), rows = PyLong_AsLong(a[6]);
     const double scale = PyFloat_AsDouble(a[7]);
     if (PyErr_Occurred()) throw Raised();
-    void *k = K.data_ptr(), *v = V.data_ptr(), *query = q.data_ptr(), *stream = stream_of(a[8]);
+    const CallStream stream(a[8], K);
+    void *k = K.data_ptr(), *v = V.data_ptr(), *query = q.data_ptr();
     const int32_t* offsets = ip(offs);
     const int layers = (int)K.size(0), batch = (int)q.size(1), d = (int)K.size(2);
     const int64_t cap = K.size(1);
@@ -556,7 +575,7 @@ PyObject* py_decode_attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
       const Unlocked u;
       out = empty(q.sizes(), at::kFloat, q);
       rc = api.decode(k, v, offsets, cap, query, layers, batch, (int)H, (int)G, d, (float)scale, (int)rows, fp(out),
-                      stream);
+                      stream.handle);
     }
     check_status(rc, "mixkv_decode_attention");
     return THPVariable_Wrap(out);

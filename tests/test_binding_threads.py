@@ -144,3 +144,32 @@ def test_calls_from_several_threads():
     for t in threads:
         t.join()
     assert found == [True] * 80, found
+
+
+@pytest.mark.gpu
+def test_what_a_call_allocates_belongs_to_its_stream():
+    # a workspace of the call's own is given back when the call returns: it may only be handed out again in the order
+    # of the stream its kernels run on, whatever the current stream is
+    import torch
+    from paper_2510_20707_b200 import binding
+    K, Q = torch.randn((4, 20000, 128), device="cuda").bfloat16(), torch.randn((1, 16, 32, 128), device="cuda").bfloat16()
+    p = binding.Params(kv_heads=4, gqa_ratio=4, budget=128)
+    need = binding.workspace_size(p, 1, 20000, 20000)
+    ref = binding.scores(K, K, Q, p)["s_comp"]
+    torch.cuda.synchronize()
+    offs, q = torch.tensor([[0, 20000]], dtype=torch.int32, device="cuda"), torch.zeros((1, 1, 4, 128), device="cuda").bfloat16()
+    for call in (lambda s: binding.scores(K, K, Q, p, stream=s), lambda s: binding.compress_layer(K, K, Q, p, stream=s),
+                 lambda s: binding.select(ref, p, stream=s), lambda s: binding.similarity_map(K, 4, stream=s),
+                 lambda s: binding.compress_layers(K[None], K[None], Q[None], p, stream=s),
+                 lambda s: binding.decode_attention(K[:1], K[:1], offs, q, 1, 4, 20000, stream=s)):
+        torch.cuda.empty_cache()
+        side = torch.cuda.Stream()
+        before = sum(seg["total_size"] for seg in torch.cuda.memory_snapshot() if seg["stream"] == 0)
+        out = call(side)
+        assert torch.cuda.current_stream() != side
+        own = sum(seg["total_size"] for seg in torch.cuda.memory_snapshot() if seg["stream"] == side.cuda_stream)
+        assert own > 0 and sum(seg["total_size"] for seg in torch.cuda.memory_snapshot() if seg["stream"] == 0) == before
+        side.synchronize()
+        if isinstance(out, dict) and "s_comp" in out:
+            assert torch.equal(out["s_comp"].view_as(ref), ref) and own >= need
+        del out
