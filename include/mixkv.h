@@ -14,7 +14,7 @@
  *    device memory and never synchronises the stream: every call only enqueues kernels
  *    on `stream` (a cudaStream_t passed as void*; NULL is the default stream).  Host
  *    state kept between calls is limited to per-device caches of attributes (SM count,
- *    compute capability, shared-memory opt-in).  The workspace needs no initialisation
+ *    compute capability, shared-memory opt-in, clusters resident at once).  The workspace needs no initialisation
  *    and no clearing between calls (every word a kernel reads was written earlier in the
  *    same call; nothing is counted across CTAs), and may be reused for other shapes; two
  *    calls that may overlap in time need a workspace each.

@@ -58,7 +58,7 @@ struct Workspace {
   float2* rowstat;    // [nt1, NQ]  softmax (reference, sum) of each window row, log2 units
   float* ksum;        // [nt1, d]      sum of unit keys
   float4* vstat;      // [nt2]         (min, max, sum, -) of |V_i| over candidates
-  float4* dstat;      // [nt2, 2]      per epilogue warpgroup: (min, max, sum) of s_div, window-count-weighted sum of s_ex_raw
+  float4* dstat;      // [nt2, 2]      per pair of epilogue warpgroups: (min, max, sum) of s_div, window-count-weighted sum of s_ex_raw
   float* exsum;       // [H, pchunks_total]   per-chunk sum of pooled s_ex (max pooling only)
   float* rbar;        // [batch*H]   redundancy of Eq. 4, left by pass 2
   int* counts;        // [batch*H]

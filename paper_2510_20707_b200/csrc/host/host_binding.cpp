@@ -4,8 +4,8 @@
 //
 // Why it is native: a call of the library enqueues two to six kernels, and the smallest calls keep the
 // GPU busy for less time than interpreted marshalling takes.  Through ctypes one decode call cost 15 us of
-// host time for 7 us of GPU time and a scores + select pair 89 us; here they cost 5.5 and 24 us, one
-// layer's compression 8.6 us.  Output tensors come from torch's caching allocator without the dispatcher.
+// host time for 7 us of GPU time and a scores + select pair 89 us; here they cost 3.2 and 18 us, one
+// layer's compression 7.4 us, a similarity map 7.1 us.  Output tensors come from torch's caching allocator without the dispatcher.
 //
 // The interpreter lock is given up around everything that can block (Unlocked, below): a launch waits while the
 // stream's queue is full, an allocation may wait for the device, and a host callback on that stream, or any

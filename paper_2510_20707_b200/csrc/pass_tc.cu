@@ -4,7 +4,7 @@
 // tcgen05.ld.
 //
 //   pass 1  K from HBM.  Logits with the window queries on the M side (one query row per TMEM
-//           lane), so the running softmax (max, sum) of a row is thread-local; alongside, key
+//           lane), so the running softmax (reference, sum) of a row is thread-local; alongside, key
 //           norms and the sum of unit keys from the shared-memory tile.  Every run of tiles
 //           of one (layer, sequence, head) inside a CTA (a segment) leaves its partial
 //           statistics.
@@ -875,8 +875,8 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     // At the start of a segment: fold the unit-key sums of the head's pass-1 segments (one
     // dimension per thread) and write the bf16 hi / lo / lo2 split of the mean unit key into the
     // three extra B rows; the CTA that starts on the head's first tile also leaves the redundancy
-    // of Eq. 4, which needs nothing but the squared norm of that sum.  Per tile: warps 12, 13 read the first 64 rows of the V
-    // tile, warps 14, 15 the last 64; one row per thread from the swizzled half tile.
+    // of Eq. 4, which needs nothing but the squared norm of that sum.  Per tile: warps 20, 21 read the first 64 rows of the V
+    // tile, warps 22, 23 the last 64; one row per thread from the swizzled half tile.
     const int vt = tid - kP2AuxWarp0 * 32;         // 0..127
     const int sub = vt >> 6, vr = vt & 63;
     int vs = sub, vph = 0, segn = 0;   // V stage of this pair of warps: half tiles sub, sub + 2, ...

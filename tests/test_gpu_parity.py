@@ -225,15 +225,16 @@ def test_prefix_longer_than_the_tail_cache():
 
 
 @pytest.mark.parametrize("H,lens,levels", [
-    (8, (16400,) * 19, 3),        # one CTA per sequence, keys not cached, no candidate list
-    (8, (16400,) * 19, 1 << 20),  # one CTA per sequence, keys not cached, candidate list
-    (8, (60016,), 5),             # cluster of eight, keys not cached, no candidate list
-    (8, (60016,), 1 << 20),       # cluster of eight, keys not cached, candidate list
+    (8, (16400,) * 19, 3),        # clusters of four, keys cached, the threshold is one of three key values
+    (8, (16400,) * 19, 1 << 20),  # clusters of four, keys cached, candidates listed and ranked
+    (8, (13016,) * 40, 700),      # clusters of two, keys not cached
+    (8, (60016,), 5),             # cluster of eight, keys not cached, the threshold is one of five key values
+    (8, (60016,), 1 << 20),       # cluster of eight, keys not cached, candidates listed and ranked
 ])
 def test_adaptive_budgets_on_many_keys_are_exact(H, lens, levels):
     # adaptive budgets on caller-supplied scores are integer work: bit-identical to the oracle.
-    # These shapes hold more keys per CTA than its shared memory caches; with few score levels
-    # the bin left after the first digit pass is larger than the candidate list.
+    # With few score levels the bin of the threshold is one key value with more keys than the
+    # candidate list takes.
     W = 16
     rng = np.random.default_rng(levels % 97)
     cu = np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
@@ -250,11 +251,31 @@ def test_adaptive_budgets_on_many_keys_are_exact(H, lens, levels):
     assert np.array_equal(got["idx"].cpu().numpy()[:offs[-1]], ref["idx"])
 
 
+def test_adaptive_budgets_by_one_cta_on_keys_it_cannot_cache():
+    # 76 (layer, sequence) pairs of 64 heads x 810 keys: more pairs than clusters of two are resident, and more keys
+    # than a CTA caches.  On the call's own scores the selection is integer work: bit-identical to the oracle
+    NL, H, W, P, B = 76, 64, 16, 810, 116
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    rand = lambda *shape: torch.randn(shape, generator=gen, device="cuda", dtype=torch.bfloat16)
+    K, Q = rand(NL, H, P + W, 128), rand(NL, 1, H, W, 128)
+    pg = binding.Params(kv_heads=H, gqa_ratio=1, window=W, budget=B, budget_mode=1)
+    po = oracle.Params(kv_heads=H, gqa_ratio=1, window=W, budget=B, budget_mode=1)
+    out = binding.compress_layers(K, K, Q, pg)
+    torch.cuda.synchronize()
+    assert int(out["status"].item()) == 0
+    for layer in (0, 37, 75):
+        ref = oracle.select(out["s_comp"][layer].cpu().numpy(), po)
+        offs = out["idx_offsets"][layer].cpu().numpy()
+        assert np.array_equal(out["counts"][layer].cpu().numpy(), ref["counts"].reshape(-1))
+        assert np.array_equal(offs, ref["idx_offsets"])
+        assert np.array_equal(out["idx"][layer].cpu().numpy()[:offs[-1]], ref["idx"])
+
+
 @pytest.mark.parametrize("levels", [0, 50, 3000000])
 def test_whole_head_ctas_select_exactly(levels):
     # 80 (sequence, head) units of 20000 candidates: one 1024-thread CTA per unit with the keys
-    # in shared memory.  Few score levels leave more keys in the bin after two digits than the
-    # key list takes (the four-pass search), many levels a few hundred (the list), levels = 0
+    # in shared memory.  Few score levels leave more keys in the bin of the threshold than the list
+    # takes (binned again, down to one key value), many levels a few dozen (the list), levels = 0
     # real-valued scores; a head of equal scores and negative zeros ride along.  Integer work:
     # bit-identical to the oracle.
     H, B, W, P = 8, 10, 16, 20000
@@ -310,7 +331,8 @@ def test_threshold_search_edges(H, n, levels, want):
 @pytest.mark.parametrize("batch,H,P", [
     (1, 8, 1024), (1, 8, 1025),                                # one CTA per sequence, two
     (15, 8, 4100), (16, 8, 4100), (30, 8, 4100),               # clusters of eight, of four
-    (31, 8, 2100), (60, 8, 1030), (61, 8, 1030)])              # of two; one CTA
+    (31, 8, 2100), (60, 8, 1030), (61, 8, 1030),               # of four; of two
+    (33, 8, 4100), (34, 8, 4100), (64, 8, 1030)])              # the last of four, of two
 def test_adaptive_budget_cluster_edges(batch, H, P):
     # levels: ties at the global threshold, which go to the lower (head, position)
     W = 16
@@ -329,7 +351,7 @@ def test_adaptive_budget_cluster_edges(batch, H, P):
 
 
 def test_long_sequence_cluster_tail():
-    # 65536 keys per head: the cluster shape of the tail kernel with 16 positions per thread
+    # 65536 keys per head: clusters of eight with 8192 positions to a CTA
     wl = synth.small_workload(H=2, G=4, W=32, seq_lens=(65536,), pool_kernel=7, budget=512,
                               seed=31, centroids=32)
     run_layer_parity(wl, variant="calibrated")

@@ -33,8 +33,8 @@ def test_random_rows_with_shared_component(H, L, block):
 
 @pytest.mark.parametrize("H,L,block", [(2, 1000, 16), (1, 700, 4), (3, 300, 2), (2, 257, 1),
                                        (1, 130, 8), (2, 2049, 16), (1, 128, 1), (2, 391, 4)])
-def test_dense_route_small_maps(H, L, block):
-    # block = 1, 2, 4, 8, 16 takes the tensor-core route: ragged last tile and last block, a zero
+def test_small_maps_and_blocks(H, L, block):
+    # blocks of which a warp takes whole ones (1, 2, 4, 8, 16 rows): ragged last tile and last block, a zero
     # row, diagonal cells without the i == j pairs
     rng = np.random.default_rng(1000 * block + L)
     X = rng.standard_normal((H, L, 128)) + 0.8 * rng.standard_normal((H, 1, 128))
@@ -62,8 +62,8 @@ def test_block_and_tile_edges(H, L, block):
 
 
 @pytest.mark.parametrize("L,block", [(8192, 1), (32768, 16)])
-def test_dense_route_full_size_sampled(L, block):
-    # The dense map of the keys of two heads at full size.  The pairwise oracle needs the L x L
+def test_full_size_sampled(L, block):
+    # The map of the keys of two heads at full size.  The pairwise oracle needs the L x L
     # matrix in fp64, so it checks sampled 128-row tiles: a cell depends only on the rows of its
     # two blocks, and the oracle run on the rows of tiles a and b gives the cells of (a, a),
     # (a, b), (b, a), (b, b).  The whole map is checked for symmetry and range, its mean against
