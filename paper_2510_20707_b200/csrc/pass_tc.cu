@@ -53,16 +53,6 @@ __device__ __forceinline__ void raise(int* status, volatile int* abort) {
   if (status) atomicExch(status, MIXKV_ERR_TIMEOUT);
 }
 
-// After an abort: let the copies in flight land before the CTA (and its shared memory) goes
-// away.  `it` loads were issued into a ring of `stages` barriers.
-__device__ __forceinline__ void drain_ring(uint64_t* full, int stages, int it) {
-  for (int k = max(0, it - stages); k < it; ++k) {
-    const unsigned long long t0 = global_ns();
-    while (!mbar_try(&full[k % stages], (k / stages) & 1) && global_ns() - t0 < kWaitLimitNs) {
-    }
-  }
-}
-
 __device__ __forceinline__ f32x2 ex2_pair(f32x2 t2) {
   float a0, a1;
   unpack2(t2, a0, a1);

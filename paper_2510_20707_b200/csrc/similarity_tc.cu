@@ -165,7 +165,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
   if (warp == 0) {
     // -------------------------------------------------------------------- TMA producer
     if (lane == 0) {
-      int s = 0, ph = 1, rown = 0;
+      int s = 0, ph = 1, rown = 0, it = 0;
       bool ok = true;
       for (GramWalk<NT> w(T, per_head, lo, hi); w.valid() && ok; w.next()) {
         if (w.fresh) {
@@ -185,12 +185,12 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
           mbar_expect_tx(&bars->bfull[s], kBHalf);
           tma_load_3d(sB + s * kBHalf, &tmB, x / P * 64, w.I * 128 + w.c * NT, x % P * H + w.h, &bars->bfull[s]);
           if (++s == kGStages) s = 0, ph ^= 1;
+          ++it;
         }
       }
-      if (*abort) {   // let the copies in flight land before the shared memory goes away
-        const unsigned long long t0 = global_ns();
-        while (global_ns() - t0 < 20000ull) {
-        }
+      if (*abort) {
+        drain_ring(bars->bfull, kGStages, it);
+        drain_ring(&bars->afull, 1, rown);
       }
     }
   } else if (warp == 1) {
