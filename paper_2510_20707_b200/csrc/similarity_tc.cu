@@ -11,7 +11,7 @@
 // epilogue of a tile overlap the MMA of the next.
 //
 // What bounds it: the output, T x T x 4 bytes per head, once T is large: a tile and its mirror image leave
-// through shared memory as 16-byte stores of full 128-byte lines.
+// as stores of 128 consecutive bytes of a row.
 //
 // NT = 128 where there are tiles enough for every SM, NT = 32 below that: a small map is one chain
 // of load, MMA and store per CTA, and a quarter of the columns shortens all three.
@@ -293,29 +293,26 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
             v[j] = __float_as_uint(x);
           }
         }
-        // Both images go through a swizzled 32 x 32 tile in shared memory (cell (i, j) of the chunk at word
-        // 4 ((j / 4) ^ (i & 7)) + j % 4 of row i) and leave as 16-byte stores, four rows of 128 bytes per
-        // instruction; where the rows of the map are not 16-byte aligned (a caller's map need only be aligned to
-        // 4 bytes), or the chunk is cut by its edge, as 4-byte stores, one row per instruction.
+        // The mirrored tile leaves straight from the registers, where 32 lanes hold 128 consecutive bytes of a row of
+        // the map (turned in shared memory first, into 16-byte stores of four rows per instruction, 4 heads of 32768 rows
+        // in blocks of 16 took 32.2 us a call, now 31.4).  The tile itself goes through a swizzled 32 x 32 tile in shared
+        // memory (cell (i, j) of the chunk at word 4 ((j / 4) ^ (i & 7)) + j % 4 of row i) and leaves as 16-byte
+        // stores, four rows of 128 bytes per instruction; where the rows of the map are not 16-byte aligned (a
+        // caller's map need only be aligned to 4 bytes), or the chunk is cut by its edge, as 4-byte stores, one row
+        // per instruction.
         const bool vec = rows16 && i0 + 32 <= T && j0 + 32 <= T;
         const int sub = lane >> 3, quad = lane & 7;   // row of a group of four, four columns of it
         if (!on_diag) {   // mirrored tile: rows J
-          if (vec) {
-            __syncwarp();
+          if (i < T) {
+            float* p = out + (size_t)j0 * T + i;
+            if (j0 + 32 <= T) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-              st[j * 32 + 4 * ((lane >> 2) ^ (j & 7)) + (lane & 3)] = __uint_as_float(v[j]);
-            __syncwarp();
-            float* p = out + (size_t)(j0 + sub) * T + i0 + 4 * quad;
+              for (int j = 0; j < 32; ++j) p[(size_t)j * T] = __uint_as_float(v[j]);
+            } else {
 #pragma unroll
-            for (int r = 0; r < 32; r += 4)
-              *reinterpret_cast<float4*>(p + (size_t)r * T) =
-                  *reinterpret_cast<const float4*>(st + (r + sub) * 32 + 4 * (quad ^ ((r + sub) & 7)));
-          } else if (i < T) {
-            float* p = out + (size_t)j0 * T + i;   // straight from the registers
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (j0 + j < T) p[(size_t)j * T] = __uint_as_float(v[j]);
+              for (int j = 0; j < 32; ++j)
+                if (j0 + j < T) p[(size_t)j * T] = __uint_as_float(v[j]);
+            }
           }
         }
         // the tile itself: rows I
