@@ -41,37 +41,50 @@ __host__ __device__ __forceinline__ int row_tiles(const int T, const int I) {
   return (T - I * 128 + NT - 1) / NT;
 }
 
-// The tiles [lo, hi) of one CTA in (head, I, c) order; column tile c covers blocks I * 128 + c * NT ...
-template <int NT>
+// The tiles of one CTA, of `total` in (head, I, c) order; column tile c covers blocks I * 128 + c * NT ...  DEALT: runs of
+// `run` tiles, dealt out in turn, else one contiguous share (see gram_run).
+template <int NT, bool DEALT>
 struct GramWalk {
-  int id, hi, T, nT, h, I, c, nc;
+  int id, hi, T, nT, h, I, c, nc, run, left;
   bool fresh;   // first tile of this CTA in its (head, I): the parts of I have to be loaded
-  __device__ GramWalk(const int T_, const int per_head, const int lo, const int hi_)
-      : id(lo), hi(hi_), T(T_), nT((T_ + 127) / 128) {
-    fresh = true;
-    h = lo / per_head;
-    c = lo - h * per_head;
+  __device__ GramWalk(const int T_, const int per_head, const int total, const int run_)
+      : T(T_), nT((T_ + 127) / 128), run(run_), left(run_) {
+    id = DEALT ? (int)blockIdx.x * run : (int)((long long)total * blockIdx.x / gridDim.x);
+    hi = DEALT ? total : (int)((long long)total * (blockIdx.x + 1) / gridDim.x);
+    h = id / per_head;
+    c = id - h * per_head;
     I = 0;
     nc = row_tiles<NT>(T, 0);
-    while (c >= nc) {
-      c -= nc;
-      nc = row_tiles<NT>(T, ++I);
+    while (c >= nc) row();
+    fresh = true;
+  }
+  __device__ __forceinline__ void row() {   // c lies behind the end of row I
+    c -= nc;
+    fresh = true;
+    if (++I == nT) {
+      I = 0;
+      ++h;
     }
+    nc = row_tiles<NT>(T, I);
   }
   __device__ __forceinline__ bool valid() const { return id < hi; }
-  // the last tile of this CTA in its (head, I)
-  __device__ __forceinline__ bool row_last() const { return id + 1 == hi || c + 1 == nc; }
+  // after this tile the parts of I are loaded again, if there is another tile
+  __device__ __forceinline__ bool row_last() const { return id + 1 == hi || c + 1 == nc || (DEALT && left == 1); }
   __device__ __forceinline__ void next() {
-    ++id;
     fresh = false;
-    if (++c == nc) {
-      c = 0;
-      fresh = true;
-      if (++I == nT) {
-        I = 0;
-        ++h;
+    if (DEALT) {
+      int ahead = 1;
+      if (--left == 0) {
+        ahead += ((int)gridDim.x - 1) * run;
+        left = run;
+        fresh = true;
       }
-      nc = row_tiles<NT>(T, I);
+      id += ahead;
+      c += ahead;
+      while (c >= nc) row();
+    } else {
+      ++id;
+      if (++c == nc) row();
     }
   }
 };
@@ -115,11 +128,11 @@ __device__ void head_mean(const float* __restrict__ us, const int* __restrict__ 
   named_bar_sync(1, 64);
 }
 
-template <int P, int NT>
+template <int P, int NT, bool DEALT>
 __global__ void __launch_bounds__(kGThreads, 1)
 k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
        const int* __restrict__ nz, const float* __restrict__ us, const int* __restrict__ nzs,
-       const int slices, const int H, const int L, const int block, const int T, const int per_head,
+       const int slices, const int H, const int L, const int block, const int T, const int per_head, const int run,
        float* __restrict__ cells, float* __restrict__ mean) {
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* base =
@@ -132,8 +145,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
   __shared__ float4 half_sum[32];   // head means
   __shared__ int half_nz;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const long long total = (long long)H * per_head;
-  const int lo = (int)(total * blockIdx.x / gridDim.x), hi = (int)(total * (blockIdx.x + 1) / gridDim.x);
+  const GramWalk<NT, DEALT> walk(T, per_head, H * per_head, run);   // (divisions: ahead of the wait)
   volatile int* abort = &bars->abort;
 
   pdl_launch_dependents();
@@ -167,7 +179,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
     if (lane == 0) {
       int s = 0, ph = 1, rown = 0, it = 0;
       bool ok = true;
-      for (GramWalk<NT> w(T, per_head, lo, hi); w.valid() && ok; w.next()) {
+      for (GramWalk<NT, DEALT> w = walk; w.valid() && ok; w.next()) {
         if (w.fresh) {
           if (rown > 0 && !mbar_wait(&bars->afree, (rown - 1) & 1, abort)) break;
           mbar_expect_tx(&bars->afull, P * kPartBytes);
@@ -201,7 +213,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
       const uint32_t a0 = umma_desc_lo(smem_u32(sA)), b0 = umma_desc_lo(smem_u32(sB));
       int s = 0, ph = 0, rown = 0, tile = 0;
       bool ok = true;
-      for (GramWalk<NT> w(T, per_head, lo, hi); w.valid() && ok; w.next()) {
+      for (GramWalk<NT, DEALT> w = walk; w.valid() && ok; w.next()) {
         if (w.fresh) {
           if (!mbar_wait(&bars->afull, rown & 1, abort)) break;
           ++rown;
@@ -252,7 +264,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
     const float inv_b = 1.0f / (float)block, last_n = (float)(L - (T - 1) * block);
     const bool rows16 = (T & 3) == 0 && (reinterpret_cast<uintptr_t>(cells) & 15) == 0;
     int tile = 0;
-    for (GramWalk<NT> w(T, per_head, lo, hi); w.valid(); w.next()) {
+    for (GramWalk<NT, DEALT> w = walk; w.valid(); w.next()) {
       const int i0 = w.I * 128 + quarter * 32, i = i0 + lane;   // this thread's block I
       const bool last_i = i == T - 1;
       const float inv_i = last_i ? 1.0f / last_n : inv_b;
@@ -344,12 +356,27 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
   if (warp == 1) tmem_dealloc(tmem, 256);
 }
 
-template <int P, int NT>
-cudaError_t launch_gram_t(const GramArgs& g, const long long per_head, cudaStream_t s) {
+// How the tiles are shared out: 0 contiguous (a CTA keeps its parts of I from tile to tile), else runs of so many in turn,
+// so that all CTAs together write whole rows of the map at a time.  That counts where the map goes to HBM: it leaves L2
+// in about the order in which it was written.
+//   Rows that do not start on 32-byte sectors (T not a multiple of 8, or a map that does not): neighbouring tiles share
+//   sectors, and a sector that leaves half written is read again.  Runs of one, from a few dozen megabytes on: 8 heads
+//   x 2500 cells a side 89 -> 71 us, 4 x 2801 66 -> 55, 4 x 5001 211 -> 177, 8 x 1500 (72 MB) 35.1 -> 33.5.
+//   Whole sectors: only the largest maps gain (pages of HBM filled in one go): 4 x 8192 269 -> 211 us in runs of one (two
+//   parts), 2 x 8192 142 -> 134 and 4 x 5000 122 -> 112 in runs of two (three parts, where the parts of I weigh more);
+//   268 MB and less are as fast or up to 5 % faster contiguous.
+int gram_run(const void* cells, const int heads, const int T, const int nparts) {
+  const double mb = (double)heads * T * T * 4e-6;
+  if (T % 8 || (reinterpret_cast<uintptr_t>(cells) & 31)) return mb > 64. ? 1 : 0;
+  return mb > 300. ? (nparts == 2 ? 1 : 2) : 0;
+}
+
+template <int P, int NT, bool DEALT>
+cudaError_t launch_gram_t(const GramArgs& g, const long long per_head, const int run, cudaStream_t s) {
   static std::atomic<bool> done[kMaxDevices];
   const size_t smem = 1024 + (size_t)P * kPartBytes + (size_t)kGStages * NT * 128 +
                       (size_t)kGEpiWarps * 4096 + sizeof(GBars);
-  const cudaError_t e = ensure_smem(k_gram<P, NT>, smem, done);
+  const cudaError_t e = ensure_smem(k_gram<P, NT, DEALT>, smem, done);
   if (e != cudaSuccess) return e;
   const long long total = per_head * g.heads;
   if (total > 0x7fffffffLL) return cudaErrorInvalidValue;
@@ -363,8 +390,9 @@ cudaError_t launch_gram_t(const GramArgs& g, const long long per_head, cudaStrea
       !encode_bf16_map(&tmB, g.parts, 3, dims, strides, boxB))
     return cudaErrorInvalidValue;
   const int grid = (int)(total < device_sm_count() ? total : device_sm_count());
-  return launch_pdl(k_gram<P, NT>, dim3((unsigned)grid), dim3(kGThreads), smem, s, 1, tmA, tmB, g.nz, g.us,
-                    g.nzs, g.slices, g.heads, g.L, g.block, g.T, (int)per_head, g.cells, g.mean);
+  return launch_pdl(k_gram<P, NT, DEALT>, dim3((unsigned)grid), dim3(kGThreads), smem, s, 1, tmA, tmB, g.nz, g.us,
+                    g.nzs, g.slices, g.heads, g.L, g.block, g.T, (int)per_head,
+                    run, g.cells, g.mean);
 }
 
 template <int NT>
@@ -380,9 +408,14 @@ cudaError_t launch_gram(const GramArgs& g, cudaStream_t s) {
   const long long wide = tiles_per_head<128>(g.T);
   const bool narrow = wide * g.heads < device_sm_count();
   const long long per_head = narrow ? tiles_per_head<32>(g.T) : wide;
+  const int run = narrow ? 0 : gram_run(g.cells, g.heads, g.T, g.nparts);
   if (g.nparts == 2)
-    return narrow ? launch_gram_t<2, 32>(g, per_head, s) : launch_gram_t<2, 128>(g, per_head, s);
-  return narrow ? launch_gram_t<3, 32>(g, per_head, s) : launch_gram_t<3, 128>(g, per_head, s);
+    return narrow ? launch_gram_t<2, 32, false>(g, per_head, 0, s)
+           : run  ? launch_gram_t<2, 128, true>(g, per_head, run, s)
+                  : launch_gram_t<2, 128, false>(g, per_head, 0, s);
+  return narrow ? launch_gram_t<3, 32, false>(g, per_head, 0, s)
+         : run  ? launch_gram_t<3, 128, true>(g, per_head, run, s)
+                : launch_gram_t<3, 128, false>(g, per_head, 0, s);
 }
 
 }  // namespace mixkv

@@ -90,6 +90,32 @@ def test_full_size_sampled(L, block):
     assert np.allclose(mean.cpu().numpy(), rbar, rtol=RTOL, atol=ATOL)
 
 
+@pytest.mark.parametrize("H,L,block", [(2, 2899, 1), (1, 8195, 2), (1, 8704, 1), (1, 17408, 2), (2, 2827, 1)])
+def test_large_maps_in_dealt_runs(H, L, block):
+    # maps whose tiles are dealt to the CTAs in runs: of one where rows split sectors (67 MB), of one and of two where
+    # they do not (303 MB), and the last below that line; in fp64 with the identity that similarity_plain is pinned to
+    # (the mean of a cell is the product of the sums of unit rows), the whole map
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    X = (torch.randn((H, L, 128), generator=gen, device="cuda") + 0.9 *
+         torch.randn((H, 1, 128), generator=gen, device="cuda")).bfloat16()
+    cells, mean = binding.similarity_map(X, block)
+    for h in range(H):
+        u = X[h].double()
+        u = u / u.norm(dim=1, keepdim=True)
+        T = -(-L // block)
+        sums = torch.zeros((T * block, 128), dtype=torch.float64, device="cuda")
+        sums[:L] = u
+        sums = sums.view(T, block, 128).sum(1)
+        n = torch.full((T,), float(block), dtype=torch.float64, device="cuda")
+        n[-1] = L - (T - 1) * block
+        ref = (sums @ sums.T) / (n[:, None] * n[None, :])
+        pairs = n * (n - 1)
+        ref.diagonal().copy_(torch.where(pairs > 0, ((sums * sums).sum(1) - n) / pairs.clamp(min=1), 0.0))
+        assert torch.allclose(cells[h].double(), ref, rtol=RTOL, atol=ATOL)
+        total = u.sum(0)
+        assert abs(float(mean[h]) - float((total @ total - L) / (L * (L - 1.0)))) <= ATOL + RTOL * abs(float(mean[h]))
+
+
 def test_keys_and_values_of_a_c2_layer():
     wl = synth.CONFIGS["C2"]
     x = synth.make_layer(wl, 7, "calibrated")
