@@ -83,6 +83,7 @@ struct P1Bars {
   uint64_t tempty[4];
   uint64_t qfull;
   uint64_t qfree;
+  TileCoord first;   // of the CTA's first tile
   uint32_t tmem_base;
   int abort;
 };
@@ -137,10 +138,10 @@ __device__ __forceinline__ float fold_key_sums(const float* ksum, const SegList&
   }
   return sum;
 }
-// The pass-1 segments of the head that segment iterator `sg` of pass 2 stands on.
-__device__ __forceinline__ SegList pass1_segments(const SeqTable& st, const RevSegIter& sg) {
-  const int per_head = (st.tile1_start[sg.b + 1] - st.tile1_start[sg.b]) / st.H;
-  return SegList(sg.layer * st.nt1 + st.tile1_start[sg.b] + sg.h * per_head, per_head, split1(st));
+// The pass-1 segments of a head.
+__device__ __forceinline__ SegList pass1_segments(const SeqTable& st, const int layer, const int b, const int h) {
+  const int per_head = (st.tile1_start[b + 1] - st.tile1_start[b]) / st.H;
+  return SegList(layer * st.nt1 + st.tile1_start[b] + h * per_head, per_head, split1(st));
 }
 
 // The running softmax statistics of a query row are a pair (m, z): z = sum over the keys seen
@@ -252,6 +253,8 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     tma_prefetch_desc(&tmK);
     tma_prefetch_desc(&tmQ);
   }
+  // (divisions: once, ahead of the wait, instead of in every role behind it)
+  if (tid == kEpiWarp0 * 32) bars->first = layer_tile_coord(st.tile1_start, st.batch, H, st.nt1, lo);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -266,7 +269,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
       if (lane == 0) {
         int s = 0, ph = 1, it = 0, segn = 0;
         bool ok = true;
-        for (SegIter sg(st.tile1_start, st.batch, H, st.nt1, lo, hi); sg.valid() && ok; sg.next()) {
+        for (SegIter sg(st.tile1_start, st.batch, H, bars->first, lo, hi); sg.valid() && ok; sg.next()) {
           if (segn > 0 && !mbar_wait(&bars->qfree, (segn - 1) & 1, abort)) break;
           mbar_expect_tx(&bars->qfull, NQ * 256);
           tma_load_3d(sQ, &tmQ, 0, sg.bh() * NQ, sg.layer, &bars->qfull);
@@ -300,7 +303,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         const uint32_t q_half = (uint32_t)(NQ * 128) >> 4;   // second 64-column half of the queries
         int s = 0, ph = 0, ts = 0, tph = 1, segn = 0;
         bool ok = true;
-        for (SegIter sg(st.tile1_start, st.batch, H, st.nt1, lo, hi); sg.valid() && ok; sg.next()) {
+        for (SegIter sg(st.tile1_start, st.batch, H, bars->first, lo, hi); sg.valid() && ok; sg.next()) {
           if (!mbar_wait(&bars->qfull, segn & 1, abort)) break;
           ++segn;
           for (int k = 0; k < sg.n; ++k) {
@@ -356,7 +359,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     constexpr int kXThreads = NU * 128;
     int ts = 0, tph = 0, segs_done = 0;
     const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + col0;
-    for (SegIter sg(st.tile1_start, st.batch, H, st.nt1, lo, hi); sg.valid(); sg.next()) {
+    for (SegIter sg(st.tile1_start, st.batch, H, bars->first, lo, hi); sg.valid(); sg.next()) {
       float m_run = -1e30f, z_run = 0.f;
       const int P = st.cu[sg.b + 1] - st.cu[sg.b] - W;
       const int t_mask = P / kTile;   // first tile that holds keys some row may not see
@@ -441,7 +444,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     const uint32_t off1 = (uint32_t)(16 * aux_w + lg) * 128 + ((uint32_t)(c ^ (lg + 4)) << 4);
     const int my_row = 16 * aux_w + 4 * (c >> 1) + lg;   // the row whose norm this lane ends with
     int s = 0, ph = 0;
-    for (SegIter sg(st.tile1_start, st.batch, H, st.nt1, lo, hi); sg.valid(); sg.next()) {
+    for (SegIter sg(st.tile1_start, st.batch, H, bars->first, lo, hi); sg.valid(); sg.next()) {
       f32x2 acc2[8];   // dims 8c .. 8c+7 of half 0, then of half 1, as packed pairs
 #pragma unroll
       for (int e = 0; e < 8; ++e) acc2[e] = pack2(0.f, 0.f);
@@ -549,6 +552,8 @@ struct P2Bars {
   uint64_t qfull;
   uint64_t qfree;
   uint64_t kbready;
+  TileCoord last;   // of the CTA's last tile
+  SegList segs;     // pass 1's segments of the head that it belongs to
   uint32_t tmem_base;
   int abort;
 };
@@ -621,6 +626,11 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     tma_prefetch_desc(&tmQ);
   }
   if (warp == kWarpTmaV && lane == 0) tma_prefetch_desc(&tmV);
+  // (divisions: once, ahead of the wait, instead of in every role behind it)
+  if (tid == kEpiWarp0 * 32) {
+    bars->last = layer_tile_coord(st.tile2_start, st.batch, H, st.nt2, hi - 1);
+    bars->segs = pass1_segments(st, bars->last.layer, bars->last.b, bars->last.h);
+  }
   if (warp >= kP2AuxWarp0) {   // B rows past the three parts of the mean key stay zero
     const int vt = tid - kP2AuxWarp0 * 32;
     unsigned char* hb = sQ + (vt >> 6) * NB * 128 + (vt & 7) * 2;
@@ -640,7 +650,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
       const uint64_t policy = l2_evict_first();
       int s = 0, ph = 1, it = 0, segn = 0;
       bool ok = true;
-      for (RevSegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
+      for (RevSegIter sg(st.tile2_start, st.batch, H, bars->last, lo, hi); sg.valid() && ok; sg.next()) {
         if (segn > 0 && !mbar_wait(&bars->qfree, (segn - 1) & 1, abort)) break;
         mbar_expect_tx(&bars->qfull, NQ * 256);
         tma_load_3d(sQ, &tmQ, 0, sg.bh() * NQ, sg.layer, &bars->qfull);
@@ -670,7 +680,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
       const uint64_t policy = l2_evict_first();
       int vit = 0, vs = 0, vph = 1;
       bool ok = true;
-      for (RevSegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
+      for (RevSegIter sg(st.tile2_start, st.batch, H, bars->last, lo, hi); sg.valid() && ok; sg.next()) {
         int y = st.cu[sg.b] + (sg.end() - 1) * kTile;
         for (int k = 0; k < 2 * sg.n; ++k, y += (k & 1) ? 64 : -64 - kTile) {   // half tiles of 64 rows
           if (!mbar_wait(&bars->vempty[vs], vph, abort)) {
@@ -698,7 +708,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     const uint32_t q_half = (uint32_t)(NB * 128) >> 4;   // second 64-column half of the B operand
     int s = 0, ph = 0, ts = 0, tph = 1, segn = 0;
     bool ok = true;
-    for (RevSegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid() && ok; sg.next()) {
+    for (RevSegIter sg(st.tile2_start, st.batch, H, bars->last, lo, hi); sg.valid() && ok; sg.next()) {
       if (!mbar_wait(&bars->qfull, segn & 1, abort)) break;
       if (!mbar_wait(&bars->kbready, segn & 1, abort)) break;
       ++segn;
@@ -750,10 +760,10 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     const uint32_t tstage = tmem + ((uint32_t)(quarter * 32) << 16) + wg * 256, taddr = tstage + ch_lo * 16;
     const float* nb = sbq + ch_lo * 16;
     int tile = 0;   // parity decides which pair owns it
-    for (RevSegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid(); sg.next()) {
+    for (RevSegIter sg(st.tile2_start, st.batch, H, bars->last, lo, hi); sg.valid(); sg.next()) {
       const int P = st.cu[sg.b + 1] - st.cu[sg.b] - W;
       {
-        const SegList sl = pass1_segments(st, sg);
+        const SegList sl = tile == 0 ? bars->segs : pass1_segments(st, sg.layer, sg.b, sg.h);
         const int q = et & 255, mid = sl.nseg > kFoldRows ? (sl.nseg + 1) >> 1 : sl.nseg;
         float2 mz = make_float2(-1e30f, 0.f);
         if (q < NQ) {
@@ -870,9 +880,10 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     const int vt = tid - kP2AuxWarp0 * 32;         // 0..127
     const int sub = vt >> 6, vr = vt & 63;
     int vs = sub, vph = 0, segn = 0;   // V stage of this pair of warps: half tiles sub, sub + 2, ...
-    for (RevSegIter sg(st.tile2_start, st.batch, H, st.nt2, lo, hi); sg.valid(); sg.next()) {
+    for (RevSegIter sg(st.tile2_start, st.batch, H, bars->last, lo, hi); sg.valid(); sg.next()) {
       const int L = st.cu[sg.b + 1] - st.cu[sg.b], P = L - W;
-      const float ks = fold_key_sums(ws.ksum, pass1_segments(st, sg), vt);
+      const float ks =
+          fold_key_sums(ws.ksum, segn == 0 ? bars->segs : pass1_segments(st, sg.layer, sg.b, sg.h), vt);
       const float kb = ks / (float)L;   // mean unit key
       __nv_bfloat16 parts[3];
       parts[0] = __float2bfloat16_rn(kb);

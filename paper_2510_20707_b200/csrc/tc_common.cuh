@@ -254,7 +254,7 @@ __device__ __forceinline__ uint32_t sw128_offset(int r, int c) {
 // ---- persistent tile schedule shared by every role of a CTA ----------------------------
 // Tiles are 128 consecutive keys of one (sequence, head), numbered in (b, h, t) order.
 struct TileCoord {
-  int b, h, t, bh;
+  int b, h, t, layer, per_head;   // per_head: tiles of each head of sequence b
 };
 
 __device__ __forceinline__ TileCoord tile_coord(const int* tile_start, int batch, int H,
@@ -266,7 +266,15 @@ __device__ __forceinline__ TileCoord tile_coord(const int* tile_start, int batch
   c.b = b;
   c.h = rem / per_head;
   c.t = rem - c.h * per_head;
-  c.bh = b * H + c.h;
+  c.layer = 0;
+  c.per_head = per_head;
+  return c;
+}
+// The same for a tile id that runs over all layers, nt tiles each.
+__device__ __forceinline__ TileCoord layer_tile_coord(const int* tile_start, int batch, int H, int nt, int id) {
+  const int layer = id / nt;
+  TileCoord c = tile_coord(tile_start, batch, H, id - layer * nt);
+  c.layer = layer;
   return c;
 }
 __host__ __device__ __forceinline__ Split split1(const SeqTable& st) {
@@ -291,17 +299,11 @@ __host__ __device__ __forceinline__ int tile_owner(int t, const Split& sp) {
 struct SegIter {
   int id, hi, layer, b, h, t0, n, per_head, H, batch;
   const int* tile_start;
-  __device__ SegIter(const int* tile_start_, int batch_, int H_, int nt, int lo, int hi_)
-      : id(lo), hi(hi_), H(H_), batch(batch_), tile_start(tile_start_) {
-    layer = b = h = t0 = n = 0;
-    per_head = 1;
-    if (lo < hi_) {
-      layer = lo / nt;
-      const TileCoord c = tile_coord(tile_start_, batch_, H_, lo - layer * nt);
-      b = c.b, h = c.h, t0 = c.t;
-      per_head = (tile_start_[b + 1] - tile_start_[b]) / H_;
-      n = min(per_head - t0, hi_ - lo);
-    }
+  // first: of tile lo
+  __device__ SegIter(const int* tile_start_, int batch_, int H_, const TileCoord& first, int lo, int hi_)
+      : id(lo), hi(hi_), layer(first.layer), b(first.b), h(first.h), t0(first.t), per_head(first.per_head), H(H_),
+        batch(batch_), tile_start(tile_start_) {
+    n = min(per_head - t0, hi - id);
   }
   __device__ __forceinline__ bool valid() const { return id < hi; }
   // (sequence, head) of the segment inside its layer, and over all layers
@@ -328,15 +330,10 @@ struct SegIter {
 struct RevSegIter {
   int id, lo, left, layer, b, h, t0, n, H, batch;
   const int* tile_start;
-  __device__ RevSegIter(const int* tile_start_, int batch_, int H_, int nt, int lo_, int hi)
-      : lo(lo_), left(hi), H(H_), batch(batch_), tile_start(tile_start_) {
-    layer = b = h = t0 = n = id = 0;
-    if (lo_ < hi) {
-      layer = (hi - 1) / nt;
-      const TileCoord c = tile_coord(tile_start_, batch_, H_, hi - 1 - layer * nt);
-      b = c.b, h = c.h;
-      set(c.t + 1);
-    }
+  // last: of tile hi - 1
+  __device__ RevSegIter(const int* tile_start_, int batch_, int H_, const TileCoord& last, int lo_, int hi)
+      : lo(lo_), left(hi), layer(last.layer), b(last.b), h(last.h), H(H_), batch(batch_), tile_start(tile_start_) {
+    set(last.t + 1);
   }
   __device__ __forceinline__ void set(int end) {   // the segment ends before tile `end` of its head
     n = min(end, left - lo);
@@ -366,6 +363,7 @@ struct RevSegIter {
 struct SegList {
   int T0, c0, nseg;
   Split sp;
+  SegList() = default;
   __device__ SegList(int T0_, int per_head, const Split& sp_) : T0(T0_), sp(sp_) {
     c0 = tile_owner(T0_, sp_);
     nseg = tile_owner(T0_ + per_head - 1, sp_) - c0 + 1;
