@@ -200,7 +200,8 @@ int enqueue_select(const LaunchCtx& c, const float* scores, int* counts, TailArg
   t.scores = scores;
   t.counts_dev = nullptr;
   t.counts_out = counts;
-  if (c.p.budget_mode == MIXKV_BUDGET_ADAPTIVE) {
+  t.adapt = !c.n_trace_events && tail_adapts(c);
+  if (c.p.budget_mode == MIXKV_BUDGET_ADAPTIVE && !t.adapt) {
     c.mark();
     if (launch_budget(c, scores, counts) != cudaSuccess) return MIXKV_ERR_CUDA;
     t.counts_dev = counts;
@@ -381,8 +382,10 @@ int compress_impl(const void* K, const void* V, const void* Qwin, int n_layers,
   }
   rc = enqueue_passes(c, K, V, Qwin, c.ws.s_div, nullptr, status_dev);
   if (rc != MIXKV_OK) return rc;
-  if (p->budget_mode == MIXKV_BUDGET_FIXED && tail_can_fuse(c)) {
-    // one kernel: mix, select, gather
+  // (a traced call keeps the stages of adaptive budgets apart)
+  t.adapt = !c.n_trace_events && tail_adapts(c);
+  if (t.adapt || (p->budget_mode == MIXKV_BUDGET_FIXED && tail_can_fuse(c))) {
+    // one kernel: mix, (budgets,) select, gather
     t.s_div = c.ws.s_div;
     t.rbar_in = rbar_in_opt;
     t.s_comp_out = s_comp_opt;   // nobody else reads the mixed scores

@@ -190,12 +190,17 @@ struct TailArgs {
   void* K_out;
   void* V_out;
   int* status_clear;   // optional word set to 0
+  bool adapt;          // adaptive budgets shared out by this kernel (tail_adapts)
 };
 // counts [layers, batch*H] <- candidates to select for budgets [layers, batch*H] given by the caller
 cudaError_t launch_given_budgets(const LaunchCtx& c, const int* budgets, int* counts);
 cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& a);
 // Whether the longest sequence is short enough for the fused mix + select + gather kernel.
 bool tail_can_fuse(const LaunchCtx& c);
+// Whether that kernel can share adaptive budgets out itself: the heads of a sequence make a cluster, every head's
+// candidates fit one CTA, and even a head that got all shared rows would not run out of candidates (the rows of a
+// sequence are then known without looking at the others).
+bool tail_adapts(const LaunchCtx& c);
 
 // Launch with programmatic dependent launch (and an optional cluster size): the kernel may
 // start while its predecessor in the stream drains; every kernel calls pdl_wait() before it

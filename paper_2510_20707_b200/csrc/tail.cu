@@ -6,6 +6,7 @@
 // copies the kept K / V rows.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <type_traits>
 
 #include "internal_api.h"
@@ -667,6 +668,7 @@ struct TailKernelArgs {
   __nv_bfloat16* K_out;
   __nv_bfloat16* V_out;
   int Bp;                     // B - W
+  int floor_slots;            // ADAPT: rows that every head gets
   int cached;                 // keys of the slice fit the shared-memory cache
   long long kv_layer_stride;  // elements between consecutive layers of K (V)
   int idx_cap;                // index-list entries reserved per layer
@@ -692,7 +694,10 @@ __device__ __forceinline__ int fixed_offset(const SeqTable& st, int bh, int Bp) 
 // raw keys and a position per thread and step in the mix); 896 heads of 2 to 7 thousand candidates (selection and
 // gather only): 47 us (119).
 // CL: launched as a cluster (else one CTA per unit, and none of the cluster's code is there to be stepped over).
-template <bool FUSED, int T, bool CL>
+// ADAPT: a cluster is the heads of a sequence, a CTA each, and shares the sequence's budget out first (the rule of
+// k_budget, from the keys that the CTAs hold anyway): a search across the cluster, then every CTA its own.  It stands for
+// mix, budget and tail kernels that each read again what the one before wrote, where tail_adapts says so.
+template <bool FUSED, int T, bool CL, bool ADAPT>
 __global__ void __launch_bounds__(T, 1024 / T)
 k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   extern __shared__ __align__(16) unsigned char tail_smem[];
@@ -700,9 +705,10 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   __shared__ int s_off, s_want;
   __shared__ float sc[8];
   __shared__ int s_rows[kTailRowCap];
+  __shared__ int s_gt[32], s_eq[32];   // (ADAPT)
   cg::cluster_group cluster = cg::this_cluster();
-  const int crank = CL ? (int)cluster.block_rank() : 0;
-  const int cs = CL ? (int)cluster.num_blocks() : 1;
+  const int crank = CL && !ADAPT ? (int)cluster.block_rank() : 0;   // (in ADAPT a unit is one CTA's)
+  const int cs = CL && !ADAPT ? (int)cluster.num_blocks() : 1;
   const int BH = st.batch * st.H;
   const int unit = blockIdx.x / cs;                    // (layer, sequence, head)
   const int layer = unit / BH, bh = unit % BH, b = bh / st.H, h = bh % st.H;
@@ -744,7 +750,7 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
       off = fixed_off;
       cnt = min(a.Bp, P);
     }
-    if (lane == 0) {
+    if (lane == 0 && !ADAPT) {
       s_off = off;
       s_want = cnt;
       if (crank == 0) {
@@ -873,8 +879,49 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
     }
   }
   __syncthreads();
-  const int want = s_want;
   auto key_at = [&](int j) -> unsigned { return cached ? skeys[j] : order_key(a.scores[poff + c0 + j]); };
+  if constexpr (ADAPT) {
+    // ---- this head's share: the floor, and the keys among the H * (Bp - floor) largest of all heads (equal ones to the
+    // lower head, then position).  No head can run out of candidates (tail_adapts), so a sequence fills H * Bp rows.
+    const int rank = (int)cluster.block_rank(), H = st.H;
+    const int N = H * (a.Bp - a.floor_slots);
+    int share = 0;
+    if (N > 0) {
+      const Threshold th = threshold_search<T>(key_at, [](int) {}, n, N, klo, khi, sm, cluster, H, rank);
+      int gt = 0, eq = 0;
+      for (int j = tid; j < n; j += T) {
+        const unsigned key = key_at(j);
+        gt += key > th.tau;
+        eq += key == th.tau;
+      }
+      gt = __reduce_add_sync(0xffffffffu, gt);
+      eq = __reduce_add_sync(0xffffffffu, eq);
+      if (lane == 0) s_gt[warp] = gt, s_eq[warp] = eq;
+      __syncthreads();
+      gt = __reduce_add_sync(0xffffffffu, lane < T / 32 ? s_gt[lane] : 0);
+      eq = __reduce_add_sync(0xffffffffu, lane < T / 32 ? s_eq[lane] : 0);
+      share = gt + max(0, min(eq, th.need_eq - th.eq_before));
+    }
+    if (tid == 0) s_want = a.floor_slots + share;
+    cluster.sync();   // the shares are there, and nobody reads another's search any more
+    const int mine = lane < H ? *cluster.map_shared_rank(&s_want, lane) : 0;
+    const int off = b * H * a.Bp + __reduce_add_sync(0xffffffffu, lane < rank ? mine : 0);
+    const int cnt = a.floor_slots + share;
+    if (tid == 0) {
+      s_off = off;
+      idx_offsets[bh] = off;
+      if (counts_out) counts_out[bh] = cnt;
+      if (out_row_offsets) out_row_offsets[bh] = off + bh * W;
+      if (bh == BH - 1) {
+        idx_offsets[BH] = off + cnt;
+        if (out_row_offsets) out_row_offsets[BH] = off + cnt + BH * W;
+      }
+    }
+    cluster.barrier_arrive();   // past this CTA's last remote read
+    for (int t = tid; t < 2 * kSelBins; t += T) (&sm.hist[0][0])[t] = 0;   // for this head's own search
+    __syncthreads();
+  }
+  const int want = s_want;
 
   int kept = 0, before = 0;   // positions this CTA keeps, and the CTAs of lower rank
   if (want >= P) {            // every candidate
@@ -982,6 +1029,7 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   }
   // a CTA's shared memory stays alive until its peers have read it
   if (cs > 1 && want > 0 && want < P) cluster.barrier_wait();
+  if constexpr (ADAPT) cluster.barrier_wait();
 }
 
 int floor_slots(const mixkv_params& p) {
@@ -1044,8 +1092,8 @@ namespace {
 int alone_clusters(const int size) {
   static std::atomic<bool> done[kMaxDevices];
   static ClusterFit fit;
-  (void)ensure_smem(k_tail<true, 1024, true>, kTailSmem, done);   // (a failure shows at the launch)
-  return fit.ask(k_tail<true, 1024, true>, 1024, 120 * 1024, size);
+  (void)ensure_smem(k_tail<true, 1024, true, false>, kTailSmem, done);   // (a failure shows at the launch)
+  return fit.ask(k_tail<true, 1024, true, false>, 1024, 120 * 1024, size);
 }
 
 // CTAs per (sequence, layer) pair: one while it has 8192 keys or less of all heads (the exchanges cost as much as
@@ -1097,13 +1145,14 @@ int tail_clusters(const long long units, const int P, const int sms, const Fit& 
   return cs;
 }
 
-TailShape tail_shape(const LaunchCtx& c) {
+// fixed_cs: so many CTAs per unit, 0: as many as the rules say.
+TailShape tail_shape(const LaunchCtx& c, const int fixed_cs = 0) {
   const long long units = (long long)c.st.layers * c.st.batch * c.st.H;
   const int P = c.max_prefix, sms = device_sm_count();
   TailShape t;
-  t.cs = tail_clusters(units, P, sms, alone_clusters);
+  t.cs = fixed_cs ? fixed_cs : tail_clusters(units, P, sms, alone_clusters);
   // What does not fit shared memory in that many CTAs takes more of them.
-  while (t.cs < kTailMaxCluster && tail_chunk(P, t.cs) > kTailCacheCap) t.cs *= 2;
+  while (!fixed_cs && t.cs < kTailMaxCluster && tail_chunk(P, t.cs) > kTailCacheCap) t.cs *= 2;
   t.chunk = tail_chunk(P, t.cs);
   // A CTA alone on its SM: 1024 threads (a block of 4096 positions), fewer when the slice is shorter.  More
   // CTAs than SMs: smaller ones side by side, as many as there are and as shared memory holds (heads of
@@ -1120,16 +1169,32 @@ TailShape tail_shape(const LaunchCtx& c) {
 
 bool tail_can_fuse(const LaunchCtx& c) { return tail_shape(c).cached; }
 
-template <bool FUSED, int T, bool CL>
+// Where it pays: whole calls, mix, budget and tail kernels against this, us.  One layer: 4 heads of 4096 keys 42.8 / 32.4,
+// eight ragged sequences of 4 heads of 2 to 7 thousand 60.9 / 51.4, 8 heads of 9000 57.1 / 47.3, of 20000 (four sequences)
+// 114 / 106; longer heads want more than a CTA each: 4 of 32768 67.1 / 67.3, 2 of 40000 62.4 / 68.3.  More CTAs than
+// are resident together lose what the launches cost: 128 units 109 / 100, 224 135 / 132, 240 299 / 292, 288 206 / 211,
+// 896 (28 layers x 8 ragged sequences) 889 / 924.
+constexpr int kAdaptMaxKeys = 24576;
+bool tail_adapts(const LaunchCtx& c) {
+  const int H = c.st.H, Bp = c.p.budget - c.p.window, f = floor_slots(c.p);
+  if (c.p.budget_mode != MIXKV_BUDGET_ADAPTIVE || H < 2 || H > kMaxCluster || c.max_prefix > kAdaptMaxKeys) return false;
+  if ((long long)c.st.layers * c.st.batch * H > device_sm_count() * 13LL / 8) return false;
+  int shortest = c.max_prefix;
+  for (int b = 0; b < c.st.batch; ++b) shortest = std::min(shortest, c.st.cu[b + 1] - c.st.cu[b] - c.st.W);
+  if ((long long)f + (long long)H * (Bp - f) > shortest) return false;
+  return tail_shape(c, 1).cached;
+}
+
+template <bool FUSED, int T, bool CL, bool ADAPT>
 cudaError_t launch_tail_t(const LaunchCtx& c, const TailKernelArgs& a, const TailShape& sh,
                           size_t smem) {
   if (smem > 20 * 1024) {   // on top of the static part
     static std::atomic<bool> done[kMaxDevices];
-    const cudaError_t e = ensure_smem(k_tail<FUSED, T, CL>, kTailSmem, done);
+    const cudaError_t e = ensure_smem(k_tail<FUSED, T, CL, ADAPT>, kTailSmem, done);
     if (e != cudaSuccess) return e;
   }
   const dim3 grid(c.st.layers * c.st.batch * c.st.H * sh.cs);
-  return launch_pdl(k_tail<FUSED, T, CL>, grid, dim3(T), smem, c.stream, sh.cs, c.st, c.ws, a);
+  return launch_pdl(k_tail<FUSED, T, CL, ADAPT>, grid, dim3(T), smem, c.stream, ADAPT ? c.st.H : sh.cs, c.st, c.ws, a);
 }
 
 cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
@@ -1148,12 +1213,13 @@ cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
   a.K_out = (__nv_bfloat16*)t.K_out;
   a.V_out = (__nv_bfloat16*)t.V_out;
   a.Bp = c.p.budget - c.p.window;
+  a.floor_slots = floor_slots(c.p);
   a.kv_layer_stride = c.kv_layer_stride;
   a.idx_cap = c.idx_cap;
   a.out_rows_cap = c.out_rows_cap;
   a.status_clear = t.status_clear;
   a.mp = mix_params(c.p);
-  const TailShape sh = tail_shape(c);
+  const TailShape sh = tail_shape(c, t.adapt ? 1 : 0);
   const bool fused = t.scores == nullptr;
   a.cached = sh.cached ? 1 : 0;
   if (fused && !a.cached) return cudaErrorInvalidValue;   // callers check tail_can_fuse() first
@@ -1163,8 +1229,11 @@ cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
   if (fused) smem += ((size_t)8 * sh.threads + 64) * 4;
   auto launch = [&](auto threads) {
     constexpr int T = decltype(threads)::value;
-    if (sh.cs > 1) return fused ? launch_tail_t<true, T, true>(c, a, sh, smem) : launch_tail_t<false, T, true>(c, a, sh, smem);
-    return fused ? launch_tail_t<true, T, false>(c, a, sh, smem) : launch_tail_t<false, T, false>(c, a, sh, smem);
+    if (t.adapt)
+      return fused ? launch_tail_t<true, T, true, true>(c, a, sh, smem) : launch_tail_t<false, T, true, true>(c, a, sh, smem);
+    if (sh.cs > 1)
+      return fused ? launch_tail_t<true, T, true, false>(c, a, sh, smem) : launch_tail_t<false, T, true, false>(c, a, sh, smem);
+    return fused ? launch_tail_t<true, T, false, false>(c, a, sh, smem) : launch_tail_t<false, T, false, false>(c, a, sh, smem);
   };
   switch (sh.threads) {
     case 256: return launch(std::integral_constant<int, 256>());

@@ -251,6 +251,29 @@ def test_adaptive_budgets_on_many_keys_are_exact(H, lens, levels):
     assert np.array_equal(got["idx"].cpu().numpy()[:offs[-1]], ref["idx"])
 
 
+@pytest.mark.parametrize("H,lens,Bp,ada_floor,levels", [
+    (3, (130,), 50, 0.2, 7), (3, (129,), 50, 0.2, 7),          # 10 + 3 * 40 = 130: a head cannot, and could, run out
+    (2, (1500, 900, 3001), 64, 0.2, 1 << 20), (5, (700, 2600), 96, 0.2, 4), (8, (12007, 1291), 144, 0.2, 1 << 20),
+    (4, (5000, 901), 80, 1.0, 50), (4, (5000, 901), 80, 0.0, 1), (7, (24576,), 300, 0.3, 900), (6, (24577,), 300, 0.3, 900)])
+def test_adaptive_budgets_shared_out_by_the_selection_are_exact(H, lens, Bp, ada_floor, levels):
+    # the heads of a sequence as a cluster that shares its budget out before each head selects: at the edges of the
+    # rule that takes it (candidates of the shortest sequence, keys of the longest), nothing to share, nothing but
+    # shared rows, scores that are all equal; integer work on caller-supplied scores, bit-identical to the oracle
+    W = 16
+    rng = np.random.default_rng(H * 1000 + Bp)
+    cu = np.concatenate([[0], np.cumsum([n + W for n in lens])]).astype(np.int32)
+    Ptot = int(cu[-1]) - len(lens) * W
+    s = (rng.integers(0, levels, size=(H, Ptot)) / np.float32(levels) - 0.25).astype(np.float32)
+    kw = dict(kv_heads=H, gqa_ratio=1, window=W, budget=W + Bp, budget_mode=1, ada_floor=ada_floor)
+    many = [int(c) for c in cu] if len(lens) > 1 else None
+    ref = oracle.select(s, oracle.Params(**kw), cu=cu if many else None)
+    got = binding.select(torch.from_numpy(s).cuda(), binding.Params(**kw), cu_seqlens=many)
+    offs = got["idx_offsets"].cpu().numpy()
+    assert np.array_equal(got["counts"].cpu().numpy(), ref["counts"].reshape(-1))
+    assert np.array_equal(offs, ref["idx_offsets"])
+    assert np.array_equal(got["idx"].cpu().numpy()[:offs[-1]], ref["idx"])
+
+
 def test_adaptive_budgets_by_one_cta_on_keys_it_cannot_cache():
     # 76 (layer, sequence) pairs of 64 heads x 810 keys: more pairs than clusters of two are resident, and more keys
     # than a CTA caches.  On the call's own scores the selection is integer work: bit-identical to the oracle
