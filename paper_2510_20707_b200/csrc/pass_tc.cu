@@ -1021,34 +1021,46 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
+// Fills a map of a bf16 tensor: dims innermost first, strides in bytes of dimensions 1 .. rank - 1, box extents; 128-byte
+// swizzle, zero fill outside.  The driver wants a current context for it.  The first call of a thread may find none (the
+// runtime binds the device's context when a call of its own needs it, and none has by then): bound here.
+bool encode_map(CUtensorMap* tm, const void* base, const cuuint32_t rank, const cuuint64_t* dims,
+                const cuuint64_t* strides, const cuuint32_t* box) {
+  EncodeTiledFn enc = encode_fn();
+  if (!enc) return false;
+  const cuuint32_t es[5] = {1, 1, 1, 1, 1};
+  auto fill = [&]() {
+    return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), dims, strides, box, es,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = fill();
+  if (r == CUDA_ERROR_INVALID_CONTEXT || r == CUDA_ERROR_NOT_INITIALIZED) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess) return false;
+    r = fill();
+  }
+  return r == CUDA_SUCCESS;
+}
+
 // X [layers, H, Ltot, d] bf16 (layer stride given in elements) as a 4-D tensor (d, Ltot, H,
 // layers) with boxes of 64 x rows x 1 x 1.  Rows past the end of the tensor read as zero.
 bool map_kv(const LaunchCtx& c, const void* X, int box_rows, CUtensorMap* tm) {
-  EncodeTiledFn enc = encode_fn();
-  if (!enc) return false;
-  cuuint64_t dims[4] = {(cuuint64_t)kHeadDim, (cuuint64_t)c.st.Ltot, (cuuint64_t)c.st.H,
-                        (cuuint64_t)c.st.layers};
-  cuuint64_t strides[3] = {(cuuint64_t)kHeadDim * 2, (cuuint64_t)c.st.Ltot * kHeadDim * 2,
-                           (cuuint64_t)c.kv_layer_stride * 2};
-  cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 1, 1};
-  cuuint32_t es[4] = {1, 1, 1, 1};
-  return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(X), dims, strides, box, es,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const cuuint64_t dims[4] = {(cuuint64_t)kHeadDim, (cuuint64_t)c.st.Ltot, (cuuint64_t)c.st.H,
+                              (cuuint64_t)c.st.layers};
+  const cuuint64_t strides[3] = {(cuuint64_t)kHeadDim * 2, (cuuint64_t)c.st.Ltot * kHeadDim * 2,
+                                 (cuuint64_t)c.kv_layer_stride * 2};
+  const cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 1, 1};
+  return encode_map(tm, X, 4, dims, strides, box);
 }
 
 // Q [layers, batch * H * NQ, d] bf16 as a 3-D tensor (d, rows, layers) with boxes of 64 x NQ x 1.
 bool map_q(const LaunchCtx& c, const void* Q, CUtensorMap* tm) {
-  EncodeTiledFn enc = encode_fn();
-  if (!enc) return false;
-  cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)c.st.batch * c.st.H * c.st.NQ,
-                        (cuuint64_t)c.st.layers};
-  cuuint64_t strides[2] = {(cuuint64_t)kHeadDim * 2, (cuuint64_t)c.q_layer_stride * 2};
-  cuuint32_t box[3] = {64, (cuuint32_t)c.st.NQ, 1};
-  cuuint32_t es[3] = {1, 1, 1};
-  return enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(Q), dims, strides, box, es,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const cuuint64_t dims[3] = {(cuuint64_t)kHeadDim, (cuuint64_t)c.st.batch * c.st.H * c.st.NQ,
+                              (cuuint64_t)c.st.layers};
+  const cuuint64_t strides[2] = {(cuuint64_t)kHeadDim * 2, (cuuint64_t)c.q_layer_stride * 2};
+  const cuuint32_t box[3] = {64, (cuuint32_t)c.st.NQ, 1};
+  return encode_map(tm, Q, 3, dims, strides, box);
 }
 
 // Dynamic shared memory of the passes: what the kernels carve up, behind up to 1023 bytes that align its start.
@@ -1078,16 +1090,11 @@ static_assert(passes_fit(), "a pass asks for more shared memory than a CTA may h
 
 bool encode_bf16_map(void* tm, const void* base, int rank, const unsigned long long* dims,
                      const unsigned long long* strides_bytes, const unsigned* box) {
-  EncodeTiledFn enc = encode_fn();
-  if (!enc) return false;
   cuuint64_t d[5], st[4];
-  cuuint32_t bx[5], es[5];
-  for (int i = 0; i < rank; ++i) d[i] = dims[i], bx[i] = box[i], es[i] = 1;
+  cuuint32_t bx[5];
+  for (int i = 0; i < rank; ++i) d[i] = dims[i], bx[i] = box[i];
   for (int i = 0; i + 1 < rank; ++i) st[i] = strides_bytes[i];
-  return enc(reinterpret_cast<CUtensorMap*>(tm), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank,
-             const_cast<void*>(base), d, st, bx, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
-             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  return encode_map(reinterpret_cast<CUtensorMap*>(tm), base, (cuuint32_t)rank, d, st, bx);
 }
 
 int device_sm_count() {

@@ -24,3 +24,9 @@ def pytest_collection_modifyitems(config, items):
     for item in items:
         if "gpu" in item.keywords:
             item.add_marker(skip)
+
+
+@pytest.fixture(scope="session")
+def fake_cuda(tmp_path_factory):
+    from fake_cuda import FakeCuda
+    return FakeCuda(str(tmp_path_factory.mktemp("fake_cuda")))

@@ -173,3 +173,37 @@ def test_what_a_call_allocates_belongs_to_its_stream():
         if isinstance(out, dict) and "s_comp" in out:
             assert torch.equal(out["s_comp"].view_as(ref), ref) and own >= need
         del out
+
+
+@pytest.mark.gpu
+def test_the_first_cuda_call_of_a_thread():
+    # a thread that has made no other CUDA call has no context bound to it, and a call that allocates nothing does not
+    # get one from the allocator either
+    import torch
+    from paper_2510_20707_b200 import binding
+    K, Q = torch.randn((4, 1000, 128), device="cuda").bfloat16(), torch.randn((1, 16, 32, 128), device="cuda").bfloat16()
+    p = binding.Params(kv_heads=4, gqa_ratio=4, budget=96)
+    ws = torch.empty(binding.workspace_size(p, 1, 1000, 1000), dtype=torch.uint8, device="cuda")
+    out = binding.compress_layer(K, K, Q, p, workspace=ws, want_aux=False)
+    s = binding.scores(K, K, Q, p)["s_comp"]
+    offs, q = torch.tensor([[0, 1000]], dtype=torch.int32, device="cuda"), torch.zeros((1, 1, 4, 128), device="cuda").bfloat16()
+    calls = [lambda: binding.compress_layer(K, K, Q, p, workspace=ws, out=out),
+             lambda: binding.scores(K, K, Q, p, workspace=ws), lambda: binding.scores_static(K, K, Q, p),
+             lambda: binding.select(s, p, workspace=ws), lambda: binding.similarity_map(K, 16),
+             lambda: binding.decode_attention(K[:1], K[:1], offs, q, 1, 4, 1000)]
+    found = []
+
+    def thread(call):
+        try:
+            call()
+            found.append(True)
+        except Exception as e:
+            found.append(e)
+
+    for call in calls:
+        call()                  # what is looked up once per device has been
+        t = threading.Thread(target=thread, args=(call,))
+        t.start()
+        t.join()
+    torch.cuda.synchronize()
+    assert found == [True] * len(calls), found
