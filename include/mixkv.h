@@ -16,8 +16,10 @@
  *    state kept between calls is limited to per-device caches of attributes (SM count,
  *    compute capability, shared-memory opt-in, clusters resident at once).  The workspace needs no initialisation
  *    and no clearing between calls (every word a kernel reads was written earlier in the
- *    same call; nothing is counted across CTAs), and may be reused for other shapes; two
- *    calls that may overlap in time need a workspace each.
+ *    same call; nothing is counted across CTAs), and may be reused for other shapes.  It belongs
+ *    to one call at a time: calls whose kernels may overlap on the GPU need one each, and so do calls that
+ *    several host threads make at once, on one stream even (a call enqueues several kernels, and those of
+ *    another thread's call may come between them; mixkv_scores_static takes care of that itself).
  *  - Shapes.  H = kv_heads, G = gqa_ratio, d = head_dim (128), W = window.
  *      K, V      [H, Ltot, d] bf16, row-major.  Ltot = L for one sequence, else
  *                cu_seqlens_host[batch]; sequence b owns rows cu[b] .. cu[b+1]-1.
@@ -145,7 +147,9 @@ int mixkv_scores(const void* K, const void* V, const void* Qwin,
  *  - All calls on one device share the one array, and it keeps whatever the previous call
  *    left in it.  Nothing in it needs to start from zero (every cell is written before it is
  *    read inside a call), but two calls whose kernels overlap on the GPU (different streams
- *    without an ordering between them) race on it: order such calls yourself.
+ *    without an ordering between them) race on it: order such calls yourself.  Several host threads
+ *    may call at once: the kernels of one call are enqueued together, and a call waits on the host
+ *    while another thread's is being enqueued on that device.
  * Arguments are those of mixkv_scores without workspace / workspace_bytes. */
 #define MIXKV_STATIC_SCRATCH_BYTES (12u << 20)
 int mixkv_scores_static(const void* K, const void* V, const void* Qwin,

@@ -11,6 +11,9 @@ The calls that enqueue work go through the native module ``_mixkv_host``
 name but for :func:`scores`, :func:`scores_static` and :func:`select`, which take the variants of
 ``csrc/internal_api.h`` (the call itself clears the status word it hands out), and
 :func:`compress_layer`, which is ``mixkv_compress_layer_traced`` with no events.
+
+The calls may be made by several threads at once (the interpreter lock is given up inside them); a
+``workspace`` then belongs to one of them at a time, on one stream too.
 """
 from __future__ import annotations
 
@@ -234,7 +237,8 @@ def scores_static(K: torch.Tensor, V: Optional[torch.Tensor], Q: torch.Tensor, p
     array, see MIXKV_STATIC_SCRATCH_BYTES in the header), so this function hands over inputs
     and outputs only; the output tensors below are the caller's, as in :func:`scores`.
     Raises MixKVError (status -6) when the problem is too large for the built-in array.
-    Calls on one device share that array: do not let two of them overlap on the GPU."""
+    Calls on one device share that array: do not let two of them overlap on the GPU (several
+    threads may call with one stream)."""
     return (_host_module or _host()).scores(K, V, Q, params, cu_seqlens, rbar_in, None, stream, True,
                                             True)
 

@@ -504,27 +504,20 @@ int mixkv_compress_layer(const void* K, const void* V, const void* Qwin,
 static __device__ __align__(256) unsigned char g_static_scratch[MIXKV_STATIC_SCRATCH_BYTES];
 
 namespace {
-std::mutex g_scratch_mutex;
-void* g_scratch_addr[kMaxDevices] = {nullptr};
+// One call at a time works in the array of a device: its lock is held until all kernels of the call are enqueued, so
+// that those of a call of another thread, on the same stream even, do not come between them.
+struct StaticScratch {
+  std::mutex enqueueing;
+  void* addr = nullptr;   // on this device; looked up once
+};
+StaticScratch g_scratch[kMaxDevices];
 
-// Device address of the scratch array on the current device; looked up once per device.
-int static_scratch(void** out) {
-  int dev = -1;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MIXKV_ERR_CUDA;
-  std::lock_guard<std::mutex> lock(g_scratch_mutex);
-  if (!g_scratch_addr[dev]) {
-    void* ptr = nullptr;
-    if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess || !ptr) return MIXKV_ERR_CUDA;
-    g_scratch_addr[dev] = ptr;
-  }
-  *out = g_scratch_addr[dev];
-  return MIXKV_OK;
-}
-
-// The scratch array for a problem that fits it.  The size is worked out on the host first: too
-// large a problem is refused before anything is enqueued (only attribute queries have run by then).
-int take_static_scratch(const mixkv_params* p, const int32_t* cu_seqlens_host, int32_t batch, int32_t L,
-                        void** scratch) {
+// mixkv_scores in the scratch array.  The size is worked out on the host first: too large a problem is refused before
+// anything is enqueued (only attribute queries have run by then).
+int scores_on_static_scratch(const void* K, const void* V, const void* Qwin, const int32_t* cu_seqlens_host,
+                             int32_t batch, int32_t L, const mixkv_params* p, float* s_comp, float* s_ex_opt,
+                             float* s_div_opt, float* rbar_opt, const float* rbar_in_opt, int32_t* status_dev,
+                             bool clear_status, void* stream) {
   int rc = check_params(p);
   if (rc != MIXKV_OK) return rc;
   SeqTable st;
@@ -534,7 +527,17 @@ int take_static_scratch(const mixkv_params* p, const int32_t* cu_seqlens_host, i
   Workspace ws;
   carve(p, st, nullptr, &ws);
   if (ws.bytes > (size_t)MIXKV_STATIC_SCRATCH_BYTES) return MIXKV_ERR_STATIC_SCRATCH_EXCEEDED;
-  return static_scratch(scratch);
+  const int dev = device_slot();
+  if (dev < 0) return MIXKV_ERR_CUDA;
+  StaticScratch& scratch = g_scratch[dev];
+  std::lock_guard<std::mutex> lock(scratch.enqueueing);
+  if (!scratch.addr) {
+    void* ptr = nullptr;
+    if (cudaGetSymbolAddress(&ptr, g_static_scratch) != cudaSuccess || !ptr) return MIXKV_ERR_CUDA;
+    scratch.addr = ptr;
+  }
+  return scores_impl(K, V, Qwin, cu_seqlens_host, batch, L, p, scratch.addr, (size_t)MIXKV_STATIC_SCRATCH_BYTES,
+                     s_comp, s_ex_opt, s_div_opt, rbar_opt, rbar_in_opt, status_dev, clear_status, stream);
 }
 }  // namespace
 
@@ -543,11 +546,9 @@ int mixkv_internal_scores(const void* K, const void* V, const void* Qwin, const 
                           void* workspace, size_t workspace_bytes, float* s_comp, float* s_ex_opt,
                           float* s_div_opt, float* rbar_opt, const float* rbar_in_opt, int32_t* status_dev,
                           void* stream) {
-  if (use_static_scratch) {
-    const int rc = take_static_scratch(p, cu_seqlens_host, batch, L, &workspace);
-    if (rc != MIXKV_OK) return rc;
-    workspace_bytes = MIXKV_STATIC_SCRATCH_BYTES;
-  }
+  if (use_static_scratch)
+    return scores_on_static_scratch(K, V, Qwin, cu_seqlens_host, batch, L, p, s_comp, s_ex_opt, s_div_opt, rbar_opt,
+                                    rbar_in_opt, status_dev, true, stream);
   return scores_impl(K, V, Qwin, cu_seqlens_host, batch, L, p, workspace, workspace_bytes, s_comp,
                      s_ex_opt, s_div_opt, rbar_opt, rbar_in_opt, status_dev, true, stream);
 }
@@ -557,12 +558,8 @@ int mixkv_scores_static(const void* K, const void* V, const void* Qwin,
                         const mixkv_params* p, float* s_comp, float* s_ex_opt, float* s_div_opt,
                         float* rbar_opt, const float* rbar_in_opt, int32_t* status_dev,
                         void* stream) {
-  void* scratch = nullptr;
-  const int rc = take_static_scratch(p, cu_seqlens_host, batch, L, &scratch);
-  if (rc != MIXKV_OK) return rc;
-  return scores_impl(K, V, Qwin, cu_seqlens_host, batch, L, p, scratch,
-                     (size_t)MIXKV_STATIC_SCRATCH_BYTES, s_comp, s_ex_opt, s_div_opt, rbar_opt,
-                     rbar_in_opt, status_dev, false, stream);
+  return scores_on_static_scratch(K, V, Qwin, cu_seqlens_host, batch, L, p, s_comp, s_ex_opt, s_div_opt, rbar_opt,
+                                  rbar_in_opt, status_dev, false, stream);
 }
 
 namespace {

@@ -207,3 +207,43 @@ def test_the_first_cuda_call_of_a_thread():
         t.join()
     torch.cuda.synchronize()
     assert found == [True] * len(calls), found
+
+
+@pytest.mark.gpu
+def test_two_threads_on_one_stream():
+    # two threads, a problem each, all calls on one stream: those that work in the library's own scratch array, and
+    # those with a workspace per thread, give the bits of calls made alone
+    import torch
+    from paper_2510_20707_b200 import binding
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    rand = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
+    stream = torch.cuda.Stream()
+    problems, found = [], []
+    for L, H, G in ((3000, 4, 4), (7001, 2, 7)):
+        p = binding.Params(kv_heads=H, gqa_ratio=G, budget=96)
+        ws = torch.empty(binding.workspace_size(p, 1, L, L), dtype=torch.uint8, device="cuda")
+        K, V, Q = rand(H, L, 128), rand(H, L, 128), rand(1, H * G, 32, 128)
+        ref = binding.scores(K, V, Q, p)
+        problems.append((K, V, Q, p, ws, ref))
+    torch.cuda.synchronize()
+    start = threading.Barrier(2)
+
+    def thread(K, V, Q, p, ws, ref):
+        try:
+            start.wait()
+            for _ in range(10):
+                outs = []
+                for _ in range(10):
+                    outs += [binding.scores_static(K, V, Q, p, stream=stream),
+                             binding.scores(K, V, Q, p, workspace=ws, stream=stream)]
+                stream.synchronize()
+                found.extend(all(torch.equal(o[k], ref[k]) for k in ("s_comp", "s_ex", "s_div", "rbar")) for o in outs)
+        except Exception as e:
+            found.append(e)
+
+    threads = [threading.Thread(target=thread, args=p) for p in problems]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert found == [True] * 400, found
