@@ -1095,6 +1095,13 @@ int alone_clusters(const int size) {
   (void)ensure_smem(k_tail<true, 1024, true, false>, kTailSmem, done);   // (a failure shows at the launch)
   return fit.ask(k_tail<true, 1024, true, false>, 1024, 120 * 1024, size);
 }
+// The same with two CTAs to an SM, of 512 threads and half of its shared memory each (adapt_pairs_fit).
+int paired_clusters(const int size) {
+  static std::atomic<bool> done[kMaxDevices];
+  static ClusterFit fit;
+  (void)ensure_smem(k_tail<true, 512, true, true>, kTailSmem, done);
+  return fit.ask(k_tail<true, 512, true, true>, 512, 113 * 1024 - 24576, size);
+}
 
 // CTAs per (sequence, layer) pair: one while it has 8192 keys or less of all heads (the exchanges cost as much as
 // the sweeps they save), else as many as leave each that much and are all resident at once, one per SM (15 clusters of
@@ -1145,14 +1152,13 @@ int tail_clusters(const long long units, const int P, const int sms, const Fit& 
   return cs;
 }
 
-// fixed_cs: so many CTAs per unit, 0: as many as the rules say.
-TailShape tail_shape(const LaunchCtx& c, const int fixed_cs = 0) {
+TailShape tail_shape(const LaunchCtx& c) {
   const long long units = (long long)c.st.layers * c.st.batch * c.st.H;
   const int P = c.max_prefix, sms = device_sm_count();
   TailShape t;
-  t.cs = fixed_cs ? fixed_cs : tail_clusters(units, P, sms, alone_clusters);
-  // What does not fit shared memory in that many CTAs takes more of them.
-  while (!fixed_cs && t.cs < kTailMaxCluster && tail_chunk(P, t.cs) > kTailCacheCap) t.cs *= 2;
+  t.cs = tail_clusters(units, P, sms, alone_clusters);
+  // What does not fit shared memory in that many CTAs takes more of them, where there is a place for such a cluster.
+  while (t.cs < kTailMaxCluster && tail_chunk(P, t.cs) > kTailCacheCap && alone_clusters(2 * t.cs) > 0) t.cs *= 2;
   t.chunk = tail_chunk(P, t.cs);
   // A CTA alone on its SM: 1024 threads (a block of 4096 positions), fewer when the slice is shorter.  More
   // CTAs than SMs: smaller ones side by side, as many as there are and as shared memory holds (heads of
@@ -1169,12 +1175,40 @@ TailShape tail_shape(const LaunchCtx& c, const int fixed_cs = 0) {
 
 bool tail_can_fuse(const LaunchCtx& c) { return tail_shape(c).cached; }
 
-// Where it pays: whole calls, mix, budget and tail kernels against this, us.  One layer: 4 heads of 4096 keys 42.8 / 32.4,
-// eight ragged sequences of 4 heads of 2 to 7 thousand 60.9 / 51.4, 8 heads of 9000 57.1 / 47.3, of 20000 (four sequences)
-// 114 / 106; longer heads want more than a CTA each: 4 of 32768 67.1 / 67.3, 2 of 40000 62.4 / 68.3.  More CTAs than
-// are resident together lose what the launches cost: 128 units 109 / 100, 224 135 / 132, 240 299 / 292, 288 206 / 211,
-// 896 (28 layers x 8 ragged sequences) 889 / 924.
+// Whether two CTAs of 512 threads share an SM (its shared memory) with a head of P candidates each.
+bool adapt_pairs_fit(const int P) {
+  return 2 * (24576 + (size_t)tail_chunk(P, 1) * 17 / 4 + 512 * 32) <= 226 * 1024;
+}
+
+// Threads of a CTA when the heads of a sequence are a cluster that shares its budget out (k_tail with ADAPT), 0: where
+// mix, budget and tail kernels are as good.  Every thread reads its bins of all heads over distributed shared memory,
+// so 1024 threads, as long as all clusters are resident with an SM to each CTA.  Where they are not, 512 threads and two
+// CTAs to an SM, all resident that way; clusters of seven and eight gain that way on long heads only.  Heads too long for
+// two to share an SM take 1024 threads in more than one wave.  One layer of so many sequences, heads x keys, whole calls,
+// three kernels / this, us (and with 256 threads for heads of 1024 keys and less, as it once was):
+//   all resident, 1024: 4 of 4 x 1024 to 8 x 24576 all faster: 4 of 8 x 760 36.2 / 31.5 (68.9), 33 of 4 x 760 47.3 / 40.0
+//     (56.1), 1 of 4 x 4300 40.3 / 32.2, 15 of 8 x 9000 159 / 150, 74 of 2 x 17000 380 / 348, 15 of 8 x 24500 471 / 427
+//   not resident (1024 threads in a second wave in brackets): 36 of 4 x 760 46.2 / 43.3 (52.3), 110 of 2 x 4300
+//     152 / 141 (153), 23 of 6 x 2300 73.4 / 71.8 (77.5), 38 of 6 x 9000 318 / 299 (306), 60 of 4 x 17000 648 / 596 (614);
+//     17 of 8 x 760 48.9 / 52.0 (56.8), x 2300 72.0 / 76.6 (81.9), x 9000 187 / 189 (195), 29 of 8 x 4300 156 / 153
+//     (160), x 17000 616 / 580 (589), 17 of 8 x 17000 361 / 353 (361)
+//   too long for pairs: 17 of 8 x 24500 511 / 497, 60 of 4 934 / 837, 23 of 6 512 / 505
+template <typename Alone, typename Paired>
+int adapt_threads(const long long sequences, const int heads, const int P, const Alone& alone, const Paired& paired) {
+  if (sequences <= alone(heads)) return 1024;
+  if (!adapt_pairs_fit(P)) return alone(heads) > 0 ? 1024 : 0;
+  return sequences <= paired(heads) && (heads <= 6 || P > 8192) ? 512 : 0;
+}
+
+// Whole calls, three kernels against this, us.  One layer: longer heads want more than a CTA each (4 of 32768 67.1 / 67.3,
+// 2 of 40000 62.4 / 68.3); more CTAs than are resident together lose what the launches cost (288 units 206 / 211, 896, 28
+// layers x 8 ragged sequences, 889 / 924).
 constexpr int kAdaptMaxKeys = 24576;
+static_assert(kAdaptMaxKeys <= kTailCacheCap, "the keys of a head stay in one CTA");
+TailShape adapt_shape(const LaunchCtx& c) {
+  return {1, adapt_threads((long long)c.st.layers * c.st.batch, c.st.H, c.max_prefix, alone_clusters, paired_clusters),
+          tail_chunk(c.max_prefix, 1), true};
+}
 bool tail_adapts(const LaunchCtx& c) {
   const int H = c.st.H, Bp = c.p.budget - c.p.window, f = floor_slots(c.p);
   if (c.p.budget_mode != MIXKV_BUDGET_ADAPTIVE || H < 2 || H > kMaxCluster || c.max_prefix > kAdaptMaxKeys) return false;
@@ -1182,7 +1216,7 @@ bool tail_adapts(const LaunchCtx& c) {
   int shortest = c.max_prefix;
   for (int b = 0; b < c.st.batch; ++b) shortest = std::min(shortest, c.st.cu[b + 1] - c.st.cu[b] - c.st.W);
   if ((long long)f + (long long)H * (Bp - f) > shortest) return false;
-  return tail_shape(c, 1).cached;
+  return adapt_shape(c).threads != 0;
 }
 
 template <bool FUSED, int T, bool CL, bool ADAPT>
@@ -1219,7 +1253,7 @@ cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
   a.out_rows_cap = c.out_rows_cap;
   a.status_clear = t.status_clear;
   a.mp = mix_params(c.p);
-  const TailShape sh = tail_shape(c, t.adapt ? 1 : 0);
+  const TailShape sh = t.adapt ? adapt_shape(c) : tail_shape(c);
   const bool fused = t.scores == nullptr;
   a.cached = sh.cached ? 1 : 0;
   if (fused && !a.cached) return cudaErrorInvalidValue;   // callers check tail_can_fuse() first
@@ -1229,8 +1263,9 @@ cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
   if (fused) smem += ((size_t)8 * sh.threads + 64) * 4;
   auto launch = [&](auto threads) {
     constexpr int T = decltype(threads)::value;
-    if (t.adapt)
-      return fused ? launch_tail_t<true, T, true, true>(c, a, sh, smem) : launch_tail_t<false, T, true, true>(c, a, sh, smem);
+    if constexpr (T >= 512)
+      if (t.adapt)
+        return fused ? launch_tail_t<true, T, true, true>(c, a, sh, smem) : launch_tail_t<false, T, true, true>(c, a, sh, smem);
     if (sh.cs > 1)
       return fused ? launch_tail_t<true, T, true, false>(c, a, sh, smem) : launch_tail_t<false, T, true, false>(c, a, sh, smem);
     return fused ? launch_tail_t<true, T, false, false>(c, a, sh, smem) : launch_tail_t<false, T, false, false>(c, a, sh, smem);
@@ -1246,6 +1281,11 @@ cudaError_t launch_tail(const LaunchCtx& c, const TailArgs& t) {
 
 extern "C" int mixkv_internal_tail_clusters(int64_t units, int32_t candidates, int32_t sms, const int32_t* alone) {
   return mixkv::tail_clusters(units, candidates, sms, [&](const int n) { return alone[n]; });
+}
+extern "C" int mixkv_internal_adapt_threads(int64_t sequences, int32_t heads, int32_t candidates, const int32_t* alone,
+                                            const int32_t* paired) {
+  return mixkv::adapt_threads(sequences, heads, candidates, [&](const int n) { return alone[n]; },
+                              [&](const int n) { return paired[n]; });
 }
 extern "C" int mixkv_internal_budget_clusters(int32_t pairs, int64_t keys_per_pair, const int32_t* alone) {
   return mixkv::budget_clusters(pairs, keys_per_pair, [&](const int n) { return alone[n]; });

@@ -1,5 +1,7 @@
 """GPU parity: the CUDA library, called through its C ABI, against the CPU oracle on the
 same seeded inputs (tolerances in tests/parity.py)."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -254,7 +256,8 @@ def test_adaptive_budgets_on_many_keys_are_exact(H, lens, levels):
 @pytest.mark.parametrize("H,lens,Bp,ada_floor,levels", [
     (3, (130,), 50, 0.2, 7), (3, (129,), 50, 0.2, 7),          # 10 + 3 * 40 = 130: a head cannot, and could, run out
     (2, (1500, 900, 3001), 64, 0.2, 1 << 20), (5, (700, 2600), 96, 0.2, 4), (8, (12007, 1291), 144, 0.2, 1 << 20),
-    (4, (5000, 901), 80, 1.0, 50), (4, (5000, 901), 80, 0.0, 1), (7, (24576,), 300, 0.3, 900), (6, (24577,), 300, 0.3, 900)])
+    (4, (5000, 901), 80, 1.0, 50), (4, (5000, 901), 80, 0.0, 1), (7, (24576,), 300, 0.3, 900), (6, (24577,), 300, 0.3, 900),
+    (8, (8193,) * 17, 100, 0.2, 700), (4, (700,) * 34, 100, 0.2, 60), (8, (18000,) * 17, 100, 0.2, 700)])
 def test_adaptive_budgets_shared_out_by_the_selection_are_exact(H, lens, Bp, ada_floor, levels):
     # the heads of a sequence as a cluster that shares its budget out before each head selects: at the edges of the
     # rule that takes it (candidates of the shortest sequence, keys of the longest), nothing to share, nothing but
@@ -272,6 +275,42 @@ def test_adaptive_budgets_shared_out_by_the_selection_are_exact(H, lens, Bp, ada
     assert np.array_equal(got["counts"].cpu().numpy(), ref["counts"].reshape(-1))
     assert np.array_equal(offs, ref["idx_offsets"])
     assert np.array_equal(got["idx"].cpu().numpy()[:offs[-1]], ref["idx"])
+
+
+@pytest.mark.parametrize("NL,H,lens,kw", [
+    (1, 2, (300,), {}), (1, 3, (1025, 777), dict(pool_mode=1)), (1, 5, (2049, 1500, 4097), dict(use_vnorm=2)),
+    (2, 8, (1290,), dict(rbar=True)), (3, 8, (9001, 12000), dict(pool_mode=1, use_vnorm=2, rbar=True)),   # 1024 threads
+    (40, 4, (700,), {}), (20, 6, (1500, 801), dict(pool_mode=1)), (90, 2, (4200,), dict(use_vnorm=0, rbar=True)),
+    (17, 8, (8225,), dict(use_vnorm=2)),                                               # 512 threads, two CTAs to an SM
+    (5, 8, (18000, 17800, 700, 18001), dict(mix_mode=3))])                             # 1024 threads, more than one wave
+def test_adaptive_budgets_have_the_bits_of_the_stages_kept_apart(NL, H, lens, kw):
+    # a call with events keeps mix, budget and tail kernels apart; without, calls of few heads share the budgets out in
+    # the tail: the same scores, the same integer work, the same bits
+    kw = dict(kw)
+    with_rbar = kw.pop("rbar", False)
+    gen = torch.Generator(device="cuda").manual_seed(H * NL)
+    rand = lambda *shape: torch.randn(shape, generator=gen, device="cuda").bfloat16()
+    total, batch, W, G = sum(lens), len(lens), 16, 2
+    K, V, Q = rand(NL, H, total, 128), rand(NL, H, total, 128), rand(NL, batch, H * G, W, 128)
+    rbar = torch.rand((NL, batch, H), generator=gen, device="cuda") if with_rbar else None
+    p = binding.Params(kv_heads=H, gqa_ratio=G, window=W, budget=W + min(200, min(lens) // H - W), budget_mode=1, **kw)
+    cu = [int(c) for c in np.concatenate([[0], np.cumsum(lens)])] if batch > 1 else None
+    traced = binding.compress_layers(K, V, Q, p, cu_seqlens=cu, rbar_in=rbar, trace_events=(ctypes.c_void_p * 1)())
+    plain = binding.compress_layers(K, V, Q, p, cu_seqlens=cu, rbar_in=rbar)
+    bare = binding.compress_layers(K, V, Q, p, cu_seqlens=cu, rbar_in=rbar, want_aux=False)
+    torch.cuda.synchronize()
+    assert int(traced["status"].item()) == 0 and int(plain["status"].item()) == 0
+    assert torch.equal(traced["s_comp"], plain["s_comp"])
+    for layer in range(NL):
+        n = int(traced["idx_offsets"][layer, -1])
+        for out in (plain, bare):
+            rows = int(traced["out_row_offsets"][layer, -1])
+            assert torch.equal(traced["out_row_offsets"][layer], out["out_row_offsets"][layer])
+            for key in ("K_out", "V_out"):
+                assert torch.equal(traced[key][layer, :rows].view(torch.int16), out[key][layer, :rows].view(torch.int16))
+        assert torch.equal(traced["counts"][layer], plain["counts"][layer])
+        assert torch.equal(traced["idx_offsets"][layer], plain["idx_offsets"][layer])
+        assert torch.equal(traced["idx"][layer, :n], plain["idx"][layer, :n])
 
 
 def test_adaptive_budgets_by_one_cta_on_keys_it_cannot_cache():

@@ -52,3 +52,33 @@ def test_calls_on_the_static_scratch_enqueue_one_after_the_other(fake_cuda):
     kernels = ["k_pass1", "k_pass2", "k_poolsum", "k_mixpool"]
     assert [x.kernel for x in calls] == kernels * 12
     assert all(len({x.caller for x in calls[i:i + 4]}) == 1 for i in range(0, 48, 4)), [x.caller for x in calls]
+
+
+@pytest.mark.parametrize("adaptive,P", [(1, 900), (1, 20000), (1, 30000), (0, 30000), (0, 50000)])
+def test_a_device_that_holds_no_cluster_gets_none(fake_cuda, adaptive, P):
+    # (a part of a device may have no group of SMs that is large enough): the call takes the kernels that need none
+    fake_cuda.reset(device=3, resident={n: 0 for n in range(2, 9)})
+    p = binding.Params(kv_heads=4, gqa_ratio=4, budget=64, budget_mode=adaptive).c()
+    rc = fake_cuda.lib.mixkv_compress_layer(ONE, ONE, ONE, None, 1, P + 32, C.byref(p), ONE, 1 << 30, None, ONE, ONE, ONE,
+                                            *[None] * 6)
+    assert rc == 0
+    calls = fake_cuda.launches()
+    assert all(x.cluster == 1 for x in calls), calls
+    unfused = adaptive or P > 40960
+    assert [x.kernel for x in calls] == ["k_pass1", "k_pass2"] + ["k_mixpool"] * unfused + ["k_budget"] * adaptive + ["k_tail"]
+
+
+@pytest.mark.parametrize("sequences,heads,P,shape", [
+    (15, 8, 700, (1024, 8)), (17, 8, 700, None), (17, 8, 9000, (512, 8)), (36, 4, 700, (512, 4)), (36, 4, 20000, (1024, 4)),
+    (60, 4, 9000, (512, 4)), (31, 8, 9000, None)])
+def test_adaptive_budgets_take_clusters_that_are_resident(fake_cuda, sequences, heads, P, shape):
+    fake_cuda.reset(device=4, resident={3: 45, 4: 33, 5: 26, 6: 22, 7: 15, 8: 15})
+    p = binding.Params(kv_heads=heads, gqa_ratio=4, budget=64, budget_mode=1).c()
+    rc = fake_cuda.lib.mixkv_compress_layers(ONE, ONE, ONE, sequences, C.c_int64(0), C.c_int64(0), None, 1, P + 32,
+                                             C.byref(p), ONE, 1 << 40, None, ONE, ONE, ONE, *[None] * 7, 0)
+    assert rc == 0
+    calls = fake_cuda.launches()[2:]
+    if shape:
+        assert [x[1:] for x in calls] == [(sequences * heads, *shape, "k_tail")]
+    else:
+        assert [x.kernel for x in calls] == ["k_mixpool", "k_budget", "k_tail"]

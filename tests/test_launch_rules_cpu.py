@@ -64,3 +64,18 @@ def test_tail_and_budget_clusters_as_measured(lib):
     budget = lambda pairs, keys: lib.mixkv_internal_budget_clusters(pairs, C.c_int64(keys), array(alone))
     assert [budget(1, 8192), budget(15, 60000), budget(16, 60000), budget(33, 60000), budget(34, 60000),
             budget(74, 60000), budget(75, 60000), budget(74, 8193)] == [1, 8, 4, 4, 2, 2, 1, 2]
+
+
+def test_adaptive_budgets_in_the_tail_as_measured(lib):
+    sms, alone, _ = B200
+    paired = tuple(2 * n for n in alone)
+    threads = lambda sequences, heads, P, alone=alone, paired=paired: lib.mixkv_internal_adapt_threads(
+        C.c_int64(sequences), heads, P, array(alone), array(paired))
+    assert [threads(15, 8, 700), threads(16, 8, 700), threads(16, 8, 8192), threads(16, 8, 8193), threads(30, 8, 8193),
+            threads(31, 8, 8193)] == [1024, 0, 0, 512, 512, 0]
+    assert [threads(33, 4, 9000), threads(34, 4, 9000), threads(66, 4, 700), threads(67, 4, 700)] == [1024, 512, 512, 0]
+    # from some 17600 keys on two CTAs do not share an SM any more
+    assert [threads(34, 4, 17000), threads(34, 4, 18000), threads(16, 8, 18000)] == [512, 1024, 1024]
+    # a device, or a part of one, that holds no such cluster
+    none = (148, 74) + (0,) * 6
+    assert [threads(1, 2, 700, none, none), threads(1, 4, 700, none, none), threads(1, 4, 20000, none, none)] == [1024, 0, 0]
