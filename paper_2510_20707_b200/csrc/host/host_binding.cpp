@@ -111,13 +111,23 @@ bool truth(PyObject* o) {
   if (t < 0) throw Raised();
   return t != 0;
 }
-long attr_int(PyObject* o, PyObject* name) {
+// The library takes 32 bits: of a larger number it would see the lower ones, another problem than the caller's.
+int32_t int32(const long x, const char* what) {
+  if (x != (int32_t)x) check_status(MIXKV_ERR_INVALID_ARG, what);
+  return (int32_t)x;
+}
+int32_t int32(PyObject* o, const char* what) {
+  const long x = PyLong_AsLong(o);
+  if (x == -1 && PyErr_Occurred()) throw Raised();
+  return int32(x, what);
+}
+int32_t attr_int(PyObject* o, PyObject* name) {
   PyObject* v = PyObject_GetAttr(o, name);
   if (!v) throw Raised();
   const long x = PyLong_AsLong(v);
   Py_DECREF(v);
   if (x == -1 && PyErr_Occurred()) throw Raised();
-  return x;
+  return int32(x, "mixkv_params");
 }
 float attr_float(PyObject* o, PyObject* name) {
   PyObject* v = PyObject_GetAttr(o, name);
@@ -129,16 +139,16 @@ float attr_float(PyObject* o, PyObject* name) {
 }
 mixkv_params params(PyObject* o) {
   mixkv_params p;
-  p.kv_heads = (int32_t)attr_int(o, nm.kv_heads);
-  p.gqa_ratio = (int32_t)attr_int(o, nm.gqa_ratio);
-  p.head_dim = (int32_t)attr_int(o, nm.head_dim);
-  p.window = (int32_t)attr_int(o, nm.window);
-  p.pool_kernel = (int32_t)attr_int(o, nm.pool_kernel);
-  p.pool_mode = (int32_t)attr_int(o, nm.pool_mode);
-  p.use_vnorm = (int32_t)attr_int(o, nm.use_vnorm);
-  p.mix_mode = (int32_t)attr_int(o, nm.mix_mode);
-  p.budget_mode = (int32_t)attr_int(o, nm.budget_mode);
-  p.budget = (int32_t)attr_int(o, nm.budget);
+  p.kv_heads = attr_int(o, nm.kv_heads);
+  p.gqa_ratio = attr_int(o, nm.gqa_ratio);
+  p.head_dim = attr_int(o, nm.head_dim);
+  p.window = attr_int(o, nm.window);
+  p.pool_kernel = attr_int(o, nm.pool_kernel);
+  p.pool_mode = attr_int(o, nm.pool_mode);
+  p.use_vnorm = attr_int(o, nm.use_vnorm);
+  p.mix_mode = attr_int(o, nm.mix_mode);
+  p.budget_mode = attr_int(o, nm.budget_mode);
+  p.budget = attr_int(o, nm.budget);
   p.ada_floor = attr_float(o, nm.ada_floor);
   p.eps = attr_float(o, nm.eps);
   p.softmax_scale = attr_float(o, nm.softmax_scale);
@@ -168,6 +178,10 @@ struct Offsets {
           Py_DECREF(seq);
           throw Raised();
         }
+      }
+      if (x != (int32_t)x) {
+        Py_DECREF(seq);
+        check_status(MIXKV_ERR_INVALID_ARG, "cu_seqlens");
       }
       v.push_back((int32_t)x);
     }
@@ -522,10 +536,7 @@ PyObject* py_similarity_map(PyObject*, PyObject* const* a, Py_ssize_t n) {
     want_dims(X, 3, "X must have three dimensions [heads, L, d]");
     if (!X.is_contiguous() || X.scalar_type() != at::kBFloat16)
       fail(PyExc_AssertionError, "X must be a contiguous bf16 tensor");
-    const long block = PyLong_AsLong(a[1]);
-    if (block == -1 && PyErr_Occurred()) throw Raised();
-    // (the library would see its lower 32 bits, and another number of cells than the map has)
-    if (block != (int32_t)block) check_status(MIXKV_ERR_INVALID_ARG, "mixkv_similarity_map");
+    const int64_t block = int32(a[1], "mixkv_similarity_map");
     const int heads = (int)X.size(0), L = (int)X.size(1);
     size_t need = 0;
     check_status(api.sim_ws_size(heads, L, (int)block, &need), "mixkv_similarity_workspace_size");
@@ -561,7 +572,8 @@ PyObject* py_decode_attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
       fail(PyExc_AssertionError, "the caches and q must be contiguous");
     if (offs.scalar_type() != at::kInt || !offs.is_contiguous())
       fail(PyExc_AssertionError, "out_row_offsets must be a contiguous int32 tensor");
-    const long H = PyLong_AsLong(a[4]), G = PyLong_AsLong(a[5]), rows = PyLong_AsLong(a[6]);
+    const char* what = "mixkv_decode_attention";
+    const int32_t H = int32(a[4], what), G = int32(a[5], what), rows = int32(a[6], what);
     const double scale = PyFloat_AsDouble(a[7]);
     if (PyErr_Occurred()) throw Raised();
     const CallStream stream(a[8], K);
@@ -574,10 +586,9 @@ PyObject* py_decode_attention(PyObject*, PyObject* const* a, Py_ssize_t n) {
     {
       const Unlocked u;
       out = empty(q.sizes(), at::kFloat, q);
-      rc = api.decode(k, v, offsets, cap, query, layers, batch, (int)H, (int)G, d, (float)scale, (int)rows, fp(out),
-                      stream.handle);
+      rc = api.decode(k, v, offsets, cap, query, layers, batch, H, G, d, (float)scale, rows, fp(out), stream.handle);
     }
-    check_status(rc, "mixkv_decode_attention");
+    check_status(rc, what);
     return THPVariable_Wrap(out);
   });
 }

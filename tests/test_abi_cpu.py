@@ -132,6 +132,31 @@ def test_binding_refuses_block_sizes_the_library_cannot_take(lib, block):
     assert e.value.status == -1
 
 
+@pytest.mark.parametrize("kw", [dict(kv_heads=(1 << 32) + 2), dict(gqa_ratio=1 - (1 << 32)), dict(max_rows=(1 << 32) + 100),
+                                dict(max_rows=1 << 31)])
+def test_binding_refuses_decode_sizes_the_library_cannot_take(lib, kw):
+    # (the lower 32 bits of each are sizes that it would take)
+    import torch
+    cache, offs = torch.zeros((1, 8, 128), dtype=torch.bfloat16), torch.zeros((1, 3), dtype=torch.int32)
+    with pytest.raises(binding.MixKVError) as e:
+        binding.decode_attention(cache, cache, offs, cache[:, None, :2], **dict(dict(kv_heads=2, gqa_ratio=1, max_rows=4), **kw))
+    assert e.value.status == -1
+
+
+@pytest.mark.parametrize("kw,cu", [(dict(kv_heads=(1 << 32) + 2), None), (dict(budget=(1 << 32) + 32), None),
+                                   (dict(pool_kernel=7 - (1 << 32)), None), ({}, [0, (1 << 32) + 64])])
+def test_binding_refuses_params_and_offsets_the_library_cannot_take(lib, kw, cu):
+    import torch
+    K, Q = torch.zeros((2, 64, 128), dtype=torch.bfloat16), torch.zeros((1, 2, 16, 128), dtype=torch.bfloat16)
+    p = binding.Params(**dict(dict(kv_heads=2, gqa_ratio=1, window=16, budget=32), **kw))
+    for call in (lambda: binding.scores(K, K, Q, p, cu_seqlens=cu), lambda: binding.compress_layer(K, K, Q, p, cu_seqlens=cu),
+                 lambda: binding.compress_layers(K[None], K[None], Q[None], p, cu_seqlens=cu),
+                 lambda: binding.select(torch.zeros((2, 48)), p, cu_seqlens=cu)):
+        with pytest.raises(binding.MixKVError) as e:
+            call()
+        assert e.value.status == -1
+
+
 def test_native_binding_is_rebuilt_for_another_torch(lib, monkeypatch):
     # the module is compiled against torch's C++ interface: a file newer than its sources does not show that
     assert build.host_matches() and not build.host_is_stale()
