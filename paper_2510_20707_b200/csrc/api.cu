@@ -16,12 +16,12 @@ int device_check(int* major_out) {
   static std::atomic<int> cached[kMaxDevices];   // 0 = unknown, else major + 1
   int dev = 0;
   if (major_out) *major_out = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return MIXKV_ERR_CUDA;
+  if (!answered(cudaGetDevice(&dev))) return MIXKV_ERR_CUDA;
   int major = 0;
   if (dev >= 0 && dev < kMaxDevices && cached[dev].load(std::memory_order_relaxed) != 0) {
     major = cached[dev].load(std::memory_order_relaxed) - 1;
   } else {
-    if (cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev) != cudaSuccess)
+    if (!answered(cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev)))
       return MIXKV_ERR_CUDA;
     if (dev >= 0 && dev < kMaxDevices) cached[dev].store(major + 1, std::memory_order_relaxed);
   }

@@ -98,10 +98,16 @@ cudaError_t launch_pass2(const LaunchCtx& c, const void* K, const void* V, const
                          float* s_div_out, float* rbar_out, int* status);
 constexpr int kMaxDevices = 64;   // what is looked up or set once per device is remembered for so many
 int device_sm_count();
+// Whether a question to the runtime was answered.  For those that a call can do without the answer of: their error is
+// not left behind as the thread's last one, where the caller's next check would take it for its own.
+inline bool answered(const cudaError_t e) {
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e == cudaSuccess;
+}
 // The current device as an index into what is remembered per device; -1: none, or one past the end.
 inline int device_slot() {
   int dev = -1;
-  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices ? dev : -1;
+  return answered(cudaGetDevice(&dev)) && dev >= 0 && dev < kMaxDevices ? dev : -1;
 }
 // Lets `kernel` have `smem` bytes of dynamic shared memory on the current device, once per device; `done` is the
 // kernel's own array (static: entry points may run in several threads at once).
@@ -114,7 +120,8 @@ cudaError_t ensure_smem(F kernel, size_t smem, std::atomic<bool> (&done)[kMaxDev
 }
 // Clusters of 1 .. 8 CTAs of one kernel that the current device holds at once.  A cluster lies in one group of SMs, and
 // how the SMs of a chip fall into groups differs between chips of one model, so the runtime is asked, once per device
-// and size (0.2 us a question); `kernel` may already have its shared memory.  Without a device: as if SMs were all alike.
+// and size (0.2 us a question); `kernel` may already have its shared memory.  No answer counts as none and is not
+// remembered.  Without a device: as if SMs were all alike.
 struct ClusterFit {
   std::atomic<int> known[kMaxDevices][kMaxCluster + 1];   // 0: not asked, else the answer + 1
   template <typename F>
@@ -132,7 +139,7 @@ struct ClusterFit {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) return device_sm_count() / size;
+    if (!answered(cudaOccupancyMaxActiveClusters(&n, kernel, &cfg))) return dev >= 0 ? 0 : device_sm_count() / size;
     if (dev >= 0) known[dev][size].store(n + 1, std::memory_order_relaxed);
     return n;
   }

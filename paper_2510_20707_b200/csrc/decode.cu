@@ -489,7 +489,7 @@ extern "C" int mixkv_decode_attention(const void* K_cache, const void* V_cache,
   auto resident = [&](const int depth) {
     return [&, depth](const int size) {
       const DecKernel k = dec_kernel(wide, depth);
-      if (ensure_smem(k, dec_smem(depth), done[variant(depth)], dev) != cudaSuccess) return 0;
+      if (!answered(ensure_smem(k, dec_smem(depth), done[variant(depth)], dev))) return 0;
       return fit[variant(depth)].ask(k, kDecThreads, dec_smem(depth), size, dev);
     };
   };

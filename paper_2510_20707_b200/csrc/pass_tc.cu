@@ -1100,11 +1100,10 @@ bool encode_bf16_map(void* tm, const void* base, int rank, const unsigned long l
 int device_sm_count() {
   static std::atomic<int> cached[kMaxDevices];
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 148;
+  if (!answered(cudaGetDevice(&dev)) || dev < 0 || dev >= kMaxDevices) return 148;
   int n = cached[dev].load(std::memory_order_relaxed);
   if (n == 0) {
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1)
-      n = 148;
+    if (!answered(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) || n < 1) return 148;
     cached[dev].store(n, std::memory_order_relaxed);
   }
   return n;

@@ -34,6 +34,10 @@ __global__ void k_wait_runs_out(int* status, unsigned long long* waited_ns) {
 extern "C" int mixkv_selftest_bounded_wait(int32_t* status_dev, unsigned long long* waited_ns_dev,
                                            void* stream) {
   if (!status_dev) return MIXKV_ERR_INVALID_ARG;
-  mixkv::k_wait_runs_out<<<1, 64, 0, (cudaStream_t)stream>>>(status_dev, waited_ns_dev);
-  return cudaGetLastError() == cudaSuccess ? MIXKV_OK : MIXKV_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(64);
+  cfg.stream = (cudaStream_t)stream;
+  return cudaLaunchKernelEx(&cfg, mixkv::k_wait_runs_out, status_dev, waited_ns_dev) == cudaSuccess ? MIXKV_OK
+                                                                                                   : MIXKV_ERR_CUDA;
 }

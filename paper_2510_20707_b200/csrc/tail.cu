@@ -1092,14 +1092,14 @@ namespace {
 int alone_clusters(const int size) {
   static std::atomic<bool> done[kMaxDevices];
   static ClusterFit fit;
-  (void)ensure_smem(k_tail<true, 1024, true, false>, kTailSmem, done);   // (a failure shows at the launch)
+  (void)answered(ensure_smem(k_tail<true, 1024, true, false>, kTailSmem, done));   // (a failure shows at the launch)
   return fit.ask(k_tail<true, 1024, true, false>, 1024, 120 * 1024, size);
 }
 // The same with two CTAs to an SM, of 512 threads and half of its shared memory each (adapt_pairs_fit).
 int paired_clusters(const int size) {
   static std::atomic<bool> done[kMaxDevices];
   static ClusterFit fit;
-  (void)ensure_smem(k_tail<true, 512, true, true>, kTailSmem, done);
+  (void)answered(ensure_smem(k_tail<true, 512, true, true>, kTailSmem, done));
   return fit.ask(k_tail<true, 512, true, true>, 512, 113 * 1024 - 24576, size);
 }
 

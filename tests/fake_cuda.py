@@ -31,9 +31,9 @@ class FakeCuda:
             binding.LIB_PATH, binding._lib = kept
         self.reset()
 
-    def reset(self, device=0, sms=148, major=10, occupancy_error=0, pause_us=0, resident={}):
+    def reset(self, device=0, sms=148, major=10, query_error=0, ask_error=0, pause_us=0, resident={}):
         """What the library keeps per device it keeps by its number: a test that changes the answers takes another."""
-        self.runtime.fake_reset(device, sms, major, occupancy_error, pause_us)
+        self.runtime.fake_reset(device, sms, major, query_error, ask_error, pause_us)
         for size, clusters in resident.items():
             self.runtime.fake_resident(size, clusters)
 

@@ -19,7 +19,7 @@ struct Launch {
 std::mutex mutex;
 std::map<const void*, std::string> names;   // host function of a kernel -> its mangled name
 std::vector<Launch> launches;
-int launch_pause_us = 0, device = 0, major = 10, sms = 148, occupancy_error = 0;
+int launch_pause_us = 0, device = 0, major = 10, sms = 148, query_error = 0, ask_error = 0;
 int resident[17];                           // clusters of n CTAs at once
 thread_local int caller = 0, last_error = 0;
 cudaError_t result(const int e) {
@@ -34,8 +34,9 @@ int encode() { return bound ? 0 : 201; }
 
 extern "C" {
 // ---- what the tests set and read
-void fake_reset(int device_, int sms_, int major_, int occupancy_error_, int pause_us) {
-  device = device_, sms = sms_, major = major_, occupancy_error = occupancy_error_, launch_pause_us = pause_us;
+// query_error: of every question about a kernel; ask_error: of those about clusters
+void fake_reset(int device_, int sms_, int major_, int query_error_, int ask_error_, int pause_us) {
+  device = device_, sms = sms_, major = major_, query_error = query_error_, ask_error = ask_error_, launch_pause_us = pause_us;
   for (int n = 1; n <= 16; ++n) resident[n] = sms_ / n;
   launches.clear();
   last_error = 0;
@@ -81,7 +82,7 @@ cudaError_t cudaPeekAtLastError() { return (cudaError_t)last_error; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) {
   bound = device >= 0;
-  return result(device < 0 ? cudaErrorNoDevice : occupancy_error);
+  return result(device < 0 ? cudaErrorNoDevice : query_error);
 }
 cudaError_t cudaSetDevice(int dev) {
   if (device < 0 || dev != device) return result(cudaErrorInvalidDevice);
@@ -100,7 +101,7 @@ cudaError_t cudaGetDriverEntryPoint(const char*, void** p, unsigned long long, c
 cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t* cfg) {
   if (device < 0) return result(cudaErrorNoDevice);
   bound = true;
-  if (occupancy_error) return result(occupancy_error);
+  if (query_error || ask_error) return result(query_error ? query_error : ask_error);
   *n = resident[cfg->attrs[0].val.clusterDim.x] * (cfg->blockDim.x <= 512 ? 2 : 1);
   return cudaSuccess;
 }

@@ -82,3 +82,40 @@ def test_adaptive_budgets_take_clusters_that_are_resident(fake_cuda, sequences, 
         assert [x[1:] for x in calls] == [(sequences * heads, *shape, "k_tail")]
     else:
         assert [x.kernel for x in calls] == ["k_mixpool", "k_budget", "k_tail"]
+
+
+@pytest.mark.parametrize("device,error", [(-1, 0), (5, 209), (5, 2)])
+def test_questions_that_fail_leave_no_error_behind(fake_cuda, device, error):
+    # no device, no image for the device, no memory: shape queries answer all the same, and the next check of the last
+    # error, in the caller's own code, must not find theirs
+    fake_cuda.reset(device=device, query_error=error)
+    lib, c = fake_cuda.lib, C.byref
+    fixed, adaptive = (binding.Params(kv_heads=4, gqa_ratio=4, budget=64, budget_mode=m).c() for m in (0, 1))
+    assert lib.mixkv_launches_for(c(fixed), 1, 1, 60000) > 0 and lib.mixkv_launches_for(c(adaptive), 1, 1, 9000) > 0
+    assert lib.mixkv_stage_name_for(c(fixed), 1, 1, 60000, 0) == b"pass1"
+    assert fake_cuda.last_error() == 0
+    size = C.c_size_t()
+    assert lib.mixkv_workspace_size(c(fixed), 1, 60000, 60000, c(size)) == 0
+    cc = C.c_int32()
+    assert lib.mixkv_device_check(c(cc)) == (-4 if device < 0 else 0)
+    assert fake_cuda.last_error() == 0
+
+
+def test_a_cluster_that_cannot_be_asked_for_is_not_launched(fake_cuda):
+    # what the runtime answers with an error is no cluster at all, and is asked again the next time
+    p = binding.Params(kv_heads=4, gqa_ratio=4, budget=64, budget_mode=1).c()
+    call = lambda: fake_cuda.lib.mixkv_compress_layer(ONE, ONE, ONE, None, 1, 20032, C.byref(p), ONE, 1 << 30, None, ONE,
+                                                      ONE, ONE, *[None] * 6)
+    fake_cuda.reset(device=6)
+    assert call() == 0 and fake_cuda.launches()[-1].cluster == 4
+    fake_cuda.reset(device=7, ask_error=912)
+    assert call() == 0 and all(x.cluster == 1 for x in fake_cuda.launches()) and fake_cuda.last_error() == 0
+    fake_cuda.reset(device=7)
+    assert call() == 0 and fake_cuda.launches()[-1].cluster == 4
+
+
+def test_an_older_error_is_not_taken_for_a_launch_that_failed(fake_cuda):
+    fake_cuda.reset()
+    fake_cuda.runtime.cudaSetDevice(99)     # an error of the caller's own, not looked at yet
+    assert fake_cuda.last_error() != 0
+    assert fake_cuda.lib.mixkv_selftest_bounded_wait(ONE, None, None) == 0
