@@ -48,11 +48,6 @@ __device__ __forceinline__ void set_regs() {
   if constexpr (N > BASE) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N));
 }
 
-__device__ __forceinline__ void raise(int* status, volatile int* abort) {
-  *abort = 1;
-  if (status) atomicExch(status, MIXKV_ERR_TIMEOUT);
-}
-
 __device__ __forceinline__ f32x2 ex2_pair(f32x2 t2) {
   float a0, a1;
   unpack2(t2, a0, a1);
@@ -83,6 +78,7 @@ struct P1Bars {
   uint64_t tempty[4];
   uint64_t qfull;
   uint64_t qfree;
+  uint64_t mmas;     // the issuer's last ones
   TileCoord first;   // of the CTA's first tile
   uint32_t tmem_base;
   int abort;
@@ -245,6 +241,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     }
     mbar_init(&bars->qfull, 1);
     mbar_init(&bars->qfree, 1);
+    mbar_init(&bars->mmas, 1);
     bars->abort = 0;
     mbar_init_fence();
   }
@@ -293,10 +290,8 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
             ++it;
           }
         }
-        if (*abort) {
-          raise(status, abort);
-          drain_ring(bars->full, kP1Stages, it);
-        }
+        drain_ring(bars->full, kP1Stages, it);
+        drain_ring(&bars->qfull, 1, segn);
       }
     } else if (warp == kP1WarpMma) {
       // ---------------------------------------------------------------- MMA issuer
@@ -339,7 +334,8 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
             if (++ts == TS) ts = 0, tph ^= 1;
           }
         }
-        if (*abort && on) raise(status, abort);
+        umma_commit(&bars->mmas, on);
+        drain_ring(&bars->mmas, 1, 1);
       }
     }
   } else if (warp < kAuxWarp0) {
@@ -557,6 +553,7 @@ struct P2Bars {
   uint64_t qfull;
   uint64_t qfree;
   uint64_t kbready;
+  uint64_t mmas;    // the issuer's last ones
   TileCoord last;   // of the CTA's last tile
   SegList segs;     // pass 1's segments of the head that it belongs to
   uint32_t tmem_base;
@@ -622,6 +619,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     mbar_init(&bars->qfull, 1);
     mbar_init(&bars->qfree, 1);
     mbar_init(&bars->kbready, 4);          // the four warps that write the mean-key rows
+    mbar_init(&bars->mmas, 1);
     bars->abort = 0;
     mbar_init_fence();
   }
@@ -674,10 +672,8 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
           ++it;
         }
       }
-      if (*abort) {
-        raise(status, abort);
-        drain_ring(bars->kfull, kP2KStages, it);
-      }
+      drain_ring(bars->kfull, kP2KStages, it);
+      drain_ring(&bars->qfull, 1, segn);
     }
   } else if (warp == kWarpTmaV) {
     // ------------------------------------------------------------------ V producer
@@ -700,10 +696,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
           ++vit;
         }
       }
-      if (*abort) {
-        raise(status, abort);
-        drain_ring(bars->vfull, vstages, vit);
-      }
+      drain_ring(bars->vfull, vstages, vit);
     }
   } else if (warp == kWarpMma) {
     // ------------------------------------------------------------------ MMA issuer
@@ -742,7 +735,8 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         tph ^= ts ^ 1;
       }
     }
-    if (*abort && on) raise(status, abort);
+    umma_commit(&bars->mmas, on);
+    drain_ring(&bars->mmas, 1, 1);
   } else if (warp >= kEpiWarp0 && warp < kEpiWarp0 + kP2EpiWarps) {
     // ------------------------------------------------------------------ epilogue
     // Alternate tiles belong to alternate pairs of warpgroups, so inside a segment the pairs never wait

@@ -31,6 +31,7 @@ struct GBars {
   uint64_t afull, afree;
   uint64_t bfull[kGStages], bempty[kGStages];
   uint64_t tfull[2], tempty[2];
+  uint64_t mmas;   // the issuer's last ones
   uint32_t tmem_base;
   int abort;
 };
@@ -160,6 +161,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
       mbar_init(&bars->tfull[s], 1);
       mbar_init(&bars->tempty[s], NT == 128 ? kGEpiWarps : 4);
     }
+    mbar_init(&bars->mmas, 1);
     bars->abort = 0;
     mbar_init_fence();
   }
@@ -200,10 +202,8 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
           ++it;
         }
       }
-      if (*abort) {
-        drain_ring(bars->bfull, kGStages, it);
-        drain_ring(&bars->afull, 1, rown);
-      }
+      drain_ring(bars->bfull, kGStages, it);
+      drain_ring(&bars->afull, 1, rown);
     }
   } else if (warp == 1) {
     // -------------------------------------------------------------------- MMA issuer
@@ -249,6 +249,8 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
         if (w.row_last()) umma_commit(&bars->afree, on);
         ++tile;
       }
+      umma_commit(&bars->mmas, on);
+      drain_ring(&bars->mmas, 1, 1);
     }
   } else if (warp < kGEpiWarp0) {
     // -------------------------------------------------------------------- head means

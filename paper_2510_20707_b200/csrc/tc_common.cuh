@@ -373,8 +373,10 @@ struct SegList {
   }
 };
 
-// After an abort: let the copies in flight land before the CTA (and its shared memory) goes
-// away.  `it` loads were issued into a ring of `stages` barriers.
+// Lets what a role has started arrive before the CTA, its shared and its tensor memory go away: `it` loads were issued into
+// a ring of `stages` barriers.  A role does this at its end, whatever ended it: when it ends early because its tiles fit the
+// ring, a wait of another role may still run out, and nobody would wait for what is under way.  Else the consumers wait
+// for the same things anyway.
 __device__ __forceinline__ void drain_ring(uint64_t* full, int stages, int it) {
   for (int k = max(0, it - stages); k < it; ++k) {
     const unsigned long long t0 = global_ns();
