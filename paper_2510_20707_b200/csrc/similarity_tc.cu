@@ -273,7 +273,9 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
       const bool on_diag = w.c * NT < 128;    // inside the diagonal 128 x 128 tile: no mirrored store
       float* out = cells + (size_t)w.h * T * T;
       const int ts = tile & 1, tph = (tile >> 1) & 1;
-      if (!mbar_wait(&bars->tfull[ts], tph, abort)) break;
+      // A wait that runs out has no status word to go to: this tile's cells, and those of the CTA's tiles behind it (their
+      // waits fail at once then), come out as NaN instead of whatever the map's memory held.
+      const float inv_j = mbar_wait(&bars->tfull[ts], tph, abort) ? inv_b : __int_as_float(0x7fffffff);
       tc_fence_after();
       const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + ts * 128 + ch * 64;
 #pragma unroll 1
@@ -289,7 +291,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
           if (lane == 0) mbar_arrive(&bars->tempty[ts]);
         }
         if (j0 >= T || i0 >= T) continue;
-        const float sc = inv_i * inv_b;
+        const float sc = inv_i * inv_j;
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * sc);
         if (j0 + 31 >= T - 1 || j0 == i0) {   // the last block, or cells of the diagonal
