@@ -402,7 +402,8 @@ DecKernel dec_kernel(const bool wide, const int depth) {
 }
 
 // CTAs per unit and depth of their rings.  shared(n) and alone(n): clusters of n CTAs that are resident at once with
-// three CTAs to an SM and with one; even: the cache has room for max_rows rows of every head, so they may be of one length.
+// three CTAs to an SM and with one; even: the cache has room for max_rows rows of every head.  They may be of one length
+// then; the caches of a layer schedule and of budgets per head have that room too and are not, and the host cannot tell.
 struct DecodeShape {
   int S, depth;
 };
@@ -442,10 +443,14 @@ DecodeShape decode_shape(const long long units, const int max_rows, const bool e
   // 41 -> 31).  Long heads of one length leave DRAM no gap then, and the SMs that get their rows first run ahead with
   // their rings while the others decide the call (SMs 81 % active, with a step in registers 89): one slot pair in
   // flight per warp keeps them level (296 units of 5000 rows 129.9 -> 120.1 us, with operands in registers 118.4; 256 of
-  // 3400 80.8 -> 74.9, registers 79.5; 296 of 1000 30.7 -> 29.5).  Ragged heads in a cache of that very size lose by it
-  // (256 units of 500 to 2000 rows 37.5 -> 39.9 us), so short ones, which gain little, keep the ring of three.
+  // 3400 80.8 -> 74.9, registers 79.5; 296 of 1000 30.7 -> 29.5).  Heads of several lengths in a cache of that very size
+  // lose by it what an SM with one head, or with one that ends early, could have had in flight.  One pair against three, from
+  // 1300 to 8000 rows, in a layer schedule of taper 0.3 / 0.5 / 0.8, per-head shares of 1/4 to 1, and equal heads: 224 units
+  // -1 to +6 % / +2 to +6 / -1 to +11 / +2 to +8, equal -3 to -7; 240 to 256 units -2 to +1 / 0 to +5 / -1 to +8 / +3 to
+  // +5, equal -4 to -8; 280 and 296 -4 to +4 / -2 to +4 / +1 to +6 / -1 to +4, equal -6 to -10; 152 units nothing either way.
+  // So from 1.6 units per SM on, where equal heads gain what the others lose at worst, and not for short ones.
   const bool pair = S == 1 && units > sms && units <= 2LL * sms;
-  return {S, !pair ? kDecDepth : even && steps >= 80 ? kDecDepthEven : kDecDepthPair};
+  return {S, !pair ? kDecDepth : even && steps >= 80 && units * 5 >= sms * 8LL ? kDecDepthEven : kDecDepthPair};
 }
 
 }  // namespace

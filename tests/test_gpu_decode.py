@@ -133,10 +133,11 @@ def test_more_units_than_one_wave(NL, batch, H, G, lo, hi):
 
 
 @pytest.mark.parametrize("units,rows,G,ragged", [
-    (224, 1280, 7, False), (296, 1265, 16, False), (296, 1300, 4, True), (223, 1281, 9, True), (296, 1264, 4, True)])
+    (224, 1280, 7, False), (296, 1265, 16, False), (296, 1300, 4, True), (223, 1281, 9, True), (296, 1264, 4, True),
+    (237, 1280, 7, False), (237, 1281, 9, True), (236, 1281, 9, True)])
 def test_two_units_per_sm_in_a_cache_of_their_size(units, rows, G, ragged):
-    # the cache has room for max_rows rows of every head: from 80 steps on one slot pair per warp in flight, whether
-    # the heads are of one length or not (none, one, a step and one, all rows among them)
+    # the cache has room for max_rows rows of every head: from 80 steps and 237 units (1.6 per SM) on one slot pair per
+    # warp in flight, else three, whether the heads are of one length or not (none, one, a step and one, all rows among them)
     rng = np.random.default_rng(units + rows)
     counts = rng.integers(0, rows + 1, units) if ragged else np.full(units, rows)
     if ragged:

@@ -51,7 +51,8 @@ def test_no_more_clusters_than_are_resident(lib, chip):
 
 @pytest.mark.parametrize("units,rows,even,want", [
     (4, 512, 1, (8, 2)), (15, 1500, 1, (8, 4)), (16, 1500, 1, (8, 2)), (16, 8000, 1, (6, 4)), (17, 1500, 1, (6, 4)),
-    (28, 2500, 0, (8, 2)), (49, 1500, 1, (7, 2)), (896, 512, 0, (1, 2)), (256, 1264, 1, (1, 3)), (256, 1265, 1, (1, 1)), (256, 3400, 0, (1, 3)), (297, 3400, 1, (1, 2)), (560, 2500, 0, (2, 2)), (12, 60, 1, (1, 2))])
+    (28, 2500, 0, (8, 2)), (49, 1500, 1, (7, 2)), (896, 512, 0, (1, 2)), (256, 1264, 1, (1, 3)), (256, 1265, 1, (1, 1)), (256, 3400, 0, (1, 3)),
+    (236, 3400, 1, (1, 3)), (237, 3400, 1, (1, 1)), (296, 8000, 1, (1, 1)), (297, 3400, 1, (1, 2)), (560, 2500, 0, (2, 2)), (12, 60, 1, (1, 2))])
 def test_decode_shapes_as_measured(lib, units, rows, even, want):
     assert decode(lib, B200, units, rows, even) == want
 
