@@ -227,8 +227,10 @@ def test_prefix_longer_than_the_tail_cache():
 
 
 @pytest.mark.parametrize("H,lens,levels", [
-    (8, (16400,) * 19, 3),        # clusters of four, keys cached, the threshold is one of three key values
-    (8, (16400,) * 19, 1 << 20),  # clusters of four, keys cached, candidates listed and ranked
+    (8, (16400,) * 19, 3),        # shared out by the tail, two CTAs to an SM, the threshold is one of three key values
+    (8, (16400,) * 19, 1 << 20),  # the same, candidates listed and ranked
+    (9, (16400,) * 19, 3),        # clusters of four, keys cached, the threshold is one of three key values
+    (9, (16400,) * 19, 1 << 20),  # clusters of four, keys cached, candidates listed and ranked
     (8, (13016,) * 40, 700),      # clusters of two, keys not cached
     (8, (60016,), 5),             # cluster of eight, keys not cached, the threshold is one of five key values
     (8, (60016,), 1 << 20),       # cluster of eight, keys not cached, candidates listed and ranked
@@ -391,8 +393,9 @@ def test_threshold_search_edges(H, n, levels, want):
 
 
 @pytest.mark.parametrize("batch,H,P", [
-    (1, 8, 1024), (1, 8, 1025),                                # one CTA per sequence, two
-    (15, 8, 4100), (16, 8, 4100), (30, 8, 4100),               # clusters of eight, of four
+    (1, 8, 1024), (1, 8, 1025), (15, 8, 4100),                 # shared out by the tail
+    (1, 16, 512), (1, 16, 513), (15, 9, 4100),                 # budget kernel: one CTA per sequence, two, clusters of eight
+    (16, 8, 4100), (30, 8, 4100),                              # clusters of four
     (31, 8, 2100), (60, 8, 1030), (61, 8, 1030),               # of four; of two
     (33, 8, 4100), (34, 8, 4100), (64, 8, 1030)])              # the last of four, of two
 def test_adaptive_budget_cluster_edges(batch, H, P):

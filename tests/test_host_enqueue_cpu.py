@@ -119,3 +119,21 @@ def test_an_older_error_is_not_taken_for_a_launch_that_failed(fake_cuda):
     fake_cuda.runtime.cudaSetDevice(99)     # an error of the caller's own, not looked at yet
     assert fake_cuda.last_error() != 0
     assert fake_cuda.lib.mixkv_selftest_bounded_wait(ONE, None, None) == 0
+
+
+@pytest.mark.parametrize("batch,H,P,budget,tail", [
+    (1, 16, 512, 1, 1), (1, 16, 513, 2, 1), (15, 9, 4100, 8, 1), (16, 8, 4100, 4, 1), (30, 8, 4100, 4, 1), (33, 8, 4100, 4, 1),
+    (34, 8, 4100, 2, 1), (31, 8, 2100, 4, 1), (60, 8, 1030, 2, 1), (61, 8, 1030, 2, 1), (64, 8, 1030, 2, 1),
+    (19, 9, 16384, 4, 1), (40, 8, 13000, 2, 1), (1, 8, 60000, 8, 8),
+    (1, 8, 1024, 0, 8), (1, 8, 1025, 0, 8), (15, 8, 4100, 0, 8), (19, 8, 16384, 0, 8)])
+def test_adaptive_selection_takes_the_clusters_its_gpu_tests_name(fake_cuda, batch, H, P, budget, tail):
+    # test_gpu_parity.py: sizes at which the selection is compared with the oracle, by the number of CTAs that share a
+    # sequence in the budget kernel (0: the tail kernel shares the budgets out)
+    fake_cuda.reset(device=8, resident={3: 45, 4: 33, 5: 26, 6: 22, 7: 15, 8: 15})
+    p = binding.Params(kv_heads=H, gqa_ratio=1, window=16, budget=116, budget_mode=1).c()
+    cu = (C.c_int32 * (batch + 1))(*[b * (P + 16) for b in range(batch + 1)])
+    rc = fake_cuda.lib.mixkv_select(ONE, cu if batch > 1 else None, batch, P + 16, C.byref(p), ONE, 1 << 40, ONE, ONE, ONE,
+                                    None, None)
+    assert rc == 0
+    calls = [(x.kernel, x.cluster) for x in fake_cuda.launches()]
+    assert calls == [("k_budget", budget)] * (budget > 0) + [("k_tail", tail)]
