@@ -27,12 +27,14 @@ int mixkv_internal_select(const float* scores, const int32_t* cu_seqlens_host, i
 // The rules that split the work of a call over clusters, as functions of the sizes and of how many clusters of n CTAs a
 // device holds at once (alone[n] with one CTA per SM, paired[n] with two, shared[n] with three, n = 1 .. 8).  No device is
 // needed.  decode: CTAs per unit and the depth of their rings; tail, budget: CTAs per unit, per (sequence, layer) pair;
-// adapt: threads of a CTA when the tail shares adaptive budgets out, 0: when it does not.
+// adapt: threads of a CTA when the tail shares adaptive budgets out, 0: when it does not; gram: tiles of a map of `cells`
+// cells a side that a CTA takes in a run, 0: one contiguous share.
 void mixkv_internal_decode_shape(int64_t units, int32_t max_rows, int32_t even, int32_t sms, const int32_t* shared,
                                  const int32_t* alone, int32_t* ctas, int32_t* depth);
 int mixkv_internal_tail_clusters(int64_t units, int32_t candidates, int32_t sms, const int32_t* alone);
 int mixkv_internal_adapt_threads(int64_t sequences, int32_t heads, int32_t candidates, const int32_t* alone,
                                  const int32_t* paired);
+int mixkv_internal_gram_run(int32_t heads, int32_t cells, int32_t parts, int32_t whole_sectors, int64_t l2_bytes);
 int mixkv_internal_budget_clusters(int32_t pairs, int64_t keys_per_pair, const int32_t* alone);
 
 #ifdef __cplusplus

@@ -360,19 +360,34 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
   if (warp == 1) tmem_dealloc(tmem, 256);
 }
 
+// Bytes of L2 on the current device.
+long long device_l2_bytes() {
+  static std::atomic<int> cached[kMaxDevices];
+  const int dev = device_slot();
+  int n = dev < 0 ? 0 : cached[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (dev < 0 || !answered(cudaDeviceGetAttribute(&n, cudaDevAttrL2CacheSize, dev)) || n < 1) return 132644864;
+    cached[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
 // How the tiles are shared out: 0 contiguous (a CTA keeps its parts of I from tile to tile), else runs of so many in turn,
 // so that all CTAs together write whole rows of the map at a time.  That counts where the map goes to HBM: it leaves L2
-// in about the order in which it was written.
+// in about the order in which it was written.  Contiguous / in runs, us, B200 (L2 of 133 MB), maps in turn on four inputs:
 //   Rows that do not start on 32-byte sectors (T not a multiple of 8, or a map that does not): neighbouring tiles share
-//   sectors, and a sector that leaves half written is read again.  Runs of one, from a few dozen megabytes on: 8 heads
-//   x 2500 cells a side 89 -> 71 us, 4 x 2801 66 -> 55, 4 x 5001 211 -> 177, 8 x 1500 (72 MB) 35.1 -> 33.5.
-//   Whole sectors: only the largest maps gain (pages of HBM filled in one go): 4 x 8192 269 -> 211 us in runs of one (two
-//   parts), 2 x 8192 142 -> 134 and 4 x 5000 122 -> 112 in runs of two (three parts, where the parts of I weigh more);
-//   268 MB and less are as fast or up to 5 % faster contiguous.
-int gram_run(const void* cells, const int heads, const int T, const int nparts) {
-  const double mb = (double)heads * T * T * 4e-6;
-  if (T % 8 || (reinterpret_cast<uintptr_t>(cells) & 31)) return mb > 64. ? 1 : 0;
-  return mb > 300. ? (nparts == 2 ? 1 : 2) : 0;
+//   sectors, and a sector that leaves half written is read again.  Runs of one from half of L2 on: 4 heads x 1801 cells a
+//   side (52 MB) 36.7 / 36.4, x 2001 (64 MB) 41.2 / 36.7, x 2401 55.8 / 47.2, x 2801 (126 MB) 69.1 / 57.3, x 5001 (400 MB)
+//   212 / 175; blocks of 16, whose sums take longer, gain less: 8 x 1450 (67 MB) 43.9 / 45.9, x 1950 70.4 / 66.4.  (One
+//   map written over and over stays in L2 and would be better off contiguous up to 100 MB: 4 x 2001 32.2 / 34.2.)
+//   Whole sectors: only the largest maps gain (pages of HBM filled in one go), from 9/4 of L2 on: runs of one with two
+//   parts (4 x 4400, 310 MB, 88.9 / 77.7, x 5000 114 / 92, one map alone 4 x 8192 283 / 218), runs of two with three parts,
+//   where the parts of I weigh more (4 x 4400 90.7 / 87.3, x 5000 119.7 / 121.3, alone 4 x 5600 149 / 140, 4 x 8192
+//   317 / 287; below, 4 x 4000, 256 MB, 75.3 / 78.0).
+int gram_run(const int heads, const int T, const int nparts, const bool whole_sectors, const long long l2) {
+  const long long bytes = 4LL * heads * T * T;
+  if (!whole_sectors) return 2 * bytes > l2 ? 1 : 0;
+  return 4 * bytes > 9 * l2 ? (nparts == 2 ? 1 : 2) : 0;
 }
 
 template <int P, int NT, bool DEALT>
@@ -412,7 +427,8 @@ cudaError_t launch_gram(const GramArgs& g, cudaStream_t s) {
   const long long wide = tiles_per_head<128>(g.T);
   const bool narrow = wide * g.heads < device_sm_count();
   const long long per_head = narrow ? tiles_per_head<32>(g.T) : wide;
-  const int run = narrow ? 0 : gram_run(g.cells, g.heads, g.T, g.nparts);
+  const bool whole_sectors = g.T % 8 == 0 && (reinterpret_cast<uintptr_t>(g.cells) & 31) == 0;
+  const int run = narrow ? 0 : gram_run(g.heads, g.T, g.nparts, whole_sectors, device_l2_bytes());
   if (g.nparts == 2)
     return narrow ? launch_gram_t<2, 32, false>(g, per_head, 0, s)
            : run  ? launch_gram_t<2, 128, true>(g, per_head, run, s)
@@ -423,3 +439,7 @@ cudaError_t launch_gram(const GramArgs& g, cudaStream_t s) {
 }
 
 }  // namespace mixkv
+
+extern "C" int mixkv_internal_gram_run(int32_t heads, int32_t cells, int32_t parts, int32_t whole_sectors, int64_t l2_bytes) {
+  return mixkv::gram_run(heads, cells, parts, whole_sectors != 0, l2_bytes);
+}

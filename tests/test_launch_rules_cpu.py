@@ -80,3 +80,11 @@ def test_adaptive_budgets_in_the_tail_as_measured(lib):
     # a device, or a part of one, that holds no such cluster
     none = (148, 74) + (0,) * 6
     assert [threads(1, 2, 700, none, none), threads(1, 4, 700, none, none), threads(1, 4, 20000, none, none)] == [1024, 0, 0]
+
+
+def test_maps_are_dealt_out_by_what_l2_holds(lib):
+    run = lambda heads, T, parts, whole, l2=132644864: lib.mixkv_internal_gram_run(heads, T, parts, whole, C.c_int64(l2))
+    assert [run(4, 2035, 2, 0), run(4, 2036, 2, 0), run(4, 2036, 3, 0)] == [0, 1, 1]
+    assert [run(4, 4312, 2, 1), run(4, 4320, 2, 1), run(4, 4320, 3, 1), run(4, 2048, 3, 1)] == [0, 1, 2, 0]
+    # half the cache: the same at half the size; a map past 32 bits of bytes
+    assert [run(2, 2036, 2, 0, 132644864 // 2), run(2, 4320, 3, 1, 132644864 // 2), run(8, 65535, 2, 0)] == [1, 2, 1]
