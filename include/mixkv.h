@@ -309,14 +309,15 @@ int mixkv_decode_attention(const void* K_cache, const void* V_cache,
                            int32_t head_dim, float softmax_scale, int32_t max_rows, float* out,
                            void* stream);
 
-/* Number of kernels one mixkv_compress_layer[s] call with events enqueues, and the name of the
+/* Number of kernels one mixkv_compress_layer[s] call WITH events enqueues, and the name of the
  * i-th of them (NULL when i is out of range), for the measurement hook.  The route depends on the
  * shape: fixed budgets take three kernels (pass1, pass2, tail; max pooling adds poolsum) while
  * the candidates of the longest sequence fit the tail kernel's shared memory (P_b <= 131072)
  * and add the unfused mix kernel beyond that; adaptive budgets take the unfused route with
- * the budget kernel (without events, calls of few heads share them out in the tail kernel: two
- * launches fewer).  The _for variants take the shape and follow the route the call
- * takes; the short forms assume the fused route where it exists. */
+ * the budget kernel.  Without events, calls of few heads with adaptive budgets share them out in the
+ * tail kernel: mixpool and budget are not launched, the results are the same bit for bit, and the
+ * hook cannot time that tail.  The _for variants take the shape and follow the route a call with
+ * events takes; the short forms assume the fused route where it exists. */
 int mixkv_launches_per_layer(const mixkv_params* p);
 const char* mixkv_stage_name(const mixkv_params* p, int32_t i);
 int mixkv_launches_for(const mixkv_params* p, int32_t n_layers, int32_t batch,

@@ -14,6 +14,11 @@ name but for :func:`scores`, :func:`scores_static` and :func:`select`, which tak
 
 The calls may be made by several threads at once (the interpreter lock is given up inside them); a
 ``workspace`` then belongs to one of them at a time, on one stream too.
+
+A call runs on ``stream`` (a torch stream; default: the current one), and what it allocates, its outputs
+among it, belongs to that stream as if it were the current one: the caller orders other streams that read
+the outputs behind it, and tells the allocator of them (``Tensor.record_stream``) before it lets go of them.
+Inputs, like those of any call on another stream than their own, are the caller's to keep until it is done.
 """
 from __future__ import annotations
 
@@ -204,8 +209,10 @@ def stage_names(params: Params):
 
 
 def stage_names_for(params: Params, n_layers: int, batch: int, max_seq_len: int):
-    """Names of the kernels a call of this shape enqueues (mixkv_launches_for /
-    mixkv_stage_name_for): the route depends on the longest sequence and the number of units."""
+    """Names of the kernels a call of this shape enqueues when it is given ``trace_events``
+    (mixkv_launches_for / mixkv_stage_name_for): the route depends on the longest sequence and the
+    number of units.  Without events, calls of few heads with adaptive budgets take another one (mix,
+    budgets and selection in one kernel, the same results): their tail cannot be timed with events."""
     pc = params.c()
     lib = load_library()
     n = int(lib.mixkv_launches_for(C.byref(pc), n_layers, batch, max_seq_len))
@@ -257,7 +264,8 @@ def compress_layer(K: torch.Tensor, V: torch.Tensor, Q: torch.Tensor, params: Pa
                    want_aux: bool = True, trace_events=None) -> Dict[str, torch.Tensor]:
     """mixkv_compress_layer.  Returns K_out / V_out [batch*H*B, 128] (rows beyond
     out_row_offsets[-1] are untouched), out_row_offsets and, if want_aux, idx / counts /
-    idx_offsets / s_comp.  `out` lets a caller reuse output tensors across calls."""
+    idx_offsets / s_comp.  `out` lets a caller reuse output tensors across calls.  `trace_events`: a
+    ctypes array of cudaEvent_t handles, recorded around the kernels of :func:`stage_names_for`."""
     events, n_events = (0, 0) if trace_events is None else _events(trace_events)
     return (_host_module or _host()).compress_layer(K, V, Q, params, cu_seqlens, rbar_in, workspace, stream,
                                                     out, want_aux, events, n_events)
@@ -293,7 +301,8 @@ def layer_budget_schedule(n_layers: int, budget: int, window: int, taper_permill
 
 def similarity_map(X: torch.Tensor, block: int, want_mean: bool = True, stream=None):
     """mixkv_similarity_map: X [heads, L, 128] bf16 device tensor -> (cells [heads, T, T] fp32,
-    mean [heads] fp32 or None): block-mean cosine similarity of the rows of every head."""
+    mean [heads] fp32 or None): block-mean cosine similarity of the rows of every head.  (A cell
+    that a wait inside the kernel ran out on is NaN: there is no status word.)"""
     return (_host_module or _host()).similarity_map(X, block, want_mean, stream)
 
 
