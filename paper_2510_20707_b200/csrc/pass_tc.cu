@@ -534,7 +534,8 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
 // 4 x 32768 keys, G*W = 224, 359 us; as here 333 us; split like this but without the pieces 359 us again.)
 //
 // A CTA walks its tiles backwards: pass 1 has read (about) the same tiles in ascending order, so the K that is
-// still in L2 from there is the end of every CTA's range.  K and V are loaded evict-first, which keeps those lines,
+// still in L2 from there is the end of every CTA's range (77 MB of it: 4 layers of 4 x 32768 keys, 268 MB of K and V, 191 MB
+// read from DRAM behind pass 1, 272 with cold caches).  K and V are loaded evict-first, which keeps those lines,
 // and the scores written for the tail, from being driven out by what is not read again.
 constexpr int kP2EpiWarps = 16;                  // warps 4..19
 constexpr int kP2AuxWarp0 = kEpiWarp0 + kP2EpiWarps;   // warps 20..23: value norms

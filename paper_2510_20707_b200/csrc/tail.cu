@@ -1184,7 +1184,7 @@ bool adapt_pairs_fit(const int P) {
 // mix, budget and tail kernels are as good.  Every thread reads its bins of all heads over distributed shared memory,
 // so 1024 threads, as long as all clusters are resident with an SM to each CTA.  Where they are not, 512 threads and two
 // CTAs to an SM, all resident that way; clusters of seven and eight gain that way on long heads only.  Heads too long for
-// two to share an SM take 1024 threads in more than one wave.  One layer of so many sequences, heads x keys, whole calls,
+// two to share an SM take 1024 threads in more than one wave.  (Layer, sequence) pairs of heads x keys, whole calls,
 // three kernels / this, us (and with 256 threads for heads of 1024 keys and less, as it once was):
 //   all resident, 1024: 4 of 4 x 1024 to 8 x 24576 all faster: 4 of 8 x 760 36.2 / 31.5 (68.9), 33 of 4 x 760 47.3 / 40.0
 //     (56.1), 1 of 4 x 4300 40.3 / 32.2, 15 of 8 x 9000 159 / 150, 74 of 2 x 17000 380 / 348, 15 of 8 x 24500 471 / 427
