@@ -228,9 +228,14 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   // reach accumulator lanes that nobody reads.
   unsigned char* sQ = base;                    // 2 halves x [NQ x 128 B]
   unsigned char* sK = sQ + 2 * NQ * 128;       // kP1Stages x 32 KB
-  float* sks = reinterpret_cast<float*>(sK + kP1Stages * kTileBytes);  // [aux warps][128] key-sum exchange
-  float2* sxs = reinterpret_cast<float2*>(sks + kP1AuxWarps * 128);    // [kP1XRows] row statistics handed over
-  P1Bars* bars = reinterpret_cast<P1Bars*>(sxs + kP1XRows);
+  // At addresses that the compiler knows.  Behind the tiles, whose place depends on NQ, every role kept the base of the
+  // barriers in a register and the epilogue spilled: 2676 clocks per tile of 28 layers of 4 x 32768 keys at G*W = 224,
+  // 2502 like this; 1563 and 1494 of 32 layers of 8 x 16384 keys at 128.  (k_pass2 comes out the other way round, 2548
+  // and 2630, and keeps its own behind its tiles.)
+  __shared__ __align__(16) float sks[kP1AuxWarps * 128];   // [aux warps][128] key-sum exchange
+  __shared__ float2 sxs[kP1XRows];                         // row statistics handed over
+  __shared__ P1Bars p1_bars;
+  P1Bars* const bars = &p1_bars;
   const int lo = cta_first_tile(blockIdx.x, split1(st));
   const int hi = cta_first_tile(blockIdx.x + 1, split1(st));
   volatile int* abort = &bars->abort;
@@ -1072,9 +1077,10 @@ bool map_q(const LaunchCtx& c, const void* Q, CUtensorMap* tm) {
 
 // Dynamic shared memory of the passes: what the kernels carve up, behind up to 1023 bytes that align its start.
 constexpr size_t pass1_smem(int NQ) {
-  return 1024 + (size_t)2 * NQ * 128 + (size_t)p1_stages(NQ) * kTileBytes + kP1AuxWarps * 128 * 4 +
-         kP1XRows * 8 + sizeof(P1Bars);
+  return 1024 + (size_t)2 * NQ * 128 + (size_t)p1_stages(NQ) * kTileBytes;
 }
+// What is left of it next to pass 1's static part.
+constexpr size_t kP1SmemLimit = kSmemLimit - (kP1AuxWarps * 128 * 4 + kP1XRows * 8 + sizeof(P1Bars) + 63) / 64 * 64;
 constexpr size_t pass2_smem(int NQ, int vstages) {
   return 1024 + (size_t)2 * (NQ + kExtraRows) * 128 + kP2KStages * kTileBytes +
          (size_t)vstages * kVSubBytes + 1024 * 4 + 64 * 4 + sizeof(P2Bars) + 64;
@@ -1087,7 +1093,7 @@ constexpr int pass2_vstages(int NQ) {
 }
 constexpr bool passes_fit() {
   for (int NQ = 16; NQ <= kMaxNQ; NQ += 16)
-    if (pass1_smem(NQ) > kSmemLimit || pass2_smem(NQ, pass2_vstages(NQ)) > kSmemLimit || p1_stages(NQ) > kP1MaxStages)
+    if (pass1_smem(NQ) > kP1SmemLimit || pass2_smem(NQ, pass2_vstages(NQ)) > kSmemLimit || p1_stages(NQ) > kP1MaxStages)
       return false;
   return true;
 }
@@ -1122,13 +1128,13 @@ cudaError_t launch_pass1(const LaunchCtx& c, const void* K, const void* Q, int* 
   static std::atomic<bool> done1[kMaxDevices], done2[kMaxDevices];
   if (c.st.NQ <= 128) {
     const size_t smem = pass1_smem(c.st.NQ);
-    cudaError_t e = ensure_smem(k_pass1<1>, kSmemLimit, done1);
+    cudaError_t e = ensure_smem(k_pass1<1>, kP1SmemLimit, done1);
     if (e != cudaSuccess) return e;
     return launch_pdl(k_pass1<1>, dim3(c.st.g1), dim3(kP1Threads), smem, c.stream, 1, tmK, tmQ, c.st,
                       c.ws, c.scale_log2e, (int)c.clear_status, status);
   }
   const size_t smem = pass1_smem(c.st.NQ);
-  cudaError_t e = ensure_smem(k_pass1<2>, kSmemLimit, done2);
+  cudaError_t e = ensure_smem(k_pass1<2>, kP1SmemLimit, done2);
   if (e != cudaSuccess) return e;
   return launch_pdl(k_pass1<2>, dim3(c.st.g1), dim3(kP1Threads), smem, c.stream, 1, tmK, tmQ, c.st,
                     c.ws, c.scale_log2e, (int)c.clear_status, status);
