@@ -2,6 +2,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "common.cuh"
@@ -54,6 +55,20 @@ int check_params(const mixkv_params* p) {
   return MIXKV_OK;
 }
 
+// How `tiles` are split over at most `sms` CTAs; per_head: the tiles of every head, 0 where heads differ.  A CTA that
+// goes from one head to the next waits for the next one's queries, and in pass 2 for its folds, with nothing to do: about
+// two tiles' time.  So no CTA works on two heads where that lengthens the longest share by a tile at most (one tile list
+// / this, us: one layer of 4 x 32768 keys 49.8 / 47.5, 4 x 6000 30.1 / 26.9, 8 x 12000 40.8 / 39.9, 8 x 30000 at G*W = 128,
+// where it is that tile, 51.7 / 50.4; 2 x 20000 and 14 layers of it level; with three tiles allowed nothing changes).
+Split split_tiles(const int tiles, const int per_head, const int sms) {
+  const int g = std::min(tiles, sms), units = per_head ? tiles / per_head : 0;
+  if (units > 0 && units <= g) {
+    const int p = std::min(per_head, g / units);
+    if ((per_head + p - 1) / p <= (tiles + g - 1) / g + 1) return {per_head, p, per_head / p, per_head % p, units * p};
+  }
+  return {tiles, g, tiles / g, tiles % g, g};
+}
+
 // Builds the sequence table from the host offsets (or a single length).
 int build_table(const mixkv_params* p, const int32_t* cu, int batch, int L, int layers,
                 SeqTable* st, int* max_len) {
@@ -87,11 +102,15 @@ int build_table(const mixkv_params* p, const int32_t* cu, int batch, int L, int 
   st->nt2 = st->tile2_start[batch];
   const long long t1 = (long long)layers * st->nt1, t2 = (long long)layers * st->nt2;
   if (t1 > 0x3fffffffLL) return MIXKV_ERR_UNSUPPORTED;
+  // tiles of every head, 0 where sequences differ
+  int head1 = st->tile1_start[1] / st->H, head2 = st->tile2_start[1] / st->H;
+  for (int b = 1; b < batch; ++b) {
+    if (st->tile1_start[b + 1] - st->tile1_start[b] != st->tile1_start[1]) head1 = 0;
+    if (st->tile2_start[b + 1] - st->tile2_start[b] != st->tile2_start[1]) head2 = 0;
+  }
   const int sms = device_sm_count();
-  st->g1 = t1 < sms ? (int)t1 : sms;
-  st->g2 = t2 < sms ? (int)t2 : sms;
-  st->q1 = (int)(t1 / st->g1), st->r1 = (int)(t1 % st->g1);
-  st->q2 = (int)(t2 / st->g2), st->r2 = (int)(t2 % st->g2);
+  st->sp1 = split_tiles((int)t1, head1, sms);
+  st->sp2 = split_tiles((int)t2, head2, sms);
   *max_len = mx;
   return MIXKV_OK;
 }
@@ -608,6 +627,13 @@ int mixkv_launches_per_layer(const mixkv_params* p) {
   if (!p) return 0;
   const char* names[8];
   return layer_stages(p, true, names);
+}
+
+int mixkv_internal_split_tiles(int32_t tiles, int32_t per_head, int32_t sms, int32_t* first, int32_t* owner) {
+  const Split sp = split_tiles(tiles, per_head, sms);
+  for (int c = 0; c <= sp.g; ++c) first[c] = cta_first_tile(c, sp);
+  for (int t = 0; t < tiles; ++t) owner[t] = tile_owner(t, sp);
+  return sp.g;
 }
 
 const char* mixkv_status_string(int status) {

@@ -22,6 +22,23 @@ constexpr int kExtraRows = 16;       // rows appended to the query tile in pass 
 constexpr int kMaxCluster = 8;       // CTAs of a cluster (the portable limit)
 constexpr float kLog2e = 1.4426950408889634f;
 
+// Tiles split contiguously over g CTAs, in (layer, sequence, head) order.  Runs of n tiles are shared out over p CTAs each
+// (p <= n): the first r of them take q + 1 tiles, the others q.  Either one run of all tiles over all CTAs, or, where
+// that makes no CTA's share longer than split_tiles() allows, a run per head, so that no CTA works on two of them.
+struct Split {
+  int n, p, q, r, g;
+};
+// First tile of CTA c.
+__host__ __device__ __forceinline__ int cta_first_tile(const int c, const Split& sp) {
+  const int run = c / sp.p, k = c - run * sp.p;
+  return run * sp.n + k * sp.q + (k < sp.r ? k : sp.r);
+}
+// CTA whose contiguous range contains tile t.
+__host__ __device__ __forceinline__ int tile_owner(const int t, const Split& sp) {
+  const int run = t / sp.n, k = t - run * sp.n, big = sp.r * (sp.q + 1);
+  return run * sp.p + (k < big ? k / (sp.q + 1) : sp.r + (k - big) / sp.q);
+}
+
 // Everything a kernel needs to find its slice of the ragged batch.
 struct SeqTable {
   int layers;                        // layers handled by one call (an outer batch dimension)
@@ -32,17 +49,10 @@ struct SeqTable {
   int pchunk_start[kMaxBatch + 1];   // prefix sum of candidate chunks
   // persistent 128-key tile schedules of the two tensor-core passes, (b, h, t) order
   // Tiles of one layer: nt1 over all L keys (pass 1), nt2 over the P candidate keys (pass 2).
-  // layers * nt tiles are split over g CTAs: layers * nt = q * g + r.
-  int nt1, g1, q1, r1;
-  int nt2, g2, q2, r2;
+  int nt1, nt2;
+  Split sp1, sp2;                    // of the tiles of all layers over the CTAs of the passes
   int tile1_start[kMaxBatch + 1];    // prefix sum of H * ceil(L_b / 128)
   int tile2_start[kMaxBatch + 1];    // prefix sum of H * ceil(P_b / 128)
-};
-
-// nt tiles split contiguously over g CTAs (g <= nt): the first r CTAs take q + 1 tiles, the
-// others q.
-struct Split {
-  int nt, g, q, r;
 };
 
 // Device workspace carve-up (all pointers into the caller's workspace).

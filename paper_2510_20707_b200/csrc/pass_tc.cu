@@ -102,51 +102,63 @@ __device__ __forceinline__ float2 merge_stats(const float2 a, const float2 b) {
 // ---- per-head folds (pass 2, at the start of a segment): what the segments of pass 1 left
 // for a (layer, sequence, head) becomes what pass 2 needs of it.
 //
-// kFoldRows row statistics and kFoldSums key sums are in flight per round and thread, two threads share a window
-// row.  Short rounds: code that runs once per segment costs its instruction fetches, and forty loads unrolled were
-// 6 KB of it (one layer of 4 x 1024 keys 23.6 us, with short rounds 22.5; 37 segments per head, a one-layer
-// call of 4 x 32768, cost the same either way).
-constexpr int kFoldRows = 6, kFoldSums = 8;
-// Window row q over segments [e_lo, e_hi): their (reference, sum) pairs merged under the largest reference.
-__device__ __forceinline__ float2 fold_row_stats(const float2* rowstat, const SegList& sl, const int e_lo,
-                                                 const int e_hi, const int NQ, const int q) {
-  float M = -1e30f, Z = 0.f;
+// Bound by round trips to L2, so a head's segments are spread over lanes (row statistics) and warps (key sums), and
+// kFoldDepth 16-byte loads of a thread are in flight together: up to 20 segments are one round, the 37 of a
+// one-layer call of 4 x 32768 keys two.  (Rounds stay short: code that runs once per segment costs its instruction
+// fetches.)  With a thread or two to a row, and one to a key dimension, that call had its normalisers 5.4 us after
+// pass 1, now 3.3; that of 4 x 1024 keys, 8 segments, 2.6 and 1.5.
+constexpr int kFoldDepth = 5;
+// Window rows 2 rp, 2 rp + 1 (rp = 8 * warp + (lane & 7)) over all segments of the head, four segments side by side
+// in a warp: (reference, sum) pairs merged under the largest reference, the same in the four lanes of a row pair.
+__device__ __forceinline__ void fold_row_stats(const float2* rowstat, const SegList& sl, const int NQ, const int rp,
+                                               const int lane, float2& s0, float2& s1) {
+  s0 = s1 = make_float2(-1e30f, 0.f);
 #pragma unroll 1
-  for (int e0 = e_lo; e0 < e_hi; e0 += kFoldRows) {
-    float2 v[kFoldRows];
+  for (int e0 = lane >> 3; e0 < sl.nseg; e0 += 4 * kFoldDepth) {
+    float4 v[kFoldDepth];
 #pragma unroll
-    for (int k = 0; k < kFoldRows; ++k) {
-      v[k] = make_float2(-1e30f, 0.f);
-      if (e0 + k < e_hi) v[k] = __ldcg(rowstat + (size_t)sl.start(e0 + k) * NQ + q);
+    for (int k = 0; k < kFoldDepth; ++k) {
+      v[k] = make_float4(-1e30f, 0.f, -1e30f, 0.f);
+      if (e0 + 4 * k < sl.nseg && 2 * rp < NQ)
+        v[k] = __ldcg(reinterpret_cast<const float4*>(rowstat + (size_t)sl.start(e0 + 4 * k) * NQ) + rp);
     }
-    float mx = M;
+    float m0 = s0.x, m1 = s1.x;
 #pragma unroll
-    for (int k = 0; k < kFoldRows; ++k) mx = fmaxf(mx, v[k].x);
-    Z *= ex2(M - mx);
+    for (int k = 0; k < kFoldDepth; ++k) m0 = fmaxf(m0, v[k].x), m1 = fmaxf(m1, v[k].z);
+    s0.y *= ex2(s0.x - m0), s1.y *= ex2(s1.x - m1);
+    s0.x = m0, s1.x = m1;
 #pragma unroll
-    for (int k = 0; k < kFoldRows; ++k) Z = fmaf(v[k].y, ex2(v[k].x - mx), Z);
-    M = mx;
+    for (int k = 0; k < kFoldDepth; ++k) {
+      s0.y = fmaf(v[k].y, ex2(v[k].x - m0), s0.y);
+      s1.y = fmaf(v[k].w, ex2(v[k].z - m1), s1.y);
+    }
   }
-  return make_float2(M, Z);
+#pragma unroll
+  for (int o = 8; o <= 16; o <<= 1) {
+    s0 = merge_stats(s0, make_float2(__shfl_xor_sync(0xffffffffu, s0.x, o), __shfl_xor_sync(0xffffffffu, s0.y, o)));
+    s1 = merge_stats(s1, make_float2(__shfl_xor_sync(0xffffffffu, s1.x, o), __shfl_xor_sync(0xffffffffu, s1.y, o)));
+  }
 }
-// Component kt of the unit-key sum over all segments of the head.
-__device__ __forceinline__ float fold_key_sums(const float* ksum, const SegList& sl, const int kt) {
-  float sum = 0.f;
+// Components 4 lane .. 4 lane + 3 of the unit-key sum over segments w, w + 4, ...
+__device__ __forceinline__ float4 fold_key_sums(const float* ksum, const SegList& sl, const int w, const int lane) {
+  float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
-  for (int e0 = 0; e0 < sl.nseg; e0 += kFoldSums) {
-    float v[kFoldSums];
+  for (int e0 = w; e0 < sl.nseg; e0 += 4 * kFoldDepth) {
+    float4 v[kFoldDepth];
 #pragma unroll
-    for (int k = 0; k < kFoldSums; ++k)
-      v[k] = e0 + k < sl.nseg ? __ldcg(ksum + (size_t)sl.start(e0 + k) * kHeadDim + kt) : 0.f;
+    for (int k = 0; k < kFoldDepth; ++k)
+      v[k] = e0 + 4 * k < sl.nseg
+                 ? __ldcg(reinterpret_cast<const float4*>(ksum + (size_t)sl.start(e0 + 4 * k) * kHeadDim) + lane)
+                 : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < kFoldSums; ++k) sum += v[k];
+    for (int k = 0; k < kFoldDepth; ++k) sum.x += v[k].x, sum.y += v[k].y, sum.z += v[k].z, sum.w += v[k].w;
   }
   return sum;
 }
 // The pass-1 segments of a head.
 __device__ __forceinline__ SegList pass1_segments(const SeqTable& st, const int layer, const int b, const int h) {
   const int per_head = (st.tile1_start[b + 1] - st.tile1_start[b]) / st.H;
-  return SegList(layer * st.nt1 + st.tile1_start[b] + h * per_head, per_head, split1(st));
+  return SegList(layer * st.nt1 + st.tile1_start[b] + h * per_head, per_head, st.sp1);
 }
 
 // The running softmax statistics of a query row are a pair (m, z): z = sum over the keys seen
@@ -236,8 +248,8 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   __shared__ float2 sxs[kP1XRows];                         // row statistics handed over
   __shared__ P1Bars p1_bars;
   P1Bars* const bars = &p1_bars;
-  const int lo = cta_first_tile(blockIdx.x, split1(st));
-  const int hi = cta_first_tile(blockIdx.x + 1, split1(st));
+  const int lo = cta_first_tile(blockIdx.x, st.sp1);
+  const int hi = cta_first_tile(blockIdx.x + 1, st.sp1);
   volatile int* abort = &bars->abort;
 
   pdl_launch_dependents();
@@ -607,13 +619,13 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   unsigned char* sV = sK + kP2KStages * kTileBytes;   // vstages x 16 KB
   float* sbq = reinterpret_cast<float*>(sV + vstages * kVSubBytes);  // [256] negated normalisers
   float* sxp = sbq + 256;                     // [2][128] partial column sums of the second column halves
-  float2* sxf = reinterpret_cast<float2*>(sxp + 256);   // [256] row statistics of the second half of the segments
-  float* sred = reinterpret_cast<float*>(sxf + 256);    // [64]: 2 x 16 epilogue, 12 value norms, 4 mean key
+  float* skp = sxp + 256;                     // [4][128] parts of the unit-key sum
+  float* sred = skp + 512;    // [64]: 2 x 16 epilogue, 12 value norms, 4 mean key
   P2Bars* bars = reinterpret_cast<P2Bars*>(sred + 64);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int lo = cta_first_tile(blockIdx.x, split2(st));
-  const int hi = cta_first_tile(blockIdx.x + 1, split2(st));
+  const int lo = cta_first_tile(blockIdx.x, st.sp2);
+  const int hi = cta_first_tile(blockIdx.x + 1, st.sp2);
   volatile int* abort = &bars->abort;
   constexpr int kWarpTmaV = 2;
 
@@ -759,7 +771,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     // ------------------------------------------------------------------ epilogue
     // Alternate tiles belong to alternate pairs of warpgroups, so inside a segment the pairs never wait
     // for each other; each pair leaves its own partial score statistics.  At the start of a segment the
-    // 512 threads fold the row statistics of the head together, two threads to a window row, into the
+    // 512 threads fold the row statistics of the head together, four lanes to a pair of window rows, into the
     // normaliser table all groups read.  Nobody leaves the tile loop early: after an abort every
     // wait fails at once, so the named barriers stay matched.
     const int quarter = warp & 3, grp = (warp - kEpiWarp0) >> 2;
@@ -780,19 +792,15 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     for (RevSegIter sg(st.tile2_start, st.batch, H, bars->last, lo, hi); sg.valid(); sg.next()) {
       const int P = st.cu[sg.b + 1] - st.cu[sg.b] - W;
       {
-        const SegList sl = pass1_segments(st, sg.layer, sg.b, sg.h);
-        const int q = et & 255, mid = sl.nseg > kFoldRows ? (sl.nseg + 1) >> 1 : sl.nseg;
-        float2 mz = make_float2(-1e30f, 0.f);
-        if (q < NQ) {
-          if (et < 256) mz = fold_row_stats(ws.rowstat, sl, 0, mid, NQ, q);
-          else sxf[q] = fold_row_stats(ws.rowstat, sl, mid, sl.nseg, NQ, q);
-        }
-        named_bar_sync(5, kP2EpiWarps * 32);   // (also: the previous segment's readers of sbq are done)
-        // the negated log2 normaliser of the row with the 1/W of the window mean folded in
-        if (et < NQ) {
-          if (mid < sl.nseg) mz = merge_stats(mz, sxf[et]);
-          sbq[et] = -(mz.x + log2f(mz.y)) - log2W;
-        }
+        // the negated log2 normalisers of the rows with the 1/W of the window mean folded in
+        const SegList sl = tile == 0 ? bars->segs : pass1_segments(st, sg.layer, sg.b, sg.h);
+        const int rp = (et >> 5) * 8 + (lane & 7);
+        float2 s0, s1;
+        fold_row_stats(ws.rowstat, sl, NQ, rp, lane, s0, s1);
+        if (tile > 0) named_bar_sync(5, kP2EpiWarps * 32);   // the previous segment's readers of sbq are done
+        if (lane < 8 && 2 * rp < NQ)
+          *reinterpret_cast<float2*>(sbq + 2 * rp) =
+              make_float2(-(s0.x + log2f(s0.y)) - log2W, -(s1.x + log2f(s1.y)) - log2W);
         named_bar_sync(5, kP2EpiWarps * 32);
       }
       float dmin = INFINITY, dmax = -INFINITY, dsum = 0.f, exw = 0.f;
@@ -889,8 +897,8 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     }
   } else if (warp >= kP2AuxWarp0) {
     // ------------------------------------------------------------------ mean key, value norms
-    // At the start of a segment: fold the unit-key sums of the head's pass-1 segments (one
-    // dimension per thread) and write the bf16 hi / lo / lo2 split of the mean unit key into the
+    // At the start of a segment: fold the unit-key sums of the head's pass-1 segments (every fourth of them
+    // per warp, then one dimension per thread) and write the bf16 hi / lo / lo2 split of the mean unit key into the
     // three extra B rows; the CTA that starts on the head's first tile also leaves the redundancy
     // of Eq. 4, which needs nothing but the squared norm of that sum.  Per tile: warps 20, 21 read the first 64 rows of the V
     // tile, warps 22, 23 the last 64; one row per thread from the swizzled half tile.
@@ -899,18 +907,21 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     int vs = sub, vph = 0, segn = 0;   // V stage of this pair of warps: half tiles sub, sub + 2, ...
     for (RevSegIter sg(st.tile2_start, st.batch, H, bars->last, lo, hi); sg.valid(); sg.next()) {
       const int L = st.cu[sg.b + 1] - st.cu[sg.b], P = L - W;
-      const float ks =
-          fold_key_sums(ws.ksum, segn == 0 ? bars->segs : pass1_segments(st, sg.layer, sg.b, sg.h), vt);
+      const float4 part =
+          fold_key_sums(ws.ksum, segn == 0 ? bars->segs : pass1_segments(st, sg.layer, sg.b, sg.h), vt >> 5, lane);
+      if (segn > 0) {   // the previous segment's MMAs must be done with the B rows, its readers with the parts
+        if (vt == 0) mbar_wait(&bars->qfree, (segn - 1) & 1, abort);
+        named_bar_sync(4, 128);
+      }
+      *reinterpret_cast<float4*>(skp + (vt >> 5) * kHeadDim + 4 * lane) = part;
+      named_bar_sync(4, 128);
+      const float ks = (skp[vt] + skp[kHeadDim + vt]) + (skp[2 * kHeadDim + vt] + skp[3 * kHeadDim + vt]);
       const float kb = ks / (float)L;   // mean unit key
       __nv_bfloat16 parts[3];
       parts[0] = __float2bfloat16_rn(kb);
       const float r1 = kb - __bfloat162float(parts[0]);
       parts[1] = __float2bfloat16_rn(r1);
       parts[2] = __float2bfloat16_rn(r1 - __bfloat162float(parts[1]));
-      if (segn > 0) {   // the previous segment's MMAs must be done with the B rows
-        if (vt == 0) mbar_wait(&bars->qfree, (segn - 1) & 1, abort);
-        named_bar_sync(4, 128);
-      }
       {
         unsigned char* hb = sQ + (vt >> 6) * NB * 128 + (vt & 7) * 2;
         const int chunk = (vt & 63) >> 3;
@@ -1130,13 +1141,13 @@ cudaError_t launch_pass1(const LaunchCtx& c, const void* K, const void* Q, int* 
     const size_t smem = pass1_smem(c.st.NQ);
     cudaError_t e = ensure_smem(k_pass1<1>, kP1SmemLimit, done1);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_pass1<1>, dim3(c.st.g1), dim3(kP1Threads), smem, c.stream, 1, tmK, tmQ, c.st,
+    return launch_pdl(k_pass1<1>, dim3(c.st.sp1.g), dim3(kP1Threads), smem, c.stream, 1, tmK, tmQ, c.st,
                       c.ws, c.scale_log2e, (int)c.clear_status, status);
   }
   const size_t smem = pass1_smem(c.st.NQ);
   cudaError_t e = ensure_smem(k_pass1<2>, kP1SmemLimit, done2);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_pass1<2>, dim3(c.st.g1), dim3(kP1Threads), smem, c.stream, 1, tmK, tmQ, c.st,
+  return launch_pdl(k_pass1<2>, dim3(c.st.sp1.g), dim3(kP1Threads), smem, c.stream, 1, tmK, tmQ, c.st,
                     c.ws, c.scale_log2e, (int)c.clear_status, status);
 }
 
@@ -1150,7 +1161,7 @@ cudaError_t launch_pass2_t(const LaunchCtx& c, const P2Maps& m, float* s_div_out
   static std::atomic<bool> done[kMaxDevices];
   cudaError_t e = ensure_smem(k_pass2<NCH>, kSmemLimit, done);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_pass2<NCH>, dim3(c.st.g2), dim3(kP2Threads), pass2_smem(c.st.NQ, vstages), c.stream, 1, m.K, m.V,
+  return launch_pdl(k_pass2<NCH>, dim3(c.st.sp2.g), dim3(kP2Threads), pass2_smem(c.st.NQ, vstages), c.stream, 1, m.K, m.V,
                     m.Q, c.st, c.ws, s_div_out, rbar_out, c.scale_log2e, c.p.use_vnorm, c.p.pool_kernel >> 1,
                     vstages, status);
 }

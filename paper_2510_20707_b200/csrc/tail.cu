@@ -146,7 +146,7 @@ __device__ __noinline__ float mix_one(const float ex, const float vn, const floa
 // The pass-2 segments of a head.
 __device__ __forceinline__ SegList pass2_segments(const SeqTable& st, const int layer, const int b, const int h) {
   const int per_head = (st.tile2_start[b + 1] - st.tile2_start[b]) / st.H;
-  return SegList(layer * st.nt2 + st.tile2_start[b] + h * per_head, per_head, split2(st));
+  return SegList(layer * st.nt2 + st.tile2_start[b] + h * per_head, per_head, st.sp2);
 }
 
 struct MixParams {

@@ -277,22 +277,6 @@ __device__ __forceinline__ TileCoord layer_tile_coord(const int* tile_start, int
   c.layer = layer;
   return c;
 }
-__host__ __device__ __forceinline__ Split split1(const SeqTable& st) {
-  return Split{st.layers * st.nt1, st.g1, st.q1, st.r1};
-}
-__host__ __device__ __forceinline__ Split split2(const SeqTable& st) {
-  return Split{st.layers * st.nt2, st.g2, st.q2, st.r2};
-}
-// First tile of CTA c.
-__host__ __device__ __forceinline__ int cta_first_tile(int c, const Split& sp) {
-  return c * sp.q + (c < sp.r ? c : sp.r);
-}
-// CTA whose contiguous range contains tile t.
-__host__ __device__ __forceinline__ int tile_owner(int t, const Split& sp) {
-  const int big = sp.r * (sp.q + 1);
-  return t < big ? t / (sp.q + 1) : sp.r + (t - big) / sp.q;
-}
-
 // Walks the tiles [lo, hi) of one CTA segment by segment: a segment is a run of tiles t0 .. t0 + n - 1 of
 // one (layer, sequence, head), so that a role's loop over the tiles of a segment carries nothing but the
 // tile index.  Tile ids run over all layers: id = layer * nt + (tile of the layer).
@@ -357,19 +341,20 @@ struct RevSegIter {
   }
 };
 
-// Segments of one (b, h) when its tiles [T0, T0 + per_head) lie in a tile list split
-// contiguously over CTAs: segment e starts at T0 for e = 0 and at the first tile of CTA
-// c0 + e otherwise (c0 = CTA that owns T0).
+// Segments of one (b, h) whose tiles [T0, T0 + per_head) lie in one run of a split: segment e starts at T0 for e = 0 and
+// at the first tile of CTA c0 + e otherwise (c0 = CTA that owns T0).
 struct SegList {
-  int T0, c0, nseg;
-  Split sp;
+  int T0, base, k0, q, r, nseg;   // base: first tile of the run, k0: c0 inside it
   SegList() = default;
-  __device__ SegList(int T0_, int per_head, const Split& sp_) : T0(T0_), sp(sp_) {
-    c0 = tile_owner(T0_, sp_);
-    nseg = tile_owner(T0_ + per_head - 1, sp_) - c0 + 1;
+  __device__ SegList(int T0_, int per_head, const Split& sp) : T0(T0_), q(sp.q), r(sp.r) {
+    const int run = T0_ / sp.n, c0 = tile_owner(T0_, sp);
+    base = run * sp.n;
+    k0 = c0 - run * sp.p;
+    nseg = tile_owner(T0_ + per_head - 1, sp) - c0 + 1;
   }
   __device__ __forceinline__ int start(int e) const {
-    return e == 0 ? T0 : cta_first_tile(c0 + e, sp);
+    const int k = k0 + e;
+    return e == 0 ? T0 : base + k * q + (k < r ? k : r);
   }
 };
 

@@ -88,3 +88,22 @@ def test_maps_are_dealt_out_by_what_l2_holds(lib):
     assert [run(4, 4312, 2, 1), run(4, 4320, 2, 1), run(4, 4320, 3, 1), run(4, 2048, 3, 1)] == [0, 1, 2, 0]
     # half the cache: the same at half the size; a map past 32 bits of bytes
     assert [run(2, 2036, 2, 0, 132644864 // 2), run(2, 4320, 3, 1, 132644864 // 2), run(8, 65535, 2, 0)] == [1, 2, 1]
+
+
+@pytest.mark.parametrize("sms", [148, 7])
+@pytest.mark.parametrize("heads,per_head", [(1, 1), (1, 300), (4, 8), (4, 47), (4, 256), (8, 24), (8, 235), (37, 5), (74, 3),
+                                            (148, 2), (149, 2), (112, 32), (5, 148), (64, 1)])
+def test_every_tile_has_one_cta(lib, heads, per_head, sms):
+    tiles = heads * per_head
+    first, owner = (C.c_int32 * (sms + 1))(), (C.c_int32 * tiles)()
+    for uniform in (per_head, 0):
+        g = lib.mixkv_internal_split_tiles(tiles, uniform, sms, first, owner)
+        assert 1 <= g <= min(tiles, sms) and first[0] == 0 and first[g] == tiles
+        shares = [first[c + 1] - first[c] for c in range(g)]
+        assert min(shares) >= 1 and sum(shares) == tiles
+        assert list(owner) == [c for c in range(g) for _ in range(shares[c])]
+        even = -(-tiles // min(tiles, sms))
+        apart = all(first[c] // per_head == (first[c + 1] - 1) // per_head for c in range(g))   # no CTA on two heads
+        assert max(shares) <= even + (1 if uniform and apart else 0)
+        if uniform and heads <= sms and -(-per_head // min(per_head, sms // heads)) <= even + 1:
+            assert apart
