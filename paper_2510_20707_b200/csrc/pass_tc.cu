@@ -252,7 +252,6 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   const int hi = cta_first_tile(blockIdx.x + 1, st.sp1);
   volatile int* abort = &bars->abort;
 
-  pdl_launch_dependents();
   if (tid == 0) {
     for (int s = 0; s < kP1Stages; ++s) {
       mbar_init(&bars->full[s], 1);
@@ -360,6 +359,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
             if (++ts == TS) ts = 0, tph ^= 1;
           }
         }
+        pdl_launch_dependents();   // (behind the wait: pass 2 reads the inputs without one of its own)
         umma_commit(&bars->mmas, on);
         drain_ring(&bars->mmas, 1, 1);
       }
@@ -629,7 +629,6 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   volatile int* abort = &bars->abort;
   constexpr int kWarpTmaV = 2;
 
-  pdl_launch_dependents();
   if (tid == 0) {
     for (int s = 0; s < kP2KStages; ++s) {
       mbar_init(&bars->kfull[s], 1);
@@ -672,7 +671,9 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
-  pdl_wait();
+  // K, V and the queries are the call's inputs: complete before pass 1 passed its own wait, behind which it lets this
+  // kernel start.  Their producers fill the rings while pass 1 ends; everybody else reads what it leaves.
+  if (warp >= kEpiWarp0) pdl_wait();
 
   if (warp == kWarpTma) {
     // ------------------------------------------------------------------ K / Q producer
@@ -764,6 +765,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         tph ^= ts ^ 1;
       }
     }
+    pdl_launch_dependents();
     if (*abort && on) raise(status, abort);
     umma_commit(&bars->mmas, on);
     drain_ring(&bars->mmas, 1, 1);

@@ -732,7 +732,6 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   float* sraw = reinterpret_cast<float*>(skeys + chunk);               // FUSED: [4 T + 64] raw scores of a block
   float* sdv = sraw + 4 * T + 64;                                      // FUSED: [4 T] diversity scores
 
-  pdl_launch_dependents();
   for (int t = tid; t < 2 * kSelBins; t += T) (&sm.hist[0][0])[t] = 0;
   const SegList sl2 = pass2_segments(st, layer, b, h);   // (divisions: ahead of the wait)
   const int fixed_off = fixed_offset(st, bh, a.Bp);
@@ -993,6 +992,8 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
     }
   }
   if (cs > 1 && want > 0 && want < P) cluster.barrier_arrive();   // past this CTA's last remote read
+
+  pdl_launch_dependents();
 
   // ---- gather: the rows this CTA keeps in ascending position order; the last CTA adds the W window rows
   if (a.K_out) {
