@@ -315,16 +315,21 @@ struct SelSmem {
   int hist[2][kSelBins];
   unsigned list[kSelListCap];    // this CTA's candidates
   int pos[kSelListCap];          // and which of its keys they are
-  unsigned all[kSelListCap];     // those of every CTA of the cluster, in rank order
+  unsigned all[kSelListCap];     // those of every CTA of the cluster, in rank order (written by all of them)
   unsigned wlo[32], whi[32];
-  unsigned range[2];             // this CTA's smallest and largest key
+  uint2 range[kSelMaxCluster];   // smallest and largest key of every CTA (each written by that CTA)
   int scan[32];
-  int off[kSelMaxCluster];       // cluster: where each rank's candidates start in `all`
-  int nlist, gt, eq;             // this CTA's candidates, its keys above them, its keys equal to the threshold
+  int nlist;                     // this CTA's candidates
   int bin, remaining, count;     // bin that holds the threshold, keys still needed from it, keys in it
+  int above_before, bin_before;  // keys above the bin and in it in the CTAs of lower rank
   unsigned tau;
   int need_eq, eq_total;
-  int gt_before, eq_before;
+};
+// What the CTAs of a cluster send each other in the rounds of a search, two rounds in turn: every rank's counts in
+// groups of 32 bins.
+constexpr int kSelGroups = kSelBins / 32;
+struct SelMail {
+  int groups[2][kSelMaxCluster][kSelGroups];
 };
 
 struct Threshold {
@@ -363,81 +368,117 @@ __device__ __forceinline__ int block_scan(const int v, int* scan, const int lane
 // than the list takes is binned again (three rounds reach single key values), so any distribution, all-equal
 // keys included, ends after a bounded number of sweeps.  The listing sweep calls above(j) for the keys that
 // are wanted in any case.  sm.hist must be zero on entry (visible to the CTA).
+//
+// Across a cluster a search is bound by its exchanges, three barriers with what has to be known behind each.  A CTA
+// sends that into its peers' shared memory ahead of the barrier (range; counts per group of 32 bins; candidates, whose place
+// in the common list the counts give), because a load from there costs another half a microsecond behind it; only the 32 counts
+// of the one group that holds the threshold are fetched, by one warp.  (Eight CTAs of 4096 keys: 7.6 us, fetched
+// from the peers behind the barriers, now 5.6; one layer of 4 x 32768 keys 47.6 -> 45.8.)
+// On entry every CTA of the cluster has started.  mail: not used when cs == 1.
 template <int T, typename KeyAt, typename Above>
 __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const Above& above_bin, const int n,
                                                       const int want, unsigned lo, unsigned hi, SelSmem& sm,
-                                                      cg::cluster_group& cluster, const int cs,
+                                                      SelMail& mail, cg::cluster_group& cluster, const int cs,
                                                       const int crank) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   constexpr int NW = T / 32, PER = kSelBins / T;
   lo = __reduce_min_sync(0xffffffffu, lo);
   hi = __reduce_max_sync(0xffffffffu, hi);
   if (lane == 0) sm.wlo[warp] = lo, sm.whi[warp] = hi;
-  if (tid == 0) sm.nlist = 0, sm.gt = 0, sm.eq = 0;
+  if (tid == 0) sm.nlist = 0;
   __syncthreads();
   lo = __reduce_min_sync(0xffffffffu, lane < NW ? sm.wlo[lane] : 0xffffffffu);
   hi = __reduce_max_sync(0xffffffffu, lane < NW ? sm.whi[lane] : 0u);
   if (cs > 1) {
-    if (tid == 0) sm.range[0] = lo, sm.range[1] = hi;
+    if (tid < cs) *cluster.map_shared_rank(&sm.range[crank], tid) = make_uint2(lo, hi);
     cluster.sync();
-    lo = 0xffffffffu, hi = 0u;
-    if (lane < cs) {
-      const uint2 r = *reinterpret_cast<const uint2*>(cluster.map_shared_rank(&sm.range[0], lane));
-      lo = r.x, hi = r.y;
-    }
+    const uint2 r = lane < cs ? sm.range[lane] : make_uint2(0xffffffffu, 0u);
+    lo = r.x, hi = r.y;
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
   }
   unsigned base = lo, span = hi - lo;   // the candidates are the keys in [base, base + span]
   int shift = span ? max(0, 32 - __clz(span) - kSelBinBits) : 0;
-  int remaining = want;
+  int remaining = want, gt_before = 0;
   for (int round = 0;; ++round) {
     int* hist = sm.hist[round & 1];
     for (int j = tid; j < n; j += T) {
       const unsigned d = key_at(j) - base;
       if (d <= span) atomicAdd(&hist[d >> shift], 1);
     }
-    if (cs > 1) cluster.sync();
-    else __syncthreads();
-    // thread t owns bins PER t .. PER t + PER - 1 (of all CTAs); `above` = keys in higher bins
+    __syncthreads();
+    // thread t owns bins PER t .. PER t + PER - 1
     int h[PER], mine = 0;
 #pragma unroll
-    for (int k = 0; k < PER; ++k) h[k] = 0;
+    for (int k = 0; k < PER; ++k) h[k] = hist[PER * tid + k], mine += h[k];
     if (cs > 1) {
-      // every rank's loads are under way before the first is used: a remote load takes half a microsecond
-      int2 v[kSelMaxCluster][PER / 2];
+      constexpr int GL = 32 / PER;   // lanes that own a group of 32 bins; they send its count to the ranks in turn
+      int sum = mine;
 #pragma unroll
-      for (int r = 0; r < kSelMaxCluster; ++r)
+      for (int o = 1; o < GL; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      int* slot = &mail.groups[round & 1][crank][tid / GL];
+      for (int r = lane % GL; r < cs; r += GL) *cluster.map_shared_rank(slot, r) = sum;
+      cluster.sync();
+      if (warp == 0) {
+        // two groups per lane, of all CTAs and of those of lower rank
+        int2 tot = make_int2(0, 0), low = tot;
 #pragma unroll
-        for (int k = 0; k < PER / 2; ++k)
-          v[r][k] = r < cs ? reinterpret_cast<const int2*>(cluster.map_shared_rank(&hist[PER * tid], r))[k]
-                           : make_int2(0, 0);
-#pragma unroll
-      for (int r = 0; r < kSelMaxCluster; ++r)
-#pragma unroll
-        for (int k = 0; k < PER / 2; ++k) h[2 * k] += v[r][k].x, h[2 * k + 1] += v[r][k].y;
-    } else {
-#pragma unroll
-      for (int k = 0; k < PER; ++k) h[k] = hist[PER * tid + k];
-    }
-#pragma unroll
-    for (int k = 0; k < PER; ++k) {
-      mine += h[k];
-      sm.hist[(round & 1) ^ 1][PER * tid + k] = 0;   // every CTA is past its reads of the other buffer
-    }
-    int above = block_scan<T, true>(mine, sm.scan, lane, warp);
-    if (above < remaining && remaining <= above + mine) {
-#pragma unroll
-      for (int k = PER - 1; k >= 0; --k) {
-        if (above < remaining && remaining <= above + h[k]) {
-          sm.bin = PER * tid + k;
-          sm.remaining = remaining - above;
-          sm.count = h[k];
+        for (int r = 0; r < kSelMaxCluster; ++r) {
+          const int2 v = r < cs ? *reinterpret_cast<const int2*>(&mail.groups[round & 1][r][2 * lane]) : make_int2(0, 0);
+          tot.x += v.x, tot.y += v.y;
+          if (r < crank) low.x += v.x, low.y += v.y;
         }
-        above += h[k];
+        auto keys_above = [&](const int v) {   // sum of v over the higher lanes
+          int incl = v;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_down_sync(0xffffffffu, incl, o);
+            if (lane + o < 32) incl += x;
+          }
+          return incl - v;
+        };
+        int above = keys_above(tot.x + tot.y);
+        const bool in_y = above < remaining && remaining <= above + tot.y;
+        const bool in_x = above + tot.y < remaining && remaining <= above + tot.y + tot.x;
+        int src = __ffs(__ballot_sync(0xffffffffu, in_x || in_y)) - 1;
+        const int group = __shfl_sync(0xffffffffu, 2 * lane + (in_y ? 1 : 0), src);
+        above = __shfl_sync(0xffffffffu, in_y ? above : above + tot.y, src);
+        int before = __reduce_add_sync(0xffffffffu, (2 * lane > group ? low.x : 0) + (2 * lane + 1 > group ? low.y : 0));
+        // the bins of that group, one per lane
+        int v[kSelMaxCluster], all = 0, lower = 0;
+#pragma unroll
+        for (int r = 0; r < kSelMaxCluster; ++r) v[r] = r < cs ? *cluster.map_shared_rank(&hist[32 * group + lane], r) : 0;
+#pragma unroll
+        for (int r = 0; r < kSelMaxCluster; ++r) all += v[r], lower += r < crank ? v[r] : 0;
+        above += keys_above(all);
+        src = __ffs(__ballot_sync(0xffffffffu, above < remaining && remaining <= above + all)) - 1;
+        before += __reduce_add_sync(0xffffffffu, lane > src ? lower : 0);
+        if (lane == src) {
+          sm.bin = 32 * group + lane;
+          sm.remaining = remaining - above;
+          sm.count = all;
+          sm.above_before = before;
+          sm.bin_before = lower;
+        }
+      }
+    } else {
+      int above = block_scan<T, true>(mine, sm.scan, lane, warp);
+      if (above < remaining && remaining <= above + mine) {
+#pragma unroll
+        for (int k = PER - 1; k >= 0; --k) {
+          if (above < remaining && remaining <= above + h[k]) {
+            sm.bin = PER * tid + k;
+            sm.remaining = remaining - above;
+            sm.count = h[k];
+          }
+          above += h[k];
+        }
       }
     }
+#pragma unroll
+    for (int k = 0; k < PER; ++k) sm.hist[(round & 1) ^ 1][PER * tid + k] = 0;   // every CTA is past its reads of it
     __syncthreads();
+    if (cs > 1) gt_before += sm.above_before;
     base += (unsigned)sm.bin << shift;
     remaining = sm.remaining;
     span = (1u << shift) - 1u;
@@ -445,60 +486,36 @@ __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const
     shift = max(0, shift - kSelBinBits);
   }
   const int count = sm.count;
+  const int before = cs > 1 ? sm.bin_before : 0;   // candidates of the lower ranks
   Threshold th;
-  th.gt_before = th.eq_before = 0;
+  th.gt_before = gt_before;
+  th.eq_before = 0;
   th.listed = shift != 0;
   if (shift == 0) {   // the bin is one key value
-    th.tau = base, th.need_eq = remaining, th.eq_total = count;
-    if (cs > 1) {
-      int gt = 0, eq = 0;
-      for (int j = tid; j < n; j += T) {
-        const unsigned key = key_at(j);
-        gt += key > base;
-        eq += key == base;
-      }
-      gt = __reduce_add_sync(0xffffffffu, gt);
-      eq = __reduce_add_sync(0xffffffffu, eq);
-      if (lane == 0) atomicAdd(&sm.gt, gt), atomicAdd(&sm.eq, eq);
-      cluster.sync();
-      const bool below = lane < crank;
-      th.gt_before = __reduce_add_sync(0xffffffffu, below ? *cluster.map_shared_rank(&sm.gt, lane) : 0);
-      th.eq_before = __reduce_add_sync(0xffffffffu, below ? *cluster.map_shared_rank(&sm.eq, lane) : 0);
-    }
+    th.tau = base, th.need_eq = remaining, th.eq_total = count, th.eq_before = before;
     return th;
   }
   // list the candidates; the keys above them are wanted in any case
-  int gt = 0;
   for (int j = tid; j < n; j += T) {
     const unsigned key = key_at(j);
     if (key >= base) {
       if (key - base <= span) {
         const int at = atomicAdd(&sm.nlist, 1);
         sm.list[at] = key, sm.pos[at] = j;
+        if (cs > 1)
+          for (int r = 0; r < cs; ++r) *cluster.map_shared_rank(&sm.all[before + at], r) = key;
       } else {
-        ++gt;
         above_bin(j);
       }
     }
   }
   const unsigned* all = sm.list;
   if (cs > 1) {
-    gt = __reduce_add_sync(0xffffffffu, gt);
-    if (lane == 0) atomicAdd(&sm.gt, gt);
-    cluster.sync();
-    if (warp < cs) {   // warp r copies rank r's candidates behind those of the lower ranks
-      const int len = lane < cs ? *cluster.map_shared_rank(&sm.nlist, lane) : 0;
-      const int start = __reduce_add_sync(0xffffffffu, lane < warp ? len : 0);
-      const int mylen = __shfl_sync(0xffffffffu, len, warp);
-      const unsigned* src = cluster.map_shared_rank(&sm.list[0], warp);
-      for (int k = lane; k < mylen; k += 32) sm.all[start + k] = src[k];
-      if (lane == 0) sm.off[warp] = start;
-    }
-    th.gt_before =
-        __reduce_add_sync(0xffffffffu, lane < crank ? *cluster.map_shared_rank(&sm.gt, lane) : 0);
     all = sm.all;
+    cluster.sync();
+  } else {
+    __syncthreads();
   }
-  __syncthreads();
   for (int k = tid; k < count; k += T) {
     const unsigned key = all[k];
     int g = 0, e = 0;
@@ -513,9 +530,8 @@ __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const
   __syncthreads();
   th.tau = sm.tau, th.need_eq = sm.need_eq, th.eq_total = sm.eq_total;
   if (cs > 1) {
-    const int below = sm.off[crank];
     int g = 0, e = 0;
-    for (int x = lane; x < below; x += 32) {
+    for (int x = lane; x < before; x += 32) {
       g += all[x] > th.tau;
       e += all[x] == th.tau;
     }
@@ -543,10 +559,12 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
   extern __shared__ unsigned bkeys[];   // [cache_cap] keys
   __shared__ __align__(16) SelSmem sm;
   __shared__ int s_gt[64], s_eq[64], t_gt[64], t_eq[64];
+  __shared__ __align__(16) SelMail mail;
   cg::cluster_group cluster = cg::this_cluster();
   const int cs = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   pdl_launch_dependents();
+  if (cs > 1) cluster.sync();   // every CTA has started: its peers may write to it
   for (int t = tid; t < 2 * kSelBins; t += kBudgetThreads) (&sm.hist[0][0])[t] = 0;
   if (tid < 64) s_gt[tid] = 0, s_eq[tid] = 0;
   pdl_wait();
@@ -600,7 +618,7 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
     return i < n ? order_key(base[(size_t)h * stride + p0 + i]) : 0u;
   };
   const Threshold th =
-      threshold_search<kBudgetThreads>(key_at, [](int) {}, local, (int)N, lo, hi, sm, cluster, cs, crank);
+      threshold_search<kBudgetThreads>(key_at, [](int) {}, local, (int)N, lo, hi, sm, mail, cluster, cs, crank);
   // a vote per word of 32; most words hold nothing that counts
   for (int h = 0; h < H; ++h) {
     for (int i0 = warp * 32; i0 < npad; i0 += kBudgetThreads) {
@@ -704,7 +722,9 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   __shared__ __align__(16) SelSmem sm;
   __shared__ int s_off, s_want;
   __shared__ float sc[8];
-  __shared__ int s_rows[kTailRowCap];
+  __shared__ __align__(16) int s_rows[kTailRowCap];   // (ahead of the compaction: what the search exchanges)
+  static_assert(sizeof(SelMail) <= sizeof(s_rows));
+  SelMail& mail = reinterpret_cast<SelMail&>(s_rows);
   __shared__ int s_gt[32], s_eq[32];   // (ADAPT)
   cg::cluster_group cluster = cg::this_cluster();
   const int crank = CL && !ADAPT ? (int)cluster.block_rank() : 0;   // (in ADAPT a unit is one CTA's)
@@ -732,6 +752,7 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   float* sraw = reinterpret_cast<float*>(skeys + chunk);               // FUSED: [4 T + 64] raw scores of a block
   float* sdv = sraw + 4 * T + 64;                                      // FUSED: [4 T] diversity scores
 
+  if (CL) cluster.barrier_arrive();   // this CTA has started: its peers may write to it
   for (int t = tid; t < 2 * kSelBins; t += T) (&sm.hist[0][0])[t] = 0;
   const SegList sl2 = pass2_segments(st, layer, b, h);   // (divisions: ahead of the wait)
   const int fixed_off = fixed_offset(st, bh, a.Bp);
@@ -878,6 +899,7 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
     }
   }
   __syncthreads();
+  if (CL) cluster.barrier_wait();
   auto key_at = [&](int j) -> unsigned { return cached ? skeys[j] : order_key(a.scores[poff + c0 + j]); };
   if constexpr (ADAPT) {
     // ---- this head's share: the floor, and the keys among the H * (Bp - floor) largest of all heads (equal ones to the
@@ -886,7 +908,7 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
     const int N = H * (a.Bp - a.floor_slots);
     int share = 0;
     if (N > 0) {
-      const Threshold th = threshold_search<T>(key_at, [](int) {}, n, N, klo, khi, sm, cluster, H, rank);
+      const Threshold th = threshold_search<T>(key_at, [](int) {}, n, N, klo, khi, sm, mail, cluster, H, rank);
       int gt = 0, eq = 0;
       for (int j = tid; j < n; j += T) {
         const unsigned key = key_at(j);
@@ -929,7 +951,7 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
   } else if (want > 0) {
     for (int w = tid; w < nwords; w += T) words[w] = 0u;   // visible after the search's first barrier
     auto keep = [&](const int j) { atomicOr(&words[j >> 5], 1u << (j & 31)); };
-    const Threshold th = threshold_search<T>(key_at, keep, n, want, klo, khi, sm, cluster, cs, crank);
+    const Threshold th = threshold_search<T>(key_at, keep, n, want, klo, khi, sm, mail, cluster, cs, crank);
     const bool all_eq = th.need_eq == th.eq_total;   // no tie to split: keep every key from tau on
     if (all_eq && th.listed) {
       for (int k = tid; k < sm.nlist; k += T)
