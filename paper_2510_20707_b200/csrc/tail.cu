@@ -24,44 +24,52 @@ namespace {
 //   s_in_scaled  = (|V_i| - sc[0]) * sc[1]
 //   s_div_scaled = (s_div_i - sc[2]) * sc[3]
 //   sc[4]        = redundancy used by the mix
-__device__ void head_scalars(const SeqTable& st, const Workspace& ws, const SegList& sl, const int layer,
+//
+// In the tail it stands between the loads of the first positions and their mix, so what it reads is asked for ahead of
+// them (load_head_parts: two segments per lane).
+struct HeadParts {
+  float4 d[2], e[2], v[2];
+  float rbar;
+};
+__device__ __forceinline__ void load_head_parts(HeadParts& hp, const Workspace& ws, const SegList& sl, const int use_vnorm,
+                                                const int e0) {
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int e = e0 + 32 * k;
+    hp.d[k] = hp.e[k] = hp.v[k] = make_float4(INFINITY, -INFINITY, 0.f, 0.f);
+    if (e < sl.nseg) {
+      const int start = sl.start(e);
+      hp.d[k] = ws.dstat[(size_t)start * 2];
+      hp.e[k] = ws.dstat[(size_t)start * 2 + 1];
+      if (use_vnorm) hp.v[k] = ws.vstat[start];
+    }
+  }
+}
+__device__ __forceinline__ void first_head_parts(HeadParts& hp, const Workspace& ws, const SegList& sl, const int unit,
+                                                 const int use_vnorm, const float* __restrict__ rbar_in, const int lane) {
+  load_head_parts(hp, ws, sl, use_vnorm, lane);
+  hp.rbar = rbar_in ? rbar_in[unit] : ws.rbar[unit];
+}
+__device__ void head_scalars(HeadParts& hp, const SeqTable& st, const Workspace& ws, const SegList& sl, const int layer,
                              const int b, const int h, const int pool_k, const int pool_mode, const int use_vnorm,
-                             const float eps, const float* __restrict__ rbar_in, const int lane,
-                             float* sc) {
-  const int unit = (layer * st.batch + b) * st.H + h;
+                             const float eps, const int lane, float* sc) {
   const int P = st.cu[b + 1] - st.cu[b] - st.W;
   float dmin = INFINITY, dmax = -INFINITY, dsum = 0.f, exw = 0.f;
   float vmin = INFINITY, vmax = -INFINITY, vsum = 0.f;
-  float rbar = 0.f;
-  if (lane == 0) rbar = rbar_in ? rbar_in[unit] : ws.rbar[unit];
-  {
-    // lanes take segments side by side, two per lane and round; all loads of a round are
-    // issued before the first is used
-    for (int e0 = lane; e0 < sl.nseg; e0 += 64) {
-      float4 d4[2], e4[2], v4[2];
+  for (int e0 = lane;;) {
 #pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int e = e0 + 32 * k;
-        d4[k] = e4[k] = make_float4(INFINITY, -INFINITY, 0.f, 0.f);
-        v4[k] = d4[k];
-        if (e < sl.nseg) {
-          const int start = sl.start(e);
-          d4[k] = ws.dstat[(size_t)start * 2];
-          e4[k] = ws.dstat[(size_t)start * 2 + 1];
-          if (use_vnorm) v4[k] = ws.vstat[start];
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        dmin = fminf(dmin, fminf(d4[k].x, e4[k].x));
-        dmax = fmaxf(dmax, fmaxf(d4[k].y, e4[k].y));
-        dsum += d4[k].z + e4[k].z;
-        exw += d4[k].w + e4[k].w;
-        vmin = fminf(vmin, v4[k].x);
-        vmax = fmaxf(vmax, v4[k].y);
-        vsum += v4[k].z;
-      }
+    for (int k = 0; k < 2; ++k) {
+      dmin = fminf(dmin, fminf(hp.d[k].x, hp.e[k].x));
+      dmax = fmaxf(dmax, fmaxf(hp.d[k].y, hp.e[k].y));
+      dsum += hp.d[k].z + hp.e[k].z;
+      exw += hp.d[k].w + hp.e[k].w;
+      vmin = fminf(vmin, hp.v[k].x);
+      vmax = fmaxf(vmax, hp.v[k].y);
+      vsum += hp.v[k].z;
     }
+    e0 += 64;
+    if (e0 - lane >= sl.nseg) break;
+    load_head_parts(hp, ws, sl, use_vnorm, e0);
   }
   float ex;
   if (pool_mode == MIXKV_POOL_AVG) {
@@ -98,7 +106,7 @@ __device__ void head_scalars(const SeqTable& st, const Workspace& ws, const SegL
     sc[1] = cin;
     sc[2] = dmin;
     sc[3] = dinv * a_div;
-    sc[4] = rbar;
+    sc[4] = hp.rbar;
   }
 }
 
@@ -196,11 +204,12 @@ __device__ __forceinline__ void mix4(const float (&ex)[4], const float4 v4, cons
 }
 
 // --------------------------------------------------------------------------- poolsum
-// Max pooling only: per-chunk sums of the pooled score (its mean enters Eq. 2).
-__global__ void __launch_bounds__(256)
+// Max pooling only: per-chunk sums of the pooled score (its mean enters Eq. 2).  A short chain with as many threads as a CTA
+// has (256 threads, eight positions each: scores and selection of three sequences 53.1 us a call, now 52.1).
+__global__ void __launch_bounds__(1024)
 k_poolsum(const SeqTable st, const Workspace ws, const int k) {
   __shared__ float tile[kPChunk + 64];
-  __shared__ float sred[8];
+  __shared__ float sred[32];
   pdl_launch_dependents();
   pdl_wait();
   const int pcx = blockIdx.x, h = blockIdx.y, layer = blockIdx.z;
@@ -210,19 +219,19 @@ k_poolsum(const SeqTable st, const Workspace ws, const int k) {
   const int p1 = min(p0 + kPChunk, P);
   const size_t poff = ppos(st, layer, h, b, 0);
   const int half = k >> 1;
-  for (int t = threadIdx.x; t < (p1 - p0) + 2 * half; t += 256) {
+  for (int t = threadIdx.x; t < (p1 - p0) + 2 * half; t += 1024) {
     const int i = p0 - half + t;
     tile[t] = (i >= 0 && i < P) ? ws.s_ex_raw[poff + i] : -INFINITY;
   }
   __syncthreads();
   float sum = 0.f;
-  for (int t = threadIdx.x; t < p1 - p0; t += 256) sum += pool_window(tile + t, k, MIXKV_POOL_MAX, 0.f);
+  for (int t = threadIdx.x; t < p1 - p0; t += 1024) sum += pool_window(tile + t, k, MIXKV_POOL_MAX, 0.f);
   sum = warp_sum(sum);
   if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = sum;
   __syncthreads();
+  if (threadIdx.x < 32) sum = warp_sum(sred[threadIdx.x]);
   if (threadIdx.x == 0) {
-    float s = 0.f;
-    for (int w = 0; w < 8; ++w) s += sred[w];
+    const float s = sum;
     ws.exsum[((size_t)layer * st.H + h) * st.pchunks_total + pcx] = s;
   }
 }
@@ -231,18 +240,23 @@ k_poolsum(const SeqTable st, const Workspace ws, const int k) {
 // Pooling and the mix over a grid of position chunks (the scores entry point, adaptive budgets).  A chunk is read
 // with consecutive threads on consecutive positions, all loads in flight at once, staged in shared memory and
 // mixed four consecutive positions per thread, as in k_tail.
+//
+// CH: positions per CTA.  A chunk is a chain (scalars, loads, stage, stores) that shorter ones shorten: where chunks of 2048
+// leave SMs without one, 512 (scores and selection of three sequences, 80 chunks, 54.9 -> 53.9 us a call).
+template <int CH>
 __global__ void __launch_bounds__(256, 4)
 k_mixpool(const SeqTable st, const Workspace ws, const float* __restrict__ s_div,
           const float* __restrict__ rbar_in, float* __restrict__ s_ex_out,
           float* __restrict__ s_comp, const MixParams mp) {
-  __shared__ __align__(16) float tile[kPChunk + 64], svn[kPChunk], sdv[kPChunk];
+  __shared__ __align__(16) float tile[CH + 64], svn[CH], sdv[CH];
   __shared__ float sc[8];
   pdl_launch_dependents();
-  const int pcx = blockIdx.x, h = blockIdx.y, layer = blockIdx.z, tid = threadIdx.x;
+  constexpr int kSplit = kPChunk / CH;
+  const int pcx = blockIdx.x / kSplit, h = blockIdx.y, layer = blockIdx.z, tid = threadIdx.x;
   const int b = find_seq(st.pchunk_start, st.batch, pcx);
   const int P = st.cu[b + 1] - st.cu[b] - st.W;
-  const int p0 = (pcx - st.pchunk_start[b]) * kPChunk;
-  const int n = min(kPChunk, P - p0);
+  const int p0 = (pcx - st.pchunk_start[b]) * kPChunk + (int)blockIdx.x % kSplit * CH;
+  const int n = min(CH, P - p0);   // (may be none of the last chunk)
   const size_t poff = ppos(st, layer, h, b, 0);
   const int half = mp.pool_k >> 1;
   const bool avg = mp.pool_mode == MIXKV_POOL_AVG;
@@ -250,7 +264,7 @@ k_mixpool(const SeqTable st, const Workspace ws, const float* __restrict__ s_div
   const SegList sl = pass2_segments(st, layer, b, h);   // (divisions: ahead of the wait)
   pdl_wait();
   // eight rounds of 256 positions (+ the pooling halo in a ninth)
-  constexpr int kRounds = kPChunk / 256;
+  constexpr int kRounds = CH / 256;
   const int nstage = n + 2 * half;
   float raw[kRounds + 1], vn[kRounds], dv[kRounds];
 #pragma unroll
@@ -264,8 +278,11 @@ k_mixpool(const SeqTable st, const Workspace ws, const float* __restrict__ s_div
     vn[e] = (mp.use_vnorm && t < n) ? ws.vnorm[poff + p0 + t] : 0.f;
     dv[e] = t < n ? s_div[poff + p0 + t] : 0.f;
   }
-  if (tid < 32)
-    head_scalars(st, ws, sl, layer, b, h, mp.pool_k, mp.pool_mode, mp.use_vnorm, mp.eps, rbar_in, tid, sc);
+  if (tid < 32) {
+    HeadParts hp;
+    first_head_parts(hp, ws, sl, (layer * st.batch + b) * st.H + h, mp.use_vnorm, rbar_in, tid);
+    head_scalars(hp, st, ws, sl, layer, b, h, mp.pool_k, mp.pool_mode, mp.use_vnorm, mp.eps, tid, sc);
+  }
 #pragma unroll
   for (int e = 0; e <= kRounds; ++e) {
     const int t = e * 256 + tid;
@@ -277,7 +294,7 @@ k_mixpool(const SeqTable st, const Workspace ws, const float* __restrict__ s_div
   const float invk = 1.0f / (float)mp.pool_k;
   // the pooled scores take the place of the value norms, the mixed ones that of the diversity scores
 #pragma unroll
-  for (int g = 0; g < kPChunk / 1024; ++g) {
+  for (int g = 0; g < (CH + 1023) / 1024; ++g) {
     const int q = g * 1024 + 4 * tid;
     if (q >= n) break;
     float ex[4], m[4];
@@ -829,10 +846,11 @@ k_tail(const SeqTable st, const Workspace ws, const TailKernelArgs a) {
         dv[e] = t < nb ? g_dv[j0 + t] : 0.f;
       }
     };
+    HeadParts hp;
+    if (warp == 1) first_head_parts(hp, ws, sl2, unit, a.mp.use_vnorm, a.rbar_in, lane);
     if (n > 0) load_block(0);
-    if (warp == 1)   // (its own share of the first block is on the way)
-      head_scalars(st, ws, sl2, layer, b, h, a.mp.pool_k, a.mp.pool_mode, a.mp.use_vnorm, a.mp.eps,
-                   a.rbar_in, lane, sc);
+    if (warp == 1)
+      head_scalars(hp, st, ws, sl2, layer, b, h, a.mp.pool_k, a.mp.pool_mode, a.mp.use_vnorm, a.mp.eps, lane, sc);
     for (int j0 = 0; j0 < n; j0 += BL) {
       const int nb = min(BL, n - j0);   // positions of this block
       __syncthreads();                  // the previous block's readers of the stage are done
@@ -1076,15 +1094,18 @@ MixParams mix_params(const mixkv_params& p) {
 }  // namespace
 
 cudaError_t launch_poolsum(const LaunchCtx& c) {
-  return launch_pdl(k_poolsum, dim3(c.st.pchunks_total, c.st.H, c.st.layers), dim3(256), 0,
+  return launch_pdl(k_poolsum, dim3(c.st.pchunks_total, c.st.H, c.st.layers), dim3(1024), 0,
                     c.stream, 1, c.st,
                     c.ws, c.p.pool_kernel);
 }
 
 cudaError_t launch_mixpool(const LaunchCtx& c, const float* s_div, const float* rbar_in,
                            float* s_ex_out, float* s_comp) {
-  return launch_pdl(k_mixpool, dim3(c.st.pchunks_total, c.st.H, c.st.layers), dim3(256), 0,
-                    c.stream, 1, c.st,
+  const long long chunks = (long long)c.st.pchunks_total * c.st.H * c.st.layers;
+  if (chunks < device_sm_count())
+    return launch_pdl(k_mixpool<512>, dim3(c.st.pchunks_total * 4, c.st.H, c.st.layers), dim3(256), 0, c.stream, 1, c.st, c.ws,
+                      s_div, rbar_in, s_ex_out, s_comp, mix_params(c.p));
+  return launch_pdl(k_mixpool<kPChunk>, dim3(c.st.pchunks_total, c.st.H, c.st.layers), dim3(256), 0, c.stream, 1, c.st,
                     c.ws, s_div, rbar_in, s_ex_out, s_comp, mix_params(c.p));
 }
 

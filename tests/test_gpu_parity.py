@@ -415,6 +415,16 @@ def test_adaptive_budget_cluster_edges(batch, H, P):
     assert np.array_equal(got["idx"].cpu().numpy()[:offs[-1]], ref["idx"])
 
 
+@pytest.mark.parametrize("H,prefixes,mode", [
+    (2, (511, 512, 513), 0), (3, (2047, 2048, 2049), 1), (1, (2561, 400, 4096), 0),   # chunks of 512 positions
+    (8, (2100,) * 9, 0), (8, (2100,) * 10, 1)])                                       # 144 chunks of 2048, the last; 160
+def test_mix_chunk_edges(H, prefixes, mode):
+    # the scores entry point, average and max pooling: positions at the edges of the mix kernel's chunks
+    wl = synth.small_workload(H=H, G=4, W=32, seq_lens=tuple(p + 32 for p in prefixes), pool_kernel=7, budget=64,
+                              seed=sum(prefixes) + H, centroids=8)
+    run_layer_parity(wl, variant="calibrated", pool_mode=mode)
+
+
 def test_long_sequence_cluster_tail():
     # 65536 keys per head: clusters of eight with 8192 positions to a CTA
     wl = synth.small_workload(H=2, G=4, W=32, seq_lens=(65536,), pool_kernel=7, budget=512,
