@@ -273,10 +273,12 @@ __device__ __forceinline__ float warp_max(const float v) {
 // Programmatic dependent launch: let the next kernel of the stream be scheduled, and wait
 // until everything before this kernel in the stream has completed and is visible.
 //
-// Where a kernel lets the next one start costs more than what that one gains by being there early: the passes do it once
-// their last MMA is issued, the tail ahead of its gather.  At the top of all three / behind their waits / as now, us a call:
-// one layer of 4 x 1024 keys 20.7 / 20.6 / 18.5, of 4 x 32768 50.0 / 48.0 / 47.4, 28 layers of 4 x 4096 108.7 / 107.4 /
-// 103.3, scores and selection of three sequences 58.6 / 57.3 / 54.8; never (at the end of a CTA) 20.9, 49.6, 104.9, 56.3.
+// Where a kernel lets the next one start costs more than what that one gains by being there early: the passes do it with
+// the last tile but one, the tail ahead of its gather.  At the top of all three / behind their waits / once the passes' last
+// MMA was issued, us a call: one layer of 4 x 1024 keys 20.7 / 20.6 / 18.5, of 4 x 32768 50.0 / 48.0 / 47.4, 28 layers of
+// 4 x 4096 108.7 / 107.4 / 103.3, scores and selection of three sequences 58.6 / 57.3 / 54.8; never (at the end of a CTA)
+// 20.9, 49.6, 104.9, 56.3.  A tile earlier than that: 18.2 -> 18.1, 45.7 -> 45.5, level, 54.9 -> 54.3 (two and three
+// tiles earlier 56.5 on the last).
 // The mix, budget, decode and similarity kernels gain nothing or lose by it (4 x 32768 rows in blocks of 16 30.6 at the top,
 // 30.9 to 32.3 later) and keep theirs at the top.
 __device__ __forceinline__ void pdl_launch_dependents() {

@@ -339,6 +339,8 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
             tc_fence_after();
             const uint32_t kb_lo = k_lo + (uint32_t)s * (kTileBytes >> 4);
             const uint32_t td = tmem + ts * (MB * 128);
+            // one tile ahead of the last (and behind the wait: pass 2 reads the inputs without one of its own)
+            if (sg.id + k == max(lo, hi - 2)) pdl_launch_dependents();
 #pragma unroll
             for (int mb = 0; mb < MB; ++mb) {
               // k-steps of 16 columns: 32 bytes apart inside a 64-column half
@@ -359,7 +361,6 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
             if (++ts == TS) ts = 0, tph ^= 1;
           }
         }
-        pdl_launch_dependents();   // (behind the wait: pass 2 reads the inputs without one of its own)
         umma_commit(&bars->mmas, on);
         drain_ring(&bars->mmas, 1, 1);
       }
@@ -748,6 +749,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         tc_fence_after();
         const uint32_t kb_lo = k_lo + (uint32_t)s * (kTileBytes >> 4);
         const uint32_t td = tmem + ts * 256;
+        if (sg.id + (sg.n - 1 - k) == min(hi - 1, lo + 1)) pdl_launch_dependents();   // one tile ahead of the last
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
           const uint32_t a_lo = kb_lo + (uint32_t)((ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2);
@@ -765,7 +767,6 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         tph ^= ts ^ 1;
       }
     }
-    pdl_launch_dependents();
     if (*abort && on) raise(status, abort);
     umma_commit(&bars->mmas, on);
     drain_ring(&bars->mmas, 1, 1);
