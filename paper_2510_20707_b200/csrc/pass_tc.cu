@@ -139,6 +139,32 @@ __device__ __forceinline__ void fold_row_stats(const float2* rowstat, const SegL
     s1 = merge_stats(s1, make_float2(__shfl_xor_sync(0xffffffffu, s1.x, o), __shfl_xor_sync(0xffffffffu, s1.y, o)));
   }
 }
+// The same for rows 2 rp, 2 rp + 1 by one lane, rp = first, first + 32, ...: log2 normalisers (negated, `shift` taken off) of
+// all rows by one warp that has the time of a whole segment for it.
+constexpr int kFoldSpare = 4;
+__device__ __forceinline__ void fold_rows_by_warp(const float2* rowstat, const SegList& sl, const int NQ, const int lane,
+                                                  const float shift, float* normaliser) {
+#pragma unroll 1
+  for (int rp = lane; 2 * rp < NQ; rp += 32) {
+    float2 s0 = make_float2(-1e30f, 0.f), s1 = s0;
+#pragma unroll 1
+    for (int e0 = 0; e0 < sl.nseg; e0 += kFoldSpare) {
+      float4 v[kFoldSpare];
+#pragma unroll
+      for (int k = 0; k < kFoldSpare; ++k) {
+        v[k] = make_float4(-1e30f, 0.f, -1e30f, 0.f);
+        if (e0 + k < sl.nseg) v[k] = __ldcg(reinterpret_cast<const float4*>(rowstat + (size_t)sl.start(e0 + k) * NQ) + rp);
+      }
+#pragma unroll
+      for (int k = 0; k < kFoldSpare; ++k) {
+        s0 = merge_stats(s0, make_float2(v[k].x, v[k].y));
+        s1 = merge_stats(s1, make_float2(v[k].z, v[k].w));
+      }
+    }
+    *reinterpret_cast<float2*>(normaliser + 2 * rp) =
+        make_float2(-(s0.x + log2f(s0.y)) - shift, -(s1.x + log2f(s1.y)) - shift);
+  }
+}
 // Components 4 lane .. 4 lane + 3 of the unit-key sum over segments w, w + 4, ...
 __device__ __forceinline__ float4 fold_key_sums(const float* ksum, const SegList& sl, const int w, const int lane) {
   float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -553,7 +579,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
 }
 
 // ======================================================================== pass 2
-// Pass 2 streams K and V.  24 warps: K/Q producer, MMA, V producer, 1 idle, four epilogue warpgroups, 4
+// Pass 2 streams K and V.  24 warps: K/Q producer, MMA, V producer, 1 spare, four epilogue warpgroups, 4
 // value-norm warps.  Epilogue warpgroup g works on accumulator stage g & 1 (alternate tiles), column half
 // g >> 1: one key per thread and half of its G*W logit columns, in pieces of 16 with the next piece on its way
 // from tensor memory; the two halves of a key meet in one word of shared memory per tile.  (With two warpgroups
@@ -581,6 +607,7 @@ struct P2Bars {
   uint64_t qfull;
   uint64_t qfree;
   uint64_t kbready;
+  uint64_t nfull[2], nempty[2];   // normalisers by the spare warp
   uint64_t mmas;    // the issuer's last ones
   TileCoord last;   // of the CTA's last tile
   SegList segs;     // pass 1's segments of the head that it belongs to
@@ -602,9 +629,11 @@ __device__ __forceinline__ void colsum16(const uint32_t (&r)[16], const float* n
   }
 }
 
-// grid = g2 persistent CTAs: K producer, MMA, V producer, 1 idle, 16 epilogue, 4 value-norm warps.
+// grid = g2 persistent CTAs: K producer, MMA, V producer, 1 spare, 16 epilogue, 4 value-norm warps.
 // NCH: pieces of 16 query columns per epilogue warp, at most.
-template <int NCH>
+// SPARE: the spare warp folds the normalisers of the CTA's segments after the first (see pass2_spare).  A template argument
+// because the code costs the calls that cannot use it 0.3 to 0.7 us.
+template <int NCH, bool SPARE>
 __global__ void __launch_bounds__(kP2Threads, 1)
 k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
         const __grid_constant__ CUtensorMap tmQ, const SeqTable st, const Workspace ws,
@@ -618,8 +647,8 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   unsigned char* sQ = base;                   // 2 halves x [NB x 128 B]
   unsigned char* sK = sQ + 2 * NB * 128;      // kP2KStages x 32 KB
   unsigned char* sV = sK + kP2KStages * kTileBytes;   // vstages x 16 KB
-  float* sbq = reinterpret_cast<float*>(sV + vstages * kVSubBytes);  // [256] negated normalisers
-  float* sxp = sbq + 256;                     // [2][128] partial column sums of the second column halves
+  float* sbq = reinterpret_cast<float*>(sV + vstages * kVSubBytes);  // [2][256] negated normalisers
+  float* sxp = sbq + 512;                     // [2][128] partial column sums of the second column halves
   float* skp = sxp + 256;                     // [4][128] parts of the unit-key sum
   float* sred = skp + 512;    // [64]: 2 x 16 epilogue, 12 value norms, 4 mean key
   P2Bars* bars = reinterpret_cast<P2Bars*>(sred + 64);
@@ -628,7 +657,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   const int lo = cta_first_tile(blockIdx.x, st.sp2);
   const int hi = cta_first_tile(blockIdx.x + 1, st.sp2);
   volatile int* abort = &bars->abort;
-  constexpr int kWarpTmaV = 2;
+  constexpr int kWarpTmaV = 2, kWarpSpare = 3;
 
   if (tid == 0) {
     for (int s = 0; s < kP2KStages; ++s) {
@@ -646,6 +675,10 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     mbar_init(&bars->qfull, 1);
     mbar_init(&bars->qfree, 1);
     mbar_init(&bars->kbready, 4);          // the four warps that write the mean-key rows
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&bars->nfull[s], 1);
+      mbar_init(&bars->nempty[s], kP2EpiWarps);
+    }
     mbar_init(&bars->mmas, 1);
     bars->abort = 0;
     mbar_init_fence();
@@ -674,7 +707,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   const uint32_t tmem = bars->tmem_base;
   // K, V and the queries are the call's inputs: complete before pass 1 passed its own wait, behind which it lets this
   // kernel start.  Their producers fill the rings while pass 1 ends; everybody else reads what it leaves.
-  if (warp >= kEpiWarp0) pdl_wait();
+  if (warp >= kEpiWarp0 || (SPARE && warp == kWarpSpare)) pdl_wait();
 
   if (warp == kWarpTma) {
     // ------------------------------------------------------------------ K / Q producer
@@ -770,13 +803,25 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     if (*abort && on) raise(status, abort);
     umma_commit(&bars->mmas, on);
     drain_ring(&bars->mmas, 1, 1);
+  } else if (SPARE && warp == kWarpSpare) {
+    // ------------------------------------------------------------------ normalisers of the segments after the first
+    // (the epilogue folds the first one's itself, all 512 threads of it, and uses the two tables in turn)
+    int segn = 0;
+    for (RevSegIter sg(st.tile2_start, st.batch, H, bars->last, lo, hi); sg.valid(); sg.next(), ++segn) {
+      if (segn == 0) continue;
+      if (segn > 1 && !mbar_wait(&bars->nempty[segn & 1], ((segn >> 1) - 1) & 1, abort)) break;
+      fold_rows_by_warp(ws.rowstat, pass1_segments(st, sg.layer, sg.b, sg.h), NQ, lane, log2f((float)W),
+                        sbq + (segn & 1) * 256);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bars->nfull[segn & 1]);
+    }
   } else if (warp >= kEpiWarp0 && warp < kEpiWarp0 + kP2EpiWarps) {
     // ------------------------------------------------------------------ epilogue
     // Alternate tiles belong to alternate pairs of warpgroups, so inside a segment the pairs never wait
     // for each other; each pair leaves its own partial score statistics.  At the start of a segment the
     // 512 threads fold the row statistics of the head together, four lanes to a pair of window rows, into the
-    // normaliser table all groups read.  Nobody leaves the tile loop early: after an abort every
-    // wait fails at once, so the named barriers stay matched.
+    // normaliser table all groups read; with SPARE the later segments' comes from the spare warp.  Nobody leaves the
+    // tile loop early: after an abort every wait fails at once, so the named barriers stay matched.
     const int quarter = warp & 3, grp = (warp - kEpiWarp0) >> 2;
     const int wg = grp & 1, chalf = grp >> 1;      // accumulator stage, column half
     const int gt = (tid - kEpiWarp0 * 32) & 127;   // thread inside the warpgroup
@@ -790,13 +835,15 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     const int xbar = 6 + wg;                       // named barriers 6, 7: partial sums handed over
     const f32x2 sc2 = pack2(scale_log2e, scale_log2e);
     const uint32_t tstage = tmem + ((uint32_t)(quarter * 32) << 16) + wg * 256, taddr = tstage + ch_lo * 16;
-    const float* nb = sbq + ch_lo * 16;
     int tile = 0;   // parity decides which pair owns it
+    int segn = 0;
     for (RevSegIter sg(st.tile2_start, st.batch, H, bars->last, lo, hi); sg.valid(); sg.next()) {
       const int P = st.cu[sg.b + 1] - st.cu[sg.b] - W;
-      {
+      if (SPARE && segn > 0) {
+        mbar_wait(&bars->nfull[segn & 1], ((segn - 1) >> 1) & 1, abort);
+      } else {
         // the negated log2 normalisers of the rows with the 1/W of the window mean folded in
-        const SegList sl = tile == 0 ? bars->segs : pass1_segments(st, sg.layer, sg.b, sg.h);
+        const SegList sl = SPARE || tile == 0 ? bars->segs : pass1_segments(st, sg.layer, sg.b, sg.h);
         const int rp = (et >> 5) * 8 + (lane & 7);
         float2 s0, s1;
         fold_row_stats(ws.rowstat, sl, NQ, rp, lane, s0, s1);
@@ -806,6 +853,7 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
               make_float2(-(s0.x + log2f(s0.y)) - log2W, -(s1.x + log2f(s1.y)) - log2W);
         named_bar_sync(5, kP2EpiWarps * 32);
       }
+      const float* nb = sbq + (SPARE ? (segn & 1) * 256 : 0) + ch_lo * 16;
       float dmin = INFINITY, dmax = -INFINITY, dsum = 0.f, exw = 0.f;
       const float* kinv = ws.kinv + kpos(st, sg.layer, sg.h, sg.b, 0);
       const size_t poff = ppos(st, sg.layer, sg.h, sg.b, 0);
@@ -878,6 +926,11 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         }
       }
       tile += sg.n;
+      if constexpr (SPARE) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bars->nempty[segn & 1]);
+        ++segn;
+      }
       if (chalf == 0) {
         // this pair's share of the segment's score statistics (neutral if it had no tile)
         const float a = warp_min(dmin), b2 = warp_max(dmax), c2 = warp_sum(dsum),
@@ -1097,7 +1150,7 @@ constexpr size_t pass1_smem(int NQ) {
 constexpr size_t kP1SmemLimit = kSmemLimit - (kP1AuxWarps * 128 * 4 + kP1XRows * 8 + sizeof(P1Bars) + 63) / 64 * 64;
 constexpr size_t pass2_smem(int NQ, int vstages) {
   return 1024 + (size_t)2 * (NQ + kExtraRows) * 128 + kP2KStages * kTileBytes +
-         (size_t)vstages * kVSubBytes + 1024 * 4 + 64 * 4 + sizeof(P2Bars) + 64;
+         (size_t)vstages * kVSubBytes + 1280 * 4 + 64 * 4 + sizeof(P2Bars) + 64;
 }
 // V stages: the two pairs of value-norm warps need one each.
 constexpr int pass2_vstages(int NQ) {
@@ -1155,18 +1208,33 @@ cudaError_t launch_pass1(const LaunchCtx& c, const void* K, const void* Q, int* 
 }
 
 namespace {
+// Whether pass 2's spare warp folds the normalisers of a CTA's second and later heads.  It has the time of a
+// head's tiles for it, with a round trip for every four segments and 64 rows: not where a head lies in many CTAs.  The
+// epilogue's own fold kept it waiting 2.5 us per head: 28 layers of 4 heads and sequences of 700, 650, 800, 900 keys 108.4
+// -> 104.4 us, of 3001, 1777, 6143 293 -> 287, of eight sequences of 2 to 7 thousand 754 -> 743 (cold), of 4096 108 -> 106.5.
+constexpr int kSpareSegments = 6;
+bool pass2_spare(const LaunchCtx& c) {
+  const int most = (c.max_seq_len + kTile - 1) / kTile;   // tiles of the longest head
+  return most / c.st.sp1.q + 2 <= kSpareSegments;
+}
 struct P2Maps {
   CUtensorMap K, V, Q;
 };
+template <int NCH, bool SPARE>
+cudaError_t launch_pass2_s(const LaunchCtx& c, const P2Maps& m, float* s_div_out, float* rbar_out, int vstages,
+                           int* status) {
+  static std::atomic<bool> done[kMaxDevices];
+  cudaError_t e = ensure_smem(k_pass2<NCH, SPARE>, kSmemLimit, done);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_pass2<NCH, SPARE>, dim3(c.st.sp2.g), dim3(kP2Threads), pass2_smem(c.st.NQ, vstages), c.stream, 1, m.K, m.V,
+                    m.Q, c.st, c.ws, s_div_out, rbar_out, c.scale_log2e, c.p.use_vnorm, c.p.pool_kernel >> 1,
+                    vstages, status);
+}
 template <int NCH>
 cudaError_t launch_pass2_t(const LaunchCtx& c, const P2Maps& m, float* s_div_out, float* rbar_out, int vstages,
                            int* status) {
-  static std::atomic<bool> done[kMaxDevices];
-  cudaError_t e = ensure_smem(k_pass2<NCH>, kSmemLimit, done);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(k_pass2<NCH>, dim3(c.st.sp2.g), dim3(kP2Threads), pass2_smem(c.st.NQ, vstages), c.stream, 1, m.K, m.V,
-                    m.Q, c.st, c.ws, s_div_out, rbar_out, c.scale_log2e, c.p.use_vnorm, c.p.pool_kernel >> 1,
-                    vstages, status);
+  return pass2_spare(c) ? launch_pass2_s<NCH, true>(c, m, s_div_out, rbar_out, vstages, status)
+                        : launch_pass2_s<NCH, false>(c, m, s_div_out, rbar_out, vstages, status);
 }
 }  // namespace
 

@@ -425,6 +425,14 @@ def test_mix_chunk_edges(H, prefixes, mode):
     run_layer_parity(wl, variant="calibrated", pool_mode=mode)
 
 
+@pytest.mark.parametrize("G,W,lens", [(7, 32, (70, 129, 300, 900)), (15, 16, (17, 200, 145)), (1, 16, (130, 1030))])
+def test_many_short_heads_per_cta(G, W, lens):
+    # CTAs of pass 2 that go through several heads, of one tile and more: the normalisers of all but the first come
+    # from its spare warp
+    wl = synth.small_workload(H=8, G=G, W=W, seq_lens=lens, pool_kernel=7, budget=W + 16, seed=G, centroids=4)
+    run_layers_parity(wl, range(12), check=(0, 5, 11))
+
+
 def test_long_sequence_cluster_tail():
     # 65536 keys per head: clusters of eight with 8192 positions to a CTA
     wl = synth.small_workload(H=2, G=4, W=32, seq_lens=(65536,), pool_kernel=7, budget=512,
