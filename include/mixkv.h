@@ -280,7 +280,7 @@ int mixkv_layer_budget_schedule(int32_t n_layers, int32_t budget, int32_t window
  *   workspace  device, mixkv_similarity_workspace_size bytes, 16-byte aligned, caller-owned
  * A zero row has cosine 0 with every row.  The cells come from the Gram matrix of the
  * per-block sums of unit rows (one streaming pass over X, then the upper triangle of tiles on the
- * tensor cores, the sums as two (block == 1) or three bf16 parts).  Errors as for the other entry
+ * tensor cores, the sums as two 16-bit parts).  Errors as for the other entry
  * points, but for a bounded wait that expires inside a kernel: there is no status word, the cells it
  * concerns are NaN. */
 int mixkv_similarity_workspace_size(int32_t heads, int32_t L, int32_t block, size_t* bytes);

@@ -178,8 +178,8 @@ __host__ __device__ __forceinline__ size_t ppos(const SeqTable& st, int layer, i
 
 // Gram matrix of the block sums of a similarity map (similarity_tc.cu).
 struct GramArgs {
-  const void* parts;   // [nparts][heads][T][d] bf16: the block sums as 2 or 3 bf16 parts
-  int nparts;
+  const void* parts;   // [2][heads][T][d] fp16 (block 1: bf16): the scaled block sums as value and remainder
+  float inv_scale2;    // one over the square of the scale
   const int* nz;       // [heads][T]       non-zero rows of a block
   const float* us;     // [heads][slices][d]  partial sums of all unit rows of a head
   const int* nzs;      // [heads][slices]

@@ -28,7 +28,7 @@ int mixkv_internal_select(const float* scores, const int32_t* cu_seqlens_host, i
 // device holds at once (alone[n] with one CTA per SM, paired[n] with two, shared[n] with three, n = 1 .. 8).  No device is
 // needed.  decode: CTAs per unit and the depth of their rings; tail, budget: CTAs per unit, per (sequence, layer) pair;
 // adapt: threads of a CTA when the tail shares adaptive budgets out, 0: when it does not; gram: tiles of a map of `cells`
-// cells a side that a CTA takes in a run, 0: one contiguous share.
+// cells a side (parts 2: of single rows, 3: of sums) that a CTA takes in a run, 0: one contiguous share.
 void mixkv_internal_decode_shape(int64_t units, int32_t max_rows, int32_t even, int32_t sms, const int32_t* shared,
                                  const int32_t* alone, int32_t* ctas, int32_t* depth);
 int mixkv_internal_tail_clusters(int64_t units, int32_t candidates, int32_t sms, const int32_t* alone);

@@ -8,6 +8,9 @@
 // only where a cell is one pair of rows.
 #include <cooperative_groups.h>
 
+#include <cuda_fp16.h>
+#include <math.h>
+
 #include "common.cuh"
 
 namespace cg = cooperative_groups;
@@ -37,25 +40,41 @@ __host__ __device__ inline int blocks_per_cta(int block) {
   return sub < kSumWarps ? kSumWarps / sub : 1;
 }
 
-// x as a sum of bf16 parts, most significant first (8 mantissa bits each).
-template <int P>
-__device__ __forceinline__ void split_parts(const float (&x)[8], uint4 (&part)[P]) {
-  __nv_bfloat16 h[P][8];
+// x (scaled) as two fp16, value and remainder: 22 mantissa bits and the remainder's sign, fp32's 24 bits in all.
+__device__ __forceinline__ void split_pair(const float (&x)[8], uint4& hi, uint4& lo) {
+  __half2 h[4], l[4];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    float r = x[e];
-#pragma unroll
-    for (int p = 0; p < P; ++p) {
-      h[p][e] = __float2bfloat16_rn(r);
-      r -= __bfloat162float(h[p][e]);
-    }
+  for (int e = 0; e < 4; ++e) {
+    h[e] = __floats2half2_rn(x[2 * e], x[2 * e + 1]);
+    const float2 b = __half22float2(h[e]);
+    l[e] = __floats2half2_rn(x[2 * e] - b.x, x[2 * e + 1] - b.y);
   }
+  hi = *reinterpret_cast<const uint4*>(h);
+  lo = *reinterpret_cast<const uint4*>(l);
+}
+// A unit row as two bf16, 16 bits for what comes from 8.
+__device__ __forceinline__ void split_row(const float (&x)[8], uint4& hi, uint4& lo) {
+  __nv_bfloat162 h[4], l[4];
 #pragma unroll
-  for (int p = 0; p < P; ++p) part[p] = *reinterpret_cast<const uint4*>(h[p]);
+  for (int e = 0; e < 4; ++e) {
+    h[e] = __floats2bfloat162_rn(x[2 * e], x[2 * e + 1]);
+    const float2 b = __bfloat1622float2(h[e]);
+    l[e] = __floats2bfloat162_rn(x[2 * e] - b.x, x[2 * e + 1] - b.y);
+  }
+  hi = *reinterpret_cast<const uint4*>(h);
+  lo = *reinterpret_cast<const uint4*>(l);
+}
+// The power of two that the sums are scaled by: a component of a block's sum is at most its rows, which go to 2^15, half of
+// fp16's range, so that the remainder of everything down to 2^-17 of that has its bits.
+inline float sum_scale(const int block) {
+  int bits = 0;
+  while (bits < 31 && (1LL << bits) < block) ++bits;
+  return ldexpf(1.f, 15 - bits);
 }
 
-// grid (slices * cluster, H).  Sums of the unit rows of every block, written as P bf16 parts
-// ([P][H][T][d]: two parts where a row stands for itself, three, fp32's 24 bits, for sums), the
+// grid (slices * cluster, H).  Sums of the unit rows of every block, times `scale`, written as two fp16 parts
+// ([2][H][T][d]; a row that stands for itself as two bf16, unscaled: 4 heads of 5000 single rows 102 us as bf16 and 105 as
+// fp16), the
 // number of non-zero rows of every block, and per slice (what one CTA or cluster read) the sum of
 // its unit rows and its non-zero rows, from which the head mean comes.
 //
@@ -65,10 +84,10 @@ __device__ __forceinline__ void split_parts(const float (&x)[8], uint4 (&part)[P
 // for 8 butterflies), bf16 pairs are widened in place and multiplied as packed fp32.
 // B: the rows per block where they are a power of two up to 16 (the places where a block ends are then known
 // to the compiler; 14 us with a test after every row, 131072 rows in blocks of 16), else 0.
-template <int MODE, int P, int B>
+template <int MODE, int B>
 __global__ void __launch_bounds__(kSumThreads, MODE == kRowsMany ? 4 : 3)
-k_block_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block_arg, const int T,
-             __nv_bfloat16* __restrict__ parts, int* __restrict__ nz, float* __restrict__ us,
+k_block_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block_arg, const int T, const float scale,
+             uint16_t* __restrict__ parts, int* __restrict__ nz, float* __restrict__ us,
              int* __restrict__ nzs) {
   const int block = B ? B : block_arg;
   __shared__ __align__(16) float part[kSumWarps][kHeadDim];
@@ -83,7 +102,7 @@ k_block_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block_a
   const int bpc = blocks_per_cta(block);
   const size_t part_stride = (size_t)H * T * kHeadDim;
   const __nv_bfloat16* base = X + (size_t)h * L * kHeadDim + 8 * c;
-  __nv_bfloat16* prow = parts + (size_t)h * T * kHeadDim + 8 * c;
+  uint16_t* prow = parts + (size_t)h * T * kHeadDim + 8 * c;
   pdl_launch_dependents();
   pdl_wait();
 
@@ -169,13 +188,11 @@ k_block_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block_a
         tot[e] = add2(tot[e], pack2(s[2 * e], s[2 * e + 1]));
       }
       if (blk < T) {
-        uint4 q[P];
-        split_parts<P>(s, q);
-        // half 0 writes parts 0 and 2, half 1 part 1
-        *reinterpret_cast<uint4*>(prow + (size_t)half * part_stride + (size_t)blk * kHeadDim) =
-            half ? q[1] : q[0];
-        if (P == 3 && half == 0)
-          *reinterpret_cast<uint4*>(prow + 2 * part_stride + (size_t)blk * kHeadDim) = q[P - 1];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s[e] *= scale;
+        uint4 hi, lo;
+        split_pair(s, hi, lo);   // half 0 writes the values, half 1 the remainders
+        *reinterpret_cast<uint4*>(prow + (size_t)half * part_stride + (size_t)blk * kHeadDim) = half ? lo : hi;
         if (lane == 0) nz[(size_t)h * T + blk] = __popc(alive & ((1u << b) - (1u << a)));
       }
       ++blk;
@@ -201,11 +218,10 @@ k_block_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block_a
           x[2 * e] = x0 * w, x[2 * e + 1] = x1 * w;
         }
         if (r < stop) {
-          uint4 o2[P];
-          split_parts<P>(x, o2);
-#pragma unroll
-          for (int k = 0; k < P; ++k)
-            *reinterpret_cast<uint4*>(prow + k * part_stride + (size_t)r * kHeadDim) = o2[k];
+          uint4 hi, lo;
+          split_row(x, hi, lo);
+          *reinterpret_cast<uint4*>(prow + (size_t)r * kHeadDim) = hi;
+          *reinterpret_cast<uint4*>(prow + part_stride + (size_t)r * kHeadDim) = lo;
           if (c == 0) nz[(size_t)h * T + r] = w > 0.f ? 1 : 0;
         }
       } else if (MODE == kRowsFew) {
@@ -292,17 +308,18 @@ k_block_sums(const __nv_bfloat16* __restrict__ X, const int L, const int block_a
         for (int e = 0; e < 4; ++e) s[e] += part[w][4 * lane + e];
         n += cnt[w];
       }
+      __half2 o[2][2];
 #pragma unroll
-      for (int k = 0; k < P; ++k) {
-        __nv_bfloat16 o[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          o[e] = __float2bfloat16_rn(s[e]);
-          s[e] -= __bfloat162float(o[e]);
-        }
-        *reinterpret_cast<uint2*>(parts + k * part_stride + ((size_t)h * T + I) * kHeadDim + 4 * lane) =
-            *reinterpret_cast<const uint2*>(o);
+      for (int e = 0; e < 2; ++e) {
+        const float x = s[2 * e] * scale, y = s[2 * e + 1] * scale;
+        o[0][e] = __floats2half2_rn(x, y);
+        const float2 b = __half22float2(o[0][e]);
+        o[1][e] = __floats2half2_rn(x - b.x, y - b.y);
       }
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        *reinterpret_cast<uint2*>(parts + k * part_stride + ((size_t)h * T + I) * kHeadDim + 4 * lane) =
+            *reinterpret_cast<const uint2*>(o[k]);
       if (lane == 0) nz[(size_t)h * T + I] = n;
     }
   }
@@ -324,14 +341,13 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 // What a call of this shape needs between its two kernels.
 struct SimPlan {
-  int T, slices, nparts;
+  int T, slices;
   size_t parts_bytes, nz_bytes, us_bytes, nzs_bytes;
   SimPlan(int heads, int L, int block) {
     T = (int)(((long long)L + block - 1) / block);
     const int bpc = blocks_per_cta(block);
     slices = (T + bpc - 1) / bpc;
-    nparts = block == 1 ? 2 : 3;
-    parts_bytes = align256((size_t)nparts * heads * T * kHeadDim * 2);
+    parts_bytes = align256((size_t)2 * heads * T * kHeadDim * 2);
     nz_bytes = align256((size_t)heads * T * 4);
     us_bytes = align256((size_t)heads * slices * kHeadDim * 4);
     nzs_bytes = align256((size_t)heads * slices * 4);
@@ -371,7 +387,8 @@ int mixkv_similarity_map(const void* X, int32_t heads, int32_t L, int32_t head_d
   }
   cudaStream_t s = (cudaStream_t)stream;
   unsigned char* wsb = reinterpret_cast<unsigned char*>(workspace);
-  __nv_bfloat16* parts = reinterpret_cast<__nv_bfloat16*>(wsb);
+  uint16_t* parts = reinterpret_cast<uint16_t*>(wsb);
+  const float scale = block == 1 ? 1.f : sum_scale(block);
   wsb += pl.parts_bytes;
   int* nz = reinterpret_cast<int*>(wsb);
   wsb += pl.nz_bytes;
@@ -388,20 +405,20 @@ int mixkv_similarity_map(const void* X, int32_t heads, int32_t L, int32_t head_d
   const __nv_bfloat16* x = reinterpret_cast<const __nv_bfloat16*>(X);
   cudaError_t e;
   auto sums = [&](auto kernel) {
-    return launch_pdl(kernel, grid, dim3(kSumThreads), 0, s, S, x, L, block, pl.T, parts, nz, us, nzs);
+    return launch_pdl(kernel, grid, dim3(kSumThreads), 0, s, S, x, L, block, pl.T, scale, parts, nz, us, nzs);
   };
-  if (sum_mode(block) == kRowsMany) e = sums(k_block_sums<kRowsMany, 3, 0>);
+  if (sum_mode(block) == kRowsMany) e = sums(k_block_sums<kRowsMany, 0>);
   else switch (block) {
-    case 1: e = sums(k_block_sums<kRowsOne, 2, 1>); break;
-    case 2: e = sums(k_block_sums<kRowsFew, 3, 2>); break;
-    case 4: e = sums(k_block_sums<kRowsFew, 3, 4>); break;
-    case 8: e = sums(k_block_sums<kRowsFew, 3, 8>); break;
-    case 16: e = sums(k_block_sums<kRowsFew, 3, 16>); break;
-    default: e = sums(k_block_sums<kRowsFew, 3, 0>); break;
+    case 1: e = sums(k_block_sums<kRowsOne, 1>); break;
+    case 2: e = sums(k_block_sums<kRowsFew, 2>); break;
+    case 4: e = sums(k_block_sums<kRowsFew, 4>); break;
+    case 8: e = sums(k_block_sums<kRowsFew, 8>); break;
+    case 16: e = sums(k_block_sums<kRowsFew, 16>); break;
+    default: e = sums(k_block_sums<kRowsFew, 0>); break;
   }
   if (e != cudaSuccess) return MIXKV_ERR_CUDA;
   GramArgs g;
-  g.parts = parts, g.nparts = pl.nparts, g.nz = nz, g.us = us, g.nzs = nzs, g.slices = pl.slices;
+  g.parts = parts, g.inv_scale2 = 1.0f / (scale * scale), g.nz = nz, g.us = us, g.nzs = nzs, g.slices = pl.slices;
   g.heads = heads, g.L = L, g.block = block, g.T = pl.T, g.cells = cells, g.mean = mean_opt;
   return launch_gram(g, s) == cudaSuccess ? MIXKV_OK : MIXKV_ERR_CUDA;
 }

@@ -1,14 +1,14 @@
 // Second kernel of the redundancy analysis: the Gram matrix of the block sums on the tensor cores,
-// cell (I, J) = u_I . u_J / pairs (similarity.cu leaves the sums u as bf16 parts).
+// cell (I, J) = u_I . u_J / pairs (similarity.cu leaves the scaled sums u as two fp16 parts, single rows as two bf16).
 //
-// The sums come as P bf16 parts, so a product is the sum of the part products that carry fp32's bits:
-//   P = 2 (one row per block: x = hi + lo, 16 mantissa bits)      hi.hi + lo.hi + hi.lo
-//   P = 3 (hi + mid + lo, 24 bits)    hi.hi + mid.hi + lo.hi + hi.mid + mid.mid + hi.lo
+// u = hi + lo carries fp32's bits, and u.u = hi.lo + lo.hi + hi.hi but for lo.lo, 2^-24 of it.  The small products are
+// accumulated first, while the sum is small: against 64 bits the cells of blocks of 16 are 3.9e-7 off (2-norm), 1.26e-6 with
+// three bf16 parts and their six products, which moved half as many bytes again (4 heads of 32768 rows in blocks of 16
+// 30.5 us a call, now 25.4; of 20000 in blocks of 4 124, now 104).
 // Persistent CTAs walk a contiguous run of tiles (head, I, J): 128 blocks I on M, NT blocks J on N,
 // only tiles that touch or lie right of the diagonal.  The parts of I stay in shared memory while
-// J runs (P x 32 KB), the parts of J go through a ring of six half parts (with three whole ones a stage was asked
-// for again only half a tile ahead of its use, less than a round trip to L2), and two accumulator stages let the
-// epilogue of a tile overlap the MMA of the next.
+// J runs (2 x 32 KB), the parts of J go through a ring of four half parts, and two accumulator stages
+// let the epilogue of a tile overlap the MMA of the next.
 //
 // What bounds it: the output, T x T x 4 bytes per head, once T is large: a tile and its mirror image leave
 // as stores of 128 consecutive bytes of a row.
@@ -25,7 +25,10 @@ namespace {
 constexpr int kGThreads = 12 * 32;   // TMA, MMA, 2 head-mean, 8 epilogue warps
 constexpr int kGEpiWarp0 = 4, kGEpiWarps = 8;
 constexpr int kPartBytes = 128 * 256;   // one part of 128 blocks: two 64-column halves of 16 KB
-constexpr int kGStages = 6;            // halves (64 columns) of one part of the blocks on N
+constexpr int kParts = 2;
+// Halves (64 columns) of one part of the blocks on N: one tile's worth.  Twice as many gain nothing, and with 64 KB less the
+// next call's first kernel finds room beside this one (4 heads of 32768 rows in blocks of 16 26.8 us a call, now 25.4).
+constexpr int kGStages = 4;
 
 struct GBars {
   uint64_t afull, afree;
@@ -129,18 +132,18 @@ __device__ void head_mean(const float* __restrict__ us, const int* __restrict__ 
   named_bar_sync(1, 64);
 }
 
-template <int P, int NT, bool DEALT>
+template <int NT, bool DEALT>
 __global__ void __launch_bounds__(kGThreads, 1)
 k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
        const int* __restrict__ nz, const float* __restrict__ us, const int* __restrict__ nzs,
        const int slices, const int H, const int L, const int block, const int T, const int per_head, const int run,
-       float* __restrict__ cells, float* __restrict__ mean) {
+       const float inv_scale2, const uint32_t idesc, float* __restrict__ cells, float* __restrict__ mean) {
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* base =
       reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
   constexpr int kBHalf = NT * 128;                      // half a part of the NT blocks on N
-  unsigned char* sA = base;                             // P parts
-  unsigned char* sB = sA + P * kPartBytes;              // kGStages x half a part
+  unsigned char* sA = base;                             // both parts
+  unsigned char* sB = sA + kParts * kPartBytes;              // kGStages x half a part
   float* sT = reinterpret_cast<float*>(sB + kGStages * kBHalf);   // [8 warps][32 x 32]
   GBars* bars = reinterpret_cast<GBars*>(sT + kGEpiWarps * 1024);
   __shared__ float4 half_sum[32];   // head means
@@ -184,20 +187,20 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
       for (GramWalk<NT, DEALT> w = walk; w.valid() && ok; w.next()) {
         if (w.fresh) {
           if (rown > 0 && !mbar_wait(&bars->afree, (rown - 1) & 1, abort)) break;
-          mbar_expect_tx(&bars->afull, P * kPartBytes);
-          for (int p = 0; p < P; ++p) {
+          mbar_expect_tx(&bars->afull, kParts * kPartBytes);
+          for (int p = 0; p < kParts; ++p) {
             tma_load_3d(sA + p * kPartBytes, &tmA, 0, w.I * 128, p * H + w.h, &bars->afull);
             tma_load_3d(sA + p * kPartBytes + 16384, &tmA, 64, w.I * 128, p * H + w.h, &bars->afull);
           }
           ++rown;
         }
-        for (int x = 0; x < 2 * P && ok; ++x) {   // half x / P of part x % P
+        for (int x = 0; x < 2 * kParts && ok; ++x) {   // both halves of the remainders, then of the values
           if (!mbar_wait(&bars->bempty[s], ph, abort)) {
             ok = false;
             break;
           }
           mbar_expect_tx(&bars->bfull[s], kBHalf);
-          tma_load_3d(sB + s * kBHalf, &tmB, x / P * 64, w.I * 128 + w.c * NT, x % P * H + w.h, &bars->bfull[s]);
+          tma_load_3d(sB + s * kBHalf, &tmB, (x & 1) * 64, w.I * 128 + w.c * NT, (x < 2 ? H : 0) + w.h, &bars->bfull[s]);
           if (++s == kGStages) s = 0, ph ^= 1;
           ++it;
         }
@@ -209,7 +212,6 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
     // -------------------------------------------------------------------- MMA issuer
     {
       const uint32_t on = elect_one();
-      constexpr uint32_t idesc = umma_idesc_bf16(128, NT);
       const uint32_t a0 = umma_desc_lo(smem_u32(sA)), b0 = umma_desc_lo(smem_u32(sB));
       int s = 0, ph = 0, rown = 0, tile = 0;
       bool ok = true;
@@ -220,29 +222,38 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
         }
         const int ts = tile & 1, tph = (tile >> 1) & 1;
         if (!mbar_wait(&bars->tempty[ts], tph ^ 1, abort)) break;
-        // half by half of the contraction, part p of J meets the parts of I whose product with it carries weight
+        // part pa of I, half `half` of the contraction, times the half part of J in stage sb
+        auto product = [&](const int pa, const int half, const int sb, const bool first) {
+          const uint32_t oa = a0 + (uint32_t)(pa * (kPartBytes >> 4) + half * (16384 >> 4));
+          const uint32_t ob = b0 + (uint32_t)sb * (kBHalf >> 4);
 #pragma unroll
-        for (int x = 0; x < 2 * P; ++x) {
-          const int p = x % P, half = x / P;
+          for (int ks = 0; ks < 4; ++ks) {
+            if (first && ks == 0) umma_bf16_lo<0>(tmem + ts * 128, oa + ks * 2, ob + ks * 2, idesc, on);
+            else umma_bf16_lo<1>(tmem + ts * 128, oa + ks * 2, ob + ks * 2, idesc, on);
+          }
+        };
+        int values0 = 0;   // stage of the values' first half
+#pragma unroll
+        for (int x = 0; x < 2 * kParts; ++x) {
           if (!mbar_wait(&bars->bfull[s], ph, abort)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t bs = b0 + (uint32_t)s * (kBHalf >> 4);
-#pragma unroll
-          for (int pa = 0; pa < P - p; ++pa) {
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {
-              const uint32_t oa = (uint32_t)(pa * (kPartBytes >> 4) + half * (16384 >> 4) + ks * 2);
-              const uint32_t ob = (uint32_t)(ks * 2);
-              if (x == 0 && pa == 0 && ks == 0)
-                umma_bf16_lo<0>(tmem + ts * 128, a0 + oa, bs + ob, idesc, on);
-              else
-                umma_bf16_lo<1>(tmem + ts * 128, a0 + oa, bs + ob, idesc, on);
+          if (x < 2) {
+            product(0, x, s, x == 0);   // hi.lo
+            umma_commit(&bars->bempty[s], on);
+          } else {
+            product(1, x & 1, s, false);   // lo.hi
+            if (x == 2) {
+              values0 = s;
+            } else {   // hi.hi
+              product(0, 0, values0, false);
+              umma_commit(&bars->bempty[values0], on);
+              product(0, 1, s, false);
+              umma_commit(&bars->bempty[s], on);
             }
           }
-          umma_commit(&bars->bempty[s], on);
           if (++s == kGStages) s = 0, ph ^= 1;
         }
         umma_commit(&bars->tfull[ts], on);
@@ -291,7 +302,7 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
           if (lane == 0) mbar_arrive(&bars->tempty[ts]);
         }
         if (j0 >= T || i0 >= T) continue;
-        const float sc = inv_i * inv_j;
+        const float sc = inv_i * inv_j * inv_scale2;
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) * sc);
         if (j0 + 31 >= T - 1 || j0 == i0) {   // the last block, or cells of the diagonal
@@ -376,32 +387,31 @@ long long device_l2_bytes() {
 // so that all CTAs together write whole rows of the map at a time.  That counts where the map goes to HBM: it leaves L2
 // in about the order in which it was written.  Contiguous / in runs, us, B200 (L2 of 133 MB), maps in turn on four inputs:
 //   Rows that do not start on 32-byte sectors (T not a multiple of 8, or a map that does not): neighbouring tiles share
-//   sectors, and a sector that leaves half written is read again.  Runs of one from half of L2 on: 4 heads x 1801 cells a
-//   side (52 MB) 36.7 / 36.4, x 2001 (64 MB) 41.2 / 36.7, x 2401 55.8 / 47.2, x 2801 (126 MB) 69.1 / 57.3, x 5001 (400 MB)
-//   212 / 175; blocks of 16, whose sums take longer, gain less: 8 x 1450 (67 MB) 43.9 / 45.9, x 1950 70.4 / 66.4.  (One
-//   map written over and over stays in L2 and would be better off contiguous up to 100 MB: 4 x 2001 32.2 / 34.2.)
-//   Whole sectors: only the largest maps gain (pages of HBM filled in one go), from 9/4 of L2 on: runs of one with two
-//   parts (4 x 4400, 310 MB, 88.9 / 77.7, x 5000 114 / 92, one map alone 4 x 8192 283 / 218), runs of two with three parts,
-//   where the parts of I weigh more (4 x 4400 90.7 / 87.3, x 5000 119.7 / 121.3, alone 4 x 5600 149 / 140, 4 x 8192
-//   317 / 287; below, 4 x 4000, 256 MB, 75.3 / 78.0).
-int gram_run(const int heads, const int T, const int nparts, const bool whole_sectors, const long long l2) {
+//   sectors, and a sector that leaves half written is read again.  Runs of one from half of L2 on: sums, 4 heads x 2401 cells
+//   a side (92 MB) 46.4 / 44.2, x 2801 (126 MB) 59.4 / 52.2, 8 x 1950 (122 MB) 63.7 / 60.3; the line lies where it was
+//   measured with longer operands (4 x 2001, 64 MB, 41.2 / 36.7 then, 30.4 / 33.0 now; 8 x 1451, 67 MB, 37.5 / 40.7).
+//   Whole sectors: only the largest maps gain (pages of HBM filled in one go), from 9/4 of L2 on: single rows in runs of
+//   one (4 x 4400, 310 MB, 86.4 / 83.7, x 5000 113 / 105), sums in runs of two (4 x 4400 89.0 / 84.3, x 5000 117 / 107,
+//   x 5600 136 / 125; 4 x 4000, 256 MB, 73.9 / 72.3).
+// kind: 2 single rows, 3 sums.
+int gram_run(const int heads, const int T, const int kind, const bool whole_sectors, const long long l2) {
   const long long bytes = 4LL * heads * T * T;
   if (!whole_sectors) return 2 * bytes > l2 ? 1 : 0;
-  return 4 * bytes > 9 * l2 ? (nparts == 2 ? 1 : 2) : 0;
+  return 4 * bytes > 9 * l2 ? (kind == 2 ? 1 : 2) : 0;
 }
 
-template <int P, int NT, bool DEALT>
+template <int NT, bool DEALT>
 cudaError_t launch_gram_t(const GramArgs& g, const long long per_head, const int run, cudaStream_t s) {
   static std::atomic<bool> done[kMaxDevices];
-  const size_t smem = 1024 + (size_t)P * kPartBytes + (size_t)kGStages * NT * 128 +
+  const size_t smem = 1024 + (size_t)kParts * kPartBytes + (size_t)kGStages * NT * 128 +
                       (size_t)kGEpiWarps * 4096 + sizeof(GBars);
-  const cudaError_t e = ensure_smem(k_gram<P, NT, DEALT>, smem, done);
+  const cudaError_t e = ensure_smem(k_gram<NT, DEALT>, smem, done);
   if (e != cudaSuccess) return e;
   const long long total = per_head * g.heads;
   if (total > 0x7fffffffLL) return cudaErrorInvalidValue;
   CUtensorMap tmA, tmB;
   const unsigned long long dims[3] = {(unsigned long long)kHeadDim, (unsigned long long)g.T,
-                                      (unsigned long long)P * g.heads};
+                                      (unsigned long long)kParts * g.heads};
   const unsigned long long strides[2] = {(unsigned long long)kHeadDim * 2,
                                          (unsigned long long)g.T * kHeadDim * 2};
   const unsigned boxA[3] = {64, 128, 1}, boxB[3] = {64, (unsigned)NT, 1};
@@ -409,9 +419,9 @@ cudaError_t launch_gram_t(const GramArgs& g, const long long per_head, const int
       !encode_bf16_map(&tmB, g.parts, 3, dims, strides, boxB))
     return cudaErrorInvalidValue;
   const int grid = (int)(total < device_sm_count() ? total : device_sm_count());
-  return launch_pdl(k_gram<P, NT, DEALT>, dim3((unsigned)grid), dim3(kGThreads), smem, s, 1, tmA, tmB, g.nz, g.us,
+  return launch_pdl(k_gram<NT, DEALT>, dim3((unsigned)grid), dim3(kGThreads), smem, s, 1, tmA, tmB, g.nz, g.us,
                     g.nzs, g.slices, g.heads, g.L, g.block, g.T, (int)per_head,
-                    run, g.cells, g.mean);
+                    run, g.inv_scale2, g.block == 1 ? umma_idesc_bf16(128, NT) : umma_idesc_f16(128, NT), g.cells, g.mean);
 }
 
 template <int NT>
@@ -428,14 +438,10 @@ cudaError_t launch_gram(const GramArgs& g, cudaStream_t s) {
   const bool narrow = wide * g.heads < device_sm_count();
   const long long per_head = narrow ? tiles_per_head<32>(g.T) : wide;
   const bool whole_sectors = g.T % 8 == 0 && (reinterpret_cast<uintptr_t>(g.cells) & 31) == 0;
-  const int run = narrow ? 0 : gram_run(g.heads, g.T, g.nparts, whole_sectors, device_l2_bytes());
-  if (g.nparts == 2)
-    return narrow ? launch_gram_t<2, 32, false>(g, per_head, 0, s)
-           : run  ? launch_gram_t<2, 128, true>(g, per_head, run, s)
-                  : launch_gram_t<2, 128, false>(g, per_head, 0, s);
-  return narrow ? launch_gram_t<3, 32, false>(g, per_head, 0, s)
-         : run  ? launch_gram_t<3, 128, true>(g, per_head, run, s)
-                : launch_gram_t<3, 128, false>(g, per_head, 0, s);
+  const int run = narrow ? 0 : gram_run(g.heads, g.T, g.block == 1 ? 2 : 3, whole_sectors, device_l2_bytes());
+  return narrow ? launch_gram_t<32, false>(g, per_head, 0, s)
+         : run  ? launch_gram_t<128, true>(g, per_head, run, s)
+                : launch_gram_t<128, false>(g, per_head, 0, s);
 }
 
 }  // namespace mixkv

@@ -114,6 +114,11 @@ __host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
          ((uint32_t)(M >> 4) << 24);
 }
 
+// The same with A and B fp16.
+__host__ __device__ constexpr uint32_t umma_idesc_f16(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+
 // A descriptor as two 32-bit halves: the high half is a constant, the low half is
 // ((address >> 4) & 0x3fff) | 1 << 16, so stepping an operand by n bytes (n a multiple of 16,
 // inside shared memory) is an integer add of n >> 4 to the low half.
