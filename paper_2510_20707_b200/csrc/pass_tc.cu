@@ -301,13 +301,9 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     tma_prefetch_desc(&tmK);
     tma_prefetch_desc(&tmQ);
   }
-  // Two query blocks: the divisions once, ahead of the wait, instead of in every role behind it (4 x 1024 keys, one layer
-  // 21.4 -> 20.8 us).  With one block the loops that come out of the compiler that way take 1 % longer (32 layers of 8 x
-  // 16384 keys 608 and 617 us): every role for itself there.
-  if (MB == 2 && tid == kEpiWarp0 * 32) bars->first = layer_tile_coord(st.tile1_start, st.batch, H, st.nt1, lo);
-  auto first_tile = [&]() -> TileCoord {
-    return MB == 2 ? bars->first : layer_tile_coord(st.tile1_start, st.batch, H, st.nt1, lo);
-  };
+  // The divisions once, ahead of the wait, instead of in every role behind it (one layer of 4 x 1024 keys 21.4 -> 20.8 us;
+  // with one query block 18.4 -> 17.8, 4 x 5000 24.9 -> 24.2, 32 layers of 8 x 16384 level).
+  if (tid == kEpiWarp0 * 32) bars->first = layer_tile_coord(st.tile1_start, st.batch, H, st.nt1, lo);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -322,7 +318,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
       if (lane == 0) {
         int s = 0, ph = 1, it = 0, segn = 0;
         bool ok = true;
-        for (SegIter sg(st.tile1_start, st.batch, H, first_tile(), lo, hi); sg.valid() && ok; sg.next()) {
+        for (SegIter sg(st.tile1_start, st.batch, H, bars->first, lo, hi); sg.valid() && ok; sg.next()) {
           if (segn > 0 && !mbar_wait(&bars->qfree, (segn - 1) & 1, abort)) break;
           mbar_expect_tx(&bars->qfull, NQ * 256);
           tma_load_3d(sQ, &tmQ, 0, sg.bh() * NQ, sg.layer, &bars->qfull);
@@ -354,7 +350,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         const uint32_t q_half = (uint32_t)(NQ * 128) >> 4;   // second 64-column half of the queries
         int s = 0, ph = 0, ts = 0, tph = 1, segn = 0;
         bool ok = true;
-        for (SegIter sg(st.tile1_start, st.batch, H, first_tile(), lo, hi); sg.valid() && ok; sg.next()) {
+        for (SegIter sg(st.tile1_start, st.batch, H, bars->first, lo, hi); sg.valid() && ok; sg.next()) {
           if (!mbar_wait(&bars->qfull, segn & 1, abort)) break;
           ++segn;
           for (int k = 0; k < sg.n; ++k) {
@@ -413,7 +409,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     constexpr int kXThreads = NU * 128;
     int ts = 0, tph = 0, segs_done = 0;
     const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + col0;
-    for (SegIter sg(st.tile1_start, st.batch, H, first_tile(), lo, hi); sg.valid(); sg.next()) {
+    for (SegIter sg(st.tile1_start, st.batch, H, bars->first, lo, hi); sg.valid(); sg.next()) {
       float m_run = -1e30f, z_run = 0.f;
       const int P = st.cu[sg.b + 1] - st.cu[sg.b] - W;
       const int t_mask = P / kTile;   // first tile that holds keys some row may not see
@@ -498,7 +494,7 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     const uint32_t off1 = (uint32_t)(16 * aux_w + lg) * 128 + ((uint32_t)(c ^ (lg + 4)) << 4);
     const int my_row = 16 * aux_w + 4 * (c >> 1) + lg;   // the row whose norm this lane ends with
     int s = 0, ph = 0;
-    for (SegIter sg(st.tile1_start, st.batch, H, first_tile(), lo, hi); sg.valid(); sg.next()) {
+    for (SegIter sg(st.tile1_start, st.batch, H, bars->first, lo, hi); sg.valid(); sg.next()) {
       f32x2 acc2[8];   // dims 8c .. 8c+7 of half 0, then of half 1, as packed pairs
 #pragma unroll
       for (int e = 0; e < 8; ++e) acc2[e] = pack2(0.f, 0.f);
