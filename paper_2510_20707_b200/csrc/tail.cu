@@ -1167,7 +1167,7 @@ cudaError_t launch_budget(const LaunchCtx& c, const float* scores, int* counts) 
   const size_t want = (size_t)c.st.H * ((chunk + 31) / 32) * 128;
   const size_t cap_bytes = 200 * 1024;
   const size_t smem = want <= cap_bytes ? want : 0;
-  if (smem > 24 * 1024) {   // on top of the search's static shared memory
+  if (smem > 20 * 1024) {   // on top of the static shared memory of the search
     static std::atomic<bool> done[kMaxDevices];
     const cudaError_t e = ensure_smem(k_budget, cap_bytes, done);
     if (e != cudaSuccess) return e;

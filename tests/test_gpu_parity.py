@@ -415,6 +415,20 @@ def test_adaptive_budget_cluster_edges(batch, H, P):
     assert np.array_equal(got["idx"].cpu().numpy()[:offs[-1]], ref["idx"])
 
 
+@pytest.mark.parametrize("P", [320, 352, 384, 416])
+def test_adaptive_budget_keys_around_the_default_shared_memory(P):
+    # 16 heads of P keys: 20, 22, 24 and 26 KB of them next to the search's own 25 KB; 48 are a kernel's without asking
+    H, W = 16, 16
+    rng = np.random.default_rng(P)
+    s = (rng.integers(0, 700, size=(H, P)) / np.float32(700)).astype(np.float32)
+    ref = oracle.select(s, oracle.Params(kv_heads=H, gqa_ratio=1, window=W, budget=W + 40, budget_mode=1))
+    got = binding.select(torch.from_numpy(s).cuda(),
+                         binding.Params(kv_heads=H, gqa_ratio=1, window=W, budget=W + 40, budget_mode=1))
+    offs = got["idx_offsets"].cpu().numpy()
+    assert np.array_equal(got["counts"].cpu().numpy(), ref["counts"].reshape(-1))
+    assert np.array_equal(got["idx"].cpu().numpy()[:offs[-1]], ref["idx"])
+
+
 @pytest.mark.parametrize("H,prefixes,mode", [
     (2, (511, 512, 513), 0), (3, (2047, 2048, 2049), 1), (1, (2561, 400, 4096), 0),   # chunks of 512 positions
     (8, (2100,) * 9, 0), (8, (2100,) * 10, 1)])                                       # 144 chunks of 2048, the last; 160
