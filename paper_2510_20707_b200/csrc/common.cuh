@@ -221,7 +221,7 @@ bool tail_adapts(const LaunchCtx& c);
 
 // Launch with programmatic dependent launch (and an optional cluster size): the kernel may
 // start while its predecessor in the stream drains; every kernel calls pdl_wait() before it
-// touches global memory.
+// touches global memory that an earlier one may still write or read (pass 2 loads the call's inputs without).
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
                        cudaStream_t stream, int cluster, Args... args) {
