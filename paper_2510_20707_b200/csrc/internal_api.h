@@ -41,6 +41,9 @@ int mixkv_internal_budget_clusters(int32_t pairs, int64_t keys_per_pair, const i
 // first[0 .. CTAs] their first tiles, owner[tiles] the CTA that pass 2 and the tail look for a tile's statistics at.
 int mixkv_internal_split_tiles(int32_t tiles, int32_t per_head, int32_t sms, int32_t* first, int32_t* owner);
 
+// Table of 16 words that the warps of a pair of pass 2's epilogue hand their statistics of a CTA's segment over in.
+int mixkv_internal_stats_table(int32_t segment, int32_t pair);
+
 #ifdef __cplusplus
 }
 #endif

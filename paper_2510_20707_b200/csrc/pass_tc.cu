@@ -625,6 +625,9 @@ __device__ __forceinline__ void colsum16(const uint32_t (&r)[16], const float* n
   }
 }
 
+// Table of 16 words in which the warps of pair `wg` of the epilogue meet at the end of segment `segn` of a CTA.
+__host__ __device__ __forceinline__ int stats_table(const int segn, const int wg) { return (segn & 1) * 2 + wg; }
+
 // grid = g2 persistent CTAs: K producer, MMA, V producer, 1 spare, 16 epilogue, 4 value-norm warps.
 // NCH: pieces of 16 query columns per epilogue warp, at most.
 // SPARE: the spare warp folds the normalisers of the CTA's segments after the first (see pass2_spare).  A template argument
@@ -646,8 +649,9 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
   float* sbq = reinterpret_cast<float*>(sV + vstages * kVSubBytes);  // [2][256] negated normalisers
   float* sxp = sbq + 512;                     // [2][128] partial column sums of the second column halves
   float* skp = sxp + 256;                     // [4][128] parts of the unit-key sum
-  float* sred = skp + 512;    // [64]: 2 x 16 epilogue, 12 value norms, 4 mean key
-  P2Bars* bars = reinterpret_cast<P2Bars*>(sred + 64);
+  float* sred = skp + 512;    // [96]: 2 x 2 x 16 epilogue, 12 value norms, 4 mean key
+  float* sred_v = sred + 64;
+  P2Bars* bars = reinterpret_cast<P2Bars*>(sred + 96);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int lo = cta_first_tile(blockIdx.x, st.sp2);
@@ -832,8 +836,8 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
     const f32x2 sc2 = pack2(scale_log2e, scale_log2e);
     const uint32_t tstage = tmem + ((uint32_t)(quarter * 32) << 16) + wg * 256, taddr = tstage + ch_lo * 16;
     int tile = 0;   // parity decides which pair owns it
-    int segn = 0;
-    for (RevSegIter sg(st.tile2_start, st.batch, H, bars->last, lo, hi); sg.valid(); sg.next()) {
+    int segn = 0;   // (counted with SPARE only)
+    for (RevSegIter sg(st.tile2_start, st.batch, H, bars->last, lo, hi); sg.valid(); sg.next(), segn += SPARE ? 1 : 0) {
       const int P = st.cu[sg.b + 1] - st.cu[sg.b] - W;
       if (SPARE && segn > 0) {
         mbar_wait(&bars->nfull[segn & 1], ((segn - 1) >> 1) & 1, abort);
@@ -925,13 +929,14 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
       if constexpr (SPARE) {
         __syncwarp();
         if (lane == 0) mbar_arrive(&bars->nempty[segn & 1]);
-        ++segn;
       }
       if (chalf == 0) {
-        // this pair's share of the segment's score statistics (neutral if it had no tile)
+        // This pair's share of the segment's score statistics (neutral if it had no tile).  With SPARE nothing holds a warp
+        // between the barrier here and its words of the next segment, if that is one tile of the other pair's, so two tables
+        // take turns: the barrier of the segment in between stands behind the read.  (Without, barrier 5 does.)
         const float a = warp_min(dmin), b2 = warp_max(dmax), c2 = warp_sum(dsum),
                     d2 = warp_sum(exw);
-        float* sr = sred + wg * 16;
+        float* sr = sred + stats_table(SPARE ? segn : 0, wg) * 16;
         if (lane == 0) {
           sr[gw] = a;
           sr[4 + gw] = b2;
@@ -986,10 +991,10 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
       if (lane == 0) mbar_arrive(&bars->kbready);   // the MMA may start: the rest is off its path
       if (sg.t0 == 0) {                 // the same in all 128 threads
         const float n2 = warp_sum(ks * ks);
-        if (lane == 0) sred[44 + (warp - kP2AuxWarp0)] = n2;
+        if (lane == 0) sred_v[12 + (warp - kP2AuxWarp0)] = n2;
         named_bar_sync(4, 128);
         if (vt == 0) {
-          const double nn = ((double)sred[44] + (double)sred[45]) + ((double)sred[46] + (double)sred[47]);
+          const double nn = ((double)sred_v[12] + (double)sred_v[13]) + ((double)sred_v[14] + (double)sred_v[15]);
           const double T = (double)L;
           const float r = (float)((nn - T) / (T * (T - 1.0)));   // Eq. 4
           ws.rbar[sg.unit()] = r;
@@ -1058,16 +1063,16 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         const float a = warp_min(vmin), b2 = warp_max(vmax), c2 = warp_sum(vsum);
         const int vw = warp - kP2AuxWarp0;
         if (lane == 0) {
-          sred[32 + vw] = a;
-          sred[36 + vw] = b2;
-          sred[40 + vw] = c2;
+          sred_v[vw] = a;
+          sred_v[4 + vw] = b2;
+          sred_v[8 + vw] = c2;
         }
         named_bar_sync(4, 128);
         if (vt == 0) {
           ws.vstat[sg.id] = make_float4(
-              fminf(fminf(sred[32], sred[33]), fminf(sred[34], sred[35])),
-              fmaxf(fmaxf(sred[36], sred[37]), fmaxf(sred[38], sred[39])),
-              (sred[40] + sred[41]) + (sred[42] + sred[43]), 0.f);
+              fminf(fminf(sred_v[0], sred_v[1]), fminf(sred_v[2], sred_v[3])),
+              fmaxf(fmaxf(sred_v[4], sred_v[5]), fmaxf(sred_v[6], sred_v[7])),
+              (sred_v[8] + sred_v[9]) + (sred_v[10] + sred_v[11]), 0.f);
         }
         named_bar_sync(4, 128);
       }
@@ -1146,7 +1151,7 @@ constexpr size_t pass1_smem(int NQ) {
 constexpr size_t kP1SmemLimit = kSmemLimit - (kP1AuxWarps * 128 * 4 + kP1XRows * 8 + sizeof(P1Bars) + 63) / 64 * 64;
 constexpr size_t pass2_smem(int NQ, int vstages) {
   return 1024 + (size_t)2 * (NQ + kExtraRows) * 128 + kP2KStages * kTileBytes +
-         (size_t)vstages * kVSubBytes + 1280 * 4 + 64 * 4 + sizeof(P2Bars) + 64;
+         (size_t)vstages * kVSubBytes + 1280 * 4 + 96 * 4 + sizeof(P2Bars) + 64;
 }
 // V stages: the two pairs of value-norm warps need one each.
 constexpr int pass2_vstages(int NQ) {
@@ -1255,3 +1260,5 @@ cudaError_t launch_pass2(const LaunchCtx& c, const void* K, const void* V, const
 }
 
 }  // namespace mixkv
+
+extern "C" int mixkv_internal_stats_table(int32_t segment, int32_t pair) { return mixkv::stats_table(segment, pair); }

@@ -488,6 +488,24 @@ def test_repeated_calls_are_bit_identical_widest_query_tile():
         assert torch.equal(first["V_out"].view(torch.int16), out["V_out"].view(torch.int16))
 
 
+def test_heads_of_one_tile_between_long_ones():
+    # CTAs of pass 2 with segments of one tile behind longer ones: statistics of neighbouring segments in tables of
+    # their own, the same bits call after call
+    wl = synth.small_workload(H=4, G=7, W=32, seq_lens=(2100, 130, 1900, 160, 97), pool_kernel=7, budget=64, seed=41,
+                              centroids=8)
+    wl = synth.replace(wl, layers=12)
+    run_layers_parity(wl, range(12), check=(0, 5, 11))
+    _, pg = params_pair(wl)
+    xs = [synth.make_layer(wl, l, "calibrated") for l in range(12)]
+    K, V, Q = (torch.stack([to_dev(x[k]) for x in xs]) for k in ("K", "V", "Q"))
+    cu = [int(c) for c in wl.cu_seqlens]
+    first = binding.compress_layers(K, V, Q, pg, cu_seqlens=cu)
+    for _ in range(200):
+        out = binding.compress_layers(K, V, Q, pg, cu_seqlens=cu)
+        assert torch.equal(first["s_comp"], out["s_comp"]) and torch.equal(first["idx_offsets"], out["idx_offsets"])
+    assert int(out["status"].item()) == 0
+
+
 def test_workspace_needs_no_clearing():
     # Every word of the workspace that a kernel reads was written earlier in the same call:
     # whatever the workspace holds (all ones, all zeros, random bytes, what an earlier call on

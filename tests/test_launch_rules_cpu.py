@@ -107,3 +107,31 @@ def test_every_tile_has_one_cta(lib, heads, per_head, sms):
         assert max(shares) <= even + (1 if uniform and apart else 0)
         if uniform and heads <= sms and -(-per_head // min(per_head, sms // heads)) <= even + 1:
             assert apart
+
+
+def pass2_segments(lib, lens, heads, layers, window, sms=148):
+    """Tiles of the segments of every CTA of pass 2, in the order in which it takes them (the last one first)."""
+    per_head = [-(-(n - window) // 128) for n in lens]
+    runs = [t for _ in range(layers) for t in per_head for _ in range(heads)]
+    tiles, uniform = sum(runs), per_head[0] if len(set(per_head)) == 1 else 0
+    first, owner = (C.c_int32 * (sms + 1))(), (C.c_int32 * tiles)()
+    g = lib.mixkv_internal_split_tiles(tiles, uniform, sms, first, owner)
+    of_cta, t = [[] for _ in range(g)], 0
+    for n in runs:
+        for c in sorted(set(owner[t:t + n])):
+            of_cta[c].append(sum(o == c for o in owner[t:t + n]))
+        t += n
+    return [segs[::-1] for segs in of_cta]
+
+
+@pytest.mark.parametrize("lens,heads,layers,window", [
+    ((4096,), 4, 28, 32), ((3001, 1777, 6143), 4, 28, 32), ((2100, 130, 1900, 160, 97), 4, 12, 32), ((130, 1030), 8, 12, 16)])
+def test_segments_of_one_tile_have_statistics_of_their_own(lib, lens, heads, layers, window):
+    # A segment of one tile is one pair's of the epilogue.  The other pair comes to its statistics with nothing in between
+    # that waits for its first warp, which may still be reading those of the segment before; only the barrier of the
+    # segment in between orders that read ahead of the writes of the one after.  So neighbours never share words.
+    segments = pass2_segments(lib, lens, heads, layers, window)
+    assert any(1 in of_cta[1:] for of_cta in segments)
+    for s in range(max(len(of_cta) for of_cta in segments)):
+        tables = {(k, wg): lib.mixkv_internal_stats_table(k, wg) for k in (s, s + 1) for wg in (0, 1)}
+        assert sorted(tables.values()) == [0, 1, 2, 3]
