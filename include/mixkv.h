@@ -118,7 +118,10 @@ int mixkv_workspace_size_layers(const mixkv_params* p, int32_t n_layers, int32_t
  *   rbar_opt      out, optional, [batch, H]
  *   rbar_in_opt   in, optional, [batch, H]: redundancy to mix with instead of the computed
  *                 one (head weights calibrated offline, Sec. 4.3)
- *   V may be NULL unless use_vnorm == MIXKV_INTRINSIC_VNORM. */
+ *   V may be NULL unless use_vnorm == MIXKV_INTRINSIC_VNORM.
+ * NaN or infinite values in K, V or Q can make every score of their head NaN, in their sequence and in the one before
+ * it in the batch.  Selection takes any scores: a NaN ranks by its bits, above every number or (sign set) below, and
+ * budgets, offsets and index lists are those of such scores, within the outputs' sizes. */
 int mixkv_scores(const void* K, const void* V, const void* Qwin,
                  const int32_t* cu_seqlens_host, int32_t batch, int32_t L,
                  const mixkv_params* p, void* workspace, size_t workspace_bytes,

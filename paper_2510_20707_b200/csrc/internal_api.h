@@ -37,6 +37,10 @@ int mixkv_internal_adapt_threads(int64_t sequences, int32_t heads, int32_t candi
 int mixkv_internal_gram_run(int32_t heads, int32_t cells, int32_t parts, int32_t whole_sectors, int64_t l2_bytes);
 int mixkv_internal_budget_clusters(int32_t pairs, int64_t keys_per_pair, const int32_t* alone);
 
+// Rounds of a threshold search among keys lo .. hi that ends at `key` without listing any: keys [base, base + span] counted
+// in bins of 2^shift.  Returns their number (three at most).
+int mixkv_internal_search_rounds(uint32_t lo, uint32_t hi, uint32_t key, uint32_t* base, uint32_t* span, int32_t* shift);
+
 // How `tiles` are split over at most `sms` CTAs (per_head: the tiles of every head, 0: heads differ): the number of CTAs;
 // first[0 .. CTAs] their first tiles, owner[tiles] the CTA that pass 2 and the tail look for a tile's statistics at.
 int mixkv_internal_split_tiles(int32_t tiles, int32_t per_head, int32_t sms, int32_t* first, int32_t* owner);

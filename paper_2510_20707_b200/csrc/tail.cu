@@ -328,6 +328,30 @@ constexpr int kSelBinBits = 11, kSelBins = 1 << kSelBinBits;
 constexpr int kSelListCap = 256;   // candidates ranked directly
 constexpr int kSelMaxCluster = kMaxCluster;
 
+// The keys that a round of a search counts, [base, base + span], in bins of 2^shift keys.  Never past the largest key there is:
+// the last bin of a range would else reach over 2^32, and keys below all others (k_budget's padding is key 0) be counted in it.
+struct SelRange {
+  unsigned base, span;
+  int shift;
+};
+// The first round's: all keys, lo the smallest and hi the largest.
+__host__ __device__ __forceinline__ SelRange sel_range(const unsigned lo, const unsigned hi) {
+  SelRange r{lo, hi - lo, 0};
+#ifdef __CUDA_ARCH__
+  const int bits = 32 - __clz(r.span);
+#else
+  const int bits = r.span ? 32 - __builtin_clz(r.span) : 0;
+#endif
+  if (bits > kSelBinBits) r.shift = bits - kSelBinBits;
+  return r;
+}
+// The keys of one bin, not yet binned again.
+__host__ __device__ __forceinline__ SelRange sel_bin(const SelRange& r, const unsigned bin, const unsigned hi) {
+  const unsigned base = r.base + (bin << r.shift), size = (1u << r.shift) - 1u;
+  return {base, size < hi - base ? size : hi - base, r.shift};
+}
+__host__ __device__ __forceinline__ int sel_next_shift(const int shift) { return shift > kSelBinBits ? shift - kSelBinBits : 0; }
+
 struct SelSmem {
   int hist[2][kSelBins];
   unsigned list[kSelListCap];    // this CTA's candidates
@@ -409,19 +433,18 @@ __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const
   if (cs > 1) {
     if (tid < cs) *cluster.map_shared_rank(&sm.range[crank], tid) = make_uint2(lo, hi);
     cluster.sync();
-    const uint2 r = lane < cs ? sm.range[lane] : make_uint2(0xffffffffu, 0u);
-    lo = r.x, hi = r.y;
+    const uint2 mine = lane < cs ? sm.range[lane] : make_uint2(0xffffffffu, 0u);
+    lo = mine.x, hi = mine.y;
     lo = __reduce_min_sync(0xffffffffu, lo);
     hi = __reduce_max_sync(0xffffffffu, hi);
   }
-  unsigned base = lo, span = hi - lo;   // the candidates are the keys in [base, base + span]
-  int shift = span ? max(0, 32 - __clz(span) - kSelBinBits) : 0;
+  SelRange r = sel_range(lo, hi);   // of the candidates
   int remaining = want, gt_before = 0;
   for (int round = 0;; ++round) {
     int* hist = sm.hist[round & 1];
     for (int j = tid; j < n; j += T) {
-      const unsigned d = key_at(j) - base;
-      if (d <= span) atomicAdd(&hist[d >> shift], 1);
+      const unsigned d = key_at(j) - r.base;
+      if (d <= r.span) atomicAdd(&hist[d >> r.shift], 1);
     }
     __syncthreads();
     // thread t owns bins PER t .. PER t + PER - 1
@@ -434,16 +457,16 @@ __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const
 #pragma unroll
       for (int o = 1; o < GL; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
       int* slot = &mail.groups[round & 1][crank][tid / GL];
-      for (int r = lane % GL; r < cs; r += GL) *cluster.map_shared_rank(slot, r) = sum;
+      for (int to = lane % GL; to < cs; to += GL) *cluster.map_shared_rank(slot, to) = sum;
       cluster.sync();
       if (warp == 0) {
         // two groups per lane, of all CTAs and of those of lower rank
         int2 tot = make_int2(0, 0), low = tot;
 #pragma unroll
-        for (int r = 0; r < kSelMaxCluster; ++r) {
-          const int2 v = r < cs ? *reinterpret_cast<const int2*>(&mail.groups[round & 1][r][2 * lane]) : make_int2(0, 0);
+        for (int of = 0; of < kSelMaxCluster; ++of) {
+          const int2 v = of < cs ? *reinterpret_cast<const int2*>(&mail.groups[round & 1][of][2 * lane]) : make_int2(0, 0);
           tot.x += v.x, tot.y += v.y;
-          if (r < crank) low.x += v.x, low.y += v.y;
+          if (of < crank) low.x += v.x, low.y += v.y;
         }
         auto keys_above = [&](const int v) {   // sum of v over the higher lanes
           int incl = v;
@@ -464,9 +487,9 @@ __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const
         // the bins of that group, one per lane
         int v[kSelMaxCluster], all = 0, lower = 0;
 #pragma unroll
-        for (int r = 0; r < kSelMaxCluster; ++r) v[r] = r < cs ? *cluster.map_shared_rank(&hist[32 * group + lane], r) : 0;
+        for (int of = 0; of < kSelMaxCluster; ++of) v[of] = of < cs ? *cluster.map_shared_rank(&hist[32 * group + lane], of) : 0;
 #pragma unroll
-        for (int r = 0; r < kSelMaxCluster; ++r) all += v[r], lower += r < crank ? v[r] : 0;
+        for (int of = 0; of < kSelMaxCluster; ++of) all += v[of], lower += of < crank ? v[of] : 0;
         above += keys_above(all);
         src = __ffs(__ballot_sync(0xffffffffu, above < remaining && remaining <= above + all)) - 1;
         before += __reduce_add_sync(0xffffffffu, lane > src ? lower : 0);
@@ -496,31 +519,30 @@ __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const
     for (int k = 0; k < PER; ++k) sm.hist[(round & 1) ^ 1][PER * tid + k] = 0;   // every CTA is past its reads of it
     __syncthreads();
     if (cs > 1) gt_before += sm.above_before;
-    base += (unsigned)sm.bin << shift;
+    r = sel_bin(r, (unsigned)sm.bin, hi);
     remaining = sm.remaining;
-    span = (1u << shift) - 1u;
-    if (shift == 0 || sm.count <= kSelListCap) break;
-    shift = max(0, shift - kSelBinBits);
+    if (r.shift == 0 || sm.count <= kSelListCap) break;
+    r.shift = sel_next_shift(r.shift);
   }
   const int count = sm.count;
   const int before = cs > 1 ? sm.bin_before : 0;   // candidates of the lower ranks
   Threshold th;
   th.gt_before = gt_before;
   th.eq_before = 0;
-  th.listed = shift != 0;
-  if (shift == 0) {   // the bin is one key value
-    th.tau = base, th.need_eq = remaining, th.eq_total = count, th.eq_before = before;
+  th.listed = r.shift != 0;
+  if (r.shift == 0) {   // the bin is one key value
+    th.tau = r.base, th.need_eq = remaining, th.eq_total = count, th.eq_before = before;
     return th;
   }
   // list the candidates; the keys above them are wanted in any case
   for (int j = tid; j < n; j += T) {
     const unsigned key = key_at(j);
-    if (key >= base) {
-      if (key - base <= span) {
+    if (key >= r.base) {
+      if (key - r.base <= r.span) {
         const int at = atomicAdd(&sm.nlist, 1);
         sm.list[at] = key, sm.pos[at] = j;
         if (cs > 1)
-          for (int r = 0; r < cs; ++r) *cluster.map_shared_rank(&sm.all[before + at], r) = key;
+          for (int to = 0; to < cs; ++to) *cluster.map_shared_rank(&sm.all[before + at], to) = key;
       } else {
         above_bin(j);
       }
@@ -560,6 +582,8 @@ __device__ __forceinline__ Threshold threshold_search(const KeyAt& key_at, const
 
 constexpr int kBudgetCluster = kMaxCluster;
 constexpr int kBudgetThreads = 1024;
+// (0 is the padding's; order_key gives it to one NaN)
+__device__ __forceinline__ unsigned budget_key(const float f) { return max(order_key(f), 1u); }
 
 // Head budgets of one sequence under the adaptive rule (see mixkv.h).  One CTA per (sequence,
 // layer) when the call has many of them, else a cluster of up to kBudgetCluster CTAs, each with a
@@ -599,7 +623,7 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
     return;
   }
   // This CTA's slice of every head: positions [p0, p0 + n).  Its keys stand head after head, every head padded
-  // to whole words of 32 with key 0 (below every key of a number), so that a word belongs to one head.
+  // to whole words of 32 with key 0 (below every score's), so that a word belongs to one head.
   const int chunk = (P + cs - 1) / cs;
   const int p0 = min(crank * chunk, P), n = min(chunk, P - p0);
   const int npad = (n + 31) & ~31, local = H * npad;
@@ -621,7 +645,7 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
         for (int k = 0; k < 4; ++k) {
           const int i = i0 + u * kBudgetThreads + tid;
           if (i < npad && h0 + k < H) {
-            const unsigned key = i < n ? order_key(v[u][k]) : 0u;
+            const unsigned key = i < n ? budget_key(v[u][k]) : 0u;
             if (cached) bkeys[(h0 + k) * npad + i] = key;
             if (i < n) lo = min(lo, key), hi = max(hi, key);
           }
@@ -632,7 +656,7 @@ k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ 
   auto key_at = [&](const int e) -> unsigned {
     if (cached) return bkeys[e];
     const int h = e / npad, i = e - h * npad;
-    return i < n ? order_key(base[(size_t)h * stride + p0 + i]) : 0u;
+    return i < n ? budget_key(base[(size_t)h * stride + p0 + i]) : 0u;
   };
   const Threshold th =
       threshold_search<kBudgetThreads>(key_at, [](int) {}, local, (int)N, lo, hi, sm, mail, cluster, cs, crank);
@@ -1330,6 +1354,16 @@ extern "C" int mixkv_internal_adapt_threads(int64_t sequences, int32_t heads, in
                                             const int32_t* paired) {
   return mixkv::adapt_threads(sequences, heads, candidates, [&](const int n) { return alone[n]; },
                               [&](const int n) { return paired[n]; });
+}
+extern "C" int mixkv_internal_search_rounds(uint32_t lo, uint32_t hi, uint32_t key, uint32_t* base, uint32_t* span,
+                                            int32_t* shift) {
+  mixkv::SelRange r = mixkv::sel_range(lo, hi);
+  for (int n = 0;; ++n) {
+    base[n] = r.base, span[n] = r.span, shift[n] = r.shift;
+    if (r.shift == 0) return n + 1;
+    r = mixkv::sel_bin(r, (key - r.base) >> r.shift, hi);
+    r.shift = mixkv::sel_next_shift(r.shift);
+  }
 }
 extern "C" int mixkv_internal_budget_clusters(int32_t pairs, int64_t keys_per_pair, const int32_t* alone) {
   return mixkv::budget_clusters(pairs, keys_per_pair, [&](const int n) { return alone[n]; });

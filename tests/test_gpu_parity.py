@@ -429,6 +429,70 @@ def test_adaptive_budget_keys_around_the_default_shared_memory(P):
     assert np.array_equal(got["idx"].cpu().numpy()[:offs[-1]], ref["idx"])
 
 
+@pytest.mark.parametrize("H,prefixes,Bp", [
+    (2, (497, 1, 284), 1), (8, (2083, 1), 1), (1, (997,), 16), (4, (3000, 20), 8), (12, (1000,), 3),   # the budget kernel
+    (8, (33000,), 1),                                                          # its clusters
+    (16, (26001,), 5),                                                         # with keys from global memory
+    (4, (3000,), 8), (4, (700,), 0)])                                          # budgets shared out in the tail; fixed ones
+@pytest.mark.parametrize("bits", [0x7fffffff, 0xffffffff, 0x7fc00000])
+def test_scores_that_are_not_numbers_keep_to_the_budget(H, prefixes, Bp, bits):
+    # A head of NaNs (and a few elsewhere), next to the padding that the budget kernel lays behind every head: each counts
+    # as one score that ranks by its bits, so the rows stay as many as the outputs have room for
+    W, fixed = 16, Bp == 0
+    Bp = Bp or 40
+    rng = np.random.default_rng(H * sum(prefixes))
+    cu = np.concatenate([[0], np.cumsum([p + W for p in prefixes])]).astype(np.int32)
+    s = rng.uniform(0.1, 2.1, size=(H, sum(prefixes))).astype(np.float32)
+    s.view(np.uint32)[0], s.view(np.uint32)[-1, 5::97] = bits, bits
+    u = s.view(np.uint32)
+    key = np.where(u >> 31 == 1, ~u, u | np.uint32(1 << 31)).astype(np.int64)
+    pg = binding.Params(kv_heads=H, gqa_ratio=1, window=W, budget=W + Bp, budget_mode=0 if fixed else 1)
+    many = len(prefixes) > 1
+    got = binding.select(torch.from_numpy(s).cuda(), pg, cu_seqlens=[int(c) for c in cu] if many else None)
+    counts, offs, idx = (got[k].cpu().numpy().reshape(-1) for k in ("counts", "idx_offsets", "idx"))
+    floor = Bp if fixed else int(0.2 * Bp)
+    n, p0 = 0, 0
+    for b, P in enumerate(prefixes):
+        k = key[:, p0:p0 + P]
+        best = np.argsort(-k.reshape(-1), kind="stable")[:H * (Bp - floor)]   # ties: lower head, lower position
+        share = np.bincount(best // P, minlength=H)
+        for h in range(H):
+            c = min(floor + int(share[h]), P)
+            assert counts[b * H + h] == c and offs[b * H + h] == n
+            assert np.array_equal(idx[n:n + c], np.sort(np.argsort(-k[h], kind="stable")[:c]))
+            n += c
+        p0 += P
+    assert offs[-1] == n
+
+
+@pytest.mark.parametrize("name,value", [("K", float("inf")), ("K", float("nan")), ("V", float("-inf")), ("Q", float("nan"))])
+@pytest.mark.parametrize("lens,mode", [((18, 17, 300, 513, 513), 1), ((300,), 1), ((300,), 0), ((300, 33, 9000), 1)])
+def test_keys_and_values_that_are_not_numbers(lens, mode, name, value):
+    # one such element in head 0 of a layer: rows within the outputs, ascending and in range; the other heads' as without it
+    H, G, W, Bp = 2, 15, 16, 1
+    wl = synth.small_workload(H=H, G=G, W=W, seq_lens=lens, pool_kernel=7, budget=W + Bp, seed=len(lens), centroids=4)
+    _, pg = params_pair(wl)
+    pg.budget_mode = mode
+    x = {k: to_dev(v) for k, v in synth.make_layer(wl, 0, "calibrated").items() if k in ("K", "V", "Q")}
+    cu = [int(c) for c in wl.cu_seqlens] if len(lens) > 1 else None
+    clean = binding.compress_layer(x["K"], x["V"], x["Q"], pg, cu_seqlens=cu)
+    if name == "Q":
+        x["Q"][0, 0, 0, 0] = value
+    else:
+        x[name][0, sum(lens) - W - 40, 3] = value
+    out = binding.compress_layer(x["K"], x["V"], x["Q"], pg, cu_seqlens=cu)
+    assert int(out["status"].item()) == 0
+    counts, offs, idx = (out[k].cpu().numpy().reshape(-1) for k in ("counts", "idx_offsets", "idx"))
+    assert offs[0] == 0 and np.array_equal(np.diff(offs), counts)
+    for b, n in enumerate(lens):
+        assert counts[b * H:(b + 1) * H].sum() == min(H * Bp, H * (n - W))
+        for h in range(H):
+            rows = idx[offs[b * H + h]:offs[b * H + h + 1]]
+            assert (np.diff(rows) > 0).all() and (len(rows) == 0 or (rows[0] >= 0 and rows[-1] < n - W))
+    assert torch.equal(clean["s_comp"][1], out["s_comp"][1])
+    assert torch.isfinite(clean["s_comp"]).all() and not torch.isfinite(out["s_comp"][0]).all()
+
+
 @pytest.mark.parametrize("H,prefixes,mode", [
     (2, (511, 512, 513), 0), (3, (2047, 2048, 2049), 1), (1, (2561, 400, 4096), 0),   # chunks of 512 positions
     (8, (2100,) * 9, 0), (8, (2100,) * 10, 1)])                                       # 144 chunks of 2048, the last; 160

@@ -135,3 +135,22 @@ def test_segments_of_one_tile_have_statistics_of_their_own(lib, lens, heads, lay
     for s in range(max(len(of_cta) for of_cta in segments)):
         tables = {(k, wg): lib.mixkv_internal_stats_table(k, wg) for k in (s, s + 1) for wg in (0, 1)}
         assert sorted(tables.values()) == [0, 1, 2, 3]
+
+
+NAN = 0xffffffff   # key of the NaN that arithmetic on the device gives
+
+
+@pytest.mark.parametrize("lo", [1, 0x400001ff, 0x42f00dad, 0x7fffffff, 0x80000000, 0xbe123456, 0xbf800001, 0xff800000, NAN])
+@pytest.mark.parametrize("hi", [0x42f00dad, 0xbf800001, 0xbf900000, 0xff800000, 0xffc00000, NAN])
+def test_a_search_counts_nothing_but_keys_there_are(lib, lo, hi):
+    # Whatever the smallest and the largest key, NaNs among them: 2048 bins, the key looked for in every round's range, and
+    # no range past the largest key or, over 2^32, at the keys below all others, where the budget kernel's padding is.
+    if lo > hi:
+        return
+    base, span, shift = (C.c_uint32 * 3)(), (C.c_uint32 * 3)(), (C.c_int32 * 3)()
+    for key in sorted({lo, hi, max(lo, hi - 1), (lo + hi) // 2, lo + (hi - lo) // 2048 * 2047}):
+        n = lib.mixkv_internal_search_rounds(C.c_uint32(lo), C.c_uint32(hi), C.c_uint32(key), base, span, shift)
+        assert 1 <= n <= 3 and shift[n - 1] == 0
+        for r in range(n):
+            assert lo <= base[r] <= key <= base[r] + span[r] <= hi, (r, hex(key), hex(base[r]), hex(span[r]))
+            assert span[r] >> shift[r] < 2048
