@@ -636,6 +636,11 @@ int mixkv_internal_split_tiles(int32_t tiles, int32_t per_head, int32_t sms, int
   return sp.g;
 }
 
+int mixkv_internal_pass2_spare(int32_t tiles1, int32_t per_head1, int32_t tiles2, int32_t per_head2, int32_t heads,
+                               int32_t longest, int32_t sms) {
+  return pass2_spare(split_tiles(tiles1, per_head1, sms), split_tiles(tiles2, per_head2, sms), tiles2, heads, longest);
+}
+
 const char* mixkv_status_string(int status) {
   switch (status) {
     case MIXKV_OK: return "ok";

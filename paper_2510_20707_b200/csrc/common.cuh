@@ -218,6 +218,9 @@ bool tail_can_fuse(const LaunchCtx& c);
 // candidates fit one CTA, and even a head that got all shared rows would not run out of candidates (the rows of a
 // sequence are then known without looking at the others).
 bool tail_adapts(const LaunchCtx& c);
+// Whether pass 2 is launched with the spare warp's folds, from the splits of both passes, the tiles of pass 2, the heads of the
+// call ((layer, sequence, head) units) and the pass-1 tiles of the longest.
+bool pass2_spare(const Split& sp1, const Split& sp2, int tiles2, int heads, int longest);
 
 // Launch with programmatic dependent launch (and an optional cluster size): the kernel may
 // start while its predecessor in the stream drains; every kernel calls pdl_wait() before it

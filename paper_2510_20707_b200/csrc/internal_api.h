@@ -45,6 +45,11 @@ int mixkv_internal_search_rounds(uint32_t lo, uint32_t hi, uint32_t key, uint32_
 // first[0 .. CTAs] their first tiles, owner[tiles] the CTA that pass 2 and the tail look for a tile's statistics at.
 int mixkv_internal_split_tiles(int32_t tiles, int32_t per_head, int32_t sms, int32_t* first, int32_t* owner);
 
+// Whether the spare warp of pass 2 folds normalisers: tiles of either pass (per_head as above), heads of the call, pass-1 tiles
+// of its longest.
+int mixkv_internal_pass2_spare(int32_t tiles1, int32_t per_head1, int32_t tiles2, int32_t per_head2, int32_t heads,
+                               int32_t longest, int32_t sms);
+
 // Table of 16 words that the warps of a pair of pass 2's epilogue hand their statistics of a CTA's segment over in.
 int mixkv_internal_stats_table(int32_t segment, int32_t pair);
 

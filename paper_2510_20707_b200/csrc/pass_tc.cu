@@ -1208,15 +1208,23 @@ cudaError_t launch_pass1(const LaunchCtx& c, const void* K, const void* Q, int* 
                     c.ws, c.scale_log2e, (int)c.clear_status, status);
 }
 
-namespace {
 // Whether pass 2's spare warp folds the normalisers of a CTA's second and later heads.  It has the time of a
 // head's tiles for it, with a round trip for every four segments and 64 rows: not where a head lies in many CTAs.  The
-// epilogue's own fold kept it waiting 2.5 us per head: 28 layers of 4 heads and sequences of 700, 650, 800, 900 keys 108.4
-// -> 104.4 us, of 3001, 1777, 6143 293 -> 287, of eight sequences of 2 to 7 thousand 754 -> 743 (cold), of 4096 108 -> 106.5.
+// epilogue's own fold kept it waiting 2.5 us per head: 28 layers of 4 heads and sequences of 700, 650, 800, 900 keys 98.6
+// -> 94.2 us, of 3001, 1777, 6143 277 -> 268, of 4096 104.7 -> 103.3.
+// Nor where no CTA has a second head, because all have CTAs of their own or every CTA takes one tile: there the code gives
+// nothing and costs (with it / without, us: one layer of five prompts of 8 x 2000 keys 28.8 / 28.3, of 4 x 500 level, 25 layers
+// of 4 x 768 38.0 / 37.7, 12 of 8 x 640 27.5 / 27.0, 10 of 4 x 1024 27.8 / 27.4).
 constexpr int kSpareSegments = 6;
+bool pass2_spare(const Split& sp1, const Split& sp2, const int tiles2, const int heads, const int longest) {
+  if (heads == 1 || sp2.n < tiles2 || sp2.g == tiles2) return false;
+  return longest / sp1.q + 2 <= kSpareSegments;
+}
+
+namespace {
 bool pass2_spare(const LaunchCtx& c) {
-  const int most = (c.max_seq_len + kTile - 1) / kTile;   // tiles of the longest head
-  return most / c.st.sp1.q + 2 <= kSpareSegments;
+  const SeqTable& st = c.st;
+  return pass2_spare(st.sp1, st.sp2, st.layers * st.nt2, st.layers * st.batch * st.H, (c.max_seq_len + kTile - 1) / kTile);
 }
 struct P2Maps {
   CUtensorMap K, V, Q;

@@ -137,6 +137,35 @@ def test_segments_of_one_tile_have_statistics_of_their_own(lib, lens, heads, lay
         assert sorted(tables.values()) == [0, 1, 2, 3]
 
 
+def pass2_spare(lib, lens, heads, layers, window, sms=148):
+    """Whether pass 2 folds normalisers in its spare warp, and whether any of its CTAs has a second head."""
+    tiles = [[-(-(n - w) // 128) for n in lens] for w in (0, window)]
+    total = [layers * heads * sum(t) for t in tiles]
+    uniform = [t[0] if len(set(t)) == 1 else 0 for t in tiles]
+    spare = lib.mixkv_internal_pass2_spare(total[0], uniform[0], total[1], uniform[1], layers * heads * len(lens),
+                                           max(tiles[0]), sms)
+    return bool(spare), any(len(of_cta) > 1 for of_cta in pass2_segments(lib, lens, heads, layers, window, sms))
+
+
+@pytest.mark.parametrize("lens,heads,layers,window,spare", [
+    ((500,), 4, 1, 32, 0), ((500,), 8, 1, 32, 0), ((1024,), 4, 10, 32, 0), ((900,), 4, 28, 32, 0), ((2000,) * 5, 8, 1, 32, 0),
+    ((768,), 4, 25, 32, 0), ((97, 130, 160), 4, 8, 32, 0), ((16384,), 1, 1, 32, 0), ((700,), 1, 1, 32, 0),   # no second head
+    ((4096,), 4, 28, 32, 1), ((3001, 1777, 6143), 4, 28, 32, 1), ((700, 650, 800, 900), 4, 28, 32, 1), ((130, 1030), 8, 12, 16, 1),
+    ((32768, 20000, 9000), 4, 1, 32, 0)])                       # second heads, but in too many segments for one warp
+def test_the_spare_warp_folds_for_second_heads_only(lib, lens, heads, layers, window, spare):
+    got, second = pass2_spare(lib, lens, heads, layers, window)
+    assert got == bool(spare) and (second or not got)
+
+
+@pytest.mark.parametrize("sms", [148, 132, 16])
+def test_the_spare_warp_folds_for_some_cta(lib, sms):
+    for heads in (1, 2, 4, 8):
+        for layers in (1, 2, 5, 14, 28):
+            for lens in ((33,), (161,), (500,), (1024,), (4096,), (300, 300), (300, 301, 40), (2000, 130, 97, 1500), (900,) * 6):
+                got, second = pass2_spare(lib, lens, heads, layers, 32, sms)
+                assert second or not got, (sms, heads, layers, lens)
+
+
 NAN = 0xffffffff   # key of the NaN that arithmetic on the device gives
 
 
