@@ -1,10 +1,12 @@
 // Second kernel of the redundancy analysis: the Gram matrix of the block sums on the tensor cores,
 // cell (I, J) = u_I . u_J / pairs (similarity.cu leaves the scaled sums u as two fp16 parts, single rows as two bf16).
 //
-// u = hi + lo carries fp32's bits, and u.u = hi.lo + lo.hi + hi.hi but for lo.lo, 2^-24 of it.  The small products are
-// accumulated first, while the sum is small: against 64 bits the cells of blocks of 16 are 3.9e-7 off (2-norm), 1.26e-6 with
-// three bf16 parts and their six products, which moved half as many bytes again (4 heads of 32768 rows in blocks of 16
-// 30.5 us a call, now 25.4; of 20000 in blocks of 4 124, now 104).
+// u = hi + lo but for up to 2^-23 of a component, and u.u = hi.lo + lo.hi + hi.hi but for lo.lo, up to 2^-22 of a term and
+// mostly 2^-24.  Both lie below what the accumulation in fp32 leaves, so the small products go first, while the sum is small:
+// against 64 bits the cells of 32768 video keys in blocks of 16 are 3.5e-7 off (2-norm); with three bf16 parts, which hold all
+// of fp32's bits, and six products in the order in which they came 1.34e-6.  Blocks of 2 to 4096 and text, random, sparse and
+// cancelling rows: 1.8e-8 to 1.8e-6, never above what the three parts left.  (They moved half as many bytes again: 4 heads of
+// 32768 rows in blocks of 16 30.5 us a call, now 25.4; of 20000 in blocks of 4 124, now 104.)
 // Persistent CTAs walk a contiguous run of tiles (head, I, J): 128 blocks I on M, NT blocks J on N,
 // only tiles that touch or lie right of the diagonal.  The parts of I stay in shared memory while
 // J runs (2 x 32 KB), the parts of J go through a ring of four half parts, and two accumulator stages

@@ -116,6 +116,31 @@ def test_large_maps_in_dealt_runs(H, L, block):
         assert abs(float(mean[h]) - float((total @ total - L) / (L * (L - 1.0)))) <= ATOL + RTOL * abs(float(mean[h]))
 
 
+@pytest.mark.parametrize("H,L,block", [(2, 1500, 2), (2, 1301, 3), (1, 4096, 16), (2, 3003, 17), (1, 4000, 31), (1, 20000, 256),
+                                       (1, 15001, 700), (1, 40000, 4096)])
+def test_maps_keep_the_bits_of_their_sums(H, L, block):
+    # Against 64 bits, tighter than what a single part of the sums, or one product of parts less, would pass: with exact
+    # accumulation those leave 1.7e-5 and more.  The bound: eight steps of the largest product truncated to fp32 2^-23 each,
+    # 9.5e-7, the parts and the product left out 2 x 2^-23 and 2^-22, the norms of two rows 2 x 2^-22, the sums 2^-23 each.
+    gen = torch.Generator(device="cuda").manual_seed(L)
+    X = (torch.randn((H, L, 128), generator=gen, device="cuda") + 1.3 *
+         torch.randn((H, 1, 128), generator=gen, device="cuda")).bfloat16()
+    cells, _ = binding.similarity_map(X, block)
+    T = -(-L // block)
+    for h in range(H):
+        u = X[h].double()
+        u = u / u.norm(dim=1, keepdim=True)
+        sums = torch.zeros((T * block, 128), dtype=torch.float64, device="cuda")
+        sums[:L] = u
+        sums = sums.view(T, block, 128).sum(1)
+        n = torch.full((T,), float(block), dtype=torch.float64, device="cuda")
+        n[-1] = L - (T - 1) * block
+        ref = (sums @ sums.T) / (n[:, None] * n[None, :])
+        pairs = n * (n - 1)
+        ref.diagonal().copy_(torch.where(pairs > 0, ((sums * sums).sum(1) - n) / pairs.clamp(min=1), 0.0))
+        assert float((cells[h].double() - ref).norm()) <= 2e-6 * float(ref.norm())
+
+
 def test_keys_and_values_of_a_c2_layer():
     wl = synth.CONFIGS["C2"]
     x = synth.make_layer(wl, 7, "calibrated")
