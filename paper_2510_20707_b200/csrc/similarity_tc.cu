@@ -389,17 +389,18 @@ long long device_l2_bytes() {
 // so that all CTAs together write whole rows of the map at a time.  That counts where the map goes to HBM: it leaves L2
 // in about the order in which it was written.  Contiguous / in runs, us, B200 (L2 of 133 MB), maps in turn on four inputs:
 //   Rows that do not start on 32-byte sectors (T not a multiple of 8, or a map that does not): neighbouring tiles share
-//   sectors, and a sector that leaves half written is read again.  Runs of one from half of L2 on: sums, 4 heads x 2401 cells
-//   a side (92 MB) 46.4 / 44.2, x 2801 (126 MB) 59.4 / 52.2, 8 x 1950 (122 MB) 63.7 / 60.3; the line lies where it was
-//   measured with longer operands (4 x 2001, 64 MB, 41.2 / 36.7 then, 30.4 / 33.0 now; 8 x 1451, 67 MB, 37.5 / 40.7).
+//   sectors, and a sector that leaves half written is read again.  Runs of one from half of L2 on: 8 heads x 1451 cells a side
+//   (67 MB) in blocks of 1, 4, 16 43.5 / 38.8, 41.1 / 36.4, 41.4 / 41.0, 4 x 2101 (71 MB) 43.9 / 37.8, 41.9 / 35.4, 42.2 / 37.4,
+//   4 x 2801 (126 MB) 66.5 / 54.3, 64.5 / 53.6, 64.6 / 54.3; below it 4 x 2001 (64 MB) 38.7 / 34.2, 36.4 / 31.6, 37.1 / 33.7,
+//   4 x 1801 (52 MB) 34.8 / 34.1, 32.4 / 31.6, 32.7 / 33.1, 4 x 1501 (36 MB) 28.2 / 28.8, 25.8 / 26.5, 24.5 / 26.8.  (One map
+//   written over and over stays in L2 and is better off contiguous up to 58 MB: 4 x 1901 32.2 / 34.0, 4 x 2001 35.5 / 34.2.)
 //   Whole sectors: only the largest maps gain (pages of HBM filled in one go), from 9/4 of L2 on: single rows in runs of
 //   one (4 x 4400, 310 MB, 86.4 / 83.7, x 5000 113 / 105), sums in runs of two (4 x 4400 89.0 / 84.3, x 5000 117 / 107,
 //   x 5600 136 / 125; 4 x 4000, 256 MB, 73.9 / 72.3).
-// kind: 2 single rows, 3 sums.
-int gram_run(const int heads, const int T, const int kind, const bool whole_sectors, const long long l2) {
+int gram_run(const int heads, const int T, const bool single_rows, const bool whole_sectors, const long long l2) {
   const long long bytes = 4LL * heads * T * T;
   if (!whole_sectors) return 2 * bytes > l2 ? 1 : 0;
-  return 4 * bytes > 9 * l2 ? (kind == 2 ? 1 : 2) : 0;
+  return 4 * bytes > 9 * l2 ? (single_rows ? 1 : 2) : 0;
 }
 
 template <int NT, bool DEALT>
@@ -440,7 +441,7 @@ cudaError_t launch_gram(const GramArgs& g, cudaStream_t s) {
   const bool narrow = wide * g.heads < device_sm_count();
   const long long per_head = narrow ? tiles_per_head<32>(g.T) : wide;
   const bool whole_sectors = g.T % 8 == 0 && (reinterpret_cast<uintptr_t>(g.cells) & 31) == 0;
-  const int run = narrow ? 0 : gram_run(g.heads, g.T, g.block == 1 ? 2 : 3, whole_sectors, device_l2_bytes());
+  const int run = narrow ? 0 : gram_run(g.heads, g.T, g.block == 1, whole_sectors, device_l2_bytes());
   return narrow ? launch_gram_t<32, false>(g, per_head, 0, s)
          : run  ? launch_gram_t<128, true>(g, per_head, run, s)
                 : launch_gram_t<128, false>(g, per_head, 0, s);
@@ -449,5 +450,5 @@ cudaError_t launch_gram(const GramArgs& g, cudaStream_t s) {
 }  // namespace mixkv
 
 extern "C" int mixkv_internal_gram_run(int32_t heads, int32_t cells, int32_t parts, int32_t whole_sectors, int64_t l2_bytes) {
-  return mixkv::gram_run(heads, cells, parts, whole_sectors != 0, l2_bytes);
+  return mixkv::gram_run(heads, cells, parts == 2, whole_sectors != 0, l2_bytes);
 }
