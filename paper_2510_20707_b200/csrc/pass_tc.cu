@@ -894,12 +894,14 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
         const float part = acc0 + acc1;
         if (chalf) {
           // The other half reads this word before it arrives on tempty, and the next tile of this stage is
-          // not complete before that: no barrier for the way back.
+          // not complete before that: no barrier for the way back.  This half waits at the barrier all the same, for no
+          // longer than it would for that tile: after an abort nothing else keeps it from a second arrival ahead of the other
+          // half's first, which would end that barrier early and leave the other half at its last one for good.
           sxp[wg * 128 + key] = part;
-          named_bar_arrive(xbar, 256);
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(&bars->tempty[wg]);
+          named_bar_sync(xbar, 256);
         } else {
           float dot = 0.f;
           if (ok) {

@@ -1,6 +1,8 @@
 """The rules that split a call's work over clusters of CTAs (csrc/internal_api.h), without a device: whatever number
 of clusters a device holds at once, no rule asks for more, which would cost a second wave."""
 import ctypes as C
+import os
+import re
 
 import pytest
 
@@ -164,6 +166,17 @@ def test_the_spare_warp_folds_for_some_cta(lib, sms):
             for lens in ((33,), (161,), (500,), (1024,), (4096,), (300, 300), (300, 301, 40), (2000, 130, 97, 1500), (900,) * 6):
                 got, second = pass2_spare(lib, lens, heads, layers, 32, sms)
                 assert second or not got, (sms, heads, layers, lens)
+
+
+def test_nobody_arrives_twice_ahead_of_a_reader():
+    # Bounded waits end at once after an abort, named barriers do not.  A role that arrives at one without waiting could come
+    # to it again ahead of the reader's first time; two such arrivals complete it, and the reader waits at its last one for
+    # good.  So there are none but in pairs: the reader of the one arrives at the other, at which the writer waits first.
+    source = open(os.path.join(os.path.dirname(build.__file__), "csrc", "pass_tc.cu")).read()
+    calls = re.findall(r"named_bar_(arrive|sync)\(([^,]+),", source)
+    assert [bar for kind, bar in calls if kind == "arrive"] == ["6 + blk", "8 + blk"]
+    assert [(kind, bar) for kind, bar in calls if "blk" in bar] == [   # the writer's, then the reader's
+        ("sync", "8 + blk"), ("arrive", "6 + blk"), ("sync", "6 + blk"), ("arrive", "8 + blk")]
 
 
 NAN = 0xffffffff   # key of the NaN that arithmetic on the device gives
