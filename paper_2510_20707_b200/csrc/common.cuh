@@ -154,9 +154,9 @@ struct ClusterFit {
     return n;
   }
 };
-// Fills a CUtensorMap (passed as void*) for a bf16 tensor of the given rank: dims innermost first,
+// Fills a CUtensorMap (passed as void*) for a tensor of 16-bit elements of the given rank: dims innermost first,
 // strides in bytes of dimensions 1 .. rank-1, box extents; 128-byte swizzle, zero fill outside.
-bool encode_bf16_map(void* tm, const void* base, int rank, const unsigned long long* dims,
+bool encode_map_16bit(void* tm, const void* base, int rank, const unsigned long long* dims,
                      const unsigned long long* strides_bytes, const unsigned* box);
 // MIXKV_OK on a compute-capability 10.x device, MIXKV_ERR_UNSUPPORTED on any other,
 // MIXKV_ERR_CUDA when none can be queried; *major_out (optional) receives the major number.

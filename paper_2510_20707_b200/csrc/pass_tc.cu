@@ -371,9 +371,9 @@ k_pass1(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
                 const uint32_t a_lo = q_lo + (ks >> 2) * q_half + (uint32_t)(mb * (16384 >> 4) + (ks & 3) * 2);
                 const uint32_t b_lo = kb_lo + (uint32_t)((ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2);
                 if (ks == 0)
-                  umma_bf16_lo<0>(td + mb * 128, a_lo, b_lo, idesc, on);
+                  umma_f16_lo<0>(td + mb * 128, a_lo, b_lo, idesc, on);
                 else
-                  umma_bf16_lo<1>(td + mb * 128, a_lo, b_lo, idesc, on);
+                  umma_f16_lo<1>(td + mb * 128, a_lo, b_lo, idesc, on);
               }
             }
             umma_commit(&bars->empty[s], on);
@@ -788,9 +788,9 @@ k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtenso
           const uint32_t a_lo = kb_lo + (uint32_t)((ks >> 2) * (kHalfBytes >> 4) + (ks & 3) * 2);
           const uint32_t b_lo = q_lo + (ks >> 2) * q_half + (uint32_t)((ks & 3) * 2);
           if (ks == 0)
-            umma_bf16_lo<0>(td, a_lo, b_lo, idesc, on);
+            umma_f16_lo<0>(td, a_lo, b_lo, idesc, on);
           else
-            umma_bf16_lo<1>(td, a_lo, b_lo, idesc, on);
+            umma_f16_lo<1>(td, a_lo, b_lo, idesc, on);
         }
         umma_commit(&bars->kempty[s], on);
         umma_commit(&bars->tfull[ts], on);
@@ -1103,7 +1103,7 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// Fills a map of a bf16 tensor: dims innermost first, strides in bytes of dimensions 1 .. rank - 1, box extents; 128-byte
+// Fills a map of a tensor of 16-bit elements: dims innermost first, strides in bytes of dimensions 1 .. rank - 1, box extents; 128-byte
 // swizzle, zero fill outside.  The driver wants a current context for it.  The first call of a thread may find none (the
 // runtime binds the device's context when a call of its own needs it, and none has by then): bound here.
 bool encode_map(CUtensorMap* tm, const void* base, const cuuint32_t rank, const cuuint64_t* dims,
@@ -1171,7 +1171,7 @@ static_assert(passes_fit(), "a pass asks for more shared memory than a CTA may h
 
 }  // namespace
 
-bool encode_bf16_map(void* tm, const void* base, int rank, const unsigned long long* dims,
+bool encode_map_16bit(void* tm, const void* base, int rank, const unsigned long long* dims,
                      const unsigned long long* strides_bytes, const unsigned* box) {
   cuuint64_t d[5], st[4];
   cuuint32_t bx[5];

@@ -230,8 +230,8 @@ k_gram(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensor
           const uint32_t ob = b0 + (uint32_t)sb * (kBHalf >> 4);
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks) {
-            if (first && ks == 0) umma_bf16_lo<0>(tmem + ts * 128, oa + ks * 2, ob + ks * 2, idesc, on);
-            else umma_bf16_lo<1>(tmem + ts * 128, oa + ks * 2, ob + ks * 2, idesc, on);
+            if (first && ks == 0) umma_f16_lo<0>(tmem + ts * 128, oa + ks * 2, ob + ks * 2, idesc, on);
+            else umma_f16_lo<1>(tmem + ts * 128, oa + ks * 2, ob + ks * 2, idesc, on);
           }
         };
         int values0 = 0;   // stage of the values' first half
@@ -418,8 +418,8 @@ cudaError_t launch_gram_t(const GramArgs& g, const long long per_head, const int
   const unsigned long long strides[2] = {(unsigned long long)kHeadDim * 2,
                                          (unsigned long long)g.T * kHeadDim * 2};
   const unsigned boxA[3] = {64, 128, 1}, boxB[3] = {64, (unsigned)NT, 1};
-  if (!encode_bf16_map(&tmA, g.parts, 3, dims, strides, boxA) ||
-      !encode_bf16_map(&tmB, g.parts, 3, dims, strides, boxB))
+  if (!encode_map_16bit(&tmA, g.parts, 3, dims, strides, boxA) ||
+      !encode_map_16bit(&tmB, g.parts, 3, dims, strides, boxB))
     return cudaErrorInvalidValue;
   const int grid = (int)(total < device_sm_count() ? total : device_sm_count());
   return launch_pdl(k_gram<NT, DEALT>, dim3((unsigned)grid), dim3(kGThreads), smem, s, 1, tmA, tmB, g.nz, g.us,

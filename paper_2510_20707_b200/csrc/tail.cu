@@ -263,7 +263,7 @@ k_mixpool(const SeqTable st, const Workspace ws, const float* __restrict__ s_div
   const float pad = avg ? 0.f : -INFINITY;
   const SegList sl = pass2_segments(st, layer, b, h);   // (divisions: ahead of the wait)
   pdl_wait();
-  // eight rounds of 256 positions (+ the pooling halo in a ninth)
+  // rounds of 256 positions (+ the pooling halo in one more)
   constexpr int kRounds = CH / 256;
   const int nstage = n + 2 * half;
   float raw[kRounds + 1], vn[kRounds], dv[kRounds];
@@ -592,8 +592,9 @@ __device__ __forceinline__ unsigned budget_key(const float f) { return max(order
 // otherwise every sweep reads them from global memory.
 // Bound by its chain of block-wide (cluster-wide) steps, not by the scores it reads: 28 layers x 8 ragged
 // sequences of 4 heads, 2 to 7 thousand candidates each, 65 us with digit passes over the raw keys, 35 us with
-// threshold_search.  In a cluster that chain also crosses four barriers (8 heads of up to 12 thousand: 19 us);
-// clusters of two, half the threads and batched reads of the peers' counts were no faster.
+// threshold_search.  In a cluster that chain also crosses six barriers or more (start, range, counts of each round, candidates,
+// heads' counts, end), with what a CTA needs of the others sent ahead of them but for the heads' counts.  Clusters of two and
+// half the threads were no faster (measured when it was fetched behind four barriers).
 __global__ void __launch_bounds__(kBudgetThreads)
 k_budget(const SeqTable st, const float* __restrict__ scores, int* __restrict__ counts,
          const int Bp, const int floor_slots, const int cache_cap) {
@@ -1173,9 +1174,9 @@ int paired_clusters(const int size) {
 
 // CTAs per (sequence, layer) pair: one while it has 8192 keys or less of all heads (the exchanges cost as much as
 // the sweeps they save), else as many as leave each that much and are all resident at once, one per SM (15 clusters of
-// eight are, 33 of four, 74 of two).  Whole calls, eight CTAs each up to 17 pairs and one
-// beyond that against this: 17 pairs of 3000 keys 50.1 / 37.9 us; 17, 20, 28 of 96000 217 / 204, 368 / 238, 439 /
-// 322 us; 28, 56 of 32000 134 / 122, 227 / 224 us.
+// eight are, 33 of four, 74 of two).  One CTA each / this, whole calls, pairs of 16 heads x keys, us: 4 of 3000 72.7 / 59.5,
+// 15 of 4000 245 / 156, 17, 20, 28 of 6000 381 / 248, 433 / 294, 526 / 392, 28, 56 of 2000 163 / 159, 290 / 291, one of
+// 30000 806 / 187; 17 of 12 x 2000 92.4 / 87.5.
 template <typename Fit>
 int budget_clusters(const int pairs, const long long keys, const Fit& alone) {
   int cs = 1;
@@ -1249,18 +1250,20 @@ bool adapt_pairs_fit(const int P) {
 }
 
 // Threads of a CTA when the heads of a sequence are a cluster that shares its budget out (k_tail with ADAPT), 0: where
-// mix, budget and tail kernels are as good.  Every thread reads its bins of all heads over distributed shared memory,
-// so 1024 threads, as long as all clusters are resident with an SM to each CTA.  Where they are not, 512 threads and two
-// CTAs to an SM, all resident that way; clusters of seven and eight gain that way on long heads only.  Heads too long for
-// two to share an SM take 1024 threads in more than one wave.  (Layer, sequence) pairs of heads x keys, whole calls,
-// three kernels / this, us (and with 256 threads for heads of 1024 keys and less, as it once was):
-//   all resident, 1024: 4 of 4 x 1024 to 8 x 24576 all faster: 4 of 8 x 760 36.2 / 31.5 (68.9), 33 of 4 x 760 47.3 / 40.0
-//     (56.1), 1 of 4 x 4300 40.3 / 32.2, 15 of 8 x 9000 159 / 150, 74 of 2 x 17000 380 / 348, 15 of 8 x 24500 471 / 427
-//   not resident (1024 threads in a second wave in brackets): 36 of 4 x 760 46.2 / 43.3 (52.3), 110 of 2 x 4300
-//     152 / 141 (153), 23 of 6 x 2300 73.4 / 71.8 (77.5), 38 of 6 x 9000 318 / 299 (306), 60 of 4 x 17000 648 / 596 (614);
-//     17 of 8 x 760 48.9 / 52.0 (56.8), x 2300 72.0 / 76.6 (81.9), x 9000 187 / 189 (195), 29 of 8 x 4300 156 / 153
-//     (160), x 17000 616 / 580 (589), 17 of 8 x 17000 361 / 353 (361)
-//   too long for pairs: 17 of 8 x 24500 511 / 497, 60 of 4 934 / 837, 23 of 6 512 / 505
+// mix, budget and tail kernels are as good.  What all threads do (sweeps, counts sent to the other heads) is most of it on
+// long heads, so 1024 threads, as long as all clusters are resident with an SM to each CTA.  Where they are not, 512 threads
+// and two CTAs to an SM, all resident that way.  Heads too long for two to share an SM take 1024 threads in more than one
+// wave.  (Layer, sequence) pairs of heads x keys, whole calls, three kernels / this, us:
+//   all resident, 1024 (512 threads in brackets): 4 of 8 x 760 32.2 / 27.7 (28.0), 33 of 4 x 760 41.5 / 37.5 (38.6), 1 of
+//     4 x 4300 34.8 / 28.3 (27.5), 15 of 8 x 9000 167 / 157 (163), 74 of 2 x 17000 352 / 338 (346), 15 of 8 x 24500 413 /
+//     399 (399)
+//   not resident (1024 threads in a second wave in brackets): 36 of 4 x 760 42.2 / 39.5 (51.3), 110 of 2 x 4300
+//     149 / 138 (154), 23 of 6 x 2300 73.5 / 65.2 (76.3), 38 of 6 x 9000 302 / 285 (296), 60 of 4 x 17000 573 / 551 (564),
+//     17 of 8 x 9000 191 / 179 (193), x 17000 335 / 324 (339), 29 of 8 x 17000 561 / 536 (548)
+//   too long for pairs: 17 of 8 x 24500 476 / 478, 60 of 4 820 / 801, 23 of 6 476 / 483
+// Seven and eight heads of 8192 keys or less in more clusters than are resident one to an SM keep the three kernels: that line
+// was drawn when a search fetched its counts from the peers (17 of 8 x 760 48.9 / 52.0).  With the counts sent, 512 threads
+// are ahead there as well: 17 of 8 x 760 44.5 / 39.5, x 2300 72.6 / 64.9, 16 of 8 x 8000 161 / 154, 29 of 8 x 4300 164 / 150.
 template <typename Alone, typename Paired>
 int adapt_threads(const long long sequences, const int heads, const int P, const Alone& alone, const Paired& paired) {
   if (sequences <= alone(heads)) return 1024;
