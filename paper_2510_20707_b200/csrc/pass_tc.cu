@@ -631,7 +631,7 @@ __host__ __device__ __forceinline__ int stats_table(const int segn, const int wg
 // grid = g2 persistent CTAs: K producer, MMA, V producer, 1 spare, 16 epilogue, 4 value-norm warps.
 // NCH: pieces of 16 query columns per epilogue warp, at most.
 // SPARE: the spare warp folds the normalisers of the CTA's segments after the first (see pass2_spare).  A template argument
-// because the code costs the calls that cannot use it 0.3 to 0.7 us.
+// because the code costs the calls that cannot use it up to half a microsecond.
 template <int NCH, bool SPARE>
 __global__ void __launch_bounds__(kP2Threads, 1)
 k_pass2(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
